@@ -1,7 +1,7 @@
 """Build the CUDA shading library ``libshshadow.so`` in-tree (sm_103a).
 
-Compiles ``csrc/shs_api.cu`` and one object of ``csrc/shs_kern.cu`` per band
-count (-DSHS_NB=1..8) in parallel with nvcc, then links them into
+Compiles ``csrc/shs_api.cu`` and one object of ``csrc/shs_kern.cu`` (1 to 5
+bands) or ``csrc/shs_hi_forward.cu`` and ``csrc/shs_hi_backward.cu`` (6 to 8) per band count in parallel with nvcc, then links them into
 ``paper_2104_00359_gb300/lib/libshshadow.so``.  Objects are cached under
 ``_build/`` and rebuilt when a source or header is newer.
 """
@@ -92,8 +92,10 @@ def build(verbose=False, jobs=None):
              (os.path.join(CSRC, "shs_chain.cu"), os.path.join(BUILD, "shs_chain.o"), []),
              (os.path.join(CSRC, "shs_tail_tc.cu"), os.path.join(BUILD, "shs_tail_tc.o"), ["-DSHS_NB=8"])]
     for n in BANDS:
-        units.append((os.path.join(CSRC, "shs_kern.cu"), os.path.join(BUILD, f"shs_kern_{n}.o"),
-                      [f"-DSHS_NB={n}"]))
+        srcs = ("shs_hi_forward", "shs_hi_backward") if n >= 6 else ("shs_kern",)
+        for src in srcs:
+            units.append((os.path.join(CSRC, src + ".cu"), os.path.join(BUILD, f"{src}_{n}.o"), [f"-DSHS_NB={n}"]))
+    units.sort(key=lambda u: "_hi_" not in u[0])   # the longest compilations first
     todo = [u for u in units if _stale(u[1], deps)]
     if todo:
         jobs = jobs or min(len(todo), max(1, os.cpu_count() or 1))

@@ -508,66 +508,7 @@ def packed_lines(lines):
     return out
 
 
-QUAD_FROM = 7   # band counts from which the triple product runs by quadrature
-
-
-def quadrature_tables(n):
-    """Separable quadrature for the truncated triple product at n bands.
-
-    y_i(theta, phi) = Leg_i(theta) T_f(i)(phi) with T_0 = 1, T_{2m-1} =
-    cos(m phi), T_{2m} = sin(m phi).  The product of three SH of degree < n is
-    a polynomial of degree <= 3(n-1) on the sphere, so NZ = 3(n-1)/2 + 1
-    Gauss-Legendre nodes in z = cos(theta) and NP = 3(n-1) + 1 uniform azimuths
-    integrate it exactly:  (a * b)_i = sum_{za, pb} w_za A B y_i.
-    Returns (leg [NZ][K], trig [NP][2n-1], w [NZ]) in float64 and checks the
-    factorisation and the exactness against the Gaunt tensor."""
-    K = n * n
-    D = 3 * (n - 1)
-    NZ, NP = D // 2 + 1, D + 1
-    z, wz = np.polynomial.legendre.leggauss(NZ)
-    H = homogeneous_polys(n)
-    N = norms(n)
-
-    def ysh(i, x, y, zz):
-        return N[i] * sum(float(v) * x ** a * y ** b * zz ** c for (a, b, c), v in H[i].items())
-
-    def f_of(m):
-        return 0 if m == 0 else (2 * m - 1 if m > 0 else 2 * (-m))
-
-    leg = np.zeros((NZ, K))
-    for za in range(NZ):
-        st = math.sqrt(1.0 - z[za] ** 2)
-        for i in range(K):
-            l = int(math.isqrt(i))
-            m = i - l * l - l
-            ph = 0.0 if m >= 0 else math.pi / (2 * (-m))
-            leg[za, i] = ysh(i, st * math.cos(ph), st * math.sin(ph), z[za])
-    phis = 2.0 * math.pi * (np.arange(NP) + 0.5) / NP
-    trig = np.zeros((NP, 2 * n - 1))
-    trig[:, 0] = 1.0
-    for m in range(1, n):
-        trig[:, 2 * m - 1] = np.cos(m * phis)
-        trig[:, 2 * m] = np.sin(m * phis)
-    w = wz * 2.0 * math.pi / NP
-    # checks: separation at an arbitrary azimuth, exactness against C_ijk
-    rng = np.random.default_rng(0)
-    for za in range(NZ):
-        st = math.sqrt(1.0 - z[za] ** 2)
-        ph = 0.731
-        for i in range(K):
-            l = int(math.isqrt(i))
-            m = i - l * l - l
-            t = 1.0 if m == 0 else (math.cos(m * ph) if m > 0 else math.sin(-m * ph))
-            assert abs(ysh(i, st * math.cos(ph), st * math.sin(ph), z[za]) - leg[za, i] * t) < 1e-12
-    fidx = [f_of(i - int(math.isqrt(i)) ** 2 - int(math.isqrt(i))) for i in range(K)]
-    Y = np.einsum("ai,bi->abi", leg, trig[:, fidx])          # [NZ, NP, K]
-    a, bb = rng.normal(size=K), rng.normal(size=K)
-    prod = np.einsum("ab,ab,abi->i", w[:, None] * (Y @ a), Y @ bb, Y)
-    ref = np.zeros(K)
-    for (i, j, k), v in gaunt_monomial(n).items():
-        ref[i] += float(v) * (a[j] * bb[k] + (a[k] * bb[j] if j != k else 0.0))
-    assert np.abs(prod - ref).max() < 1e-10 * max(1.0, np.abs(ref).max()), np.abs(prod - ref).max()
-    return leg, trig, w
+LANE_PAIR_FROM = 6   # band counts from which a pair of lanes shares a point and products run by quadrature
 
 
 def exp_rule_tables(n):
@@ -628,15 +569,110 @@ def emit_exp_rule(n):
             "#endif"]
 
 
-def emit_quadrature(n):
-    leg, trig, w = quadrature_tables(n)
+def lane_pair_legs(n):
+    """(m, r) of the Legendre factors one lane of a lane pair holds: lane
+    parity b owns the coefficients with l + |m| = b mod 2, l = m + b + 2 r."""
+    return [(m, r) for m in range(n) for r in range((n - m + 1) // 2)]
+
+
+def lane_pair_rule(n, nz, quads):
+    """A rule of nz (even) Gauss-Legendre nodes in z and 4 * quads azimuths
+    2 pi (b + 1/2) / (4 quads), arranged for a pair of lanes: step t holds the
+    nodes z_t > 0 (even lane) and -z_t (odd lane), with Leg_lm(z_t) of each
+    lane's own coefficients (l + |m| even, odd; 0 where l >= n).  The four
+    azimuths phi, -phi, pi - phi, pi + phi of a quad share cos(m phi),
+    sin(m phi).  Returns (leg [nz/2][2][legs], w [nz/2], phi [quads])."""
+    z, wz = np.polynomial.legendre.leggauss(nz)
+    H = homogeneous_polys(n)
+    N = norms(n)
+    legs = lane_pair_legs(n)
+    leg = np.zeros((nz // 2, 2, len(legs)))
+    w = np.zeros(nz // 2)
+    for t in range(nz // 2):
+        zt = z[nz - 1 - t]
+        assert zt > 0 and abs(zt + z[t]) < 1e-15
+        w[t] = wz[t] * 2.0 * math.pi / (4 * quads)
+        st = math.sqrt(1.0 - zt * zt)
+        for b in range(2):
+            for e, (m, r) in enumerate(legs):
+                l = m + b + 2 * r
+                if l < n:
+                    leg[t, b, e] = N[l * l + l + m] * sum(float(v) * st ** a * 0.0 ** bb * zt ** c
+                                                          for (a, bb, c), v in H[l * l + l + m].items())
+    return leg, w, 2.0 * math.pi * (np.arange(quads) + 0.5) / (4 * quads)
+
+
+def lane_pair_product_rule(n):
+    """The lane-pair rule of the truncated triple product: degree 3 (n - 1) is
+    integrated exactly by an even number of nodes >= 3 (n - 1) / 2 + 1 / 2 and
+    a multiple of four azimuths > 3 (n - 1).  Each Legendre factor carries the
+    cube root of the node's weight (an integrand has three factors).  Checked
+    against the Gaunt tensor."""
+    D = 3 * (n - 1)
+    nz = (D // 2 + 1) + (D // 2 + 1) % 2
+    quads = (D + 4) // 4
+    leg, w, phi = lane_pair_rule(n, nz, quads)
+    leg = leg * np.cbrt(w)[:, None, None]
+    K = n * n
+    cols = []
+    for t in range(nz // 2):
+        for sz in (1.0, -1.0):
+            for q in range(quads):
+                for ph in (phi[q], -phi[q], math.pi - phi[q], math.pi + phi[q]):
+                    y = np.zeros(K)
+                    for b in range(2):
+                        for e, (m, r) in enumerate(lane_pair_legs(n)):
+                            l = m + b + 2 * r
+                            if l < n:
+                                v = leg[t, b, e] * (sz if b else 1.0)
+                                y[l * l + l + m] = v * math.cos(m * ph)
+                                if m:
+                                    y[l * l + l - m] = v * math.sin(m * ph)
+                    cols.append(y)
+    Y = np.array(cols)
+    rng = np.random.default_rng(0)
+    a, bb = rng.normal(size=K), rng.normal(size=K)
+    prod = ((Y @ a) * (Y @ bb)) @ Y
+    ref = np.zeros(K)
+    for (i, j, k), v in gaunt_monomial(n).items():
+        ref[i] += float(v) * (a[j] * bb[k] + (a[k] * bb[j] if j != k else 0.0))
+    assert np.abs(prod - ref).max() < 1e-10 * max(1.0, np.abs(ref).max())
+    return leg, phi
+
+
+def emit_lane_pair(n):
+    """(tables, members of SH<n>) of the lane-pair rules."""
+    leg, phi = lane_pair_product_rule(n)
+    eleg, ew, ephi = lane_pair_rule(n, 2 * n, n)
 
     def arr(name, a):
         vals = ", ".join(fmt(("c", float(v))) for v in np.asarray(a).ravel())
-        return f"static __constant__ float {name}[{np.asarray(a).size}] = {{{vals}}};"
-    return [f"#if defined(SHS_NB) && SHS_NB == {n}",
-            arr(f"kQuadLeg{n}", leg), arr(f"kQuadTrig{n}", trig), arr(f"kQuadW{n}", w),
-            "#endif"], leg.shape[0], trig.shape[0]
+        return f"static __device__ const float {name}[{np.asarray(a).size}] = {{{vals}}};"
+
+    def trig(name, phis):
+        out = [f"    __device__ __forceinline__ static float {name}(int b, int h) {{   // h = 2m - 1: cos(m phi_b), 2m: sin",
+               f"        switch (b * {2 * n - 1} + h) {{"]
+        for b, ph in enumerate(phis):
+            for h in range(1, 2 * n - 1):
+                m = (h + 1) // 2
+                v = math.cos(m * ph) if h % 2 else math.sin(m * ph)
+                out.append(f"            case {b * (2 * n - 1) + h}: return {fmt(('c', v))};")
+        return out + ["            default: return 1.0f;", "        }", "    }"]
+    def rows(phis):   # [quads][2n - 1]: 1, cos m phi, sin m phi
+        return [[1.0] + [(math.cos if h % 2 else math.sin)((h + 1) // 2 * ph) for h in range(1, 2 * n - 1)] for ph in phis]
+    tables = [f"#if defined(SHS_NB) && SHS_NB == {n}", "// lane-pair rules: product, then projected exponential (plain, weighted)",
+              arr(f"kLpLeg{n}", leg), arr(f"kLeLeg{n}", np.stack([eleg, eleg * ew[:, None, None]])),
+              arr(f"kLpTrig{n}", rows(phi)).replace("__device__ const", "__constant__"), "#endif"]
+    members = [f"    static constexpr int LPS = {leg.shape[0]};   // lane-pair product rule: node pairs",
+               f"    static constexpr int LPQ = {len(phi)};   // ... and azimuth quads",
+               f"    static constexpr int LES = {n};   // lane-pair projected-exponential rule: node pairs",
+               f"    static constexpr int LEQ = {n};   // ... and azimuth quads",
+               f"#if defined(SHS_NB) && SHS_NB == {n}",
+               f"    __device__ __forceinline__ static const float* lp_leg() {{ return kLpLeg{n}; }}",
+               f"    __device__ __forceinline__ static const float* le_leg() {{ return kLeLeg{n}; }}",
+               f"    __device__ __forceinline__ static const float* lp_trig_row(int b) {{ return kLpTrig{n} + b * {2 * n - 1}; }}",
+               "#endif"] + trig("lp_trig", phi) + trig("le_trig", ephi)
+    return tables, members
 
 
 def indent(lines, k=8):
@@ -648,7 +684,7 @@ def generate():
         "// Generated by gen_tables.py -- do not edit.",
         "// Real SH polynomials, their reverse-mode gradients, and the truncated",
         "// SH triple product (Sec. 3.2, Eq. 3 and Eq. 6-7), unrolled per band count",
-        "// (from 7 bands, quadrature tables for the triple product instead).",
+        "// (from 6 bands, lane-pair quadrature tables for the triple product instead).",
         "#pragma once",
         "",
         "namespace shsgen {",
@@ -662,22 +698,21 @@ def generate():
         code, outs = build_ybar(n)
         fwd = emit_forward(code, outs, "Y")
         vjp = emit_forward(code, [], "Y") + emit_vjp(code, outs)
-        mul_l, sqr_l = emit_gaunt(n, C) if n < QUAD_FROM else ([], [])
+        mul_l, sqr_l = emit_gaunt(n, C) if n < LANE_PAIR_FROM else ([], [])
         N = norms(n)
         A = ahat(n)
-        if n >= QUAD_FROM:
-            parts.extend(emit_quadrature(n)[0])
-        parts.extend(emit_exp_rule(n))
+        parts.extend(emit_exp_rule(n) if n < LANE_PAIR_FROM else emit_lane_pair(n)[0])
         parts.append(f"template <> struct SH<{n}> {{")
         parts.append(f"    static constexpr int K = {K};")
         parts.append(f"    static constexpr int NNZ_SYM = {len(C)};   // entries (i, j <= k)")
         parts.append(f"    static constexpr int EZ = {2 * n};    // projected-exponential rule: Gauss-Legendre nodes")
         parts.append(f"    static constexpr int EP = {4 * n};    // projected-exponential rule: uniform azimuths")
-        parts.append("#if defined(SHS_NB) && SHS_NB == " + str(n))
-        parts.append(f"    __device__ __forceinline__ static const float* eleg() {{ return kExpLeg{n}; }}")
-        parts.append(f"    __device__ __forceinline__ static const float* etrig() {{ return kExpTrig{n}; }}")
-        parts.append(f"    __device__ __forceinline__ static const float* ew() {{ return kExpW{n}; }}")
-        parts.append("#endif")
+        if n < LANE_PAIR_FROM:
+            parts.append("#if defined(SHS_NB) && SHS_NB == " + str(n))
+            parts.append(f"    __device__ __forceinline__ static const float* eleg() {{ return kExpLeg{n}; }}")
+            parts.append(f"    __device__ __forceinline__ static const float* etrig() {{ return kExpTrig{n}; }}")
+            parts.append(f"    __device__ __forceinline__ static const float* ew() {{ return kExpW{n}; }}")
+            parts.append("#endif")
         parts.append("    __device__ __forceinline__ static float norm(int i) {")
         parts.append("        switch (i) {")
         for i, v in enumerate(N):
@@ -701,38 +736,33 @@ def generate():
         parts.append("        (void)x; (void)y; (void)z; (void)w;")
         parts.append(indent([ln for ln in vjp if not ln.startswith("Y[")]))
         parts.append("    }")
-        na, ng, ml, acc_l, m2f_l, gc_l, ge_l = emit_monomial_route(n)
-        parts.append(f"    static constexpr int NA = {na};   // monomials of degree < n")
-        parts.append(f"    static constexpr int NG = {max(ng, 1)};   // gradient coefficients, bands >= 1")
-        parts.append("    __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {")
-        parts.append("        (void)x; (void)y; (void)z;")
-        parts.append(indent(ml + acc_l))
-        parts.append("    }")
-        parts.append("    // the same for two pairs at once, one per half of each float2")
-        parts.append("    __device__ __forceinline__ static void accumulate2(const float2* G, float2 x, float2 y, float2 z,")
-        parts.append("                                                       float2* acc) {")
-        parts.append("        (void)x; (void)y; (void)z;")
-        parts.append(indent(packed_lines(ml + acc_l)))
-        parts.append("    }")
-        parts.append("    __device__ __forceinline__ static void mono_to_f(const float* acc, float* f) {")
-        parts.append(indent(m2f_l))
-        parts.append("    }")
-        parts.append("    __device__ __forceinline__ static void grad_coeffs(const float* w, float* gq) {")
-        parts.append("        (void)w; (void)gq;")
-        parts.append(indent(gc_l))
-        parts.append("    }")
-        parts.append("    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,")
-        parts.append("                                                     float* gx, float* gy, float* gz) {")
-        parts.append("        (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;")
-        parts.append(indent(ge_l))
-        parts.append("    }")
-        # From 7 bands on the products are tens of thousands of FMAs each:
-        # one out-of-line copy per translation unit instead of one per call
-        # site keeps compile time and the instruction footprint bounded (the
-        # operands of an out-of-line call live in local memory, a few hundred
-        # bytes against ~10^4 FMAs per call; the operands never alias, which
-        # lets every input stay in a register while the outputs are stored).
-        if n < QUAD_FROM:
+        if n < LANE_PAIR_FROM:
+            na, ng, ml, acc_l, m2f_l, gc_l, ge_l = emit_monomial_route(n)
+            parts.append(f"    static constexpr int NA = {na};   // monomials of degree < n")
+            parts.append(f"    static constexpr int NG = {max(ng, 1)};   // gradient coefficients, bands >= 1")
+            parts.append("    __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {")
+            parts.append("        (void)x; (void)y; (void)z;")
+            parts.append(indent(ml + acc_l))
+            parts.append("    }")
+            parts.append("    // the same for two pairs at once, one per half of each float2")
+            parts.append("    __device__ __forceinline__ static void accumulate2(const float2* G, float2 x, float2 y, float2 z,")
+            parts.append("                                                       float2* acc) {")
+            parts.append("        (void)x; (void)y; (void)z;")
+            parts.append(indent(packed_lines(ml + acc_l)))
+            parts.append("    }")
+            parts.append("    __device__ __forceinline__ static void mono_to_f(const float* acc, float* f) {")
+            parts.append(indent(m2f_l))
+            parts.append("    }")
+            parts.append("    __device__ __forceinline__ static void grad_coeffs(const float* w, float* gq) {")
+            parts.append("        (void)w; (void)gq;")
+            parts.append(indent(gc_l))
+            parts.append("    }")
+            parts.append("    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,")
+            parts.append("                                                     float* gx, float* gy, float* gz) {")
+            parts.append("        (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;")
+            parts.append(indent(ge_l))
+            parts.append("    }")
+        if n < LANE_PAIR_FROM:
             parts.append("    __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,")
             parts.append("                                               float* __restrict__ o) {")
             parts.append(indent(mul_l))
@@ -741,18 +771,7 @@ def generate():
             parts.append(indent(sqr_l))
             parts.append("    }")
         else:
-            # The unrolled products would be 10^4 FMAs of straight-line code
-            # each (instruction-fetch bound); these band counts use the
-            # separable quadrature of quadrature_tables() instead.
-            _, nz, npp = emit_quadrature(n)
-            parts.append(f"    static constexpr int QZ = {nz};    // Gauss-Legendre nodes in cos(theta)")
-            parts.append(f"    static constexpr int QP = {npp};    // uniform azimuths")
-            parts.append(f"    static constexpr int QF = {2 * n - 1};    // azimuthal harmonics 1, cos m phi, sin m phi")
-            parts.append("#if defined(SHS_NB) && SHS_NB == " + str(n))
-            parts.append(f"    __device__ __forceinline__ static const float* qleg() {{ return kQuadLeg{n}; }}")
-            parts.append(f"    __device__ __forceinline__ static const float* qtrig() {{ return kQuadTrig{n}; }}")
-            parts.append(f"    __device__ __forceinline__ static const float* qw() {{ return kQuadW{n}; }}")
-            parts.append("#endif")
+            parts.extend(emit_lane_pair(n)[1])
         parts.append("};")
         parts.append("")
     parts.append("}  // namespace shsgen")

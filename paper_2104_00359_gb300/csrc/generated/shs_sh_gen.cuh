@@ -1,7 +1,7 @@
 // Generated by gen_tables.py -- do not edit.
 // Real SH polynomials, their reverse-mode gradients, and the truncated
 // SH triple product (Sec. 3.2, Eq. 3 and Eq. 6-7), unrolled per band count
-// (from 7 bands, quadrature tables for the triple product instead).
+// (from 6 bands, lane-pair quadrature tables for the triple product instead).
 #pragma once
 
 namespace shsgen {
@@ -1331,20 +1331,16 @@ template <> struct SH<5> {
 };
 
 #if defined(SHS_NB) && SHS_NB == 6
-static __constant__ float kExpLeg6[432] = {0.282094806432724f, 0.0933968797326088f, -0.4795929789543152f, 0.0933968797326088f, 0.019960161298513412f, -0.20499086380004883f, 0.5962111353874207f, -0.20499086380004883f, 0.019960161298513412f, 0.004121108911931515f, -0.05183584615588188f, 0.33349815011024475f, -0.66567063331604f, 0.33349815011024475f, -0.05183584615588188f, 0.004121108911931515f, 0.0008355395984835923f, -0.012135355733335018f, 0.09929478168487549f, -0.47001588344573975f, 0.6966167688369751f, -0.47001588344573975f, 0.09929478168487549f, -0.012135355733335018f, 0.0008355395984835923f, 0.0001675097446423024f, -0.002720072865486145f, 0.026212655007839203f, -0.16249744594097137f, 0.6064973473548889f, -0.6931184530258179f, 0.6064973473548889f, -0.16249744594097137f, 0.026212655007839203f, -0.002720072865486145f, 0.0001675097446423024f, 0.282094806432724f, 0.20877224206924438f, -0.44175395369529724f, 0.20877224206924438f, 0.099734365940094f, -0.4220680892467499f, 0.4580381512641907f, -0.4220680892467499f, 0.099734365940094f, 0.04602940008044243f, -0.23857153952121735f, 0.6028831005096436f, -0.3667958080768585f, 0.6028831005096436f, -0.23857153952121735f, 0.04602940008044243f, 0.020860688760876656f, -0.12484792619943619f, 0.40785059332847595f, -0.7035349011421204f, 0.19715876877307892f, -0.7035349011421204f, 0.40785059332847595f, -0.12484792619943619f, 0.020860688760876656f, 0.00934850238263607f, -0.06255322694778442f, 0.2426128387451172f, -0.5745615363121033f, 0.694404661655426f, 0.013120017945766449f, 0.694404661655426f, -0.5745615363121033f, 0.2426128387451172f, -0.06255322694778442f, 0.00934850238263607f, 0.282094806432724f, 0.31180721521377563f, -0.3761763870716095f, 0.31180721521377563f, 0.22247010469436646f, -0.5367931723594666f, 0.2454536110162735f, -0.5367931723594666f, 0.22247010469436646f, 0.15334708988666534f, -0.4531651437282562f, 0.5727651119232178f, 0.010414783842861652f, 0.5727651119232178f, -0.4531651437282562f, 0.15334708988666534f, 0.10379639267921448f, -0.35418701171875f, 0.6067496538162231f, -0.37777870893478394f, -0.2628938853740692f, -0.37777870893478394f, 0.6067496538162231f, -0.35418701171875f, 0.10379639267921448f, 0.06947188824415207f, -0.2650418281555176f, 0.5511578917503357f, -0.5848469138145447f, 0.02309684082865715f, 0.3923318088054657f, 0.02309684082865715f, -0.5848469138145447f, 0.5511578917503357f, -0.2650418281555176f, 0.06947188824415207f, 0.282094806432724f, 0.3954535126686096f, -0.2869650423526764f, 0.3954535126686096f, 0.3578410744667053f, -0.5193423628807068f, 0.010984186083078384f, -0.5193423628807068f, 0.3578410744667053f, 0.31282636523246765f, -0.5560482740402222f, 0.2680802643299103f, 0.27950891852378845f, 0.2680802643299103f, -0.5560482740402222f, 0.31282636523246765f, 0.2685464322566986f, -0.5511856079101562f, 0.43838274478912354f, 0.1861763745546341f, -0.3367987275123596f, 0.1861763745546341f, 0.43838274478912354f, -0.5511856079101562f, 0.2685464322566986f, 0.2279583215713501f, -0.5231051445007324f, 0.5458644032478333f, -0.032114166766405106f, -0.4877561032772064f, 0.11332645267248154f, -0.4877561032772064f, -0.032114166766405106f, 0.5458644032478333f, -0.5231051445007324f, 0.2279583215713501f, 0.282094806432724f, 0.45434778928756714f, -0.17972339689731598f, 0.45434778928756714f, 0.47236329317092896f, -0.3736993372440338f, -0.18737411499023438f, -0.3736993372440338f, 0.47236329317092896f, 0.4744410812854767f, -0.4596995711326599f, -0.13748858869075775f, 0.3189375698566437f, -0.13748858869075775f, -0.4596995711326599f, 0.4744410812854767f, 0.46794116497039795f, -0.523543119430542f, -0.021640226244926453f, 0.4697921574115753f, -0.044248729944229126f, 0.4697921574115753f, -0.021640226244926453f, -0.523543119430542f, 0.46794116497039795f, 0.4563734233379364f, -0.5708690881729126f, 0.08564011752605438f, 0.4528975486755371f, -0.21471181511878967f, -0.28745853900909424f, -0.21471181511878967f, 0.4528975486755371f, 0.08564011752605438f, -0.5708690881729126f, 0.4563734233379364f, 0.282094806432724f, 0.48475590348243713f, -0.061189357191324234f, 0.48475590348243713f, 0.5377067923545837f, -0.13574638962745667f, -0.3005523085594177f, -0.13574638962745667f, 0.5377067923545837f, 0.5762172937393188f, -0.1781618595123291f, -0.4178895950317383f, 0.13653768599033356f, -0.4178895950317383f, -0.1781618595123291f, 0.5762172937393188f, 0.6063591837882996f, -0.21648497879505157f, -0.414544939994812f, 0.24025601148605347f, 0.26849499344825745f, 0.24025601148605347f, -0.414544939994812f, -0.21648497879505157f, 0.6063591837882996f, 0.6309481859207153f, -0.2518526315689087f, -0.4103360176086426f, 0.2815471291542053f, 0.3530324697494507f, -0.2038392275571823f, 0.3530324697494507f, 0.2815471291542053f, -0.4103360176086426f, -0.2518526315689087f, 0.6309481859207153f, 0.282094806432724f, 0.48475590348243713f, 0.061189357191324234f, 0.48475590348243713f, 0.5377067923545837f, 0.13574638962745667f, -0.3005523085594177f, 0.13574638962745667f, 0.5377067923545837f, 0.5762172937393188f, 0.1781618595123291f, -0.4178895950317383f, -0.13653768599033356f, -0.4178895950317383f, 0.1781618595123291f, 0.5762172937393188f, 0.6063591837882996f, 0.21648497879505157f, -0.414544939994812f, -0.24025601148605347f, 0.26849499344825745f, -0.24025601148605347f, -0.414544939994812f, 0.21648497879505157f, 0.6063591837882996f, 0.6309481859207153f, 0.2518526315689087f, -0.4103360176086426f, -0.2815471291542053f, 0.3530324697494507f, 0.2038392275571823f, 0.3530324697494507f, -0.2815471291542053f, -0.4103360176086426f, 0.2518526315689087f, 0.6309481859207153f, 0.282094806432724f, 0.45434778928756714f, 0.17972339689731598f, 0.45434778928756714f, 0.47236329317092896f, 0.3736993372440338f, -0.18737411499023438f, 0.3736993372440338f, 0.47236329317092896f, 0.4744410812854767f, 0.4596995711326599f, -0.13748858869075775f, -0.3189375698566437f, -0.13748858869075775f, 0.4596995711326599f, 0.4744410812854767f, 0.46794116497039795f, 0.523543119430542f, -0.021640226244926453f, -0.4697921574115753f, -0.044248729944229126f, -0.4697921574115753f, -0.021640226244926453f, 0.523543119430542f, 0.46794116497039795f, 0.4563734233379364f, 0.5708690881729126f, 0.08564011752605438f, -0.4528975486755371f, -0.21471181511878967f, 0.28745853900909424f, -0.21471181511878967f, -0.4528975486755371f, 0.08564011752605438f, 0.5708690881729126f, 0.4563734233379364f, 0.282094806432724f, 0.3954535126686096f, 0.2869650423526764f, 0.3954535126686096f, 0.3578410744667053f, 0.5193423628807068f, 0.010984186083078384f, 0.5193423628807068f, 0.3578410744667053f, 0.31282636523246765f, 0.5560482740402222f, 0.2680802643299103f, -0.27950891852378845f, 0.2680802643299103f, 0.5560482740402222f, 0.31282636523246765f, 0.2685464322566986f, 0.5511856079101562f, 0.43838274478912354f, -0.1861763745546341f, -0.3367987275123596f, -0.1861763745546341f, 0.43838274478912354f, 0.5511856079101562f, 0.2685464322566986f, 0.2279583215713501f, 0.5231051445007324f, 0.5458644032478333f, 0.032114166766405106f, -0.4877561032772064f, -0.11332645267248154f, -0.4877561032772064f, 0.032114166766405106f, 0.5458644032478333f, 0.5231051445007324f, 0.2279583215713501f, 0.282094806432724f, 0.31180721521377563f, 0.3761763870716095f, 0.31180721521377563f, 0.22247010469436646f, 0.5367931723594666f, 0.2454536110162735f, 0.5367931723594666f, 0.22247010469436646f, 0.15334708988666534f, 0.4531651437282562f, 0.5727651119232178f, -0.010414783842861652f, 0.5727651119232178f, 0.4531651437282562f, 0.15334708988666534f, 0.10379639267921448f, 0.35418701171875f, 0.6067496538162231f, 0.37777870893478394f, -0.2628938853740692f, 0.37777870893478394f, 0.6067496538162231f, 0.35418701171875f, 0.10379639267921448f, 0.06947188824415207f, 0.2650418281555176f, 0.5511578917503357f, 0.5848469138145447f, 0.02309684082865715f, -0.3923318088054657f, 0.02309684082865715f, 0.5848469138145447f, 0.5511578917503357f, 0.2650418281555176f, 0.06947188824415207f, 0.282094806432724f, 0.20877224206924438f, 0.44175395369529724f, 0.20877224206924438f, 0.099734365940094f, 0.4220680892467499f, 0.4580381512641907f, 0.4220680892467499f, 0.099734365940094f, 0.04602940008044243f, 0.23857153952121735f, 0.6028831005096436f, 0.3667958080768585f, 0.6028831005096436f, 0.23857153952121735f, 0.04602940008044243f, 0.020860688760876656f, 0.12484792619943619f, 0.40785059332847595f, 0.7035349011421204f, 0.19715876877307892f, 0.7035349011421204f, 0.40785059332847595f, 0.12484792619943619f, 0.020860688760876656f, 0.00934850238263607f, 0.06255322694778442f, 0.2426128387451172f, 0.5745615363121033f, 0.694404661655426f, -0.013120017945766449f, 0.694404661655426f, 0.5745615363121033f, 0.2426128387451172f, 0.06255322694778442f, 0.00934850238263607f, 0.282094806432724f, 0.0933968797326088f, 0.4795929789543152f, 0.0933968797326088f, 0.019960161298513412f, 0.20499086380004883f, 0.5962111353874207f, 0.20499086380004883f, 0.019960161298513412f, 0.004121108911931515f, 0.05183584615588188f, 0.33349815011024475f, 0.66567063331604f, 0.33349815011024475f, 0.05183584615588188f, 0.004121108911931515f, 0.0008355395984835923f, 0.012135355733335018f, 0.09929478168487549f, 0.47001588344573975f, 0.6966167688369751f, 0.47001588344573975f, 0.09929478168487549f, 0.012135355733335018f, 0.0008355395984835923f, 0.0001675097446423024f, 0.002720072865486145f, 0.026212655007839203f, 0.16249744594097137f, 0.6064973473548889f, 0.6931184530258179f, 0.6064973473548889f, 0.16249744594097137f, 0.026212655007839203f, 0.002720072865486145f, 0.0001675097446423024f};
-static __constant__ float kExpTrig6[264] = {1.0f, 0.9914448857307434f, 0.13052618503570557f, 0.9659258127212524f, 0.258819043636322f, 0.9238795042037964f, 0.3826834261417389f, 0.8660253882408142f, 0.5f, 0.7933533191680908f, 0.6087614297866821f, 1.0f, 0.9238795042037964f, 0.3826834261417389f, 0.7071067690849304f, 0.7071067690849304f, 0.3826834261417389f, 0.9238795042037964f, 6.123234262925839e-17f, 1.0f, -0.3826834261417389f, 0.9238795042037964f, 1.0f, 0.7933533191680908f, 0.6087614297866821f, 0.258819043636322f, 0.9659258127212524f, -0.3826834261417389f, 0.9238795042037964f, -0.8660253882408142f, 0.5f, -0.9914448857307434f, -0.13052618503570557f, 1.0f, 0.6087614297866821f, 0.7933533191680908f, -0.258819043636322f, 0.9659258127212524f, -0.9238795042037964f, 0.3826834261417389f, -0.8660253882408142f, -0.5f, -0.13052618503570557f, -0.9914448857307434f, 1.0f, 0.3826834261417389f, 0.9238795042037964f, -0.7071067690849304f, 0.7071067690849304f, -0.9238795042037964f, -0.3826834261417389f, -1.8369701465288538e-16f, -1.0f, 0.9238795042037964f, -0.3826834261417389f, 1.0f, 0.13052618503570557f, 0.9914448857307434f, -0.9659258127212524f, 0.258819043636322f, -0.3826834261417389f, -0.9238795042037964f, 0.8660253882408142f, -0.5f, 0.6087614297866821f, 0.7933533191680908f, 1.0f, -0.13052618503570557f, 0.9914448857307434f, -0.9659258127212524f, -0.258819043636322f, 0.3826834261417389f, -0.9238795042037964f, 0.8660253882408142f, 0.5f, -0.6087614297866821f, 0.7933533191680908f, 1.0f, -0.3826834261417389f, 0.9238795042037964f, -0.7071067690849304f, -0.7071067690849304f, 0.9238795042037964f, -0.3826834261417389f, 1.1943400666719682e-15f, 1.0f, -0.9238795042037964f, -0.3826834261417389f, 1.0f, -0.6087614297866821f, 0.7933533191680908f, -0.258819043636322f, -0.9659258127212524f, 0.9238795042037964f, 0.3826834261417389f, -0.8660253882408142f, 0.5f, 0.13052618503570557f, -0.9914448857307434f, 1.0f, -0.7933533191680908f, 0.6087614297866821f, 0.258819043636322f, -0.9659258127212524f, 0.3826834261417389f, 0.9238795042037964f, -0.8660253882408142f, -0.5f, 0.9914448857307434f, -0.13052618503570557f, 1.0f, -0.9238795042037964f, 0.3826834261417389f, 0.7071067690849304f, -0.7071067690849304f, -0.3826834261417389f, 0.9238795042037964f, -4.2862638516991895e-16f, -1.0f, 0.3826834261417389f, 0.9238795042037964f, 1.0f, -0.9914448857307434f, 0.13052618503570557f, 0.9659258127212524f, -0.258819043636322f, -0.9238795042037964f, 0.3826834261417389f, 0.8660253882408142f, -0.5f, -0.7933533191680908f, 0.6087614297866821f, 1.0f, -0.9914448857307434f, -0.13052618503570557f, 0.9659258127212524f, 0.258819043636322f, -0.9238795042037964f, -0.3826834261417389f, 0.8660253882408142f, 0.5f, -0.7933533191680908f, -0.6087614297866821f, 1.0f, -0.9238795042037964f, -0.3826834261417389f, 0.7071067690849304f, 0.7071067690849304f, -0.3826834261417389f, -0.9238795042037964f, 5.510910704284357e-16f, 1.0f, 0.3826834261417389f, -0.9238795042037964f, 1.0f, -0.7933533191680908f, -0.6087614297866821f, 0.258819043636322f, 0.9659258127212524f, 0.3826834261417389f, -0.9238795042037964f, -0.8660253882408142f, 0.5f, 0.9914448857307434f, 0.13052618503570557f, 1.0f, -0.6087614297866821f, -0.7933533191680908f, -0.258819043636322f, 0.9659258127212524f, 0.9238795042037964f, -0.3826834261417389f, -0.8660253882408142f, -0.5f, 0.13052618503570557f, 0.9914448857307434f, 1.0f, -0.3826834261417389f, -0.9238795042037964f, -0.7071067690849304f, 0.7071067690849304f, 0.9238795042037964f, 0.3826834261417389f, 1.1028011101830775e-15f, -1.0f, -0.9238795042037964f, 0.3826834261417389f, 1.0f, -0.13052618503570557f, -0.9914448857307434f, -0.9659258127212524f, 0.258819043636322f, 0.3826834261417389f, 0.9238795042037964f, 0.8660253882408142f, -0.5f, -0.6087614297866821f, -0.7933533191680908f, 1.0f, 0.13052618503570557f, -0.9914448857307434f, -0.9659258127212524f, -0.258819043636322f, -0.3826834261417389f, 0.9238795042037964f, 0.8660253882408142f, 0.5f, 0.6087614297866821f, -0.7933533191680908f, 1.0f, 0.3826834261417389f, -0.9238795042037964f, -0.7071067690849304f, -0.7071067690849304f, -0.9238795042037964f, 0.3826834261417389f, 2.5723772274061606e-15f, 1.0f, 0.9238795042037964f, 0.3826834261417389f, 1.0f, 0.6087614297866821f, -0.7933533191680908f, -0.258819043636322f, -0.9659258127212524f, -0.9238795042037964f, -0.3826834261417389f, -0.8660253882408142f, 0.5f, -0.13052618503570557f, 0.9914448857307434f, 1.0f, 0.7933533191680908f, -0.6087614297866821f, 0.258819043636322f, -0.9659258127212524f, -0.3826834261417389f, -0.9238795042037964f, -0.8660253882408142f, -0.5f, -0.9914448857307434f, 0.13052618503570557f, 1.0f, 0.9238795042037964f, -0.3826834261417389f, 0.7071067690849304f, -0.7071067690849304f, 0.3826834261417389f, -0.9238795042037964f, 8.57871739666044e-16f, -1.0f, -0.3826834261417389f, -0.9238795042037964f, 1.0f, 0.9914448857307434f, -0.13052618503570557f, 0.9659258127212524f, -0.258819043636322f, 0.9238795042037964f, -0.3826834261417389f, 0.8660253882408142f, -0.5f, 0.7933533191680908f, -0.6087614297866821f};
-static __constant__ float kExpW6[12] = {0.01235047448426485f, 0.027996649965643883f, 0.04190840944647789f, 0.05318910628557205f, 0.06112820282578468f, 0.06522654742002487f, 0.06522654742002487f, 0.06112820282578468f, 0.05318910628557205f, 0.04190840944647789f, 0.027996649965643883f, 0.01235047448426485f};
+// lane-pair rules: product, then projected exponential (plain, weighted)
+static __device__ const float kLpLeg6[96] = {0.09627555310726166f, 0.19014164805412292f, 0.18406742811203003f, 0.04652512073516846f, 0.15714223682880402f, 0.25652122497558594f, 0.014512873254716396f, 0.06856247037649155f, 0.004373585805296898f, 0.026470474898815155f, 0.0012942698085680604f, 0.00037873201654292643f, 0.16013231873512268f, 0.19700372219085693f, 0.15417835116386414f, 0.09990215301513672f, 0.21137355268001556f, 0.0f, 0.036872684955596924f, 0.1080133244395256f, 0.012599730864167213f, 0.0f, 0.004122147336602211f, 0.0f, 0.12515482306480408f, 0.12649886310100555f, -0.09113376587629318f, 0.13102267682552338f, 0.2663714289665222f, 0.06967514008283615f, 0.08854003250598907f, 0.2639823257923126f, 0.05780312418937683f, 0.22584053874015808f, 0.03705662116408348f, 0.023490939289331436f, 0.17269699275493622f, 0.022869709879159927f, -0.16741353273391724f, 0.23340384662151337f, 0.20621128380298615f, 0.0f, 0.18662303686141968f, 0.279779314994812f, 0.1381494402885437f, 0.0f, 0.09791262447834015f, 0.0f, 0.1403641700744629f, -0.026905516162514687f, -0.1376871019601822f, 0.20683826506137848f, 0.07370050996541977f, -0.2425079345703125f, 0.19674327969551086f, 0.1590183526277542f, 0.180795356631279f, 0.22271154820919037f, 0.16314642131328583f, 0.1455753594636917f, 0.12776632606983185f, -0.15799476206302643f, 0.014452863484621048f, 0.24306106567382812f, -0.1587732434272766f, 0.0f, 0.2735573649406433f, -0.07777585834264755f, 0.2850414514541626f, 0.0f, 0.2843632102012634f, 0.0f, 0.14731866121292114f, -0.14808091521263123f, 0.1121562197804451f, 0.25083374977111816f, -0.1951584368944168f, 0.1285189688205719f, 0.27568212151527405f, -0.18251359462738037f, 0.2927181124687195f, -0.16920839250087738f, 0.305206298828125f, 0.31467151641845703f, 0.04680580645799637f, -0.10123119503259659f, 0.142460435628891f, 0.10288506746292114f, -0.17417211830615997f, 0.0f, 0.13379472494125366f, -0.1994764804840088f, 0.16108393669128418f, 0.0f, 0.18568259477615356f, 0.0f};
+static __device__ const float kLeLeg6[288] = {0.282094806432724f, 0.5962111353874207f, 0.6966167688369751f, 0.0933968797326088f, 0.33349815011024475f, 0.6064973473548889f, 0.019960161298513412f, 0.09929478168487549f, 0.004121108911931515f, 0.026212655007839203f, 0.0008355395984835923f, 0.0001675097446423024f, 0.4795929789543152f, 0.66567063331604f, 0.6931184530258179f, 0.20499086380004883f, 0.47001588344573975f, 0.0f, 0.05183584615588188f, 0.16249744594097137f, 0.012135355733335018f, 0.0f, 0.002720072865486145f, 0.0f, 0.282094806432724f, 0.4580381512641907f, 0.19715876877307892f, 0.20877224206924438f, 0.6028831005096436f, 0.694404661655426f, 0.099734365940094f, 0.40785059332847595f, 0.04602940008044243f, 0.2426128387451172f, 0.020860688760876656f, 0.00934850238263607f, 0.44175395369529724f, 0.3667958080768585f, -0.013120017945766449f, 0.4220680892467499f, 0.7035349011421204f, 0.0f, 0.23857153952121735f, 0.5745615363121033f, 0.12484792619943619f, 0.0f, 0.06255322694778442f, 0.0f, 0.282094806432724f, 0.2454536110162735f, -0.2628938853740692f, 0.31180721521377563f, 0.5727651119232178f, 0.02309684082865715f, 0.22247010469436646f, 0.6067496538162231f, 0.15334708988666534f, 0.5511578917503357f, 0.10379639267921448f, 0.06947188824415207f, 0.3761763870716095f, -0.010414783842861652f, -0.3923318088054657f, 0.5367931723594666f, 0.37777870893478394f, 0.0f, 0.4531651437282562f, 0.5848469138145447f, 0.35418701171875f, 0.0f, 0.2650418281555176f, 0.0f, 0.282094806432724f, 0.010984186083078384f, -0.3367987275123596f, 0.3954535126686096f, 0.2680802643299103f, -0.4877561032772064f, 0.3578410744667053f, 0.43838274478912354f, 0.31282636523246765f, 0.5458644032478333f, 0.2685464322566986f, 0.2279583215713501f, 0.2869650423526764f, -0.27950891852378845f, -0.11332645267248154f, 0.5193423628807068f, -0.1861763745546341f, 0.0f, 0.5560482740402222f, 0.032114166766405106f, 0.5511856079101562f, 0.0f, 0.5231051445007324f, 0.0f, 0.282094806432724f, -0.18737411499023438f, -0.044248729944229126f, 0.45434778928756714f, -0.13748858869075775f, -0.21471181511878967f, 0.47236329317092896f, -0.021640226244926453f, 0.4744410812854767f, 0.08564011752605438f, 0.46794116497039795f, 0.4563734233379364f, 0.17972339689731598f, -0.3189375698566437f, 0.28745853900909424f, 0.3736993372440338f, -0.4697921574115753f, 0.0f, 0.4596995711326599f, -0.4528975486755371f, 0.523543119430542f, 0.0f, 0.5708690881729126f, 0.0f, 0.282094806432724f, -0.3005523085594177f, 0.26849499344825745f, 0.48475590348243713f, -0.4178895950317383f, 0.3530324697494507f, 0.5377067923545837f, -0.414544939994812f, 0.5762172937393188f, -0.4103360176086426f, 0.6063591837882996f, 0.6309481859207153f, 0.061189357191324234f, -0.13653768599033356f, 0.2038392275571823f, 0.13574638962745667f, -0.24025601148605347f, 0.0f, 0.1781618595123291f, -0.2815471291542053f, 0.21648497879505157f, 0.0f, 0.2518526315689087f, 0.0f, 0.003484004409983754f, 0.007363489829003811f, 0.008603546768426895f, 0.0011534957448020577f, 0.004118860233575106f, 0.007490530144423246f, 0.00024651744752191007f, 0.0012263376265764236f, 5.08976518176496e-05f, 0.000323738728184253f, 1.0319310604245402e-05f, 2.068824642265099e-06f, 0.005923200864344835f, 0.008221347816288471f, 0.008560341782867908f, 0.0025317342951893806f, 0.005804919172078371f, 0.0f, 0.0006401973078027368f, 0.0020069205202162266f, 0.00014987739268690348f, 0.0f, 3.3594187698327005e-05f, 0.0f, 0.007897709496319294f, 0.01282353326678276f, 0.005519785452634096f, 0.005844923667609692f, 0.016878707334399223f, 0.01944100484251976f, 0.0027922282461076975f, 0.011418450623750687f, 0.0012886689510196447f, 0.006792346481233835f, 0.00058402941795066f, 0.0002617267600726336f, 0.012367631308734417f, 0.010269053280353546f, -0.00036731656291522086f, 0.011816493235528469f, 0.019696621224284172f, 0.0f, 0.006679203826934099f, 0.016085797920823097f, 0.0034953237045556307f, 0.0f, 0.0017512808553874493f, 0.0f, 0.011822143569588661f, 0.010286569595336914f, -0.011017464101314545f, 0.013067344203591347f, 0.02400367334485054f, 0.0009679518989287317f, 0.009323367848992348f, 0.025427913293242455f, 0.006426532287150621f, 0.02309815213084221f, 0.004349941853433847f, 0.002911456162109971f, 0.015764953568577766f, -0.0004364670312497765f, -0.01644200086593628f, 0.022496148943901062f, 0.01583210565149784f, 0.0f, 0.01899143122136593f, 0.024510003626346588f, 0.014843413606286049f, 0.0f, 0.011107482016086578f, 0.0f, 0.015004370361566544f, 0.0005842390237376094f, -0.017914025112986565f, 0.021033819764852524f, 0.01425895094871521f, -0.025943312793970108f, 0.019033247604966164f, 0.023317188024520874f, 0.01663895510137081f, 0.029034042730927467f, 0.014283744618296623f, 0.01212489977478981f, 0.01526341401040554f, -0.014866829849779606f, -0.006027732975780964f, 0.027623355388641357f, -0.009902555495500565f, 0.0f, 0.029575711116194725f, 0.0017081238329410553f, 0.02931707166135311f, 0.0f, 0.027823494747281075f, 0.0f, 0.017243947833776474f, -0.011453842744231224f, -0.0027048452757298946f, 0.02777346409857273f, -0.008404430001974106f, -0.013124947436153889f, 0.028874719515442848f, -0.001322828116826713f, 0.02900172956287861f, 0.005235026590526104f, 0.028604403138160706f, 0.027897287160158157f, 0.010986167937517166f, -0.01949607953429222f, 0.01757182367146015f, 0.02284356951713562f, -0.02871754951775074f, 0.0f, 0.02810060791671276f, -0.027684813365340233f, 0.0320032499730587f, 0.0f, 0.03489620238542557f, 0.0f, 0.01840006746351719f, -0.019603990018367767f, 0.017513001337647438f, 0.03161895275115967f, -0.027257494628429413f, 0.0230270866304636f, 0.03507275506854057f, -0.027039334177970886f, 0.037584662437438965f, -0.026764800772070885f, 0.03955071419477463f, 0.04115457087755203f, 0.003991170320659876f, -0.008905881084501743f, 0.013295728713274002f, 0.008854268118739128f, -0.01567106880247593f, 0.0f, 0.011620881967246532f, -0.018364345654845238f, 0.01412056665867567f, 0.0f, 0.016427477821707726f, 0.0f};
+static __constant__ float kLpTrig6[44] = {1.0f, 0.9807852506637573f, 0.19509032368659973f, 0.9238795042037964f, 0.3826834261417389f, 0.8314695954322815f, 0.5555702447891235f, 0.7071067690849304f, 0.7071067690849304f, 0.5555702447891235f, 0.8314695954322815f, 1.0f, 0.8314695954322815f, 0.5555702447891235f, 0.3826834261417389f, 0.9238795042037964f, -0.19509032368659973f, 0.9807852506637573f, -0.7071067690849304f, 0.7071067690849304f, -0.9807852506637573f, 0.19509032368659973f, 1.0f, 0.5555702447891235f, 0.8314695954322815f, -0.3826834261417389f, 0.9238795042037964f, -0.9807852506637573f, 0.19509032368659973f, -0.7071067690849304f, -0.7071067690849304f, 0.19509032368659973f, -0.9807852506637573f, 1.0f, 0.19509032368659973f, 0.9807852506637573f, -0.9238795042037964f, 0.3826834261417389f, -0.5555702447891235f, -0.8314695954322815f, 0.7071067690849304f, -0.7071067690849304f, 0.8314695954322815f, 0.5555702447891235f};
 #endif
 template <> struct SH<6> {
     static constexpr int K = 36;
     static constexpr int NNZ_SYM = 1517;   // entries (i, j <= k)
     static constexpr int EZ = 12;    // projected-exponential rule: Gauss-Legendre nodes
     static constexpr int EP = 24;    // projected-exponential rule: uniform azimuths
-#if defined(SHS_NB) && SHS_NB == 6
-    __device__ __forceinline__ static const float* eleg() { return kExpLeg6; }
-    __device__ __forceinline__ static const float* etrig() { return kExpTrig6; }
-    __device__ __forceinline__ static const float* ew() { return kExpW6; }
-#endif
     __device__ __forceinline__ static float norm(int i) {
         switch (i) {
             case 0: return 0.282094806432724f;
@@ -1728,500 +1724,138 @@ template <> struct SH<6> {
         gy = w[1] + t50 * a_t86 + t46 * a_t78 + t42 * a_t72 + t39 * a_t68 + t14 * a_t22 + t17 * a_t19 + t8 * a_t16 + t11 * a_t13 + t2 * a_t10 + t5 * a_t7 + x * a_t4 + x * a_t3 + y * a_t1 + y * a_t1;
         gz = w[2] + 105.0f * a_t65 + t61 * a_t62 + 15.0f * a_t60 + t55 * a_t56 + t52 * a_t53 + 3.0f * a_t51 + t46 * a_t47 + t42 * a_t43 + t39 * a_t40 + 3.0f * a_t39 + t34 * a_t35 + t30 * a_t31 + 0.6666666865348816f * a_t29 + t26 * a_t27 + z * a_t24 + z * a_t24;
     }
-    static constexpr int NA = 56;   // monomials of degree < n
-    static constexpr int NG = 105;   // gradient coefficients, bands >= 1
-    __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
-        (void)x; (void)y; (void)z;
-        const float m1_0_0 = x;
-        const float m0_1_0 = y;
-        const float m0_0_1 = z;
-        const float m2_0_0 = x * m1_0_0;
-        const float m1_1_0 = x * m0_1_0;
-        const float m1_0_1 = x * m0_0_1;
-        const float m0_2_0 = y * m0_1_0;
-        const float m0_1_1 = y * m0_0_1;
-        const float m0_0_2 = z * m0_0_1;
-        const float m3_0_0 = x * m2_0_0;
-        const float m2_1_0 = x * m1_1_0;
-        const float m2_0_1 = x * m1_0_1;
-        const float m1_2_0 = x * m0_2_0;
-        const float m1_1_1 = x * m0_1_1;
-        const float m1_0_2 = x * m0_0_2;
-        const float m0_3_0 = y * m0_2_0;
-        const float m0_2_1 = y * m0_1_1;
-        const float m0_1_2 = y * m0_0_2;
-        const float m0_0_3 = z * m0_0_2;
-        const float m4_0_0 = x * m3_0_0;
-        const float m3_1_0 = x * m2_1_0;
-        const float m3_0_1 = x * m2_0_1;
-        const float m2_2_0 = x * m1_2_0;
-        const float m2_1_1 = x * m1_1_1;
-        const float m2_0_2 = x * m1_0_2;
-        const float m1_3_0 = x * m0_3_0;
-        const float m1_2_1 = x * m0_2_1;
-        const float m1_1_2 = x * m0_1_2;
-        const float m1_0_3 = x * m0_0_3;
-        const float m0_4_0 = y * m0_3_0;
-        const float m0_3_1 = y * m0_2_1;
-        const float m0_2_2 = y * m0_1_2;
-        const float m0_1_3 = y * m0_0_3;
-        const float m0_0_4 = z * m0_0_3;
-        const float gtx = G[5] * x;
-        const float gty = G[5] * y;
-        const float gtz = G[5] * z;
-        acc[0] = fmaf(G[0], 1.0f, acc[0]);
-        acc[1] = fmaf(G[1], m1_0_0, acc[1]);
-        acc[2] = fmaf(G[1], m0_1_0, acc[2]);
-        acc[3] = fmaf(G[1], m0_0_1, acc[3]);
-        acc[4] = fmaf(G[2], m2_0_0, acc[4]);
-        acc[5] = fmaf(G[2], m1_1_0, acc[5]);
-        acc[6] = fmaf(G[2], m1_0_1, acc[6]);
-        acc[7] = fmaf(G[2], m0_2_0, acc[7]);
-        acc[8] = fmaf(G[2], m0_1_1, acc[8]);
-        acc[9] = fmaf(G[2], m0_0_2, acc[9]);
-        acc[10] = fmaf(G[3], m3_0_0, acc[10]);
-        acc[11] = fmaf(G[3], m2_1_0, acc[11]);
-        acc[12] = fmaf(G[3], m2_0_1, acc[12]);
-        acc[13] = fmaf(G[3], m1_2_0, acc[13]);
-        acc[14] = fmaf(G[3], m1_1_1, acc[14]);
-        acc[15] = fmaf(G[3], m1_0_2, acc[15]);
-        acc[16] = fmaf(G[3], m0_3_0, acc[16]);
-        acc[17] = fmaf(G[3], m0_2_1, acc[17]);
-        acc[18] = fmaf(G[3], m0_1_2, acc[18]);
-        acc[19] = fmaf(G[3], m0_0_3, acc[19]);
-        acc[20] = fmaf(G[4], m4_0_0, acc[20]);
-        acc[21] = fmaf(G[4], m3_1_0, acc[21]);
-        acc[22] = fmaf(G[4], m3_0_1, acc[22]);
-        acc[23] = fmaf(G[4], m2_2_0, acc[23]);
-        acc[24] = fmaf(G[4], m2_1_1, acc[24]);
-        acc[25] = fmaf(G[4], m2_0_2, acc[25]);
-        acc[26] = fmaf(G[4], m1_3_0, acc[26]);
-        acc[27] = fmaf(G[4], m1_2_1, acc[27]);
-        acc[28] = fmaf(G[4], m1_1_2, acc[28]);
-        acc[29] = fmaf(G[4], m1_0_3, acc[29]);
-        acc[30] = fmaf(G[4], m0_4_0, acc[30]);
-        acc[31] = fmaf(G[4], m0_3_1, acc[31]);
-        acc[32] = fmaf(G[4], m0_2_2, acc[32]);
-        acc[33] = fmaf(G[4], m0_1_3, acc[33]);
-        acc[34] = fmaf(G[4], m0_0_4, acc[34]);
-        acc[35] = fmaf(gtx, m4_0_0, acc[35]);
-        acc[36] = fmaf(gtx, m3_1_0, acc[36]);
-        acc[37] = fmaf(gtx, m3_0_1, acc[37]);
-        acc[38] = fmaf(gtx, m2_2_0, acc[38]);
-        acc[39] = fmaf(gtx, m2_1_1, acc[39]);
-        acc[40] = fmaf(gtx, m2_0_2, acc[40]);
-        acc[41] = fmaf(gtx, m1_3_0, acc[41]);
-        acc[42] = fmaf(gtx, m1_2_1, acc[42]);
-        acc[43] = fmaf(gtx, m1_1_2, acc[43]);
-        acc[44] = fmaf(gtx, m1_0_3, acc[44]);
-        acc[45] = fmaf(gtx, m0_4_0, acc[45]);
-        acc[46] = fmaf(gtx, m0_3_1, acc[46]);
-        acc[47] = fmaf(gtx, m0_2_2, acc[47]);
-        acc[48] = fmaf(gtx, m0_1_3, acc[48]);
-        acc[49] = fmaf(gtx, m0_0_4, acc[49]);
-        acc[50] = fmaf(gty, m0_4_0, acc[50]);
-        acc[51] = fmaf(gty, m0_3_1, acc[51]);
-        acc[52] = fmaf(gty, m0_2_2, acc[52]);
-        acc[53] = fmaf(gty, m0_1_3, acc[53]);
-        acc[54] = fmaf(gty, m0_0_4, acc[54]);
-        acc[55] = fmaf(gtz, m0_0_4, acc[55]);
+    static constexpr int LPS = 4;   // lane-pair product rule: node pairs
+    static constexpr int LPQ = 4;   // ... and azimuth quads
+    static constexpr int LES = 6;   // lane-pair projected-exponential rule: node pairs
+    static constexpr int LEQ = 6;   // ... and azimuth quads
+#if defined(SHS_NB) && SHS_NB == 6
+    __device__ __forceinline__ static const float* lp_leg() { return kLpLeg6; }
+    __device__ __forceinline__ static const float* le_leg() { return kLeLeg6; }
+    __device__ __forceinline__ static const float* lp_trig_row(int b) { return kLpTrig6 + b * 11; }
+#endif
+    __device__ __forceinline__ static float lp_trig(int b, int h) {   // h = 2m - 1: cos(m phi_b), 2m: sin
+        switch (b * 11 + h) {
+            case 1: return 0.9807852506637573f;
+            case 2: return 0.19509032368659973f;
+            case 3: return 0.9238795042037964f;
+            case 4: return 0.3826834261417389f;
+            case 5: return 0.8314695954322815f;
+            case 6: return 0.5555702447891235f;
+            case 7: return 0.7071067690849304f;
+            case 8: return 0.7071067690849304f;
+            case 9: return 0.5555702447891235f;
+            case 10: return 0.8314695954322815f;
+            case 12: return 0.8314695954322815f;
+            case 13: return 0.5555702447891235f;
+            case 14: return 0.3826834261417389f;
+            case 15: return 0.9238795042037964f;
+            case 16: return -0.19509032368659973f;
+            case 17: return 0.9807852506637573f;
+            case 18: return -0.7071067690849304f;
+            case 19: return 0.7071067690849304f;
+            case 20: return -0.9807852506637573f;
+            case 21: return 0.19509032368659973f;
+            case 23: return 0.5555702447891235f;
+            case 24: return 0.8314695954322815f;
+            case 25: return -0.3826834261417389f;
+            case 26: return 0.9238795042037964f;
+            case 27: return -0.9807852506637573f;
+            case 28: return 0.19509032368659973f;
+            case 29: return -0.7071067690849304f;
+            case 30: return -0.7071067690849304f;
+            case 31: return 0.19509032368659973f;
+            case 32: return -0.9807852506637573f;
+            case 34: return 0.19509032368659973f;
+            case 35: return 0.9807852506637573f;
+            case 36: return -0.9238795042037964f;
+            case 37: return 0.3826834261417389f;
+            case 38: return -0.5555702447891235f;
+            case 39: return -0.8314695954322815f;
+            case 40: return 0.7071067690849304f;
+            case 41: return -0.7071067690849304f;
+            case 42: return 0.8314695954322815f;
+            case 43: return 0.5555702447891235f;
+            default: return 1.0f;
+        }
     }
-    // the same for two pairs at once, one per half of each float2
-    __device__ __forceinline__ static void accumulate2(const float2* G, float2 x, float2 y, float2 z,
-                                                       float2* acc) {
-        (void)x; (void)y; (void)z;
-        const float2 m1_0_0 = x;
-        const float2 m0_1_0 = y;
-        const float2 m0_0_1 = z;
-        const float2 m2_0_0 = __fmul2_rn(x, m1_0_0);
-        const float2 m1_1_0 = __fmul2_rn(x, m0_1_0);
-        const float2 m1_0_1 = __fmul2_rn(x, m0_0_1);
-        const float2 m0_2_0 = __fmul2_rn(y, m0_1_0);
-        const float2 m0_1_1 = __fmul2_rn(y, m0_0_1);
-        const float2 m0_0_2 = __fmul2_rn(z, m0_0_1);
-        const float2 m3_0_0 = __fmul2_rn(x, m2_0_0);
-        const float2 m2_1_0 = __fmul2_rn(x, m1_1_0);
-        const float2 m2_0_1 = __fmul2_rn(x, m1_0_1);
-        const float2 m1_2_0 = __fmul2_rn(x, m0_2_0);
-        const float2 m1_1_1 = __fmul2_rn(x, m0_1_1);
-        const float2 m1_0_2 = __fmul2_rn(x, m0_0_2);
-        const float2 m0_3_0 = __fmul2_rn(y, m0_2_0);
-        const float2 m0_2_1 = __fmul2_rn(y, m0_1_1);
-        const float2 m0_1_2 = __fmul2_rn(y, m0_0_2);
-        const float2 m0_0_3 = __fmul2_rn(z, m0_0_2);
-        const float2 m4_0_0 = __fmul2_rn(x, m3_0_0);
-        const float2 m3_1_0 = __fmul2_rn(x, m2_1_0);
-        const float2 m3_0_1 = __fmul2_rn(x, m2_0_1);
-        const float2 m2_2_0 = __fmul2_rn(x, m1_2_0);
-        const float2 m2_1_1 = __fmul2_rn(x, m1_1_1);
-        const float2 m2_0_2 = __fmul2_rn(x, m1_0_2);
-        const float2 m1_3_0 = __fmul2_rn(x, m0_3_0);
-        const float2 m1_2_1 = __fmul2_rn(x, m0_2_1);
-        const float2 m1_1_2 = __fmul2_rn(x, m0_1_2);
-        const float2 m1_0_3 = __fmul2_rn(x, m0_0_3);
-        const float2 m0_4_0 = __fmul2_rn(y, m0_3_0);
-        const float2 m0_3_1 = __fmul2_rn(y, m0_2_1);
-        const float2 m0_2_2 = __fmul2_rn(y, m0_1_2);
-        const float2 m0_1_3 = __fmul2_rn(y, m0_0_3);
-        const float2 m0_0_4 = __fmul2_rn(z, m0_0_3);
-        const float2 gtx = __fmul2_rn(G[5], x);
-        const float2 gty = __fmul2_rn(G[5], y);
-        const float2 gtz = __fmul2_rn(G[5], z);
-        acc[0] = __fadd2_rn(G[0], acc[0]);
-        acc[1] = __ffma2_rn(G[1], m1_0_0, acc[1]);
-        acc[2] = __ffma2_rn(G[1], m0_1_0, acc[2]);
-        acc[3] = __ffma2_rn(G[1], m0_0_1, acc[3]);
-        acc[4] = __ffma2_rn(G[2], m2_0_0, acc[4]);
-        acc[5] = __ffma2_rn(G[2], m1_1_0, acc[5]);
-        acc[6] = __ffma2_rn(G[2], m1_0_1, acc[6]);
-        acc[7] = __ffma2_rn(G[2], m0_2_0, acc[7]);
-        acc[8] = __ffma2_rn(G[2], m0_1_1, acc[8]);
-        acc[9] = __ffma2_rn(G[2], m0_0_2, acc[9]);
-        acc[10] = __ffma2_rn(G[3], m3_0_0, acc[10]);
-        acc[11] = __ffma2_rn(G[3], m2_1_0, acc[11]);
-        acc[12] = __ffma2_rn(G[3], m2_0_1, acc[12]);
-        acc[13] = __ffma2_rn(G[3], m1_2_0, acc[13]);
-        acc[14] = __ffma2_rn(G[3], m1_1_1, acc[14]);
-        acc[15] = __ffma2_rn(G[3], m1_0_2, acc[15]);
-        acc[16] = __ffma2_rn(G[3], m0_3_0, acc[16]);
-        acc[17] = __ffma2_rn(G[3], m0_2_1, acc[17]);
-        acc[18] = __ffma2_rn(G[3], m0_1_2, acc[18]);
-        acc[19] = __ffma2_rn(G[3], m0_0_3, acc[19]);
-        acc[20] = __ffma2_rn(G[4], m4_0_0, acc[20]);
-        acc[21] = __ffma2_rn(G[4], m3_1_0, acc[21]);
-        acc[22] = __ffma2_rn(G[4], m3_0_1, acc[22]);
-        acc[23] = __ffma2_rn(G[4], m2_2_0, acc[23]);
-        acc[24] = __ffma2_rn(G[4], m2_1_1, acc[24]);
-        acc[25] = __ffma2_rn(G[4], m2_0_2, acc[25]);
-        acc[26] = __ffma2_rn(G[4], m1_3_0, acc[26]);
-        acc[27] = __ffma2_rn(G[4], m1_2_1, acc[27]);
-        acc[28] = __ffma2_rn(G[4], m1_1_2, acc[28]);
-        acc[29] = __ffma2_rn(G[4], m1_0_3, acc[29]);
-        acc[30] = __ffma2_rn(G[4], m0_4_0, acc[30]);
-        acc[31] = __ffma2_rn(G[4], m0_3_1, acc[31]);
-        acc[32] = __ffma2_rn(G[4], m0_2_2, acc[32]);
-        acc[33] = __ffma2_rn(G[4], m0_1_3, acc[33]);
-        acc[34] = __ffma2_rn(G[4], m0_0_4, acc[34]);
-        acc[35] = __ffma2_rn(gtx, m4_0_0, acc[35]);
-        acc[36] = __ffma2_rn(gtx, m3_1_0, acc[36]);
-        acc[37] = __ffma2_rn(gtx, m3_0_1, acc[37]);
-        acc[38] = __ffma2_rn(gtx, m2_2_0, acc[38]);
-        acc[39] = __ffma2_rn(gtx, m2_1_1, acc[39]);
-        acc[40] = __ffma2_rn(gtx, m2_0_2, acc[40]);
-        acc[41] = __ffma2_rn(gtx, m1_3_0, acc[41]);
-        acc[42] = __ffma2_rn(gtx, m1_2_1, acc[42]);
-        acc[43] = __ffma2_rn(gtx, m1_1_2, acc[43]);
-        acc[44] = __ffma2_rn(gtx, m1_0_3, acc[44]);
-        acc[45] = __ffma2_rn(gtx, m0_4_0, acc[45]);
-        acc[46] = __ffma2_rn(gtx, m0_3_1, acc[46]);
-        acc[47] = __ffma2_rn(gtx, m0_2_2, acc[47]);
-        acc[48] = __ffma2_rn(gtx, m0_1_3, acc[48]);
-        acc[49] = __ffma2_rn(gtx, m0_0_4, acc[49]);
-        acc[50] = __ffma2_rn(gty, m0_4_0, acc[50]);
-        acc[51] = __ffma2_rn(gty, m0_3_1, acc[51]);
-        acc[52] = __ffma2_rn(gty, m0_2_2, acc[52]);
-        acc[53] = __ffma2_rn(gty, m0_1_3, acc[53]);
-        acc[54] = __ffma2_rn(gty, m0_0_4, acc[54]);
-        acc[55] = __ffma2_rn(gtz, m0_0_4, acc[55]);
-    }
-    __device__ __forceinline__ static void mono_to_f(const float* acc, float* f) {
-        f[0] = 1.0f * acc[0];
-        f[1] = 1.0f * acc[2];
-        f[2] = 1.0f * acc[3];
-        f[3] = 1.0f * acc[1];
-        f[4] = 6.0f * acc[5];
-        f[5] = 3.0f * acc[8];
-        f[6] = ((1.0f * acc[9] + -0.5f * acc[7]) + -0.5f * acc[4]);
-        f[7] = 3.0f * acc[6];
-        f[8] = (-3.0f * acc[7] + 3.0f * acc[4]);
-        f[9] = (-15.0f * acc[16] + 45.0f * acc[11]);
-        f[10] = 30.0f * acc[14];
-        f[11] = ((6.0f * acc[18] + -1.5f * acc[16]) + -1.5f * acc[11]);
-        f[12] = ((1.0f * acc[19] + -1.5f * acc[17]) + -1.5f * acc[12]);
-        f[13] = ((6.0f * acc[15] + -1.5f * acc[13]) + -1.5f * acc[10]);
-        f[14] = (-15.0f * acc[17] + 15.0f * acc[12]);
-        f[15] = (-45.0f * acc[13] + 15.0f * acc[10]);
-        f[16] = (-420.0f * acc[26] + 420.0f * acc[21]);
-        f[17] = (-105.0f * acc[31] + 315.0f * acc[24]);
-        f[18] = ((90.0f * acc[28] + -15.0f * acc[26]) + -15.0f * acc[21]);
-        f[19] = ((10.0f * acc[33] + -7.5f * acc[31]) + -7.5f * acc[24]);
-        f[20] = ((fmaf(0.75f, acc[23], 1.0f * acc[34]) + fmaf(0.375f, acc[20], -3.0f * acc[32])) + (0.375f * acc[30] + -3.0f * acc[25]));
-        f[21] = ((10.0f * acc[29] + -7.5f * acc[27]) + -7.5f * acc[22]);
-        f[22] = ((-45.0f * acc[32] + 7.5f * acc[30]) + (45.0f * acc[25] + -7.5f * acc[20]));
-        f[23] = (-315.0f * acc[27] + 105.0f * acc[22]);
-        f[24] = ((105.0f * acc[30] + -630.0f * acc[23]) + 105.0f * acc[20]);
-        f[25] = ((945.0f * acc[50] + -9450.0f * acc[41]) + 4725.0f * acc[36]);
-        f[26] = (-3780.0f * acc[46] + 3780.0f * acc[39]);
-        f[27] = ((fmaf(-157.5f, acc[36], -420.0f * acc[52]) + 52.5f * acc[50]) + (1260.0f * acc[43] + -105.0f * acc[41]));
-        f[28] = ((210.0f * acc[48] + -105.0f * acc[46]) + -105.0f * acc[39]);
-        f[29] = ((fmaf(3.75f, acc[41], 15.0f * acc[54]) + fmaf(1.875f, acc[36], -22.5f * acc[52])) + (1.875f * acc[50] + -22.5f * acc[43]));
-        f[30] = ((fmaf(3.75f, acc[42], 1.0f * acc[55]) + fmaf(1.875f, acc[37], -5.0f * acc[53])) + (1.875f * acc[51] + -5.0f * acc[44]));
-        f[31] = ((fmaf(3.75f, acc[38], 15.0f * acc[49]) + fmaf(1.875f, acc[35], -22.5f * acc[47])) + (1.875f * acc[45] + -22.5f * acc[40]));
-        f[32] = ((-105.0f * acc[53] + 52.5f * acc[51]) + (105.0f * acc[44] + -52.5f * acc[37]));
-        f[33] = ((fmaf(-52.5f, acc[35], -1260.0f * acc[47]) + 157.5f * acc[45]) + (420.0f * acc[40] + 105.0f * acc[38]));
-        f[34] = ((945.0f * acc[51] + -5670.0f * acc[42]) + 945.0f * acc[37]);
-        f[35] = ((4725.0f * acc[45] + -9450.0f * acc[38]) + 945.0f * acc[35]);
-    }
-    __device__ __forceinline__ static void grad_coeffs(const float* w, float* gq) {
-        (void)w; (void)gq;
-        gq[0] = 1.0f * w[3];
-        gq[1] = 1.0f * w[1];
-        gq[2] = 1.0f * w[2];
-        gq[3] = (-1.0f * w[6] + 6.0f * w[8]);
-        gq[4] = 6.0f * w[4];
-        gq[5] = 3.0f * w[7];
-        gq[6] = 6.0f * w[4];
-        gq[7] = (-1.0f * w[6] + -6.0f * w[8]);
-        gq[8] = 3.0f * w[5];
-        gq[9] = 3.0f * w[7];
-        gq[10] = 3.0f * w[5];
-        gq[11] = 2.0f * w[6];
-        gq[12] = (-4.5f * w[13] + 45.0f * w[15]);
-        gq[13] = (90.0f * w[9] + -3.0f * w[11]);
-        gq[14] = (-3.0f * w[12] + 30.0f * w[14]);
-        gq[15] = (-1.5f * w[13] + -45.0f * w[15]);
-        gq[16] = 30.0f * w[10];
-        gq[17] = 6.0f * w[13];
-        gq[18] = (45.0f * w[9] + -1.5f * w[11]);
-        gq[19] = (-3.0f * w[13] + -90.0f * w[15]);
-        gq[20] = 30.0f * w[10];
-        gq[21] = (-45.0f * w[9] + -4.5f * w[11]);
-        gq[22] = (-3.0f * w[12] + -30.0f * w[14]);
-        gq[23] = 6.0f * w[11];
-        gq[24] = (-1.5f * w[12] + 15.0f * w[14]);
-        gq[25] = 30.0f * w[10];
-        gq[26] = 12.0f * w[13];
-        gq[27] = (-1.5f * w[12] + -15.0f * w[14]);
-        gq[28] = 12.0f * w[11];
-        gq[29] = 3.0f * w[12];
-        gq[30] = ((1.5f * w[20] + -30.0f * w[22]) + 420.0f * w[24]);
-        gq[31] = (1260.0f * w[16] + -45.0f * w[18]);
-        gq[32] = (-22.5f * w[21] + 315.0f * w[23]);
-        gq[33] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[34] = (630.0f * w[17] + -15.0f * w[19]);
-        gq[35] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[36] = (-420.0f * w[16] + -15.0f * w[18]);
-        gq[37] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[38] = 90.0f * w[18];
-        gq[39] = 10.0f * w[21];
-        gq[40] = (420.0f * w[16] + -15.0f * w[18]);
-        gq[41] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[42] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[43] = (-1260.0f * w[16] + -45.0f * w[18]);
-        gq[44] = (-15.0f * w[21] + -630.0f * w[23]);
-        gq[45] = 90.0f * w[18];
-        gq[46] = ((1.5f * w[20] + 30.0f * w[22]) + 420.0f * w[24]);
-        gq[47] = (-315.0f * w[17] + -22.5f * w[19]);
-        gq[48] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[49] = 10.0f * w[19];
-        gq[50] = (-7.5f * w[21] + 105.0f * w[23]);
-        gq[51] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[52] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[53] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[54] = 180.0f * w[18];
-        gq[55] = 30.0f * w[21];
-        gq[56] = (-105.0f * w[17] + -7.5f * w[19]);
-        gq[57] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[58] = 30.0f * w[19];
-        gq[59] = 4.0f * w[20];
-        gq[60] = ((9.375f * w[31] + -262.5f * w[33]) + 4725.0f * w[35]);
-        gq[61] = ((18900.0f * w[25] + -630.0f * w[27]) + 7.5f * w[29]);
-        gq[62] = ((7.5f * w[30] + -210.0f * w[32]) + 3780.0f * w[34]);
-        gq[63] = ((11.25f * w[31] + 315.0f * w[33]) + -28350.0f * w[35]);
-        gq[64] = (11340.0f * w[26] + -315.0f * w[28]);
-        gq[65] = (-67.5f * w[31] + 1260.0f * w[33]);
-        gq[66] = ((-18900.0f * w[25] + -210.0f * w[27]) + 7.5f * w[29]);
-        gq[67] = (7.5f * w[30] + -11340.0f * w[34]);
-        gq[68] = (2520.0f * w[27] + -45.0f * w[29]);
-        gq[69] = (-10.0f * w[30] + 210.0f * w[32]);
-        gq[70] = ((1.875f * w[31] + 157.5f * w[33]) + 4725.0f * w[35]);
-        gq[71] = (-3780.0f * w[26] + -105.0f * w[28]);
-        gq[72] = (-22.5f * w[31] + -1260.0f * w[33]);
-        gq[73] = 210.0f * w[28];
-        gq[74] = 15.0f * w[31];
-        gq[75] = ((4725.0f * w[25] + -157.5f * w[27]) + 1.875f * w[29]);
-        gq[76] = ((7.5f * w[31] + 210.0f * w[33]) + -18900.0f * w[35]);
-        gq[77] = (3780.0f * w[26] + -105.0f * w[28]);
-        gq[78] = ((-28350.0f * w[25] + -315.0f * w[27]) + 11.25f * w[29]);
-        gq[79] = (7.5f * w[30] + -11340.0f * w[34]);
-        gq[80] = (1260.0f * w[27] + -22.5f * w[29]);
-        gq[81] = ((7.5f * w[31] + 630.0f * w[33]) + 18900.0f * w[35]);
-        gq[82] = (-11340.0f * w[26] + -315.0f * w[28]);
-        gq[83] = (-45.0f * w[31] + -2520.0f * w[33]);
-        gq[84] = 210.0f * w[28];
-        gq[85] = ((4725.0f * w[25] + 262.5f * w[27]) + 9.375f * w[29]);
-        gq[86] = ((7.5f * w[30] + 210.0f * w[32]) + 3780.0f * w[34]);
-        gq[87] = (-1260.0f * w[27] + -67.5f * w[29]);
-        gq[88] = (-10.0f * w[30] + -210.0f * w[32]);
-        gq[89] = 15.0f * w[29];
-        gq[90] = ((1.875f * w[30] + -52.5f * w[32]) + 945.0f * w[34]);
-        gq[91] = (3780.0f * w[26] + -105.0f * w[28]);
-        gq[92] = (-45.0f * w[31] + 840.0f * w[33]);
-        gq[93] = (3.75f * w[30] + -5670.0f * w[34]);
-        gq[94] = (2520.0f * w[27] + -45.0f * w[29]);
-        gq[95] = (-15.0f * w[30] + 315.0f * w[32]);
-        gq[96] = (-3780.0f * w[26] + -105.0f * w[28]);
-        gq[97] = (-45.0f * w[31] + -2520.0f * w[33]);
-        gq[98] = 630.0f * w[28];
-        gq[99] = 60.0f * w[31];
-        gq[100] = ((1.875f * w[30] + 52.5f * w[32]) + 945.0f * w[34]);
-        gq[101] = (-840.0f * w[27] + -45.0f * w[29]);
-        gq[102] = (-15.0f * w[30] + -315.0f * w[32]);
-        gq[103] = 60.0f * w[29];
-        gq[104] = 5.0f * w[30];
-    }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
-        (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        const float u1_0_0 = x;
-        const float u0_1_0 = y;
-        const float u0_0_1 = z;
-        const float u2_0_0 = x * u1_0_0;
-        const float u1_1_0 = x * u0_1_0;
-        const float u1_0_1 = x * u0_0_1;
-        const float u0_2_0 = y * u0_1_0;
-        const float u0_1_1 = y * u0_0_1;
-        const float u0_0_2 = z * u0_0_1;
-        const float u3_0_0 = x * u2_0_0;
-        const float u2_1_0 = x * u1_1_0;
-        const float u2_0_1 = x * u1_0_1;
-        const float u1_2_0 = x * u0_2_0;
-        const float u1_1_1 = x * u0_1_1;
-        const float u1_0_2 = x * u0_0_2;
-        const float u0_3_0 = y * u0_2_0;
-        const float u0_2_1 = y * u0_1_1;
-        const float u0_1_2 = y * u0_0_2;
-        const float u0_0_3 = z * u0_0_2;
-        const float u4_0_0 = x * u3_0_0;
-        const float u3_1_0 = x * u2_1_0;
-        const float u3_0_1 = x * u2_0_1;
-        const float u2_2_0 = x * u1_2_0;
-        const float u2_1_1 = x * u1_1_1;
-        const float u2_0_2 = x * u1_0_2;
-        const float u1_3_0 = x * u0_3_0;
-        const float u1_2_1 = x * u0_2_1;
-        const float u1_1_2 = x * u0_1_2;
-        const float u1_0_3 = x * u0_0_3;
-        const float u0_4_0 = y * u0_3_0;
-        const float u0_3_1 = y * u0_2_1;
-        const float u0_2_2 = y * u0_1_2;
-        const float u0_1_3 = y * u0_0_3;
-        const float u0_0_4 = z * u0_0_3;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
-        gx[1] = gq[3] * u1_0_0 + gq[4] * u0_1_0 + gq[5] * u0_0_1;
-        gy[1] = gq[6] * u1_0_0 + gq[7] * u0_1_0 + gq[8] * u0_0_1;
-        gz[1] = gq[9] * u1_0_0 + gq[10] * u0_1_0 + gq[11] * u0_0_1;
-        gx[2] = gq[12] * u2_0_0 + gq[13] * u1_1_0 + gq[14] * u1_0_1 + gq[15] * u0_2_0 + gq[16] * u0_1_1 + gq[17] * u0_0_2;
-        gy[2] = gq[18] * u2_0_0 + gq[19] * u1_1_0 + gq[20] * u1_0_1 + gq[21] * u0_2_0 + gq[22] * u0_1_1 + gq[23] * u0_0_2;
-        gz[2] = gq[24] * u2_0_0 + gq[25] * u1_1_0 + gq[26] * u1_0_1 + gq[27] * u0_2_0 + gq[28] * u0_1_1 + gq[29] * u0_0_2;
-        gx[3] = gq[30] * u3_0_0 + gq[31] * u2_1_0 + gq[32] * u2_0_1 + gq[33] * u1_2_0 + gq[34] * u1_1_1 + gq[35] * u1_0_2 + gq[36] * u0_3_0 + gq[37] * u0_2_1 + gq[38] * u0_1_2 + gq[39] * u0_0_3;
-        gy[3] = gq[40] * u3_0_0 + gq[41] * u2_1_0 + gq[42] * u2_0_1 + gq[43] * u1_2_0 + gq[44] * u1_1_1 + gq[45] * u1_0_2 + gq[46] * u0_3_0 + gq[47] * u0_2_1 + gq[48] * u0_1_2 + gq[49] * u0_0_3;
-        gz[3] = gq[50] * u3_0_0 + gq[51] * u2_1_0 + gq[52] * u2_0_1 + gq[53] * u1_2_0 + gq[54] * u1_1_1 + gq[55] * u1_0_2 + gq[56] * u0_3_0 + gq[57] * u0_2_1 + gq[58] * u0_1_2 + gq[59] * u0_0_3;
-        gx[4] = gq[60] * u4_0_0 + gq[61] * u3_1_0 + gq[62] * u3_0_1 + gq[63] * u2_2_0 + gq[64] * u2_1_1 + gq[65] * u2_0_2 + gq[66] * u1_3_0 + gq[67] * u1_2_1 + gq[68] * u1_1_2 + gq[69] * u1_0_3 + gq[70] * u0_4_0 + gq[71] * u0_3_1 + gq[72] * u0_2_2 + gq[73] * u0_1_3 + gq[74] * u0_0_4;
-        gy[4] = gq[75] * u4_0_0 + gq[76] * u3_1_0 + gq[77] * u3_0_1 + gq[78] * u2_2_0 + gq[79] * u2_1_1 + gq[80] * u2_0_2 + gq[81] * u1_3_0 + gq[82] * u1_2_1 + gq[83] * u1_1_2 + gq[84] * u1_0_3 + gq[85] * u0_4_0 + gq[86] * u0_3_1 + gq[87] * u0_2_2 + gq[88] * u0_1_3 + gq[89] * u0_0_4;
-        gz[4] = gq[90] * u4_0_0 + gq[91] * u3_1_0 + gq[92] * u3_0_1 + gq[93] * u2_2_0 + gq[94] * u2_1_1 + gq[95] * u2_0_2 + gq[96] * u1_3_0 + gq[97] * u1_2_1 + gq[98] * u1_1_2 + gq[99] * u1_0_3 + gq[100] * u0_4_0 + gq[101] * u0_3_1 + gq[102] * u0_2_2 + gq[103] * u0_1_3 + gq[104] * u0_0_4;
-    }
-    __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,
-                                               float* __restrict__ o) {
-        o[0] = ((fmaf(0.282094806432724f, a[32] * b[32], fmaf(0.282094806432724f, a[28] * b[28], fmaf(0.282094806432724f, a[24] * b[24], fmaf(0.282094806432724f, a[20] * b[20], fmaf(0.282094806432724f, a[16] * b[16], fmaf(0.282094806432724f, a[12] * b[12], fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])))))))) + fmaf(0.282094806432724f, a[33] * b[33], fmaf(0.282094806432724f, a[29] * b[29], fmaf(0.282094806432724f, a[25] * b[25], fmaf(0.282094806432724f, a[21] * b[21], fmaf(0.282094806432724f, a[17] * b[17], fmaf(0.282094806432724f, a[13] * b[13], fmaf(0.282094806432724f, a[9] * b[9], fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1]))))))))) + (fmaf(0.282094806432724f, a[34] * b[34], fmaf(0.282094806432724f, a[30] * b[30], fmaf(0.282094806432724f, a[26] * b[26], fmaf(0.282094806432724f, a[22] * b[22], fmaf(0.282094806432724f, a[18] * b[18], fmaf(0.282094806432724f, a[14] * b[14], fmaf(0.282094806432724f, a[10] * b[10], fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2])))))))) + fmaf(0.282094806432724f, a[35] * b[35], fmaf(0.282094806432724f, a[31] * b[31], fmaf(0.282094806432724f, a[27] * b[27], fmaf(0.282094806432724f, a[23] * b[23], fmaf(0.282094806432724f, a[19] * b[19], fmaf(0.282094806432724f, a[15] * b[15], fmaf(0.282094806432724f, a[11] * b[11], fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3]))))))))));
-        o[1] = ((fmaf(0.034723468124866486f, (a[24] * b[27] + a[27] * b[24]), fmaf(0.08505477756261826f, (a[22] * b[29] + a[29] * b[22]), fmaf(-0.15912292897701263f, (a[19] * b[32] + a[32] * b[19]), fmaf(-0.2083408087491989f, (a[17] * b[34] + a[34] * b[17]), fmaf(0.04352817311882973f, (a[15] * b[18] + a[18] * b[15]), fmaf(0.16858388483524323f, (a[13] * b[18] + a[18] * b[13]), fmaf(-0.1994711458683014f, (a[10] * b[23] + a[23] * b[10]), fmaf(0.05839917063713074f, (a[8] * b[11] + a[11] * b[8]), fmaf(-0.18467439711093903f, (a[5] * b[14] + a[14] * b[5]), fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0]))))))))))) + fmaf(0.2083408087491989f, (a[23] * b[26] + a[26] * b[23]), fmaf(0.19018827378749847f, (a[20] * b[29] + a[29] * b[20]), fmaf(-0.08505477756261826f, (a[18] * b[31] + a[31] * b[18]), fmaf(-0.034723468124866486f, (a[16] * b[33] + a[33] * b[16]), fmaf(0.1994711458683014f, (a[14] * b[17] + a[17] * b[14]), fmaf(-0.15078601241111755f, (a[11] * b[20] + a[20] * b[11]), fmaf(-0.04352817311882973f, (a[9] * b[22] + a[22] * b[9]), fmaf(0.20230065286159515f, (a[6] * b[11] + a[11] * b[6]), fmaf(-0.05839917063713074f, (a[4] * b[13] + a[13] * b[4]), -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1]))))))))))) + (fmaf(0.06014281138777733f, (a[23] * b[28] + a[28] * b[23]), fmaf(0.15912292897701263f, (a[21] * b[28] + a[28] * b[21]), fmaf(-0.1837393194437027f, (a[18] * b[33] + a[33] * b[18]), fmaf(-0.23293210566043854f, (a[16] * b[35] + a[35] * b[16]), fmaf(0.07539300620555878f, (a[14] * b[19] + a[19] * b[14]), fmaf(-0.16858388483524323f, (a[11] * b[22] + a[22] * b[11]), fmaf(-0.23032943904399872f, (a[9] * b[24] + a[24] * b[9]), fmaf(0.18467439711093903f, (a[7] * b[10] + a[10] * b[7]), fmaf(-0.22617901861667633f, (a[4] * b[15] + a[15] * b[4]), -0.21850968897342682f * (a[1] * b[8] + a[8] * b[1])))))))))) + fmaf(0.23293210566043854f, (a[24] * b[25] + a[25] * b[24]), fmaf(0.1837393194437027f, (a[22] * b[27] + a[27] * b[22]), fmaf(-0.15528807044029236f, (a[19] * b[30] + a[30] * b[19]), fmaf(-0.06014281138777733f, (a[17] * b[32] + a[32] * b[17]), fmaf(0.23032943904399872f, (a[15] * b[16] + a[16] * b[15]), fmaf(0.1946638971567154f, (a[12] * b[19] + a[19] * b[12]), fmaf(-0.07539300620555878f, (a[10] * b[21] + a[21] * b[10]), fmaf(0.22617901861667633f, (a[8] * b[9] + a[9] * b[8]), fmaf(-0.14304816722869873f, (a[5] * b[12] + a[12] * b[5]), 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2]))))))))))));
-        o[2] = ((fmaf(0.14731919765472412f, (a[24] * b[34] + a[34] * b[24]), fmaf(0.24553200602531433f, (a[20] * b[30] + a[30] * b[20]), fmaf(0.14731919765472412f, (a[16] * b[26] + a[26] * b[16]), fmaf(0.2462325245141983f, (a[12] * b[20] + a[20] * b[12]), fmaf(0.18467439711093903f, (a[8] * b[14] + a[14] * b[8]), fmaf(0.18467439711093903f, (a[4] * b[10] + a[10] * b[4]), 0.282094806432724f * (a[0] * b[2] + a[2] * b[0]))))))) + fmaf(0.24057124555110931f, (a[21] * b[31] + a[31] * b[21]), fmaf(0.19642560184001923f, (a[17] * b[27] + a[27] * b[17]), fmaf(0.23841361701488495f, (a[13] * b[21] + a[21] * b[13]), fmaf(0.1628675013780594f, (a[9] * b[17] + a[17] * b[9]), fmaf(0.23359668254852295f, (a[5] * b[11] + a[11] * b[5]), 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1]))))))) + (fmaf(0.22503378987312317f, (a[22] * b[32] + a[32] * b[22]), fmaf(0.22503378987312317f, (a[18] * b[28] + a[28] * b[18]), fmaf(0.21324361860752106f, (a[14] * b[22] + a[22] * b[14]), fmaf(0.21324361860752106f, (a[10] * b[18] + a[18] * b[10]), fmaf(0.24776668846607208f, (a[6] * b[12] + a[12] * b[6]), 0.2523132562637329f * (a[2] * b[6] + a[6] * b[2])))))) + fmaf(0.19642560184001923f, (a[23] * b[33] + a[33] * b[23]), fmaf(0.24057124555110931f, (a[19] * b[29] + a[29] * b[19]), fmaf(0.1628675013780594f, (a[15] * b[23] + a[23] * b[15]), fmaf(0.23841361701488495f, (a[11] * b[19] + a[19] * b[11]), fmaf(0.23359668254852295f, (a[7] * b[13] + a[13] * b[7]), 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3]))))))));
-        o[3] = ((fmaf(0.23293210566043854f, (a[24] * b[35] + a[35] * b[24]), fmaf(0.1837393194437027f, (a[22] * b[33] + a[33] * b[22]), fmaf(0.19018827378749847f, (a[20] * b[31] + a[31] * b[20]), fmaf(-0.06014281138777733f, (a[17] * b[28] + a[28] * b[17]), fmaf(0.23032943904399872f, (a[15] * b[24] + a[24] * b[15]), fmaf(0.16858388483524323f, (a[13] * b[22] + a[22] * b[13]), fmaf(-0.07539300620555878f, (a[10] * b[19] + a[19] * b[10]), fmaf(0.22617901861667633f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.20230065286159515f, (a[6] * b[13] + a[13] * b[6]), fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0]))))))))))) + fmaf(-0.06014281138777733f, (a[23] * b[32] + a[32] * b[23]), fmaf(-0.15528807044029236f, (a[21] * b[30] + a[30] * b[21]), fmaf(0.1837393194437027f, (a[18] * b[27] + a[27] * b[18]), fmaf(0.23293210566043854f, (a[16] * b[25] + a[25] * b[16]), fmaf(-0.07539300620555878f, (a[14] * b[21] + a[21] * b[14]), fmaf(0.16858388483524323f, (a[11] * b[18] + a[18] * b[11]), fmaf(0.23032943904399872f, (a[9] * b[16] + a[16] * b[9]), fmaf(-0.14304816722869873f, (a[7] * b[12] + a[12] * b[7]), fmaf(0.22617901861667633f, (a[4] * b[9] + a[9] * b[4]), 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1]))))))))))) + (fmaf(0.2083408087491989f, (a[23] * b[34] + a[34] * b[23]), fmaf(0.15912292897701263f, (a[21] * b[32] + a[32] * b[21]), fmaf(-0.08505477756261826f, (a[18] * b[29] + a[29] * b[18]), fmaf(-0.034723468124866486f, (a[16] * b[27] + a[27] * b[16]), fmaf(0.1994711458683014f, (a[14] * b[23] + a[23] * b[14]), fmaf(0.1946638971567154f, (a[12] * b[21] + a[21] * b[12]), fmaf(-0.04352817311882973f, (a[9] * b[18] + a[18] * b[9]), fmaf(0.18467439711093903f, (a[7] * b[14] + a[14] * b[7]), fmaf(-0.05839917063713074f, (a[4] * b[11] + a[11] * b[4]), 0.21850968897342682f * (a[2] * b[7] + a[7] * b[2])))))))))) + fmaf(-0.034723468124866486f, (a[24] * b[33] + a[33] * b[24]), fmaf(-0.08505477756261826f, (a[22] * b[31] + a[31] * b[22]), fmaf(0.15912292897701263f, (a[19] * b[28] + a[28] * b[19]), fmaf(0.2083408087491989f, (a[17] * b[26] + a[26] * b[17]), fmaf(-0.04352817311882973f, (a[15] * b[22] + a[22] * b[15]), fmaf(-0.15078601241111755f, (a[13] * b[20] + a[20] * b[13]), fmaf(0.1994711458683014f, (a[10] * b[17] + a[17] * b[10]), fmaf(-0.05839917063713074f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.18467439711093903f, (a[5] * b[10] + a[10] * b[5]), -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3]))))))))))));
-        o[4] = ((fmaf(0.09704355895519257f, (a[28] * b[34] + a[34] * b[28]), fmaf(-0.09704355895519257f, (a[26] * b[32] + a[32] * b[26]), fmaf(0.07508081942796707f, (a[18] * b[24] + a[24] * b[18]), fmaf(-0.016943316906690598f, (a[15] * b[29] + a[29] * b[15]), fmaf(0.14175796508789062f, (a[13] * b[27] + a[27] * b[13]), fmaf(0.09403159469366074f, (a[11] * b[15] + a[15] * b[11]), fmaf(-0.18806318938732147f, (a[10] * b[12] + a[12] * b[10]), fmaf(0.23841361701488495f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.16858388483524323f, (a[5] * b[23] + a[23] * b[5]), fmaf(0.04029925540089607f, (a[4] * b[20] + a[20] * b[4]), fmaf(0.18467439711093903f, (a[2] * b[10] + a[10] * b[2]), 0.282094806432724f * (a[0] * b[4] + a[4] * b[0])))))))))))) + fmaf(0.14007030427455902f, (a[29] * b[31] + a[31] * b[29]), fmaf(-0.12103458493947983f, (a[27] * b[31] + a[31] * b[27]), fmaf(0.14188940823078156f, (a[19] * b[21] + a[21] * b[19]), fmaf(-0.07508081942796707f, (a[16] * b[22] + a[22] * b[16]), fmaf(-0.06562118977308273f, (a[13] * b[29] + a[29] * b[13]), fmaf(-0.06562118977308273f, (a[11] * b[31] + a[31] * b[11]), fmaf(0.05357947573065758f, (a[10] * b[30] + a[30] * b[10]), fmaf(-0.09403159469366074f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.15607835352420807f, (a[6] * b[18] + a[18] * b[6]), fmaf(-0.23841361701488495f, (a[4] * b[24] + a[24] * b[4]), fmaf(0.22617901861667633f, (a[3] * b[9] + a[9] * b[3]), 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1]))))))))))))) + (fmaf(0.12103458493947983f, (a[29] * b[33] + a[33] * b[29]), fmaf(0.06264134496450424f, (a[27] * b[35] + a[35] * b[27]), fmaf(0.11262122541666031f, (a[19] * b[23] + a[23] * b[19]), fmaf(-0.11262122541666031f, (a[17] * b[21] + a[21] * b[17]), fmaf(0.19018827378749847f, (a[14] * b[26] + a[26] * b[14]), fmaf(-0.14175796508789062f, (a[11] * b[33] + a[33] * b[11]), fmaf(-0.19018827378749847f, (a[10] * b[34] + a[34] * b[10]), fmaf(0.016943316906690598f, (a[9] * b[31] + a[31] * b[9]), fmaf(0.16858388483524323f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.15607835352420807f, (a[5] * b[7] + a[7] * b[5]), fmaf(-0.05839917063713074f, (a[3] * b[11] + a[11] * b[3]), -0.05839917063713074f * (a[1] * b[13] + a[13] * b[1])))))))))))) + fmaf(-0.19137248396873474f, (a[28] * b[30] + a[30] * b[28]), fmaf(-0.06264134496450424f, (a[25] * b[33] + a[33] * b[25]), fmaf(-0.19036461412906647f, (a[18] * b[20] + a[20] * b[18]), fmaf(0.24553200602531433f, (a[15] * b[25] + a[25] * b[15]), fmaf(0.14175796508789062f, (a[12] * b[28] + a[28] * b[12]), fmaf(0.14567312598228455f, (a[11] * b[13] + a[13] * b[11]), fmaf(-0.24553200602531433f, (a[9] * b[35] + a[35] * b[9]), fmaf(-0.06371872127056122f, (a[7] * b[19] + a[19] * b[7]), fmaf(-0.06371872127056122f, (a[5] * b[21] + a[21] * b[5]), fmaf(-0.180223748087883f, (a[4] * b[6] + a[6] * b[4]), -0.22617901861667633f * (a[1] * b[15] + a[15] * b[1])))))))))))));
-        o[5] = ((fmaf(0.0361659973859787f, (a[29] * b[30] + a[30] * b[29]), fmaf(0.11436693370342255f, (a[27] * b[32] + a[32] * b[27]), fmaf(-0.09029786288738251f, (a[19] * b[22] + a[22] * b[19]), fmaf(-0.14046335220336914f, (a[17] * b[24] + a[24] * b[17]), fmaf(0.15528807044029236f, (a[15] * b[26] + a[26] * b[15]), fmaf(0.2143179029226303f, (a[12] * b[29] + a[29] * b[12]), fmaf(0.059470802545547485f, (a[11] * b[12] + a[12] * b[11]), fmaf(0.11516471952199936f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.06371872127056122f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.180223748087883f, (a[5] * b[22] + a[22] * b[5]), fmaf(-0.16858388483524323f, (a[4] * b[23] + a[23] * b[4]), fmaf(0.23359668254852295f, (a[2] * b[11] + a[11] * b[2]), 0.282094806432724f * (a[0] * b[5] + a[5] * b[0]))))))))))))) + fmaf(-0.0741182416677475f, (a[29] * b[32] + a[32] * b[29]), fmaf(-0.13866253197193146f, (a[27] * b[34] + a[34] * b[27]), fmaf(0.13288237154483795f, (a[25] * b[34] + a[34] * b[25]), fmaf(0.09029786288738251f, (a[18] * b[21] + a[21] * b[18]), fmaf(0.04482780396938324f, (a[15] * b[28] + a[28] * b[15]), fmaf(0.17361734807491302f, (a[13] * b[28] + a[28] * b[13]), fmaf(-0.11516471952199936f, (a[11] * b[14] + a[14] * b[11]), fmaf(-0.1486770063638687f, (a[10] * b[15] + a[15] * b[10]), fmaf(0.1486770063638687f, (a[9] * b[14] + a[14] * b[9]), fmaf(0.22072811424732208f, (a[6] * b[19] + a[19] * b[6]), fmaf(0.0901118740439415f, (a[5] * b[6] + a[6] * b[5]), fmaf(0.18467439711093903f, (a[3] * b[10] + a[10] * b[3]), 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1])))))))))))))) + (fmaf(0.0741182416677475f, (a[28] * b[31] + a[31] * b[28]), fmaf(0.13866253197193146f, (a[26] * b[33] + a[33] * b[26]), fmaf(-0.13272538781166077f, (a[18] * b[23] + a[23] * b[18]), fmaf(0.14046335220336914f, (a[16] * b[23] + a[23] * b[16]), fmaf(0.17931121587753296f, (a[14] * b[27] + a[27] * b[14]), fmaf(-0.16943317651748657f, (a[11] * b[30] + a[30] * b[11]), fmaf(-0.08300496637821198f, (a[10] * b[31] + a[31] * b[10]), fmaf(-0.04482780396938324f, (a[9] * b[32] + a[32] * b[9]), fmaf(0.180223748087883f, (a[7] * b[18] + a[18] * b[7]), fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[7] + a[7] * b[4]), -0.14304816722869873f * (a[1] * b[12] + a[12] * b[1])))))))))))) + fmaf(-0.11436693370342255f, (a[28] * b[33] + a[33] * b[28]), fmaf(-0.13288237154483795f, (a[26] * b[35] + a[35] * b[26]), fmaf(0.04486937075853348f, (a[19] * b[20] + a[20] * b[19]), fmaf(0.13272538781166077f, (a[17] * b[22] + a[22] * b[17]), fmaf(0.08300496637821198f, (a[14] * b[29] + a[29] * b[14]), fmaf(-0.17361734807491302f, (a[11] * b[32] + a[32] * b[11]), fmaf(-0.17931121587753296f, (a[10] * b[33] + a[33] * b[10]), fmaf(-0.15528807044029236f, (a[9] * b[34] + a[34] * b[9]), fmaf(0.16858388483524323f, (a[8] * b[17] + a[17] * b[8]), fmaf(-0.1611970216035843f, (a[5] * b[20] + a[20] * b[5]), fmaf(-0.06371872127056122f, (a[4] * b[21] + a[21] * b[4]), -0.18467439711093903f * (a[1] * b[14] + a[14] * b[1]))))))))))))));
-        o[6] = ((fmaf(-0.24260888993740082f, a[35] * b[35], fmaf(0.14556533098220825f, a[31] * b[31], fmaf(0.01617392711341381f, a[27] * b[27], fmaf(-0.057343922555446625f, a[23] * b[23], fmaf(0.1392638087272644f, a[19] * b[19], fmaf(0.12679217755794525f, (a[15] * b[33] + a[33] * b[15]), fmaf(0.12615662813186646f, a[13] * b[13], fmaf(0.12615662813186646f, a[11] * b[11], fmaf(0.15607835352420807f, (a[8] * b[22] + a[22] * b[8]), fmaf(0.24179553985595703f, (a[6] * b[20] + a[20] * b[6]), fmaf(0.15607835352420807f, (a[4] * b[18] + a[18] * b[4]), fmaf(0.24776668846607208f, (a[2] * b[12] + a[12] * b[2]), 0.282094806432724f * (a[0] * b[6] + a[6] * b[0]))))))))))))) + fmaf(0.09704355895519257f, a[32] * b[32], fmaf(0.09704355895519257f, a[28] * b[28], fmaf(-0.2293756902217865f, a[24] * b[24], fmaf(0.16383977234363556f, a[20] * b[20], fmaf(-0.2293756902217865f, a[16] * b[16], fmaf(0.22731846570968628f, (a[13] * b[31] + a[31] * b[13]), fmaf(0.22731846570968628f, (a[11] * b[29] + a[29] * b[11]), fmaf(-0.2102610468864441f, a[9] * b[9], fmaf(0.0901118740439415f, a[7] * b[7], fmaf(0.0901118740439415f, a[5] * b[5], fmaf(-0.12615662813186646f, a[3] * b[3], -0.12615662813186646f * a[1] * b[1])))))))))))) + (fmaf(0.01617392711341381f, a[33] * b[33], fmaf(0.14556533098220825f, a[29] * b[29], fmaf(-0.24260888993740082f, a[25] * b[25], fmaf(0.1392638087272644f, a[21] * b[21], fmaf(-0.057343922555446625f, a[17] * b[17], fmaf(0.19018827378749847f, (a[14] * b[32] + a[32] * b[14]), fmaf(0.16820883750915527f, a[12] * b[12], fmaf(0.12679217755794525f, (a[9] * b[27] + a[27] * b[9]), fmaf(0.22072811424732208f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.22072811424732208f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.20230065286159515f, (a[3] * b[13] + a[13] * b[3]), 0.20230065286159515f * (a[1] * b[11] + a[11] * b[1])))))))))))) + fmaf(-0.09704355895519257f, a[34] * b[34], fmaf(0.1617392599582672f, a[30] * b[30], fmaf(-0.09704355895519257f, a[26] * b[26], fmaf(0.06553591042757034f, a[22] * b[22], fmaf(0.06553591042757034f, a[18] * b[18], fmaf(-0.2102610468864441f, a[15] * b[15], fmaf(0.23961469531059265f, (a[12] * b[30] + a[30] * b[12]), fmaf(0.19018827378749847f, (a[10] * b[28] + a[28] * b[10]), fmaf(-0.180223748087883f, a[8] * b[8], fmaf(0.180223748087883f, a[6] * b[6], fmaf(-0.180223748087883f, a[4] * b[4], 0.2523132562637329f * a[2] * b[2])))))))))))));
-        o[7] = ((fmaf(0.13866253197193146f, (a[33] * b[34] + a[34] * b[33]), fmaf(0.0741182416677475f, (a[28] * b[29] + a[29] * b[28]), fmaf(0.14046335220336914f, (a[23] * b[24] + a[24] * b[23]), fmaf(0.09029786288738251f, (a[18] * b[19] + a[19] * b[18]), fmaf(-0.04482780396938324f, (a[15] * b[32] + a[32] * b[15]), fmaf(0.17361734807491302f, (a[13] * b[32] + a[32] * b[13]), fmaf(0.059470802545547485f, (a[12] * b[13] + a[13] * b[12]), fmaf(0.11516471952199936f, (a[10] * b[11] + a[11] * b[10]), fmaf(0.16858388483524323f, (a[8] * b[23] + a[23] * b[8]), fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), fmaf(-0.06371872127056122f, (a[4] * b[19] + a[19] * b[4]), fmaf(-0.14304816722869873f, (a[3] * b[12] + a[12] * b[3]), 0.282094806432724f * (a[0] * b[7] + a[7] * b[0]))))))))))))) + fmaf(0.13288237154483795f, (a[34] * b[35] + a[35] * b[34]), fmaf(0.0361659973859787f, (a[30] * b[31] + a[31] * b[30]), fmaf(0.13288237154483795f, (a[25] * b[26] + a[26] * b[25]), fmaf(0.04486937075853348f, (a[20] * b[21] + a[21] * b[20]), fmaf(0.15528807044029236f, (a[15] * b[34] + a[34] * b[15]), fmaf(0.1486770063638687f, (a[14] * b[15] + a[15] * b[14]), fmaf(0.2143179029226303f, (a[12] * b[31] + a[31] * b[12]), fmaf(0.17931121587753296f, (a[10] * b[27] + a[27] * b[10]), fmaf(0.1486770063638687f, (a[9] * b[10] + a[10] * b[9]), fmaf(-0.1611970216035843f, (a[7] * b[20] + a[20] * b[7]), fmaf(0.180223748087883f, (a[5] * b[18] + a[18] * b[5]), fmaf(0.18467439711093903f, (a[3] * b[14] + a[14] * b[3]), 0.18467439711093903f * (a[1] * b[10] + a[10] * b[1])))))))))))))) + (fmaf(0.0741182416677475f, (a[31] * b[32] + a[32] * b[31]), fmaf(0.13866253197193146f, (a[26] * b[27] + a[27] * b[26]), fmaf(0.09029786288738251f, (a[21] * b[22] + a[22] * b[21]), fmaf(0.14046335220336914f, (a[16] * b[17] + a[17] * b[16]), fmaf(-0.08300496637821198f, (a[14] * b[31] + a[31] * b[14]), fmaf(0.11516471952199936f, (a[13] * b[14] + a[14] * b[13]), fmaf(-0.08300496637821198f, (a[10] * b[29] + a[29] * b[10]), fmaf(0.15528807044029236f, (a[9] * b[26] + a[26] * b[9]), fmaf(0.180223748087883f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.0901118740439415f, (a[6] * b[7] + a[7] * b[6]), fmaf(0.15607835352420807f, (a[4] * b[5] + a[5] * b[4]), 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2])))))))))))) + fmaf(0.11436693370342255f, (a[32] * b[33] + a[33] * b[32]), fmaf(0.11436693370342255f, (a[27] * b[28] + a[28] * b[27]), fmaf(0.13272538781166077f, (a[22] * b[23] + a[23] * b[22]), fmaf(0.13272538781166077f, (a[17] * b[18] + a[18] * b[17]), fmaf(0.17931121587753296f, (a[14] * b[33] + a[33] * b[14]), fmaf(-0.16943317651748657f, (a[13] * b[30] + a[30] * b[13]), fmaf(0.17361734807491302f, (a[11] * b[28] + a[28] * b[11]), fmaf(-0.04482780396938324f, (a[9] * b[28] + a[28] * b[9]), fmaf(-0.06371872127056122f, (a[8] * b[21] + a[21] * b[8]), fmaf(0.22072811424732208f, (a[6] * b[21] + a[21] * b[6]), fmaf(0.16858388483524323f, (a[4] * b[17] + a[17] * b[4]), 0.23359668254852295f * (a[2] * b[13] + a[13] * b[2]))))))))))))));
-        o[8] = ((fmaf(0.14007030427455902f, a[31] * b[31], fmaf(-0.09704355895519257f, (a[26] * b[28] + a[28] * b[26]), fmaf(0.14188940823078156f, a[21] * b[21], fmaf(-0.07508081942796707f, (a[16] * b[18] + a[18] * b[16]), fmaf(0.05357947573065758f, (a[14] * b[30] + a[30] * b[14]), fmaf(0.14567312598228455f, a[13] * b[13], fmaf(0.14175796508789062f, (a[11] * b[27] + a[27] * b[11]), fmaf(0.24553200602531433f, (a[9] * b[25] + a[25] * b[9]), fmaf(0.16858388483524323f, (a[7] * b[23] + a[23] * b[7]), fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), fmaf(0.23841361701488495f, (a[4] * b[16] + a[16] * b[4]), fmaf(0.18467439711093903f, (a[2] * b[14] + a[14] * b[2]), 0.282094806432724f * (a[0] * b[8] + a[8] * b[0]))))))))))))) + fmaf(-0.12103458493947983f, (a[31] * b[33] + a[33] * b[31]), fmaf(-0.12103458493947983f, (a[27] * b[29] + a[29] * b[27]), fmaf(-0.11262122541666031f, (a[21] * b[23] + a[23] * b[21]), fmaf(-0.11262122541666031f, (a[17] * b[19] + a[19] * b[17]), fmaf(0.19018827378749847f, (a[14] * b[34] + a[34] * b[14]), fmaf(-0.09403159469366074f, (a[13] * b[15] + a[15] * b[13]), fmaf(0.06562118977308273f, (a[11] * b[29] + a[29] * b[11]), fmaf(0.016943316906690598f, (a[9] * b[29] + a[29] * b[9]), fmaf(0.04029925540089607f, (a[8] * b[20] + a[20] * b[8]), fmaf(0.15607835352420807f, (a[6] * b[22] + a[22] * b[6]), fmaf(-0.15607835352420807f, a[5] * b[5], fmaf(0.21850968897342682f, a[3] * b[3], -0.21850968897342682f * a[1] * b[1]))))))))))))) + (fmaf(-0.09704355895519257f, (a[32] * b[34] + a[34] * b[32]), fmaf(-0.14007030427455902f, a[29] * b[29], fmaf(-0.07508081942796707f, (a[22] * b[24] + a[24] * b[22]), fmaf(-0.14188940823078156f, a[19] * b[19], fmaf(0.016943316906690598f, (a[15] * b[31] + a[31] * b[15]), fmaf(-0.06562118977308273f, (a[13] * b[31] + a[31] * b[13]), fmaf(-0.18806318938732147f, (a[12] * b[14] + a[14] * b[12]), fmaf(0.19018827378749847f, (a[10] * b[26] + a[26] * b[10]), fmaf(0.23841361701488495f, (a[8] * b[24] + a[24] * b[8]), fmaf(0.15607835352420807f, a[7] * b[7], fmaf(0.16858388483524323f, (a[5] * b[17] + a[17] * b[5]), fmaf(-0.05839917063713074f, (a[3] * b[13] + a[13] * b[3]), 0.22617901861667633f * (a[1] * b[9] + a[9] * b[1]))))))))))))) + fmaf(-0.06264134496450424f, (a[33] * b[35] + a[35] * b[33]), fmaf(-0.19137248396873474f, (a[30] * b[32] + a[32] * b[30]), fmaf(-0.06264134496450424f, (a[25] * b[27] + a[27] * b[25]), fmaf(-0.19036461412906647f, (a[20] * b[22] + a[22] * b[20]), fmaf(0.24553200602531433f, (a[15] * b[35] + a[35] * b[15]), fmaf(0.14175796508789062f, (a[13] * b[33] + a[33] * b[13]), fmaf(0.14175796508789062f, (a[12] * b[32] + a[32] * b[12]), fmaf(-0.14567312598228455f, a[11] * b[11], fmaf(-0.09403159469366074f, (a[9] * b[11] + a[11] * b[9]), fmaf(-0.06371872127056122f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.06371872127056122f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.22617901861667633f, (a[3] * b[15] + a[15] * b[3]), 0.05839917063713074f * (a[1] * b[11] + a[11] * b[1])))))))))))))));
-        o[9] = ((fmaf(-0.10158468782901764f, (a[22] * b[29] + a[29] * b[22]), fmaf(-0.19628025591373444f, (a[20] * b[27] + a[27] * b[20]), fmaf(-0.10158468782901764f, (a[18] * b[31] + a[31] * b[18]), fmaf(0.1332552284002304f, (a[13] * b[18] + a[18] * b[13]), fmaf(0.1332552284002304f, (a[11] * b[22] + a[22] * b[11]), fmaf(0.24553200602531433f, (a[8] * b[25] + a[25] * b[8]), fmaf(0.1486770063638687f, (a[7] * b[10] + a[10] * b[7]), fmaf(-0.04482780396938324f, (a[5] * b[32] + a[32] * b[5]), fmaf(-0.09403159469366074f, (a[4] * b[13] + a[13] * b[4]), fmaf(0.1628675013780594f, (a[2] * b[17] + a[17] * b[2]), 0.282094806432724f * (a[0] * b[9] + a[9] * b[0]))))))))))) + fmaf(-0.03583570942282677f, (a[24] * b[29] + a[29] * b[24]), fmaf(-0.1316688060760498f, (a[21] * b[26] + a[26] * b[21]), fmaf(0.09814012795686722f, (a[18] * b[35] + a[35] * b[18]), fmaf(-0.09932258725166321f, (a[14] * b[19] + a[19] * b[14]), fmaf(0.11752006411552429f, (a[11] * b[24] + a[24] * b[11]), fmaf(0.016943316906690598f, (a[8] * b[29] + a[29] * b[8]), fmaf(0.15528807044029236f, (a[7] * b[26] + a[26] * b[7]), fmaf(-0.15528807044029236f, (a[5] * b[34] + a[34] * b[5]), fmaf(0.016943316906690598f, (a[4] * b[31] + a[31] * b[4]), fmaf(0.22617901861667633f, (a[3] * b[4] + a[4] * b[3]), 0.22617901861667633f * (a[1] * b[8] + a[8] * b[1])))))))))))) + (fmaf(0.1266983598470688f, (a[21] * b[28] + a[28] * b[21]), fmaf(0.1266983598470688f, (a[19] * b[32] + a[32] * b[19]), fmaf(0.03583570942282677f, (a[16] * b[31] + a[31] * b[16]), fmaf(-0.20355072617530823f, (a[12] * b[17] + a[17] * b[12]), fmaf(0.07693494111299515f, (a[9] * b[20] + a[20] * b[9]), fmaf(-0.04482780396938324f, (a[7] * b[28] + a[28] * b[7]), fmaf(-0.2102610468864441f, (a[6] * b[9] + a[9] * b[6]), fmaf(-0.24553200602531433f, (a[4] * b[35] + a[35] * b[4]), fmaf(0.23032943904399872f, (a[3] * b[16] + a[16] * b[3]), -0.04352817311882973f * (a[1] * b[22] + a[22] * b[1])))))))))) + fmaf(-0.09814012795686722f, (a[22] * b[25] + a[25] * b[22]), fmaf(0.1316688060760498f, (a[19] * b[34] + a[34] * b[19]), fmaf(0.09814012795686722f, (a[17] * b[30] + a[30] * b[17]), fmaf(-0.11752006411552429f, (a[13] * b[16] + a[16] * b[13]), fmaf(-0.09932258725166321f, (a[10] * b[21] + a[21] * b[10]), fmaf(-0.09403159469366074f, (a[8] * b[11] + a[11] * b[8]), fmaf(0.12679217755794525f, (a[6] * b[27] + a[27] * b[6]), fmaf(0.1486770063638687f, (a[5] * b[14] + a[14] * b[5]), fmaf(-0.04352817311882973f, (a[3] * b[18] + a[18] * b[3]), -0.23032943904399872f * (a[1] * b[24] + a[24] * b[1]))))))))))));
-        o[10] = ((fmaf(0.11379365622997284f, (a[23] * b[29] + a[29] * b[23]), fmaf(0.025339672341942787f, (a[21] * b[27] + a[27] * b[21]), fmaf(-0.10135868936777115f, (a[18] * b[34] + a[34] * b[18]), fmaf(-0.07741397619247437f, (a[16] * b[32] + a[32] * b[16]), fmaf(0.06785023957490921f, (a[13] * b[17] + a[17] * b[13]), fmaf(-0.15171775221824646f, (a[10] * b[24] + a[24] * b[10]), fmaf(-0.08300496637821198f, (a[7] * b[29] + a[29] * b[7]), fmaf(0.19018827378749847f, (a[6] * b[28] + a[28] * b[6]), fmaf(0.11516471952199936f, (a[5] * b[13] + a[13] * b[5]), fmaf(-0.07539300620555878f, (a[3] * b[19] + a[19] * b[3]), fmaf(0.18467439711093903f, (a[2] * b[4] + a[4] * b[2]), 0.282094806432724f * (a[0] * b[10] + a[10] * b[0])))))))))))) + fmaf(0.07741397619247437f, (a[24] * b[28] + a[28] * b[24]), fmaf(0.09774991124868393f, (a[21] * b[29] + a[29] * b[21]), fmaf(0.09774991124868393f, (a[19] * b[31] + a[31] * b[19]), fmaf(-0.11379365622997284f, (a[17] * b[31] + a[31] * b[17]), fmaf(0.10257992148399353f, (a[13] * b[19] + a[19] * b[13]), fmaf(0.10257992148399353f, (a[11] * b[21] + a[21] * b[11]), fmaf(0.19018827378749847f, (a[8] * b[26] + a[26] * b[8]), fmaf(0.1486770063638687f, (a[7] * b[9] + a[9] * b[7]), fmaf(-0.1486770063638687f, (a[5] * b[15] + a[15] * b[5]), fmaf(-0.18806318938732147f, (a[4] * b[12] + a[12] * b[4]), fmaf(0.21324361860752106f, (a[2] * b[18] + a[18] * b[2]), 0.18467439711093903f * (a[1] * b[7] + a[7] * b[1]))))))))))))) + (fmaf(0.10135868936777115f, (a[22] * b[26] + a[26] * b[22]), fmaf(-0.025339672341942787f, (a[19] * b[33] + a[33] * b[19]), fmaf(-0.1499115228652954f, (a[17] * b[35] + a[35] * b[17]), fmaf(0.15171775221824646f, (a[14] * b[16] + a[16] * b[14]), fmaf(-0.06785023957490921f, (a[11] * b[23] + a[23] * b[11]), fmaf(-0.09932258725166321f, (a[9] * b[21] + a[21] * b[9]), fmaf(0.11516471952199936f, (a[7] * b[11] + a[11] * b[7]), fmaf(-0.08300496637821198f, (a[5] * b[31] + a[31] * b[5]), fmaf(0.05357947573065758f, (a[4] * b[30] + a[30] * b[4]), fmaf(0.18467439711093903f, (a[3] * b[5] + a[5] * b[3]), -0.07539300620555878f * (a[1] * b[21] + a[21] * b[1]))))))))))) + fmaf(0.1499115228652954f, (a[23] * b[25] + a[25] * b[23]), fmaf(-0.06542675197124481f, (a[20] * b[28] + a[28] * b[20]), fmaf(-0.17132745683193207f, (a[18] * b[30] + a[30] * b[18]), fmaf(0.09932258725166321f, (a[15] * b[19] + a[19] * b[15]), fmaf(-0.04441840946674347f, (a[12] * b[18] + a[18] * b[12]), fmaf(-0.17951487004756927f, (a[10] * b[20] + a[20] * b[10]), fmaf(0.17931121587753296f, (a[7] * b[27] + a[27] * b[7]), fmaf(-0.17931121587753296f, (a[5] * b[33] + a[33] * b[5]), fmaf(-0.19018827378749847f, (a[4] * b[34] + a[34] * b[4]), fmaf(0.1994711458683014f, (a[3] * b[17] + a[17] * b[3]), -0.1994711458683014f * (a[1] * b[23] + a[23] * b[1])))))))))))));
-        o[11] = ((fmaf(-0.1199292242527008f, (a[24] * b[27] + a[27] * b[24]), fmaf(-0.07518995553255081f, (a[22] * b[29] + a[29] * b[22]), fmaf(-0.1046828031539917f, (a[19] * b[32] + a[32] * b[19]), fmaf(-0.0299823060631752f, (a[17] * b[34] + a[34] * b[17]), fmaf(-0.1332552284002304f, (a[15] * b[18] + a[18] * b[15]), fmaf(0.11468784511089325f, (a[13] * b[18] + a[18] * b[13]), fmaf(-0.06785023957490921f, (a[10] * b[23] + a[23] * b[10]), fmaf(0.06562118977308273f, (a[8] * b[29] + a[29] * b[8]), fmaf(0.17361734807491302f, (a[7] * b[28] + a[28] * b[7]), fmaf(-0.17361734807491302f, (a[5] * b[32] + a[32] * b[5]), fmaf(-0.14175796508789062f, (a[4] * b[33] + a[33] * b[4]), fmaf(0.16858388483524323f, (a[3] * b[18] + a[18] * b[3]), fmaf(-0.16858388483524323f, (a[1] * b[22] + a[22] * b[1]), 0.282094806432724f * (a[0] * b[11] + a[11] * b[0])))))))))))))) + fmaf(0.0299823060631752f, (a[23] * b[26] + a[26] * b[23]), fmaf(0.08601991832256317f, (a[20] * b[29] + a[29] * b[20]), fmaf(0.07518995553255081f, (a[18] * b[31] + a[31] * b[18]), fmaf(0.1199292242527008f, (a[16] * b[33] + a[33] * b[16]), fmaf(0.06785023957490921f, (a[14] * b[17] + a[17] * b[14]), fmaf(0.025644980370998383f, (a[11] * b[20] + a[20] * b[11]), fmaf(0.1332552284002304f, (a[9] * b[22] + a[22] * b[9]), fmaf(-0.09403159469366074f, (a[8] * b[9] + a[9] * b[8]), fmaf(0.12615662813186646f, (a[6] * b[11] + a[11] * b[6]), fmaf(0.059470802545547485f, (a[5] * b[12] + a[12] * b[5]), fmaf(0.14567312598228455f, (a[4] * b[13] + a[13] * b[4]), fmaf(0.23359668254852295f, (a[2] * b[5] + a[5] * b[2]), 0.20230065286159515f * (a[1] * b[6] + a[6] * b[1])))))))))))))) + (fmaf(-0.12117204070091248f, (a[23] * b[28] + a[28] * b[23]), fmaf(0.1046828031539917f, (a[21] * b[28] + a[28] * b[21]), fmaf(-0.1019902154803276f, (a[18] * b[33] + a[33] * b[18]), fmaf(0.13408493995666504f, (a[16] * b[35] + a[35] * b[16]), fmaf(-0.10257992148399353f, (a[14] * b[19] + a[19] * b[14]), fmaf(-0.11468784511089325f, (a[11] * b[22] + a[22] * b[11]), fmaf(0.11752006411552429f, (a[9] * b[24] + a[24] * b[9]), fmaf(-0.14567312598228455f, (a[8] * b[11] + a[11] * b[8]), fmaf(0.22731846570968628f, (a[6] * b[29] + a[29] * b[6]), fmaf(-0.11516471952199936f, (a[5] * b[14] + a[14] * b[5]), fmaf(0.09403159469366074f, (a[4] * b[15] + a[15] * b[4]), fmaf(0.23841361701488495f, (a[2] * b[19] + a[19] * b[2]), 0.05839917063713074f * (a[1] * b[8] + a[8] * b[1]))))))))))))) + fmaf(-0.13408493995666504f, (a[24] * b[25] + a[25] * b[24]), fmaf(0.1019902154803276f, (a[22] * b[27] + a[27] * b[22]), fmaf(0.009577495977282524f, (a[19] * b[30] + a[30] * b[19]), fmaf(0.12117204070091248f, (a[17] * b[32] + a[32] * b[17]), fmaf(-0.11752006411552429f, (a[15] * b[16] + a[16] * b[15]), fmaf(0.09932258725166321f, (a[12] * b[19] + a[19] * b[12]), fmaf(0.10257992148399353f, (a[10] * b[21] + a[21] * b[10]), fmaf(0.14175796508789062f, (a[8] * b[27] + a[27] * b[8]), fmaf(0.11516471952199936f, (a[7] * b[10] + a[10] * b[7]), fmaf(-0.16943317651748657f, (a[5] * b[30] + a[30] * b[5]), fmaf(-0.06562118977308273f, (a[4] * b[31] + a[31] * b[4]), fmaf(-0.05839917063713074f, (a[3] * b[4] + a[4] * b[3]), -0.15078601241111755f * (a[1] * b[20] + a[20] * b[1])))))))))))))));
-        o[12] = ((fmaf(-0.2077234983444214f, (a[24] * b[34] + a[34] * b[24]), fmaf(0.14837393164634705f, (a[20] * b[30] + a[30] * b[20]), fmaf(-0.2077234983444214f, (a[16] * b[26] + a[26] * b[16]), fmaf(0.1538698822259903f, (a[12] * b[20] + a[20] * b[12]), fmaf(0.14175796508789062f, (a[8] * b[32] + a[32] * b[8]), fmaf(0.23961469531059265f, (a[6] * b[30] + a[30] * b[6]), fmaf(0.14175796508789062f, (a[4] * b[28] + a[28] * b[4]), fmaf(0.2462325245141983f, (a[2] * b[20] + a[20] * b[2]), 0.282094806432724f * (a[0] * b[12] + a[12] * b[0]))))))))) + fmaf(0.11508946865797043f, (a[21] * b[31] + a[31] * b[21]), fmaf(-0.1038617491722107f, (a[17] * b[27] + a[27] * b[17]), fmaf(0.09932258725166321f, (a[13] * b[21] + a[21] * b[13]), fmaf(-0.20355072617530823f, (a[9] * b[17] + a[17] * b[9]), fmaf(0.059470802545547485f, (a[7] * b[13] + a[13] * b[7]), fmaf(0.059470802545547485f, (a[5] * b[11] + a[11] * b[5]), fmaf(-0.14304816722869873f, (a[3] * b[7] + a[7] * b[3]), -0.14304816722869873f * (a[1] * b[5] + a[5] * b[1]))))))))) + (fmaf(0.022664492949843407f, (a[22] * b[32] + a[32] * b[22]), fmaf(0.022664492949843407f, (a[18] * b[28] + a[28] * b[18]), fmaf(-0.04441840946674347f, (a[14] * b[22] + a[22] * b[14]), fmaf(-0.04441840946674347f, (a[10] * b[18] + a[18] * b[10]), fmaf(0.2143179029226303f, (a[7] * b[31] + a[31] * b[7]), fmaf(0.2143179029226303f, (a[5] * b[29] + a[29] * b[5]), fmaf(0.1946638971567154f, (a[3] * b[21] + a[21] * b[3]), 0.1946638971567154f * (a[1] * b[19] + a[19] * b[1])))))))) + fmaf(-0.1038617491722107f, (a[23] * b[33] + a[33] * b[23]), fmaf(0.11508946865797043f, (a[19] * b[29] + a[29] * b[19]), fmaf(-0.20355072617530823f, (a[15] * b[23] + a[23] * b[15]), fmaf(0.09932258725166321f, (a[11] * b[19] + a[19] * b[11]), fmaf(-0.18806318938732147f, (a[8] * b[14] + a[14] * b[8]), fmaf(0.16820883750915527f, (a[6] * b[12] + a[12] * b[6]), fmaf(-0.18806318938732147f, (a[4] * b[10] + a[10] * b[4]), 0.24776668846607208f * (a[2] * b[6] + a[6] * b[2]))))))))));
-        o[13] = ((fmaf(-0.13408493995666504f, (a[24] * b[35] + a[35] * b[24]), fmaf(0.1019902154803276f, (a[22] * b[33] + a[33] * b[22]), fmaf(0.08601991832256317f, (a[20] * b[31] + a[31] * b[20]), fmaf(0.12117204070091248f, (a[17] * b[28] + a[28] * b[17]), fmaf(-0.11752006411552429f, (a[15] * b[24] + a[24] * b[15]), fmaf(0.11468784511089325f, (a[13] * b[22] + a[22] * b[13]), fmaf(0.10257992148399353f, (a[10] * b[19] + a[19] * b[10]), fmaf(0.14175796508789062f, (a[8] * b[33] + a[33] * b[8]), fmaf(0.17361734807491302f, (a[7] * b[32] + a[32] * b[7]), fmaf(0.22731846570968628f, (a[6] * b[31] + a[31] * b[6]), fmaf(-0.06562118977308273f, (a[4] * b[29] + a[29] * b[4]), fmaf(0.16858388483524323f, (a[3] * b[22] + a[22] * b[3]), fmaf(0.23841361701488495f, (a[2] * b[21] + a[21] * b[2]), 0.282094806432724f * (a[0] * b[13] + a[13] * b[0])))))))))))))) + fmaf(0.12117204070091248f, (a[23] * b[32] + a[32] * b[23]), fmaf(0.009577495977282524f, (a[21] * b[30] + a[30] * b[21]), fmaf(0.1019902154803276f, (a[18] * b[27] + a[27] * b[18]), fmaf(-0.13408493995666504f, (a[16] * b[25] + a[25] * b[16]), fmaf(0.10257992148399353f, (a[14] * b[21] + a[21] * b[14]), fmaf(0.11468784511089325f, (a[11] * b[18] + a[18] * b[11]), fmaf(-0.11752006411552429f, (a[9] * b[16] + a[16] * b[9]), fmaf(0.14567312598228455f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.059470802545547485f, (a[7] * b[12] + a[12] * b[7]), fmaf(0.11516471952199936f, (a[5] * b[10] + a[10] * b[5]), fmaf(-0.09403159469366074f, (a[4] * b[9] + a[9] * b[4]), fmaf(0.20230065286159515f, (a[3] * b[6] + a[6] * b[3]), -0.05839917063713074f * (a[1] * b[4] + a[4] * b[1])))))))))))))) + (fmaf(0.0299823060631752f, (a[23] * b[34] + a[34] * b[23]), fmaf(0.1046828031539917f, (a[21] * b[32] + a[32] * b[21]), fmaf(0.07518995553255081f, (a[18] * b[29] + a[29] * b[18]), fmaf(0.1199292242527008f, (a[16] * b[27] + a[27] * b[16]), fmaf(0.06785023957490921f, (a[14] * b[23] + a[23] * b[14]), fmaf(0.09932258725166321f, (a[12] * b[21] + a[21] * b[12]), fmaf(0.1332552284002304f, (a[9] * b[18] + a[18] * b[9]), fmaf(-0.09403159469366074f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.11516471952199936f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.17361734807491302f, (a[5] * b[28] + a[28] * b[5]), fmaf(0.14567312598228455f, (a[4] * b[11] + a[11] * b[4]), fmaf(-0.05839917063713074f, (a[3] * b[8] + a[8] * b[3]), 0.16858388483524323f * (a[1] * b[18] + a[18] * b[1]))))))))))))) + fmaf(0.1199292242527008f, (a[24] * b[33] + a[33] * b[24]), fmaf(0.07518995553255081f, (a[22] * b[31] + a[31] * b[22]), fmaf(0.1046828031539917f, (a[19] * b[28] + a[28] * b[19]), fmaf(0.0299823060631752f, (a[17] * b[26] + a[26] * b[17]), fmaf(0.1332552284002304f, (a[15] * b[22] + a[22] * b[15]), fmaf(0.025644980370998383f, (a[13] * b[20] + a[20] * b[13]), fmaf(0.06785023957490921f, (a[10] * b[17] + a[17] * b[10]), fmaf(-0.06562118977308273f, (a[8] * b[31] + a[31] * b[8]), fmaf(-0.16943317651748657f, (a[7] * b[30] + a[30] * b[7]), fmaf(0.12615662813186646f, (a[6] * b[13] + a[13] * b[6]), fmaf(0.14175796508789062f, (a[4] * b[27] + a[27] * b[4]), fmaf(-0.15078601241111755f, (a[3] * b[20] + a[20] * b[3]), 0.23359668254852295f * (a[2] * b[7] + a[7] * b[2])))))))))))))));
-        o[14] = ((fmaf(0.1499115228652954f, (a[23] * b[35] + a[35] * b[23]), fmaf(0.025339672341942787f, (a[21] * b[33] + a[33] * b[21]), fmaf(0.025339672341942787f, (a[19] * b[27] + a[27] * b[19]), fmaf(-0.07741397619247437f, (a[16] * b[28] + a[28] * b[16]), fmaf(0.06785023957490921f, (a[13] * b[23] + a[23] * b[13]), fmaf(0.06785023957490921f, (a[11] * b[17] + a[17] * b[11]), fmaf(0.05357947573065758f, (a[8] * b[30] + a[30] * b[8]), fmaf(0.1486770063638687f, (a[7] * b[15] + a[15] * b[7]), fmaf(0.17931121587753296f, (a[5] * b[27] + a[27] * b[5]), fmaf(0.1994711458683014f, (a[3] * b[23] + a[23] * b[3]), fmaf(0.18467439711093903f, (a[2] * b[8] + a[8] * b[2]), 0.282094806432724f * (a[0] * b[14] + a[14] * b[0])))))))))))) + fmaf(-0.07741397619247437f, (a[24] * b[32] + a[32] * b[24]), fmaf(-0.17132745683193207f, (a[22] * b[30] + a[30] * b[22]), fmaf(-0.09774991124868393f, (a[19] * b[29] + a[29] * b[19]), fmaf(0.1499115228652954f, (a[17] * b[25] + a[25] * b[17]), fmaf(-0.17951487004756927f, (a[14] * b[20] + a[20] * b[14]), fmaf(-0.10257992148399353f, (a[11] * b[19] + a[19] * b[11]), fmaf(0.19018827378749847f, (a[8] * b[34] + a[34] * b[8]), fmaf(-0.08300496637821198f, (a[7] * b[31] + a[31] * b[7]), fmaf(0.08300496637821198f, (a[5] * b[29] + a[29] * b[5]), fmaf(0.19018827378749847f, (a[4] * b[26] + a[26] * b[4]), fmaf(0.21324361860752106f, (a[2] * b[22] + a[22] * b[2]), -0.18467439711093903f * (a[1] * b[5] + a[5] * b[1]))))))))))))) + (fmaf(0.10135868936777115f, (a[22] * b[34] + a[34] * b[22]), fmaf(-0.06542675197124481f, (a[20] * b[32] + a[32] * b[20]), fmaf(-0.11379365622997284f, (a[17] * b[29] + a[29] * b[17]), fmaf(0.15171775221824646f, (a[14] * b[24] + a[24] * b[14]), fmaf(-0.04441840946674347f, (a[12] * b[22] + a[22] * b[12]), fmaf(-0.09932258725166321f, (a[9] * b[19] + a[19] * b[9]), fmaf(0.17931121587753296f, (a[7] * b[33] + a[33] * b[7]), fmaf(0.19018827378749847f, (a[6] * b[32] + a[32] * b[6]), fmaf(0.1486770063638687f, (a[5] * b[9] + a[9] * b[5]), fmaf(0.18467439711093903f, (a[3] * b[7] + a[7] * b[3]), 0.1994711458683014f * (a[1] * b[17] + a[17] * b[1]))))))))))) + fmaf(-0.11379365622997284f, (a[23] * b[31] + a[31] * b[23]), fmaf(0.09774991124868393f, (a[21] * b[31] + a[31] * b[21]), fmaf(0.10135868936777115f, (a[18] * b[26] + a[26] * b[18]), fmaf(-0.09932258725166321f, (a[15] * b[21] + a[21] * b[15]), fmaf(0.10257992148399353f, (a[13] * b[21] + a[21] * b[13]), fmaf(0.15171775221824646f, (a[10] * b[16] + a[16] * b[10]), fmaf(-0.18806318938732147f, (a[8] * b[12] + a[12] * b[8]), fmaf(0.11516471952199936f, (a[7] * b[13] + a[13] * b[7]), fmaf(-0.11516471952199936f, (a[5] * b[11] + a[11] * b[5]), fmaf(-0.07539300620555878f, (a[3] * b[21] + a[21] * b[3]), 0.07539300620555878f * (a[1] * b[19] + a[19] * b[1])))))))))))));
-        o[15] = ((fmaf(0.09814012795686722f, (a[23] * b[30] + a[30] * b[23]), fmaf(0.1266983598470688f, (a[21] * b[32] + a[32] * b[21]), fmaf(0.10158468782901764f, (a[18] * b[29] + a[29] * b[18]), fmaf(-0.09932258725166321f, (a[14] * b[21] + a[21] * b[14]), fmaf(-0.1332552284002304f, (a[11] * b[18] + a[18] * b[11]), fmaf(0.016943316906690598f, (a[8] * b[31] + a[31] * b[8]), fmaf(0.1486770063638687f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.15528807044029236f, (a[5] * b[26] + a[26] * b[5]), fmaf(0.09403159469366074f, (a[4] * b[11] + a[11] * b[4]), fmaf(0.1628675013780594f, (a[2] * b[23] + a[23] * b[2]), 0.282094806432724f * (a[0] * b[15] + a[15] * b[0]))))))))))) + fmaf(0.03583570942282677f, (a[24] * b[31] + a[31] * b[24]), fmaf(-0.1316688060760498f, (a[21] * b[34] + a[34] * b[21]), fmaf(-0.1316688060760498f, (a[19] * b[26] + a[26] * b[19]), fmaf(0.07693494111299515f, (a[15] * b[20] + a[20] * b[15]), fmaf(-0.20355072617530823f, (a[12] * b[23] + a[23] * b[12]), fmaf(0.24553200602531433f, (a[8] * b[35] + a[35] * b[8]), fmaf(-0.04482780396938324f, (a[7] * b[32] + a[32] * b[7]), fmaf(0.04482780396938324f, (a[5] * b[28] + a[28] * b[5]), fmaf(0.24553200602531433f, (a[4] * b[25] + a[25] * b[4]), fmaf(0.22617901861667633f, (a[3] * b[8] + a[8] * b[3]), -0.22617901861667633f * (a[1] * b[4] + a[4] * b[1])))))))))))) + (fmaf(-0.10158468782901764f, (a[22] * b[31] + a[31] * b[22]), fmaf(-0.1266983598470688f, (a[19] * b[28] + a[28] * b[19]), fmaf(0.03583570942282677f, (a[16] * b[29] + a[29] * b[16]), fmaf(0.1332552284002304f, (a[13] * b[22] + a[22] * b[13]), fmaf(0.09932258725166321f, (a[10] * b[19] + a[19] * b[10]), fmaf(0.15528807044029236f, (a[7] * b[34] + a[34] * b[7]), fmaf(-0.2102610468864441f, (a[6] * b[15] + a[15] * b[6]), fmaf(-0.016943316906690598f, (a[4] * b[29] + a[29] * b[4]), fmaf(-0.04352817311882973f, (a[3] * b[22] + a[22] * b[3]), 0.23032943904399872f * (a[1] * b[16] + a[16] * b[1])))))))))) + fmaf(-0.09814012795686722f, (a[22] * b[35] + a[35] * b[22]), fmaf(-0.19628025591373444f, (a[20] * b[33] + a[33] * b[20]), fmaf(-0.09814012795686722f, (a[18] * b[25] + a[25] * b[18]), fmaf(-0.11752006411552429f, (a[13] * b[24] + a[24] * b[13]), fmaf(-0.11752006411552429f, (a[11] * b[16] + a[16] * b[11]), fmaf(-0.09403159469366074f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.12679217755794525f, (a[6] * b[33] + a[33] * b[6]), fmaf(-0.1486770063638687f, (a[5] * b[10] + a[10] * b[5]), fmaf(0.23032943904399872f, (a[3] * b[24] + a[24] * b[3]), 0.04352817311882973f * (a[1] * b[18] + a[18] * b[1]))))))))))));
-        o[16] = ((fmaf(-0.1188535988330841f, (a[27] * b[31] + a[31] * b[27]), fmaf(0.13504546880722046f, (a[18] * b[22] + a[22] * b[18]), fmaf(-0.07741397619247437f, (a[14] * b[28] + a[28] * b[14]), fmaf(0.13408493995666504f, (a[11] * b[35] + a[35] * b[11]), fmaf(0.15171775221824646f, (a[10] * b[14] + a[14] * b[10]), fmaf(0.14046335220336914f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.23841361701488495f, (a[4] * b[8] + a[8] * b[4]), fmaf(0.14731919765472412f, (a[2] * b[26] + a[26] * b[2]), 0.282094806432724f * (a[0] * b[16] + a[16] * b[0]))))))))) + fmaf(0.1283765584230423f, (a[28] * b[32] + a[32] * b[28]), fmaf(-0.11909890919923782f, (a[19] * b[23] + a[23] * b[19]), fmaf(0.03583570942282677f, (a[15] * b[29] + a[29] * b[15]), fmaf(-0.2077234983444214f, (a[12] * b[26] + a[26] * b[12]), fmaf(-0.07741397619247437f, (a[10] * b[32] + a[32] * b[10]), fmaf(-0.07508081942796707f, (a[8] * b[18] + a[18] * b[8]), fmaf(-0.07508081942796707f, (a[4] * b[22] + a[22] * b[4]), fmaf(0.23032943904399872f, (a[3] * b[9] + a[9] * b[3]), 0.23032943904399872f * (a[1] * b[15] + a[15] * b[1])))))))))) + (fmaf(-0.1188535988330841f, (a[29] * b[33] + a[33] * b[29]), fmaf(0.05315294489264488f, (a[25] * b[31] + a[31] * b[25]), fmaf(0.10652530938386917f, (a[16] * b[20] + a[20] * b[16]), fmaf(-0.13408493995666504f, (a[13] * b[25] + a[25] * b[13]), fmaf(-0.11752006411552429f, (a[11] * b[15] + a[15] * b[11]), fmaf(-0.11752006411552429f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.14046335220336914f, (a[5] * b[23] + a[23] * b[5]), fmaf(0.23293210566043854f, (a[3] * b[25] + a[25] * b[3]), -0.034723468124866486f * (a[1] * b[33] + a[33] * b[1]))))))))) + fmaf(-0.05315294489264488f, (a[29] * b[35] + a[35] * b[29]), fmaf(0.13019759953022003f, (a[26] * b[30] + a[30] * b[26]), fmaf(-0.11909890919923782f, (a[17] * b[21] + a[21] * b[17]), fmaf(0.1199292242527008f, (a[13] * b[27] + a[27] * b[13]), fmaf(0.1199292242527008f, (a[11] * b[33] + a[33] * b[11]), fmaf(0.03583570942282677f, (a[9] * b[31] + a[31] * b[9]), fmaf(-0.2293756902217865f, (a[6] * b[16] + a[16] * b[6]), fmaf(-0.034723468124866486f, (a[3] * b[27] + a[27] * b[3]), -0.23293210566043854f * (a[1] * b[35] + a[35] * b[1])))))))))));
-        o[17] = ((fmaf(0.09944005310535431f, (a[28] * b[35] + a[35] * b[28]), fmaf(-0.09944005310535431f, (a[25] * b[32] + a[32] * b[25]), fmaf(-0.15978795289993286f, (a[17] * b[20] + a[20] * b[17]), fmaf(0.12117204070091248f, (a[13] * b[28] + a[28] * b[13]), fmaf(0.12117204070091248f, (a[11] * b[32] + a[32] * b[11]), fmaf(0.06785023957490921f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.13272538781166077f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.13272538781166077f, (a[5] * b[22] + a[22] * b[5]), fmaf(-0.06014281138777733f, (a[3] * b[28] + a[28] * b[3]), fmaf(0.1628675013780594f, (a[2] * b[9] + a[9] * b[2]), 0.282094806432724f * (a[0] * b[17] + a[17] * b[0]))))))))))) + fmaf(0.034310080111026764f, (a[29] * b[32] + a[32] * b[29]), fmaf(-0.1188535988330841f, (a[26] * b[31] + a[31] * b[26]), fmaf(0.045015156269073486f, (a[18] * b[21] + a[21] * b[18]), fmaf(0.1499115228652954f, (a[14] * b[25] + a[25] * b[14]), fmaf(-0.0299823060631752f, (a[11] * b[34] + a[34] * b[11]), fmaf(-0.11379365622997284f, (a[10] * b[31] + a[31] * b[10]), fmaf(-0.11262122541666031f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[24] + a[24] * b[5]), fmaf(0.16858388483524323f, (a[4] * b[7] + a[7] * b[4]), fmaf(0.19642560184001923f, (a[2] * b[27] + a[27] * b[2]), 0.1994711458683014f * (a[1] * b[14] + a[14] * b[1])))))))))))) + (fmaf(0.1188535988330841f, (a[29] * b[34] + a[34] * b[29]), fmaf(-0.13019759953022003f, (a[27] * b[30] + a[30] * b[27]), fmaf(0.045015156269073486f, (a[19] * b[22] + a[22] * b[19]), fmaf(-0.11379365622997284f, (a[14] * b[29] + a[29] * b[14]), fmaf(-0.1038617491722107f, (a[12] * b[27] + a[27] * b[12]), fmaf(-0.1499115228652954f, (a[10] * b[35] + a[35] * b[10]), fmaf(-0.20355072617530823f, (a[9] * b[12] + a[12] * b[9]), fmaf(-0.057343922555446625f, (a[6] * b[17] + a[17] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[21] + a[21] * b[4]), fmaf(0.1994711458683014f, (a[3] * b[10] + a[10] * b[3]), -0.06014281138777733f * (a[1] * b[32] + a[32] * b[1]))))))))))) + fmaf(0.034310080111026764f, (a[28] * b[31] + a[31] * b[28]), fmaf(0.11909890919923782f, (a[19] * b[24] + a[24] * b[19]), fmaf(-0.11909890919923782f, (a[16] * b[21] + a[21] * b[16]), fmaf(0.0299823060631752f, (a[13] * b[26] + a[26] * b[13]), fmaf(0.06785023957490921f, (a[11] * b[14] + a[14] * b[11]), fmaf(0.09814012795686722f, (a[9] * b[30] + a[30] * b[9]), fmaf(0.14046335220336914f, (a[7] * b[16] + a[16] * b[7]), fmaf(0.16858388483524323f, (a[5] * b[8] + a[8] * b[5]), fmaf(0.2083408087491989f, (a[3] * b[26] + a[26] * b[3]), -0.2083408087491989f * (a[1] * b[34] + a[34] * b[1]))))))))))));
-        o[18] = ((fmaf(0.09704355895519257f, (a[29] * b[31] + a[31] * b[29]), fmaf(0.08404218405485153f, (a[26] * b[32] + a[32] * b[26]), fmaf(-0.13504546880722046f, (a[18] * b[24] + a[24] * b[18]), fmaf(0.10158468782901764f, (a[15] * b[29] + a[29] * b[15]), fmaf(0.1019902154803276f, (a[13] * b[27] + a[27] * b[13]), fmaf(-0.1332552284002304f, (a[11] * b[15] + a[15] * b[11]), fmaf(-0.04441840946674347f, (a[10] * b[12] + a[12] * b[10]), fmaf(-0.07508081942796707f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.13272538781166077f, (a[5] * b[23] + a[23] * b[5]), fmaf(-0.19036461412906647f, (a[4] * b[20] + a[20] * b[4]), fmaf(0.16858388483524323f, (a[3] * b[11] + a[11] * b[3]), fmaf(-0.1837393194437027f, (a[1] * b[33] + a[33] * b[1]), 0.282094806432724f * (a[0] * b[18] + a[18] * b[0]))))))))))))) + fmaf(-0.13019759953022003f, (a[27] * b[35] + a[35] * b[27]), fmaf(0.10208478569984436f, (a[19] * b[21] + a[21] * b[19]), fmaf(0.13504546880722046f, (a[16] * b[22] + a[22] * b[16]), fmaf(0.07518995553255081f, (a[13] * b[29] + a[29] * b[13]), fmaf(0.07518995553255081f, (a[11] * b[31] + a[31] * b[11]), fmaf(-0.17132745683193207f, (a[10] * b[30] + a[30] * b[10]), fmaf(0.1332552284002304f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.06553591042757034f, (a[6] * b[18] + a[18] * b[6]), fmaf(0.07508081942796707f, (a[4] * b[24] + a[24] * b[4]), fmaf(0.1837393194437027f, (a[3] * b[27] + a[27] * b[3]), fmaf(0.21324361860752106f, (a[2] * b[10] + a[10] * b[2]), 0.16858388483524323f * (a[1] * b[13] + a[13] * b[1]))))))))))))) + (fmaf(-0.09944005310535431f, (a[28] * b[30] + a[30] * b[28]), fmaf(-0.045015156269073486f, (a[19] * b[23] + a[23] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[21] + a[21] * b[17]), fmaf(0.10135868936777115f, (a[14] * b[26] + a[26] * b[14]), fmaf(-0.1019902154803276f, (a[11] * b[33] + a[33] * b[11]), fmaf(-0.10135868936777115f, (a[10] * b[34] + a[34] * b[10]), fmaf(-0.10158468782901764f, (a[9] * b[31] + a[31] * b[9]), fmaf(0.13272538781166077f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.180223748087883f, (a[5] * b[7] + a[7] * b[5]), fmaf(-0.08505477756261826f, (a[3] * b[29] + a[29] * b[3]), fmaf(0.22503378987312317f, (a[2] * b[28] + a[28] * b[2]), 0.04352817311882973f * (a[1] * b[15] + a[15] * b[1])))))))))))) + fmaf(-0.08404218405485153f, (a[28] * b[34] + a[34] * b[28]), fmaf(0.13019759953022003f, (a[25] * b[33] + a[33] * b[25]), fmaf(-0.08369845151901245f, (a[18] * b[20] + a[20] * b[18]), fmaf(-0.09814012795686722f, (a[15] * b[25] + a[25] * b[15]), fmaf(0.022664492949843407f, (a[12] * b[28] + a[28] * b[12]), fmaf(0.11468784511089325f, (a[11] * b[13] + a[13] * b[11]), fmaf(0.09814012795686722f, (a[9] * b[35] + a[35] * b[9]), fmaf(0.09029786288738251f, (a[7] * b[19] + a[19] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[21] + a[21] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[6] + a[6] * b[4]), fmaf(-0.04352817311882973f, (a[3] * b[9] + a[9] * b[3]), -0.08505477756261826f * (a[1] * b[31] + a[31] * b[1]))))))))))))));
-        o[19] = ((fmaf(-0.08404218405485153f, (a[28] * b[33] + a[33] * b[28]), fmaf(-0.13019759953022003f, (a[25] * b[34] + a[34] * b[25]), fmaf(0.10208478569984436f, (a[18] * b[21] + a[21] * b[18]), fmaf(-0.1266983598470688f, (a[15] * b[28] + a[28] * b[15]), fmaf(0.1046828031539917f, (a[13] * b[28] + a[28] * b[13]), fmaf(-0.10257992148399353f, (a[11] * b[14] + a[14] * b[11]), fmaf(0.09932258725166321f, (a[10] * b[15] + a[15] * b[10]), fmaf(-0.09932258725166321f, (a[9] * b[14] + a[14] * b[9]), fmaf(0.1392638087272644f, (a[6] * b[19] + a[19] * b[6]), fmaf(0.22072811424732208f, (a[5] * b[6] + a[6] * b[5]), fmaf(0.15912292897701263f, (a[3] * b[28] + a[28] * b[3]), fmaf(-0.15912292897701263f, (a[1] * b[32] + a[32] * b[1]), 0.282094806432724f * (a[0] * b[19] + a[19] * b[0]))))))))))))) + fmaf(0.05315294489264488f, (a[29] * b[30] + a[30] * b[29]), fmaf(0.13019759953022003f, (a[26] * b[35] + a[35] * b[26]), fmaf(-0.045015156269073486f, (a[18] * b[23] + a[23] * b[18]), fmaf(-0.11909890919923782f, (a[16] * b[23] + a[23] * b[16]), fmaf(0.025339672341942787f, (a[14] * b[27] + a[27] * b[14]), fmaf(0.009577495977282524f, (a[11] * b[30] + a[30] * b[11]), fmaf(0.09774991124868393f, (a[10] * b[31] + a[31] * b[10]), fmaf(0.1266983598470688f, (a[9] * b[32] + a[32] * b[9]), fmaf(0.09029786288738251f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.06371872127056122f, (a[5] * b[8] + a[8] * b[5]), fmaf(-0.06371872127056122f, (a[4] * b[7] + a[7] * b[4]), fmaf(0.23841361701488495f, (a[2] * b[11] + a[11] * b[2]), 0.1946638971567154f * (a[1] * b[12] + a[12] * b[1])))))))))))))) + (fmaf(-0.09077593684196472f, (a[29] * b[32] + a[32] * b[29]), fmaf(0.08404218405485153f, (a[27] * b[32] + a[32] * b[27]), fmaf(0.06848055124282837f, (a[19] * b[20] + a[20] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[22] + a[22] * b[17]), fmaf(-0.09774991124868393f, (a[14] * b[29] + a[29] * b[14]), fmaf(-0.1046828031539917f, (a[11] * b[32] + a[32] * b[11]), fmaf(-0.025339672341942787f, (a[10] * b[33] + a[33] * b[10]), fmaf(0.1316688060760498f, (a[9] * b[34] + a[34] * b[9]), fmaf(-0.11262122541666031f, (a[8] * b[17] + a[17] * b[8]), fmaf(0.04486937075853348f, (a[5] * b[20] + a[20] * b[5]), fmaf(0.14188940823078156f, (a[4] * b[21] + a[21] * b[4]), fmaf(0.24057124555110931f, (a[2] * b[29] + a[29] * b[2]), 0.07539300620555878f * (a[1] * b[14] + a[14] * b[1]))))))))))))) + fmaf(0.09077593684196472f, (a[28] * b[31] + a[31] * b[28]), fmaf(-0.10208478569984436f, (a[19] * b[22] + a[22] * b[19]), fmaf(0.11909890919923782f, (a[17] * b[24] + a[24] * b[17]), fmaf(-0.1316688060760498f, (a[15] * b[26] + a[26] * b[15]), fmaf(0.11508946865797043f, (a[12] * b[29] + a[29] * b[12]), fmaf(0.09932258725166321f, (a[11] * b[12] + a[12] * b[11]), fmaf(0.10257992148399353f, (a[10] * b[13] + a[13] * b[10]), fmaf(-0.14188940823078156f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.09029786288738251f, (a[5] * b[22] + a[22] * b[5]), fmaf(0.11262122541666031f, (a[4] * b[23] + a[23] * b[4]), fmaf(-0.07539300620555878f, (a[3] * b[10] + a[10] * b[3]), -0.15528807044029236f * (a[1] * b[30] + a[30] * b[1]))))))))))))));
-        o[20] = ((fmaf(-0.13019759953022003f, a[33] * b[33], fmaf(0.08679839968681335f, a[29] * b[29], fmaf(0.13019759953022003f, a[25] * b[25], fmaf(0.06848055124282837f, a[21] * b[21], fmaf(-0.15978795289993286f, a[17] * b[17], fmaf(-0.06542675197124481f, (a[14] * b[32] + a[32] * b[14]), fmaf(0.14837393164634705f, (a[12] * b[30] + a[30] * b[12]), fmaf(-0.06542675197124481f, (a[10] * b[28] + a[28] * b[10]), fmaf(-0.19036461412906647f, (a[8] * b[22] + a[22] * b[8]), fmaf(0.16383977234363556f, (a[6] * b[20] + a[20] * b[6]), fmaf(-0.19036461412906647f, (a[4] * b[18] + a[18] * b[4]), fmaf(0.24553200602531433f, (a[2] * b[30] + a[30] * b[2]), 0.282094806432724f * (a[0] * b[20] + a[20] * b[0]))))))))))))) + fmaf(-0.13019759953022003f, a[34] * b[34], fmaf(0.13019759953022003f, a[30] * b[30], fmaf(-0.13019759953022003f, a[26] * b[26], fmaf(-0.08369845151901245f, a[22] * b[22], fmaf(-0.08369845151901245f, a[18] * b[18], fmaf(0.07693494111299515f, a[15] * b[15], fmaf(0.025644980370998383f, a[13] * b[13], fmaf(0.025644980370998383f, a[11] * b[11], fmaf(0.07693494111299515f, a[9] * b[9], fmaf(-0.1611970216035843f, a[7] * b[7], fmaf(-0.1611970216035843f, a[5] * b[5], fmaf(-0.15078601241111755f, (a[3] * b[13] + a[13] * b[3]), -0.15078601241111755f * (a[1] * b[11] + a[11] * b[1])))))))))))))) + (fmaf(0.13019759953022003f, a[35] * b[35], fmaf(0.08679839968681335f, a[31] * b[31], fmaf(-0.13019759953022003f, a[27] * b[27], fmaf(-0.15978795289993286f, a[23] * b[23], fmaf(0.06848055124282837f, a[19] * b[19], fmaf(-0.19628025591373444f, (a[15] * b[33] + a[33] * b[15]), fmaf(0.08601991832256317f, (a[13] * b[31] + a[31] * b[13]), fmaf(0.08601991832256317f, (a[11] * b[29] + a[29] * b[11]), fmaf(-0.19628025591373444f, (a[9] * b[27] + a[27] * b[9]), fmaf(0.04486937075853348f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.04486937075853348f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.19018827378749847f, (a[3] * b[31] + a[31] * b[3]), 0.19018827378749847f * (a[1] * b[29] + a[29] * b[1]))))))))))))) + fmaf(-0.02169959992170334f, a[32] * b[32], fmaf(-0.02169959992170334f, a[28] * b[28], fmaf(0.10652530938386917f, a[24] * b[24], fmaf(0.13696110248565674f, a[20] * b[20], fmaf(0.10652530938386917f, a[16] * b[16], fmaf(-0.17951487004756927f, a[14] * b[14], fmaf(0.1538698822259903f, a[12] * b[12], fmaf(-0.17951487004756927f, a[10] * b[10], fmaf(0.04029925540089607f, a[8] * b[8], fmaf(0.24179553985595703f, a[6] * b[6], fmaf(0.04029925540089607f, a[4] * b[4], 0.2462325245141983f * (a[2] * b[12] + a[12] * b[2]))))))))))))));
-        o[21] = ((fmaf(0.09077593684196472f, (a[31] * b[32] + a[32] * b[31]), fmaf(-0.13019759953022003f, (a[25] * b[26] + a[26] * b[25]), fmaf(0.06848055124282837f, (a[20] * b[21] + a[21] * b[20]), fmaf(-0.1316688060760498f, (a[15] * b[34] + a[34] * b[15]), fmaf(-0.09932258725166321f, (a[14] * b[15] + a[15] * b[14]), fmaf(0.11508946865797043f, (a[12] * b[31] + a[31] * b[12]), fmaf(0.025339672341942787f, (a[10] * b[27] + a[27] * b[10]), fmaf(-0.09932258725166321f, (a[9] * b[10] + a[10] * b[9]), fmaf(0.04486937075853348f, (a[7] * b[20] + a[20] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[18] + a[18] * b[5]), fmaf(0.15912292897701263f, (a[3] * b[32] + a[32] * b[3]), fmaf(0.24057124555110931f, (a[2] * b[31] + a[31] * b[2]), 0.282094806432724f * (a[0] * b[21] + a[21] * b[0]))))))))))))) + fmaf(0.08404218405485153f, (a[32] * b[33] + a[33] * b[32]), fmaf(0.08404218405485153f, (a[27] * b[28] + a[28] * b[27]), fmaf(0.10208478569984436f, (a[21] * b[22] + a[22] * b[21]), fmaf(-0.11909890919923782f, (a[16] * b[17] + a[17] * b[16]), fmaf(0.09774991124868393f, (a[14] * b[31] + a[31] * b[14]), fmaf(0.10257992148399353f, (a[13] * b[14] + a[14] * b[13]), fmaf(0.09774991124868393f, (a[10] * b[29] + a[29] * b[10]), fmaf(-0.1316688060760498f, (a[9] * b[26] + a[26] * b[9]), fmaf(0.09029786288738251f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.22072811424732208f, (a[6] * b[7] + a[7] * b[6]), fmaf(-0.06371872127056122f, (a[4] * b[5] + a[5] * b[4]), fmaf(0.1946638971567154f, (a[3] * b[12] + a[12] * b[3]), -0.07539300620555878f * (a[1] * b[10] + a[10] * b[1])))))))))))))) + (fmaf(-0.13019759953022003f, (a[34] * b[35] + a[35] * b[34]), fmaf(0.09077593684196472f, (a[28] * b[29] + a[29] * b[28]), fmaf(0.045015156269073486f, (a[22] * b[23] + a[23] * b[22]), fmaf(0.045015156269073486f, (a[17] * b[18] + a[18] * b[17]), fmaf(0.025339672341942787f, (a[14] * b[33] + a[33] * b[14]), fmaf(0.009577495977282524f, (a[13] * b[30] + a[30] * b[13]), fmaf(0.1046828031539917f, (a[11] * b[28] + a[28] * b[11]), fmaf(0.1266983598470688f, (a[9] * b[28] + a[28] * b[9]), fmaf(0.14188940823078156f, (a[8] * b[21] + a[21] * b[8]), fmaf(0.1392638087272644f, (a[6] * b[21] + a[21] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[17] + a[17] * b[4]), fmaf(-0.07539300620555878f, (a[3] * b[14] + a[14] * b[3]), 0.15912292897701263f * (a[1] * b[28] + a[28] * b[1]))))))))))))) + fmaf(0.05315294489264488f, (a[30] * b[31] + a[31] * b[30]), fmaf(-0.11909890919923782f, (a[23] * b[24] + a[24] * b[23]), fmaf(0.10208478569984436f, (a[18] * b[19] + a[19] * b[18]), fmaf(0.1266983598470688f, (a[15] * b[32] + a[32] * b[15]), fmaf(0.1046828031539917f, (a[13] * b[32] + a[32] * b[13]), fmaf(0.09932258725166321f, (a[12] * b[13] + a[13] * b[12]), fmaf(0.10257992148399353f, (a[10] * b[11] + a[11] * b[10]), fmaf(-0.11262122541666031f, (a[8] * b[23] + a[23] * b[8]), fmaf(-0.06371872127056122f, (a[7] * b[8] + a[8] * b[7]), fmaf(0.14188940823078156f, (a[4] * b[19] + a[19] * b[4]), fmaf(-0.15528807044029236f, (a[3] * b[30] + a[30] * b[3]), 0.23841361701488495f * (a[2] * b[13] + a[13] * b[2]))))))))))))));
-        o[22] = ((fmaf(0.13019759953022003f, (a[33] * b[35] + a[35] * b[33]), fmaf(-0.09704355895519257f, a[29] * b[29], fmaf(0.045015156269073486f, (a[21] * b[23] + a[23] * b[21]), fmaf(0.045015156269073486f, (a[17] * b[19] + a[19] * b[17]), fmaf(0.10135868936777115f, (a[14] * b[34] + a[34] * b[14]), fmaf(0.1332552284002304f, (a[13] * b[15] + a[15] * b[13]), fmaf(-0.07518995553255081f, (a[11] * b[29] + a[29] * b[11]), fmaf(-0.10158468782901764f, (a[9] * b[29] + a[29] * b[9]), fmaf(-0.19036461412906647f, (a[8] * b[20] + a[20] * b[8]), fmaf(0.06553591042757034f, (a[6] * b[22] + a[22] * b[6]), fmaf(-0.180223748087883f, a[5] * b[5], fmaf(-0.04352817311882973f, (a[3] * b[15] + a[15] * b[3]), fmaf(0.08505477756261826f, (a[1] * b[29] + a[29] * b[1]), 0.282094806432724f * (a[0] * b[22] + a[22] * b[0])))))))))))))) + fmaf(-0.09944005310535431f, (a[30] * b[32] + a[32] * b[30]), fmaf(0.13504546880722046f, (a[22] * b[24] + a[24] * b[22]), fmaf(-0.10208478569984436f, a[19] * b[19], fmaf(-0.10158468782901764f, (a[15] * b[31] + a[31] * b[15]), fmaf(0.07518995553255081f, (a[13] * b[31] + a[31] * b[13]), fmaf(-0.04441840946674347f, (a[12] * b[14] + a[14] * b[12]), fmaf(0.10135868936777115f, (a[10] * b[26] + a[26] * b[10]), fmaf(-0.07508081942796707f, (a[8] * b[24] + a[24] * b[8]), fmaf(0.180223748087883f, a[7] * b[7], fmaf(0.13272538781166077f, (a[5] * b[17] + a[17] * b[5]), fmaf(-0.08505477756261826f, (a[3] * b[31] + a[31] * b[3]), fmaf(0.21324361860752106f, (a[2] * b[14] + a[14] * b[2]), -0.04352817311882973f * (a[1] * b[9] + a[9] * b[1])))))))))))))) + (fmaf(0.09704355895519257f, a[31] * b[31], fmaf(0.13019759953022003f, (a[25] * b[27] + a[27] * b[25]), fmaf(-0.08369845151901245f, (a[20] * b[22] + a[22] * b[20]), fmaf(-0.09814012795686722f, (a[15] * b[35] + a[35] * b[15]), fmaf(0.1019902154803276f, (a[13] * b[33] + a[33] * b[13]), fmaf(0.022664492949843407f, (a[12] * b[32] + a[32] * b[12]), fmaf(-0.11468784511089325f, a[11] * b[11], fmaf(0.1332552284002304f, (a[9] * b[11] + a[11] * b[9]), fmaf(0.09029786288738251f, (a[7] * b[21] + a[21] * b[7]), fmaf(-0.09029786288738251f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.1837393194437027f, (a[3] * b[33] + a[33] * b[3]), fmaf(0.22503378987312317f, (a[2] * b[32] + a[32] * b[2]), -0.16858388483524323f * (a[1] * b[11] + a[11] * b[1]))))))))))))) + fmaf(0.08404218405485153f, (a[32] * b[34] + a[34] * b[32]), fmaf(0.08404218405485153f, (a[26] * b[28] + a[28] * b[26]), fmaf(0.10208478569984436f, a[21] * b[21], fmaf(0.13504546880722046f, (a[16] * b[18] + a[18] * b[16]), fmaf(-0.17132745683193207f, (a[14] * b[30] + a[30] * b[14]), fmaf(0.11468784511089325f, a[13] * b[13], fmaf(0.1019902154803276f, (a[11] * b[27] + a[27] * b[11]), fmaf(-0.09814012795686722f, (a[9] * b[25] + a[25] * b[9]), fmaf(0.13272538781166077f, (a[7] * b[23] + a[23] * b[7]), fmaf(0.15607835352420807f, (a[6] * b[8] + a[8] * b[6]), fmaf(-0.07508081942796707f, (a[4] * b[16] + a[16] * b[4]), fmaf(0.16858388483524323f, (a[3] * b[13] + a[13] * b[3]), 0.1837393194437027f * (a[1] * b[27] + a[27] * b[1])))))))))))))));
-        o[23] = ((fmaf(0.034310080111026764f, (a[31] * b[32] + a[32] * b[31]), fmaf(-0.09944005310535431f, (a[25] * b[28] + a[28] * b[25]), fmaf(-0.045015156269073486f, (a[18] * b[19] + a[19] * b[18]), fmaf(-0.11379365622997284f, (a[14] * b[31] + a[31] * b[14]), fmaf(-0.1038617491722107f, (a[12] * b[33] + a[33] * b[12]), fmaf(0.11379365622997284f, (a[10] * b[29] + a[29] * b[10]), fmaf(0.14046335220336914f, (a[7] * b[24] + a[24] * b[7]), fmaf(-0.13272538781166077f, (a[5] * b[18] + a[18] * b[5]), fmaf(0.2083408087491989f, (a[3] * b[34] + a[34] * b[3]), fmaf(0.1628675013780594f, (a[2] * b[15] + a[15] * b[2]), 0.282094806432724f * (a[0] * b[23] + a[23] * b[0]))))))))))) + fmaf(-0.1188535988330841f, (a[31] * b[34] + a[34] * b[31]), fmaf(-0.1188535988330841f, (a[26] * b[29] + a[29] * b[26]), fmaf(-0.15978795289993286f, (a[20] * b[23] + a[23] * b[20]), fmaf(0.1499115228652954f, (a[14] * b[35] + a[35] * b[14]), fmaf(0.06785023957490921f, (a[13] * b[14] + a[14] * b[13]), fmaf(0.0299823060631752f, (a[11] * b[26] + a[26] * b[11]), fmaf(-0.11262122541666031f, (a[8] * b[21] + a[21] * b[8]), fmaf(-0.057343922555446625f, (a[6] * b[23] + a[23] * b[6]), fmaf(-0.16858388483524323f, (a[4] * b[5] + a[5] * b[4]), fmaf(0.19642560184001923f, (a[2] * b[33] + a[33] * b[2]), -0.1994711458683014f * (a[1] * b[10] + a[10] * b[1])))))))))))) + (fmaf(-0.09944005310535431f, (a[32] * b[35] + a[35] * b[32]), fmaf(-0.034310080111026764f, (a[28] * b[29] + a[29] * b[28]), fmaf(0.045015156269073486f, (a[21] * b[22] + a[22] * b[21]), fmaf(0.09814012795686722f, (a[15] * b[30] + a[30] * b[15]), fmaf(0.12117204070091248f, (a[13] * b[32] + a[32] * b[13]), fmaf(-0.12117204070091248f, (a[11] * b[28] + a[28] * b[11]), fmaf(-0.06785023957490921f, (a[10] * b[11] + a[11] * b[10]), fmaf(0.16858388483524323f, (a[7] * b[8] + a[8] * b[7]), fmaf(0.11262122541666031f, (a[4] * b[19] + a[19] * b[4]), fmaf(0.1994711458683014f, (a[3] * b[14] + a[14] * b[3]), 0.2083408087491989f * (a[1] * b[26] + a[26] * b[1]))))))))))) + fmaf(-0.13019759953022003f, (a[30] * b[33] + a[33] * b[30]), fmaf(-0.11909890919923782f, (a[21] * b[24] + a[24] * b[21]), fmaf(-0.11909890919923782f, (a[16] * b[19] + a[19] * b[16]), fmaf(0.0299823060631752f, (a[13] * b[34] + a[34] * b[13]), fmaf(-0.20355072617530823f, (a[12] * b[15] + a[15] * b[12]), fmaf(0.1499115228652954f, (a[10] * b[25] + a[25] * b[10]), fmaf(0.13272538781166077f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.14046335220336914f, (a[5] * b[16] + a[16] * b[5]), fmaf(-0.06014281138777733f, (a[3] * b[32] + a[32] * b[3]), 0.06014281138777733f * (a[1] * b[28] + a[28] * b[1]))))))))))));
-        o[24] = ((fmaf(0.13019759953022003f, (a[30] * b[34] + a[34] * b[30]), fmaf(0.13504546880722046f, a[22] * b[22], fmaf(0.11909890919923782f, (a[17] * b[19] + a[19] * b[17]), fmaf(-0.13408493995666504f, (a[13] * b[35] + a[35] * b[13]), fmaf(-0.1199292242527008f, (a[11] * b[27] + a[27] * b[11]), fmaf(-0.03583570942282677f, (a[9] * b[29] + a[29] * b[9]), fmaf(0.14046335220336914f, (a[7] * b[23] + a[23] * b[7]), fmaf(-0.23841361701488495f, a[4] * b[4], fmaf(0.14731919765472412f, (a[2] * b[34] + a[34] * b[2]), 0.282094806432724f * (a[0] * b[24] + a[24] * b[0])))))))))) + fmaf(-0.1188535988330841f, (a[31] * b[33] + a[33] * b[31]), fmaf(0.05315294489264488f, (a[25] * b[29] + a[29] * b[25]), fmaf(-0.13504546880722046f, a[18] * b[18], fmaf(0.15171775221824646f, a[14] * b[14], fmaf(-0.2077234983444214f, (a[12] * b[34] + a[34] * b[12]), fmaf(-0.15171775221824646f, a[10] * b[10], fmaf(0.23841361701488495f, a[8] * b[8], fmaf(0.07508081942796707f, (a[4] * b[18] + a[18] * b[4]), fmaf(0.23032943904399872f, (a[3] * b[15] + a[15] * b[3]), -0.23032943904399872f * (a[1] * b[9] + a[9] * b[1]))))))))))) + (fmaf(0.05315294489264488f, (a[31] * b[35] + a[35] * b[31]), fmaf(0.1188535988330841f, (a[27] * b[29] + a[29] * b[27]), fmaf(0.10652530938386917f, (a[20] * b[24] + a[24] * b[20]), fmaf(-0.07741397619247437f, (a[14] * b[32] + a[32] * b[14]), fmaf(-0.11752006411552429f, (a[13] * b[15] + a[15] * b[13]), fmaf(0.07741397619247437f, (a[10] * b[28] + a[28] * b[10]), fmaf(-0.07508081942796707f, (a[8] * b[22] + a[22] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[17] + a[17] * b[5]), fmaf(-0.034723468124866486f, (a[3] * b[33] + a[33] * b[3]), 0.23293210566043854f * (a[1] * b[25] + a[25] * b[1])))))))))) + fmaf(0.1283765584230423f, a[32] * b[32], fmaf(-0.1283765584230423f, a[28] * b[28], fmaf(-0.11909890919923782f, (a[21] * b[23] + a[23] * b[21]), fmaf(0.03583570942282677f, (a[15] * b[31] + a[31] * b[15]), fmaf(0.1199292242527008f, (a[13] * b[33] + a[33] * b[13]), fmaf(-0.13408493995666504f, (a[11] * b[25] + a[25] * b[11]), fmaf(0.11752006411552429f, (a[9] * b[11] + a[11] * b[9]), fmaf(-0.2293756902217865f, (a[6] * b[24] + a[24] * b[6]), fmaf(0.23293210566043854f, (a[3] * b[35] + a[35] * b[3]), 0.034723468124866486f * (a[1] * b[27] + a[27] * b[1]))))))))))));
-        o[25] = ((fmaf(0.05315294489264488f, (a[24] * b[29] + a[29] * b[24]), fmaf(0.13019759953022003f, (a[20] * b[25] + a[25] * b[20]), fmaf(0.05315294489264488f, (a[16] * b[31] + a[31] * b[16]), fmaf(-0.13408493995666504f, (a[11] * b[24] + a[24] * b[11]), fmaf(0.24553200602531433f, (a[8] * b[9] + a[9] * b[8]), fmaf(-0.06264134496450424f, (a[4] * b[33] + a[33] * b[4]), 0.282094806432724f * (a[0] * b[25] + a[25] * b[0]))))))) + fmaf(-0.13019759953022003f, (a[21] * b[26] + a[26] * b[21]), fmaf(-0.09944005310535431f, (a[17] * b[32] + a[32] * b[17]), fmaf(-0.13408493995666504f, (a[13] * b[16] + a[16] * b[13]), fmaf(-0.06264134496450424f, (a[8] * b[27] + a[27] * b[8]), fmaf(0.13288237154483795f, (a[5] * b[34] + a[34] * b[5]), 0.23293210566043854f * (a[1] * b[24] + a[24] * b[1]))))))) + (fmaf(0.13019759953022003f, (a[22] * b[27] + a[27] * b[22]), fmaf(0.13019759953022003f, (a[18] * b[33] + a[33] * b[18]), fmaf(0.1499115228652954f, (a[14] * b[17] + a[17] * b[14]), fmaf(-0.09814012795686722f, (a[9] * b[22] + a[22] * b[9]), fmaf(-0.24260888993740082f, (a[6] * b[25] + a[25] * b[6]), 0.23293210566043854f * (a[3] * b[16] + a[16] * b[3])))))) + fmaf(-0.09944005310535431f, (a[23] * b[28] + a[28] * b[23]), fmaf(-0.13019759953022003f, (a[19] * b[34] + a[34] * b[19]), fmaf(-0.09814012795686722f, (a[15] * b[18] + a[18] * b[15]), fmaf(0.1499115228652954f, (a[10] * b[23] + a[23] * b[10]), fmaf(0.13288237154483795f, (a[7] * b[26] + a[26] * b[7]), 0.24553200602531433f * (a[4] * b[15] + a[15] * b[4]))))))));
-        o[26] = ((fmaf(0.08404218405485153f, (a[22] * b[28] + a[28] * b[22]), fmaf(0.08404218405485153f, (a[18] * b[32] + a[32] * b[18]), fmaf(0.10135868936777115f, (a[14] * b[18] + a[18] * b[14]), fmaf(0.10135868936777115f, (a[10] * b[22] + a[22] * b[10]), fmaf(0.13866253197193146f, (a[7] * b[27] + a[27] * b[7]), fmaf(-0.13288237154483795f, (a[5] * b[35] + a[35] * b[5]), fmaf(0.19018827378749847f, (a[4] * b[14] + a[14] * b[4]), 0.282094806432724f * (a[0] * b[26] + a[26] * b[0])))))))) + fmaf(-0.1188535988330841f, (a[23] * b[29] + a[29] * b[23]), fmaf(0.13019759953022003f, (a[19] * b[35] + a[35] * b[19]), fmaf(-0.1316688060760498f, (a[15] * b[19] + a[19] * b[15]), fmaf(0.0299823060631752f, (a[11] * b[23] + a[23] * b[11]), fmaf(0.19018827378749847f, (a[8] * b[10] + a[10] * b[8]), fmaf(-0.09704355895519257f, (a[6] * b[26] + a[26] * b[6]), fmaf(-0.09704355895519257f, (a[4] * b[32] + a[32] * b[4]), 0.2083408087491989f * (a[1] * b[23] + a[23] * b[1]))))))))) + (fmaf(-0.13019759953022003f, (a[20] * b[26] + a[26] * b[20]), fmaf(0.13019759953022003f, (a[16] * b[30] + a[30] * b[16]), fmaf(-0.2077234983444214f, (a[12] * b[16] + a[16] * b[12]), fmaf(-0.09704355895519257f, (a[8] * b[28] + a[28] * b[8]), fmaf(0.15528807044029236f, (a[7] * b[9] + a[9] * b[7]), fmaf(0.15528807044029236f, (a[5] * b[15] + a[15] * b[5]), 0.14731919765472412f * (a[2] * b[16] + a[16] * b[2]))))))) + fmaf(-0.13019759953022003f, (a[21] * b[25] + a[25] * b[21]), fmaf(-0.1188535988330841f, (a[17] * b[31] + a[31] * b[17]), fmaf(0.0299823060631752f, (a[13] * b[17] + a[17] * b[13]), fmaf(-0.1316688060760498f, (a[9] * b[21] + a[21] * b[9]), fmaf(0.13288237154483795f, (a[7] * b[25] + a[25] * b[7]), fmaf(0.13866253197193146f, (a[5] * b[33] + a[33] * b[5]), 0.2083408087491989f * (a[3] * b[17] + a[17] * b[3])))))))));
-        o[27] = ((fmaf(-0.13019759953022003f, (a[20] * b[27] + a[27] * b[20]), fmaf(-0.1188535988330841f, (a[16] * b[31] + a[31] * b[16]), fmaf(-0.1038617491722107f, (a[12] * b[17] + a[17] * b[12]), fmaf(-0.19628025591373444f, (a[9] * b[20] + a[20] * b[9]), fmaf(0.11436693370342255f, (a[7] * b[28] + a[28] * b[7]), fmaf(0.12679217755794525f, (a[6] * b[9] + a[9] * b[6]), fmaf(0.06264134496450424f, (a[4] * b[35] + a[35] * b[4]), fmaf(-0.034723468124866486f, (a[3] * b[16] + a[16] * b[3]), 0.282094806432724f * (a[0] * b[27] + a[27] * b[0]))))))))) + fmaf(0.08404218405485153f, (a[21] * b[28] + a[28] * b[21]), fmaf(-0.13019759953022003f, (a[17] * b[30] + a[30] * b[17]), fmaf(0.1199292242527008f, (a[13] * b[16] + a[16] * b[13]), fmaf(0.025339672341942787f, (a[10] * b[21] + a[21] * b[10]), fmaf(0.14175796508789062f, (a[8] * b[11] + a[11] * b[8]), fmaf(0.01617392711341381f, (a[6] * b[27] + a[27] * b[6]), fmaf(0.17931121587753296f, (a[5] * b[14] + a[14] * b[5]), fmaf(0.1837393194437027f, (a[3] * b[18] + a[18] * b[3]), 0.1837393194437027f * (a[1] * b[22] + a[22] * b[1])))))))))) + (fmaf(0.13019759953022003f, (a[22] * b[25] + a[25] * b[22]), fmaf(-0.13019759953022003f, (a[18] * b[35] + a[35] * b[18]), fmaf(0.1019902154803276f, (a[13] * b[18] + a[18] * b[13]), fmaf(0.1019902154803276f, (a[11] * b[22] + a[22] * b[11]), fmaf(-0.06264134496450424f, (a[8] * b[25] + a[25] * b[8]), fmaf(0.17931121587753296f, (a[7] * b[10] + a[10] * b[7]), fmaf(0.11436693370342255f, (a[5] * b[32] + a[32] * b[5]), fmaf(0.14175796508789062f, (a[4] * b[13] + a[13] * b[4]), 0.034723468124866486f * (a[1] * b[24] + a[24] * b[1]))))))))) + fmaf(0.1188535988330841f, (a[24] * b[29] + a[29] * b[24]), fmaf(0.08404218405485153f, (a[19] * b[32] + a[32] * b[19]), fmaf(0.025339672341942787f, (a[14] * b[19] + a[19] * b[14]), fmaf(-0.1199292242527008f, (a[11] * b[24] + a[24] * b[11]), fmaf(-0.12103458493947983f, (a[8] * b[29] + a[29] * b[8]), fmaf(0.13866253197193146f, (a[7] * b[26] + a[26] * b[7]), fmaf(-0.13866253197193146f, (a[5] * b[34] + a[34] * b[5]), fmaf(-0.12103458493947983f, (a[4] * b[31] + a[31] * b[4]), 0.19642560184001923f * (a[2] * b[17] + a[17] * b[2])))))))))));
-        o[28] = ((fmaf(0.08404218405485153f, (a[22] * b[26] + a[26] * b[22]), fmaf(-0.08404218405485153f, (a[19] * b[33] + a[33] * b[19]), fmaf(0.09944005310535431f, (a[17] * b[35] + a[35] * b[17]), fmaf(-0.07741397619247437f, (a[14] * b[16] + a[16] * b[14]), fmaf(-0.12117204070091248f, (a[11] * b[23] + a[23] * b[11]), fmaf(0.1266983598470688f, (a[9] * b[21] + a[21] * b[9]), fmaf(0.17361734807491302f, (a[7] * b[11] + a[11] * b[7]), fmaf(-0.11436693370342255f, (a[5] * b[33] + a[33] * b[5]), fmaf(0.09704355895519257f, (a[4] * b[34] + a[34] * b[4]), fmaf(-0.06014281138777733f, (a[3] * b[17] + a[17] * b[3]), 0.282094806432724f * (a[0] * b[28] + a[28] * b[0]))))))))))) + fmaf(-0.09944005310535431f, (a[23] * b[25] + a[25] * b[23]), fmaf(-0.02169959992170334f, (a[20] * b[28] + a[28] * b[20]), fmaf(-0.09944005310535431f, (a[18] * b[30] + a[30] * b[18]), fmaf(-0.1266983598470688f, (a[15] * b[19] + a[19] * b[15]), fmaf(0.022664492949843407f, (a[12] * b[18] + a[18] * b[12]), fmaf(-0.06542675197124481f, (a[10] * b[20] + a[20] * b[10]), fmaf(0.11436693370342255f, (a[7] * b[27] + a[27] * b[7]), fmaf(0.19018827378749847f, (a[6] * b[10] + a[10] * b[6]), fmaf(0.17361734807491302f, (a[5] * b[13] + a[13] * b[5]), fmaf(0.15912292897701263f, (a[3] * b[19] + a[19] * b[3]), 0.15912292897701263f * (a[1] * b[21] + a[21] * b[1])))))))))))) + (fmaf(-0.034310080111026764f, (a[23] * b[29] + a[29] * b[23]), fmaf(0.08404218405485153f, (a[21] * b[27] + a[27] * b[21]), fmaf(-0.08404218405485153f, (a[18] * b[34] + a[34] * b[18]), fmaf(0.1283765584230423f, (a[16] * b[32] + a[32] * b[16]), fmaf(0.12117204070091248f, (a[13] * b[17] + a[17] * b[13]), fmaf(0.07741397619247437f, (a[10] * b[24] + a[24] * b[10]), fmaf(0.0741182416677475f, (a[7] * b[29] + a[29] * b[7]), fmaf(0.09704355895519257f, (a[6] * b[28] + a[28] * b[6]), fmaf(0.04482780396938324f, (a[5] * b[15] + a[15] * b[5]), fmaf(0.14175796508789062f, (a[4] * b[12] + a[12] * b[4]), 0.06014281138777733f * (a[1] * b[23] + a[23] * b[1]))))))))))) + fmaf(-0.1283765584230423f, (a[24] * b[28] + a[28] * b[24]), fmaf(0.09077593684196472f, (a[21] * b[29] + a[29] * b[21]), fmaf(0.09077593684196472f, (a[19] * b[31] + a[31] * b[19]), fmaf(0.034310080111026764f, (a[17] * b[31] + a[31] * b[17]), fmaf(0.1046828031539917f, (a[13] * b[19] + a[19] * b[13]), fmaf(0.1046828031539917f, (a[11] * b[21] + a[21] * b[11]), fmaf(-0.09704355895519257f, (a[8] * b[26] + a[26] * b[8]), fmaf(-0.04482780396938324f, (a[7] * b[9] + a[9] * b[7]), fmaf(0.0741182416677475f, (a[5] * b[31] + a[31] * b[5]), fmaf(-0.19137248396873474f, (a[4] * b[30] + a[30] * b[4]), 0.22503378987312317f * (a[2] * b[18] + a[18] * b[2])))))))))))));
-        o[29] = ((fmaf(-0.034310080111026764f, (a[23] * b[28] + a[28] * b[23]), fmaf(0.08679839968681335f, (a[20] * b[29] + a[29] * b[20]), fmaf(0.1188535988330841f, (a[17] * b[34] + a[34] * b[17]), fmaf(0.10158468782901764f, (a[15] * b[18] + a[18] * b[15]), fmaf(0.07518995553255081f, (a[13] * b[18] + a[18] * b[13]), fmaf(0.11379365622997284f, (a[10] * b[23] + a[23] * b[10]), fmaf(-0.14007030427455902f, (a[8] * b[29] + a[29] * b[8]), fmaf(0.0741182416677475f, (a[7] * b[28] + a[28] * b[7]), fmaf(-0.0741182416677475f, (a[5] * b[32] + a[32] * b[5]), fmaf(0.12103458493947983f, (a[4] * b[33] + a[33] * b[4]), fmaf(-0.08505477756261826f, (a[3] * b[18] + a[18] * b[3]), 0.282094806432724f * (a[0] * b[29] + a[29] * b[0])))))))))))) + fmaf(0.05315294489264488f, (a[24] * b[25] + a[25] * b[24]), fmaf(0.09077593684196472f, (a[21] * b[28] + a[28] * b[21]), fmaf(0.09704355895519257f, (a[18] * b[31] + a[31] * b[18]), fmaf(-0.1188535988330841f, (a[16] * b[33] + a[33] * b[16]), fmaf(-0.11379365622997284f, (a[14] * b[17] + a[17] * b[14]), fmaf(0.08601991832256317f, (a[11] * b[20] + a[20] * b[11]), fmaf(-0.10158468782901764f, (a[9] * b[22] + a[22] * b[9]), fmaf(0.016943316906690598f, (a[8] * b[9] + a[9] * b[8]), fmaf(0.22731846570968628f, (a[6] * b[11] + a[11] * b[6]), fmaf(0.2143179029226303f, (a[5] * b[12] + a[12] * b[5]), fmaf(-0.06562118977308273f, (a[4] * b[13] + a[13] * b[4]), 0.19018827378749847f * (a[1] * b[20] + a[20] * b[1]))))))))))))) + (fmaf(0.1188535988330841f, (a[24] * b[27] + a[27] * b[24]), fmaf(-0.09704355895519257f, (a[22] * b[29] + a[29] * b[22]), fmaf(0.05315294489264488f, (a[19] * b[30] + a[30] * b[19]), fmaf(-0.05315294489264488f, (a[16] * b[35] + a[35] * b[16]), fmaf(-0.09774991124868393f, (a[14] * b[19] + a[19] * b[14]), fmaf(-0.07518995553255081f, (a[11] * b[22] + a[22] * b[11]), fmaf(-0.03583570942282677f, (a[9] * b[24] + a[24] * b[9]), fmaf(0.06562118977308273f, (a[8] * b[11] + a[11] * b[8]), fmaf(0.14556533098220825f, (a[6] * b[29] + a[29] * b[6]), fmaf(0.08300496637821198f, (a[5] * b[14] + a[14] * b[5]), fmaf(-0.016943316906690598f, (a[4] * b[15] + a[15] * b[4]), 0.08505477756261826f * (a[1] * b[22] + a[22] * b[1])))))))))))) + fmaf(-0.1188535988330841f, (a[23] * b[26] + a[26] * b[23]), fmaf(-0.09077593684196472f, (a[19] * b[32] + a[32] * b[19]), fmaf(0.034310080111026764f, (a[17] * b[32] + a[32] * b[17]), fmaf(0.03583570942282677f, (a[15] * b[16] + a[16] * b[15]), fmaf(0.11508946865797043f, (a[12] * b[19] + a[19] * b[12]), fmaf(0.09774991124868393f, (a[10] * b[21] + a[21] * b[10]), fmaf(-0.12103458493947983f, (a[8] * b[27] + a[27] * b[8]), fmaf(-0.08300496637821198f, (a[7] * b[10] + a[10] * b[7]), fmaf(0.0361659973859787f, (a[5] * b[30] + a[30] * b[5]), fmaf(0.14007030427455902f, (a[4] * b[31] + a[31] * b[4]), 0.24057124555110931f * (a[2] * b[19] + a[19] * b[2])))))))))))));
-        o[30] = ((fmaf(-0.13019759953022003f, (a[23] * b[33] + a[33] * b[23]), fmaf(0.05315294489264488f, (a[19] * b[29] + a[29] * b[19]), fmaf(0.09814012795686722f, (a[15] * b[23] + a[23] * b[15]), fmaf(0.009577495977282524f, (a[11] * b[19] + a[19] * b[11]), fmaf(0.05357947573065758f, (a[8] * b[14] + a[14] * b[8]), fmaf(0.23961469531059265f, (a[6] * b[12] + a[12] * b[6]), fmaf(0.05357947573065758f, (a[4] * b[10] + a[10] * b[4]), 0.282094806432724f * (a[0] * b[30] + a[30] * b[0])))))))) + fmaf(0.13019759953022003f, (a[24] * b[34] + a[34] * b[24]), fmaf(0.13019759953022003f, (a[20] * b[30] + a[30] * b[20]), fmaf(0.13019759953022003f, (a[16] * b[26] + a[26] * b[16]), fmaf(0.14837393164634705f, (a[12] * b[20] + a[20] * b[12]), fmaf(-0.19137248396873474f, (a[8] * b[32] + a[32] * b[8]), fmaf(0.1617392599582672f, (a[6] * b[30] + a[30] * b[6]), fmaf(-0.19137248396873474f, (a[4] * b[28] + a[28] * b[4]), -0.15528807044029236f * (a[1] * b[19] + a[19] * b[1]))))))))) + (fmaf(0.05315294489264488f, (a[21] * b[31] + a[31] * b[21]), fmaf(-0.13019759953022003f, (a[17] * b[27] + a[27] * b[17]), fmaf(0.009577495977282524f, (a[13] * b[21] + a[21] * b[13]), fmaf(0.09814012795686722f, (a[9] * b[17] + a[17] * b[9]), fmaf(-0.16943317651748657f, (a[7] * b[13] + a[13] * b[7]), fmaf(-0.16943317651748657f, (a[5] * b[11] + a[11] * b[5]), 0.24553200602531433f * (a[2] * b[20] + a[20] * b[2]))))))) + fmaf(-0.09944005310535431f, (a[22] * b[32] + a[32] * b[22]), fmaf(-0.09944005310535431f, (a[18] * b[28] + a[28] * b[18]), fmaf(-0.17132745683193207f, (a[14] * b[22] + a[22] * b[14]), fmaf(-0.17132745683193207f, (a[10] * b[18] + a[18] * b[10]), fmaf(0.0361659973859787f, (a[7] * b[31] + a[31] * b[7]), fmaf(0.0361659973859787f, (a[5] * b[29] + a[29] * b[5]), -0.15528807044029236f * (a[3] * b[21] + a[21] * b[3])))))))));
-        o[31] = ((fmaf(-0.1188535988330841f, (a[23] * b[34] + a[34] * b[23]), fmaf(0.05315294489264488f, (a[21] * b[30] + a[30] * b[21]), fmaf(0.034310080111026764f, (a[17] * b[28] + a[28] * b[17]), fmaf(0.03583570942282677f, (a[15] * b[24] + a[24] * b[15]), fmaf(0.07518995553255081f, (a[13] * b[22] + a[22] * b[13]), fmaf(0.09774991124868393f, (a[10] * b[19] + a[19] * b[10]), fmaf(-0.12103458493947983f, (a[8] * b[33] + a[33] * b[8]), fmaf(0.0741182416677475f, (a[7] * b[32] + a[32] * b[7]), fmaf(0.14556533098220825f, (a[6] * b[31] + a[31] * b[6]), fmaf(0.14007030427455902f, (a[4] * b[29] + a[29] * b[4]), fmaf(-0.08505477756261826f, (a[3] * b[22] + a[22] * b[3]), 0.282094806432724f * (a[0] * b[31] + a[31] * b[0])))))))))))) + fmaf(-0.1188535988330841f, (a[24] * b[33] + a[33] * b[24]), fmaf(0.09077593684196472f, (a[21] * b[32] + a[32] * b[21]), fmaf(0.09704355895519257f, (a[18] * b[29] + a[29] * b[18]), fmaf(0.05315294489264488f, (a[16] * b[25] + a[25] * b[16]), fmaf(0.09774991124868393f, (a[14] * b[21] + a[21] * b[14]), fmaf(0.07518995553255081f, (a[11] * b[18] + a[18] * b[11]), fmaf(0.03583570942282677f, (a[9] * b[16] + a[16] * b[9]), fmaf(-0.06562118977308273f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.2143179029226303f, (a[7] * b[12] + a[12] * b[7]), fmaf(-0.08300496637821198f, (a[5] * b[10] + a[10] * b[5]), fmaf(0.016943316906690598f, (a[4] * b[9] + a[9] * b[4]), -0.08505477756261826f * (a[1] * b[18] + a[18] * b[1]))))))))))))) + (fmaf(0.05315294489264488f, (a[24] * b[35] + a[35] * b[24]), fmaf(0.09704355895519257f, (a[22] * b[31] + a[31] * b[22]), fmaf(0.09077593684196472f, (a[19] * b[28] + a[28] * b[19]), fmaf(-0.1188535988330841f, (a[16] * b[27] + a[27] * b[16]), fmaf(-0.11379365622997284f, (a[14] * b[23] + a[23] * b[14]), fmaf(0.11508946865797043f, (a[12] * b[21] + a[21] * b[12]), fmaf(-0.10158468782901764f, (a[9] * b[18] + a[18] * b[9]), fmaf(0.016943316906690598f, (a[8] * b[15] + a[15] * b[8]), fmaf(-0.08300496637821198f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.0741182416677475f, (a[5] * b[28] + a[28] * b[5]), fmaf(-0.06562118977308273f, (a[4] * b[11] + a[11] * b[4]), 0.24057124555110931f * (a[2] * b[21] + a[21] * b[2])))))))))))) + fmaf(0.034310080111026764f, (a[23] * b[32] + a[32] * b[23]), fmaf(0.08679839968681335f, (a[20] * b[31] + a[31] * b[20]), fmaf(-0.1188535988330841f, (a[17] * b[26] + a[26] * b[17]), fmaf(-0.10158468782901764f, (a[15] * b[22] + a[22] * b[15]), fmaf(0.08601991832256317f, (a[13] * b[20] + a[20] * b[13]), fmaf(-0.11379365622997284f, (a[10] * b[17] + a[17] * b[10]), fmaf(0.14007030427455902f, (a[8] * b[31] + a[31] * b[8]), fmaf(0.0361659973859787f, (a[7] * b[30] + a[30] * b[7]), fmaf(0.22731846570968628f, (a[6] * b[13] + a[13] * b[6]), fmaf(-0.12103458493947983f, (a[4] * b[27] + a[27] * b[4]), 0.19018827378749847f * (a[3] * b[20] + a[20] * b[3])))))))))))));
-        o[32] = ((fmaf(0.08404218405485153f, (a[22] * b[34] + a[34] * b[22]), fmaf(-0.02169959992170334f, (a[20] * b[32] + a[32] * b[20]), fmaf(0.034310080111026764f, (a[17] * b[29] + a[29] * b[17]), fmaf(-0.07741397619247437f, (a[14] * b[24] + a[24] * b[14]), fmaf(0.022664492949843407f, (a[12] * b[22] + a[22] * b[12]), fmaf(0.1266983598470688f, (a[9] * b[19] + a[19] * b[9]), fmaf(0.11436693370342255f, (a[7] * b[33] + a[33] * b[7]), fmaf(0.09704355895519257f, (a[6] * b[32] + a[32] * b[6]), fmaf(-0.17361734807491302f, (a[5] * b[11] + a[11] * b[5]), fmaf(0.15912292897701263f, (a[3] * b[21] + a[21] * b[3]), 0.282094806432724f * (a[0] * b[32] + a[32] * b[0]))))))))))) + fmaf(0.034310080111026764f, (a[23] * b[31] + a[31] * b[23]), fmaf(0.09077593684196472f, (a[21] * b[31] + a[31] * b[21]), fmaf(0.08404218405485153f, (a[18] * b[26] + a[26] * b[18]), fmaf(0.1266983598470688f, (a[15] * b[21] + a[21] * b[15]), fmaf(0.1046828031539917f, (a[13] * b[21] + a[21] * b[13]), fmaf(-0.07741397619247437f, (a[10] * b[16] + a[16] * b[10]), fmaf(0.14175796508789062f, (a[8] * b[12] + a[12] * b[8]), fmaf(0.17361734807491302f, (a[7] * b[13] + a[13] * b[7]), fmaf(0.11436693370342255f, (a[5] * b[27] + a[27] * b[5]), fmaf(-0.06014281138777733f, (a[3] * b[23] + a[23] * b[3]), -0.06014281138777733f * (a[1] * b[17] + a[17] * b[1])))))))))))) + (fmaf(-0.09944005310535431f, (a[23] * b[35] + a[35] * b[23]), fmaf(0.08404218405485153f, (a[21] * b[33] + a[33] * b[21]), fmaf(0.08404218405485153f, (a[19] * b[27] + a[27] * b[19]), fmaf(0.1283765584230423f, (a[16] * b[28] + a[28] * b[16]), fmaf(0.12117204070091248f, (a[13] * b[23] + a[23] * b[13]), fmaf(0.12117204070091248f, (a[11] * b[17] + a[17] * b[11]), fmaf(-0.19137248396873474f, (a[8] * b[30] + a[30] * b[8]), fmaf(-0.04482780396938324f, (a[7] * b[15] + a[15] * b[7]), fmaf(-0.0741182416677475f, (a[5] * b[29] + a[29] * b[5]), fmaf(-0.09704355895519257f, (a[4] * b[26] + a[26] * b[4]), -0.15912292897701263f * (a[1] * b[19] + a[19] * b[1]))))))))))) + fmaf(0.1283765584230423f, (a[24] * b[32] + a[32] * b[24]), fmaf(-0.09944005310535431f, (a[22] * b[30] + a[30] * b[22]), fmaf(-0.09077593684196472f, (a[19] * b[29] + a[29] * b[19]), fmaf(-0.09944005310535431f, (a[17] * b[25] + a[25] * b[17]), fmaf(-0.06542675197124481f, (a[14] * b[20] + a[20] * b[14]), fmaf(-0.1046828031539917f, (a[11] * b[19] + a[19] * b[11]), fmaf(-0.09704355895519257f, (a[8] * b[34] + a[34] * b[8]), fmaf(0.0741182416677475f, (a[7] * b[31] + a[31] * b[7]), fmaf(0.19018827378749847f, (a[6] * b[14] + a[14] * b[6]), fmaf(-0.04482780396938324f, (a[5] * b[9] + a[9] * b[5]), 0.22503378987312317f * (a[2] * b[22] + a[22] * b[2])))))))))))));
-        o[33] = ((fmaf(0.08404218405485153f, (a[21] * b[32] + a[32] * b[21]), fmaf(-0.1188535988330841f, (a[16] * b[29] + a[29] * b[16]), fmaf(0.1019902154803276f, (a[13] * b[22] + a[22] * b[13]), fmaf(-0.025339672341942787f, (a[10] * b[19] + a[19] * b[10]), fmaf(0.13866253197193146f, (a[7] * b[34] + a[34] * b[7]), fmaf(0.12679217755794525f, (a[6] * b[15] + a[15] * b[6]), fmaf(0.12103458493947983f, (a[4] * b[29] + a[29] * b[4]), fmaf(0.1837393194437027f, (a[3] * b[22] + a[22] * b[3]), 0.282094806432724f * (a[0] * b[33] + a[33] * b[0]))))))))) + fmaf(0.13019759953022003f, (a[22] * b[35] + a[35] * b[22]), fmaf(0.13019759953022003f, (a[18] * b[25] + a[25] * b[18]), fmaf(0.1199292242527008f, (a[13] * b[24] + a[24] * b[13]), fmaf(0.1199292242527008f, (a[11] * b[16] + a[16] * b[11]), fmaf(0.14175796508789062f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.01617392711341381f, (a[6] * b[33] + a[33] * b[6]), fmaf(-0.17931121587753296f, (a[5] * b[10] + a[10] * b[5]), fmaf(-0.034723468124866486f, (a[3] * b[24] + a[24] * b[3]), -0.034723468124866486f * (a[1] * b[16] + a[16] * b[1])))))))))) + (fmaf(-0.13019759953022003f, (a[23] * b[30] + a[30] * b[23]), fmaf(-0.08404218405485153f, (a[19] * b[28] + a[28] * b[19]), fmaf(0.025339672341942787f, (a[14] * b[21] + a[21] * b[14]), fmaf(-0.1019902154803276f, (a[11] * b[18] + a[18] * b[11]), fmaf(-0.12103458493947983f, (a[8] * b[31] + a[31] * b[8]), fmaf(0.17931121587753296f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.13866253197193146f, (a[5] * b[26] + a[26] * b[5]), fmaf(-0.14175796508789062f, (a[4] * b[11] + a[11] * b[4]), -0.1837393194437027f * (a[1] * b[18] + a[18] * b[1]))))))))) + fmaf(-0.1188535988330841f, (a[24] * b[31] + a[31] * b[24]), fmaf(-0.13019759953022003f, (a[20] * b[33] + a[33] * b[20]), fmaf(-0.19628025591373444f, (a[15] * b[20] + a[20] * b[15]), fmaf(-0.1038617491722107f, (a[12] * b[23] + a[23] * b[12]), fmaf(-0.06264134496450424f, (a[8] * b[35] + a[35] * b[8]), fmaf(0.11436693370342255f, (a[7] * b[32] + a[32] * b[7]), fmaf(-0.11436693370342255f, (a[5] * b[28] + a[28] * b[5]), fmaf(-0.06264134496450424f, (a[4] * b[25] + a[25] * b[4]), 0.19642560184001923f * (a[2] * b[23] + a[23] * b[2])))))))))));
-        o[34] = ((fmaf(-0.1188535988330841f, (a[23] * b[31] + a[31] * b[23]), fmaf(-0.13019759953022003f, (a[19] * b[25] + a[25] * b[19]), fmaf(0.10135868936777115f, (a[14] * b[22] + a[22] * b[14]), fmaf(-0.10135868936777115f, (a[10] * b[18] + a[18] * b[10]), fmaf(0.13288237154483795f, (a[7] * b[35] + a[35] * b[7]), fmaf(-0.13866253197193146f, (a[5] * b[27] + a[27] * b[5]), fmaf(-0.19018827378749847f, (a[4] * b[10] + a[10] * b[4]), 0.282094806432724f * (a[0] * b[34] + a[34] * b[0])))))))) + fmaf(0.13019759953022003f, (a[24] * b[30] + a[30] * b[24]), fmaf(-0.13019759953022003f, (a[20] * b[34] + a[34] * b[20]), fmaf(-0.1316688060760498f, (a[15] * b[21] + a[21] * b[15]), fmaf(-0.0299823060631752f, (a[11] * b[17] + a[17] * b[11]), fmaf(0.19018827378749847f, (a[8] * b[14] + a[14] * b[8]), fmaf(-0.09704355895519257f, (a[6] * b[34] + a[34] * b[6]), fmaf(0.09704355895519257f, (a[4] * b[28] + a[28] * b[4]), -0.2083408087491989f * (a[1] * b[17] + a[17] * b[1]))))))))) + (fmaf(-0.13019759953022003f, (a[21] * b[35] + a[35] * b[21]), fmaf(0.1188535988330841f, (a[17] * b[29] + a[29] * b[17]), fmaf(-0.2077234983444214f, (a[12] * b[24] + a[24] * b[12]), fmaf(-0.09704355895519257f, (a[8] * b[32] + a[32] * b[8]), fmaf(0.15528807044029236f, (a[7] * b[15] + a[15] * b[7]), fmaf(-0.15528807044029236f, (a[5] * b[9] + a[9] * b[5]), 0.14731919765472412f * (a[2] * b[24] + a[24] * b[2]))))))) + fmaf(0.08404218405485153f, (a[22] * b[32] + a[32] * b[22]), fmaf(-0.08404218405485153f, (a[18] * b[28] + a[28] * b[18]), fmaf(0.0299823060631752f, (a[13] * b[23] + a[23] * b[13]), fmaf(0.1316688060760498f, (a[9] * b[19] + a[19] * b[9]), fmaf(0.13866253197193146f, (a[7] * b[33] + a[33] * b[7]), fmaf(0.13288237154483795f, (a[5] * b[25] + a[25] * b[5]), 0.2083408087491989f * (a[3] * b[23] + a[23] * b[3])))))))));
-        o[35] = ((fmaf(0.05315294489264488f, (a[24] * b[31] + a[31] * b[24]), fmaf(0.13019759953022003f, (a[20] * b[35] + a[35] * b[20]), fmaf(-0.05315294489264488f, (a[16] * b[29] + a[29] * b[16]), fmaf(0.13408493995666504f, (a[11] * b[16] + a[16] * b[11]), fmaf(0.24553200602531433f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.06264134496450424f, (a[4] * b[27] + a[27] * b[4]), 0.282094806432724f * (a[0] * b[35] + a[35] * b[0]))))))) + fmaf(-0.13019759953022003f, (a[21] * b[34] + a[34] * b[21]), fmaf(0.09944005310535431f, (a[17] * b[28] + a[28] * b[17]), fmaf(-0.13408493995666504f, (a[13] * b[24] + a[24] * b[13]), fmaf(-0.06264134496450424f, (a[8] * b[33] + a[33] * b[8]), fmaf(-0.13288237154483795f, (a[5] * b[26] + a[26] * b[5]), -0.23293210566043854f * (a[1] * b[16] + a[16] * b[1]))))))) + (fmaf(0.13019759953022003f, (a[22] * b[33] + a[33] * b[22]), fmaf(-0.13019759953022003f, (a[18] * b[27] + a[27] * b[18]), fmaf(0.1499115228652954f, (a[14] * b[23] + a[23] * b[14]), fmaf(0.09814012795686722f, (a[9] * b[18] + a[18] * b[9]), fmaf(-0.24260888993740082f, (a[6] * b[35] + a[35] * b[6]), 0.23293210566043854f * (a[3] * b[24] + a[24] * b[3])))))) + fmaf(-0.09944005310535431f, (a[23] * b[32] + a[32] * b[23]), fmaf(0.13019759953022003f, (a[19] * b[26] + a[26] * b[19]), fmaf(-0.09814012795686722f, (a[15] * b[22] + a[22] * b[15]), fmaf(-0.1499115228652954f, (a[10] * b[17] + a[17] * b[10]), fmaf(0.13288237154483795f, (a[7] * b[34] + a[34] * b[7]), -0.24553200602531433f * (a[4] * b[9] + a[9] * b[4]))))))));
-    }
-    __device__ __forceinline__ static void sqr(const float* __restrict__ a, float* __restrict__ o) {
-        o[0] = ((fmaf(0.282094806432724f, a[32] * a[32], fmaf(0.282094806432724f, a[28] * a[28], fmaf(0.282094806432724f, a[24] * a[24], fmaf(0.282094806432724f, a[20] * a[20], fmaf(0.282094806432724f, a[16] * a[16], fmaf(0.282094806432724f, a[12] * a[12], fmaf(0.282094806432724f, a[8] * a[8], fmaf(0.282094806432724f, a[4] * a[4], 0.282094806432724f * a[0] * a[0])))))))) + fmaf(0.282094806432724f, a[33] * a[33], fmaf(0.282094806432724f, a[29] * a[29], fmaf(0.282094806432724f, a[25] * a[25], fmaf(0.282094806432724f, a[21] * a[21], fmaf(0.282094806432724f, a[17] * a[17], fmaf(0.282094806432724f, a[13] * a[13], fmaf(0.282094806432724f, a[9] * a[9], fmaf(0.282094806432724f, a[5] * a[5], 0.282094806432724f * a[1] * a[1]))))))))) + (fmaf(0.282094806432724f, a[34] * a[34], fmaf(0.282094806432724f, a[30] * a[30], fmaf(0.282094806432724f, a[26] * a[26], fmaf(0.282094806432724f, a[22] * a[22], fmaf(0.282094806432724f, a[18] * a[18], fmaf(0.282094806432724f, a[14] * a[14], fmaf(0.282094806432724f, a[10] * a[10], fmaf(0.282094806432724f, a[6] * a[6], 0.282094806432724f * a[2] * a[2])))))))) + fmaf(0.282094806432724f, a[35] * a[35], fmaf(0.282094806432724f, a[31] * a[31], fmaf(0.282094806432724f, a[27] * a[27], fmaf(0.282094806432724f, a[23] * a[23], fmaf(0.282094806432724f, a[19] * a[19], fmaf(0.282094806432724f, a[15] * a[15], fmaf(0.282094806432724f, a[11] * a[11], fmaf(0.282094806432724f, a[7] * a[7], 0.282094806432724f * a[3] * a[3]))))))))));
-        o[1] = ((fmaf(0.06944693624973297f, a[24] * a[27], fmaf(0.1701095551252365f, a[22] * a[29], fmaf(-0.31824585795402527f, a[19] * a[32], fmaf(-0.4166816174983978f, a[17] * a[34], fmaf(0.08705634623765945f, a[15] * a[18], fmaf(0.33716776967048645f, a[13] * a[18], fmaf(-0.3989422917366028f, a[10] * a[23], fmaf(0.11679834127426147f, a[8] * a[11], fmaf(-0.36934879422187805f, a[5] * a[14], fmaf(0.43701937794685364f, a[3] * a[4], 0.564189612865448f * a[0] * a[1])))))))))) + fmaf(0.4166816174983978f, a[23] * a[26], fmaf(0.38037654757499695f, a[20] * a[29], fmaf(-0.1701095551252365f, a[18] * a[31], fmaf(-0.06944693624973297f, a[16] * a[33], fmaf(0.3989422917366028f, a[14] * a[17], fmaf(-0.3015720248222351f, a[11] * a[20], fmaf(-0.08705634623765945f, a[9] * a[22], fmaf(0.4046013057231903f, a[6] * a[11], fmaf(-0.11679834127426147f, a[4] * a[13], -0.2523132562637329f * a[1] * a[6])))))))))) + (fmaf(0.12028562277555466f, a[23] * a[28], fmaf(0.31824585795402527f, a[21] * a[28], fmaf(-0.3674786388874054f, a[18] * a[33], fmaf(-0.4658642113208771f, a[16] * a[35], fmaf(0.15078601241111755f, a[14] * a[19], fmaf(-0.33716776967048645f, a[11] * a[22], fmaf(-0.46065887808799744f, a[9] * a[24], fmaf(0.36934879422187805f, a[7] * a[10], fmaf(-0.45235803723335266f, a[4] * a[15], -0.43701937794685364f * a[1] * a[8]))))))))) + fmaf(0.4658642113208771f, a[24] * a[25], fmaf(0.3674786388874054f, a[22] * a[27], fmaf(-0.3105761408805847f, a[19] * a[30], fmaf(-0.12028562277555466f, a[17] * a[32], fmaf(0.46065887808799744f, a[15] * a[16], fmaf(0.3893277943134308f, a[12] * a[19], fmaf(-0.15078601241111755f, a[10] * a[21], fmaf(0.45235803723335266f, a[8] * a[9], fmaf(-0.28609633445739746f, a[5] * a[12], 0.43701937794685364f * a[2] * a[5])))))))))));
-        o[2] = ((fmaf(0.29463839530944824f, a[24] * a[34], fmaf(0.49106401205062866f, a[20] * a[30], fmaf(0.29463839530944824f, a[16] * a[26], fmaf(0.4924650490283966f, a[12] * a[20], fmaf(0.36934879422187805f, a[8] * a[14], fmaf(0.36934879422187805f, a[4] * a[10], 0.564189612865448f * a[0] * a[2])))))) + fmaf(0.48114249110221863f, a[21] * a[31], fmaf(0.39285120368003845f, a[17] * a[27], fmaf(0.4768272340297699f, a[13] * a[21], fmaf(0.3257350027561188f, a[9] * a[17], fmaf(0.4671933650970459f, a[5] * a[11], 0.43701937794685364f * a[1] * a[5])))))) + (fmaf(0.45006757974624634f, a[22] * a[32], fmaf(0.45006757974624634f, a[18] * a[28], fmaf(0.4264872372150421f, a[14] * a[22], fmaf(0.4264872372150421f, a[10] * a[18], fmaf(0.49553337693214417f, a[6] * a[12], 0.5046265125274658f * a[2] * a[6]))))) + fmaf(0.39285120368003845f, a[23] * a[33], fmaf(0.48114249110221863f, a[19] * a[29], fmaf(0.3257350027561188f, a[15] * a[23], fmaf(0.4768272340297699f, a[11] * a[19], fmaf(0.4671933650970459f, a[7] * a[13], 0.43701937794685364f * a[3] * a[7])))))));
-        o[3] = ((fmaf(0.4658642113208771f, a[24] * a[35], fmaf(0.3674786388874054f, a[22] * a[33], fmaf(0.38037654757499695f, a[20] * a[31], fmaf(-0.12028562277555466f, a[17] * a[28], fmaf(0.46065887808799744f, a[15] * a[24], fmaf(0.33716776967048645f, a[13] * a[22], fmaf(-0.15078601241111755f, a[10] * a[19], fmaf(0.45235803723335266f, a[8] * a[15], fmaf(0.4046013057231903f, a[6] * a[13], fmaf(0.43701937794685364f, a[3] * a[8], 0.564189612865448f * a[0] * a[3])))))))))) + fmaf(-0.12028562277555466f, a[23] * a[32], fmaf(-0.3105761408805847f, a[21] * a[30], fmaf(0.3674786388874054f, a[18] * a[27], fmaf(0.4658642113208771f, a[16] * a[25], fmaf(-0.15078601241111755f, a[14] * a[21], fmaf(0.33716776967048645f, a[11] * a[18], fmaf(0.46065887808799744f, a[9] * a[16], fmaf(-0.28609633445739746f, a[7] * a[12], fmaf(0.45235803723335266f, a[4] * a[9], 0.43701937794685364f * a[1] * a[4])))))))))) + (fmaf(0.4166816174983978f, a[23] * a[34], fmaf(0.31824585795402527f, a[21] * a[32], fmaf(-0.1701095551252365f, a[18] * a[29], fmaf(-0.06944693624973297f, a[16] * a[27], fmaf(0.3989422917366028f, a[14] * a[23], fmaf(0.3893277943134308f, a[12] * a[21], fmaf(-0.08705634623765945f, a[9] * a[18], fmaf(0.36934879422187805f, a[7] * a[14], fmaf(-0.11679834127426147f, a[4] * a[11], 0.43701937794685364f * a[2] * a[7]))))))))) + fmaf(-0.06944693624973297f, a[24] * a[33], fmaf(-0.1701095551252365f, a[22] * a[31], fmaf(0.31824585795402527f, a[19] * a[28], fmaf(0.4166816174983978f, a[17] * a[26], fmaf(-0.08705634623765945f, a[15] * a[22], fmaf(-0.3015720248222351f, a[13] * a[20], fmaf(0.3989422917366028f, a[10] * a[17], fmaf(-0.11679834127426147f, a[8] * a[13], fmaf(0.36934879422187805f, a[5] * a[10], -0.2523132562637329f * a[3] * a[6])))))))))));
-        o[4] = ((fmaf(0.19408711791038513f, a[28] * a[34], fmaf(-0.19408711791038513f, a[26] * a[32], fmaf(0.15016163885593414f, a[18] * a[24], fmaf(-0.033886633813381195f, a[15] * a[29], fmaf(0.28351593017578125f, a[13] * a[27], fmaf(0.18806318938732147f, a[11] * a[15], fmaf(-0.37612637877464294f, a[10] * a[12], fmaf(0.4768272340297699f, a[8] * a[16], fmaf(-0.33716776967048645f, a[5] * a[23], fmaf(0.08059851080179214f, a[4] * a[20], fmaf(0.36934879422187805f, a[2] * a[10], 0.564189612865448f * a[0] * a[4]))))))))))) + fmaf(0.28014060854911804f, a[29] * a[31], fmaf(-0.24206916987895966f, a[27] * a[31], fmaf(0.2837788164615631f, a[19] * a[21], fmaf(-0.15016163885593414f, a[16] * a[22], fmaf(-0.13124237954616547f, a[13] * a[29], fmaf(-0.13124237954616547f, a[11] * a[31], fmaf(0.10715895146131516f, a[10] * a[30], fmaf(-0.18806318938732147f, a[9] * a[13], fmaf(0.31215670704841614f, a[6] * a[18], fmaf(-0.4768272340297699f, a[4] * a[24], fmaf(0.45235803723335266f, a[3] * a[9], 0.43701937794685364f * a[1] * a[3])))))))))))) + (fmaf(0.24206916987895966f, a[29] * a[33], fmaf(0.12528268992900848f, a[27] * a[35], fmaf(0.22524245083332062f, a[19] * a[23], fmaf(-0.22524245083332062f, a[17] * a[21], fmaf(0.38037654757499695f, a[14] * a[26], fmaf(-0.28351593017578125f, a[11] * a[33], fmaf(-0.38037654757499695f, a[10] * a[34], fmaf(0.033886633813381195f, a[9] * a[31], fmaf(0.33716776967048645f, a[7] * a[17], fmaf(0.31215670704841614f, a[5] * a[7], fmaf(-0.11679834127426147f, a[3] * a[11], -0.11679834127426147f * a[1] * a[13]))))))))))) + fmaf(-0.3827449679374695f, a[28] * a[30], fmaf(-0.12528268992900848f, a[25] * a[33], fmaf(-0.38072922825813293f, a[18] * a[20], fmaf(0.49106401205062866f, a[15] * a[25], fmaf(0.28351593017578125f, a[12] * a[28], fmaf(0.2913462519645691f, a[11] * a[13], fmaf(-0.49106401205062866f, a[9] * a[35], fmaf(-0.12743744254112244f, a[7] * a[19], fmaf(-0.12743744254112244f, a[5] * a[21], fmaf(-0.360447496175766f, a[4] * a[6], -0.45235803723335266f * a[1] * a[15]))))))))))));
-        o[5] = ((fmaf(0.0723319947719574f, a[29] * a[30], fmaf(0.2287338674068451f, a[27] * a[32], fmaf(-0.18059572577476501f, a[19] * a[22], fmaf(-0.2809267044067383f, a[17] * a[24], fmaf(0.3105761408805847f, a[15] * a[26], fmaf(0.4286358058452606f, a[12] * a[29], fmaf(0.11894160509109497f, a[11] * a[12], fmaf(0.23032943904399872f, a[10] * a[13], fmaf(0.12743744254112244f, a[8] * a[19], fmaf(-0.360447496175766f, a[5] * a[22], fmaf(-0.33716776967048645f, a[4] * a[23], fmaf(0.4671933650970459f, a[2] * a[11], 0.564189612865448f * a[0] * a[5])))))))))))) + fmaf(-0.148236483335495f, a[29] * a[32], fmaf(-0.2773250639438629f, a[27] * a[34], fmaf(0.2657647430896759f, a[25] * a[34], fmaf(0.18059572577476501f, a[18] * a[21], fmaf(0.08965560793876648f, a[15] * a[28], fmaf(0.34723469614982605f, a[13] * a[28], fmaf(-0.23032943904399872f, a[11] * a[14], fmaf(-0.2973540127277374f, a[10] * a[15], fmaf(0.2973540127277374f, a[9] * a[14], fmaf(0.44145622849464417f, a[6] * a[19], fmaf(0.180223748087883f, a[5] * a[6], fmaf(0.36934879422187805f, a[3] * a[10], 0.43701937794685364f * a[1] * a[2]))))))))))))) + (fmaf(0.148236483335495f, a[28] * a[31], fmaf(0.2773250639438629f, a[26] * a[33], fmaf(-0.26545077562332153f, a[18] * a[23], fmaf(0.2809267044067383f, a[16] * a[23], fmaf(0.3586224317550659f, a[14] * a[27], fmaf(-0.33886635303497314f, a[11] * a[30], fmaf(-0.16600993275642395f, a[10] * a[31], fmaf(-0.08965560793876648f, a[9] * a[32], fmaf(0.360447496175766f, a[7] * a[18], fmaf(-0.31215670704841614f, a[5] * a[8], fmaf(0.31215670704841614f, a[4] * a[7], -0.28609633445739746f * a[1] * a[12]))))))))))) + fmaf(-0.2287338674068451f, a[28] * a[33], fmaf(-0.2657647430896759f, a[26] * a[35], fmaf(0.08973874151706696f, a[19] * a[20], fmaf(0.26545077562332153f, a[17] * a[22], fmaf(0.16600993275642395f, a[14] * a[29], fmaf(-0.34723469614982605f, a[11] * a[32], fmaf(-0.3586224317550659f, a[10] * a[33], fmaf(-0.3105761408805847f, a[9] * a[34], fmaf(0.33716776967048645f, a[8] * a[17], fmaf(-0.3223940432071686f, a[5] * a[20], fmaf(-0.12743744254112244f, a[4] * a[21], -0.36934879422187805f * a[1] * a[14])))))))))))));
-        o[6] = ((fmaf(-0.24260888993740082f, a[35] * a[35], fmaf(0.14556533098220825f, a[31] * a[31], fmaf(0.01617392711341381f, a[27] * a[27], fmaf(-0.057343922555446625f, a[23] * a[23], fmaf(0.1392638087272644f, a[19] * a[19], fmaf(0.2535843551158905f, a[15] * a[33], fmaf(0.12615662813186646f, a[13] * a[13], fmaf(0.12615662813186646f, a[11] * a[11], fmaf(0.31215670704841614f, a[8] * a[22], fmaf(0.48359107971191406f, a[6] * a[20], fmaf(0.31215670704841614f, a[4] * a[18], fmaf(0.49553337693214417f, a[2] * a[12], 0.564189612865448f * a[0] * a[6])))))))))))) + fmaf(0.09704355895519257f, a[32] * a[32], fmaf(0.09704355895519257f, a[28] * a[28], fmaf(-0.2293756902217865f, a[24] * a[24], fmaf(0.16383977234363556f, a[20] * a[20], fmaf(-0.2293756902217865f, a[16] * a[16], fmaf(0.45463693141937256f, a[13] * a[31], fmaf(0.45463693141937256f, a[11] * a[29], fmaf(-0.2102610468864441f, a[9] * a[9], fmaf(0.0901118740439415f, a[7] * a[7], fmaf(0.0901118740439415f, a[5] * a[5], fmaf(-0.12615662813186646f, a[3] * a[3], -0.12615662813186646f * a[1] * a[1])))))))))))) + (fmaf(0.01617392711341381f, a[33] * a[33], fmaf(0.14556533098220825f, a[29] * a[29], fmaf(-0.24260888993740082f, a[25] * a[25], fmaf(0.1392638087272644f, a[21] * a[21], fmaf(-0.057343922555446625f, a[17] * a[17], fmaf(0.38037654757499695f, a[14] * a[32], fmaf(0.16820883750915527f, a[12] * a[12], fmaf(0.2535843551158905f, a[9] * a[27], fmaf(0.44145622849464417f, a[7] * a[21], fmaf(0.44145622849464417f, a[5] * a[19], fmaf(0.4046013057231903f, a[3] * a[13], 0.4046013057231903f * a[1] * a[11]))))))))))) + fmaf(-0.09704355895519257f, a[34] * a[34], fmaf(0.1617392599582672f, a[30] * a[30], fmaf(-0.09704355895519257f, a[26] * a[26], fmaf(0.06553591042757034f, a[22] * a[22], fmaf(0.06553591042757034f, a[18] * a[18], fmaf(-0.2102610468864441f, a[15] * a[15], fmaf(0.4792293906211853f, a[12] * a[30], fmaf(0.38037654757499695f, a[10] * a[28], fmaf(-0.180223748087883f, a[8] * a[8], fmaf(0.180223748087883f, a[6] * a[6], fmaf(-0.180223748087883f, a[4] * a[4], 0.2523132562637329f * a[2] * a[2])))))))))))));
-        o[7] = ((fmaf(0.2773250639438629f, a[33] * a[34], fmaf(0.148236483335495f, a[28] * a[29], fmaf(0.2809267044067383f, a[23] * a[24], fmaf(0.18059572577476501f, a[18] * a[19], fmaf(-0.08965560793876648f, a[15] * a[32], fmaf(0.34723469614982605f, a[13] * a[32], fmaf(0.11894160509109497f, a[12] * a[13], fmaf(0.23032943904399872f, a[10] * a[11], fmaf(0.33716776967048645f, a[8] * a[23], fmaf(0.31215670704841614f, a[7] * a[8], fmaf(-0.12743744254112244f, a[4] * a[19], fmaf(-0.28609633445739746f, a[3] * a[12], 0.564189612865448f * a[0] * a[7])))))))))))) + fmaf(0.2657647430896759f, a[34] * a[35], fmaf(0.0723319947719574f, a[30] * a[31], fmaf(0.2657647430896759f, a[25] * a[26], fmaf(0.08973874151706696f, a[20] * a[21], fmaf(0.3105761408805847f, a[15] * a[34], fmaf(0.2973540127277374f, a[14] * a[15], fmaf(0.4286358058452606f, a[12] * a[31], fmaf(0.3586224317550659f, a[10] * a[27], fmaf(0.2973540127277374f, a[9] * a[10], fmaf(-0.3223940432071686f, a[7] * a[20], fmaf(0.360447496175766f, a[5] * a[18], fmaf(0.36934879422187805f, a[3] * a[14], 0.36934879422187805f * a[1] * a[10]))))))))))))) + (fmaf(0.148236483335495f, a[31] * a[32], fmaf(0.2773250639438629f, a[26] * a[27], fmaf(0.18059572577476501f, a[21] * a[22], fmaf(0.2809267044067383f, a[16] * a[17], fmaf(-0.16600993275642395f, a[14] * a[31], fmaf(0.23032943904399872f, a[13] * a[14], fmaf(-0.16600993275642395f, a[10] * a[29], fmaf(0.3105761408805847f, a[9] * a[26], fmaf(0.360447496175766f, a[7] * a[22], fmaf(0.180223748087883f, a[6] * a[7], fmaf(0.31215670704841614f, a[4] * a[5], 0.43701937794685364f * a[2] * a[3]))))))))))) + fmaf(0.2287338674068451f, a[32] * a[33], fmaf(0.2287338674068451f, a[27] * a[28], fmaf(0.26545077562332153f, a[22] * a[23], fmaf(0.26545077562332153f, a[17] * a[18], fmaf(0.3586224317550659f, a[14] * a[33], fmaf(-0.33886635303497314f, a[13] * a[30], fmaf(0.34723469614982605f, a[11] * a[28], fmaf(-0.08965560793876648f, a[9] * a[28], fmaf(-0.12743744254112244f, a[8] * a[21], fmaf(0.44145622849464417f, a[6] * a[21], fmaf(0.33716776967048645f, a[4] * a[17], 0.4671933650970459f * a[2] * a[13])))))))))))));
-        o[8] = ((fmaf(0.14007030427455902f, a[31] * a[31], fmaf(-0.19408711791038513f, a[26] * a[28], fmaf(0.14188940823078156f, a[21] * a[21], fmaf(-0.15016163885593414f, a[16] * a[18], fmaf(0.10715895146131516f, a[14] * a[30], fmaf(0.14567312598228455f, a[13] * a[13], fmaf(0.28351593017578125f, a[11] * a[27], fmaf(0.49106401205062866f, a[9] * a[25], fmaf(0.33716776967048645f, a[7] * a[23], fmaf(-0.360447496175766f, a[6] * a[8], fmaf(0.4768272340297699f, a[4] * a[16], fmaf(0.36934879422187805f, a[2] * a[14], 0.564189612865448f * a[0] * a[8])))))))))))) + fmaf(-0.24206916987895966f, a[31] * a[33], fmaf(-0.24206916987895966f, a[27] * a[29], fmaf(-0.22524245083332062f, a[21] * a[23], fmaf(-0.22524245083332062f, a[17] * a[19], fmaf(0.38037654757499695f, a[14] * a[34], fmaf(-0.18806318938732147f, a[13] * a[15], fmaf(0.13124237954616547f, a[11] * a[29], fmaf(0.033886633813381195f, a[9] * a[29], fmaf(0.08059851080179214f, a[8] * a[20], fmaf(0.31215670704841614f, a[6] * a[22], fmaf(-0.15607835352420807f, a[5] * a[5], fmaf(0.21850968897342682f, a[3] * a[3], -0.21850968897342682f * a[1] * a[1]))))))))))))) + (fmaf(-0.19408711791038513f, a[32] * a[34], fmaf(-0.14007030427455902f, a[29] * a[29], fmaf(-0.15016163885593414f, a[22] * a[24], fmaf(-0.14188940823078156f, a[19] * a[19], fmaf(0.033886633813381195f, a[15] * a[31], fmaf(-0.13124237954616547f, a[13] * a[31], fmaf(-0.37612637877464294f, a[12] * a[14], fmaf(0.38037654757499695f, a[10] * a[26], fmaf(0.4768272340297699f, a[8] * a[24], fmaf(0.15607835352420807f, a[7] * a[7], fmaf(0.33716776967048645f, a[5] * a[17], fmaf(-0.11679834127426147f, a[3] * a[13], 0.45235803723335266f * a[1] * a[9])))))))))))) + fmaf(-0.12528268992900848f, a[33] * a[35], fmaf(-0.3827449679374695f, a[30] * a[32], fmaf(-0.12528268992900848f, a[25] * a[27], fmaf(-0.38072922825813293f, a[20] * a[22], fmaf(0.49106401205062866f, a[15] * a[35], fmaf(0.28351593017578125f, a[13] * a[33], fmaf(0.28351593017578125f, a[12] * a[32], fmaf(-0.14567312598228455f, a[11] * a[11], fmaf(-0.18806318938732147f, a[9] * a[11], fmaf(-0.12743744254112244f, a[7] * a[21], fmaf(0.12743744254112244f, a[5] * a[19], fmaf(0.45235803723335266f, a[3] * a[15], 0.11679834127426147f * a[1] * a[11]))))))))))))));
-        o[9] = ((fmaf(-0.20316937565803528f, a[22] * a[29], fmaf(-0.39256051182746887f, a[20] * a[27], fmaf(-0.20316937565803528f, a[18] * a[31], fmaf(0.2665104568004608f, a[13] * a[18], fmaf(0.2665104568004608f, a[11] * a[22], fmaf(0.49106401205062866f, a[8] * a[25], fmaf(0.2973540127277374f, a[7] * a[10], fmaf(-0.08965560793876648f, a[5] * a[32], fmaf(-0.18806318938732147f, a[4] * a[13], fmaf(0.3257350027561188f, a[2] * a[17], 0.564189612865448f * a[0] * a[9])))))))))) + fmaf(-0.07167141884565353f, a[24] * a[29], fmaf(-0.2633376121520996f, a[21] * a[26], fmaf(0.19628025591373444f, a[18] * a[35], fmaf(-0.19864517450332642f, a[14] * a[19], fmaf(0.23504012823104858f, a[11] * a[24], fmaf(0.033886633813381195f, a[8] * a[29], fmaf(0.3105761408805847f, a[7] * a[26], fmaf(-0.3105761408805847f, a[5] * a[34], fmaf(0.033886633813381195f, a[4] * a[31], fmaf(0.45235803723335266f, a[3] * a[4], 0.45235803723335266f * a[1] * a[8]))))))))))) + (fmaf(0.2533967196941376f, a[21] * a[28], fmaf(0.2533967196941376f, a[19] * a[32], fmaf(0.07167141884565353f, a[16] * a[31], fmaf(-0.40710145235061646f, a[12] * a[17], fmaf(0.1538698822259903f, a[9] * a[20], fmaf(-0.08965560793876648f, a[7] * a[28], fmaf(-0.4205220937728882f, a[6] * a[9], fmaf(-0.49106401205062866f, a[4] * a[35], fmaf(0.46065887808799744f, a[3] * a[16], -0.08705634623765945f * a[1] * a[22]))))))))) + fmaf(-0.19628025591373444f, a[22] * a[25], fmaf(0.2633376121520996f, a[19] * a[34], fmaf(0.19628025591373444f, a[17] * a[30], fmaf(-0.23504012823104858f, a[13] * a[16], fmaf(-0.19864517450332642f, a[10] * a[21], fmaf(-0.18806318938732147f, a[8] * a[11], fmaf(0.2535843551158905f, a[6] * a[27], fmaf(0.2973540127277374f, a[5] * a[14], fmaf(-0.08705634623765945f, a[3] * a[18], -0.46065887808799744f * a[1] * a[24])))))))))));
-        o[10] = ((fmaf(0.22758731245994568f, a[23] * a[29], fmaf(0.050679344683885574f, a[21] * a[27], fmaf(-0.2027173787355423f, a[18] * a[34], fmaf(-0.15482795238494873f, a[16] * a[32], fmaf(0.13570047914981842f, a[13] * a[17], fmaf(-0.3034355044364929f, a[10] * a[24], fmaf(-0.16600993275642395f, a[7] * a[29], fmaf(0.38037654757499695f, a[6] * a[28], fmaf(0.23032943904399872f, a[5] * a[13], fmaf(-0.15078601241111755f, a[3] * a[19], fmaf(0.36934879422187805f, a[2] * a[4], 0.564189612865448f * a[0] * a[10]))))))))))) + fmaf(0.15482795238494873f, a[24] * a[28], fmaf(0.19549982249736786f, a[21] * a[29], fmaf(0.19549982249736786f, a[19] * a[31], fmaf(-0.22758731245994568f, a[17] * a[31], fmaf(0.20515984296798706f, a[13] * a[19], fmaf(0.20515984296798706f, a[11] * a[21], fmaf(0.38037654757499695f, a[8] * a[26], fmaf(0.2973540127277374f, a[7] * a[9], fmaf(-0.2973540127277374f, a[5] * a[15], fmaf(-0.37612637877464294f, a[4] * a[12], fmaf(0.4264872372150421f, a[2] * a[18], 0.36934879422187805f * a[1] * a[7])))))))))))) + (fmaf(0.2027173787355423f, a[22] * a[26], fmaf(-0.050679344683885574f, a[19] * a[33], fmaf(-0.2998230457305908f, a[17] * a[35], fmaf(0.3034355044364929f, a[14] * a[16], fmaf(-0.13570047914981842f, a[11] * a[23], fmaf(-0.19864517450332642f, a[9] * a[21], fmaf(0.23032943904399872f, a[7] * a[11], fmaf(-0.16600993275642395f, a[5] * a[31], fmaf(0.10715895146131516f, a[4] * a[30], fmaf(0.36934879422187805f, a[3] * a[5], -0.15078601241111755f * a[1] * a[21])))))))))) + fmaf(0.2998230457305908f, a[23] * a[25], fmaf(-0.13085350394248962f, a[20] * a[28], fmaf(-0.34265491366386414f, a[18] * a[30], fmaf(0.19864517450332642f, a[15] * a[19], fmaf(-0.08883681893348694f, a[12] * a[18], fmaf(-0.35902974009513855f, a[10] * a[20], fmaf(0.3586224317550659f, a[7] * a[27], fmaf(-0.3586224317550659f, a[5] * a[33], fmaf(-0.38037654757499695f, a[4] * a[34], fmaf(0.3989422917366028f, a[3] * a[17], -0.3989422917366028f * a[1] * a[23]))))))))))));
-        o[11] = ((fmaf(-0.2398584485054016f, a[24] * a[27], fmaf(-0.15037991106510162f, a[22] * a[29], fmaf(-0.2093656063079834f, a[19] * a[32], fmaf(-0.0599646121263504f, a[17] * a[34], fmaf(-0.2665104568004608f, a[15] * a[18], fmaf(0.2293756902217865f, a[13] * a[18], fmaf(-0.13570047914981842f, a[10] * a[23], fmaf(0.13124237954616547f, a[8] * a[29], fmaf(0.34723469614982605f, a[7] * a[28], fmaf(-0.34723469614982605f, a[5] * a[32], fmaf(-0.28351593017578125f, a[4] * a[33], fmaf(0.33716776967048645f, a[3] * a[18], fmaf(-0.33716776967048645f, a[1] * a[22], 0.564189612865448f * a[0] * a[11]))))))))))))) + fmaf(0.0599646121263504f, a[23] * a[26], fmaf(0.17203983664512634f, a[20] * a[29], fmaf(0.15037991106510162f, a[18] * a[31], fmaf(0.2398584485054016f, a[16] * a[33], fmaf(0.13570047914981842f, a[14] * a[17], fmaf(0.051289960741996765f, a[11] * a[20], fmaf(0.2665104568004608f, a[9] * a[22], fmaf(-0.18806318938732147f, a[8] * a[9], fmaf(0.2523132562637329f, a[6] * a[11], fmaf(0.11894160509109497f, a[5] * a[12], fmaf(0.2913462519645691f, a[4] * a[13], fmaf(0.4671933650970459f, a[2] * a[5], 0.4046013057231903f * a[1] * a[6]))))))))))))) + (fmaf(-0.24234408140182495f, a[23] * a[28], fmaf(0.2093656063079834f, a[21] * a[28], fmaf(-0.2039804309606552f, a[18] * a[33], fmaf(0.2681698799133301f, a[16] * a[35], fmaf(-0.20515984296798706f, a[14] * a[19], fmaf(-0.2293756902217865f, a[11] * a[22], fmaf(0.23504012823104858f, a[9] * a[24], fmaf(-0.2913462519645691f, a[8] * a[11], fmaf(0.45463693141937256f, a[6] * a[29], fmaf(-0.23032943904399872f, a[5] * a[14], fmaf(0.18806318938732147f, a[4] * a[15], fmaf(0.4768272340297699f, a[2] * a[19], 0.11679834127426147f * a[1] * a[8])))))))))))) + fmaf(-0.2681698799133301f, a[24] * a[25], fmaf(0.2039804309606552f, a[22] * a[27], fmaf(0.019154991954565048f, a[19] * a[30], fmaf(0.24234408140182495f, a[17] * a[32], fmaf(-0.23504012823104858f, a[15] * a[16], fmaf(0.19864517450332642f, a[12] * a[19], fmaf(0.20515984296798706f, a[10] * a[21], fmaf(0.28351593017578125f, a[8] * a[27], fmaf(0.23032943904399872f, a[7] * a[10], fmaf(-0.33886635303497314f, a[5] * a[30], fmaf(-0.13124237954616547f, a[4] * a[31], fmaf(-0.11679834127426147f, a[3] * a[4], -0.3015720248222351f * a[1] * a[20]))))))))))))));
-        o[12] = ((fmaf(-0.4154469966888428f, a[24] * a[34], fmaf(0.2967478632926941f, a[20] * a[30], fmaf(-0.4154469966888428f, a[16] * a[26], fmaf(0.3077397644519806f, a[12] * a[20], fmaf(0.28351593017578125f, a[8] * a[32], fmaf(0.4792293906211853f, a[6] * a[30], fmaf(0.28351593017578125f, a[4] * a[28], fmaf(0.4924650490283966f, a[2] * a[20], 0.564189612865448f * a[0] * a[12])))))))) + fmaf(0.23017893731594086f, a[21] * a[31], fmaf(-0.2077234983444214f, a[17] * a[27], fmaf(0.19864517450332642f, a[13] * a[21], fmaf(-0.40710145235061646f, a[9] * a[17], fmaf(0.11894160509109497f, a[7] * a[13], fmaf(0.11894160509109497f, a[5] * a[11], fmaf(-0.28609633445739746f, a[3] * a[7], -0.28609633445739746f * a[1] * a[5])))))))) + (fmaf(0.04532898589968681f, a[22] * a[32], fmaf(0.04532898589968681f, a[18] * a[28], fmaf(-0.08883681893348694f, a[14] * a[22], fmaf(-0.08883681893348694f, a[10] * a[18], fmaf(0.4286358058452606f, a[7] * a[31], fmaf(0.4286358058452606f, a[5] * a[29], fmaf(0.3893277943134308f, a[3] * a[21], 0.3893277943134308f * a[1] * a[19]))))))) + fmaf(-0.2077234983444214f, a[23] * a[33], fmaf(0.23017893731594086f, a[19] * a[29], fmaf(-0.40710145235061646f, a[15] * a[23], fmaf(0.19864517450332642f, a[11] * a[19], fmaf(-0.37612637877464294f, a[8] * a[14], fmaf(0.33641767501831055f, a[6] * a[12], fmaf(-0.37612637877464294f, a[4] * a[10], 0.49553337693214417f * a[2] * a[6])))))))));
-        o[13] = ((fmaf(-0.2681698799133301f, a[24] * a[35], fmaf(0.2039804309606552f, a[22] * a[33], fmaf(0.17203983664512634f, a[20] * a[31], fmaf(0.24234408140182495f, a[17] * a[28], fmaf(-0.23504012823104858f, a[15] * a[24], fmaf(0.2293756902217865f, a[13] * a[22], fmaf(0.20515984296798706f, a[10] * a[19], fmaf(0.28351593017578125f, a[8] * a[33], fmaf(0.34723469614982605f, a[7] * a[32], fmaf(0.45463693141937256f, a[6] * a[31], fmaf(-0.13124237954616547f, a[4] * a[29], fmaf(0.33716776967048645f, a[3] * a[22], fmaf(0.4768272340297699f, a[2] * a[21], 0.564189612865448f * a[0] * a[13]))))))))))))) + fmaf(0.24234408140182495f, a[23] * a[32], fmaf(0.019154991954565048f, a[21] * a[30], fmaf(0.2039804309606552f, a[18] * a[27], fmaf(-0.2681698799133301f, a[16] * a[25], fmaf(0.20515984296798706f, a[14] * a[21], fmaf(0.2293756902217865f, a[11] * a[18], fmaf(-0.23504012823104858f, a[9] * a[16], fmaf(0.2913462519645691f, a[8] * a[13], fmaf(0.11894160509109497f, a[7] * a[12], fmaf(0.23032943904399872f, a[5] * a[10], fmaf(-0.18806318938732147f, a[4] * a[9], fmaf(0.4046013057231903f, a[3] * a[6], -0.11679834127426147f * a[1] * a[4]))))))))))))) + (fmaf(0.0599646121263504f, a[23] * a[34], fmaf(0.2093656063079834f, a[21] * a[32], fmaf(0.15037991106510162f, a[18] * a[29], fmaf(0.2398584485054016f, a[16] * a[27], fmaf(0.13570047914981842f, a[14] * a[23], fmaf(0.19864517450332642f, a[12] * a[21], fmaf(0.2665104568004608f, a[9] * a[18], fmaf(-0.18806318938732147f, a[8] * a[15], fmaf(0.23032943904399872f, a[7] * a[14], fmaf(0.34723469614982605f, a[5] * a[28], fmaf(0.2913462519645691f, a[4] * a[11], fmaf(-0.11679834127426147f, a[3] * a[8], 0.33716776967048645f * a[1] * a[18])))))))))))) + fmaf(0.2398584485054016f, a[24] * a[33], fmaf(0.15037991106510162f, a[22] * a[31], fmaf(0.2093656063079834f, a[19] * a[28], fmaf(0.0599646121263504f, a[17] * a[26], fmaf(0.2665104568004608f, a[15] * a[22], fmaf(0.051289960741996765f, a[13] * a[20], fmaf(0.13570047914981842f, a[10] * a[17], fmaf(-0.13124237954616547f, a[8] * a[31], fmaf(-0.33886635303497314f, a[7] * a[30], fmaf(0.2523132562637329f, a[6] * a[13], fmaf(0.28351593017578125f, a[4] * a[27], fmaf(-0.3015720248222351f, a[3] * a[20], 0.4671933650970459f * a[2] * a[7]))))))))))))));
-        o[14] = ((fmaf(0.2998230457305908f, a[23] * a[35], fmaf(0.050679344683885574f, a[21] * a[33], fmaf(0.050679344683885574f, a[19] * a[27], fmaf(-0.15482795238494873f, a[16] * a[28], fmaf(0.13570047914981842f, a[13] * a[23], fmaf(0.13570047914981842f, a[11] * a[17], fmaf(0.10715895146131516f, a[8] * a[30], fmaf(0.2973540127277374f, a[7] * a[15], fmaf(0.3586224317550659f, a[5] * a[27], fmaf(0.3989422917366028f, a[3] * a[23], fmaf(0.36934879422187805f, a[2] * a[8], 0.564189612865448f * a[0] * a[14]))))))))))) + fmaf(-0.15482795238494873f, a[24] * a[32], fmaf(-0.34265491366386414f, a[22] * a[30], fmaf(-0.19549982249736786f, a[19] * a[29], fmaf(0.2998230457305908f, a[17] * a[25], fmaf(-0.35902974009513855f, a[14] * a[20], fmaf(-0.20515984296798706f, a[11] * a[19], fmaf(0.38037654757499695f, a[8] * a[34], fmaf(-0.16600993275642395f, a[7] * a[31], fmaf(0.16600993275642395f, a[5] * a[29], fmaf(0.38037654757499695f, a[4] * a[26], fmaf(0.4264872372150421f, a[2] * a[22], -0.36934879422187805f * a[1] * a[5])))))))))))) + (fmaf(0.2027173787355423f, a[22] * a[34], fmaf(-0.13085350394248962f, a[20] * a[32], fmaf(-0.22758731245994568f, a[17] * a[29], fmaf(0.3034355044364929f, a[14] * a[24], fmaf(-0.08883681893348694f, a[12] * a[22], fmaf(-0.19864517450332642f, a[9] * a[19], fmaf(0.3586224317550659f, a[7] * a[33], fmaf(0.38037654757499695f, a[6] * a[32], fmaf(0.2973540127277374f, a[5] * a[9], fmaf(0.36934879422187805f, a[3] * a[7], 0.3989422917366028f * a[1] * a[17])))))))))) + fmaf(-0.22758731245994568f, a[23] * a[31], fmaf(0.19549982249736786f, a[21] * a[31], fmaf(0.2027173787355423f, a[18] * a[26], fmaf(-0.19864517450332642f, a[15] * a[21], fmaf(0.20515984296798706f, a[13] * a[21], fmaf(0.3034355044364929f, a[10] * a[16], fmaf(-0.37612637877464294f, a[8] * a[12], fmaf(0.23032943904399872f, a[7] * a[13], fmaf(-0.23032943904399872f, a[5] * a[11], fmaf(-0.15078601241111755f, a[3] * a[21], 0.15078601241111755f * a[1] * a[19]))))))))))));
-        o[15] = ((fmaf(0.19628025591373444f, a[23] * a[30], fmaf(0.2533967196941376f, a[21] * a[32], fmaf(0.20316937565803528f, a[18] * a[29], fmaf(-0.19864517450332642f, a[14] * a[21], fmaf(-0.2665104568004608f, a[11] * a[18], fmaf(0.033886633813381195f, a[8] * a[31], fmaf(0.2973540127277374f, a[7] * a[14], fmaf(0.3105761408805847f, a[5] * a[26], fmaf(0.18806318938732147f, a[4] * a[11], fmaf(0.3257350027561188f, a[2] * a[23], 0.564189612865448f * a[0] * a[15])))))))))) + fmaf(0.07167141884565353f, a[24] * a[31], fmaf(-0.2633376121520996f, a[21] * a[34], fmaf(-0.2633376121520996f, a[19] * a[26], fmaf(0.1538698822259903f, a[15] * a[20], fmaf(-0.40710145235061646f, a[12] * a[23], fmaf(0.49106401205062866f, a[8] * a[35], fmaf(-0.08965560793876648f, a[7] * a[32], fmaf(0.08965560793876648f, a[5] * a[28], fmaf(0.49106401205062866f, a[4] * a[25], fmaf(0.45235803723335266f, a[3] * a[8], -0.45235803723335266f * a[1] * a[4]))))))))))) + (fmaf(-0.20316937565803528f, a[22] * a[31], fmaf(-0.2533967196941376f, a[19] * a[28], fmaf(0.07167141884565353f, a[16] * a[29], fmaf(0.2665104568004608f, a[13] * a[22], fmaf(0.19864517450332642f, a[10] * a[19], fmaf(0.3105761408805847f, a[7] * a[34], fmaf(-0.4205220937728882f, a[6] * a[15], fmaf(-0.033886633813381195f, a[4] * a[29], fmaf(-0.08705634623765945f, a[3] * a[22], 0.46065887808799744f * a[1] * a[16]))))))))) + fmaf(-0.19628025591373444f, a[22] * a[35], fmaf(-0.39256051182746887f, a[20] * a[33], fmaf(-0.19628025591373444f, a[18] * a[25], fmaf(-0.23504012823104858f, a[13] * a[24], fmaf(-0.23504012823104858f, a[11] * a[16], fmaf(-0.18806318938732147f, a[8] * a[13], fmaf(0.2535843551158905f, a[6] * a[33], fmaf(-0.2973540127277374f, a[5] * a[10], fmaf(0.46065887808799744f, a[3] * a[24], 0.08705634623765945f * a[1] * a[18])))))))))));
-        o[16] = ((fmaf(-0.2377071976661682f, a[27] * a[31], fmaf(0.2700909376144409f, a[18] * a[22], fmaf(-0.15482795238494873f, a[14] * a[28], fmaf(0.2681698799133301f, a[11] * a[35], fmaf(0.3034355044364929f, a[10] * a[14], fmaf(0.2809267044067383f, a[7] * a[17], fmaf(0.4768272340297699f, a[4] * a[8], fmaf(0.29463839530944824f, a[2] * a[26], 0.564189612865448f * a[0] * a[16])))))))) + fmaf(0.2567531168460846f, a[28] * a[32], fmaf(-0.23819781839847565f, a[19] * a[23], fmaf(0.07167141884565353f, a[15] * a[29], fmaf(-0.4154469966888428f, a[12] * a[26], fmaf(-0.15482795238494873f, a[10] * a[32], fmaf(-0.15016163885593414f, a[8] * a[18], fmaf(-0.15016163885593414f, a[4] * a[22], fmaf(0.46065887808799744f, a[3] * a[9], 0.46065887808799744f * a[1] * a[15]))))))))) + (fmaf(-0.2377071976661682f, a[29] * a[33], fmaf(0.10630588978528976f, a[25] * a[31], fmaf(0.21305061876773834f, a[16] * a[20], fmaf(-0.2681698799133301f, a[13] * a[25], fmaf(-0.23504012823104858f, a[11] * a[15], fmaf(-0.23504012823104858f, a[9] * a[13], fmaf(0.2809267044067383f, a[5] * a[23], fmaf(0.4658642113208771f, a[3] * a[25], -0.06944693624973297f * a[1] * a[33])))))))) + fmaf(-0.10630588978528976f, a[29] * a[35], fmaf(0.26039519906044006f, a[26] * a[30], fmaf(-0.23819781839847565f, a[17] * a[21], fmaf(0.2398584485054016f, a[13] * a[27], fmaf(0.2398584485054016f, a[11] * a[33], fmaf(0.07167141884565353f, a[9] * a[31], fmaf(-0.458751380443573f, a[6] * a[16], fmaf(-0.06944693624973297f, a[3] * a[27], -0.4658642113208771f * a[1] * a[35]))))))))));
-        o[17] = ((fmaf(0.19888010621070862f, a[28] * a[35], fmaf(-0.19888010621070862f, a[25] * a[32], fmaf(-0.3195759057998657f, a[17] * a[20], fmaf(0.24234408140182495f, a[13] * a[28], fmaf(0.24234408140182495f, a[11] * a[32], fmaf(0.13570047914981842f, a[10] * a[13], fmaf(0.26545077562332153f, a[7] * a[18], fmaf(0.26545077562332153f, a[5] * a[22], fmaf(-0.12028562277555466f, a[3] * a[28], fmaf(0.3257350027561188f, a[2] * a[9], 0.564189612865448f * a[0] * a[17])))))))))) + fmaf(0.06862016022205353f, a[29] * a[32], fmaf(-0.2377071976661682f, a[26] * a[31], fmaf(0.09003031253814697f, a[18] * a[21], fmaf(0.2998230457305908f, a[14] * a[25], fmaf(-0.0599646121263504f, a[11] * a[34], fmaf(-0.22758731245994568f, a[10] * a[31], fmaf(-0.22524245083332062f, a[8] * a[19], fmaf(-0.2809267044067383f, a[5] * a[24], fmaf(0.33716776967048645f, a[4] * a[7], fmaf(0.39285120368003845f, a[2] * a[27], 0.3989422917366028f * a[1] * a[14]))))))))))) + (fmaf(0.2377071976661682f, a[29] * a[34], fmaf(-0.26039519906044006f, a[27] * a[30], fmaf(0.09003031253814697f, a[19] * a[22], fmaf(-0.22758731245994568f, a[14] * a[29], fmaf(-0.2077234983444214f, a[12] * a[27], fmaf(-0.2998230457305908f, a[10] * a[35], fmaf(-0.40710145235061646f, a[9] * a[12], fmaf(-0.11468784511089325f, a[6] * a[17], fmaf(-0.22524245083332062f, a[4] * a[21], fmaf(0.3989422917366028f, a[3] * a[10], -0.12028562277555466f * a[1] * a[32])))))))))) + fmaf(0.06862016022205353f, a[28] * a[31], fmaf(0.23819781839847565f, a[19] * a[24], fmaf(-0.23819781839847565f, a[16] * a[21], fmaf(0.0599646121263504f, a[13] * a[26], fmaf(0.13570047914981842f, a[11] * a[14], fmaf(0.19628025591373444f, a[9] * a[30], fmaf(0.2809267044067383f, a[7] * a[16], fmaf(0.33716776967048645f, a[5] * a[8], fmaf(0.4166816174983978f, a[3] * a[26], -0.4166816174983978f * a[1] * a[34])))))))))));
-        o[18] = ((fmaf(0.19408711791038513f, a[29] * a[31], fmaf(0.16808436810970306f, a[26] * a[32], fmaf(-0.2700909376144409f, a[18] * a[24], fmaf(0.20316937565803528f, a[15] * a[29], fmaf(0.2039804309606552f, a[13] * a[27], fmaf(-0.2665104568004608f, a[11] * a[15], fmaf(-0.08883681893348694f, a[10] * a[12], fmaf(-0.15016163885593414f, a[8] * a[16], fmaf(-0.26545077562332153f, a[5] * a[23], fmaf(-0.38072922825813293f, a[4] * a[20], fmaf(0.33716776967048645f, a[3] * a[11], fmaf(-0.3674786388874054f, a[1] * a[33], 0.564189612865448f * a[0] * a[18])))))))))))) + fmaf(-0.26039519906044006f, a[27] * a[35], fmaf(0.20416957139968872f, a[19] * a[21], fmaf(0.2700909376144409f, a[16] * a[22], fmaf(0.15037991106510162f, a[13] * a[29], fmaf(0.15037991106510162f, a[11] * a[31], fmaf(-0.34265491366386414f, a[10] * a[30], fmaf(0.2665104568004608f, a[9] * a[13], fmaf(0.13107182085514069f, a[6] * a[18], fmaf(0.15016163885593414f, a[4] * a[24], fmaf(0.3674786388874054f, a[3] * a[27], fmaf(0.4264872372150421f, a[2] * a[10], 0.33716776967048645f * a[1] * a[13])))))))))))) + (fmaf(-0.19888010621070862f, a[28] * a[30], fmaf(-0.09003031253814697f, a[19] * a[23], fmaf(0.09003031253814697f, a[17] * a[21], fmaf(0.2027173787355423f, a[14] * a[26], fmaf(-0.2039804309606552f, a[11] * a[33], fmaf(-0.2027173787355423f, a[10] * a[34], fmaf(-0.20316937565803528f, a[9] * a[31], fmaf(0.26545077562332153f, a[7] * a[17], fmaf(0.360447496175766f, a[5] * a[7], fmaf(-0.1701095551252365f, a[3] * a[29], fmaf(0.45006757974624634f, a[2] * a[28], 0.08705634623765945f * a[1] * a[15]))))))))))) + fmaf(-0.16808436810970306f, a[28] * a[34], fmaf(0.26039519906044006f, a[25] * a[33], fmaf(-0.1673969030380249f, a[18] * a[20], fmaf(-0.19628025591373444f, a[15] * a[25], fmaf(0.04532898589968681f, a[12] * a[28], fmaf(0.2293756902217865f, a[11] * a[13], fmaf(0.19628025591373444f, a[9] * a[35], fmaf(0.18059572577476501f, a[7] * a[19], fmaf(0.18059572577476501f, a[5] * a[21], fmaf(0.31215670704841614f, a[4] * a[6], fmaf(-0.08705634623765945f, a[3] * a[9], -0.1701095551252365f * a[1] * a[31])))))))))))));
-        o[19] = ((fmaf(-0.16808436810970306f, a[28] * a[33], fmaf(-0.26039519906044006f, a[25] * a[34], fmaf(0.20416957139968872f, a[18] * a[21], fmaf(-0.2533967196941376f, a[15] * a[28], fmaf(0.2093656063079834f, a[13] * a[28], fmaf(-0.20515984296798706f, a[11] * a[14], fmaf(0.19864517450332642f, a[10] * a[15], fmaf(-0.19864517450332642f, a[9] * a[14], fmaf(0.2785276174545288f, a[6] * a[19], fmaf(0.44145622849464417f, a[5] * a[6], fmaf(0.31824585795402527f, a[3] * a[28], fmaf(-0.31824585795402527f, a[1] * a[32], 0.564189612865448f * a[0] * a[19])))))))))))) + fmaf(0.10630588978528976f, a[29] * a[30], fmaf(0.26039519906044006f, a[26] * a[35], fmaf(-0.09003031253814697f, a[18] * a[23], fmaf(-0.23819781839847565f, a[16] * a[23], fmaf(0.050679344683885574f, a[14] * a[27], fmaf(0.019154991954565048f, a[11] * a[30], fmaf(0.19549982249736786f, a[10] * a[31], fmaf(0.2533967196941376f, a[9] * a[32], fmaf(0.18059572577476501f, a[7] * a[18], fmaf(0.12743744254112244f, a[5] * a[8], fmaf(-0.12743744254112244f, a[4] * a[7], fmaf(0.4768272340297699f, a[2] * a[11], 0.3893277943134308f * a[1] * a[12]))))))))))))) + (fmaf(-0.18155187368392944f, a[29] * a[32], fmaf(0.16808436810970306f, a[27] * a[32], fmaf(0.13696110248565674f, a[19] * a[20], fmaf(0.09003031253814697f, a[17] * a[22], fmaf(-0.19549982249736786f, a[14] * a[29], fmaf(-0.2093656063079834f, a[11] * a[32], fmaf(-0.050679344683885574f, a[10] * a[33], fmaf(0.2633376121520996f, a[9] * a[34], fmaf(-0.22524245083332062f, a[8] * a[17], fmaf(0.08973874151706696f, a[5] * a[20], fmaf(0.2837788164615631f, a[4] * a[21], fmaf(0.48114249110221863f, a[2] * a[29], 0.15078601241111755f * a[1] * a[14])))))))))))) + fmaf(0.18155187368392944f, a[28] * a[31], fmaf(-0.20416957139968872f, a[19] * a[22], fmaf(0.23819781839847565f, a[17] * a[24], fmaf(-0.2633376121520996f, a[15] * a[26], fmaf(0.23017893731594086f, a[12] * a[29], fmaf(0.19864517450332642f, a[11] * a[12], fmaf(0.20515984296798706f, a[10] * a[13], fmaf(-0.2837788164615631f, a[8] * a[19], fmaf(-0.18059572577476501f, a[5] * a[22], fmaf(0.22524245083332062f, a[4] * a[23], fmaf(-0.15078601241111755f, a[3] * a[10], -0.3105761408805847f * a[1] * a[30])))))))))))));
-        o[20] = ((fmaf(-0.13019759953022003f, a[33] * a[33], fmaf(0.08679839968681335f, a[29] * a[29], fmaf(0.13019759953022003f, a[25] * a[25], fmaf(0.06848055124282837f, a[21] * a[21], fmaf(-0.15978795289993286f, a[17] * a[17], fmaf(-0.13085350394248962f, a[14] * a[32], fmaf(0.2967478632926941f, a[12] * a[30], fmaf(-0.13085350394248962f, a[10] * a[28], fmaf(-0.38072922825813293f, a[8] * a[22], fmaf(0.3276795446872711f, a[6] * a[20], fmaf(-0.38072922825813293f, a[4] * a[18], fmaf(0.49106401205062866f, a[2] * a[30], 0.564189612865448f * a[0] * a[20])))))))))))) + fmaf(-0.13019759953022003f, a[34] * a[34], fmaf(0.13019759953022003f, a[30] * a[30], fmaf(-0.13019759953022003f, a[26] * a[26], fmaf(-0.08369845151901245f, a[22] * a[22], fmaf(-0.08369845151901245f, a[18] * a[18], fmaf(0.07693494111299515f, a[15] * a[15], fmaf(0.025644980370998383f, a[13] * a[13], fmaf(0.025644980370998383f, a[11] * a[11], fmaf(0.07693494111299515f, a[9] * a[9], fmaf(-0.1611970216035843f, a[7] * a[7], fmaf(-0.1611970216035843f, a[5] * a[5], fmaf(-0.3015720248222351f, a[3] * a[13], -0.3015720248222351f * a[1] * a[11]))))))))))))) + (fmaf(0.13019759953022003f, a[35] * a[35], fmaf(0.08679839968681335f, a[31] * a[31], fmaf(-0.13019759953022003f, a[27] * a[27], fmaf(-0.15978795289993286f, a[23] * a[23], fmaf(0.06848055124282837f, a[19] * a[19], fmaf(-0.39256051182746887f, a[15] * a[33], fmaf(0.17203983664512634f, a[13] * a[31], fmaf(0.17203983664512634f, a[11] * a[29], fmaf(-0.39256051182746887f, a[9] * a[27], fmaf(0.08973874151706696f, a[7] * a[21], fmaf(0.08973874151706696f, a[5] * a[19], fmaf(0.38037654757499695f, a[3] * a[31], 0.38037654757499695f * a[1] * a[29])))))))))))) + fmaf(-0.02169959992170334f, a[32] * a[32], fmaf(-0.02169959992170334f, a[28] * a[28], fmaf(0.10652530938386917f, a[24] * a[24], fmaf(0.13696110248565674f, a[20] * a[20], fmaf(0.10652530938386917f, a[16] * a[16], fmaf(-0.17951487004756927f, a[14] * a[14], fmaf(0.1538698822259903f, a[12] * a[12], fmaf(-0.17951487004756927f, a[10] * a[10], fmaf(0.04029925540089607f, a[8] * a[8], fmaf(0.24179553985595703f, a[6] * a[6], fmaf(0.04029925540089607f, a[4] * a[4], 0.4924650490283966f * a[2] * a[12])))))))))))));
-        o[21] = ((fmaf(0.18155187368392944f, a[31] * a[32], fmaf(-0.26039519906044006f, a[25] * a[26], fmaf(0.13696110248565674f, a[20] * a[21], fmaf(-0.2633376121520996f, a[15] * a[34], fmaf(-0.19864517450332642f, a[14] * a[15], fmaf(0.23017893731594086f, a[12] * a[31], fmaf(0.050679344683885574f, a[10] * a[27], fmaf(-0.19864517450332642f, a[9] * a[10], fmaf(0.08973874151706696f, a[7] * a[20], fmaf(0.18059572577476501f, a[5] * a[18], fmaf(0.31824585795402527f, a[3] * a[32], fmaf(0.48114249110221863f, a[2] * a[31], 0.564189612865448f * a[0] * a[21])))))))))))) + fmaf(0.16808436810970306f, a[32] * a[33], fmaf(0.16808436810970306f, a[27] * a[28], fmaf(0.20416957139968872f, a[21] * a[22], fmaf(-0.23819781839847565f, a[16] * a[17], fmaf(0.19549982249736786f, a[14] * a[31], fmaf(0.20515984296798706f, a[13] * a[14], fmaf(0.19549982249736786f, a[10] * a[29], fmaf(-0.2633376121520996f, a[9] * a[26], fmaf(0.18059572577476501f, a[7] * a[22], fmaf(0.44145622849464417f, a[6] * a[7], fmaf(-0.12743744254112244f, a[4] * a[5], fmaf(0.3893277943134308f, a[3] * a[12], -0.15078601241111755f * a[1] * a[10]))))))))))))) + (fmaf(-0.26039519906044006f, a[34] * a[35], fmaf(0.18155187368392944f, a[28] * a[29], fmaf(0.09003031253814697f, a[22] * a[23], fmaf(0.09003031253814697f, a[17] * a[18], fmaf(0.050679344683885574f, a[14] * a[33], fmaf(0.019154991954565048f, a[13] * a[30], fmaf(0.2093656063079834f, a[11] * a[28], fmaf(0.2533967196941376f, a[9] * a[28], fmaf(0.2837788164615631f, a[8] * a[21], fmaf(0.2785276174545288f, a[6] * a[21], fmaf(-0.22524245083332062f, a[4] * a[17], fmaf(-0.15078601241111755f, a[3] * a[14], 0.31824585795402527f * a[1] * a[28])))))))))))) + fmaf(0.10630588978528976f, a[30] * a[31], fmaf(-0.23819781839847565f, a[23] * a[24], fmaf(0.20416957139968872f, a[18] * a[19], fmaf(0.2533967196941376f, a[15] * a[32], fmaf(0.2093656063079834f, a[13] * a[32], fmaf(0.19864517450332642f, a[12] * a[13], fmaf(0.20515984296798706f, a[10] * a[11], fmaf(-0.22524245083332062f, a[8] * a[23], fmaf(-0.12743744254112244f, a[7] * a[8], fmaf(0.2837788164615631f, a[4] * a[19], fmaf(-0.3105761408805847f, a[3] * a[30], 0.4768272340297699f * a[2] * a[13])))))))))))));
-        o[22] = ((fmaf(0.26039519906044006f, a[33] * a[35], fmaf(-0.09704355895519257f, a[29] * a[29], fmaf(0.09003031253814697f, a[21] * a[23], fmaf(0.09003031253814697f, a[17] * a[19], fmaf(0.2027173787355423f, a[14] * a[34], fmaf(0.2665104568004608f, a[13] * a[15], fmaf(-0.15037991106510162f, a[11] * a[29], fmaf(-0.20316937565803528f, a[9] * a[29], fmaf(-0.38072922825813293f, a[8] * a[20], fmaf(0.13107182085514069f, a[6] * a[22], fmaf(-0.180223748087883f, a[5] * a[5], fmaf(-0.08705634623765945f, a[3] * a[15], fmaf(0.1701095551252365f, a[1] * a[29], 0.564189612865448f * a[0] * a[22]))))))))))))) + fmaf(-0.19888010621070862f, a[30] * a[32], fmaf(0.2700909376144409f, a[22] * a[24], fmaf(-0.10208478569984436f, a[19] * a[19], fmaf(-0.20316937565803528f, a[15] * a[31], fmaf(0.15037991106510162f, a[13] * a[31], fmaf(-0.08883681893348694f, a[12] * a[14], fmaf(0.2027173787355423f, a[10] * a[26], fmaf(-0.15016163885593414f, a[8] * a[24], fmaf(0.180223748087883f, a[7] * a[7], fmaf(0.26545077562332153f, a[5] * a[17], fmaf(-0.1701095551252365f, a[3] * a[31], fmaf(0.4264872372150421f, a[2] * a[14], -0.08705634623765945f * a[1] * a[9]))))))))))))) + (fmaf(0.09704355895519257f, a[31] * a[31], fmaf(0.26039519906044006f, a[25] * a[27], fmaf(-0.1673969030380249f, a[20] * a[22], fmaf(-0.19628025591373444f, a[15] * a[35], fmaf(0.2039804309606552f, a[13] * a[33], fmaf(0.04532898589968681f, a[12] * a[32], fmaf(-0.11468784511089325f, a[11] * a[11], fmaf(0.2665104568004608f, a[9] * a[11], fmaf(0.18059572577476501f, a[7] * a[21], fmaf(-0.18059572577476501f, a[5] * a[19], fmaf(0.3674786388874054f, a[3] * a[33], fmaf(0.45006757974624634f, a[2] * a[32], -0.33716776967048645f * a[1] * a[11])))))))))))) + fmaf(0.16808436810970306f, a[32] * a[34], fmaf(0.16808436810970306f, a[26] * a[28], fmaf(0.10208478569984436f, a[21] * a[21], fmaf(0.2700909376144409f, a[16] * a[18], fmaf(-0.34265491366386414f, a[14] * a[30], fmaf(0.11468784511089325f, a[13] * a[13], fmaf(0.2039804309606552f, a[11] * a[27], fmaf(-0.19628025591373444f, a[9] * a[25], fmaf(0.26545077562332153f, a[7] * a[23], fmaf(0.31215670704841614f, a[6] * a[8], fmaf(-0.15016163885593414f, a[4] * a[16], fmaf(0.33716776967048645f, a[3] * a[13], 0.3674786388874054f * a[1] * a[27]))))))))))))));
-        o[23] = ((fmaf(0.06862016022205353f, a[31] * a[32], fmaf(-0.19888010621070862f, a[25] * a[28], fmaf(-0.09003031253814697f, a[18] * a[19], fmaf(-0.22758731245994568f, a[14] * a[31], fmaf(-0.2077234983444214f, a[12] * a[33], fmaf(0.22758731245994568f, a[10] * a[29], fmaf(0.2809267044067383f, a[7] * a[24], fmaf(-0.26545077562332153f, a[5] * a[18], fmaf(0.4166816174983978f, a[3] * a[34], fmaf(0.3257350027561188f, a[2] * a[15], 0.564189612865448f * a[0] * a[23])))))))))) + fmaf(-0.2377071976661682f, a[31] * a[34], fmaf(-0.2377071976661682f, a[26] * a[29], fmaf(-0.3195759057998657f, a[20] * a[23], fmaf(0.2998230457305908f, a[14] * a[35], fmaf(0.13570047914981842f, a[13] * a[14], fmaf(0.0599646121263504f, a[11] * a[26], fmaf(-0.22524245083332062f, a[8] * a[21], fmaf(-0.11468784511089325f, a[6] * a[23], fmaf(-0.33716776967048645f, a[4] * a[5], fmaf(0.39285120368003845f, a[2] * a[33], -0.3989422917366028f * a[1] * a[10]))))))))))) + (fmaf(-0.19888010621070862f, a[32] * a[35], fmaf(-0.06862016022205353f, a[28] * a[29], fmaf(0.09003031253814697f, a[21] * a[22], fmaf(0.19628025591373444f, a[15] * a[30], fmaf(0.24234408140182495f, a[13] * a[32], fmaf(-0.24234408140182495f, a[11] * a[28], fmaf(-0.13570047914981842f, a[10] * a[11], fmaf(0.33716776967048645f, a[7] * a[8], fmaf(0.22524245083332062f, a[4] * a[19], fmaf(0.3989422917366028f, a[3] * a[14], 0.4166816174983978f * a[1] * a[26])))))))))) + fmaf(-0.26039519906044006f, a[30] * a[33], fmaf(-0.23819781839847565f, a[21] * a[24], fmaf(-0.23819781839847565f, a[16] * a[19], fmaf(0.0599646121263504f, a[13] * a[34], fmaf(-0.40710145235061646f, a[12] * a[15], fmaf(0.2998230457305908f, a[10] * a[25], fmaf(0.26545077562332153f, a[7] * a[22], fmaf(0.2809267044067383f, a[5] * a[16], fmaf(-0.12028562277555466f, a[3] * a[32], 0.12028562277555466f * a[1] * a[28])))))))))));
-        o[24] = ((fmaf(0.26039519906044006f, a[30] * a[34], fmaf(0.13504546880722046f, a[22] * a[22], fmaf(0.23819781839847565f, a[17] * a[19], fmaf(-0.2681698799133301f, a[13] * a[35], fmaf(-0.2398584485054016f, a[11] * a[27], fmaf(-0.07167141884565353f, a[9] * a[29], fmaf(0.2809267044067383f, a[7] * a[23], fmaf(-0.23841361701488495f, a[4] * a[4], fmaf(0.29463839530944824f, a[2] * a[34], 0.564189612865448f * a[0] * a[24]))))))))) + fmaf(-0.2377071976661682f, a[31] * a[33], fmaf(0.10630588978528976f, a[25] * a[29], fmaf(-0.13504546880722046f, a[18] * a[18], fmaf(0.15171775221824646f, a[14] * a[14], fmaf(-0.4154469966888428f, a[12] * a[34], fmaf(-0.15171775221824646f, a[10] * a[10], fmaf(0.23841361701488495f, a[8] * a[8], fmaf(0.15016163885593414f, a[4] * a[18], fmaf(0.46065887808799744f, a[3] * a[15], -0.46065887808799744f * a[1] * a[9])))))))))) + (fmaf(0.10630588978528976f, a[31] * a[35], fmaf(0.2377071976661682f, a[27] * a[29], fmaf(0.21305061876773834f, a[20] * a[24], fmaf(-0.15482795238494873f, a[14] * a[32], fmaf(-0.23504012823104858f, a[13] * a[15], fmaf(0.15482795238494873f, a[10] * a[28], fmaf(-0.15016163885593414f, a[8] * a[22], fmaf(-0.2809267044067383f, a[5] * a[17], fmaf(-0.06944693624973297f, a[3] * a[33], 0.4658642113208771f * a[1] * a[25]))))))))) + fmaf(0.1283765584230423f, a[32] * a[32], fmaf(-0.1283765584230423f, a[28] * a[28], fmaf(-0.23819781839847565f, a[21] * a[23], fmaf(0.07167141884565353f, a[15] * a[31], fmaf(0.2398584485054016f, a[13] * a[33], fmaf(-0.2681698799133301f, a[11] * a[25], fmaf(0.23504012823104858f, a[9] * a[11], fmaf(-0.458751380443573f, a[6] * a[24], fmaf(0.4658642113208771f, a[3] * a[35], 0.06944693624973297f * a[1] * a[27])))))))))));
-        o[25] = ((fmaf(0.10630588978528976f, a[24] * a[29], fmaf(0.26039519906044006f, a[20] * a[25], fmaf(0.10630588978528976f, a[16] * a[31], fmaf(-0.2681698799133301f, a[11] * a[24], fmaf(0.49106401205062866f, a[8] * a[9], fmaf(-0.12528268992900848f, a[4] * a[33], 0.564189612865448f * a[0] * a[25])))))) + fmaf(-0.26039519906044006f, a[21] * a[26], fmaf(-0.19888010621070862f, a[17] * a[32], fmaf(-0.2681698799133301f, a[13] * a[16], fmaf(-0.12528268992900848f, a[8] * a[27], fmaf(0.2657647430896759f, a[5] * a[34], 0.4658642113208771f * a[1] * a[24])))))) + (fmaf(0.26039519906044006f, a[22] * a[27], fmaf(0.26039519906044006f, a[18] * a[33], fmaf(0.2998230457305908f, a[14] * a[17], fmaf(-0.19628025591373444f, a[9] * a[22], fmaf(-0.48521777987480164f, a[6] * a[25], 0.4658642113208771f * a[3] * a[16]))))) + fmaf(-0.19888010621070862f, a[23] * a[28], fmaf(-0.26039519906044006f, a[19] * a[34], fmaf(-0.19628025591373444f, a[15] * a[18], fmaf(0.2998230457305908f, a[10] * a[23], fmaf(0.2657647430896759f, a[7] * a[26], 0.49106401205062866f * a[4] * a[15])))))));
-        o[26] = ((fmaf(0.16808436810970306f, a[22] * a[28], fmaf(0.16808436810970306f, a[18] * a[32], fmaf(0.2027173787355423f, a[14] * a[18], fmaf(0.2027173787355423f, a[10] * a[22], fmaf(0.2773250639438629f, a[7] * a[27], fmaf(-0.2657647430896759f, a[5] * a[35], fmaf(0.38037654757499695f, a[4] * a[14], 0.564189612865448f * a[0] * a[26]))))))) + fmaf(-0.2377071976661682f, a[23] * a[29], fmaf(0.26039519906044006f, a[19] * a[35], fmaf(-0.2633376121520996f, a[15] * a[19], fmaf(0.0599646121263504f, a[11] * a[23], fmaf(0.38037654757499695f, a[8] * a[10], fmaf(-0.19408711791038513f, a[6] * a[26], fmaf(-0.19408711791038513f, a[4] * a[32], 0.4166816174983978f * a[1] * a[23])))))))) + (fmaf(-0.26039519906044006f, a[20] * a[26], fmaf(0.26039519906044006f, a[16] * a[30], fmaf(-0.4154469966888428f, a[12] * a[16], fmaf(-0.19408711791038513f, a[8] * a[28], fmaf(0.3105761408805847f, a[7] * a[9], fmaf(0.3105761408805847f, a[5] * a[15], 0.29463839530944824f * a[2] * a[16])))))) + fmaf(-0.26039519906044006f, a[21] * a[25], fmaf(-0.2377071976661682f, a[17] * a[31], fmaf(0.0599646121263504f, a[13] * a[17], fmaf(-0.2633376121520996f, a[9] * a[21], fmaf(0.2657647430896759f, a[7] * a[25], fmaf(0.2773250639438629f, a[5] * a[33], 0.4166816174983978f * a[3] * a[17]))))))));
-        o[27] = ((fmaf(-0.26039519906044006f, a[20] * a[27], fmaf(-0.2377071976661682f, a[16] * a[31], fmaf(-0.2077234983444214f, a[12] * a[17], fmaf(-0.39256051182746887f, a[9] * a[20], fmaf(0.2287338674068451f, a[7] * a[28], fmaf(0.2535843551158905f, a[6] * a[9], fmaf(0.12528268992900848f, a[4] * a[35], fmaf(-0.06944693624973297f, a[3] * a[16], 0.564189612865448f * a[0] * a[27])))))))) + fmaf(0.16808436810970306f, a[21] * a[28], fmaf(-0.26039519906044006f, a[17] * a[30], fmaf(0.2398584485054016f, a[13] * a[16], fmaf(0.050679344683885574f, a[10] * a[21], fmaf(0.28351593017578125f, a[8] * a[11], fmaf(0.03234785422682762f, a[6] * a[27], fmaf(0.3586224317550659f, a[5] * a[14], fmaf(0.3674786388874054f, a[3] * a[18], 0.3674786388874054f * a[1] * a[22]))))))))) + (fmaf(0.26039519906044006f, a[22] * a[25], fmaf(-0.26039519906044006f, a[18] * a[35], fmaf(0.2039804309606552f, a[13] * a[18], fmaf(0.2039804309606552f, a[11] * a[22], fmaf(-0.12528268992900848f, a[8] * a[25], fmaf(0.3586224317550659f, a[7] * a[10], fmaf(0.2287338674068451f, a[5] * a[32], fmaf(0.28351593017578125f, a[4] * a[13], 0.06944693624973297f * a[1] * a[24])))))))) + fmaf(0.2377071976661682f, a[24] * a[29], fmaf(0.16808436810970306f, a[19] * a[32], fmaf(0.050679344683885574f, a[14] * a[19], fmaf(-0.2398584485054016f, a[11] * a[24], fmaf(-0.24206916987895966f, a[8] * a[29], fmaf(0.2773250639438629f, a[7] * a[26], fmaf(-0.2773250639438629f, a[5] * a[34], fmaf(-0.24206916987895966f, a[4] * a[31], 0.39285120368003845f * a[2] * a[17]))))))))));
-        o[28] = ((fmaf(0.16808436810970306f, a[22] * a[26], fmaf(-0.16808436810970306f, a[19] * a[33], fmaf(0.19888010621070862f, a[17] * a[35], fmaf(-0.15482795238494873f, a[14] * a[16], fmaf(-0.24234408140182495f, a[11] * a[23], fmaf(0.2533967196941376f, a[9] * a[21], fmaf(0.34723469614982605f, a[7] * a[11], fmaf(-0.2287338674068451f, a[5] * a[33], fmaf(0.19408711791038513f, a[4] * a[34], fmaf(-0.12028562277555466f, a[3] * a[17], 0.564189612865448f * a[0] * a[28])))))))))) + fmaf(-0.19888010621070862f, a[23] * a[25], fmaf(-0.04339919984340668f, a[20] * a[28], fmaf(-0.19888010621070862f, a[18] * a[30], fmaf(-0.2533967196941376f, a[15] * a[19], fmaf(0.04532898589968681f, a[12] * a[18], fmaf(-0.13085350394248962f, a[10] * a[20], fmaf(0.2287338674068451f, a[7] * a[27], fmaf(0.38037654757499695f, a[6] * a[10], fmaf(0.34723469614982605f, a[5] * a[13], fmaf(0.31824585795402527f, a[3] * a[19], 0.31824585795402527f * a[1] * a[21]))))))))))) + (fmaf(-0.06862016022205353f, a[23] * a[29], fmaf(0.16808436810970306f, a[21] * a[27], fmaf(-0.16808436810970306f, a[18] * a[34], fmaf(0.2567531168460846f, a[16] * a[32], fmaf(0.24234408140182495f, a[13] * a[17], fmaf(0.15482795238494873f, a[10] * a[24], fmaf(0.148236483335495f, a[7] * a[29], fmaf(0.19408711791038513f, a[6] * a[28], fmaf(0.08965560793876648f, a[5] * a[15], fmaf(0.28351593017578125f, a[4] * a[12], 0.12028562277555466f * a[1] * a[23])))))))))) + fmaf(-0.2567531168460846f, a[24] * a[28], fmaf(0.18155187368392944f, a[21] * a[29], fmaf(0.18155187368392944f, a[19] * a[31], fmaf(0.06862016022205353f, a[17] * a[31], fmaf(0.2093656063079834f, a[13] * a[19], fmaf(0.2093656063079834f, a[11] * a[21], fmaf(-0.19408711791038513f, a[8] * a[26], fmaf(-0.08965560793876648f, a[7] * a[9], fmaf(0.148236483335495f, a[5] * a[31], fmaf(-0.3827449679374695f, a[4] * a[30], 0.45006757974624634f * a[2] * a[18]))))))))))));
-        o[29] = ((fmaf(-0.06862016022205353f, a[23] * a[28], fmaf(0.1735967993736267f, a[20] * a[29], fmaf(0.2377071976661682f, a[17] * a[34], fmaf(0.20316937565803528f, a[15] * a[18], fmaf(0.15037991106510162f, a[13] * a[18], fmaf(0.22758731245994568f, a[10] * a[23], fmaf(-0.28014060854911804f, a[8] * a[29], fmaf(0.148236483335495f, a[7] * a[28], fmaf(-0.148236483335495f, a[5] * a[32], fmaf(0.24206916987895966f, a[4] * a[33], fmaf(-0.1701095551252365f, a[3] * a[18], 0.564189612865448f * a[0] * a[29]))))))))))) + fmaf(0.10630588978528976f, a[24] * a[25], fmaf(0.18155187368392944f, a[21] * a[28], fmaf(0.19408711791038513f, a[18] * a[31], fmaf(-0.2377071976661682f, a[16] * a[33], fmaf(-0.22758731245994568f, a[14] * a[17], fmaf(0.17203983664512634f, a[11] * a[20], fmaf(-0.20316937565803528f, a[9] * a[22], fmaf(0.033886633813381195f, a[8] * a[9], fmaf(0.45463693141937256f, a[6] * a[11], fmaf(0.4286358058452606f, a[5] * a[12], fmaf(-0.13124237954616547f, a[4] * a[13], 0.38037654757499695f * a[1] * a[20])))))))))))) + (fmaf(0.2377071976661682f, a[24] * a[27], fmaf(-0.19408711791038513f, a[22] * a[29], fmaf(0.10630588978528976f, a[19] * a[30], fmaf(-0.10630588978528976f, a[16] * a[35], fmaf(-0.19549982249736786f, a[14] * a[19], fmaf(-0.15037991106510162f, a[11] * a[22], fmaf(-0.07167141884565353f, a[9] * a[24], fmaf(0.13124237954616547f, a[8] * a[11], fmaf(0.2911306619644165f, a[6] * a[29], fmaf(0.16600993275642395f, a[5] * a[14], fmaf(-0.033886633813381195f, a[4] * a[15], 0.1701095551252365f * a[1] * a[22]))))))))))) + fmaf(-0.2377071976661682f, a[23] * a[26], fmaf(-0.18155187368392944f, a[19] * a[32], fmaf(0.06862016022205353f, a[17] * a[32], fmaf(0.07167141884565353f, a[15] * a[16], fmaf(0.23017893731594086f, a[12] * a[19], fmaf(0.19549982249736786f, a[10] * a[21], fmaf(-0.24206916987895966f, a[8] * a[27], fmaf(-0.16600993275642395f, a[7] * a[10], fmaf(0.0723319947719574f, a[5] * a[30], fmaf(0.28014060854911804f, a[4] * a[31], 0.48114249110221863f * a[2] * a[19]))))))))))));
-        o[30] = ((fmaf(-0.26039519906044006f, a[23] * a[33], fmaf(0.10630588978528976f, a[19] * a[29], fmaf(0.19628025591373444f, a[15] * a[23], fmaf(0.019154991954565048f, a[11] * a[19], fmaf(0.10715895146131516f, a[8] * a[14], fmaf(0.4792293906211853f, a[6] * a[12], fmaf(0.10715895146131516f, a[4] * a[10], 0.564189612865448f * a[0] * a[30]))))))) + fmaf(0.26039519906044006f, a[24] * a[34], fmaf(0.26039519906044006f, a[20] * a[30], fmaf(0.26039519906044006f, a[16] * a[26], fmaf(0.2967478632926941f, a[12] * a[20], fmaf(-0.3827449679374695f, a[8] * a[32], fmaf(0.3234785199165344f, a[6] * a[30], fmaf(-0.3827449679374695f, a[4] * a[28], -0.3105761408805847f * a[1] * a[19])))))))) + (fmaf(0.10630588978528976f, a[21] * a[31], fmaf(-0.26039519906044006f, a[17] * a[27], fmaf(0.019154991954565048f, a[13] * a[21], fmaf(0.19628025591373444f, a[9] * a[17], fmaf(-0.33886635303497314f, a[7] * a[13], fmaf(-0.33886635303497314f, a[5] * a[11], 0.49106401205062866f * a[2] * a[20])))))) + fmaf(-0.19888010621070862f, a[22] * a[32], fmaf(-0.19888010621070862f, a[18] * a[28], fmaf(-0.34265491366386414f, a[14] * a[22], fmaf(-0.34265491366386414f, a[10] * a[18], fmaf(0.0723319947719574f, a[7] * a[31], fmaf(0.0723319947719574f, a[5] * a[29], -0.3105761408805847f * a[3] * a[21]))))))));
-        o[31] = ((fmaf(-0.2377071976661682f, a[23] * a[34], fmaf(0.10630588978528976f, a[21] * a[30], fmaf(0.06862016022205353f, a[17] * a[28], fmaf(0.07167141884565353f, a[15] * a[24], fmaf(0.15037991106510162f, a[13] * a[22], fmaf(0.19549982249736786f, a[10] * a[19], fmaf(-0.24206916987895966f, a[8] * a[33], fmaf(0.148236483335495f, a[7] * a[32], fmaf(0.2911306619644165f, a[6] * a[31], fmaf(0.28014060854911804f, a[4] * a[29], fmaf(-0.1701095551252365f, a[3] * a[22], 0.564189612865448f * a[0] * a[31]))))))))))) + fmaf(-0.2377071976661682f, a[24] * a[33], fmaf(0.18155187368392944f, a[21] * a[32], fmaf(0.19408711791038513f, a[18] * a[29], fmaf(0.10630588978528976f, a[16] * a[25], fmaf(0.19549982249736786f, a[14] * a[21], fmaf(0.15037991106510162f, a[11] * a[18], fmaf(0.07167141884565353f, a[9] * a[16], fmaf(-0.13124237954616547f, a[8] * a[13], fmaf(0.4286358058452606f, a[7] * a[12], fmaf(-0.16600993275642395f, a[5] * a[10], fmaf(0.033886633813381195f, a[4] * a[9], -0.1701095551252365f * a[1] * a[18])))))))))))) + (fmaf(0.10630588978528976f, a[24] * a[35], fmaf(0.19408711791038513f, a[22] * a[31], fmaf(0.18155187368392944f, a[19] * a[28], fmaf(-0.2377071976661682f, a[16] * a[27], fmaf(-0.22758731245994568f, a[14] * a[23], fmaf(0.23017893731594086f, a[12] * a[21], fmaf(-0.20316937565803528f, a[9] * a[18], fmaf(0.033886633813381195f, a[8] * a[15], fmaf(-0.16600993275642395f, a[7] * a[14], fmaf(0.148236483335495f, a[5] * a[28], fmaf(-0.13124237954616547f, a[4] * a[11], 0.48114249110221863f * a[2] * a[21]))))))))))) + fmaf(0.06862016022205353f, a[23] * a[32], fmaf(0.1735967993736267f, a[20] * a[31], fmaf(-0.2377071976661682f, a[17] * a[26], fmaf(-0.20316937565803528f, a[15] * a[22], fmaf(0.17203983664512634f, a[13] * a[20], fmaf(-0.22758731245994568f, a[10] * a[17], fmaf(0.28014060854911804f, a[8] * a[31], fmaf(0.0723319947719574f, a[7] * a[30], fmaf(0.45463693141937256f, a[6] * a[13], fmaf(-0.24206916987895966f, a[4] * a[27], 0.38037654757499695f * a[3] * a[20]))))))))))));
-        o[32] = ((fmaf(0.16808436810970306f, a[22] * a[34], fmaf(-0.04339919984340668f, a[20] * a[32], fmaf(0.06862016022205353f, a[17] * a[29], fmaf(-0.15482795238494873f, a[14] * a[24], fmaf(0.04532898589968681f, a[12] * a[22], fmaf(0.2533967196941376f, a[9] * a[19], fmaf(0.2287338674068451f, a[7] * a[33], fmaf(0.19408711791038513f, a[6] * a[32], fmaf(-0.34723469614982605f, a[5] * a[11], fmaf(0.31824585795402527f, a[3] * a[21], 0.564189612865448f * a[0] * a[32])))))))))) + fmaf(0.06862016022205353f, a[23] * a[31], fmaf(0.18155187368392944f, a[21] * a[31], fmaf(0.16808436810970306f, a[18] * a[26], fmaf(0.2533967196941376f, a[15] * a[21], fmaf(0.2093656063079834f, a[13] * a[21], fmaf(-0.15482795238494873f, a[10] * a[16], fmaf(0.28351593017578125f, a[8] * a[12], fmaf(0.34723469614982605f, a[7] * a[13], fmaf(0.2287338674068451f, a[5] * a[27], fmaf(-0.12028562277555466f, a[3] * a[23], -0.12028562277555466f * a[1] * a[17]))))))))))) + (fmaf(-0.19888010621070862f, a[23] * a[35], fmaf(0.16808436810970306f, a[21] * a[33], fmaf(0.16808436810970306f, a[19] * a[27], fmaf(0.2567531168460846f, a[16] * a[28], fmaf(0.24234408140182495f, a[13] * a[23], fmaf(0.24234408140182495f, a[11] * a[17], fmaf(-0.3827449679374695f, a[8] * a[30], fmaf(-0.08965560793876648f, a[7] * a[15], fmaf(-0.148236483335495f, a[5] * a[29], fmaf(-0.19408711791038513f, a[4] * a[26], -0.31824585795402527f * a[1] * a[19])))))))))) + fmaf(0.2567531168460846f, a[24] * a[32], fmaf(-0.19888010621070862f, a[22] * a[30], fmaf(-0.18155187368392944f, a[19] * a[29], fmaf(-0.19888010621070862f, a[17] * a[25], fmaf(-0.13085350394248962f, a[14] * a[20], fmaf(-0.2093656063079834f, a[11] * a[19], fmaf(-0.19408711791038513f, a[8] * a[34], fmaf(0.148236483335495f, a[7] * a[31], fmaf(0.38037654757499695f, a[6] * a[14], fmaf(-0.08965560793876648f, a[5] * a[9], 0.45006757974624634f * a[2] * a[22]))))))))))));
-        o[33] = ((fmaf(0.16808436810970306f, a[21] * a[32], fmaf(-0.2377071976661682f, a[16] * a[29], fmaf(0.2039804309606552f, a[13] * a[22], fmaf(-0.050679344683885574f, a[10] * a[19], fmaf(0.2773250639438629f, a[7] * a[34], fmaf(0.2535843551158905f, a[6] * a[15], fmaf(0.24206916987895966f, a[4] * a[29], fmaf(0.3674786388874054f, a[3] * a[22], 0.564189612865448f * a[0] * a[33])))))))) + fmaf(0.26039519906044006f, a[22] * a[35], fmaf(0.26039519906044006f, a[18] * a[25], fmaf(0.2398584485054016f, a[13] * a[24], fmaf(0.2398584485054016f, a[11] * a[16], fmaf(0.28351593017578125f, a[8] * a[13], fmaf(0.03234785422682762f, a[6] * a[33], fmaf(-0.3586224317550659f, a[5] * a[10], fmaf(-0.06944693624973297f, a[3] * a[24], -0.06944693624973297f * a[1] * a[16]))))))))) + (fmaf(-0.26039519906044006f, a[23] * a[30], fmaf(-0.16808436810970306f, a[19] * a[28], fmaf(0.050679344683885574f, a[14] * a[21], fmaf(-0.2039804309606552f, a[11] * a[18], fmaf(-0.24206916987895966f, a[8] * a[31], fmaf(0.3586224317550659f, a[7] * a[14], fmaf(0.2773250639438629f, a[5] * a[26], fmaf(-0.28351593017578125f, a[4] * a[11], -0.3674786388874054f * a[1] * a[18])))))))) + fmaf(-0.2377071976661682f, a[24] * a[31], fmaf(-0.26039519906044006f, a[20] * a[33], fmaf(-0.39256051182746887f, a[15] * a[20], fmaf(-0.2077234983444214f, a[12] * a[23], fmaf(-0.12528268992900848f, a[8] * a[35], fmaf(0.2287338674068451f, a[7] * a[32], fmaf(-0.2287338674068451f, a[5] * a[28], fmaf(-0.12528268992900848f, a[4] * a[25], 0.39285120368003845f * a[2] * a[23]))))))))));
-        o[34] = ((fmaf(-0.2377071976661682f, a[23] * a[31], fmaf(-0.26039519906044006f, a[19] * a[25], fmaf(0.2027173787355423f, a[14] * a[22], fmaf(-0.2027173787355423f, a[10] * a[18], fmaf(0.2657647430896759f, a[7] * a[35], fmaf(-0.2773250639438629f, a[5] * a[27], fmaf(-0.38037654757499695f, a[4] * a[10], 0.564189612865448f * a[0] * a[34]))))))) + fmaf(0.26039519906044006f, a[24] * a[30], fmaf(-0.26039519906044006f, a[20] * a[34], fmaf(-0.2633376121520996f, a[15] * a[21], fmaf(-0.0599646121263504f, a[11] * a[17], fmaf(0.38037654757499695f, a[8] * a[14], fmaf(-0.19408711791038513f, a[6] * a[34], fmaf(0.19408711791038513f, a[4] * a[28], -0.4166816174983978f * a[1] * a[17])))))))) + (fmaf(-0.26039519906044006f, a[21] * a[35], fmaf(0.2377071976661682f, a[17] * a[29], fmaf(-0.4154469966888428f, a[12] * a[24], fmaf(-0.19408711791038513f, a[8] * a[32], fmaf(0.3105761408805847f, a[7] * a[15], fmaf(-0.3105761408805847f, a[5] * a[9], 0.29463839530944824f * a[2] * a[24])))))) + fmaf(0.16808436810970306f, a[22] * a[32], fmaf(-0.16808436810970306f, a[18] * a[28], fmaf(0.0599646121263504f, a[13] * a[23], fmaf(0.2633376121520996f, a[9] * a[19], fmaf(0.2773250639438629f, a[7] * a[33], fmaf(0.2657647430896759f, a[5] * a[25], 0.4166816174983978f * a[3] * a[23]))))))));
-        o[35] = ((fmaf(0.10630588978528976f, a[24] * a[31], fmaf(0.26039519906044006f, a[20] * a[35], fmaf(-0.10630588978528976f, a[16] * a[29], fmaf(0.2681698799133301f, a[11] * a[16], fmaf(0.49106401205062866f, a[8] * a[15], fmaf(0.12528268992900848f, a[4] * a[27], 0.564189612865448f * a[0] * a[35])))))) + fmaf(-0.26039519906044006f, a[21] * a[34], fmaf(0.19888010621070862f, a[17] * a[28], fmaf(-0.2681698799133301f, a[13] * a[24], fmaf(-0.12528268992900848f, a[8] * a[33], fmaf(-0.2657647430896759f, a[5] * a[26], -0.4658642113208771f * a[1] * a[16])))))) + (fmaf(0.26039519906044006f, a[22] * a[33], fmaf(-0.26039519906044006f, a[18] * a[27], fmaf(0.2998230457305908f, a[14] * a[23], fmaf(0.19628025591373444f, a[9] * a[18], fmaf(-0.48521777987480164f, a[6] * a[35], 0.4658642113208771f * a[3] * a[24]))))) + fmaf(-0.19888010621070862f, a[23] * a[32], fmaf(0.26039519906044006f, a[19] * a[26], fmaf(-0.19628025591373444f, a[15] * a[22], fmaf(-0.2998230457305908f, a[10] * a[17], fmaf(0.2657647430896759f, a[7] * a[34], -0.49106401205062866f * a[4] * a[9])))))));
+    __device__ __forceinline__ static float le_trig(int b, int h) {   // h = 2m - 1: cos(m phi_b), 2m: sin
+        switch (b * 11 + h) {
+            case 1: return 0.9914448857307434f;
+            case 2: return 0.13052618503570557f;
+            case 3: return 0.9659258127212524f;
+            case 4: return 0.258819043636322f;
+            case 5: return 0.9238795042037964f;
+            case 6: return 0.3826834261417389f;
+            case 7: return 0.8660253882408142f;
+            case 8: return 0.5f;
+            case 9: return 0.7933533191680908f;
+            case 10: return 0.6087614297866821f;
+            case 12: return 0.9238795042037964f;
+            case 13: return 0.3826834261417389f;
+            case 14: return 0.7071067690849304f;
+            case 15: return 0.7071067690849304f;
+            case 16: return 0.3826834261417389f;
+            case 17: return 0.9238795042037964f;
+            case 18: return 6.123234262925839e-17f;
+            case 19: return 1.0f;
+            case 20: return -0.3826834261417389f;
+            case 21: return 0.9238795042037964f;
+            case 23: return 0.7933533191680908f;
+            case 24: return 0.6087614297866821f;
+            case 25: return 0.258819043636322f;
+            case 26: return 0.9659258127212524f;
+            case 27: return -0.3826834261417389f;
+            case 28: return 0.9238795042037964f;
+            case 29: return -0.8660253882408142f;
+            case 30: return 0.5f;
+            case 31: return -0.9914448857307434f;
+            case 32: return -0.13052618503570557f;
+            case 34: return 0.6087614297866821f;
+            case 35: return 0.7933533191680908f;
+            case 36: return -0.258819043636322f;
+            case 37: return 0.9659258127212524f;
+            case 38: return -0.9238795042037964f;
+            case 39: return 0.3826834261417389f;
+            case 40: return -0.8660253882408142f;
+            case 41: return -0.5f;
+            case 42: return -0.13052618503570557f;
+            case 43: return -0.9914448857307434f;
+            case 45: return 0.3826834261417389f;
+            case 46: return 0.9238795042037964f;
+            case 47: return -0.7071067690849304f;
+            case 48: return 0.7071067690849304f;
+            case 49: return -0.9238795042037964f;
+            case 50: return -0.3826834261417389f;
+            case 51: return -1.8369701465288538e-16f;
+            case 52: return -1.0f;
+            case 53: return 0.9238795042037964f;
+            case 54: return -0.3826834261417389f;
+            case 56: return 0.13052618503570557f;
+            case 57: return 0.9914448857307434f;
+            case 58: return -0.9659258127212524f;
+            case 59: return 0.258819043636322f;
+            case 60: return -0.3826834261417389f;
+            case 61: return -0.9238795042037964f;
+            case 62: return 0.8660253882408142f;
+            case 63: return -0.5f;
+            case 64: return 0.6087614297866821f;
+            case 65: return 0.7933533191680908f;
+            default: return 1.0f;
+        }
     }
 };
 
 #if defined(SHS_NB) && SHS_NB == 7
-static __constant__ float kQuadLeg7[490] = {0.282094806432724f, 0.11088809370994568f, -0.47585317492485046f, 0.11088809370994568f, 0.028136439621448517f, -0.24148334562778473f, 0.5820493698120117f, -0.24148334562778473f, 0.028136439621448517f, 0.006897183135151863f, -0.07249957323074341f, 0.3881925940513611f, -0.6332811713218689f, 0.3881925940513611f, -0.07249957323074341f, 0.006897183135151863f, 0.0016602643299847841f, -0.020151635631918907f, 0.13741593062877655f, -0.5381947755813599f, 0.6381627321243286f, -0.5381947755813599f, 0.13741593062877655f, -0.020151635631918907f, 0.0016602643299847841f, 0.0003951871476601809f, -0.005362791009247303f, 0.043099742382764816f, -0.2218766212463379f, 0.6798455715179443f, -0.6017029285430908f, 0.6798455715179443f, -0.2218766212463379f, 0.043099742382764816f, -0.005362791009247303f, 0.0003951871476601809f, 9.33497358346358e-05f, -0.0013876877492293715f, 0.012627102434635162f, -0.07795622199773788f, 0.3230060040950775f, -0.802699089050293f, 0.528781533241272f, -0.802699089050293f, 0.3230060040950775f, -0.07795622199773788f, 0.012627102434635162f, -0.0013876877492293715f, 9.33497358346358e-05f, 0.282094806432724f, 0.24511361122131348f, -0.4226721227169037f, 0.24511361122131348f, 0.137478306889534f, -0.4741331934928894f, 0.39266371726989746f, -0.4741331934928894f, 0.137478306889534f, 0.0744936540722847f, -0.3146524429321289f, 0.6286184787750244f, -0.23942779004573822f, 0.6286184787750244f, -0.3146524429321289f, 0.0744936540722847f, 0.039637595415115356f, -0.1933251917362213f, 0.5046157836914062f, -0.6498939394950867f, 0.015881182625889778f, -0.6498939394950867f, 0.5046157836914062f, -0.1933251917362213f, 0.039637595415115356f, 0.020855247974395752f, -0.11372384428977966f, 0.3542337715625763f, -0.6496331095695496f, 0.5188519954681396f, 0.2127721607685089f, 0.5188519954681396f, -0.6496331095695496f, 0.3542337715625763f, -0.11372384428977966f, 0.020855247974395752f, 0.010889505036175251f, -0.06504815071821213f, 0.23110173642635345f, -0.5263574719429016f, 0.6966809034347534f, -0.2604548931121826f, -0.3827480673789978f, -0.2604548931121826f, 0.6966809034347534f, -0.5263574719429016f, 0.23110173642635345f, -0.06504815071821213f, 0.010889505036175251f, 0.282094806432724f, 0.3585166037082672f, -0.3319612145423889f, 0.3585166037082672f, 0.29411548376083374f, -0.5446605682373047f, 0.1213601753115654f, -0.5446605682373047f, 0.29411548376083374f, 0.23310139775276184f, -0.5286869406700134f, 0.438648521900177f, 0.17545272409915924f, 0.438648521900177f, -0.5286869406700134f, 0.23310139775276184f, 0.1814156323671341f, -0.47511395812034607f, 0.5683075189590454f, -0.07710716128349304f, -0.3586549460887909f, -0.07710716128349304f, 0.5683075189590454f, -0.47511395812034607f, 0.1814156323671341f, 0.13961261510849f, -0.40879231691360474f, 0.6096698641777039f, -0.3373580276966095f, -0.3283151686191559f, 0.3089510500431061f, -0.3283151686191559f, -0.3373580276966095f, 0.6096698641777039f, -0.40879231691360474f, 0.13961261510849f, 0.10662505775690079f, -0.34200146794319153f, 0.5963935256004333f, -0.5136942267417908f, -0.06878549605607986f, 0.5276145935058594f, -0.05914037674665451f, 0.5276145935058594f, -0.06878549605607986f, -0.5136942267417908f, 0.5963935256004333f, -0.34200146794319153f, 0.10662505775690079f, 0.282094806432724f, 0.44033047556877136f, -0.2117580771446228f, 0.44033047556877136f, 0.4436666667461395f, -0.42672494053840637f, -0.13767008483409882f, -0.42672494053840637f, 0.4436666667461395f, 0.4318702220916748f, -0.5087332725524902f, -0.025060366839170456f, 0.3333059847354889f, -0.025060366839170456f, -0.5087332725524902f, 0.4318702220916748f, 0.4128122329711914f, -0.5615116953849792f, 0.12096259742975235f, 0.440361887216568f, -0.1481127291917801f, 0.440361887216568f, 0.12096259742975235f, -0.5615116953849792f, 0.4128122329711914f, 0.39018625020980835f, -0.5933803915977478f, 0.24725398421287537f, 0.3682527244091034f, -0.3627842366695404f, -0.20651771128177643f, -0.3627842366695404f, 0.3682527244091034f, 0.24725398421287537f, -0.5933803915977478f, 0.39018625020980835f, 0.36599576473236084f, -0.6097164750099182f, 0.35483497381210327f, 0.2728903889656067f, -0.4551534950733185f, -0.12045054137706757f, 0.32672613859176636f, -0.12045054137706757f, -0.4551534950733185f, 0.2728903889656067f, 0.35483497381210327f, -0.6097164750099182f, 0.36599576473236084f, 0.282094806432724f, 0.48315757513046265f, -0.07274037599563599f, 0.48315757513046265f, 0.5341668128967285f, -0.16083984076976776f, -0.2944209575653076f, -0.16083984076976776f, 0.5341668128967285f, 0.5705364942550659f, -0.21040001511573792f, -0.40186813473701477f, 0.1605125069618225f, -0.40186813473701477f, -0.21040001511573792f, 0.5705364942550659f, 0.598401665687561f, -0.2548147141933441f, -0.3908316493034363f, 0.2802008390426636f, 0.24883784353733063f, 0.2802008390426636f, -0.3908316493034363f, -0.2548147141933441f, 0.598401665687561f, 0.6206149458885193f, -0.29546698927879333f, -0.37870079278945923f, 0.3257097601890564f, 0.31354087591171265f, -0.23469020426273346f, 0.31354087591171265f, 0.3257097601890564f, -0.37870079278945923f, -0.29546698927879333f, 0.6206149458885193f, 0.6387580633163452f, -0.33313000202178955f, -0.36482664942741394f, 0.36549919843673706f, 0.2780129909515381f, -0.3732146918773651f, -0.17958590388298035f, -0.3732146918773651f, 0.2780129909515381f, 0.36549919843673706f, -0.36482664942741394f, -0.33313000202178955f, 0.6387580633163452f, 0.282094806432724f, 0.48315757513046265f, 0.07274037599563599f, 0.48315757513046265f, 0.5341668128967285f, 0.16083984076976776f, -0.2944209575653076f, 0.16083984076976776f, 0.5341668128967285f, 0.5705364942550659f, 0.21040001511573792f, -0.40186813473701477f, -0.1605125069618225f, -0.40186813473701477f, 0.21040001511573792f, 0.5705364942550659f, 0.598401665687561f, 0.2548147141933441f, -0.3908316493034363f, -0.2802008390426636f, 0.24883784353733063f, -0.2802008390426636f, -0.3908316493034363f, 0.2548147141933441f, 0.598401665687561f, 0.6206149458885193f, 0.29546698927879333f, -0.37870079278945923f, -0.3257097601890564f, 0.31354087591171265f, 0.23469020426273346f, 0.31354087591171265f, -0.3257097601890564f, -0.37870079278945923f, 0.29546698927879333f, 0.6206149458885193f, 0.6387580633163452f, 0.33313000202178955f, -0.36482664942741394f, -0.36549919843673706f, 0.2780129909515381f, 0.3732146918773651f, -0.17958590388298035f, 0.3732146918773651f, 0.2780129909515381f, -0.36549919843673706f, -0.36482664942741394f, 0.33313000202178955f, 0.6387580633163452f, 0.282094806432724f, 0.44033047556877136f, 0.2117580771446228f, 0.44033047556877136f, 0.4436666667461395f, 0.42672494053840637f, -0.13767008483409882f, 0.42672494053840637f, 0.4436666667461395f, 0.4318702220916748f, 0.5087332725524902f, -0.025060366839170456f, -0.3333059847354889f, -0.025060366839170456f, 0.5087332725524902f, 0.4318702220916748f, 0.4128122329711914f, 0.5615116953849792f, 0.12096259742975235f, -0.440361887216568f, -0.1481127291917801f, -0.440361887216568f, 0.12096259742975235f, 0.5615116953849792f, 0.4128122329711914f, 0.39018625020980835f, 0.5933803915977478f, 0.24725398421287537f, -0.3682527244091034f, -0.3627842366695404f, 0.20651771128177643f, -0.3627842366695404f, -0.3682527244091034f, 0.24725398421287537f, 0.5933803915977478f, 0.39018625020980835f, 0.36599576473236084f, 0.6097164750099182f, 0.35483497381210327f, -0.2728903889656067f, -0.4551534950733185f, 0.12045054137706757f, 0.32672613859176636f, 0.12045054137706757f, -0.4551534950733185f, -0.2728903889656067f, 0.35483497381210327f, 0.6097164750099182f, 0.36599576473236084f, 0.282094806432724f, 0.3585166037082672f, 0.3319612145423889f, 0.3585166037082672f, 0.29411548376083374f, 0.5446605682373047f, 0.1213601753115654f, 0.5446605682373047f, 0.29411548376083374f, 0.23310139775276184f, 0.5286869406700134f, 0.438648521900177f, -0.17545272409915924f, 0.438648521900177f, 0.5286869406700134f, 0.23310139775276184f, 0.1814156323671341f, 0.47511395812034607f, 0.5683075189590454f, 0.07710716128349304f, -0.3586549460887909f, 0.07710716128349304f, 0.5683075189590454f, 0.47511395812034607f, 0.1814156323671341f, 0.13961261510849f, 0.40879231691360474f, 0.6096698641777039f, 0.3373580276966095f, -0.3283151686191559f, -0.3089510500431061f, -0.3283151686191559f, 0.3373580276966095f, 0.6096698641777039f, 0.40879231691360474f, 0.13961261510849f, 0.10662505775690079f, 0.34200146794319153f, 0.5963935256004333f, 0.5136942267417908f, -0.06878549605607986f, -0.5276145935058594f, -0.05914037674665451f, -0.5276145935058594f, -0.06878549605607986f, 0.5136942267417908f, 0.5963935256004333f, 0.34200146794319153f, 0.10662505775690079f, 0.282094806432724f, 0.24511361122131348f, 0.4226721227169037f, 0.24511361122131348f, 0.137478306889534f, 0.4741331934928894f, 0.39266371726989746f, 0.4741331934928894f, 0.137478306889534f, 0.0744936540722847f, 0.3146524429321289f, 0.6286184787750244f, 0.23942779004573822f, 0.6286184787750244f, 0.3146524429321289f, 0.0744936540722847f, 0.039637595415115356f, 0.1933251917362213f, 0.5046157836914062f, 0.6498939394950867f, 0.015881182625889778f, 0.6498939394950867f, 0.5046157836914062f, 0.1933251917362213f, 0.039637595415115356f, 0.020855247974395752f, 0.11372384428977966f, 0.3542337715625763f, 0.6496331095695496f, 0.5188519954681396f, -0.2127721607685089f, 0.5188519954681396f, 0.6496331095695496f, 0.3542337715625763f, 0.11372384428977966f, 0.020855247974395752f, 0.010889505036175251f, 0.06504815071821213f, 0.23110173642635345f, 0.5263574719429016f, 0.6966809034347534f, 0.2604548931121826f, -0.3827480673789978f, 0.2604548931121826f, 0.6966809034347534f, 0.5263574719429016f, 0.23110173642635345f, 0.06504815071821213f, 0.010889505036175251f, 0.282094806432724f, 0.11088809370994568f, 0.47585317492485046f, 0.11088809370994568f, 0.028136439621448517f, 0.24148334562778473f, 0.5820493698120117f, 0.24148334562778473f, 0.028136439621448517f, 0.006897183135151863f, 0.07249957323074341f, 0.3881925940513611f, 0.6332811713218689f, 0.3881925940513611f, 0.07249957323074341f, 0.006897183135151863f, 0.0016602643299847841f, 0.020151635631918907f, 0.13741593062877655f, 0.5381947755813599f, 0.6381627321243286f, 0.5381947755813599f, 0.13741593062877655f, 0.020151635631918907f, 0.0016602643299847841f, 0.0003951871476601809f, 0.005362791009247303f, 0.043099742382764816f, 0.2218766212463379f, 0.6798455715179443f, 0.6017029285430908f, 0.6798455715179443f, 0.2218766212463379f, 0.043099742382764816f, 0.005362791009247303f, 0.0003951871476601809f, 9.33497358346358e-05f, 0.0013876877492293715f, 0.012627102434635162f, 0.07795622199773788f, 0.3230060040950775f, 0.802699089050293f, 0.528781533241272f, 0.802699089050293f, 0.3230060040950775f, 0.07795622199773788f, 0.012627102434635162f, 0.0013876877492293715f, 9.33497358346358e-05f};
-static __constant__ float kQuadTrig7[247] = {1.0f, 0.9863613247871399f, 0.1645945906639099f, 0.945817232131958f, 0.3246994614601135f, 0.8794737458229065f, 0.47594738006591797f, 0.789140522480011f, 0.614212691783905f, 0.6772815585136414f, 0.7357239127159119f, 0.5469481348991394f, 0.8371664881706238f, 1.0f, 0.8794737458229065f, 0.47594738006591797f, 0.5469481348991394f, 0.8371664881706238f, 0.0825793445110321f, 0.9965844750404358f, -0.4016954302787781f, 0.915773332118988f, -0.789140522480011f, 0.614212691783905f, -0.9863613247871399f, 0.1645945906639099f, 1.0f, 0.6772815585136414f, 0.7357239127159119f, -0.0825793445110321f, 0.9965844750404358f, -0.789140522480011f, 0.614212691783905f, -0.9863613247871399f, -0.1645945906639099f, -0.5469481348991394f, -0.8371664881706238f, 0.24548548460006714f, -0.9694002866744995f, 1.0f, 0.4016954302787781f, 0.915773332118988f, -0.6772815585136414f, 0.7357239127159119f, -0.945817232131958f, -0.3246994614601135f, -0.0825793445110321f, -0.9965844750404358f, 0.8794737458229065f, -0.47594738006591797f, 0.789140522480011f, 0.614212691783905f, 1.0f, 0.0825793445110321f, 0.9965844750404358f, -0.9863613247871399f, 0.1645945906639099f, -0.24548548460006714f, -0.9694002866744995f, 0.945817232131958f, -0.3246994614601135f, 0.4016954302787781f, 0.915773332118988f, -0.8794737458229065f, 0.47594738006591797f, 1.0f, -0.24548548460006714f, 0.9694002866744995f, -0.8794737458229065f, -0.47594738006591797f, 0.6772815585136414f, -0.7357239127159119f, 0.5469481348991394f, 0.8371664881706238f, -0.945817232131958f, 0.3246994614601135f, -0.0825793445110321f, -0.9965844750404358f, 1.0f, -0.5469481348991394f, 0.8371664881706238f, -0.4016954302787781f, -0.915773332118988f, 0.9863613247871399f, 0.1645945906639099f, -0.6772815585136414f, 0.7357239127159119f, -0.24548548460006714f, -0.9694002866744995f, 0.945817232131958f, 0.3246994614601135f, 1.0f, -0.789140522480011f, 0.614212691783905f, 0.24548548460006714f, -0.9694002866744995f, 0.4016954302787781f, 0.915773332118988f, -0.8794737458229065f, -0.47594738006591797f, 0.9863613247871399f, -0.1645945906639099f, -0.6772815585136414f, 0.7357239127159119f, 1.0f, -0.945817232131958f, 0.3246994614601135f, 0.789140522480011f, -0.614212691783905f, -0.5469481348991394f, 0.8371664881706238f, 0.24548548460006714f, -0.9694002866744995f, 0.0825793445110321f, 0.9965844750404358f, -0.4016954302787781f, -0.915773332118988f, 1.0f, -1.0f, 1.2246468525851679e-16f, 1.0f, -2.4492937051703357e-16f, -1.0f, 3.6739402930577075e-16f, 1.0f, -4.898587410340671e-16f, -1.0f, 6.123233998228043e-16f, 1.0f, -7.347880586115415e-16f, 1.0f, -0.945817232131958f, -0.3246994614601135f, 0.789140522480011f, 0.614212691783905f, -0.5469481348991394f, -0.8371664881706238f, 0.24548548460006714f, 0.9694002866744995f, 0.0825793445110321f, -0.9965844750404358f, -0.4016954302787781f, 0.915773332118988f, 1.0f, -0.789140522480011f, -0.614212691783905f, 0.24548548460006714f, 0.9694002866744995f, 0.4016954302787781f, -0.915773332118988f, -0.8794737458229065f, 0.47594738006591797f, 0.9863613247871399f, 0.1645945906639099f, -0.6772815585136414f, -0.7357239127159119f, 1.0f, -0.5469481348991394f, -0.8371664881706238f, -0.4016954302787781f, 0.915773332118988f, 0.9863613247871399f, -0.1645945906639099f, -0.6772815585136414f, -0.7357239127159119f, -0.24548548460006714f, 0.9694002866744995f, 0.945817232131958f, -0.3246994614601135f, 1.0f, -0.24548548460006714f, -0.9694002866744995f, -0.8794737458229065f, 0.47594738006591797f, 0.6772815585136414f, 0.7357239127159119f, 0.5469481348991394f, -0.8371664881706238f, -0.945817232131958f, -0.3246994614601135f, -0.0825793445110321f, 0.9965844750404358f, 1.0f, 0.0825793445110321f, -0.9965844750404358f, -0.9863613247871399f, -0.1645945906639099f, -0.24548548460006714f, 0.9694002866744995f, 0.945817232131958f, 0.3246994614601135f, 0.4016954302787781f, -0.915773332118988f, -0.8794737458229065f, -0.47594738006591797f, 1.0f, 0.4016954302787781f, -0.915773332118988f, -0.6772815585136414f, -0.7357239127159119f, -0.945817232131958f, 0.3246994614601135f, -0.0825793445110321f, 0.9965844750404358f, 0.8794737458229065f, 0.47594738006591797f, 0.789140522480011f, -0.614212691783905f, 1.0f, 0.6772815585136414f, -0.7357239127159119f, -0.0825793445110321f, -0.9965844750404358f, -0.789140522480011f, -0.614212691783905f, -0.9863613247871399f, 0.1645945906639099f, -0.5469481348991394f, 0.8371664881706238f, 0.24548548460006714f, 0.9694002866744995f, 1.0f, 0.8794737458229065f, -0.47594738006591797f, 0.5469481348991394f, -0.8371664881706238f, 0.0825793445110321f, -0.9965844750404358f, -0.4016954302787781f, -0.915773332118988f, -0.789140522480011f, -0.614212691783905f, -0.9863613247871399f, -0.1645945906639099f, 1.0f, 0.9863613247871399f, -0.1645945906639099f, 0.945817232131958f, -0.3246994614601135f, 0.8794737458229065f, -0.47594738006591797f, 0.789140522480011f, -0.614212691783905f, 0.6772815585136414f, -0.7357239127159119f, 0.5469481348991394f, -0.8371664881706238f};
-static __constant__ float kQuadW7[10] = {0.02204781025648117f, 0.04942265897989273f, 0.07245054095983505f, 0.08904487639665604f, 0.09772807359695435f, 0.09772807359695435f, 0.08904487639665604f, 0.07245054095983505f, 0.04942265897989273f, 0.02204781025648117f};
-#endif
-#if defined(SHS_NB) && SHS_NB == 7
-static __constant__ float kExpLeg7[686] = {0.282094806432724f, 0.08064790815114975f, -0.48190075159072876f, 0.08064790815114975f, 0.014882830902934074f, -0.17786070704460144f, 0.6050053238868713f, -0.17786070704460144f, 0.014882830902934074f, 0.00265336106531322f, -0.03883617743849754f, 0.2914804220199585f, -0.6859782338142395f, 0.2914804220199585f, -0.03883617743849754f, 0.00265336106531322f, 0.000464526005089283f, -0.00785090122371912f, 0.07487541437149048f, -0.4148964583873749f, 0.7337506413459778f, -0.4148964583873749f, 0.07487541437149048f, -0.00785090122371912f, 0.000464526005089283f, 8.041624823817983e-05f, -0.0015195264713838696f, 0.017060957849025726f, -0.12354122847318649f, 0.5422344207763672f, -0.7521823048591614f, 0.5422344207763672f, -0.12354122847318649f, 0.017060957849025726f, -0.0015195264713838696f, 8.041624823817983e-05f, 1.3815361853630748e-05f, -0.0002859679516404867f, 0.003632891923189163f, -0.03146146610379219f, 0.18467740714550018f, -0.6680772304534912f, 0.7436875104904175f, -0.6680772304534912f, 0.18467740714550018f, -0.03146146610379219f, 0.003632891923189163f, -0.0002859679516404867f, 1.3815361853630748e-05f, 0.282094806432724f, 0.1815134733915329f, -0.4536356031894684f, 0.1815134733915329f, 0.07539057731628418f, -0.3768298625946045f, 0.5002028346061707f, -0.3768298625946045f, 0.07539057731628418f, 0.03025127202272415f, -0.18519000709056854f, 0.5619985461235046f, -0.4538605809211731f, 0.5619985461235046f, -0.18519000709056854f, 0.03025127202272415f, 0.01191991288214922f, -0.08425901085138321f, 0.32866668701171875f, -0.700112521648407f, 0.33283063769340515f, -0.700112521648407f, 0.32866668701171875f, -0.08425901085138321f, 0.01191991288214922f, 0.004644325003027916f, -0.03670463338494301f, 0.169509157538414f, -0.4870571792125702f, 0.7632161974906921f, -0.15976978838443756f, 0.7632161974906921f, -0.4870571792125702f, 0.169509157538414f, -0.03670463338494301f, 0.004644325003027916f, 0.0017957952804863453f, -0.015546969138085842f, 0.08151230216026306f, -0.2842300832271576f, 0.6359331011772156f, -0.7355261445045471f, -0.037704091519117355f, -0.7355261445045471f, 0.6359331011772156f, -0.2842300832271576f, 0.08151230216026306f, -0.015546969138085842f, 0.0017957952804863453f, 0.282094806432724f, 0.2745485305786133f, -0.4041726291179657f, 0.2745485305786133f, 0.1724795252084732f, -0.5078264474868774f, 0.33203983306884766f, -0.5078264474868774f, 0.1724795252084732f, 0.1046825647354126f, -0.3774833381175995f, 0.6218326687812805f, -0.1300550252199173f, 0.6218326687812805f, -0.3774833381175995f, 0.1046825647354126f, 0.062389861792325974f, -0.2597806453704834f, 0.5660937428474426f, -0.5566006898880005f, -0.1206328421831131f, -0.5566006898880005f, 0.5660937428474426f, -0.2597806453704834f, 0.062389861792325974f, 0.03676832094788551f, -0.17116761207580566f, 0.4477361738681793f, -0.6590285897254944f, 0.31886351108551025f, 0.32900097966194153f, 0.31886351108551025f, -0.6590285897254944f, 0.4477361738681793f, -0.17116761207580566f, 0.03676832094788551f, 0.021503949537873268f, -0.10966213047504425f, 0.3283042311668396f, -0.6120079755783081f, 0.6012592911720276f, 0.020793095231056213f, -0.4215880334377289f, 0.020793095231056213f, 0.6012592911720276f, -0.6120079755783081f, 0.3283042311668396f, -0.10966213047504425f, 0.021503949537873268f, 0.282094806432724f, 0.35491126775741577f, -0.335813045501709f, 0.35491126775741577f, 0.2882298231124878f, -0.545439600944519f, 0.13155442476272583f, -0.545439600944519f, 0.2882298231124878f, 0.22613950073719025f, -0.5241189002990723f, 0.45212191343307495f, 0.16367165744304657f, 0.45212191343307495f, -0.5241189002990723f, 0.22613950073719025f, 0.1742275357246399f, -0.4662722051143646f, 0.5757606625556946f, -0.10240838676691055f, -0.35559025406837463f, -0.10240838676691055f, 0.5757606625556946f, -0.4662722051143646f, 0.1742275357246399f, 0.13273249566555023f, -0.3971503973007202f, 0.6096431016921997f, -0.36253634095191956f, -0.3051152229309082f, 0.32220059633255005f, -0.3051152229309082f, -0.36253634095191956f, 0.6096431016921997f, -0.3971503973007202f, 0.13273249566555023f, 0.10035116225481033f, -0.3289203643798828f, 0.5894106030464172f, -0.5328931212425232f, -0.03383835777640343f, 0.5257964134216309f, -0.08521328866481781f, 0.5257964134216309f, -0.03383835777640343f, -0.5328931212425232f, 0.5894106030464172f, -0.3289203643798828f, 0.10035116225481033f, 0.282094806432724f, 0.4187522530555725f, -0.25175178050994873f, 0.4187522530555725f, 0.4012486934661865f, -0.4824574589729309f, -0.0642000138759613f, -0.4824574589729309f, 0.4012486934661865f, 0.3714398741722107f, -0.546990156173706f, 0.12824709713459015f, 0.32160407304763794f, 0.12824709713459015f, -0.546990156173706f, 0.3714398741722107f, 0.3376496136188507f, -0.5741516351699829f, 0.2982756793498993f, 0.33728790283203125f, -0.2642127573490143f, 0.33728790283203125f, 0.2982756793498993f, -0.5741516351699829f, 0.3376496136188507f, 0.30350375175476074f, -0.5770047903060913f, 0.42788830399513245f, 0.18464216589927673f, -0.4800601899623871f, -0.0516158863902092f, -0.4800601899623871f, 0.18464216589927673f, 0.42788830399513245f, -0.5770047903060913f, 0.30350375175476074f, 0.27073636651039124f, -0.5638357400894165f, 0.5227455496788025f, 0.023816371336579323f, -0.4915175139904022f, 0.16429507732391357f, 0.3176251947879791f, 0.16429507732391357f, -0.4915175139904022f, 0.023816371336579323f, 0.5227455496788025f, -0.5638357400894165f, 0.27073636651039124f, 0.282094806432724f, 0.46305686235427856f, -0.15591910481452942f, 0.46305686235427856f, 0.4906456470489502f, -0.3304174244403839f, -0.21904003620147705f, -0.3304174244403839f, 0.4906456470489502f, 0.5022500157356262f, -0.41424816846847534f, -0.21260583400726318f, 0.296621710062027f, -0.21260583400726318f, -0.41424816846847534f, 0.5022500157356262f, 0.504864513874054f, -0.4808225631713867f, -0.12202231585979462f, 0.4627828299999237f, 0.03257828578352928f, 0.4627828299999237f, -0.12202231585979462f, -0.4808225631713867f, 0.504864513874054f, 0.5018221139907837f, -0.5343364477157593f, -0.03477540984749794f, 0.477090060710907f, -0.0892399251461029f, -0.31815603375434875f, -0.0892399251461029f, 0.477090060710907f, -0.03477540984749794f, -0.5343364477157593f, 0.5018221139907837f, 0.4950048625469208f, -0.5773844718933105f, 0.04890919476747513f, 0.47038865089416504f, -0.2030356377363205f, -0.4030117094516754f, 0.16972026228904724f, -0.4030117094516754f, -0.2030356377363205f, 0.47038865089416504f, 0.04890919476747513f, -0.5773844718933105f, 0.4950048625469208f, 0.282094806432724f, 0.4857417047023773f, -0.05279592052102089f, 0.4857417047023773f, 0.5398960113525391f, -0.11736404150724411f, -0.30434414744377136f, -0.11736404150724411f, 0.5398960113525391f, 0.5797399282455444f, -0.15434898436069489f, -0.42784395813941956f, 0.11861658841371536f, -0.42784395813941956f, -0.15434898436069489f, 0.5797399282455444f, 0.6113067269325256f, -0.18793129920959473f, -0.4293491542339325f, 0.20973744988441467f, 0.280807226896286f, 0.20973744988441467f, -0.4293491542339325f, -0.18793129920959473f, 0.6113067269325256f, 0.6373898983001709f, -0.21907870471477509f, -0.4301821291446686f, 0.24699321389198303f, 0.377977579832077f, -0.1793360412120819f, 0.377977579832077f, 0.24699321389198303f, -0.4301821291446686f, -0.21907870471477509f, 0.6373898983001709f, 0.6595321297645569f, -0.24832561612129211f, -0.4295520782470703f, 0.28084641695022583f, 0.36160001158714294f, -0.29129156470298767f, -0.24261875450611115f, -0.29129156470298767f, 0.36160001158714294f, 0.28084641695022583f, -0.4295520782470703f, -0.24832561612129211f, 0.6595321297645569f, 0.282094806432724f, 0.4857417047023773f, 0.05279592052102089f, 0.4857417047023773f, 0.5398960113525391f, 0.11736404150724411f, -0.30434414744377136f, 0.11736404150724411f, 0.5398960113525391f, 0.5797399282455444f, 0.15434898436069489f, -0.42784395813941956f, -0.11861658841371536f, -0.42784395813941956f, 0.15434898436069489f, 0.5797399282455444f, 0.6113067269325256f, 0.18793129920959473f, -0.4293491542339325f, -0.20973744988441467f, 0.280807226896286f, -0.20973744988441467f, -0.4293491542339325f, 0.18793129920959473f, 0.6113067269325256f, 0.6373898983001709f, 0.21907870471477509f, -0.4301821291446686f, -0.24699321389198303f, 0.377977579832077f, 0.1793360412120819f, 0.377977579832077f, -0.24699321389198303f, -0.4301821291446686f, 0.21907870471477509f, 0.6373898983001709f, 0.6595321297645569f, 0.24832561612129211f, -0.4295520782470703f, -0.28084641695022583f, 0.36160001158714294f, 0.29129156470298767f, -0.24261875450611115f, 0.29129156470298767f, 0.36160001158714294f, -0.28084641695022583f, -0.4295520782470703f, 0.24832561612129211f, 0.6595321297645569f, 0.282094806432724f, 0.46305686235427856f, 0.15591910481452942f, 0.46305686235427856f, 0.4906456470489502f, 0.3304174244403839f, -0.21904003620147705f, 0.3304174244403839f, 0.4906456470489502f, 0.5022500157356262f, 0.41424816846847534f, -0.21260583400726318f, -0.296621710062027f, -0.21260583400726318f, 0.41424816846847534f, 0.5022500157356262f, 0.504864513874054f, 0.4808225631713867f, -0.12202231585979462f, -0.4627828299999237f, 0.03257828578352928f, -0.4627828299999237f, -0.12202231585979462f, 0.4808225631713867f, 0.504864513874054f, 0.5018221139907837f, 0.5343364477157593f, -0.03477540984749794f, -0.477090060710907f, -0.0892399251461029f, 0.31815603375434875f, -0.0892399251461029f, -0.477090060710907f, -0.03477540984749794f, 0.5343364477157593f, 0.5018221139907837f, 0.4950048625469208f, 0.5773844718933105f, 0.04890919476747513f, -0.47038865089416504f, -0.2030356377363205f, 0.4030117094516754f, 0.16972026228904724f, 0.4030117094516754f, -0.2030356377363205f, -0.47038865089416504f, 0.04890919476747513f, 0.5773844718933105f, 0.4950048625469208f, 0.282094806432724f, 0.4187522530555725f, 0.25175178050994873f, 0.4187522530555725f, 0.4012486934661865f, 0.4824574589729309f, -0.0642000138759613f, 0.4824574589729309f, 0.4012486934661865f, 0.3714398741722107f, 0.546990156173706f, 0.12824709713459015f, -0.32160407304763794f, 0.12824709713459015f, 0.546990156173706f, 0.3714398741722107f, 0.3376496136188507f, 0.5741516351699829f, 0.2982756793498993f, -0.33728790283203125f, -0.2642127573490143f, -0.33728790283203125f, 0.2982756793498993f, 0.5741516351699829f, 0.3376496136188507f, 0.30350375175476074f, 0.5770047903060913f, 0.42788830399513245f, -0.18464216589927673f, -0.4800601899623871f, 0.0516158863902092f, -0.4800601899623871f, -0.18464216589927673f, 0.42788830399513245f, 0.5770047903060913f, 0.30350375175476074f, 0.27073636651039124f, 0.5638357400894165f, 0.5227455496788025f, -0.023816371336579323f, -0.4915175139904022f, -0.16429507732391357f, 0.3176251947879791f, -0.16429507732391357f, -0.4915175139904022f, -0.023816371336579323f, 0.5227455496788025f, 0.5638357400894165f, 0.27073636651039124f, 0.282094806432724f, 0.35491126775741577f, 0.335813045501709f, 0.35491126775741577f, 0.2882298231124878f, 0.545439600944519f, 0.13155442476272583f, 0.545439600944519f, 0.2882298231124878f, 0.22613950073719025f, 0.5241189002990723f, 0.45212191343307495f, -0.16367165744304657f, 0.45212191343307495f, 0.5241189002990723f, 0.22613950073719025f, 0.1742275357246399f, 0.4662722051143646f, 0.5757606625556946f, 0.10240838676691055f, -0.35559025406837463f, 0.10240838676691055f, 0.5757606625556946f, 0.4662722051143646f, 0.1742275357246399f, 0.13273249566555023f, 0.3971503973007202f, 0.6096431016921997f, 0.36253634095191956f, -0.3051152229309082f, -0.32220059633255005f, -0.3051152229309082f, 0.36253634095191956f, 0.6096431016921997f, 0.3971503973007202f, 0.13273249566555023f, 0.10035116225481033f, 0.3289203643798828f, 0.5894106030464172f, 0.5328931212425232f, -0.03383835777640343f, -0.5257964134216309f, -0.08521328866481781f, -0.5257964134216309f, -0.03383835777640343f, 0.5328931212425232f, 0.5894106030464172f, 0.3289203643798828f, 0.10035116225481033f, 0.282094806432724f, 0.2745485305786133f, 0.4041726291179657f, 0.2745485305786133f, 0.1724795252084732f, 0.5078264474868774f, 0.33203983306884766f, 0.5078264474868774f, 0.1724795252084732f, 0.1046825647354126f, 0.3774833381175995f, 0.6218326687812805f, 0.1300550252199173f, 0.6218326687812805f, 0.3774833381175995f, 0.1046825647354126f, 0.062389861792325974f, 0.2597806453704834f, 0.5660937428474426f, 0.5566006898880005f, -0.1206328421831131f, 0.5566006898880005f, 0.5660937428474426f, 0.2597806453704834f, 0.062389861792325974f, 0.03676832094788551f, 0.17116761207580566f, 0.4477361738681793f, 0.6590285897254944f, 0.31886351108551025f, -0.32900097966194153f, 0.31886351108551025f, 0.6590285897254944f, 0.4477361738681793f, 0.17116761207580566f, 0.03676832094788551f, 0.021503949537873268f, 0.10966213047504425f, 0.3283042311668396f, 0.6120079755783081f, 0.6012592911720276f, -0.020793095231056213f, -0.4215880334377289f, -0.020793095231056213f, 0.6012592911720276f, 0.6120079755783081f, 0.3283042311668396f, 0.10966213047504425f, 0.021503949537873268f, 0.282094806432724f, 0.1815134733915329f, 0.4536356031894684f, 0.1815134733915329f, 0.07539057731628418f, 0.3768298625946045f, 0.5002028346061707f, 0.3768298625946045f, 0.07539057731628418f, 0.03025127202272415f, 0.18519000709056854f, 0.5619985461235046f, 0.4538605809211731f, 0.5619985461235046f, 0.18519000709056854f, 0.03025127202272415f, 0.01191991288214922f, 0.08425901085138321f, 0.32866668701171875f, 0.700112521648407f, 0.33283063769340515f, 0.700112521648407f, 0.32866668701171875f, 0.08425901085138321f, 0.01191991288214922f, 0.004644325003027916f, 0.03670463338494301f, 0.169509157538414f, 0.4870571792125702f, 0.7632161974906921f, 0.15976978838443756f, 0.7632161974906921f, 0.4870571792125702f, 0.169509157538414f, 0.03670463338494301f, 0.004644325003027916f, 0.0017957952804863453f, 0.015546969138085842f, 0.08151230216026306f, 0.2842300832271576f, 0.6359331011772156f, 0.7355261445045471f, -0.037704091519117355f, 0.7355261445045471f, 0.6359331011772156f, 0.2842300832271576f, 0.08151230216026306f, 0.015546969138085842f, 0.0017957952804863453f, 0.282094806432724f, 0.08064790815114975f, 0.48190075159072876f, 0.08064790815114975f, 0.014882830902934074f, 0.17786070704460144f, 0.6050053238868713f, 0.17786070704460144f, 0.014882830902934074f, 0.00265336106531322f, 0.03883617743849754f, 0.2914804220199585f, 0.6859782338142395f, 0.2914804220199585f, 0.03883617743849754f, 0.00265336106531322f, 0.000464526005089283f, 0.00785090122371912f, 0.07487541437149048f, 0.4148964583873749f, 0.7337506413459778f, 0.4148964583873749f, 0.07487541437149048f, 0.00785090122371912f, 0.000464526005089283f, 8.041624823817983e-05f, 0.0015195264713838696f, 0.017060957849025726f, 0.12354122847318649f, 0.5422344207763672f, 0.7521823048591614f, 0.5422344207763672f, 0.12354122847318649f, 0.017060957849025726f, 0.0015195264713838696f, 8.041624823817983e-05f, 1.3815361853630748e-05f, 0.0002859679516404867f, 0.003632891923189163f, 0.03146146610379219f, 0.18467740714550018f, 0.6680772304534912f, 0.7436875104904175f, 0.6680772304534912f, 0.18467740714550018f, 0.03146146610379219f, 0.003632891923189163f, 0.0002859679516404867f, 1.3815361853630748e-05f};
-static __constant__ float kExpTrig7[364] = {1.0f, 0.9937121868133545f, 0.11196447908878326f, 0.9749279022216797f, 0.22252093255519867f, 0.9438833594322205f, 0.33027905225753784f, 0.9009688496589661f, 0.4338837265968323f, 0.8467242121696472f, 0.5320320725440979f, 0.7818315029144287f, 0.6234897971153259f, 1.0f, 0.9438833594322205f, 0.33027905225753784f, 0.7818315029144287f, 0.6234897971153259f, 0.5320320725440979f, 0.8467242121696472f, 0.22252093255519867f, 0.9749279022216797f, -0.11196447908878326f, 0.9937121868133545f, -0.4338837265968323f, 0.9009688496589661f, 1.0f, 0.8467242121696472f, 0.5320320725440979f, 0.4338837265968323f, 0.9009688496589661f, -0.11196447908878326f, 0.9937121868133545f, -0.6234897971153259f, 0.7818315029144287f, -0.9438833594322205f, 0.33027905225753784f, -0.9749279022216797f, -0.22252093255519867f, 1.0f, 0.7071067690849304f, 0.7071067690849304f, 6.123234262925839e-17f, 1.0f, -0.7071067690849304f, 0.7071067690849304f, -1.0f, 1.2246468525851679e-16f, -0.7071067690849304f, -0.7071067690849304f, -1.8369701465288538e-16f, -1.0f, 1.0f, 0.5320320725440979f, 0.8467242121696472f, -0.4338837265968323f, 0.9009688496589661f, -0.9937121868133545f, 0.11196447908878326f, -0.6234897971153259f, -0.7818315029144287f, 0.33027905225753784f, -0.9438833594322205f, 0.9749279022216797f, -0.22252093255519867f, 1.0f, 0.33027905225753784f, 0.9438833594322205f, -0.7818315029144287f, 0.6234897971153259f, -0.8467242121696472f, -0.5320320725440979f, 0.22252093255519867f, -0.9749279022216797f, 0.9937121868133545f, -0.11196447908878326f, 0.4338837265968323f, 0.9009688496589661f, 1.0f, 0.11196447908878326f, 0.9937121868133545f, -0.9749279022216797f, 0.22252093255519867f, -0.33027905225753784f, -0.9438833594322205f, 0.9009688496589661f, -0.4338837265968323f, 0.5320320725440979f, 0.8467242121696472f, -0.7818315029144287f, 0.6234897971153259f, 1.0f, -0.11196447908878326f, 0.9937121868133545f, -0.9749279022216797f, -0.22252093255519867f, 0.33027905225753784f, -0.9438833594322205f, 0.9009688496589661f, 0.4338837265968323f, -0.5320320725440979f, 0.8467242121696472f, -0.7818315029144287f, -0.6234897971153259f, 1.0f, -0.33027905225753784f, 0.9438833594322205f, -0.7818315029144287f, -0.6234897971153259f, 0.8467242121696472f, -0.5320320725440979f, 0.22252093255519867f, 0.9749279022216797f, -0.9937121868133545f, -0.11196447908878326f, 0.4338837265968323f, -0.9009688496589661f, 1.0f, -0.5320320725440979f, 0.8467242121696472f, -0.4338837265968323f, -0.9009688496589661f, 0.9937121868133545f, 0.11196447908878326f, -0.6234897971153259f, 0.7818315029144287f, -0.33027905225753784f, -0.9438833594322205f, 0.9749279022216797f, 0.22252093255519867f, 1.0f, -0.7071067690849304f, 0.7071067690849304f, -1.8369701465288538e-16f, -1.0f, 0.7071067690849304f, 0.7071067690849304f, -1.0f, 3.6739402930577075e-16f, 0.7071067690849304f, -0.7071067690849304f, 5.510910704284357e-16f, 1.0f, 1.0f, -0.8467242121696472f, 0.5320320725440979f, 0.4338837265968323f, -0.9009688496589661f, 0.11196447908878326f, 0.9937121868133545f, -0.6234897971153259f, -0.7818315029144287f, 0.9438833594322205f, 0.33027905225753784f, -0.9749279022216797f, 0.22252093255519867f, 1.0f, -0.9438833594322205f, 0.33027905225753784f, 0.7818315029144287f, -0.6234897971153259f, -0.5320320725440979f, 0.8467242121696472f, 0.22252093255519867f, -0.9749279022216797f, 0.11196447908878326f, 0.9937121868133545f, -0.4338837265968323f, -0.9009688496589661f, 1.0f, -0.9937121868133545f, 0.11196447908878326f, 0.9749279022216797f, -0.22252093255519867f, -0.9438833594322205f, 0.33027905225753784f, 0.9009688496589661f, -0.4338837265968323f, -0.8467242121696472f, 0.5320320725440979f, 0.7818315029144287f, -0.6234897971153259f, 1.0f, -0.9937121868133545f, -0.11196447908878326f, 0.9749279022216797f, 0.22252093255519867f, -0.9438833594322205f, -0.33027905225753784f, 0.9009688496589661f, 0.4338837265968323f, -0.8467242121696472f, -0.5320320725440979f, 0.7818315029144287f, 0.6234897971153259f, 1.0f, -0.9438833594322205f, -0.33027905225753784f, 0.7818315029144287f, 0.6234897971153259f, -0.5320320725440979f, -0.8467242121696472f, 0.22252093255519867f, 0.9749279022216797f, 0.11196447908878326f, -0.9937121868133545f, -0.4338837265968323f, 0.9009688496589661f, 1.0f, -0.8467242121696472f, -0.5320320725440979f, 0.4338837265968323f, 0.9009688496589661f, 0.11196447908878326f, -0.9937121868133545f, -0.6234897971153259f, 0.7818315029144287f, 0.9438833594322205f, -0.33027905225753784f, -0.9749279022216797f, -0.22252093255519867f, 1.0f, -0.7071067690849304f, -0.7071067690849304f, 3.0616169991140216e-16f, 1.0f, 0.7071067690849304f, -0.7071067690849304f, -1.0f, 6.123233998228043e-16f, 0.7071067690849304f, 0.7071067690849304f, -2.6948418861948977e-15f, -1.0f, 1.0f, -0.5320320725440979f, -0.8467242121696472f, -0.4338837265968323f, 0.9009688496589661f, 0.9937121868133545f, -0.11196447908878326f, -0.6234897971153259f, -0.7818315029144287f, -0.33027905225753784f, 0.9438833594322205f, 0.9749279022216797f, -0.22252093255519867f, 1.0f, -0.33027905225753784f, -0.9438833594322205f, -0.7818315029144287f, 0.6234897971153259f, 0.8467242121696472f, 0.5320320725440979f, 0.22252093255519867f, -0.9749279022216797f, -0.9937121868133545f, 0.11196447908878326f, 0.4338837265968323f, 0.9009688496589661f, 1.0f, -0.11196447908878326f, -0.9937121868133545f, -0.9749279022216797f, 0.22252093255519867f, 0.33027905225753784f, 0.9438833594322205f, 0.9009688496589661f, -0.4338837265968323f, -0.5320320725440979f, -0.8467242121696472f, -0.7818315029144287f, 0.6234897971153259f, 1.0f, 0.11196447908878326f, -0.9937121868133545f, -0.9749279022216797f, -0.22252093255519867f, -0.33027905225753784f, 0.9438833594322205f, 0.9009688496589661f, 0.4338837265968323f, 0.5320320725440979f, -0.8467242121696472f, -0.7818315029144287f, -0.6234897971153259f, 1.0f, 0.33027905225753784f, -0.9438833594322205f, -0.7818315029144287f, -0.6234897971153259f, -0.8467242121696472f, 0.5320320725440979f, 0.22252093255519867f, 0.9749279022216797f, 0.9937121868133545f, 0.11196447908878326f, 0.4338837265968323f, -0.9009688496589661f, 1.0f, 0.5320320725440979f, -0.8467242121696472f, -0.4338837265968323f, -0.9009688496589661f, -0.9937121868133545f, -0.11196447908878326f, -0.6234897971153259f, 0.7818315029144287f, 0.33027905225753784f, 0.9438833594322205f, 0.9749279022216797f, 0.22252093255519867f, 1.0f, 0.7071067690849304f, -0.7071067690849304f, -4.2862638516991895e-16f, -1.0f, -0.7071067690849304f, -0.7071067690849304f, -1.0f, 8.572527703398379e-16f, -0.7071067690849304f, 0.7071067690849304f, -4.904777103602732e-16f, 1.0f, 1.0f, 0.8467242121696472f, -0.5320320725440979f, 0.4338837265968323f, -0.9009688496589661f, -0.11196447908878326f, -0.9937121868133545f, -0.6234897971153259f, -0.7818315029144287f, -0.9438833594322205f, -0.33027905225753784f, -0.9749279022216797f, 0.22252093255519867f, 1.0f, 0.9438833594322205f, -0.33027905225753784f, 0.7818315029144287f, -0.6234897971153259f, 0.5320320725440979f, -0.8467242121696472f, 0.22252093255519867f, -0.9749279022216797f, -0.11196447908878326f, -0.9937121868133545f, -0.4338837265968323f, -0.9009688496589661f, 1.0f, 0.9937121868133545f, -0.11196447908878326f, 0.9749279022216797f, -0.22252093255519867f, 0.9438833594322205f, -0.33027905225753784f, 0.9009688496589661f, -0.4338837265968323f, 0.8467242121696472f, -0.5320320725440979f, 0.7818315029144287f, -0.6234897971153259f};
-static __constant__ float kExpW7[14] = {0.007880788296461105f, 0.017987431958317757f, 0.027268704026937485f, 0.03527630865573883f, 0.04163471981883049f, 0.0460464283823967f, 0.04830509424209595f, 0.04830509424209595f, 0.0460464283823967f, 0.04163471981883049f, 0.03527630865573883f, 0.027268704026937485f, 0.017987431958317757f, 0.007880788296461105f};
+// lane-pair rules: product, then projected exponential (plain, weighted)
+static __device__ const float kLpLeg7[160] = {0.07776033133268356f, 0.1604437679052353f, 0.17591159045696259f, 0.14576031267642975f, 0.030566656962037086f, 0.10700652748346329f, 0.18740160763263702f, 0.007755899336189032f, 0.03787914291024208f, 0.08903763443231583f, 0.0019012305419892073f, 0.011880581267178059f, 0.0004576571809593588f, 0.003480701008811593f, 0.00010893459693761542f, 2.5732151698321104e-05f, 0.13117045164108276f, 0.17456598579883575f, 0.1658613383769989f, 0.0f, 0.06656565517187119f, 0.14835511147975922f, 0.22126656770706177f, 0.019984738901257515f, 0.06116100028157234f, 0.0f, 0.0055548627860844135f, 0.02148888260126114f, 0.0014782703947275877f, 0.0f, 0.0003825205785688013f, 0.0f, 0.10176809132099152f, 0.1416567713022232f, 0.0057292720302939415f, -0.13807961344718933f, 0.08842682093381882f, 0.22677944600582123f, 0.1871802657842636f, 0.04959646612405777f, 0.18204443156719208f, 0.2513335645198822f, 0.026874219998717308f, 0.1277928352355957f, 0.014299598522484303f, 0.08337191492319107f, 0.0075237080454826355f, 0.003928481601178646f, 0.15248256921768188f, 0.08637560904026031f, -0.07675936818122864f, 0.0f, 0.17104756832122803f, 0.23445476591587067f, 0.09396131336688995f, 0.11351354420185089f, 0.23436066508293152f, 0.0f, 0.06974370777606964f, 0.18988792598247528f, 0.04102684557437897f, 0.0f, 0.023466672748327255f, 0.0f, 0.11560682207345963f, 0.049735285341739655f, -0.1469823718070984f, -0.024236643686890602f, 0.1469256728887558f, 0.17976497113704681f, -0.13454866409301758f, 0.12053308635950089f, 0.23290126025676727f, -0.028189362958073616f, 0.09552856534719467f, 0.24985216557979584f, 0.07434694468975067f, 0.24441133439540863f, 0.05721541494131088f, 0.043696604669094086f, 0.13604286313056946f, -0.07190325111150742f, -0.12661293148994446f, 0.0f, 0.22321036458015442f, 0.03159971162676811f, -0.21622465550899506f, 0.21666410565376282f, 0.1382545530796051f, 0.0f, 0.19470907747745514f, 0.21051988005638123f, 0.16752943396568298f, 0.0f, 0.1401575207710266f, 0.0f, 0.12383381277322769f, -0.060434337705373764f, -0.06501844525337219f, 0.1434260606765747f, 0.19329603016376495f, -0.011000985279679298f, -0.15925481915473938f, 0.1947605460882187f, 0.0531000941991806f, -0.19980302453041077f, 0.18958215415477753f, 0.10853941738605499f, 0.18121609091758728f, 0.15576526522636414f, 0.17128373682498932f, 0.1606646180152893f, 0.09295744448900223f, -0.14631447196006775f, 0.09065702557563782f, 0.0f, 0.18732348084449768f, -0.19330981373786926f, 0.05287531390786171f, 0.22332343459129333f, -0.16165538132190704f, 0.0f, 0.24649208784103394f, -0.11979328095912933f, 0.2604818046092987f, 0.0f, 0.2676529884338379f, 0.0f, 0.12773483991622925f, -0.13331623375415802f, 0.11267582327127457f, -0.0813179761171341f, 0.21877773106098175f, -0.18196919560432434f, 0.14197389781475067f, 0.24187514185905457f, -0.17697179317474365f, 0.12588657438755035f, 0.2583436071872711f, -0.17147885262966156f, 0.270961195230484f, -0.1651965230703354f, 0.28101956844329834f, 0.2892349064350128f, 0.032937441021203995f, -0.07268138229846954f, 0.10626965761184692f, 0.0f, 0.07282960414886475f, -0.12687724828720093f, 0.16899468004703522f, 0.09527086466550827f, -0.14748406410217285f, 0.0f, 0.11538220942020416f, -0.16550104320049286f, 0.13378988206386566f, 0.0f, 0.150844007730484f, 0.0f};
+static __device__ const float kLeLeg7[448] = {0.282094806432724f, 0.6050053238868713f, 0.7337506413459778f, 0.7436875104904175f, 0.08064790815114975f, 0.2914804220199585f, 0.5422344207763672f, 0.014882830902934074f, 0.07487541437149048f, 0.18467740714550018f, 0.00265336106531322f, 0.017060957849025726f, 0.000464526005089283f, 0.003632891923189163f, 8.041624823817983e-05f, 1.3815361853630748e-05f, 0.48190075159072876f, 0.6859782338142395f, 0.7521823048591614f, 0.0f, 0.17786070704460144f, 0.4148964583873749f, 0.6680772304534912f, 0.03883617743849754f, 0.12354122847318649f, 0.0f, 0.00785090122371912f, 0.03146146610379219f, 0.0015195264713838696f, 0.0f, 0.0002859679516404867f, 0.0f, 0.282094806432724f, 0.5002028346061707f, 0.33283063769340515f, -0.037704091519117355f, 0.1815134733915329f, 0.5619985461235046f, 0.7632161974906921f, 0.07539057731628418f, 0.32866668701171875f, 0.6359331011772156f, 0.03025127202272415f, 0.169509157538414f, 0.01191991288214922f, 0.08151230216026306f, 0.004644325003027916f, 0.0017957952804863453f, 0.4536356031894684f, 0.4538605809211731f, 0.15976978838443756f, 0.0f, 0.3768298625946045f, 0.700112521648407f, 0.7355261445045471f, 0.18519000709056854f, 0.4870571792125702f, 0.0f, 0.08425901085138321f, 0.2842300832271576f, 0.03670463338494301f, 0.0f, 0.015546969138085842f, 0.0f, 0.282094806432724f, 0.33203983306884766f, -0.1206328421831131f, -0.4215880334377289f, 0.2745485305786133f, 0.6218326687812805f, 0.31886351108551025f, 0.1724795252084732f, 0.5660937428474426f, 0.6012592911720276f, 0.1046825647354126f, 0.4477361738681793f, 0.062389861792325974f, 0.3283042311668396f, 0.03676832094788551f, 0.021503949537873268f, 0.4041726291179657f, 0.1300550252199173f, -0.32900097966194153f, 0.0f, 0.5078264474868774f, 0.5566006898880005f, -0.020793095231056213f, 0.3774833381175995f, 0.6590285897254944f, 0.0f, 0.2597806453704834f, 0.6120079755783081f, 0.17116761207580566f, 0.0f, 0.10966213047504425f, 0.0f, 0.282094806432724f, 0.13155442476272583f, -0.35559025406837463f, -0.08521328866481781f, 0.35491126775741577f, 0.45212191343307495f, -0.3051152229309082f, 0.2882298231124878f, 0.5757606625556946f, -0.03383835777640343f, 0.22613950073719025f, 0.6096431016921997f, 0.1742275357246399f, 0.5894106030464172f, 0.13273249566555023f, 0.10035116225481033f, 0.335813045501709f, -0.16367165744304657f, -0.32220059633255005f, 0.0f, 0.545439600944519f, 0.10240838676691055f, -0.5257964134216309f, 0.5241189002990723f, 0.36253634095191956f, 0.0f, 0.4662722051143646f, 0.5328931212425232f, 0.3971503973007202f, 0.0f, 0.3289203643798828f, 0.0f, 0.282094806432724f, -0.0642000138759613f, -0.2642127573490143f, 0.3176251947879791f, 0.4187522530555725f, 0.12824709713459015f, -0.4800601899623871f, 0.4012486934661865f, 0.2982756793498993f, -0.4915175139904022f, 0.3714398741722107f, 0.42788830399513245f, 0.3376496136188507f, 0.5227455496788025f, 0.30350375175476074f, 0.27073636651039124f, 0.25175178050994873f, -0.32160407304763794f, 0.0516158863902092f, 0.0f, 0.4824574589729309f, -0.33728790283203125f, -0.16429507732391357f, 0.546990156173706f, -0.18464216589927673f, 0.0f, 0.5741516351699829f, -0.023816371336579323f, 0.5770047903060913f, 0.0f, 0.5638357400894165f, 0.0f, 0.282094806432724f, -0.21904003620147705f, 0.03257828578352928f, 0.16972026228904724f, 0.46305686235427856f, -0.21260583400726318f, -0.0892399251461029f, 0.4906456470489502f, -0.12202231585979462f, -0.2030356377363205f, 0.5022500157356262f, -0.03477540984749794f, 0.504864513874054f, 0.04890919476747513f, 0.5018221139907837f, 0.4950048625469208f, 0.15591910481452942f, -0.296621710062027f, 0.31815603375434875f, 0.0f, 0.3304174244403839f, -0.4627828299999237f, 0.4030117094516754f, 0.41424816846847534f, -0.477090060710907f, 0.0f, 0.4808225631713867f, -0.47038865089416504f, 0.5343364477157593f, 0.0f, 0.5773844718933105f, 0.0f, 0.282094806432724f, -0.30434414744377136f, 0.280807226896286f, -0.24261875450611115f, 0.4857417047023773f, -0.42784395813941956f, 0.377977579832077f, 0.5398960113525391f, -0.4293491542339325f, 0.36160001158714294f, 0.5797399282455444f, -0.4301821291446686f, 0.6113067269325256f, -0.4295520782470703f, 0.6373898983001709f, 0.6595321297645569f, 0.05279592052102089f, -0.11861658841371536f, 0.1793360412120819f, 0.0f, 0.11736404150724411f, -0.20973744988441467f, 0.29129156470298767f, 0.15434898436069489f, -0.24699321389198303f, 0.0f, 0.18793129920959473f, -0.28084641695022583f, 0.21907870471477509f, 0.0f, 0.24832561612129211f, 0.0f, 0.0022231293842196465f, 0.004767918959259987f, 0.005782533437013626f, 0.005860844161361456f, 0.0006355691002681851f, 0.002297095488756895f, 0.0042732348665595055f, 0.00011728843674063683f, 0.0005900773103348911f, 0.001455403515137732f, 2.091057649522554e-05f, 0.00013445380318444222f, 3.6608312257158104e-06f, 2.8630052838707343e-05f, 6.33743411526666e-07f, 1.0887594470432305e-07f, 0.0037977579049766064f, 0.00540604954585433f, 0.005927789490669966f, 0.0f, 0.0014016826171427965f, 0.0032697112765163183f, 0.005264975130558014f, 0.00030605969368480146f, 0.0009736022911965847f, 0.0f, 6.187129474710673e-05f, 0.00024794114870019257f, 1.1975066627201159e-05f, 0.0f, 2.2536530650540954e-06f, 0.0f, 0.005074161104857922f, 0.008997364901006222f, 0.005986768752336502f, -0.0006781998090445995f, 0.0032649615313857794f, 0.01010891143232584f, 0.013728300109505653f, 0.0013560829684138298f, 0.005911869928240776f, 0.011438804678618908f, 0.0005441427347250283f, 0.0030490346252918243f, 0.00021440863201860338f, 0.0014661969617009163f, 8.353948214789852e-05f, 3.230174843338318e-05f, 0.008159739896655083f, 0.008163786493241787f, 0.0028738481923937798f, 0.0f, 0.006778202019631863f, 0.012593227438628674f, 0.013230226933956146f, 0.0033310926519334316f, 0.0087609076872468f, 0.0f, 0.001515603275038302f, 0.005112569313496351f, 0.0006602220819331706f, 0.0f, 0.0002796500630211085f, 0.0f, 0.007692359387874603f, 0.009054295718669891f, -0.0032895011827349663f, -0.011496159248054028f, 0.007486582268029451f, 0.016956571489572525f, 0.008694995194673538f, 0.004703293088823557f, 0.015436642803251743f, 0.016395561397075653f, 0.0028545577079057693f, 0.012209185399115086f, 0.0017012906027957797f, 0.008952430449426174f, 0.001002624398097396f, 0.0005863848491571844f, 0.011021263897418976f, 0.003546432126313448f, -0.008971430361270905f, 0.0f, 0.013847769238054752f, 0.015177778899669647f, -0.0005670007667504251f, 0.010293480940163136f, 0.0179708544164896f, 0.0f, 0.00708388164639473f, 0.016688663512468338f, 0.00466751866042614f, 0.0f, 0.002990344073623419f, 0.0f, 0.00995126273483038f, 0.0046407547779381275f, -0.01254391111433506f, -0.003006010316312313f, 0.0125199593603611f, 0.0159491915255785f, -0.010763337835669518f, 0.010167684406042099f, 0.02031070925295353f, -0.0011936923256143928f, 0.00797736644744873f, 0.02150595746934414f, 0.006146104075014591f, 0.02079222910106182f, 0.004682312253862619f, 0.0035400185734033585f, 0.01184624433517456f, -0.0057737319730222225f, -0.011366047896444798f, 0.0f, 0.0192410945892334f, 0.0036125897895544767f, -0.018548157066106796f, 0.01848897896707058f, 0.012788943946361542f, 0.0f, 0.016448361799120903f, 0.018798502162098885f, 0.014009999111294746f, 0.0f, 0.0116030965000391f, 0.0f, 0.011744937859475613f, -0.0026729495730251074f, -0.011000423692166805f, 0.013224235735833645f, 0.017434632405638695f, 0.005339531693607569f, -0.01998717151582241f, 0.01670587621629238f, 0.012418624013662338f, -0.02046419307589531f, 0.015464793890714645f, 0.017815008759498596f, 0.014057946391403675f, 0.0217643640935421f, 0.012636292725801468f, 0.01127203181385994f, 0.010481614619493484f, -0.013389894738793373f, 0.0021490128710865974f, 0.0f, 0.02008698135614395f, -0.014042886905372143f, -0.0068403794430196285f, 0.022773781791329384f, -0.007687524892389774f, 0.0f, 0.023904642090201378f, -0.0009915879927575588f, 0.024023432284593582f, 0.0f, 0.02347514219582081f, 0.0f, 0.012989457696676254f, -0.01008601114153862f, 0.0015001136343926191f, 0.007815011776983738f, 0.021322114393115044f, -0.009789738804101944f, -0.004109179601073265f, 0.02259247936308384f, -0.00561869191005826f, -0.009349065832793713f, 0.023126818239688873f, -0.0016012833220884204f, 0.023247206583619118f, 0.0022520937491208315f, 0.023107115179300308f, 0.022793205454945564f, 0.007179517764598131f, -0.013658370822668076f, 0.014649949036538601f, 0.0f, 0.015214542858302593f, -0.021309496834874153f, 0.018557248637080193f, 0.01907464861869812f, -0.0219682939350605f, 0.0f, 0.02214016206562519f, -0.021659716963768005f, 0.02460428513586521f, 0.0f, 0.026586493477225304f, 0.0f, 0.013626615516841412f, -0.01470137294381857f, 0.01356441993266344f, -0.011719722300767899f, 0.02346380054950714f, -0.020667042583227158f, 0.018258243799209595f, 0.026079727336764336f, -0.020739750936627388f, 0.01746712438762188f, 0.028004391118884087f, -0.020779989659786224f, 0.029529228806495667f, -0.02074955403804779f, 0.03078918159008026f, 0.03185876086354256f, 0.002550311852246523f, -0.005729785654693842f, 0.008662845008075237f, 0.0f, 0.005669281352311373f, -0.01013138797134161f, 0.01407086756080389f, 0.007455842569470406f, -0.011931031011044979f, 0.0f, 0.009078038856387138f, -0.01356631238013506f, 0.010582617484033108f, 0.0f, 0.011995392851531506f, 0.0f};
+static __constant__ float kLpTrig7[65] = {1.0f, 0.9876883625984192f, 0.15643446147441864f, 0.9510565400123596f, 0.30901700258255005f, 0.8910065293312073f, 0.45399048924446106f, 0.80901700258255f, 0.5877852439880371f, 0.7071067690849304f, 0.7071067690849304f, 0.5877852439880371f, 0.80901700258255f, 1.0f, 0.8910065293312073f, 0.45399048924446106f, 0.5877852439880371f, 0.80901700258255f, 0.15643446147441864f, 0.9876883625984192f, -0.30901700258255005f, 0.9510565400123596f, -0.7071067690849304f, 0.7071067690849304f, -0.9510565400123596f, 0.30901700258255005f, 1.0f, 0.7071067690849304f, 0.7071067690849304f, 6.123234262925839e-17f, 1.0f, -0.7071067690849304f, 0.7071067690849304f, -1.0f, 1.2246468525851679e-16f, -0.7071067690849304f, -0.7071067690849304f, -1.8369701465288538e-16f, -1.0f, 1.0f, 0.45399048924446106f, 0.8910065293312073f, -0.5877852439880371f, 0.80901700258255f, -0.9876883625984192f, -0.15643446147441864f, -0.30901700258255005f, -0.9510565400123596f, 0.7071067690849304f, -0.7071067690849304f, 0.9510565400123596f, 0.30901700258255005f, 1.0f, 0.15643446147441864f, 0.9876883625984192f, -0.9510565400123596f, 0.30901700258255005f, -0.45399048924446106f, -0.8910065293312073f, 0.80901700258255f, -0.5877852439880371f, 0.7071067690849304f, 0.7071067690849304f, -0.5877852439880371f, 0.80901700258255f};
 #endif
 template <> struct SH<7> {
     static constexpr int K = 49;
     static constexpr int NNZ_SYM = 3348;   // entries (i, j <= k)
     static constexpr int EZ = 14;    // projected-exponential rule: Gauss-Legendre nodes
     static constexpr int EP = 28;    // projected-exponential rule: uniform azimuths
-#if defined(SHS_NB) && SHS_NB == 7
-    __device__ __forceinline__ static const float* eleg() { return kExpLeg7; }
-    __device__ __forceinline__ static const float* etrig() { return kExpTrig7; }
-    __device__ __forceinline__ static const float* ew() { return kExpW7; }
-#endif
     __device__ __forceinline__ static float norm(int i) {
         switch (i) {
             case 0: return 0.282094806432724f;
@@ -2749,629 +2383,182 @@ template <> struct SH<7> {
         gy = w[1] + t64 * a_t123 + t60 * a_t113 + t56 * a_t105 + t52 * a_t99 + t49 * a_t95 + t20 * a_t28 + t23 * a_t25 + t14 * a_t22 + t17 * a_t19 + t8 * a_t16 + t11 * a_t13 + t2 * a_t10 + t5 * a_t7 + x * a_t4 + x * a_t3 + y * a_t1 + y * a_t1;
         gz = w[2] + 945.0f * a_t92 + t88 * a_t89 + 105.0f * a_t87 + t82 * a_t83 + t79 * a_t80 + 15.0f * a_t78 + t73 * a_t74 + t69 * a_t70 + t66 * a_t67 + 3.0f * a_t65 + t60 * a_t61 + t56 * a_t57 + t52 * a_t53 + t49 * a_t50 + 3.0f * a_t49 + t44 * a_t45 + t40 * a_t41 + t36 * a_t37 + 0.6666666865348816f * a_t35 + t32 * a_t33 + z * a_t30 + z * a_t30;
     }
-    static constexpr int NA = 84;   // monomials of degree < n
-    static constexpr int NG = 168;   // gradient coefficients, bands >= 1
-    __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
-        (void)x; (void)y; (void)z;
-        const float m1_0_0 = x;
-        const float m0_1_0 = y;
-        const float m0_0_1 = z;
-        const float m2_0_0 = x * m1_0_0;
-        const float m1_1_0 = x * m0_1_0;
-        const float m1_0_1 = x * m0_0_1;
-        const float m0_2_0 = y * m0_1_0;
-        const float m0_1_1 = y * m0_0_1;
-        const float m0_0_2 = z * m0_0_1;
-        const float m3_0_0 = x * m2_0_0;
-        const float m2_1_0 = x * m1_1_0;
-        const float m2_0_1 = x * m1_0_1;
-        const float m1_2_0 = x * m0_2_0;
-        const float m1_1_1 = x * m0_1_1;
-        const float m1_0_2 = x * m0_0_2;
-        const float m0_3_0 = y * m0_2_0;
-        const float m0_2_1 = y * m0_1_1;
-        const float m0_1_2 = y * m0_0_2;
-        const float m0_0_3 = z * m0_0_2;
-        const float m4_0_0 = x * m3_0_0;
-        const float m3_1_0 = x * m2_1_0;
-        const float m3_0_1 = x * m2_0_1;
-        const float m2_2_0 = x * m1_2_0;
-        const float m2_1_1 = x * m1_1_1;
-        const float m2_0_2 = x * m1_0_2;
-        const float m1_3_0 = x * m0_3_0;
-        const float m1_2_1 = x * m0_2_1;
-        const float m1_1_2 = x * m0_1_2;
-        const float m1_0_3 = x * m0_0_3;
-        const float m0_4_0 = y * m0_3_0;
-        const float m0_3_1 = y * m0_2_1;
-        const float m0_2_2 = y * m0_1_2;
-        const float m0_1_3 = y * m0_0_3;
-        const float m0_0_4 = z * m0_0_3;
-        const float m5_0_0 = x * m4_0_0;
-        const float m4_1_0 = x * m3_1_0;
-        const float m4_0_1 = x * m3_0_1;
-        const float m3_2_0 = x * m2_2_0;
-        const float m3_1_1 = x * m2_1_1;
-        const float m3_0_2 = x * m2_0_2;
-        const float m2_3_0 = x * m1_3_0;
-        const float m2_2_1 = x * m1_2_1;
-        const float m2_1_2 = x * m1_1_2;
-        const float m2_0_3 = x * m1_0_3;
-        const float m1_4_0 = x * m0_4_0;
-        const float m1_3_1 = x * m0_3_1;
-        const float m1_2_2 = x * m0_2_2;
-        const float m1_1_3 = x * m0_1_3;
-        const float m1_0_4 = x * m0_0_4;
-        const float m0_5_0 = y * m0_4_0;
-        const float m0_4_1 = y * m0_3_1;
-        const float m0_3_2 = y * m0_2_2;
-        const float m0_2_3 = y * m0_1_3;
-        const float m0_1_4 = y * m0_0_4;
-        const float m0_0_5 = z * m0_0_4;
-        const float gtx = G[6] * x;
-        const float gty = G[6] * y;
-        const float gtz = G[6] * z;
-        acc[0] = fmaf(G[0], 1.0f, acc[0]);
-        acc[1] = fmaf(G[1], m1_0_0, acc[1]);
-        acc[2] = fmaf(G[1], m0_1_0, acc[2]);
-        acc[3] = fmaf(G[1], m0_0_1, acc[3]);
-        acc[4] = fmaf(G[2], m2_0_0, acc[4]);
-        acc[5] = fmaf(G[2], m1_1_0, acc[5]);
-        acc[6] = fmaf(G[2], m1_0_1, acc[6]);
-        acc[7] = fmaf(G[2], m0_2_0, acc[7]);
-        acc[8] = fmaf(G[2], m0_1_1, acc[8]);
-        acc[9] = fmaf(G[2], m0_0_2, acc[9]);
-        acc[10] = fmaf(G[3], m3_0_0, acc[10]);
-        acc[11] = fmaf(G[3], m2_1_0, acc[11]);
-        acc[12] = fmaf(G[3], m2_0_1, acc[12]);
-        acc[13] = fmaf(G[3], m1_2_0, acc[13]);
-        acc[14] = fmaf(G[3], m1_1_1, acc[14]);
-        acc[15] = fmaf(G[3], m1_0_2, acc[15]);
-        acc[16] = fmaf(G[3], m0_3_0, acc[16]);
-        acc[17] = fmaf(G[3], m0_2_1, acc[17]);
-        acc[18] = fmaf(G[3], m0_1_2, acc[18]);
-        acc[19] = fmaf(G[3], m0_0_3, acc[19]);
-        acc[20] = fmaf(G[4], m4_0_0, acc[20]);
-        acc[21] = fmaf(G[4], m3_1_0, acc[21]);
-        acc[22] = fmaf(G[4], m3_0_1, acc[22]);
-        acc[23] = fmaf(G[4], m2_2_0, acc[23]);
-        acc[24] = fmaf(G[4], m2_1_1, acc[24]);
-        acc[25] = fmaf(G[4], m2_0_2, acc[25]);
-        acc[26] = fmaf(G[4], m1_3_0, acc[26]);
-        acc[27] = fmaf(G[4], m1_2_1, acc[27]);
-        acc[28] = fmaf(G[4], m1_1_2, acc[28]);
-        acc[29] = fmaf(G[4], m1_0_3, acc[29]);
-        acc[30] = fmaf(G[4], m0_4_0, acc[30]);
-        acc[31] = fmaf(G[4], m0_3_1, acc[31]);
-        acc[32] = fmaf(G[4], m0_2_2, acc[32]);
-        acc[33] = fmaf(G[4], m0_1_3, acc[33]);
-        acc[34] = fmaf(G[4], m0_0_4, acc[34]);
-        acc[35] = fmaf(G[5], m5_0_0, acc[35]);
-        acc[36] = fmaf(G[5], m4_1_0, acc[36]);
-        acc[37] = fmaf(G[5], m4_0_1, acc[37]);
-        acc[38] = fmaf(G[5], m3_2_0, acc[38]);
-        acc[39] = fmaf(G[5], m3_1_1, acc[39]);
-        acc[40] = fmaf(G[5], m3_0_2, acc[40]);
-        acc[41] = fmaf(G[5], m2_3_0, acc[41]);
-        acc[42] = fmaf(G[5], m2_2_1, acc[42]);
-        acc[43] = fmaf(G[5], m2_1_2, acc[43]);
-        acc[44] = fmaf(G[5], m2_0_3, acc[44]);
-        acc[45] = fmaf(G[5], m1_4_0, acc[45]);
-        acc[46] = fmaf(G[5], m1_3_1, acc[46]);
-        acc[47] = fmaf(G[5], m1_2_2, acc[47]);
-        acc[48] = fmaf(G[5], m1_1_3, acc[48]);
-        acc[49] = fmaf(G[5], m1_0_4, acc[49]);
-        acc[50] = fmaf(G[5], m0_5_0, acc[50]);
-        acc[51] = fmaf(G[5], m0_4_1, acc[51]);
-        acc[52] = fmaf(G[5], m0_3_2, acc[52]);
-        acc[53] = fmaf(G[5], m0_2_3, acc[53]);
-        acc[54] = fmaf(G[5], m0_1_4, acc[54]);
-        acc[55] = fmaf(G[5], m0_0_5, acc[55]);
-        acc[56] = fmaf(gtx, m5_0_0, acc[56]);
-        acc[57] = fmaf(gtx, m4_1_0, acc[57]);
-        acc[58] = fmaf(gtx, m4_0_1, acc[58]);
-        acc[59] = fmaf(gtx, m3_2_0, acc[59]);
-        acc[60] = fmaf(gtx, m3_1_1, acc[60]);
-        acc[61] = fmaf(gtx, m3_0_2, acc[61]);
-        acc[62] = fmaf(gtx, m2_3_0, acc[62]);
-        acc[63] = fmaf(gtx, m2_2_1, acc[63]);
-        acc[64] = fmaf(gtx, m2_1_2, acc[64]);
-        acc[65] = fmaf(gtx, m2_0_3, acc[65]);
-        acc[66] = fmaf(gtx, m1_4_0, acc[66]);
-        acc[67] = fmaf(gtx, m1_3_1, acc[67]);
-        acc[68] = fmaf(gtx, m1_2_2, acc[68]);
-        acc[69] = fmaf(gtx, m1_1_3, acc[69]);
-        acc[70] = fmaf(gtx, m1_0_4, acc[70]);
-        acc[71] = fmaf(gtx, m0_5_0, acc[71]);
-        acc[72] = fmaf(gtx, m0_4_1, acc[72]);
-        acc[73] = fmaf(gtx, m0_3_2, acc[73]);
-        acc[74] = fmaf(gtx, m0_2_3, acc[74]);
-        acc[75] = fmaf(gtx, m0_1_4, acc[75]);
-        acc[76] = fmaf(gtx, m0_0_5, acc[76]);
-        acc[77] = fmaf(gty, m0_5_0, acc[77]);
-        acc[78] = fmaf(gty, m0_4_1, acc[78]);
-        acc[79] = fmaf(gty, m0_3_2, acc[79]);
-        acc[80] = fmaf(gty, m0_2_3, acc[80]);
-        acc[81] = fmaf(gty, m0_1_4, acc[81]);
-        acc[82] = fmaf(gty, m0_0_5, acc[82]);
-        acc[83] = fmaf(gtz, m0_0_5, acc[83]);
-    }
-    // the same for two pairs at once, one per half of each float2
-    __device__ __forceinline__ static void accumulate2(const float2* G, float2 x, float2 y, float2 z,
-                                                       float2* acc) {
-        (void)x; (void)y; (void)z;
-        const float2 m1_0_0 = x;
-        const float2 m0_1_0 = y;
-        const float2 m0_0_1 = z;
-        const float2 m2_0_0 = __fmul2_rn(x, m1_0_0);
-        const float2 m1_1_0 = __fmul2_rn(x, m0_1_0);
-        const float2 m1_0_1 = __fmul2_rn(x, m0_0_1);
-        const float2 m0_2_0 = __fmul2_rn(y, m0_1_0);
-        const float2 m0_1_1 = __fmul2_rn(y, m0_0_1);
-        const float2 m0_0_2 = __fmul2_rn(z, m0_0_1);
-        const float2 m3_0_0 = __fmul2_rn(x, m2_0_0);
-        const float2 m2_1_0 = __fmul2_rn(x, m1_1_0);
-        const float2 m2_0_1 = __fmul2_rn(x, m1_0_1);
-        const float2 m1_2_0 = __fmul2_rn(x, m0_2_0);
-        const float2 m1_1_1 = __fmul2_rn(x, m0_1_1);
-        const float2 m1_0_2 = __fmul2_rn(x, m0_0_2);
-        const float2 m0_3_0 = __fmul2_rn(y, m0_2_0);
-        const float2 m0_2_1 = __fmul2_rn(y, m0_1_1);
-        const float2 m0_1_2 = __fmul2_rn(y, m0_0_2);
-        const float2 m0_0_3 = __fmul2_rn(z, m0_0_2);
-        const float2 m4_0_0 = __fmul2_rn(x, m3_0_0);
-        const float2 m3_1_0 = __fmul2_rn(x, m2_1_0);
-        const float2 m3_0_1 = __fmul2_rn(x, m2_0_1);
-        const float2 m2_2_0 = __fmul2_rn(x, m1_2_0);
-        const float2 m2_1_1 = __fmul2_rn(x, m1_1_1);
-        const float2 m2_0_2 = __fmul2_rn(x, m1_0_2);
-        const float2 m1_3_0 = __fmul2_rn(x, m0_3_0);
-        const float2 m1_2_1 = __fmul2_rn(x, m0_2_1);
-        const float2 m1_1_2 = __fmul2_rn(x, m0_1_2);
-        const float2 m1_0_3 = __fmul2_rn(x, m0_0_3);
-        const float2 m0_4_0 = __fmul2_rn(y, m0_3_0);
-        const float2 m0_3_1 = __fmul2_rn(y, m0_2_1);
-        const float2 m0_2_2 = __fmul2_rn(y, m0_1_2);
-        const float2 m0_1_3 = __fmul2_rn(y, m0_0_3);
-        const float2 m0_0_4 = __fmul2_rn(z, m0_0_3);
-        const float2 m5_0_0 = __fmul2_rn(x, m4_0_0);
-        const float2 m4_1_0 = __fmul2_rn(x, m3_1_0);
-        const float2 m4_0_1 = __fmul2_rn(x, m3_0_1);
-        const float2 m3_2_0 = __fmul2_rn(x, m2_2_0);
-        const float2 m3_1_1 = __fmul2_rn(x, m2_1_1);
-        const float2 m3_0_2 = __fmul2_rn(x, m2_0_2);
-        const float2 m2_3_0 = __fmul2_rn(x, m1_3_0);
-        const float2 m2_2_1 = __fmul2_rn(x, m1_2_1);
-        const float2 m2_1_2 = __fmul2_rn(x, m1_1_2);
-        const float2 m2_0_3 = __fmul2_rn(x, m1_0_3);
-        const float2 m1_4_0 = __fmul2_rn(x, m0_4_0);
-        const float2 m1_3_1 = __fmul2_rn(x, m0_3_1);
-        const float2 m1_2_2 = __fmul2_rn(x, m0_2_2);
-        const float2 m1_1_3 = __fmul2_rn(x, m0_1_3);
-        const float2 m1_0_4 = __fmul2_rn(x, m0_0_4);
-        const float2 m0_5_0 = __fmul2_rn(y, m0_4_0);
-        const float2 m0_4_1 = __fmul2_rn(y, m0_3_1);
-        const float2 m0_3_2 = __fmul2_rn(y, m0_2_2);
-        const float2 m0_2_3 = __fmul2_rn(y, m0_1_3);
-        const float2 m0_1_4 = __fmul2_rn(y, m0_0_4);
-        const float2 m0_0_5 = __fmul2_rn(z, m0_0_4);
-        const float2 gtx = __fmul2_rn(G[6], x);
-        const float2 gty = __fmul2_rn(G[6], y);
-        const float2 gtz = __fmul2_rn(G[6], z);
-        acc[0] = __fadd2_rn(G[0], acc[0]);
-        acc[1] = __ffma2_rn(G[1], m1_0_0, acc[1]);
-        acc[2] = __ffma2_rn(G[1], m0_1_0, acc[2]);
-        acc[3] = __ffma2_rn(G[1], m0_0_1, acc[3]);
-        acc[4] = __ffma2_rn(G[2], m2_0_0, acc[4]);
-        acc[5] = __ffma2_rn(G[2], m1_1_0, acc[5]);
-        acc[6] = __ffma2_rn(G[2], m1_0_1, acc[6]);
-        acc[7] = __ffma2_rn(G[2], m0_2_0, acc[7]);
-        acc[8] = __ffma2_rn(G[2], m0_1_1, acc[8]);
-        acc[9] = __ffma2_rn(G[2], m0_0_2, acc[9]);
-        acc[10] = __ffma2_rn(G[3], m3_0_0, acc[10]);
-        acc[11] = __ffma2_rn(G[3], m2_1_0, acc[11]);
-        acc[12] = __ffma2_rn(G[3], m2_0_1, acc[12]);
-        acc[13] = __ffma2_rn(G[3], m1_2_0, acc[13]);
-        acc[14] = __ffma2_rn(G[3], m1_1_1, acc[14]);
-        acc[15] = __ffma2_rn(G[3], m1_0_2, acc[15]);
-        acc[16] = __ffma2_rn(G[3], m0_3_0, acc[16]);
-        acc[17] = __ffma2_rn(G[3], m0_2_1, acc[17]);
-        acc[18] = __ffma2_rn(G[3], m0_1_2, acc[18]);
-        acc[19] = __ffma2_rn(G[3], m0_0_3, acc[19]);
-        acc[20] = __ffma2_rn(G[4], m4_0_0, acc[20]);
-        acc[21] = __ffma2_rn(G[4], m3_1_0, acc[21]);
-        acc[22] = __ffma2_rn(G[4], m3_0_1, acc[22]);
-        acc[23] = __ffma2_rn(G[4], m2_2_0, acc[23]);
-        acc[24] = __ffma2_rn(G[4], m2_1_1, acc[24]);
-        acc[25] = __ffma2_rn(G[4], m2_0_2, acc[25]);
-        acc[26] = __ffma2_rn(G[4], m1_3_0, acc[26]);
-        acc[27] = __ffma2_rn(G[4], m1_2_1, acc[27]);
-        acc[28] = __ffma2_rn(G[4], m1_1_2, acc[28]);
-        acc[29] = __ffma2_rn(G[4], m1_0_3, acc[29]);
-        acc[30] = __ffma2_rn(G[4], m0_4_0, acc[30]);
-        acc[31] = __ffma2_rn(G[4], m0_3_1, acc[31]);
-        acc[32] = __ffma2_rn(G[4], m0_2_2, acc[32]);
-        acc[33] = __ffma2_rn(G[4], m0_1_3, acc[33]);
-        acc[34] = __ffma2_rn(G[4], m0_0_4, acc[34]);
-        acc[35] = __ffma2_rn(G[5], m5_0_0, acc[35]);
-        acc[36] = __ffma2_rn(G[5], m4_1_0, acc[36]);
-        acc[37] = __ffma2_rn(G[5], m4_0_1, acc[37]);
-        acc[38] = __ffma2_rn(G[5], m3_2_0, acc[38]);
-        acc[39] = __ffma2_rn(G[5], m3_1_1, acc[39]);
-        acc[40] = __ffma2_rn(G[5], m3_0_2, acc[40]);
-        acc[41] = __ffma2_rn(G[5], m2_3_0, acc[41]);
-        acc[42] = __ffma2_rn(G[5], m2_2_1, acc[42]);
-        acc[43] = __ffma2_rn(G[5], m2_1_2, acc[43]);
-        acc[44] = __ffma2_rn(G[5], m2_0_3, acc[44]);
-        acc[45] = __ffma2_rn(G[5], m1_4_0, acc[45]);
-        acc[46] = __ffma2_rn(G[5], m1_3_1, acc[46]);
-        acc[47] = __ffma2_rn(G[5], m1_2_2, acc[47]);
-        acc[48] = __ffma2_rn(G[5], m1_1_3, acc[48]);
-        acc[49] = __ffma2_rn(G[5], m1_0_4, acc[49]);
-        acc[50] = __ffma2_rn(G[5], m0_5_0, acc[50]);
-        acc[51] = __ffma2_rn(G[5], m0_4_1, acc[51]);
-        acc[52] = __ffma2_rn(G[5], m0_3_2, acc[52]);
-        acc[53] = __ffma2_rn(G[5], m0_2_3, acc[53]);
-        acc[54] = __ffma2_rn(G[5], m0_1_4, acc[54]);
-        acc[55] = __ffma2_rn(G[5], m0_0_5, acc[55]);
-        acc[56] = __ffma2_rn(gtx, m5_0_0, acc[56]);
-        acc[57] = __ffma2_rn(gtx, m4_1_0, acc[57]);
-        acc[58] = __ffma2_rn(gtx, m4_0_1, acc[58]);
-        acc[59] = __ffma2_rn(gtx, m3_2_0, acc[59]);
-        acc[60] = __ffma2_rn(gtx, m3_1_1, acc[60]);
-        acc[61] = __ffma2_rn(gtx, m3_0_2, acc[61]);
-        acc[62] = __ffma2_rn(gtx, m2_3_0, acc[62]);
-        acc[63] = __ffma2_rn(gtx, m2_2_1, acc[63]);
-        acc[64] = __ffma2_rn(gtx, m2_1_2, acc[64]);
-        acc[65] = __ffma2_rn(gtx, m2_0_3, acc[65]);
-        acc[66] = __ffma2_rn(gtx, m1_4_0, acc[66]);
-        acc[67] = __ffma2_rn(gtx, m1_3_1, acc[67]);
-        acc[68] = __ffma2_rn(gtx, m1_2_2, acc[68]);
-        acc[69] = __ffma2_rn(gtx, m1_1_3, acc[69]);
-        acc[70] = __ffma2_rn(gtx, m1_0_4, acc[70]);
-        acc[71] = __ffma2_rn(gtx, m0_5_0, acc[71]);
-        acc[72] = __ffma2_rn(gtx, m0_4_1, acc[72]);
-        acc[73] = __ffma2_rn(gtx, m0_3_2, acc[73]);
-        acc[74] = __ffma2_rn(gtx, m0_2_3, acc[74]);
-        acc[75] = __ffma2_rn(gtx, m0_1_4, acc[75]);
-        acc[76] = __ffma2_rn(gtx, m0_0_5, acc[76]);
-        acc[77] = __ffma2_rn(gty, m0_5_0, acc[77]);
-        acc[78] = __ffma2_rn(gty, m0_4_1, acc[78]);
-        acc[79] = __ffma2_rn(gty, m0_3_2, acc[79]);
-        acc[80] = __ffma2_rn(gty, m0_2_3, acc[80]);
-        acc[81] = __ffma2_rn(gty, m0_1_4, acc[81]);
-        acc[82] = __ffma2_rn(gty, m0_0_5, acc[82]);
-        acc[83] = __ffma2_rn(gtz, m0_0_5, acc[83]);
-    }
-    __device__ __forceinline__ static void mono_to_f(const float* acc, float* f) {
-        f[0] = 1.0f * acc[0];
-        f[1] = 1.0f * acc[2];
-        f[2] = 1.0f * acc[3];
-        f[3] = 1.0f * acc[1];
-        f[4] = 6.0f * acc[5];
-        f[5] = 3.0f * acc[8];
-        f[6] = ((1.0f * acc[9] + -0.5f * acc[7]) + -0.5f * acc[4]);
-        f[7] = 3.0f * acc[6];
-        f[8] = (-3.0f * acc[7] + 3.0f * acc[4]);
-        f[9] = (-15.0f * acc[16] + 45.0f * acc[11]);
-        f[10] = 30.0f * acc[14];
-        f[11] = ((6.0f * acc[18] + -1.5f * acc[16]) + -1.5f * acc[11]);
-        f[12] = ((1.0f * acc[19] + -1.5f * acc[17]) + -1.5f * acc[12]);
-        f[13] = ((6.0f * acc[15] + -1.5f * acc[13]) + -1.5f * acc[10]);
-        f[14] = (-15.0f * acc[17] + 15.0f * acc[12]);
-        f[15] = (-45.0f * acc[13] + 15.0f * acc[10]);
-        f[16] = (-420.0f * acc[26] + 420.0f * acc[21]);
-        f[17] = (-105.0f * acc[31] + 315.0f * acc[24]);
-        f[18] = ((90.0f * acc[28] + -15.0f * acc[26]) + -15.0f * acc[21]);
-        f[19] = ((10.0f * acc[33] + -7.5f * acc[31]) + -7.5f * acc[24]);
-        f[20] = ((fmaf(0.75f, acc[23], 1.0f * acc[34]) + fmaf(0.375f, acc[20], -3.0f * acc[32])) + (0.375f * acc[30] + -3.0f * acc[25]));
-        f[21] = ((10.0f * acc[29] + -7.5f * acc[27]) + -7.5f * acc[22]);
-        f[22] = ((-45.0f * acc[32] + 7.5f * acc[30]) + (45.0f * acc[25] + -7.5f * acc[20]));
-        f[23] = (-315.0f * acc[27] + 105.0f * acc[22]);
-        f[24] = ((105.0f * acc[30] + -630.0f * acc[23]) + 105.0f * acc[20]);
-        f[25] = ((945.0f * acc[50] + -9450.0f * acc[41]) + 4725.0f * acc[36]);
-        f[26] = (-3780.0f * acc[46] + 3780.0f * acc[39]);
-        f[27] = ((fmaf(-157.5f, acc[36], -420.0f * acc[52]) + 52.5f * acc[50]) + (1260.0f * acc[43] + -105.0f * acc[41]));
-        f[28] = ((210.0f * acc[48] + -105.0f * acc[46]) + -105.0f * acc[39]);
-        f[29] = ((fmaf(3.75f, acc[41], 15.0f * acc[54]) + fmaf(1.875f, acc[36], -22.5f * acc[52])) + (1.875f * acc[50] + -22.5f * acc[43]));
-        f[30] = ((fmaf(3.75f, acc[42], 1.0f * acc[55]) + fmaf(1.875f, acc[37], -5.0f * acc[53])) + (1.875f * acc[51] + -5.0f * acc[44]));
-        f[31] = ((fmaf(3.75f, acc[38], 15.0f * acc[49]) + fmaf(1.875f, acc[35], -22.5f * acc[47])) + (1.875f * acc[45] + -22.5f * acc[40]));
-        f[32] = ((-105.0f * acc[53] + 52.5f * acc[51]) + (105.0f * acc[44] + -52.5f * acc[37]));
-        f[33] = ((fmaf(-52.5f, acc[35], -1260.0f * acc[47]) + 157.5f * acc[45]) + (420.0f * acc[40] + 105.0f * acc[38]));
-        f[34] = ((945.0f * acc[51] + -5670.0f * acc[42]) + 945.0f * acc[37]);
-        f[35] = ((4725.0f * acc[45] + -9450.0f * acc[38]) + 945.0f * acc[35]);
-        f[36] = ((62370.0f * acc[71] + -207900.0f * acc[62]) + 62370.0f * acc[57]);
-        f[37] = ((10395.0f * acc[78] + -103950.0f * acc[67]) + 51975.0f * acc[60]);
-        f[38] = ((-18900.0f * acc[73] + 1890.0f * acc[71]) + (18900.0f * acc[64] + -1890.0f * acc[57]));
-        f[39] = ((fmaf(-1417.5f, acc[60], -1260.0f * acc[80]) + 472.5f * acc[78]) + (3780.0f * acc[69] + -945.0f * acc[67]));
-        f[40] = ((fmaf(52.5f, acc[62], 420.0f * acc[75]) + fmaf(26.25f, acc[57], -420.0f * acc[73])) + (26.25f * acc[71] + -420.0f * acc[64]));
-        f[41] = ((fmaf(26.25f, acc[67], 21.0f * acc[82]) + fmaf(13.125f, acc[60], -52.5f * acc[80])) + (13.125f * acc[78] + -52.5f * acc[69]));
-        f[42] = ((fmaf(-0.9375f, acc[59], fmaf(-7.5f, acc[70], 1.0f * acc[83])) + fmaf(-0.3125f, acc[56], fmaf(11.25f, acc[68], -7.5f * acc[81]))) + (fmaf(-0.9375f, acc[66], 5.625f * acc[79]) + fmaf(5.625f, acc[61], -0.3125f * acc[77])));
-        f[43] = ((fmaf(26.25f, acc[63], 21.0f * acc[76]) + fmaf(13.125f, acc[58], -52.5f * acc[74])) + (13.125f * acc[72] + -52.5f * acc[65]));
-        f[44] = ((fmaf(-13.125f, acc[66], -210.0f * acc[81]) + fmaf(-210.0f, acc[61], 210.0f * acc[79])) + (fmaf(13.125f, acc[59], -13.125f * acc[77]) + fmaf(13.125f, acc[56], 210.0f * acc[70])));
-        f[45] = ((fmaf(-472.5f, acc[58], -3780.0f * acc[74]) + 1417.5f * acc[72]) + (1260.0f * acc[65] + 945.0f * acc[63]));
-        f[46] = ((fmaf(4725.0f, acc[61], 4725.0f * acc[79]) + fmaf(2362.5f, acc[59], -472.5f * acc[77])) + (fmaf(-472.5f, acc[56], -28350.0f * acc[68]) + 2362.5f * acc[66]));
-        f[47] = ((51975.0f * acc[72] + -103950.0f * acc[63]) + 10395.0f * acc[58]);
-        f[48] = ((-10395.0f * acc[77] + 155925.0f * acc[66]) + (-155925.0f * acc[59] + 10395.0f * acc[56]));
-    }
-    __device__ __forceinline__ static void grad_coeffs(const float* w, float* gq) {
-        (void)w; (void)gq;
-        gq[0] = 1.0f * w[3];
-        gq[1] = 1.0f * w[1];
-        gq[2] = 1.0f * w[2];
-        gq[3] = (-1.0f * w[6] + 6.0f * w[8]);
-        gq[4] = 6.0f * w[4];
-        gq[5] = 3.0f * w[7];
-        gq[6] = 6.0f * w[4];
-        gq[7] = (-1.0f * w[6] + -6.0f * w[8]);
-        gq[8] = 3.0f * w[5];
-        gq[9] = 3.0f * w[7];
-        gq[10] = 3.0f * w[5];
-        gq[11] = 2.0f * w[6];
-        gq[12] = (-4.5f * w[13] + 45.0f * w[15]);
-        gq[13] = (90.0f * w[9] + -3.0f * w[11]);
-        gq[14] = (-3.0f * w[12] + 30.0f * w[14]);
-        gq[15] = (-1.5f * w[13] + -45.0f * w[15]);
-        gq[16] = 30.0f * w[10];
-        gq[17] = 6.0f * w[13];
-        gq[18] = (45.0f * w[9] + -1.5f * w[11]);
-        gq[19] = (-3.0f * w[13] + -90.0f * w[15]);
-        gq[20] = 30.0f * w[10];
-        gq[21] = (-45.0f * w[9] + -4.5f * w[11]);
-        gq[22] = (-3.0f * w[12] + -30.0f * w[14]);
-        gq[23] = 6.0f * w[11];
-        gq[24] = (-1.5f * w[12] + 15.0f * w[14]);
-        gq[25] = 30.0f * w[10];
-        gq[26] = 12.0f * w[13];
-        gq[27] = (-1.5f * w[12] + -15.0f * w[14]);
-        gq[28] = 12.0f * w[11];
-        gq[29] = 3.0f * w[12];
-        gq[30] = ((1.5f * w[20] + -30.0f * w[22]) + 420.0f * w[24]);
-        gq[31] = (1260.0f * w[16] + -45.0f * w[18]);
-        gq[32] = (-22.5f * w[21] + 315.0f * w[23]);
-        gq[33] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[34] = (630.0f * w[17] + -15.0f * w[19]);
-        gq[35] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[36] = (-420.0f * w[16] + -15.0f * w[18]);
-        gq[37] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[38] = 90.0f * w[18];
-        gq[39] = 10.0f * w[21];
-        gq[40] = (420.0f * w[16] + -15.0f * w[18]);
-        gq[41] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[42] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[43] = (-1260.0f * w[16] + -45.0f * w[18]);
-        gq[44] = (-15.0f * w[21] + -630.0f * w[23]);
-        gq[45] = 90.0f * w[18];
-        gq[46] = ((1.5f * w[20] + 30.0f * w[22]) + 420.0f * w[24]);
-        gq[47] = (-315.0f * w[17] + -22.5f * w[19]);
-        gq[48] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[49] = 10.0f * w[19];
-        gq[50] = (-7.5f * w[21] + 105.0f * w[23]);
-        gq[51] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[52] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[53] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[54] = 180.0f * w[18];
-        gq[55] = 30.0f * w[21];
-        gq[56] = (-105.0f * w[17] + -7.5f * w[19]);
-        gq[57] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[58] = 30.0f * w[19];
-        gq[59] = 4.0f * w[20];
-        gq[60] = ((9.375f * w[31] + -262.5f * w[33]) + 4725.0f * w[35]);
-        gq[61] = ((18900.0f * w[25] + -630.0f * w[27]) + 7.5f * w[29]);
-        gq[62] = ((7.5f * w[30] + -210.0f * w[32]) + 3780.0f * w[34]);
-        gq[63] = ((11.25f * w[31] + 315.0f * w[33]) + -28350.0f * w[35]);
-        gq[64] = (11340.0f * w[26] + -315.0f * w[28]);
-        gq[65] = (-67.5f * w[31] + 1260.0f * w[33]);
-        gq[66] = ((-18900.0f * w[25] + -210.0f * w[27]) + 7.5f * w[29]);
-        gq[67] = (7.5f * w[30] + -11340.0f * w[34]);
-        gq[68] = (2520.0f * w[27] + -45.0f * w[29]);
-        gq[69] = (-10.0f * w[30] + 210.0f * w[32]);
-        gq[70] = ((1.875f * w[31] + 157.5f * w[33]) + 4725.0f * w[35]);
-        gq[71] = (-3780.0f * w[26] + -105.0f * w[28]);
-        gq[72] = (-22.5f * w[31] + -1260.0f * w[33]);
-        gq[73] = 210.0f * w[28];
-        gq[74] = 15.0f * w[31];
-        gq[75] = ((4725.0f * w[25] + -157.5f * w[27]) + 1.875f * w[29]);
-        gq[76] = ((7.5f * w[31] + 210.0f * w[33]) + -18900.0f * w[35]);
-        gq[77] = (3780.0f * w[26] + -105.0f * w[28]);
-        gq[78] = ((-28350.0f * w[25] + -315.0f * w[27]) + 11.25f * w[29]);
-        gq[79] = (7.5f * w[30] + -11340.0f * w[34]);
-        gq[80] = (1260.0f * w[27] + -22.5f * w[29]);
-        gq[81] = ((7.5f * w[31] + 630.0f * w[33]) + 18900.0f * w[35]);
-        gq[82] = (-11340.0f * w[26] + -315.0f * w[28]);
-        gq[83] = (-45.0f * w[31] + -2520.0f * w[33]);
-        gq[84] = 210.0f * w[28];
-        gq[85] = ((4725.0f * w[25] + 262.5f * w[27]) + 9.375f * w[29]);
-        gq[86] = ((7.5f * w[30] + 210.0f * w[32]) + 3780.0f * w[34]);
-        gq[87] = (-1260.0f * w[27] + -67.5f * w[29]);
-        gq[88] = (-10.0f * w[30] + -210.0f * w[32]);
-        gq[89] = 15.0f * w[29];
-        gq[90] = ((1.875f * w[30] + -52.5f * w[32]) + 945.0f * w[34]);
-        gq[91] = (3780.0f * w[26] + -105.0f * w[28]);
-        gq[92] = (-45.0f * w[31] + 840.0f * w[33]);
-        gq[93] = (3.75f * w[30] + -5670.0f * w[34]);
-        gq[94] = (2520.0f * w[27] + -45.0f * w[29]);
-        gq[95] = (-15.0f * w[30] + 315.0f * w[32]);
-        gq[96] = (-3780.0f * w[26] + -105.0f * w[28]);
-        gq[97] = (-45.0f * w[31] + -2520.0f * w[33]);
-        gq[98] = 630.0f * w[28];
-        gq[99] = 60.0f * w[31];
-        gq[100] = ((1.875f * w[30] + 52.5f * w[32]) + 945.0f * w[34]);
-        gq[101] = (-840.0f * w[27] + -45.0f * w[29]);
-        gq[102] = (-15.0f * w[30] + -315.0f * w[32]);
-        gq[103] = 60.0f * w[29];
-        gq[104] = 5.0f * w[30];
-        gq[105] = ((-1.875f * w[42] + 78.75f * w[44]) + (-2835.0f * w[46] + 62370.0f * w[48]));
-        gq[106] = ((311850.0f * w[36] + -9450.0f * w[38]) + 131.25f * w[40]);
-        gq[107] = ((65.625f * w[43] + -2362.5f * w[45]) + 51975.0f * w[47]);
-        gq[108] = ((-3.75f * w[42] + 52.5f * w[44]) + (9450.0f * w[46] + -623700.0f * w[48]));
-        gq[109] = ((207900.0f * w[37] + -5670.0f * w[39]) + 52.5f * w[41]);
-        gq[110] = ((22.5f * w[42] + -840.0f * w[44]) + 18900.0f * w[46]);
-        gq[111] = (-623700.0f * w[36] + 157.5f * w[40]);
-        gq[112] = ((78.75f * w[43] + 2835.0f * w[45]) + -311850.0f * w[47]);
-        gq[113] = (56700.0f * w[38] + -1260.0f * w[40]);
-        gq[114] = (-157.5f * w[43] + 3780.0f * w[45]);
-        gq[115] = ((-1.875f * w[42] + -26.25f * w[44]) + (4725.0f * w[46] + 311850.0f * w[48]));
-        gq[116] = ((-207900.0f * w[37] + -1890.0f * w[39]) + 52.5f * w[41]);
-        gq[117] = (22.5f * w[42] + -56700.0f * w[46]);
-        gq[118] = (7560.0f * w[39] + -105.0f * w[41]);
-        gq[119] = (-15.0f * w[42] + 420.0f * w[44]);
-        gq[120] = ((62370.0f * w[36] + 1890.0f * w[38]) + 26.25f * w[40]);
-        gq[121] = ((13.125f * w[43] + 1417.5f * w[45]) + 51975.0f * w[47]);
-        gq[122] = (-18900.0f * w[38] + -420.0f * w[40]);
-        gq[123] = (-52.5f * w[43] + -3780.0f * w[45]);
-        gq[124] = 420.0f * w[40];
-        gq[125] = 21.0f * w[43];
-        gq[126] = ((62370.0f * w[36] + -1890.0f * w[38]) + 26.25f * w[40]);
-        gq[127] = ((-1.875f * w[42] + 26.25f * w[44]) + (4725.0f * w[46] + -311850.0f * w[48]));
-        gq[128] = ((51975.0f * w[37] + -1417.5f * w[39]) + 13.125f * w[41]);
-        gq[129] = (-623700.0f * w[36] + 157.5f * w[40]);
-        gq[130] = ((52.5f * w[43] + 1890.0f * w[45]) + -207900.0f * w[47]);
-        gq[131] = (18900.0f * w[38] + -420.0f * w[40]);
-        gq[132] = ((-3.75f * w[42] + -52.5f * w[44]) + (9450.0f * w[46] + 623700.0f * w[48]));
-        gq[133] = ((-311850.0f * w[37] + -2835.0f * w[39]) + 78.75f * w[41]);
-        gq[134] = (22.5f * w[42] + -56700.0f * w[46]);
-        gq[135] = (3780.0f * w[39] + -52.5f * w[41]);
-        gq[136] = ((311850.0f * w[36] + 9450.0f * w[38]) + 131.25f * w[40]);
-        gq[137] = ((52.5f * w[43] + 5670.0f * w[45]) + 207900.0f * w[47]);
-        gq[138] = (-56700.0f * w[38] + -1260.0f * w[40]);
-        gq[139] = (-105.0f * w[43] + -7560.0f * w[45]);
-        gq[140] = 420.0f * w[40];
-        gq[141] = ((-1.875f * w[42] + -78.75f * w[44]) + (-2835.0f * w[46] + -62370.0f * w[48]));
-        gq[142] = ((51975.0f * w[37] + 2362.5f * w[39]) + 65.625f * w[41]);
-        gq[143] = ((22.5f * w[42] + 840.0f * w[44]) + 18900.0f * w[46]);
-        gq[144] = (-3780.0f * w[39] + -157.5f * w[41]);
-        gq[145] = (-15.0f * w[42] + -420.0f * w[44]);
-        gq[146] = 21.0f * w[41];
-        gq[147] = ((13.125f * w[43] + -472.5f * w[45]) + 10395.0f * w[47]);
-        gq[148] = ((51975.0f * w[37] + -1417.5f * w[39]) + 13.125f * w[41]);
-        gq[149] = ((11.25f * w[42] + -420.0f * w[44]) + 9450.0f * w[46]);
-        gq[150] = ((26.25f * w[43] + 945.0f * w[45]) + -103950.0f * w[47]);
-        gq[151] = (37800.0f * w[38] + -840.0f * w[40]);
-        gq[152] = (-157.5f * w[43] + 3780.0f * w[45]);
-        gq[153] = ((-103950.0f * w[37] + -945.0f * w[39]) + 26.25f * w[41]);
-        gq[154] = (22.5f * w[42] + -56700.0f * w[46]);
-        gq[155] = (11340.0f * w[39] + -157.5f * w[41]);
-        gq[156] = (-30.0f * w[42] + 840.0f * w[44]);
-        gq[157] = ((13.125f * w[43] + 1417.5f * w[45]) + 51975.0f * w[47]);
-        gq[158] = (-37800.0f * w[38] + -840.0f * w[40]);
-        gq[159] = (-157.5f * w[43] + -11340.0f * w[45]);
-        gq[160] = 1680.0f * w[40];
-        gq[161] = 105.0f * w[43];
-        gq[162] = ((10395.0f * w[37] + 472.5f * w[39]) + 13.125f * w[41]);
-        gq[163] = ((11.25f * w[42] + 420.0f * w[44]) + 9450.0f * w[46]);
-        gq[164] = (-3780.0f * w[39] + -157.5f * w[41]);
-        gq[165] = (-30.0f * w[42] + -840.0f * w[44]);
-        gq[166] = 105.0f * w[41];
-        gq[167] = 6.0f * w[42];
-    }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
-        (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        const float u1_0_0 = x;
-        const float u0_1_0 = y;
-        const float u0_0_1 = z;
-        const float u2_0_0 = x * u1_0_0;
-        const float u1_1_0 = x * u0_1_0;
-        const float u1_0_1 = x * u0_0_1;
-        const float u0_2_0 = y * u0_1_0;
-        const float u0_1_1 = y * u0_0_1;
-        const float u0_0_2 = z * u0_0_1;
-        const float u3_0_0 = x * u2_0_0;
-        const float u2_1_0 = x * u1_1_0;
-        const float u2_0_1 = x * u1_0_1;
-        const float u1_2_0 = x * u0_2_0;
-        const float u1_1_1 = x * u0_1_1;
-        const float u1_0_2 = x * u0_0_2;
-        const float u0_3_0 = y * u0_2_0;
-        const float u0_2_1 = y * u0_1_1;
-        const float u0_1_2 = y * u0_0_2;
-        const float u0_0_3 = z * u0_0_2;
-        const float u4_0_0 = x * u3_0_0;
-        const float u3_1_0 = x * u2_1_0;
-        const float u3_0_1 = x * u2_0_1;
-        const float u2_2_0 = x * u1_2_0;
-        const float u2_1_1 = x * u1_1_1;
-        const float u2_0_2 = x * u1_0_2;
-        const float u1_3_0 = x * u0_3_0;
-        const float u1_2_1 = x * u0_2_1;
-        const float u1_1_2 = x * u0_1_2;
-        const float u1_0_3 = x * u0_0_3;
-        const float u0_4_0 = y * u0_3_0;
-        const float u0_3_1 = y * u0_2_1;
-        const float u0_2_2 = y * u0_1_2;
-        const float u0_1_3 = y * u0_0_3;
-        const float u0_0_4 = z * u0_0_3;
-        const float u5_0_0 = x * u4_0_0;
-        const float u4_1_0 = x * u3_1_0;
-        const float u4_0_1 = x * u3_0_1;
-        const float u3_2_0 = x * u2_2_0;
-        const float u3_1_1 = x * u2_1_1;
-        const float u3_0_2 = x * u2_0_2;
-        const float u2_3_0 = x * u1_3_0;
-        const float u2_2_1 = x * u1_2_1;
-        const float u2_1_2 = x * u1_1_2;
-        const float u2_0_3 = x * u1_0_3;
-        const float u1_4_0 = x * u0_4_0;
-        const float u1_3_1 = x * u0_3_1;
-        const float u1_2_2 = x * u0_2_2;
-        const float u1_1_3 = x * u0_1_3;
-        const float u1_0_4 = x * u0_0_4;
-        const float u0_5_0 = y * u0_4_0;
-        const float u0_4_1 = y * u0_3_1;
-        const float u0_3_2 = y * u0_2_2;
-        const float u0_2_3 = y * u0_1_3;
-        const float u0_1_4 = y * u0_0_4;
-        const float u0_0_5 = z * u0_0_4;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
-        gx[1] = gq[3] * u1_0_0 + gq[4] * u0_1_0 + gq[5] * u0_0_1;
-        gy[1] = gq[6] * u1_0_0 + gq[7] * u0_1_0 + gq[8] * u0_0_1;
-        gz[1] = gq[9] * u1_0_0 + gq[10] * u0_1_0 + gq[11] * u0_0_1;
-        gx[2] = gq[12] * u2_0_0 + gq[13] * u1_1_0 + gq[14] * u1_0_1 + gq[15] * u0_2_0 + gq[16] * u0_1_1 + gq[17] * u0_0_2;
-        gy[2] = gq[18] * u2_0_0 + gq[19] * u1_1_0 + gq[20] * u1_0_1 + gq[21] * u0_2_0 + gq[22] * u0_1_1 + gq[23] * u0_0_2;
-        gz[2] = gq[24] * u2_0_0 + gq[25] * u1_1_0 + gq[26] * u1_0_1 + gq[27] * u0_2_0 + gq[28] * u0_1_1 + gq[29] * u0_0_2;
-        gx[3] = gq[30] * u3_0_0 + gq[31] * u2_1_0 + gq[32] * u2_0_1 + gq[33] * u1_2_0 + gq[34] * u1_1_1 + gq[35] * u1_0_2 + gq[36] * u0_3_0 + gq[37] * u0_2_1 + gq[38] * u0_1_2 + gq[39] * u0_0_3;
-        gy[3] = gq[40] * u3_0_0 + gq[41] * u2_1_0 + gq[42] * u2_0_1 + gq[43] * u1_2_0 + gq[44] * u1_1_1 + gq[45] * u1_0_2 + gq[46] * u0_3_0 + gq[47] * u0_2_1 + gq[48] * u0_1_2 + gq[49] * u0_0_3;
-        gz[3] = gq[50] * u3_0_0 + gq[51] * u2_1_0 + gq[52] * u2_0_1 + gq[53] * u1_2_0 + gq[54] * u1_1_1 + gq[55] * u1_0_2 + gq[56] * u0_3_0 + gq[57] * u0_2_1 + gq[58] * u0_1_2 + gq[59] * u0_0_3;
-        gx[4] = gq[60] * u4_0_0 + gq[61] * u3_1_0 + gq[62] * u3_0_1 + gq[63] * u2_2_0 + gq[64] * u2_1_1 + gq[65] * u2_0_2 + gq[66] * u1_3_0 + gq[67] * u1_2_1 + gq[68] * u1_1_2 + gq[69] * u1_0_3 + gq[70] * u0_4_0 + gq[71] * u0_3_1 + gq[72] * u0_2_2 + gq[73] * u0_1_3 + gq[74] * u0_0_4;
-        gy[4] = gq[75] * u4_0_0 + gq[76] * u3_1_0 + gq[77] * u3_0_1 + gq[78] * u2_2_0 + gq[79] * u2_1_1 + gq[80] * u2_0_2 + gq[81] * u1_3_0 + gq[82] * u1_2_1 + gq[83] * u1_1_2 + gq[84] * u1_0_3 + gq[85] * u0_4_0 + gq[86] * u0_3_1 + gq[87] * u0_2_2 + gq[88] * u0_1_3 + gq[89] * u0_0_4;
-        gz[4] = gq[90] * u4_0_0 + gq[91] * u3_1_0 + gq[92] * u3_0_1 + gq[93] * u2_2_0 + gq[94] * u2_1_1 + gq[95] * u2_0_2 + gq[96] * u1_3_0 + gq[97] * u1_2_1 + gq[98] * u1_1_2 + gq[99] * u1_0_3 + gq[100] * u0_4_0 + gq[101] * u0_3_1 + gq[102] * u0_2_2 + gq[103] * u0_1_3 + gq[104] * u0_0_4;
-        gx[5] = gq[105] * u5_0_0 + gq[106] * u4_1_0 + gq[107] * u4_0_1 + gq[108] * u3_2_0 + gq[109] * u3_1_1 + gq[110] * u3_0_2 + gq[111] * u2_3_0 + gq[112] * u2_2_1 + gq[113] * u2_1_2 + gq[114] * u2_0_3 + gq[115] * u1_4_0 + gq[116] * u1_3_1 + gq[117] * u1_2_2 + gq[118] * u1_1_3 + gq[119] * u1_0_4 + gq[120] * u0_5_0 + gq[121] * u0_4_1 + gq[122] * u0_3_2 + gq[123] * u0_2_3 + gq[124] * u0_1_4 + gq[125] * u0_0_5;
-        gy[5] = gq[126] * u5_0_0 + gq[127] * u4_1_0 + gq[128] * u4_0_1 + gq[129] * u3_2_0 + gq[130] * u3_1_1 + gq[131] * u3_0_2 + gq[132] * u2_3_0 + gq[133] * u2_2_1 + gq[134] * u2_1_2 + gq[135] * u2_0_3 + gq[136] * u1_4_0 + gq[137] * u1_3_1 + gq[138] * u1_2_2 + gq[139] * u1_1_3 + gq[140] * u1_0_4 + gq[141] * u0_5_0 + gq[142] * u0_4_1 + gq[143] * u0_3_2 + gq[144] * u0_2_3 + gq[145] * u0_1_4 + gq[146] * u0_0_5;
-        gz[5] = gq[147] * u5_0_0 + gq[148] * u4_1_0 + gq[149] * u4_0_1 + gq[150] * u3_2_0 + gq[151] * u3_1_1 + gq[152] * u3_0_2 + gq[153] * u2_3_0 + gq[154] * u2_2_1 + gq[155] * u2_1_2 + gq[156] * u2_0_3 + gq[157] * u1_4_0 + gq[158] * u1_3_1 + gq[159] * u1_2_2 + gq[160] * u1_1_3 + gq[161] * u1_0_4 + gq[162] * u0_5_0 + gq[163] * u0_4_1 + gq[164] * u0_3_2 + gq[165] * u0_2_3 + gq[166] * u0_1_4 + gq[167] * u0_0_5;
-    }
-    static constexpr int QZ = 10;    // Gauss-Legendre nodes in cos(theta)
-    static constexpr int QP = 19;    // uniform azimuths
-    static constexpr int QF = 13;    // azimuthal harmonics 1, cos m phi, sin m phi
+    static constexpr int LPS = 5;   // lane-pair product rule: node pairs
+    static constexpr int LPQ = 5;   // ... and azimuth quads
+    static constexpr int LES = 7;   // lane-pair projected-exponential rule: node pairs
+    static constexpr int LEQ = 7;   // ... and azimuth quads
 #if defined(SHS_NB) && SHS_NB == 7
-    __device__ __forceinline__ static const float* qleg() { return kQuadLeg7; }
-    __device__ __forceinline__ static const float* qtrig() { return kQuadTrig7; }
-    __device__ __forceinline__ static const float* qw() { return kQuadW7; }
+    __device__ __forceinline__ static const float* lp_leg() { return kLpLeg7; }
+    __device__ __forceinline__ static const float* le_leg() { return kLeLeg7; }
+    __device__ __forceinline__ static const float* lp_trig_row(int b) { return kLpTrig7 + b * 13; }
 #endif
+    __device__ __forceinline__ static float lp_trig(int b, int h) {   // h = 2m - 1: cos(m phi_b), 2m: sin
+        switch (b * 13 + h) {
+            case 1: return 0.9876883625984192f;
+            case 2: return 0.15643446147441864f;
+            case 3: return 0.9510565400123596f;
+            case 4: return 0.30901700258255005f;
+            case 5: return 0.8910065293312073f;
+            case 6: return 0.45399048924446106f;
+            case 7: return 0.80901700258255f;
+            case 8: return 0.5877852439880371f;
+            case 9: return 0.7071067690849304f;
+            case 10: return 0.7071067690849304f;
+            case 11: return 0.5877852439880371f;
+            case 12: return 0.80901700258255f;
+            case 14: return 0.8910065293312073f;
+            case 15: return 0.45399048924446106f;
+            case 16: return 0.5877852439880371f;
+            case 17: return 0.80901700258255f;
+            case 18: return 0.15643446147441864f;
+            case 19: return 0.9876883625984192f;
+            case 20: return -0.30901700258255005f;
+            case 21: return 0.9510565400123596f;
+            case 22: return -0.7071067690849304f;
+            case 23: return 0.7071067690849304f;
+            case 24: return -0.9510565400123596f;
+            case 25: return 0.30901700258255005f;
+            case 27: return 0.7071067690849304f;
+            case 28: return 0.7071067690849304f;
+            case 29: return 6.123234262925839e-17f;
+            case 30: return 1.0f;
+            case 31: return -0.7071067690849304f;
+            case 32: return 0.7071067690849304f;
+            case 33: return -1.0f;
+            case 34: return 1.2246468525851679e-16f;
+            case 35: return -0.7071067690849304f;
+            case 36: return -0.7071067690849304f;
+            case 37: return -1.8369701465288538e-16f;
+            case 38: return -1.0f;
+            case 40: return 0.45399048924446106f;
+            case 41: return 0.8910065293312073f;
+            case 42: return -0.5877852439880371f;
+            case 43: return 0.80901700258255f;
+            case 44: return -0.9876883625984192f;
+            case 45: return -0.15643446147441864f;
+            case 46: return -0.30901700258255005f;
+            case 47: return -0.9510565400123596f;
+            case 48: return 0.7071067690849304f;
+            case 49: return -0.7071067690849304f;
+            case 50: return 0.9510565400123596f;
+            case 51: return 0.30901700258255005f;
+            case 53: return 0.15643446147441864f;
+            case 54: return 0.9876883625984192f;
+            case 55: return -0.9510565400123596f;
+            case 56: return 0.30901700258255005f;
+            case 57: return -0.45399048924446106f;
+            case 58: return -0.8910065293312073f;
+            case 59: return 0.80901700258255f;
+            case 60: return -0.5877852439880371f;
+            case 61: return 0.7071067690849304f;
+            case 62: return 0.7071067690849304f;
+            case 63: return -0.5877852439880371f;
+            case 64: return 0.80901700258255f;
+            default: return 1.0f;
+        }
+    }
+    __device__ __forceinline__ static float le_trig(int b, int h) {   // h = 2m - 1: cos(m phi_b), 2m: sin
+        switch (b * 13 + h) {
+            case 1: return 0.9937121868133545f;
+            case 2: return 0.11196447908878326f;
+            case 3: return 0.9749279022216797f;
+            case 4: return 0.22252093255519867f;
+            case 5: return 0.9438833594322205f;
+            case 6: return 0.33027905225753784f;
+            case 7: return 0.9009688496589661f;
+            case 8: return 0.4338837265968323f;
+            case 9: return 0.8467242121696472f;
+            case 10: return 0.5320320725440979f;
+            case 11: return 0.7818315029144287f;
+            case 12: return 0.6234897971153259f;
+            case 14: return 0.9438833594322205f;
+            case 15: return 0.33027905225753784f;
+            case 16: return 0.7818315029144287f;
+            case 17: return 0.6234897971153259f;
+            case 18: return 0.5320320725440979f;
+            case 19: return 0.8467242121696472f;
+            case 20: return 0.22252093255519867f;
+            case 21: return 0.9749279022216797f;
+            case 22: return -0.11196447908878326f;
+            case 23: return 0.9937121868133545f;
+            case 24: return -0.4338837265968323f;
+            case 25: return 0.9009688496589661f;
+            case 27: return 0.8467242121696472f;
+            case 28: return 0.5320320725440979f;
+            case 29: return 0.4338837265968323f;
+            case 30: return 0.9009688496589661f;
+            case 31: return -0.11196447908878326f;
+            case 32: return 0.9937121868133545f;
+            case 33: return -0.6234897971153259f;
+            case 34: return 0.7818315029144287f;
+            case 35: return -0.9438833594322205f;
+            case 36: return 0.33027905225753784f;
+            case 37: return -0.9749279022216797f;
+            case 38: return -0.22252093255519867f;
+            case 40: return 0.7071067690849304f;
+            case 41: return 0.7071067690849304f;
+            case 42: return 6.123234262925839e-17f;
+            case 43: return 1.0f;
+            case 44: return -0.7071067690849304f;
+            case 45: return 0.7071067690849304f;
+            case 46: return -1.0f;
+            case 47: return 1.2246468525851679e-16f;
+            case 48: return -0.7071067690849304f;
+            case 49: return -0.7071067690849304f;
+            case 50: return -1.8369701465288538e-16f;
+            case 51: return -1.0f;
+            case 53: return 0.5320320725440979f;
+            case 54: return 0.8467242121696472f;
+            case 55: return -0.4338837265968323f;
+            case 56: return 0.9009688496589661f;
+            case 57: return -0.9937121868133545f;
+            case 58: return 0.11196447908878326f;
+            case 59: return -0.6234897971153259f;
+            case 60: return -0.7818315029144287f;
+            case 61: return 0.33027905225753784f;
+            case 62: return -0.9438833594322205f;
+            case 63: return 0.9749279022216797f;
+            case 64: return -0.22252093255519867f;
+            case 66: return 0.33027905225753784f;
+            case 67: return 0.9438833594322205f;
+            case 68: return -0.7818315029144287f;
+            case 69: return 0.6234897971153259f;
+            case 70: return -0.8467242121696472f;
+            case 71: return -0.5320320725440979f;
+            case 72: return 0.22252093255519867f;
+            case 73: return -0.9749279022216797f;
+            case 74: return 0.9937121868133545f;
+            case 75: return -0.11196447908878326f;
+            case 76: return 0.4338837265968323f;
+            case 77: return 0.9009688496589661f;
+            case 79: return 0.11196447908878326f;
+            case 80: return 0.9937121868133545f;
+            case 81: return -0.9749279022216797f;
+            case 82: return 0.22252093255519867f;
+            case 83: return -0.33027905225753784f;
+            case 84: return -0.9438833594322205f;
+            case 85: return 0.9009688496589661f;
+            case 86: return -0.4338837265968323f;
+            case 87: return 0.5320320725440979f;
+            case 88: return 0.8467242121696472f;
+            case 89: return -0.7818315029144287f;
+            case 90: return 0.6234897971153259f;
+            default: return 1.0f;
+        }
+    }
 };
 
 #if defined(SHS_NB) && SHS_NB == 8
-static __constant__ float kQuadLeg8[704] = {0.282094806432724f, 0.10139966756105423f, -0.47796496748924255f, 0.10139966756105423f, 0.023527316749095917f, -0.22180019319057465f, 0.5900326371192932f, -0.22180019319057465f, 0.023527316749095917f, 0.005273836199194193f, -0.060892216861248016f, 0.358977347612381f, -0.6514920592308044f, 0.358977347612381f, -0.060892216861248016f, 0.005273836199194193f, 0.0011608704226091504f, -0.015477052889764309f, 0.11610877513885498f, -0.5023488402366638f, 0.6709103584289551f, -0.5023488402366638f, 0.11610877513885498f, -0.015477052889764309f, 0.0011608704226091504f, 0.0002526742173358798f, -0.0037663481198251247f, 0.03328768163919449f, -0.1889096200466156f, 0.6423048377037048f, -0.6526771783828735f, 0.6423048377037048f, -0.1889096200466156f, 0.03328768163919449f, -0.0037663481198251247f, 0.0002526742173358798f, 5.457865336211398e-05f, -0.0008911954937502742f, 0.008915836922824383f, -0.06062023714184761f, 0.2776050269603729f, -0.7700836658477783f, 0.6005485653877258f, -0.7700836658477783f, 0.2776050269603729f, -0.06062023714184761f, 0.008915836922824383f, -0.0008911954937502742f, 5.457865336211398e-05f, 1.1724255273293238e-05f, -0.00020678013970609754f, 0.002285235794261098f, -0.01777736470103264f, 0.09899555146694183f, -0.3792743682861328f, 0.8778833150863647f, -0.5186641216278076f, 0.8778833150863647f, -0.3792743682861328f, 0.09899555146694183f, -0.01777736470103264f, 0.002285235794261098f, -0.00020678013970609754f, 1.1724255273293238e-05f, 0.282094806432724f, 0.2255629450082779f, -0.4334210157394409f, 0.2255629450082779f, 0.11642193049192429f, -0.44741135835647583f, 0.42913442850112915f, -0.44741135835647583f, 0.11642193049192429f, 0.05805240944027901f, -0.27323609590530396f, 0.6191432476043701f, -0.3093152344226837f, 0.6191432476043701f, -0.27323609590530396f, 0.05805240944027901f, 0.02842552773654461f, -0.15448835492134094f, 0.45453232526779175f, -0.6871917843818665f, 0.11265167593955994f, -0.6871917843818665f, 0.45453232526779175f, -0.15448835492134094f, 0.02842552773654461f, 0.013763121329247952f, -0.08362943679094315f, 0.2927502989768982f, -0.6165207624435425f, 0.6244769096374512f, 0.11134136468172073f, 0.6244769096374512f, -0.6165207624435425f, 0.2927502989768982f, -0.08362943679094315f, 0.013763121329247952f, 0.006613175384700298f, -0.04401927441358566f, 0.1754482388496399f, -0.4547070562839508f, 0.7135617136955261f, -0.43579602241516113f, -0.3096718490123749f, -0.43579602241516113f, 0.7135617136955261f, -0.4547070562839508f, 0.1754482388496399f, -0.04401927441358566f, 0.006613175384700298f, 0.0031601209193468094f, -0.022720083594322205f, 0.10042279958724976f, -0.30229702591896057f, 0.6097151041030884f, -0.710532546043396f, 0.1564732939004898f, 0.4365486800670624f, 0.1564732939004898f, -0.710532546043396f, 0.6097151041030884f, -0.30229702591896057f, 0.10042279958724976f, -0.022720083594322205f, 0.0031601209193468094f, 0.282094806432724f, 0.33385464549064636f, -0.3567540943622589f, 0.33385464549064636f, 0.2550434470176697f, -0.5450742840766907f, 0.18903493881225586f, -0.5450742840766907f, 0.2550434470176697f, 0.18823018670082092f, -0.49269306659698486f, 0.5201573371887207f, 0.0911131277680397f, 0.5201573371887207f, -0.49269306659698486f, 0.18823018670082092f, 0.13641661405563354f, -0.4123099446296692f, 0.6033957004547119f, -0.24428431689739227f, -0.3222220242023468f, -0.24428431689739227f, 0.6033957004547119f, -0.4123099446296692f, 0.13641661405563354f, 0.09776093065738678f, -0.33035197854042053f, 0.5927775502204895f, -0.48970529437065125f, -0.15323173999786377f, 0.3768104314804077f, -0.15323173999786377f, -0.48970529437065125f, 0.5927775502204895f, -0.33035197854042053f, 0.09776093065738678f, 0.06952614337205887f, -0.25736549496650696f, 0.5349928736686707f, -0.6146100759506226f, 0.16838739812374115f, 0.46926796436309814f, -0.2256249189376831f, 0.46926796436309814f, 0.16838739812374115f, -0.6146100759506226f, 0.5349928736686707f, -0.25736549496650696f, 0.06952614337205887f, 0.04917353764176369f, -0.19661064445972443f, 0.45835599303245544f, -0.6492382884025574f, 0.4221198260784149f, 0.22629094123840332f, -0.5378110408782959f, -0.048520419746637344f, -0.5378110408782959f, 0.22629094123840332f, 0.4221198260784149f, -0.6492382884025574f, 0.45835599303245544f, -0.19661064445972443f, 0.04917353764176369f, 0.282094806432724f, 0.4176163077354431f, -0.25363168120384216f, 0.4176163077354431f, 0.3990747332572937f, -0.48474156856536865f, -0.06043458357453346f, -0.48474156856536865f, 0.3990747332572937f, 0.36842525005340576f, -0.5480889678001404f, 0.13567231595516205f, 0.3201510012149811f, 0.13567231595516205f, -0.5480889678001404f, 0.36842525005340576f, 0.33400073647499084f, -0.5737443566322327f, 0.30628740787506104f, 0.33061546087265015f, -0.26896023750305176f, 0.33061546087265015f, 0.30628740787506104f, -0.5737443566322327f, 0.33400073647499084f, 0.2994094789028168f, -0.5750313997268677f, 0.43535691499710083f, 0.17416177690029144f, -0.48301979899406433f, -0.043231651186943054f, -0.48301979899406433f, 0.17416177690029144f, 0.43535691499710083f, -0.5750313997268677f, 0.2994094789028168f, 0.2663595974445343f, -0.5603830218315125f, 0.5288844108581543f, 0.010728582739830017f, -0.4893190264701843f, 0.17777447402477264f, 0.3141016364097595f, 0.17777447402477264f, -0.4893190264701843f, 0.010728582739830017f, 0.5288844108581543f, -0.5603830218315125f, 0.2663595974445343f, 0.23565231263637543f, -0.5355027914047241f, 0.592467725276947f, -0.14461760222911835f, -0.42997920513153076f, 0.3572480082511902f, 0.29564520716667175f, -0.28199321031570435f, 0.29564520716667175f, 0.3572480082511902f, -0.42997920513153076f, -0.14461760222911835f, 0.592467725276947f, -0.5355027914047241f, 0.23565231263637543f, 0.282094806432724f, 0.4705184996128082f, -0.13169945776462555f, 0.4705184996128082f, 0.5065854787826538f, -0.2835894227027893f, -0.2466486543416977f, -0.2835894227027893f, 0.5065854787826538f, 0.5269230008125305f, -0.36126846075057983f, -0.2802448868751526f, 0.26522132754325867f, -0.2802448868751526f, -0.36126846075057983f, 0.5269230008125305f, 0.5382009148597717f, -0.4260854423046112f, -0.21559613943099976f, 0.4326667785644531f, 0.10632962733507156f, 0.4326667785644531f, -0.21559613943099976f, -0.4260854423046112f, 0.5382009148597717f, 0.5435779094696045f, -0.48113733530044556f, -0.15121962130069733f, 0.4685167074203491f, 0.040870290249586105f, -0.3230115473270416f, 0.040870290249586105f, 0.4685167074203491f, -0.15121962130069733f, -0.48113733530044556f, 0.5435779094696045f, 0.5448335409164429f, -0.5282770991325378f, -0.08713434636592865f, 0.4880121052265167f, -0.05705355480313301f, -0.4528689384460449f, 0.0670318454504013f, -0.4528689384460449f, -0.05705355480313301f, 0.4880121052265167f, -0.08713434636592865f, -0.5282770991325378f, 0.5448335409164429f, 0.5430833101272583f, -0.5687714219093323f, -0.023852212354540825f, 0.49448996782302856f, -0.1453525573015213f, -0.42935067415237427f, 0.2052813470363617f, 0.28726741671562195f, 0.2052813470363617f, -0.42935067415237427f, -0.1453525573015213f, 0.49448996782302856f, -0.023852212354540825f, -0.5687714219093323f, 0.5430833101272583f, 0.282094806432724f, 0.48860251903533936f, 0.0f, 0.48860251903533936f, 0.5462742447853088f, 0.0f, -0.31539157032966614f, 0.0f, 0.5462742447853088f, 0.5900436043739319f, 0.0f, -0.4570457935333252f, 0.0f, -0.4570457935333252f, 0.0f, 0.5900436043739319f, 0.6258357167243958f, 0.0f, -0.473087340593338f, 0.0f, 0.3173566460609436f, 0.0f, -0.473087340593338f, 0.0f, 0.6258357167243958f, 0.6563820838928223f, 0.0f, -0.48923829197883606f, 0.0f, 0.45294666290283203f, 0.0f, 0.45294666290283203f, 0.0f, -0.48923829197883606f, 0.0f, 0.6563820838928223f, 0.6831840872764587f, 0.0f, -0.5045648813247681f, 0.0f, 0.46060264110565186f, 0.0f, -0.31784600019454956f, 0.0f, 0.46060264110565186f, 0.0f, -0.5045648813247681f, 0.0f, 0.6831840872764587f, 0.7071627378463745f, 0.0f, -0.518915593624115f, 0.0f, 0.469376802444458f, 0.0f, -0.4516580402851105f, 0.0f, -0.4516580402851105f, 0.0f, 0.469376802444458f, 0.0f, -0.518915593624115f, 0.0f, 0.7071627378463745f, 0.282094806432724f, 0.4705184996128082f, 0.13169945776462555f, 0.4705184996128082f, 0.5065854787826538f, 0.2835894227027893f, -0.2466486543416977f, 0.2835894227027893f, 0.5065854787826538f, 0.5269230008125305f, 0.36126846075057983f, -0.2802448868751526f, -0.26522132754325867f, -0.2802448868751526f, 0.36126846075057983f, 0.5269230008125305f, 0.5382009148597717f, 0.4260854423046112f, -0.21559613943099976f, -0.4326667785644531f, 0.10632962733507156f, -0.4326667785644531f, -0.21559613943099976f, 0.4260854423046112f, 0.5382009148597717f, 0.5435779094696045f, 0.48113733530044556f, -0.15121962130069733f, -0.4685167074203491f, 0.040870290249586105f, 0.3230115473270416f, 0.040870290249586105f, -0.4685167074203491f, -0.15121962130069733f, 0.48113733530044556f, 0.5435779094696045f, 0.5448335409164429f, 0.5282770991325378f, -0.08713434636592865f, -0.4880121052265167f, -0.05705355480313301f, 0.4528689384460449f, 0.0670318454504013f, 0.4528689384460449f, -0.05705355480313301f, -0.4880121052265167f, -0.08713434636592865f, 0.5282770991325378f, 0.5448335409164429f, 0.5430833101272583f, 0.5687714219093323f, -0.023852212354540825f, -0.49448996782302856f, -0.1453525573015213f, 0.42935067415237427f, 0.2052813470363617f, -0.28726741671562195f, 0.2052813470363617f, 0.42935067415237427f, -0.1453525573015213f, -0.49448996782302856f, -0.023852212354540825f, 0.5687714219093323f, 0.5430833101272583f, 0.282094806432724f, 0.4176163077354431f, 0.25363168120384216f, 0.4176163077354431f, 0.3990747332572937f, 0.48474156856536865f, -0.06043458357453346f, 0.48474156856536865f, 0.3990747332572937f, 0.36842525005340576f, 0.5480889678001404f, 0.13567231595516205f, -0.3201510012149811f, 0.13567231595516205f, 0.5480889678001404f, 0.36842525005340576f, 0.33400073647499084f, 0.5737443566322327f, 0.30628740787506104f, -0.33061546087265015f, -0.26896023750305176f, -0.33061546087265015f, 0.30628740787506104f, 0.5737443566322327f, 0.33400073647499084f, 0.2994094789028168f, 0.5750313997268677f, 0.43535691499710083f, -0.17416177690029144f, -0.48301979899406433f, 0.043231651186943054f, -0.48301979899406433f, -0.17416177690029144f, 0.43535691499710083f, 0.5750313997268677f, 0.2994094789028168f, 0.2663595974445343f, 0.5603830218315125f, 0.5288844108581543f, -0.010728582739830017f, -0.4893190264701843f, -0.17777447402477264f, 0.3141016364097595f, -0.17777447402477264f, -0.4893190264701843f, -0.010728582739830017f, 0.5288844108581543f, 0.5603830218315125f, 0.2663595974445343f, 0.23565231263637543f, 0.5355027914047241f, 0.592467725276947f, 0.14461760222911835f, -0.42997920513153076f, -0.3572480082511902f, 0.29564520716667175f, 0.28199321031570435f, 0.29564520716667175f, -0.3572480082511902f, -0.42997920513153076f, 0.14461760222911835f, 0.592467725276947f, 0.5355027914047241f, 0.23565231263637543f, 0.282094806432724f, 0.33385464549064636f, 0.3567540943622589f, 0.33385464549064636f, 0.2550434470176697f, 0.5450742840766907f, 0.18903493881225586f, 0.5450742840766907f, 0.2550434470176697f, 0.18823018670082092f, 0.49269306659698486f, 0.5201573371887207f, -0.0911131277680397f, 0.5201573371887207f, 0.49269306659698486f, 0.18823018670082092f, 0.13641661405563354f, 0.4123099446296692f, 0.6033957004547119f, 0.24428431689739227f, -0.3222220242023468f, 0.24428431689739227f, 0.6033957004547119f, 0.4123099446296692f, 0.13641661405563354f, 0.09776093065738678f, 0.33035197854042053f, 0.5927775502204895f, 0.48970529437065125f, -0.15323173999786377f, -0.3768104314804077f, -0.15323173999786377f, 0.48970529437065125f, 0.5927775502204895f, 0.33035197854042053f, 0.09776093065738678f, 0.06952614337205887f, 0.25736549496650696f, 0.5349928736686707f, 0.6146100759506226f, 0.16838739812374115f, -0.46926796436309814f, -0.2256249189376831f, -0.46926796436309814f, 0.16838739812374115f, 0.6146100759506226f, 0.5349928736686707f, 0.25736549496650696f, 0.06952614337205887f, 0.04917353764176369f, 0.19661064445972443f, 0.45835599303245544f, 0.6492382884025574f, 0.4221198260784149f, -0.22629094123840332f, -0.5378110408782959f, 0.048520419746637344f, -0.5378110408782959f, -0.22629094123840332f, 0.4221198260784149f, 0.6492382884025574f, 0.45835599303245544f, 0.19661064445972443f, 0.04917353764176369f, 0.282094806432724f, 0.2255629450082779f, 0.4334210157394409f, 0.2255629450082779f, 0.11642193049192429f, 0.44741135835647583f, 0.42913442850112915f, 0.44741135835647583f, 0.11642193049192429f, 0.05805240944027901f, 0.27323609590530396f, 0.6191432476043701f, 0.3093152344226837f, 0.6191432476043701f, 0.27323609590530396f, 0.05805240944027901f, 0.02842552773654461f, 0.15448835492134094f, 0.45453232526779175f, 0.6871917843818665f, 0.11265167593955994f, 0.6871917843818665f, 0.45453232526779175f, 0.15448835492134094f, 0.02842552773654461f, 0.013763121329247952f, 0.08362943679094315f, 0.2927502989768982f, 0.6165207624435425f, 0.6244769096374512f, -0.11134136468172073f, 0.6244769096374512f, 0.6165207624435425f, 0.2927502989768982f, 0.08362943679094315f, 0.013763121329247952f, 0.006613175384700298f, 0.04401927441358566f, 0.1754482388496399f, 0.4547070562839508f, 0.7135617136955261f, 0.43579602241516113f, -0.3096718490123749f, 0.43579602241516113f, 0.7135617136955261f, 0.4547070562839508f, 0.1754482388496399f, 0.04401927441358566f, 0.006613175384700298f, 0.0031601209193468094f, 0.022720083594322205f, 0.10042279958724976f, 0.30229702591896057f, 0.6097151041030884f, 0.710532546043396f, 0.1564732939004898f, -0.4365486800670624f, 0.1564732939004898f, 0.710532546043396f, 0.6097151041030884f, 0.30229702591896057f, 0.10042279958724976f, 0.022720083594322205f, 0.0031601209193468094f, 0.282094806432724f, 0.10139966756105423f, 0.47796496748924255f, 0.10139966756105423f, 0.023527316749095917f, 0.22180019319057465f, 0.5900326371192932f, 0.22180019319057465f, 0.023527316749095917f, 0.005273836199194193f, 0.060892216861248016f, 0.358977347612381f, 0.6514920592308044f, 0.358977347612381f, 0.060892216861248016f, 0.005273836199194193f, 0.0011608704226091504f, 0.015477052889764309f, 0.11610877513885498f, 0.5023488402366638f, 0.6709103584289551f, 0.5023488402366638f, 0.11610877513885498f, 0.015477052889764309f, 0.0011608704226091504f, 0.0002526742173358798f, 0.0037663481198251247f, 0.03328768163919449f, 0.1889096200466156f, 0.6423048377037048f, 0.6526771783828735f, 0.6423048377037048f, 0.1889096200466156f, 0.03328768163919449f, 0.0037663481198251247f, 0.0002526742173358798f, 5.457865336211398e-05f, 0.0008911954937502742f, 0.008915836922824383f, 0.06062023714184761f, 0.2776050269603729f, 0.7700836658477783f, 0.6005485653877258f, 0.7700836658477783f, 0.2776050269603729f, 0.06062023714184761f, 0.008915836922824383f, 0.0008911954937502742f, 5.457865336211398e-05f, 1.1724255273293238e-05f, 0.00020678013970609754f, 0.002285235794261098f, 0.01777736470103264f, 0.09899555146694183f, 0.3792743682861328f, 0.8778833150863647f, 0.5186641216278076f, 0.8778833150863647f, 0.3792743682861328f, 0.09899555146694183f, 0.01777736470103264f, 0.002285235794261098f, 0.00020678013970609754f, 1.1724255273293238e-05f};
-static __constant__ float kQuadTrig8[330] = {1.0f, 0.9898214340209961f, 0.1423148363828659f, 0.9594929814338684f, 0.28173255920410156f, 0.9096319675445557f, 0.4154150187969208f, 0.8412535190582275f, 0.5406408309936523f, 0.7557495832443237f, 0.6548607349395752f, 0.6548607349395752f, 0.7557495832443237f, 0.5406408309936523f, 0.8412535190582275f, 1.0f, 0.9096319675445557f, 0.4154150187969208f, 0.6548607349395752f, 0.7557495832443237f, 0.28173255920410156f, 0.9594929814338684f, -0.1423148363828659f, 0.9898214340209961f, -0.5406408309936523f, 0.8412535190582275f, -0.8412535190582275f, 0.5406408309936523f, -0.9898214340209961f, 0.1423148363828659f, 1.0f, 0.7557495832443237f, 0.6548607349395752f, 0.1423148363828659f, 0.9898214340209961f, -0.5406408309936523f, 0.8412535190582275f, -0.9594929814338684f, 0.28173255920410156f, -0.9096319675445557f, -0.4154150187969208f, -0.4154150187969208f, -0.9096319675445557f, 0.28173255920410156f, -0.9594929814338684f, 1.0f, 0.5406408309936523f, 0.8412535190582275f, -0.4154150187969208f, 0.9096319675445557f, -0.9898214340209961f, 0.1423148363828659f, -0.6548607349395752f, -0.7557495832443237f, 0.28173255920410156f, -0.9594929814338684f, 0.9594929814338684f, -0.28173255920410156f, 0.7557495832443237f, 0.6548607349395752f, 1.0f, 0.28173255920410156f, 0.9594929814338684f, -0.8412535190582275f, 0.5406408309936523f, -0.7557495832443237f, -0.6548607349395752f, 0.4154150187969208f, -0.9096319675445557f, 0.9898214340209961f, 0.1423148363828659f, 0.1423148363828659f, 0.9898214340209961f, -0.9096319675445557f, 0.4154150187969208f, 1.0f, 2.832769343193999e-16f, 1.0f, -1.0f, 5.665538686387998e-16f, -1.071875407883231e-15f, -1.0f, 1.0f, -1.1331077372775996e-15f, 1.1943400666719682e-15f, 1.0f, -1.0f, 2.143750815766462e-15f, -2.204983251039949e-15f, -1.0f, 1.0f, -0.28173255920410156f, 0.9594929814338684f, -0.8412535190582275f, -0.5406408309936523f, 0.7557495832443237f, -0.6548607349395752f, 0.4154150187969208f, 0.9096319675445557f, -0.9898214340209961f, 0.1423148363828659f, 0.1423148363828659f, -0.9898214340209961f, 0.9096319675445557f, 0.4154150187969208f, 1.0f, -0.5406408309936523f, 0.8412535190582275f, -0.4154150187969208f, -0.9096319675445557f, 0.9898214340209961f, 0.1423148363828659f, -0.6548607349395752f, 0.7557495832443237f, -0.28173255920410156f, -0.9594929814338684f, 0.9594929814338684f, 0.28173255920410156f, -0.7557495832443237f, 0.6548607349395752f, 1.0f, -0.7557495832443237f, 0.6548607349395752f, 0.1423148363828659f, -0.9898214340209961f, 0.5406408309936523f, 0.8412535190582275f, -0.9594929814338684f, -0.28173255920410156f, 0.9096319675445557f, -0.4154150187969208f, -0.4154150187969208f, 0.9096319675445557f, -0.28173255920410156f, -0.9594929814338684f, 1.0f, -0.9096319675445557f, 0.4154150187969208f, 0.6548607349395752f, -0.7557495832443237f, -0.28173255920410156f, 0.9594929814338684f, -0.1423148363828659f, -0.9898214340209961f, 0.5406408309936523f, 0.8412535190582275f, -0.8412535190582275f, -0.5406408309936523f, 0.9898214340209961f, 0.1423148363828659f, 1.0f, -0.9898214340209961f, 0.1423148363828659f, 0.9594929814338684f, -0.28173255920410156f, -0.9096319675445557f, 0.4154150187969208f, 0.8412535190582275f, -0.5406408309936523f, -0.7557495832443237f, 0.6548607349395752f, 0.6548607349395752f, -0.7557495832443237f, -0.5406408309936523f, 0.8412535190582275f, 1.0f, -0.9898214340209961f, -0.1423148363828659f, 0.9594929814338684f, 0.28173255920410156f, -0.9096319675445557f, -0.4154150187969208f, 0.8412535190582275f, 0.5406408309936523f, -0.7557495832443237f, -0.6548607349395752f, 0.6548607349395752f, 0.7557495832443237f, -0.5406408309936523f, -0.8412535190582275f, 1.0f, -0.9096319675445557f, -0.4154150187969208f, 0.6548607349395752f, 0.7557495832443237f, -0.28173255920410156f, -0.9594929814338684f, -0.1423148363828659f, 0.9898214340209961f, 0.5406408309936523f, -0.8412535190582275f, -0.8412535190582275f, 0.5406408309936523f, 0.9898214340209961f, -0.1423148363828659f, 1.0f, -0.7557495832443237f, -0.6548607349395752f, 0.1423148363828659f, 0.9898214340209961f, 0.5406408309936523f, -0.8412535190582275f, -0.9594929814338684f, 0.28173255920410156f, 0.9096319675445557f, 0.4154150187969208f, -0.4154150187969208f, -0.9096319675445557f, -0.28173255920410156f, 0.9594929814338684f, 1.0f, -0.5406408309936523f, -0.8412535190582275f, -0.4154150187969208f, 0.9096319675445557f, 0.9898214340209961f, -0.1423148363828659f, -0.6548607349395752f, -0.7557495832443237f, -0.28173255920410156f, 0.9594929814338684f, 0.9594929814338684f, -0.28173255920410156f, -0.7557495832443237f, -0.6548607349395752f, 1.0f, -0.28173255920410156f, -0.9594929814338684f, -0.8412535190582275f, 0.5406408309936523f, 0.7557495832443237f, 0.6548607349395752f, 0.4154150187969208f, -0.9096319675445557f, -0.9898214340209961f, -0.1423148363828659f, 0.1423148363828659f, 0.9898214340209961f, 0.9096319675445557f, -0.4154150187969208f, 1.0f, -1.8369701465288538e-16f, -1.0f, -1.0f, 3.6739402930577075e-16f, 5.510910704284357e-16f, 1.0f, 1.0f, -7.347880586115415e-16f, -2.6948418861948977e-15f, -1.0f, -1.0f, 1.1021821408568715e-15f, -4.904777103602732e-16f, 1.0f, 1.0f, 0.28173255920410156f, -0.9594929814338684f, -0.8412535190582275f, -0.5406408309936523f, -0.7557495832443237f, 0.6548607349395752f, 0.4154150187969208f, 0.9096319675445557f, 0.9898214340209961f, -0.1423148363828659f, 0.1423148363828659f, -0.9898214340209961f, -0.9096319675445557f, -0.4154150187969208f, 1.0f, 0.5406408309936523f, -0.8412535190582275f, -0.4154150187969208f, -0.9096319675445557f, -0.9898214340209961f, -0.1423148363828659f, -0.6548607349395752f, 0.7557495832443237f, 0.28173255920410156f, 0.9594929814338684f, 0.9594929814338684f, 0.28173255920410156f, 0.7557495832443237f, -0.6548607349395752f, 1.0f, 0.7557495832443237f, -0.6548607349395752f, 0.1423148363828659f, -0.9898214340209961f, -0.5406408309936523f, -0.8412535190582275f, -0.9594929814338684f, -0.28173255920410156f, -0.9096319675445557f, 0.4154150187969208f, -0.4154150187969208f, 0.9096319675445557f, 0.28173255920410156f, 0.9594929814338684f, 1.0f, 0.9096319675445557f, -0.4154150187969208f, 0.6548607349395752f, -0.7557495832443237f, 0.28173255920410156f, -0.9594929814338684f, -0.1423148363828659f, -0.9898214340209961f, -0.5406408309936523f, -0.8412535190582275f, -0.8412535190582275f, -0.5406408309936523f, -0.9898214340209961f, -0.1423148363828659f, 1.0f, 0.9898214340209961f, -0.1423148363828659f, 0.9594929814338684f, -0.28173255920410156f, 0.9096319675445557f, -0.4154150187969208f, 0.8412535190582275f, -0.5406408309936523f, 0.7557495832443237f, -0.6548607349395752f, 0.6548607349395752f, -0.7557495832443237f, 0.5406408309936523f, -0.8412535190582275f};
-static __constant__ float kQuadW8[11] = {0.01589890569448471f, 0.035865668207407f, 0.053204361349344254f, 0.06659997999668121f, 0.07505679875612259f, 0.0779472216963768f, 0.07505679875612259f, 0.06659997999668121f, 0.053204361349344254f, 0.035865668207407f, 0.01589890569448471f};
-#endif
-#if defined(SHS_NB) && SHS_NB == 8
-static __constant__ float kExpLeg8[1024] = {0.282094806432724f, 0.07094971090555191f, -0.48342376947402954f, 0.07094971090555191f, 0.011518623679876328f, -0.15696685016155243f, 0.6108322739601135f, -0.15696685016155243f, 0.011518623679876328f, 0.0018066286575049162f, -0.030152400955557823f, 0.2584724724292755f, -0.6995154619216919f, 0.2584724724292755f, -0.030152400955557823f, 0.0018066286575049162f, 0.00027825316647067666f, -0.00536244036629796f, 0.05838014557957649f, -0.3703010082244873f, 0.7587076425552368f, -0.3703010082244873f, 0.05838014557957649f, -0.00536244036629796f, 0.00027825316647067666f, 4.237711618770845e-05f, -0.0009130798862315714f, 0.011699545197188854f, -0.09684120118618011f, 0.48795923590660095f, -0.7922953963279724f, 0.48795923590660095f, -0.09684120118618011f, 0.011699545197188854f, -0.0009130798862315714f, 4.237711618770845e-05f, 6.4048267631733324e-06f, -0.00015117340080905706f, 0.0021913156379014254f, -0.02167833410203457f, 0.14570735394954681f, -0.6073318123817444f, 0.8024648427963257f, -0.6073318123817444f, 0.14570735394954681f, -0.02167833410203457f, 0.0021913156379014254f, -0.00015117340080905706f, 6.4048267631733324e-06f, 9.626843393562012e-07f, -2.454286914144177e-05f, 0.000392841175198555f, -0.004440254531800747f, 0.0361325666308403f, -0.204736590385437f, 0.7245708703994751f, -0.7908328771591187f, 0.7245708703994751f, -0.204736590385437f, 0.0361325666308403f, -0.004440254531800747f, 0.000392841175198555f, -2.454286914144177e-05f, 9.626843393562012e-07f, 0.282094806432724f, 0.16040606796741486f, -0.461521714925766f, 0.16040606796741486f, 0.05887635797262192f, -0.3387991189956665f, 0.5288062691688538f, -0.3387991189956665f, 0.05887635797262192f, 0.020877545699477196f, -0.14713852107524872f, 0.5193262100219727f, -0.5150310397148132f, 0.5193262100219727f, -0.14713852107524872f, 0.020877545699477196f, 0.007269772235304117f, -0.0591612234711647f, 0.26746249198913574f, -0.6733590960502625f, 0.4332386255264282f, -0.6733590960502625f, 0.26746249198913574f, -0.0591612234711647f, 0.007269772235304117f, 0.002503123367205262f, -0.022774748504161835f, 0.12169450521469116f, -0.4091092348098755f, 0.7771311402320862f, -0.29784974455833435f, 0.7771311402320862f, -0.4091092348098755f, 0.12169450521469116f, -0.022774748504161835f, 0.002503123367205262f, 0.0008553196093998849f, -0.008524921722710133f, 0.051662128418684006f, -0.20980627834796906f, 0.5564955472946167f, -0.8136188983917236f, 0.12681901454925537f, -0.8136188983917236f, 0.5564955472946167f, -0.20980627834796906f, 0.051662128418684006f, -0.008524921722710133f, 0.0008553196093998849f, 0.000290653231786564f, -0.0031290357001125813f, 0.020974058657884598f, -0.09791873395442963f, 0.32081058621406555f, -0.691368579864502f, 0.774089515209198f, 0.05915773659944534f, 0.774089515209198f, -0.691368579864502f, 0.32081058621406555f, -0.09791873395442963f, 0.020974058657884598f, -0.0031290357001125813f, 0.000290653231786564f, 0.282094806432724f, 0.24463455379009247f, -0.42294958233833313f, 0.24463455379009247f, 0.13694144785404205f, -0.47351714968681335f, 0.39359357953071594f, -0.47351714968681335f, 0.13694144785404205f, 0.07405773550271988f, -0.3136294484138489f, 0.6285143494606018f, -0.24117226898670197f, 0.6285143494606018f, -0.3136294484138489f, 0.07405773550271988f, 0.03932863101363182f, -0.1923200637102127f, 0.5034611225128174f, -0.6510443687438965f, 0.018211757764220238f, -0.6510443687438965f, 0.5034611225128174f, -0.1923200637102127f, 0.03932863101363182f, 0.020652245730161667f, -0.11291147023439407f, 0.3527039885520935f, -0.6490544676780701f, 0.5217272043228149f, 0.21048904955387115f, 0.5217272043228149f, -0.6490544676780701f, 0.3527039885520935f, -0.11291147023439407f, 0.020652245730161667f, 0.010762432590126991f, -0.06445726007223129f, 0.22964313626289368f, -0.524702787399292f, 0.6975259780883789f, -0.26493629813194275f, -0.38138410449028015f, -0.26493629813194275f, 0.6975259780883789f, -0.524702787399292f, 0.22964313626289368f, -0.06445726007223129f, 0.010762432590126991f, 0.005577687174081802f, -0.036081865429878235f, 0.1427166610956192f, -0.3805752098560333f, 0.6644591093063354f, -0.6177658438682556f, -0.0579991415143013f, 0.44790521264076233f, -0.0579991415143013f, -0.6177658438682556f, 0.6644591093063354f, -0.3805752098560333f, 0.1427166610956192f, -0.036081865429878235f, 0.005577687174081802f, 0.282094806432724f, 0.3201611340045929f, -0.36909249424934387f, 0.3201611340045929f, 0.2345505803823471f, -0.5407955646514893f, 0.22452960908412933f, -0.5407955646514893f, 0.2345505803823471f, 0.16600562632083893f, -0.4687756597995758f, 0.5549961924552917f, 0.04138867184519768f, 0.5549961924552917f, -0.4687756597995758f, 0.16600562632083893f, 0.11537507176399231f, -0.37620416283607483f, 0.6082530617713928f, -0.32933056354522705f, -0.2879684865474701f, -0.32933056354522705f, 0.6082530617713928f, -0.37620416283607483f, 0.11537507176399231f, 0.07929050922393799f, -0.2890598773956299f, 0.5692598223686218f, -0.5534201264381409f, -0.044748563319444656f, 0.3913777768611908f, -0.044748563319444656f, -0.5534201264381409f, 0.5692598223686218f, -0.2890598773956299f, 0.07929050922393799f, 0.05407732352614403f, -0.2159595489501953f, 0.4908573031425476f, -0.6415792107582092f, 0.29154467582702637f, 0.39608559012413025f, -0.3008277714252472f, 0.39608559012413025f, 0.29154467582702637f, -0.6415792107582092f, 0.4908573031425476f, -0.2159595489501953f, 0.05407732352614403f, 0.03667834401130676f, -0.1582123339176178f, 0.402326762676239f, -0.6385716795921326f, 0.5239323973655701f, 0.08651652932167053f, -0.5584453344345093f, 0.06159166991710663f, -0.5584453344345093f, 0.08651652932167053f, 0.5239323973655701f, -0.6385716795921326f, 0.402326762676239f, -0.1582123339176178f, 0.03667834401130676f, 0.282094806432724f, 0.384176105260849f, -0.3018958866596222f, 0.384176105260849f, 0.3377225399017334f, -0.5307828187942505f, 0.04583054408431053f, -0.5307828187942505f, 0.3377225399017334f, 0.28681913018226624f, -0.5520908832550049f, 0.32660973072052f, 0.25159263610839844f, 0.32660973072052f, -0.5520908832550049f, 0.28681913018226624f, 0.23919881880283356f, -0.5316561460494995f, 0.48913657665252686f, 0.10648290067911148f, -0.35458382964134216f, 0.10648290067911148f, 0.48913657665252686f, -0.5316561460494995f, 0.23919881880283356f, 0.1972559243440628f, -0.49018144607543945f, 0.57930988073349f, -0.13303987681865692f, -0.4573071599006653f, 0.1836709827184677f, -0.4573071599006653f, -0.13303987681865692f, 0.57930988073349f, -0.49018144607543945f, 0.1972559243440628f, 0.16143056750297546f, -0.4394436776638031f, 0.6170144081115723f, -0.331875741481781f, -0.30245769023895264f, 0.4651665985584259f, 0.12894819676876068f, 0.4651665985584259f, -0.30245769023895264f, -0.331875741481781f, 0.6170144081115723f, -0.4394436776638031f, 0.16143056750297546f, 0.13138386607170105f, -0.3863072693347931f, 0.6180117130279541f, -0.4811188876628876f, -0.10303568840026855f, 0.5200333595275879f, -0.12329808622598648f, -0.34278231859207153f, -0.12329808622598648f, 0.5200333595275879f, -0.10303568840026855f, -0.4811188876628876f, 0.6180117130279541f, -0.3863072693347931f, 0.13138386607170105f, 0.282094806432724f, 0.43434005975723267f, -0.22378814220428467f, 0.43434005975723267f, 0.4316771626472473f, -0.4448322653770447f, -0.1169036328792572f, -0.4448322653770447f, 0.4316771626472473f, 0.4144829213619232f, -0.5231057405471802f, 0.01986619643867016f, 0.3334845304489136f, 0.01986619643867016f, -0.5231057405471802f, 0.4144829213619232f, 0.390802264213562f, -0.5695204138755798f, 0.1751290261745453f, 0.4171973168849945f, -0.18545503914356232f, 0.4171973168849945f, 0.1751290261745453f, -0.5695204138755798f, 0.390802264213562f, 0.3643574118614197f, -0.5936559438705444f, 0.30518484115600586f, 0.3215390741825104f, -0.40778017044067383f, -0.1654045134782791f, -0.40778017044067383f, 0.3215390741825104f, 0.30518484115600586f, -0.5936559438705444f, 0.3643574118614197f, 0.3371187150478363f, -0.6017009019851685f, 0.4119834005832672f, 0.20522691309452057f, -0.4818282127380371f, -0.03768457472324371f, 0.33673009276390076f, -0.03768457472324371f, -0.4818282127380371f, 0.20522691309452057f, 0.4119834005832672f, -0.6017009019851685f, 0.3371187150478363f, 0.31019774079322815f, -0.5980119705200195f, 0.4975000023841858f, 0.08099491894245148f, -0.5003358721733093f, 0.14276351034641266f, 0.44140905141830444f, -0.14211028814315796f, 0.44140905141830444f, 0.14276351034641266f, -0.5003358721733093f, 0.08099491894245148f, 0.4975000023841858f, -0.5980119705200195f, 0.31019774079322815f, 0.282094806432724f, 0.4688291847705841f, -0.13759219646453857f, 0.4688291847705841f, 0.502954363822937f, -0.29521456360816956f, -0.2403593808412552f, -0.29521456360816956f, 0.502954363822937f, 0.521267831325531f, -0.37472763657569885f, -0.264663428068161f, 0.27359575033187866f, -0.264663428068161f, -0.37472763657569885f, 0.521267831325531f, 0.5305131077766418f, -0.44037261605262756f, -0.1937839388847351f, 0.44199138879776f, 0.0889744758605957f, 0.44199138879776f, -0.1937839388847351f, -0.44037261605262756f, 0.5305131077766418f, 0.5338895320892334f, -0.4954850971698761f, -0.12374024838209152f, 0.4735797047615051f, 0.009497372433543205f, -0.3242362141609192f, 0.009497372433543205f, 0.4735797047615051f, -0.12374024838209152f, -0.4954850971698761f, 0.5338895320892334f, 0.5332015156745911f, -0.5420773029327393f, -0.05461635813117027f, 0.4876188635826111f, -0.09324891865253448f, -0.4452876150608063f, 0.09286528080701828f, -0.4452876150608063f, -0.09324891865253448f, 0.4876188635826111f, -0.05461635813117027f, -0.5420773029327393f, 0.5332015156745911f, 0.5295804738998413f, -0.5815340280532837f, 0.013045242987573147f, 0.4878280460834503f, -0.18446695804595947f, -0.41168612241744995f, 0.24327048659324646f, 0.27236804366111755f, 0.24327048659324646f, -0.41168612241744995f, -0.18446695804595947f, 0.4878280460834503f, 0.013045242987573147f, -0.5815340280532837f, 0.5295804738998413f, 0.282094806432724f, 0.4863921105861664f, -0.046423349529504776f, 0.4863921105861664f, 0.5413427948951721f, -0.1033361628651619f, -0.3068500757217407f, -0.1033361628651619f, 0.5413427948951721f, 0.582071840763092f, -0.1360824704170227f, -0.43444186449050903f, 0.10476886481046677f, -0.43444186449050903f, -0.1360824704170227f, 0.582071840763092f, 0.6145874261856079f, -0.16591231524944305f, -0.4391913115978241f, 0.1858418732881546f, 0.2890093922615051f, 0.1858418732881546f, -0.4391913115978241f, -0.16591231524944305f, 0.6145874261856079f, 0.6416686773300171f, -0.19366930425167084f, -0.44341665506362915f, 0.21955569088459015f, 0.394683301448822f, -0.15971150994300842f, 0.394683301448822f, 0.21955569088459015f, -0.44341665506362915f, -0.19366930425167084f, 0.6416686773300171f, 0.6648485660552979f, -0.21981802582740784f, -0.4462928771972656f, 0.2504565119743347f, 0.38350313901901245f, -0.2607538104057312f, -0.2592114210128784f, -0.2607538104057312f, 0.38350313901901245f, 0.2504565119743347f, -0.4462928771972656f, -0.21981802582740784f, 0.6648485660552979f, 0.6850703358650208f, -0.24465221166610718f, -0.44775089621543884f, 0.27913984656333923f, 0.37287411093711853f, -0.2920544147491455f, -0.34362509846687317f, 0.2089904397726059f, -0.34362509846687317f, -0.2920544147491455f, 0.37287411093711853f, 0.27913984656333923f, -0.44775089621543884f, -0.24465221166610718f, 0.6850703358650208f, 0.282094806432724f, 0.4863921105861664f, 0.046423349529504776f, 0.4863921105861664f, 0.5413427948951721f, 0.1033361628651619f, -0.3068500757217407f, 0.1033361628651619f, 0.5413427948951721f, 0.582071840763092f, 0.1360824704170227f, -0.43444186449050903f, -0.10476886481046677f, -0.43444186449050903f, 0.1360824704170227f, 0.582071840763092f, 0.6145874261856079f, 0.16591231524944305f, -0.4391913115978241f, -0.1858418732881546f, 0.2890093922615051f, -0.1858418732881546f, -0.4391913115978241f, 0.16591231524944305f, 0.6145874261856079f, 0.6416686773300171f, 0.19366930425167084f, -0.44341665506362915f, -0.21955569088459015f, 0.394683301448822f, 0.15971150994300842f, 0.394683301448822f, -0.21955569088459015f, -0.44341665506362915f, 0.19366930425167084f, 0.6416686773300171f, 0.6648485660552979f, 0.21981802582740784f, -0.4462928771972656f, -0.2504565119743347f, 0.38350313901901245f, 0.2607538104057312f, -0.2592114210128784f, 0.2607538104057312f, 0.38350313901901245f, -0.2504565119743347f, -0.4462928771972656f, 0.21981802582740784f, 0.6648485660552979f, 0.6850703358650208f, 0.24465221166610718f, -0.44775089621543884f, -0.27913984656333923f, 0.37287411093711853f, 0.2920544147491455f, -0.34362509846687317f, -0.2089904397726059f, -0.34362509846687317f, 0.2920544147491455f, 0.37287411093711853f, -0.27913984656333923f, -0.44775089621543884f, 0.24465221166610718f, 0.6850703358650208f, 0.282094806432724f, 0.4688291847705841f, 0.13759219646453857f, 0.4688291847705841f, 0.502954363822937f, 0.29521456360816956f, -0.2403593808412552f, 0.29521456360816956f, 0.502954363822937f, 0.521267831325531f, 0.37472763657569885f, -0.264663428068161f, -0.27359575033187866f, -0.264663428068161f, 0.37472763657569885f, 0.521267831325531f, 0.5305131077766418f, 0.44037261605262756f, -0.1937839388847351f, -0.44199138879776f, 0.0889744758605957f, -0.44199138879776f, -0.1937839388847351f, 0.44037261605262756f, 0.5305131077766418f, 0.5338895320892334f, 0.4954850971698761f, -0.12374024838209152f, -0.4735797047615051f, 0.009497372433543205f, 0.3242362141609192f, 0.009497372433543205f, -0.4735797047615051f, -0.12374024838209152f, 0.4954850971698761f, 0.5338895320892334f, 0.5332015156745911f, 0.5420773029327393f, -0.05461635813117027f, -0.4876188635826111f, -0.09324891865253448f, 0.4452876150608063f, 0.09286528080701828f, 0.4452876150608063f, -0.09324891865253448f, -0.4876188635826111f, -0.05461635813117027f, 0.5420773029327393f, 0.5332015156745911f, 0.5295804738998413f, 0.5815340280532837f, 0.013045242987573147f, -0.4878280460834503f, -0.18446695804595947f, 0.41168612241744995f, 0.24327048659324646f, -0.27236804366111755f, 0.24327048659324646f, 0.41168612241744995f, -0.18446695804595947f, -0.4878280460834503f, 0.013045242987573147f, 0.5815340280532837f, 0.5295804738998413f, 0.282094806432724f, 0.43434005975723267f, 0.22378814220428467f, 0.43434005975723267f, 0.4316771626472473f, 0.4448322653770447f, -0.1169036328792572f, 0.4448322653770447f, 0.4316771626472473f, 0.4144829213619232f, 0.5231057405471802f, 0.01986619643867016f, -0.3334845304489136f, 0.01986619643867016f, 0.5231057405471802f, 0.4144829213619232f, 0.390802264213562f, 0.5695204138755798f, 0.1751290261745453f, -0.4171973168849945f, -0.18545503914356232f, -0.4171973168849945f, 0.1751290261745453f, 0.5695204138755798f, 0.390802264213562f, 0.3643574118614197f, 0.5936559438705444f, 0.30518484115600586f, -0.3215390741825104f, -0.40778017044067383f, 0.1654045134782791f, -0.40778017044067383f, -0.3215390741825104f, 0.30518484115600586f, 0.5936559438705444f, 0.3643574118614197f, 0.3371187150478363f, 0.6017009019851685f, 0.4119834005832672f, -0.20522691309452057f, -0.4818282127380371f, 0.03768457472324371f, 0.33673009276390076f, 0.03768457472324371f, -0.4818282127380371f, -0.20522691309452057f, 0.4119834005832672f, 0.6017009019851685f, 0.3371187150478363f, 0.31019774079322815f, 0.5980119705200195f, 0.4975000023841858f, -0.08099491894245148f, -0.5003358721733093f, -0.14276351034641266f, 0.44140905141830444f, 0.14211028814315796f, 0.44140905141830444f, -0.14276351034641266f, -0.5003358721733093f, -0.08099491894245148f, 0.4975000023841858f, 0.5980119705200195f, 0.31019774079322815f, 0.282094806432724f, 0.384176105260849f, 0.3018958866596222f, 0.384176105260849f, 0.3377225399017334f, 0.5307828187942505f, 0.04583054408431053f, 0.5307828187942505f, 0.3377225399017334f, 0.28681913018226624f, 0.5520908832550049f, 0.32660973072052f, -0.25159263610839844f, 0.32660973072052f, 0.5520908832550049f, 0.28681913018226624f, 0.23919881880283356f, 0.5316561460494995f, 0.48913657665252686f, -0.10648290067911148f, -0.35458382964134216f, -0.10648290067911148f, 0.48913657665252686f, 0.5316561460494995f, 0.23919881880283356f, 0.1972559243440628f, 0.49018144607543945f, 0.57930988073349f, 0.13303987681865692f, -0.4573071599006653f, -0.1836709827184677f, -0.4573071599006653f, 0.13303987681865692f, 0.57930988073349f, 0.49018144607543945f, 0.1972559243440628f, 0.16143056750297546f, 0.4394436776638031f, 0.6170144081115723f, 0.331875741481781f, -0.30245769023895264f, -0.4651665985584259f, 0.12894819676876068f, -0.4651665985584259f, -0.30245769023895264f, 0.331875741481781f, 0.6170144081115723f, 0.4394436776638031f, 0.16143056750297546f, 0.13138386607170105f, 0.3863072693347931f, 0.6180117130279541f, 0.4811188876628876f, -0.10303568840026855f, -0.5200333595275879f, -0.12329808622598648f, 0.34278231859207153f, -0.12329808622598648f, -0.5200333595275879f, -0.10303568840026855f, 0.4811188876628876f, 0.6180117130279541f, 0.3863072693347931f, 0.13138386607170105f, 0.282094806432724f, 0.3201611340045929f, 0.36909249424934387f, 0.3201611340045929f, 0.2345505803823471f, 0.5407955646514893f, 0.22452960908412933f, 0.5407955646514893f, 0.2345505803823471f, 0.16600562632083893f, 0.4687756597995758f, 0.5549961924552917f, -0.04138867184519768f, 0.5549961924552917f, 0.4687756597995758f, 0.16600562632083893f, 0.11537507176399231f, 0.37620416283607483f, 0.6082530617713928f, 0.32933056354522705f, -0.2879684865474701f, 0.32933056354522705f, 0.6082530617713928f, 0.37620416283607483f, 0.11537507176399231f, 0.07929050922393799f, 0.2890598773956299f, 0.5692598223686218f, 0.5534201264381409f, -0.044748563319444656f, -0.3913777768611908f, -0.044748563319444656f, 0.5534201264381409f, 0.5692598223686218f, 0.2890598773956299f, 0.07929050922393799f, 0.05407732352614403f, 0.2159595489501953f, 0.4908573031425476f, 0.6415792107582092f, 0.29154467582702637f, -0.39608559012413025f, -0.3008277714252472f, -0.39608559012413025f, 0.29154467582702637f, 0.6415792107582092f, 0.4908573031425476f, 0.2159595489501953f, 0.05407732352614403f, 0.03667834401130676f, 0.1582123339176178f, 0.402326762676239f, 0.6385716795921326f, 0.5239323973655701f, -0.08651652932167053f, -0.5584453344345093f, -0.06159166991710663f, -0.5584453344345093f, -0.08651652932167053f, 0.5239323973655701f, 0.6385716795921326f, 0.402326762676239f, 0.1582123339176178f, 0.03667834401130676f, 0.282094806432724f, 0.24463455379009247f, 0.42294958233833313f, 0.24463455379009247f, 0.13694144785404205f, 0.47351714968681335f, 0.39359357953071594f, 0.47351714968681335f, 0.13694144785404205f, 0.07405773550271988f, 0.3136294484138489f, 0.6285143494606018f, 0.24117226898670197f, 0.6285143494606018f, 0.3136294484138489f, 0.07405773550271988f, 0.03932863101363182f, 0.1923200637102127f, 0.5034611225128174f, 0.6510443687438965f, 0.018211757764220238f, 0.6510443687438965f, 0.5034611225128174f, 0.1923200637102127f, 0.03932863101363182f, 0.020652245730161667f, 0.11291147023439407f, 0.3527039885520935f, 0.6490544676780701f, 0.5217272043228149f, -0.21048904955387115f, 0.5217272043228149f, 0.6490544676780701f, 0.3527039885520935f, 0.11291147023439407f, 0.020652245730161667f, 0.010762432590126991f, 0.06445726007223129f, 0.22964313626289368f, 0.524702787399292f, 0.6975259780883789f, 0.26493629813194275f, -0.38138410449028015f, 0.26493629813194275f, 0.6975259780883789f, 0.524702787399292f, 0.22964313626289368f, 0.06445726007223129f, 0.010762432590126991f, 0.005577687174081802f, 0.036081865429878235f, 0.1427166610956192f, 0.3805752098560333f, 0.6644591093063354f, 0.6177658438682556f, -0.0579991415143013f, -0.44790521264076233f, -0.0579991415143013f, 0.6177658438682556f, 0.6644591093063354f, 0.3805752098560333f, 0.1427166610956192f, 0.036081865429878235f, 0.005577687174081802f, 0.282094806432724f, 0.16040606796741486f, 0.461521714925766f, 0.16040606796741486f, 0.05887635797262192f, 0.3387991189956665f, 0.5288062691688538f, 0.3387991189956665f, 0.05887635797262192f, 0.020877545699477196f, 0.14713852107524872f, 0.5193262100219727f, 0.5150310397148132f, 0.5193262100219727f, 0.14713852107524872f, 0.020877545699477196f, 0.007269772235304117f, 0.0591612234711647f, 0.26746249198913574f, 0.6733590960502625f, 0.4332386255264282f, 0.6733590960502625f, 0.26746249198913574f, 0.0591612234711647f, 0.007269772235304117f, 0.002503123367205262f, 0.022774748504161835f, 0.12169450521469116f, 0.4091092348098755f, 0.7771311402320862f, 0.29784974455833435f, 0.7771311402320862f, 0.4091092348098755f, 0.12169450521469116f, 0.022774748504161835f, 0.002503123367205262f, 0.0008553196093998849f, 0.008524921722710133f, 0.051662128418684006f, 0.20980627834796906f, 0.5564955472946167f, 0.8136188983917236f, 0.12681901454925537f, 0.8136188983917236f, 0.5564955472946167f, 0.20980627834796906f, 0.051662128418684006f, 0.008524921722710133f, 0.0008553196093998849f, 0.000290653231786564f, 0.0031290357001125813f, 0.020974058657884598f, 0.09791873395442963f, 0.32081058621406555f, 0.691368579864502f, 0.774089515209198f, -0.05915773659944534f, 0.774089515209198f, 0.691368579864502f, 0.32081058621406555f, 0.09791873395442963f, 0.020974058657884598f, 0.0031290357001125813f, 0.000290653231786564f, 0.282094806432724f, 0.07094971090555191f, 0.48342376947402954f, 0.07094971090555191f, 0.011518623679876328f, 0.15696685016155243f, 0.6108322739601135f, 0.15696685016155243f, 0.011518623679876328f, 0.0018066286575049162f, 0.030152400955557823f, 0.2584724724292755f, 0.6995154619216919f, 0.2584724724292755f, 0.030152400955557823f, 0.0018066286575049162f, 0.00027825316647067666f, 0.00536244036629796f, 0.05838014557957649f, 0.3703010082244873f, 0.7587076425552368f, 0.3703010082244873f, 0.05838014557957649f, 0.00536244036629796f, 0.00027825316647067666f, 4.237711618770845e-05f, 0.0009130798862315714f, 0.011699545197188854f, 0.09684120118618011f, 0.48795923590660095f, 0.7922953963279724f, 0.48795923590660095f, 0.09684120118618011f, 0.011699545197188854f, 0.0009130798862315714f, 4.237711618770845e-05f, 6.4048267631733324e-06f, 0.00015117340080905706f, 0.0021913156379014254f, 0.02167833410203457f, 0.14570735394954681f, 0.6073318123817444f, 0.8024648427963257f, 0.6073318123817444f, 0.14570735394954681f, 0.02167833410203457f, 0.0021913156379014254f, 0.00015117340080905706f, 6.4048267631733324e-06f, 9.626843393562012e-07f, 2.454286914144177e-05f, 0.000392841175198555f, 0.004440254531800747f, 0.0361325666308403f, 0.204736590385437f, 0.7245708703994751f, 0.7908328771591187f, 0.7245708703994751f, 0.204736590385437f, 0.0361325666308403f, 0.004440254531800747f, 0.000392841175198555f, 2.454286914144177e-05f, 9.626843393562012e-07f};
-static __constant__ float kExpTrig8[480] = {1.0f, 0.9951847195625305f, 0.0980171412229538f, 0.9807852506637573f, 0.19509032368659973f, 0.9569403529167175f, 0.290284663438797f, 0.9238795042037964f, 0.3826834261417389f, 0.8819212913513184f, 0.4713967442512512f, 0.8314695954322815f, 0.5555702447891235f, 0.7730104327201843f, 0.6343932747840881f, 1.0f, 0.9569403529167175f, 0.290284663438797f, 0.8314695954322815f, 0.5555702447891235f, 0.6343932747840881f, 0.7730104327201843f, 0.3826834261417389f, 0.9238795042037964f, 0.0980171412229538f, 0.9951847195625305f, -0.19509032368659973f, 0.9807852506637573f, -0.4713967442512512f, 0.8819212913513184f, 1.0f, 0.8819212913513184f, 0.4713967442512512f, 0.5555702447891235f, 0.8314695954322815f, 0.0980171412229538f, 0.9951847195625305f, -0.3826834261417389f, 0.9238795042037964f, -0.7730104327201843f, 0.6343932747840881f, -0.9807852506637573f, 0.19509032368659973f, -0.9569403529167175f, -0.290284663438797f, 1.0f, 0.7730104327201843f, 0.6343932747840881f, 0.19509032368659973f, 0.9807852506637573f, -0.4713967442512512f, 0.8819212913513184f, -0.9238795042037964f, 0.3826834261417389f, -0.9569403529167175f, -0.290284663438797f, -0.5555702447891235f, -0.8314695954322815f, 0.0980171412229538f, -0.9951847195625305f, 1.0f, 0.6343932747840881f, 0.7730104327201843f, -0.19509032368659973f, 0.9807852506637573f, -0.8819212913513184f, 0.4713967442512512f, -0.9238795042037964f, -0.3826834261417389f, -0.290284663438797f, -0.9569403529167175f, 0.5555702447891235f, -0.8314695954322815f, 0.9951847195625305f, -0.0980171412229538f, 1.0f, 0.4713967442512512f, 0.8819212913513184f, -0.5555702447891235f, 0.8314695954322815f, -0.9951847195625305f, -0.0980171412229538f, -0.3826834261417389f, -0.9238795042037964f, 0.6343932747840881f, -0.7730104327201843f, 0.9807852506637573f, 0.19509032368659973f, 0.290284663438797f, 0.9569403529167175f, 1.0f, 0.290284663438797f, 0.9569403529167175f, -0.8314695954322815f, 0.5555702447891235f, -0.7730104327201843f, -0.6343932747840881f, 0.3826834261417389f, -0.9238795042037964f, 0.9951847195625305f, 0.0980171412229538f, 0.19509032368659973f, 0.9807852506637573f, -0.8819212913513184f, 0.4713967442512512f, 1.0f, 0.0980171412229538f, 0.9951847195625305f, -0.9807852506637573f, 0.19509032368659973f, -0.290284663438797f, -0.9569403529167175f, 0.9238795042037964f, -0.3826834261417389f, 0.4713967442512512f, 0.8819212913513184f, -0.8314695954322815f, 0.5555702447891235f, -0.6343932747840881f, -0.7730104327201843f, 1.0f, -0.0980171412229538f, 0.9951847195625305f, -0.9807852506637573f, -0.19509032368659973f, 0.290284663438797f, -0.9569403529167175f, 0.9238795042037964f, 0.3826834261417389f, -0.4713967442512512f, 0.8819212913513184f, -0.8314695954322815f, -0.5555702447891235f, 0.6343932747840881f, -0.7730104327201843f, 1.0f, -0.290284663438797f, 0.9569403529167175f, -0.8314695954322815f, -0.5555702447891235f, 0.7730104327201843f, -0.6343932747840881f, 0.3826834261417389f, 0.9238795042037964f, -0.9951847195625305f, 0.0980171412229538f, 0.19509032368659973f, -0.9807852506637573f, 0.8819212913513184f, 0.4713967442512512f, 1.0f, -0.4713967442512512f, 0.8819212913513184f, -0.5555702447891235f, -0.8314695954322815f, 0.9951847195625305f, -0.0980171412229538f, -0.3826834261417389f, 0.9238795042037964f, -0.6343932747840881f, -0.7730104327201843f, 0.9807852506637573f, -0.19509032368659973f, -0.290284663438797f, 0.9569403529167175f, 1.0f, -0.6343932747840881f, 0.7730104327201843f, -0.19509032368659973f, -0.9807852506637573f, 0.8819212913513184f, 0.4713967442512512f, -0.9238795042037964f, 0.3826834261417389f, 0.290284663438797f, -0.9569403529167175f, 0.5555702447891235f, 0.8314695954322815f, -0.9951847195625305f, -0.0980171412229538f, 1.0f, -0.7730104327201843f, 0.6343932747840881f, 0.19509032368659973f, -0.9807852506637573f, 0.4713967442512512f, 0.8819212913513184f, -0.9238795042037964f, -0.3826834261417389f, 0.9569403529167175f, -0.290284663438797f, -0.5555702447891235f, 0.8314695954322815f, -0.0980171412229538f, -0.9951847195625305f, 1.0f, -0.8819212913513184f, 0.4713967442512512f, 0.5555702447891235f, -0.8314695954322815f, -0.0980171412229538f, 0.9951847195625305f, -0.3826834261417389f, -0.9238795042037964f, 0.7730104327201843f, 0.6343932747840881f, -0.9807852506637573f, -0.19509032368659973f, 0.9569403529167175f, -0.290284663438797f, 1.0f, -0.9569403529167175f, 0.290284663438797f, 0.8314695954322815f, -0.5555702447891235f, -0.6343932747840881f, 0.7730104327201843f, 0.3826834261417389f, -0.9238795042037964f, -0.0980171412229538f, 0.9951847195625305f, -0.19509032368659973f, -0.9807852506637573f, 0.4713967442512512f, 0.8819212913513184f, 1.0f, -0.9951847195625305f, 0.0980171412229538f, 0.9807852506637573f, -0.19509032368659973f, -0.9569403529167175f, 0.290284663438797f, 0.9238795042037964f, -0.3826834261417389f, -0.8819212913513184f, 0.4713967442512512f, 0.8314695954322815f, -0.5555702447891235f, -0.7730104327201843f, 0.6343932747840881f, 1.0f, -0.9951847195625305f, -0.0980171412229538f, 0.9807852506637573f, 0.19509032368659973f, -0.9569403529167175f, -0.290284663438797f, 0.9238795042037964f, 0.3826834261417389f, -0.8819212913513184f, -0.4713967442512512f, 0.8314695954322815f, 0.5555702447891235f, -0.7730104327201843f, -0.6343932747840881f, 1.0f, -0.9569403529167175f, -0.290284663438797f, 0.8314695954322815f, 0.5555702447891235f, -0.6343932747840881f, -0.7730104327201843f, 0.3826834261417389f, 0.9238795042037964f, -0.0980171412229538f, -0.9951847195625305f, -0.19509032368659973f, 0.9807852506637573f, 0.4713967442512512f, -0.8819212913513184f, 1.0f, -0.8819212913513184f, -0.4713967442512512f, 0.5555702447891235f, 0.8314695954322815f, -0.0980171412229538f, -0.9951847195625305f, -0.3826834261417389f, 0.9238795042037964f, 0.7730104327201843f, -0.6343932747840881f, -0.9807852506637573f, 0.19509032368659973f, 0.9569403529167175f, 0.290284663438797f, 1.0f, -0.7730104327201843f, -0.6343932747840881f, 0.19509032368659973f, 0.9807852506637573f, 0.4713967442512512f, -0.8819212913513184f, -0.9238795042037964f, 0.3826834261417389f, 0.9569403529167175f, 0.290284663438797f, -0.5555702447891235f, -0.8314695954322815f, -0.0980171412229538f, 0.9951847195625305f, 1.0f, -0.6343932747840881f, -0.7730104327201843f, -0.19509032368659973f, 0.9807852506637573f, 0.8819212913513184f, -0.4713967442512512f, -0.9238795042037964f, -0.3826834261417389f, 0.290284663438797f, 0.9569403529167175f, 0.5555702447891235f, -0.8314695954322815f, -0.9951847195625305f, 0.0980171412229538f, 1.0f, -0.4713967442512512f, -0.8819212913513184f, -0.5555702447891235f, 0.8314695954322815f, 0.9951847195625305f, 0.0980171412229538f, -0.3826834261417389f, -0.9238795042037964f, -0.6343932747840881f, 0.7730104327201843f, 0.9807852506637573f, 0.19509032368659973f, -0.290284663438797f, -0.9569403529167175f, 1.0f, -0.290284663438797f, -0.9569403529167175f, -0.8314695954322815f, 0.5555702447891235f, 0.7730104327201843f, 0.6343932747840881f, 0.3826834261417389f, -0.9238795042037964f, -0.9951847195625305f, -0.0980171412229538f, 0.19509032368659973f, 0.9807852506637573f, 0.8819212913513184f, -0.4713967442512512f, 1.0f, -0.0980171412229538f, -0.9951847195625305f, -0.9807852506637573f, 0.19509032368659973f, 0.290284663438797f, 0.9569403529167175f, 0.9238795042037964f, -0.3826834261417389f, -0.4713967442512512f, -0.8819212913513184f, -0.8314695954322815f, 0.5555702447891235f, 0.6343932747840881f, 0.7730104327201843f, 1.0f, 0.0980171412229538f, -0.9951847195625305f, -0.9807852506637573f, -0.19509032368659973f, -0.290284663438797f, 0.9569403529167175f, 0.9238795042037964f, 0.3826834261417389f, 0.4713967442512512f, -0.8819212913513184f, -0.8314695954322815f, -0.5555702447891235f, -0.6343932747840881f, 0.7730104327201843f, 1.0f, 0.290284663438797f, -0.9569403529167175f, -0.8314695954322815f, -0.5555702447891235f, -0.7730104327201843f, 0.6343932747840881f, 0.3826834261417389f, 0.9238795042037964f, 0.9951847195625305f, -0.0980171412229538f, 0.19509032368659973f, -0.9807852506637573f, -0.8819212913513184f, -0.4713967442512512f, 1.0f, 0.4713967442512512f, -0.8819212913513184f, -0.5555702447891235f, -0.8314695954322815f, -0.9951847195625305f, 0.0980171412229538f, -0.3826834261417389f, 0.9238795042037964f, 0.6343932747840881f, 0.7730104327201843f, 0.9807852506637573f, -0.19509032368659973f, 0.290284663438797f, -0.9569403529167175f, 1.0f, 0.6343932747840881f, -0.7730104327201843f, -0.19509032368659973f, -0.9807852506637573f, -0.8819212913513184f, -0.4713967442512512f, -0.9238795042037964f, 0.3826834261417389f, -0.290284663438797f, 0.9569403529167175f, 0.5555702447891235f, 0.8314695954322815f, 0.9951847195625305f, 0.0980171412229538f, 1.0f, 0.7730104327201843f, -0.6343932747840881f, 0.19509032368659973f, -0.9807852506637573f, -0.4713967442512512f, -0.8819212913513184f, -0.9238795042037964f, -0.3826834261417389f, -0.9569403529167175f, 0.290284663438797f, -0.5555702447891235f, 0.8314695954322815f, 0.0980171412229538f, 0.9951847195625305f, 1.0f, 0.8819212913513184f, -0.4713967442512512f, 0.5555702447891235f, -0.8314695954322815f, 0.0980171412229538f, -0.9951847195625305f, -0.3826834261417389f, -0.9238795042037964f, -0.7730104327201843f, -0.6343932747840881f, -0.9807852506637573f, -0.19509032368659973f, -0.9569403529167175f, 0.290284663438797f, 1.0f, 0.9569403529167175f, -0.290284663438797f, 0.8314695954322815f, -0.5555702447891235f, 0.6343932747840881f, -0.7730104327201843f, 0.3826834261417389f, -0.9238795042037964f, 0.0980171412229538f, -0.9951847195625305f, -0.19509032368659973f, -0.9807852506637573f, -0.4713967442512512f, -0.8819212913513184f, 1.0f, 0.9951847195625305f, -0.0980171412229538f, 0.9807852506637573f, -0.19509032368659973f, 0.9569403529167175f, -0.290284663438797f, 0.9238795042037964f, -0.3826834261417389f, 0.8819212913513184f, -0.4713967442512512f, 0.8314695954322815f, -0.5555702447891235f, 0.7730104327201843f, -0.6343932747840881f};
-static __constant__ float kExpW8[16] = {0.00533137284219265f, 0.012223450466990471f, 0.018684329465031624f, 0.024470841512084007f, 0.029373103752732277f, 0.03321380540728569f, 0.035854097455739975f, 0.037198539823293686f, 0.037198539823293686f, 0.035854097455739975f, 0.03321380540728569f, 0.029373103752732277f, 0.024470841512084007f, 0.018684329465031624f, 0.012223450466990471f, 0.00533137284219265f};
+// lane-pair rules: product, then projected exponential (plain, weighted)
+static __device__ const float kLpLeg8[240] = {0.06520631164312363f, 0.13781440258026123f, 0.16102319955825806f, 0.15215513110160828f, 0.021588720381259918f, 0.07708820700645447f, 0.14019207656383514f, 0.19657686352729797f, 0.00461379811167717f, 0.022952022030949593f, 0.05559203401207924f, 0.0009525957866571844f, 0.006059064529836178f, 0.01822534203529358f, 0.00019313527445774525f, 0.0014945222064852715f, 3.87199324904941e-05f, 0.0003527893277350813f, 7.703575647610705e-06f, 1.5242303561535664e-06f, 0.11085808277130127f, 0.15386998653411865f, 0.16021457314491272f, 0.13757289946079254f, 0.04738370701670647f, 0.10864433646202087f, 0.1700213998556137f, 0.0f, 0.011981873773038387f, 0.03756134212017059f, 0.07660231739282608f, 0.0028050916735082865f, 0.011091789230704308f, 0.0f, 0.0006287457654252648f, 0.0029944006819278f, 0.0001370324462186545f, 0.0f, 2.9285665732459165e-05f, 0.0f, 0.08565717935562134f, 0.13908180594444275f, 0.05986662954092026f, -0.06713762134313583f, 0.0633930191397667f, 0.18306352198123932f, 0.21085374057292938f, 0.10451316833496094f, 0.03028402104973793f, 0.1238425225019455f, 0.21286974847316742f, 0.013976679183542728f, 0.07366860657930374f, 0.16529589891433716f, 0.00633428106084466f, 0.04081254079937935f, 0.0028386428020894527f, 0.021603398025035858f, 0.0012624345254153013f, 0.0005583513411693275f, 0.13413716852664948f, 0.11137636750936508f, -0.003983851056545973f, -0.11710293591022491f, 0.12815962731838226f, 0.21362611651420593f, 0.17273001372814178f, 0.0f, 0.0724414810538292f, 0.17446376383304596f, 0.22883576154708862f, 0.037909671664237976f, 0.11820931732654572f, 0.0f, 0.018994087353348732f, 0.07242981344461441f, 0.009253524243831635f, 0.0f, 0.004420579876750708f, 0.0f, 0.09798557311296463f, 0.08525826036930084f, -0.09131614118814468f, -0.11765225976705551f, 0.10830617696046829f, 0.19894984364509583f, 0.008022683672606945f, -0.19128155708312988f, 0.07727494835853577f, 0.2107543796300888f, 0.1254342496395111f, 0.053265079855918884f, 0.19144459068775177f, 0.19945865869522095f, 0.03605365753173828f, 0.16045929491519928f, 0.0241310466080904f, 0.12792740762233734f, 0.016028307378292084f, 0.010587655007839203f, 0.13066479563713074f, -0.003617573296651244f, -0.13627637922763824f, -0.04429611191153526f, 0.18645501136779785f, 0.13122136890888214f, -0.11810997873544693f, 0.0f, 0.15740682184696198f, 0.20314645767211914f, 0.0009861834114417434f, 0.1230267807841301f, 0.2253846824169159f, 0.0f, 0.09206223487854004f, 0.21661099791526794f, 0.06698594242334366f, 0.0f, 0.04779353365302086f, 0.0f, 0.10608874261379242f, 0.00413087522611022f, -0.1266615241765976f, 0.07696889340877533f, 0.14872010052204132f, 0.10081823915243149f, -0.18343278765678406f, 0.007615973707288504f, 0.1345750093460083f, 0.1648647040128708f, -0.14551927149295807f, 0.11764611303806305f, 0.20528586208820343f, -0.08582877367734909f, 0.10099354386329651f, 0.22752733528614044f, 0.08572938293218613f, 0.23614519834518433f, 0.07221883535385132f, 0.060502298176288605f, 0.1079203188419342f, -0.10511626303195953f, -0.04261922463774681f, 0.13283823430538177f, 0.1953115612268448f, -0.07001624256372452f, -0.14808103442192078f, 0.0f, 0.20911574363708496f, 0.012077328749001026f, -0.18980476260185242f, 0.2072870284318924f, 0.08569271862506866f, 0.0f, 0.19672666490077972f, 0.1459958702325821f, 0.18154096603393555f, 0.0f, 0.1642742156982422f, 0.0f, 0.11112427711486816f, -0.07381140440702438f, -0.01743069291114807f, 0.10047222673892975f, 0.1789790838956833f, -0.054160233587026596f, -0.08458041399717331f, 0.17426559329032898f, 0.1860758513212204f, -0.008524632081389427f, -0.13042566180229187f, 0.18689434230327606f, 0.033735811710357666f, -0.16413705050945282f, 0.18433387577533722f, 0.07256858795881271f, 0.17977702617645264f, 0.10785961151123047f, 0.17399948835372925f, 0.1674797534942627f, 0.07079759240150452f, -0.12563757598400116f, 0.11323718726634979f, -0.039617281407117844f, 0.14720962941646576f, -0.18506301939487457f, 0.12129383534193039f, 0.0f, 0.18108728528022766f, -0.17840780317783356f, 0.07581662386655807f, 0.20623688399791718f, -0.1622493416070938f, 0.0f, 0.22487977147102356f, -0.139549121260643f, 0.23842665553092957f, 0.0f, 0.24788059294223785f, 0.0f, 0.11355419456958771f, -0.12098407745361328f, 0.10807975381612778f, -0.08776627480983734f, 0.19513322412967682f, -0.16821692883968353f, 0.14210937917232513f, -0.10832967609167099f, 0.21644802391529083f, -0.16687056422233582f, 0.13246333599090576f, 0.23195002973079681f, -0.16517631709575653f, 0.12301430851221085f, 0.24408331513404846f, -0.1628371924161911f, 0.253981351852417f, -0.15985198318958282f, 0.2622710168361664f, 0.26933905482292175f, 0.024631112813949585f, -0.054961759597063065f, 0.0820532739162445f, -0.1040557399392128f, 0.054643236100673676f, -0.09671244770288467f, 0.13222384452819824f, 0.0f, 0.07171712070703506f, -0.11333373934030533f, 0.14613576233386993f, 0.087143674492836f, -0.12822918593883514f, 0.0f, 0.10138054937124252f, -0.14173586666584015f, 0.11468159407377243f, 0.0f, 0.12720850110054016f, 0.0f};
+static __device__ const float kLeLeg8[640] = {0.282094806432724f, 0.6108322739601135f, 0.7587076425552368f, 0.8024648427963257f, 0.07094971090555191f, 0.2584724724292755f, 0.48795923590660095f, 0.7245708703994751f, 0.011518623679876328f, 0.05838014557957649f, 0.14570735394954681f, 0.0018066286575049162f, 0.011699545197188854f, 0.0361325666308403f, 0.00027825316647067666f, 0.0021913156379014254f, 4.237711618770845e-05f, 0.000392841175198555f, 6.4048267631733324e-06f, 9.626843393562012e-07f, 0.48342376947402954f, 0.6995154619216919f, 0.7922953963279724f, 0.7908328771591187f, 0.15696685016155243f, 0.3703010082244873f, 0.6073318123817444f, 0.0f, 0.030152400955557823f, 0.09684120118618011f, 0.204736590385437f, 0.00536244036629796f, 0.02167833410203457f, 0.0f, 0.0009130798862315714f, 0.004440254531800747f, 0.00015117340080905706f, 0.0f, 2.454286914144177e-05f, 0.0f, 0.282094806432724f, 0.5288062691688538f, 0.4332386255264282f, 0.12681901454925537f, 0.16040606796741486f, 0.5193262100219727f, 0.7771311402320862f, 0.774089515209198f, 0.05887635797262192f, 0.26746249198913574f, 0.5564955472946167f, 0.020877545699477196f, 0.12169450521469116f, 0.32081058621406555f, 0.007269772235304117f, 0.051662128418684006f, 0.002503123367205262f, 0.020974058657884598f, 0.0008553196093998849f, 0.000290653231786564f, 0.461521714925766f, 0.5150310397148132f, 0.29784974455833435f, -0.05915773659944534f, 0.3387991189956665f, 0.6733590960502625f, 0.8136188983917236f, 0.0f, 0.14713852107524872f, 0.4091092348098755f, 0.691368579864502f, 0.0591612234711647f, 0.20980627834796906f, 0.0f, 0.022774748504161835f, 0.09791873395442963f, 0.008524921722710133f, 0.0f, 0.0031290357001125813f, 0.0f, 0.282094806432724f, 0.39359357953071594f, 0.018211757764220238f, -0.38138410449028015f, 0.24463455379009247f, 0.6285143494606018f, 0.5217272043228149f, -0.0579991415143013f, 0.13694144785404205f, 0.5034611225128174f, 0.6975259780883789f, 0.07405773550271988f, 0.3527039885520935f, 0.6644591093063354f, 0.03932863101363182f, 0.22964313626289368f, 0.020652245730161667f, 0.1427166610956192f, 0.010762432590126991f, 0.005577687174081802f, 0.42294958233833313f, 0.24117226898670197f, -0.21048904955387115f, -0.44790521264076233f, 0.47351714968681335f, 0.6510443687438965f, 0.26493629813194275f, 0.0f, 0.3136294484138489f, 0.6490544676780701f, 0.6177658438682556f, 0.1923200637102127f, 0.524702787399292f, 0.0f, 0.11291147023439407f, 0.3805752098560333f, 0.06445726007223129f, 0.0f, 0.036081865429878235f, 0.0f, 0.282094806432724f, 0.22452960908412933f, -0.2879684865474701f, -0.3008277714252472f, 0.3201611340045929f, 0.5549961924552917f, -0.044748563319444656f, -0.5584453344345093f, 0.2345505803823471f, 0.6082530617713928f, 0.29154467582702637f, 0.16600562632083893f, 0.5692598223686218f, 0.5239323973655701f, 0.11537507176399231f, 0.4908573031425476f, 0.07929050922393799f, 0.402326762676239f, 0.05407732352614403f, 0.03667834401130676f, 0.36909249424934387f, -0.04138867184519768f, -0.3913777768611908f, -0.06159166991710663f, 0.5407955646514893f, 0.32933056354522705f, -0.39608559012413025f, 0.0f, 0.4687756597995758f, 0.5534201264381409f, -0.08651652932167053f, 0.37620416283607483f, 0.6415792107582092f, 0.0f, 0.2890598773956299f, 0.6385716795921326f, 0.2159595489501953f, 0.0f, 0.1582123339176178f, 0.0f, 0.282094806432724f, 0.04583054408431053f, -0.35458382964134216f, 0.12894819676876068f, 0.384176105260849f, 0.32660973072052f, -0.4573071599006653f, -0.12329808622598648f, 0.3377225399017334f, 0.48913657665252686f, -0.30245769023895264f, 0.28681913018226624f, 0.57930988073349f, -0.10303568840026855f, 0.23919881880283356f, 0.6170144081115723f, 0.1972559243440628f, 0.6180117130279541f, 0.16143056750297546f, 0.13138386607170105f, 0.3018958866596222f, -0.25159263610839844f, -0.1836709827184677f, 0.34278231859207153f, 0.5307828187942505f, -0.10648290067911148f, -0.4651665985584259f, 0.0f, 0.5520908832550049f, 0.13303987681865692f, -0.5200333595275879f, 0.5316561460494995f, 0.331875741481781f, 0.0f, 0.49018144607543945f, 0.4811188876628876f, 0.4394436776638031f, 0.0f, 0.3863072693347931f, 0.0f, 0.282094806432724f, -0.1169036328792572f, -0.18545503914356232f, 0.33673009276390076f, 0.43434005975723267f, 0.01986619643867016f, -0.40778017044067383f, 0.44140905141830444f, 0.4316771626472473f, 0.1751290261745453f, -0.4818282127380371f, 0.4144829213619232f, 0.30518484115600586f, -0.5003358721733093f, 0.390802264213562f, 0.4119834005832672f, 0.3643574118614197f, 0.4975000023841858f, 0.3371187150478363f, 0.31019774079322815f, 0.22378814220428467f, -0.3334845304489136f, 0.1654045134782791f, 0.14211028814315796f, 0.4448322653770447f, -0.4171973168849945f, 0.03768457472324371f, 0.0f, 0.5231057405471802f, -0.3215390741825104f, -0.14276351034641266f, 0.5695204138755798f, -0.20522691309452057f, 0.0f, 0.5936559438705444f, -0.08099491894245148f, 0.6017009019851685f, 0.0f, 0.5980119705200195f, 0.0f, 0.282094806432724f, -0.2403593808412552f, 0.0889744758605957f, 0.09286528080701828f, 0.4688291847705841f, -0.264663428068161f, 0.009497372433543205f, 0.24327048659324646f, 0.502954363822937f, -0.1937839388847351f, -0.09324891865253448f, 0.521267831325531f, -0.12374024838209152f, -0.18446695804595947f, 0.5305131077766418f, -0.05461635813117027f, 0.5338895320892334f, 0.013045242987573147f, 0.5332015156745911f, 0.5295804738998413f, 0.13759219646453857f, -0.27359575033187866f, 0.3242362141609192f, -0.27236804366111755f, 0.29521456360816956f, -0.44199138879776f, 0.4452876150608063f, 0.0f, 0.37472763657569885f, -0.4735797047615051f, 0.41168612241744995f, 0.44037261605262756f, -0.4876188635826111f, 0.0f, 0.4954850971698761f, -0.4878280460834503f, 0.5420773029327393f, 0.0f, 0.5815340280532837f, 0.0f, 0.282094806432724f, -0.3068500757217407f, 0.2890093922615051f, -0.2592114210128784f, 0.4863921105861664f, -0.43444186449050903f, 0.394683301448822f, -0.34362509846687317f, 0.5413427948951721f, -0.4391913115978241f, 0.38350313901901245f, 0.582071840763092f, -0.44341665506362915f, 0.37287411093711853f, 0.6145874261856079f, -0.4462928771972656f, 0.6416686773300171f, -0.44775089621543884f, 0.6648485660552979f, 0.6850703358650208f, 0.046423349529504776f, -0.10476886481046677f, 0.15971150994300842f, -0.2089904397726059f, 0.1033361628651619f, -0.1858418732881546f, 0.2607538104057312f, 0.0f, 0.1360824704170227f, -0.21955569088459015f, 0.2920544147491455f, 0.16591231524944305f, -0.2504565119743347f, 0.0f, 0.19366930425167084f, -0.27913984656333923f, 0.21981802582740784f, 0.0f, 0.24465221166610718f, 0.0f, 0.0015039525460451841f, 0.0032565747387707233f, 0.0040449537336826324f, 0.004278239328414202f, 0.0003782593703363091f, 0.001378013170324266f, 0.0026014926843345165f, 0.0038629574701189995f, 6.141007906990126e-05f, 0.00031124631641432643f, 0.0007768202922306955f, 9.631811735744122e-06f, 6.237463821889833e-05f, 0.00019263618742115796f, 1.4834713510936126e-06f, 1.1682720469252672e-05f, 2.2592820414502057e-07f, 2.094382807626971e-06f, 3.4146520278000025e-08f, 5.132429592435983e-09f, 0.002577312523499131f, 0.0037293776404112577f, 0.004224022384732962f, 0.0042162248864769936f, 0.000836848805192858f, 0.0019742127042263746f, 0.0032379121985286474f, 0.0f, 0.00016075369785539806f, 0.000516296538989991f, 0.0010915271705016494f, 2.8589169232873246e-05f, 0.00011557528341654688f, 0.0f, 4.867969437327702e-06f, 2.367265369684901e-05f, 8.059617471189995e-07f, 0.0f, 1.3084718375466764e-07f, 0.0f, 0.0034481717739254236f, 0.006463837809860706f, 0.005295671056956053f, 0.0015501659363508224f, 0.0019607157446444035f, 0.006347957998514175f, 0.009499224834144115f, 0.009462045505642891f, 0.0007196722435764968f, 0.0032693147659301758f, 0.00680229626595974f, 0.0002551956567913294f, 0.001487526809796691f, 0.003921412397176027f, 8.886170689947903e-05f, 0.000631489499937743f, 3.059680602746084e-05f, 0.0002563753805588931f, 1.0454957191541325e-05f, 3.552785528881941e-06f, 0.005641388241201639f, 0.006295457016676664f, 0.0036407518200576305f, -0.0007231116760522127f, 0.004141294397413731f, 0.008230771869421005f, 0.009945230558514595f, 0.0f, 0.001798540586605668f, 0.005000726785510778f, 0.00845090951770544f, 0.0007231542840600014f, 0.0025645566638559103f, 0.0f, 0.00027838602545671165f, 0.001196904806420207f, 0.00010420395847177133f, 0.0f, 3.8247613701969385e-05f, 0.0f, 0.005270752124488354f, 0.007354032248258591f, 0.0003402744769118726f, -0.0071259066462516785f, 0.004570832941681147f, 0.01174336951225996f, 0.009748122654855251f, -0.0010836750734597445f, 0.0025586592964828014f, 0.009406833909451962f, 0.013032806105911732f, 0.0013837191509082913f, 0.006590037606656551f, 0.012414973229169846f, 0.0007348291110247374f, 0.004290727898478508f, 0.00038587336894124746f, 0.0026665651239454746f, 0.00020108884200453758f, 0.00010421535262139514f, 0.007902529090642929f, 0.004506142344325781f, -0.003932847175747156f, -0.008368808776140213f, 0.008847351185977459f, 0.012164327315986156f, 0.00495015736669302f, 0.0f, 0.00585995614528656f, 0.012127147056162357f, 0.011542540974915028f, 0.003593371482565999f, 0.009803719818592072f, 0.0f, 0.0021096752025187016f, 0.0071107931435108185f, 0.0012043407186865807f, 0.0f, 0.0006741654360666871f, 0.0f, 0.006903097033500671f, 0.0054944283328950405f, -0.007046831306070089f, -0.0073615084402263165f, 0.007834612391889095f, 0.013581224717199802f, -0.0010950349969789386f, -0.013665626756846905f, 0.005739650223404169f, 0.01488446444272995f, 0.007134343963116407f, 0.004062297288328409f, 0.013930266723036766f, 0.012821067124605179f, 0.0028233251068741083f, 0.012011690996587276f, 0.0019403055775910616f, 0.00984527450054884f, 0.0013233176432549953f, 0.0008975499076768756f, 0.009032003581523895f, -0.0010128156282007694f, -0.009577343240380287f, -0.0015072000678628683f, 0.013233722187578678f, 0.008058995939791203f, -0.009692547842860222f, 0.0f, 0.011471334844827652f, 0.013542655855417252f, -0.002117132069543004f, 0.009206032380461693f, 0.01569998264312744f, 0.0f, 0.007073538843542337f, 0.015626385807991028f, 0.005284711718559265f, 0.0f, 0.003871588734909892f, 0.0f, 0.008285999298095703f, 0.0013461853377521038f, -0.01041522715240717f, 0.0037876085843890905f, 0.011284444481134415f, 0.009593541733920574f, -0.01343253068625927f, -0.0036216473672538996f, 0.009919959120452404f, 0.01436745934188366f, -0.008884121663868427f, 0.008424768224358559f, 0.017016129568219185f, -0.0030264779925346375f, 0.00702601158991456f, 0.018123628571629524f, 0.005794018507003784f, 0.01815292239189148f, 0.004741716664284468f, 0.003859151853248477f, 0.008867619559168816f, -0.007390057202428579f, -0.00539498683065176f, 0.010068580508232117f, 0.01559073943644762f, -0.0031277332454919815f, -0.013663386926054955f, 0.0f, 0.016216622665524483f, 0.0039077941328287125f, -0.015274993143975735f, 0.015616391785442829f, 0.009748220443725586f, 0.0f, 0.014398150146007538f, 0.014131954871118069f, 0.012907824479043484f, 0.0f, 0.011347043327987194f, 0.0f, 0.00936944130808115f, -0.0038828144315630198f, -0.006159667391330004f, 0.011184087023139f, 0.014426086097955704f, 0.0006598319741897285f, -0.0135439308360219f, 0.01466087345033884f, 0.014337641187012196f, 0.005816700868308544f, -0.01600334793329239f, 0.013766555115580559f, 0.010136350058019161f, -0.01661805808544159f, 0.012980030849575996f, 0.013683537021279335f, 0.012101695872843266f, 0.01652386784553528f, 0.01119699515402317f, 0.010302847251296043f, 0.007432855665683746f, -0.011076290160417557f, 0.005493713077157736f, 0.004720023367553949f, 0.014774571172893047f, -0.013856709934771061f, 0.0012516481801867485f, 0.0f, 0.017374331131577492f, -0.010679536499083042f, -0.0047417194582521915f, 0.018915940076112747f, -0.00681636668741703f, 0.0f, 0.019717572256922722f, -0.002690149238333106f, 0.0199847761541605f, 0.0f, 0.019862251356244087f, 0.0f, 0.010114253498613834f, -0.008617868646979332f, 0.0031900994945317507f, 0.0033296009059995413f, 0.01680944673717022f, -0.009489268064498901f, 0.0003405197348911315f, 0.008722243830561638f, 0.018032973632216454f, -0.006947948131710291f, -0.0033433556091040373f, 0.018689587712287903f, -0.004436594899743795f, -0.006613896228373051f, 0.019021067768335342f, -0.0019582202658057213f, 0.01914212666451931f, 0.0004677253891713917f, 0.019117459654808044f, 0.0189876276999712f, 0.0049332440830767155f, -0.009809528477489948f, 0.011625195853412151f, -0.009765510447323322f, 0.010584651492536068f, -0.015847202390432358f, 0.015965385362505913f, 0.0f, 0.01343552116304636f, -0.016979772597551346f, 0.014760633930563927f, 0.01578916236758232f, -0.01748313382267952f, 0.0f, 0.017765169963240623f, -0.017490632832050323f, 0.019435690715909004f, 0.0f, 0.020850377157330513f, 0.0f, 0.010493514128029346f, -0.01141437515616417f, 0.010750727728009224f, -0.009642287157475948f, 0.018093077465891838f, -0.01616060361266136f, 0.01468164287507534f, -0.012782352045178413f, 0.020137161016464233f, -0.016337275505065918f, 0.0142657570540905f, 0.0216522216796875f, -0.016494451090693474f, 0.01387037243694067f, 0.022861754521727562f, -0.01660144329071045f, 0.023869138211011887f, -0.016655679792165756f, 0.02473139576613903f, 0.025483615696430206f, 0.0017268809024244547f, -0.003897249000146985f, 0.005941035225987434f, -0.007774139288812876f, 0.003843954298645258f, -0.0069130463525652885f, 0.00969966035336256f, 0.0f, 0.0050620692782104015f, -0.008167151361703873f, 0.010863997973501682f, 0.00617169588804245f, -0.00931661669164896f, 0.0f, 0.007204215507954359f, -0.010383594781160355f, 0.008176909759640694f, 0.0f, 0.00910070538520813f, 0.0f};
+static __constant__ float kLpTrig8[90] = {1.0f, 0.9914448857307434f, 0.13052618503570557f, 0.9659258127212524f, 0.258819043636322f, 0.9238795042037964f, 0.3826834261417389f, 0.8660253882408142f, 0.5f, 0.7933533191680908f, 0.6087614297866821f, 0.7071067690849304f, 0.7071067690849304f, 0.6087614297866821f, 0.7933533191680908f, 1.0f, 0.9238795042037964f, 0.3826834261417389f, 0.7071067690849304f, 0.7071067690849304f, 0.3826834261417389f, 0.9238795042037964f, 6.123234262925839e-17f, 1.0f, -0.3826834261417389f, 0.9238795042037964f, -0.7071067690849304f, 0.7071067690849304f, -0.9238795042037964f, 0.3826834261417389f, 1.0f, 0.7933533191680908f, 0.6087614297866821f, 0.258819043636322f, 0.9659258127212524f, -0.3826834261417389f, 0.9238795042037964f, -0.8660253882408142f, 0.5f, -0.9914448857307434f, -0.13052618503570557f, -0.7071067690849304f, -0.7071067690849304f, -0.13052618503570557f, -0.9914448857307434f, 1.0f, 0.6087614297866821f, 0.7933533191680908f, -0.258819043636322f, 0.9659258127212524f, -0.9238795042037964f, 0.3826834261417389f, -0.8660253882408142f, -0.5f, -0.13052618503570557f, -0.9914448857307434f, 0.7071067690849304f, -0.7071067690849304f, 0.9914448857307434f, 0.13052618503570557f, 1.0f, 0.3826834261417389f, 0.9238795042037964f, -0.7071067690849304f, 0.7071067690849304f, -0.9238795042037964f, -0.3826834261417389f, -1.8369701465288538e-16f, -1.0f, 0.9238795042037964f, -0.3826834261417389f, 0.7071067690849304f, 0.7071067690849304f, -0.3826834261417389f, 0.9238795042037964f, 1.0f, 0.13052618503570557f, 0.9914448857307434f, -0.9659258127212524f, 0.258819043636322f, -0.3826834261417389f, -0.9238795042037964f, 0.8660253882408142f, -0.5f, 0.6087614297866821f, 0.7933533191680908f, -0.7071067690849304f, 0.7071067690849304f, -0.7933533191680908f, -0.6087614297866821f};
 #endif
 template <> struct SH<8> {
     static constexpr int K = 64;
     static constexpr int NNZ_SYM = 6588;   // entries (i, j <= k)
     static constexpr int EZ = 16;    // projected-exponential rule: Gauss-Legendre nodes
     static constexpr int EP = 32;    // projected-exponential rule: uniform azimuths
-#if defined(SHS_NB) && SHS_NB == 8
-    __device__ __forceinline__ static const float* eleg() { return kExpLeg8; }
-    __device__ __forceinline__ static const float* etrig() { return kExpTrig8; }
-    __device__ __forceinline__ static const float* ew() { return kExpW8; }
-#endif
     __device__ __forceinline__ static float norm(int i) {
         switch (i) {
             case 0: return 0.282094806432724f;
@@ -4065,865 +3252,221 @@ template <> struct SH<8> {
         gy = w[1] + t78 * a_t166 + t74 * a_t154 + t70 * a_t144 + t66 * a_t136 + t62 * a_t130 + t59 * a_t126 + t26 * a_t34 + t29 * a_t31 + t20 * a_t28 + t23 * a_t25 + t14 * a_t22 + t17 * a_t19 + t8 * a_t16 + t11 * a_t13 + t2 * a_t10 + t5 * a_t7 + x * a_t4 + x * a_t3 + y * a_t1 + y * a_t1;
         gz = w[2] + 10395.0f * a_t123 + t119 * a_t120 + 945.0f * a_t118 + t113 * a_t114 + t110 * a_t111 + 105.0f * a_t109 + t104 * a_t105 + t100 * a_t101 + t97 * a_t98 + 15.0f * a_t96 + t91 * a_t92 + t87 * a_t88 + t83 * a_t84 + t80 * a_t81 + 3.0f * a_t79 + t74 * a_t75 + t70 * a_t71 + t66 * a_t67 + t62 * a_t63 + t59 * a_t60 + 3.0f * a_t59 + t54 * a_t55 + t50 * a_t51 + t46 * a_t47 + t42 * a_t43 + 0.6666666865348816f * a_t41 + t38 * a_t39 + z * a_t36 + z * a_t36;
     }
-    static constexpr int NA = 120;   // monomials of degree < n
-    static constexpr int NG = 252;   // gradient coefficients, bands >= 1
-    __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
-        (void)x; (void)y; (void)z;
-        const float m1_0_0 = x;
-        const float m0_1_0 = y;
-        const float m0_0_1 = z;
-        const float m2_0_0 = x * m1_0_0;
-        const float m1_1_0 = x * m0_1_0;
-        const float m1_0_1 = x * m0_0_1;
-        const float m0_2_0 = y * m0_1_0;
-        const float m0_1_1 = y * m0_0_1;
-        const float m0_0_2 = z * m0_0_1;
-        const float m3_0_0 = x * m2_0_0;
-        const float m2_1_0 = x * m1_1_0;
-        const float m2_0_1 = x * m1_0_1;
-        const float m1_2_0 = x * m0_2_0;
-        const float m1_1_1 = x * m0_1_1;
-        const float m1_0_2 = x * m0_0_2;
-        const float m0_3_0 = y * m0_2_0;
-        const float m0_2_1 = y * m0_1_1;
-        const float m0_1_2 = y * m0_0_2;
-        const float m0_0_3 = z * m0_0_2;
-        const float m4_0_0 = x * m3_0_0;
-        const float m3_1_0 = x * m2_1_0;
-        const float m3_0_1 = x * m2_0_1;
-        const float m2_2_0 = x * m1_2_0;
-        const float m2_1_1 = x * m1_1_1;
-        const float m2_0_2 = x * m1_0_2;
-        const float m1_3_0 = x * m0_3_0;
-        const float m1_2_1 = x * m0_2_1;
-        const float m1_1_2 = x * m0_1_2;
-        const float m1_0_3 = x * m0_0_3;
-        const float m0_4_0 = y * m0_3_0;
-        const float m0_3_1 = y * m0_2_1;
-        const float m0_2_2 = y * m0_1_2;
-        const float m0_1_3 = y * m0_0_3;
-        const float m0_0_4 = z * m0_0_3;
-        const float m5_0_0 = x * m4_0_0;
-        const float m4_1_0 = x * m3_1_0;
-        const float m4_0_1 = x * m3_0_1;
-        const float m3_2_0 = x * m2_2_0;
-        const float m3_1_1 = x * m2_1_1;
-        const float m3_0_2 = x * m2_0_2;
-        const float m2_3_0 = x * m1_3_0;
-        const float m2_2_1 = x * m1_2_1;
-        const float m2_1_2 = x * m1_1_2;
-        const float m2_0_3 = x * m1_0_3;
-        const float m1_4_0 = x * m0_4_0;
-        const float m1_3_1 = x * m0_3_1;
-        const float m1_2_2 = x * m0_2_2;
-        const float m1_1_3 = x * m0_1_3;
-        const float m1_0_4 = x * m0_0_4;
-        const float m0_5_0 = y * m0_4_0;
-        const float m0_4_1 = y * m0_3_1;
-        const float m0_3_2 = y * m0_2_2;
-        const float m0_2_3 = y * m0_1_3;
-        const float m0_1_4 = y * m0_0_4;
-        const float m0_0_5 = z * m0_0_4;
-        const float m6_0_0 = x * m5_0_0;
-        const float m5_1_0 = x * m4_1_0;
-        const float m5_0_1 = x * m4_0_1;
-        const float m4_2_0 = x * m3_2_0;
-        const float m4_1_1 = x * m3_1_1;
-        const float m4_0_2 = x * m3_0_2;
-        const float m3_3_0 = x * m2_3_0;
-        const float m3_2_1 = x * m2_2_1;
-        const float m3_1_2 = x * m2_1_2;
-        const float m3_0_3 = x * m2_0_3;
-        const float m2_4_0 = x * m1_4_0;
-        const float m2_3_1 = x * m1_3_1;
-        const float m2_2_2 = x * m1_2_2;
-        const float m2_1_3 = x * m1_1_3;
-        const float m2_0_4 = x * m1_0_4;
-        const float m1_5_0 = x * m0_5_0;
-        const float m1_4_1 = x * m0_4_1;
-        const float m1_3_2 = x * m0_3_2;
-        const float m1_2_3 = x * m0_2_3;
-        const float m1_1_4 = x * m0_1_4;
-        const float m1_0_5 = x * m0_0_5;
-        const float m0_6_0 = y * m0_5_0;
-        const float m0_5_1 = y * m0_4_1;
-        const float m0_4_2 = y * m0_3_2;
-        const float m0_3_3 = y * m0_2_3;
-        const float m0_2_4 = y * m0_1_4;
-        const float m0_1_5 = y * m0_0_5;
-        const float m0_0_6 = z * m0_0_5;
-        const float gtx = G[7] * x;
-        const float gty = G[7] * y;
-        const float gtz = G[7] * z;
-        acc[0] = fmaf(G[0], 1.0f, acc[0]);
-        acc[1] = fmaf(G[1], m1_0_0, acc[1]);
-        acc[2] = fmaf(G[1], m0_1_0, acc[2]);
-        acc[3] = fmaf(G[1], m0_0_1, acc[3]);
-        acc[4] = fmaf(G[2], m2_0_0, acc[4]);
-        acc[5] = fmaf(G[2], m1_1_0, acc[5]);
-        acc[6] = fmaf(G[2], m1_0_1, acc[6]);
-        acc[7] = fmaf(G[2], m0_2_0, acc[7]);
-        acc[8] = fmaf(G[2], m0_1_1, acc[8]);
-        acc[9] = fmaf(G[2], m0_0_2, acc[9]);
-        acc[10] = fmaf(G[3], m3_0_0, acc[10]);
-        acc[11] = fmaf(G[3], m2_1_0, acc[11]);
-        acc[12] = fmaf(G[3], m2_0_1, acc[12]);
-        acc[13] = fmaf(G[3], m1_2_0, acc[13]);
-        acc[14] = fmaf(G[3], m1_1_1, acc[14]);
-        acc[15] = fmaf(G[3], m1_0_2, acc[15]);
-        acc[16] = fmaf(G[3], m0_3_0, acc[16]);
-        acc[17] = fmaf(G[3], m0_2_1, acc[17]);
-        acc[18] = fmaf(G[3], m0_1_2, acc[18]);
-        acc[19] = fmaf(G[3], m0_0_3, acc[19]);
-        acc[20] = fmaf(G[4], m4_0_0, acc[20]);
-        acc[21] = fmaf(G[4], m3_1_0, acc[21]);
-        acc[22] = fmaf(G[4], m3_0_1, acc[22]);
-        acc[23] = fmaf(G[4], m2_2_0, acc[23]);
-        acc[24] = fmaf(G[4], m2_1_1, acc[24]);
-        acc[25] = fmaf(G[4], m2_0_2, acc[25]);
-        acc[26] = fmaf(G[4], m1_3_0, acc[26]);
-        acc[27] = fmaf(G[4], m1_2_1, acc[27]);
-        acc[28] = fmaf(G[4], m1_1_2, acc[28]);
-        acc[29] = fmaf(G[4], m1_0_3, acc[29]);
-        acc[30] = fmaf(G[4], m0_4_0, acc[30]);
-        acc[31] = fmaf(G[4], m0_3_1, acc[31]);
-        acc[32] = fmaf(G[4], m0_2_2, acc[32]);
-        acc[33] = fmaf(G[4], m0_1_3, acc[33]);
-        acc[34] = fmaf(G[4], m0_0_4, acc[34]);
-        acc[35] = fmaf(G[5], m5_0_0, acc[35]);
-        acc[36] = fmaf(G[5], m4_1_0, acc[36]);
-        acc[37] = fmaf(G[5], m4_0_1, acc[37]);
-        acc[38] = fmaf(G[5], m3_2_0, acc[38]);
-        acc[39] = fmaf(G[5], m3_1_1, acc[39]);
-        acc[40] = fmaf(G[5], m3_0_2, acc[40]);
-        acc[41] = fmaf(G[5], m2_3_0, acc[41]);
-        acc[42] = fmaf(G[5], m2_2_1, acc[42]);
-        acc[43] = fmaf(G[5], m2_1_2, acc[43]);
-        acc[44] = fmaf(G[5], m2_0_3, acc[44]);
-        acc[45] = fmaf(G[5], m1_4_0, acc[45]);
-        acc[46] = fmaf(G[5], m1_3_1, acc[46]);
-        acc[47] = fmaf(G[5], m1_2_2, acc[47]);
-        acc[48] = fmaf(G[5], m1_1_3, acc[48]);
-        acc[49] = fmaf(G[5], m1_0_4, acc[49]);
-        acc[50] = fmaf(G[5], m0_5_0, acc[50]);
-        acc[51] = fmaf(G[5], m0_4_1, acc[51]);
-        acc[52] = fmaf(G[5], m0_3_2, acc[52]);
-        acc[53] = fmaf(G[5], m0_2_3, acc[53]);
-        acc[54] = fmaf(G[5], m0_1_4, acc[54]);
-        acc[55] = fmaf(G[5], m0_0_5, acc[55]);
-        acc[56] = fmaf(G[6], m6_0_0, acc[56]);
-        acc[57] = fmaf(G[6], m5_1_0, acc[57]);
-        acc[58] = fmaf(G[6], m5_0_1, acc[58]);
-        acc[59] = fmaf(G[6], m4_2_0, acc[59]);
-        acc[60] = fmaf(G[6], m4_1_1, acc[60]);
-        acc[61] = fmaf(G[6], m4_0_2, acc[61]);
-        acc[62] = fmaf(G[6], m3_3_0, acc[62]);
-        acc[63] = fmaf(G[6], m3_2_1, acc[63]);
-        acc[64] = fmaf(G[6], m3_1_2, acc[64]);
-        acc[65] = fmaf(G[6], m3_0_3, acc[65]);
-        acc[66] = fmaf(G[6], m2_4_0, acc[66]);
-        acc[67] = fmaf(G[6], m2_3_1, acc[67]);
-        acc[68] = fmaf(G[6], m2_2_2, acc[68]);
-        acc[69] = fmaf(G[6], m2_1_3, acc[69]);
-        acc[70] = fmaf(G[6], m2_0_4, acc[70]);
-        acc[71] = fmaf(G[6], m1_5_0, acc[71]);
-        acc[72] = fmaf(G[6], m1_4_1, acc[72]);
-        acc[73] = fmaf(G[6], m1_3_2, acc[73]);
-        acc[74] = fmaf(G[6], m1_2_3, acc[74]);
-        acc[75] = fmaf(G[6], m1_1_4, acc[75]);
-        acc[76] = fmaf(G[6], m1_0_5, acc[76]);
-        acc[77] = fmaf(G[6], m0_6_0, acc[77]);
-        acc[78] = fmaf(G[6], m0_5_1, acc[78]);
-        acc[79] = fmaf(G[6], m0_4_2, acc[79]);
-        acc[80] = fmaf(G[6], m0_3_3, acc[80]);
-        acc[81] = fmaf(G[6], m0_2_4, acc[81]);
-        acc[82] = fmaf(G[6], m0_1_5, acc[82]);
-        acc[83] = fmaf(G[6], m0_0_6, acc[83]);
-        acc[84] = fmaf(gtx, m6_0_0, acc[84]);
-        acc[85] = fmaf(gtx, m5_1_0, acc[85]);
-        acc[86] = fmaf(gtx, m5_0_1, acc[86]);
-        acc[87] = fmaf(gtx, m4_2_0, acc[87]);
-        acc[88] = fmaf(gtx, m4_1_1, acc[88]);
-        acc[89] = fmaf(gtx, m4_0_2, acc[89]);
-        acc[90] = fmaf(gtx, m3_3_0, acc[90]);
-        acc[91] = fmaf(gtx, m3_2_1, acc[91]);
-        acc[92] = fmaf(gtx, m3_1_2, acc[92]);
-        acc[93] = fmaf(gtx, m3_0_3, acc[93]);
-        acc[94] = fmaf(gtx, m2_4_0, acc[94]);
-        acc[95] = fmaf(gtx, m2_3_1, acc[95]);
-        acc[96] = fmaf(gtx, m2_2_2, acc[96]);
-        acc[97] = fmaf(gtx, m2_1_3, acc[97]);
-        acc[98] = fmaf(gtx, m2_0_4, acc[98]);
-        acc[99] = fmaf(gtx, m1_5_0, acc[99]);
-        acc[100] = fmaf(gtx, m1_4_1, acc[100]);
-        acc[101] = fmaf(gtx, m1_3_2, acc[101]);
-        acc[102] = fmaf(gtx, m1_2_3, acc[102]);
-        acc[103] = fmaf(gtx, m1_1_4, acc[103]);
-        acc[104] = fmaf(gtx, m1_0_5, acc[104]);
-        acc[105] = fmaf(gtx, m0_6_0, acc[105]);
-        acc[106] = fmaf(gtx, m0_5_1, acc[106]);
-        acc[107] = fmaf(gtx, m0_4_2, acc[107]);
-        acc[108] = fmaf(gtx, m0_3_3, acc[108]);
-        acc[109] = fmaf(gtx, m0_2_4, acc[109]);
-        acc[110] = fmaf(gtx, m0_1_5, acc[110]);
-        acc[111] = fmaf(gtx, m0_0_6, acc[111]);
-        acc[112] = fmaf(gty, m0_6_0, acc[112]);
-        acc[113] = fmaf(gty, m0_5_1, acc[113]);
-        acc[114] = fmaf(gty, m0_4_2, acc[114]);
-        acc[115] = fmaf(gty, m0_3_3, acc[115]);
-        acc[116] = fmaf(gty, m0_2_4, acc[116]);
-        acc[117] = fmaf(gty, m0_1_5, acc[117]);
-        acc[118] = fmaf(gty, m0_0_6, acc[118]);
-        acc[119] = fmaf(gtz, m0_0_6, acc[119]);
-    }
-    // the same for two pairs at once, one per half of each float2
-    __device__ __forceinline__ static void accumulate2(const float2* G, float2 x, float2 y, float2 z,
-                                                       float2* acc) {
-        (void)x; (void)y; (void)z;
-        const float2 m1_0_0 = x;
-        const float2 m0_1_0 = y;
-        const float2 m0_0_1 = z;
-        const float2 m2_0_0 = __fmul2_rn(x, m1_0_0);
-        const float2 m1_1_0 = __fmul2_rn(x, m0_1_0);
-        const float2 m1_0_1 = __fmul2_rn(x, m0_0_1);
-        const float2 m0_2_0 = __fmul2_rn(y, m0_1_0);
-        const float2 m0_1_1 = __fmul2_rn(y, m0_0_1);
-        const float2 m0_0_2 = __fmul2_rn(z, m0_0_1);
-        const float2 m3_0_0 = __fmul2_rn(x, m2_0_0);
-        const float2 m2_1_0 = __fmul2_rn(x, m1_1_0);
-        const float2 m2_0_1 = __fmul2_rn(x, m1_0_1);
-        const float2 m1_2_0 = __fmul2_rn(x, m0_2_0);
-        const float2 m1_1_1 = __fmul2_rn(x, m0_1_1);
-        const float2 m1_0_2 = __fmul2_rn(x, m0_0_2);
-        const float2 m0_3_0 = __fmul2_rn(y, m0_2_0);
-        const float2 m0_2_1 = __fmul2_rn(y, m0_1_1);
-        const float2 m0_1_2 = __fmul2_rn(y, m0_0_2);
-        const float2 m0_0_3 = __fmul2_rn(z, m0_0_2);
-        const float2 m4_0_0 = __fmul2_rn(x, m3_0_0);
-        const float2 m3_1_0 = __fmul2_rn(x, m2_1_0);
-        const float2 m3_0_1 = __fmul2_rn(x, m2_0_1);
-        const float2 m2_2_0 = __fmul2_rn(x, m1_2_0);
-        const float2 m2_1_1 = __fmul2_rn(x, m1_1_1);
-        const float2 m2_0_2 = __fmul2_rn(x, m1_0_2);
-        const float2 m1_3_0 = __fmul2_rn(x, m0_3_0);
-        const float2 m1_2_1 = __fmul2_rn(x, m0_2_1);
-        const float2 m1_1_2 = __fmul2_rn(x, m0_1_2);
-        const float2 m1_0_3 = __fmul2_rn(x, m0_0_3);
-        const float2 m0_4_0 = __fmul2_rn(y, m0_3_0);
-        const float2 m0_3_1 = __fmul2_rn(y, m0_2_1);
-        const float2 m0_2_2 = __fmul2_rn(y, m0_1_2);
-        const float2 m0_1_3 = __fmul2_rn(y, m0_0_3);
-        const float2 m0_0_4 = __fmul2_rn(z, m0_0_3);
-        const float2 m5_0_0 = __fmul2_rn(x, m4_0_0);
-        const float2 m4_1_0 = __fmul2_rn(x, m3_1_0);
-        const float2 m4_0_1 = __fmul2_rn(x, m3_0_1);
-        const float2 m3_2_0 = __fmul2_rn(x, m2_2_0);
-        const float2 m3_1_1 = __fmul2_rn(x, m2_1_1);
-        const float2 m3_0_2 = __fmul2_rn(x, m2_0_2);
-        const float2 m2_3_0 = __fmul2_rn(x, m1_3_0);
-        const float2 m2_2_1 = __fmul2_rn(x, m1_2_1);
-        const float2 m2_1_2 = __fmul2_rn(x, m1_1_2);
-        const float2 m2_0_3 = __fmul2_rn(x, m1_0_3);
-        const float2 m1_4_0 = __fmul2_rn(x, m0_4_0);
-        const float2 m1_3_1 = __fmul2_rn(x, m0_3_1);
-        const float2 m1_2_2 = __fmul2_rn(x, m0_2_2);
-        const float2 m1_1_3 = __fmul2_rn(x, m0_1_3);
-        const float2 m1_0_4 = __fmul2_rn(x, m0_0_4);
-        const float2 m0_5_0 = __fmul2_rn(y, m0_4_0);
-        const float2 m0_4_1 = __fmul2_rn(y, m0_3_1);
-        const float2 m0_3_2 = __fmul2_rn(y, m0_2_2);
-        const float2 m0_2_3 = __fmul2_rn(y, m0_1_3);
-        const float2 m0_1_4 = __fmul2_rn(y, m0_0_4);
-        const float2 m0_0_5 = __fmul2_rn(z, m0_0_4);
-        const float2 m6_0_0 = __fmul2_rn(x, m5_0_0);
-        const float2 m5_1_0 = __fmul2_rn(x, m4_1_0);
-        const float2 m5_0_1 = __fmul2_rn(x, m4_0_1);
-        const float2 m4_2_0 = __fmul2_rn(x, m3_2_0);
-        const float2 m4_1_1 = __fmul2_rn(x, m3_1_1);
-        const float2 m4_0_2 = __fmul2_rn(x, m3_0_2);
-        const float2 m3_3_0 = __fmul2_rn(x, m2_3_0);
-        const float2 m3_2_1 = __fmul2_rn(x, m2_2_1);
-        const float2 m3_1_2 = __fmul2_rn(x, m2_1_2);
-        const float2 m3_0_3 = __fmul2_rn(x, m2_0_3);
-        const float2 m2_4_0 = __fmul2_rn(x, m1_4_0);
-        const float2 m2_3_1 = __fmul2_rn(x, m1_3_1);
-        const float2 m2_2_2 = __fmul2_rn(x, m1_2_2);
-        const float2 m2_1_3 = __fmul2_rn(x, m1_1_3);
-        const float2 m2_0_4 = __fmul2_rn(x, m1_0_4);
-        const float2 m1_5_0 = __fmul2_rn(x, m0_5_0);
-        const float2 m1_4_1 = __fmul2_rn(x, m0_4_1);
-        const float2 m1_3_2 = __fmul2_rn(x, m0_3_2);
-        const float2 m1_2_3 = __fmul2_rn(x, m0_2_3);
-        const float2 m1_1_4 = __fmul2_rn(x, m0_1_4);
-        const float2 m1_0_5 = __fmul2_rn(x, m0_0_5);
-        const float2 m0_6_0 = __fmul2_rn(y, m0_5_0);
-        const float2 m0_5_1 = __fmul2_rn(y, m0_4_1);
-        const float2 m0_4_2 = __fmul2_rn(y, m0_3_2);
-        const float2 m0_3_3 = __fmul2_rn(y, m0_2_3);
-        const float2 m0_2_4 = __fmul2_rn(y, m0_1_4);
-        const float2 m0_1_5 = __fmul2_rn(y, m0_0_5);
-        const float2 m0_0_6 = __fmul2_rn(z, m0_0_5);
-        const float2 gtx = __fmul2_rn(G[7], x);
-        const float2 gty = __fmul2_rn(G[7], y);
-        const float2 gtz = __fmul2_rn(G[7], z);
-        acc[0] = __fadd2_rn(G[0], acc[0]);
-        acc[1] = __ffma2_rn(G[1], m1_0_0, acc[1]);
-        acc[2] = __ffma2_rn(G[1], m0_1_0, acc[2]);
-        acc[3] = __ffma2_rn(G[1], m0_0_1, acc[3]);
-        acc[4] = __ffma2_rn(G[2], m2_0_0, acc[4]);
-        acc[5] = __ffma2_rn(G[2], m1_1_0, acc[5]);
-        acc[6] = __ffma2_rn(G[2], m1_0_1, acc[6]);
-        acc[7] = __ffma2_rn(G[2], m0_2_0, acc[7]);
-        acc[8] = __ffma2_rn(G[2], m0_1_1, acc[8]);
-        acc[9] = __ffma2_rn(G[2], m0_0_2, acc[9]);
-        acc[10] = __ffma2_rn(G[3], m3_0_0, acc[10]);
-        acc[11] = __ffma2_rn(G[3], m2_1_0, acc[11]);
-        acc[12] = __ffma2_rn(G[3], m2_0_1, acc[12]);
-        acc[13] = __ffma2_rn(G[3], m1_2_0, acc[13]);
-        acc[14] = __ffma2_rn(G[3], m1_1_1, acc[14]);
-        acc[15] = __ffma2_rn(G[3], m1_0_2, acc[15]);
-        acc[16] = __ffma2_rn(G[3], m0_3_0, acc[16]);
-        acc[17] = __ffma2_rn(G[3], m0_2_1, acc[17]);
-        acc[18] = __ffma2_rn(G[3], m0_1_2, acc[18]);
-        acc[19] = __ffma2_rn(G[3], m0_0_3, acc[19]);
-        acc[20] = __ffma2_rn(G[4], m4_0_0, acc[20]);
-        acc[21] = __ffma2_rn(G[4], m3_1_0, acc[21]);
-        acc[22] = __ffma2_rn(G[4], m3_0_1, acc[22]);
-        acc[23] = __ffma2_rn(G[4], m2_2_0, acc[23]);
-        acc[24] = __ffma2_rn(G[4], m2_1_1, acc[24]);
-        acc[25] = __ffma2_rn(G[4], m2_0_2, acc[25]);
-        acc[26] = __ffma2_rn(G[4], m1_3_0, acc[26]);
-        acc[27] = __ffma2_rn(G[4], m1_2_1, acc[27]);
-        acc[28] = __ffma2_rn(G[4], m1_1_2, acc[28]);
-        acc[29] = __ffma2_rn(G[4], m1_0_3, acc[29]);
-        acc[30] = __ffma2_rn(G[4], m0_4_0, acc[30]);
-        acc[31] = __ffma2_rn(G[4], m0_3_1, acc[31]);
-        acc[32] = __ffma2_rn(G[4], m0_2_2, acc[32]);
-        acc[33] = __ffma2_rn(G[4], m0_1_3, acc[33]);
-        acc[34] = __ffma2_rn(G[4], m0_0_4, acc[34]);
-        acc[35] = __ffma2_rn(G[5], m5_0_0, acc[35]);
-        acc[36] = __ffma2_rn(G[5], m4_1_0, acc[36]);
-        acc[37] = __ffma2_rn(G[5], m4_0_1, acc[37]);
-        acc[38] = __ffma2_rn(G[5], m3_2_0, acc[38]);
-        acc[39] = __ffma2_rn(G[5], m3_1_1, acc[39]);
-        acc[40] = __ffma2_rn(G[5], m3_0_2, acc[40]);
-        acc[41] = __ffma2_rn(G[5], m2_3_0, acc[41]);
-        acc[42] = __ffma2_rn(G[5], m2_2_1, acc[42]);
-        acc[43] = __ffma2_rn(G[5], m2_1_2, acc[43]);
-        acc[44] = __ffma2_rn(G[5], m2_0_3, acc[44]);
-        acc[45] = __ffma2_rn(G[5], m1_4_0, acc[45]);
-        acc[46] = __ffma2_rn(G[5], m1_3_1, acc[46]);
-        acc[47] = __ffma2_rn(G[5], m1_2_2, acc[47]);
-        acc[48] = __ffma2_rn(G[5], m1_1_3, acc[48]);
-        acc[49] = __ffma2_rn(G[5], m1_0_4, acc[49]);
-        acc[50] = __ffma2_rn(G[5], m0_5_0, acc[50]);
-        acc[51] = __ffma2_rn(G[5], m0_4_1, acc[51]);
-        acc[52] = __ffma2_rn(G[5], m0_3_2, acc[52]);
-        acc[53] = __ffma2_rn(G[5], m0_2_3, acc[53]);
-        acc[54] = __ffma2_rn(G[5], m0_1_4, acc[54]);
-        acc[55] = __ffma2_rn(G[5], m0_0_5, acc[55]);
-        acc[56] = __ffma2_rn(G[6], m6_0_0, acc[56]);
-        acc[57] = __ffma2_rn(G[6], m5_1_0, acc[57]);
-        acc[58] = __ffma2_rn(G[6], m5_0_1, acc[58]);
-        acc[59] = __ffma2_rn(G[6], m4_2_0, acc[59]);
-        acc[60] = __ffma2_rn(G[6], m4_1_1, acc[60]);
-        acc[61] = __ffma2_rn(G[6], m4_0_2, acc[61]);
-        acc[62] = __ffma2_rn(G[6], m3_3_0, acc[62]);
-        acc[63] = __ffma2_rn(G[6], m3_2_1, acc[63]);
-        acc[64] = __ffma2_rn(G[6], m3_1_2, acc[64]);
-        acc[65] = __ffma2_rn(G[6], m3_0_3, acc[65]);
-        acc[66] = __ffma2_rn(G[6], m2_4_0, acc[66]);
-        acc[67] = __ffma2_rn(G[6], m2_3_1, acc[67]);
-        acc[68] = __ffma2_rn(G[6], m2_2_2, acc[68]);
-        acc[69] = __ffma2_rn(G[6], m2_1_3, acc[69]);
-        acc[70] = __ffma2_rn(G[6], m2_0_4, acc[70]);
-        acc[71] = __ffma2_rn(G[6], m1_5_0, acc[71]);
-        acc[72] = __ffma2_rn(G[6], m1_4_1, acc[72]);
-        acc[73] = __ffma2_rn(G[6], m1_3_2, acc[73]);
-        acc[74] = __ffma2_rn(G[6], m1_2_3, acc[74]);
-        acc[75] = __ffma2_rn(G[6], m1_1_4, acc[75]);
-        acc[76] = __ffma2_rn(G[6], m1_0_5, acc[76]);
-        acc[77] = __ffma2_rn(G[6], m0_6_0, acc[77]);
-        acc[78] = __ffma2_rn(G[6], m0_5_1, acc[78]);
-        acc[79] = __ffma2_rn(G[6], m0_4_2, acc[79]);
-        acc[80] = __ffma2_rn(G[6], m0_3_3, acc[80]);
-        acc[81] = __ffma2_rn(G[6], m0_2_4, acc[81]);
-        acc[82] = __ffma2_rn(G[6], m0_1_5, acc[82]);
-        acc[83] = __ffma2_rn(G[6], m0_0_6, acc[83]);
-        acc[84] = __ffma2_rn(gtx, m6_0_0, acc[84]);
-        acc[85] = __ffma2_rn(gtx, m5_1_0, acc[85]);
-        acc[86] = __ffma2_rn(gtx, m5_0_1, acc[86]);
-        acc[87] = __ffma2_rn(gtx, m4_2_0, acc[87]);
-        acc[88] = __ffma2_rn(gtx, m4_1_1, acc[88]);
-        acc[89] = __ffma2_rn(gtx, m4_0_2, acc[89]);
-        acc[90] = __ffma2_rn(gtx, m3_3_0, acc[90]);
-        acc[91] = __ffma2_rn(gtx, m3_2_1, acc[91]);
-        acc[92] = __ffma2_rn(gtx, m3_1_2, acc[92]);
-        acc[93] = __ffma2_rn(gtx, m3_0_3, acc[93]);
-        acc[94] = __ffma2_rn(gtx, m2_4_0, acc[94]);
-        acc[95] = __ffma2_rn(gtx, m2_3_1, acc[95]);
-        acc[96] = __ffma2_rn(gtx, m2_2_2, acc[96]);
-        acc[97] = __ffma2_rn(gtx, m2_1_3, acc[97]);
-        acc[98] = __ffma2_rn(gtx, m2_0_4, acc[98]);
-        acc[99] = __ffma2_rn(gtx, m1_5_0, acc[99]);
-        acc[100] = __ffma2_rn(gtx, m1_4_1, acc[100]);
-        acc[101] = __ffma2_rn(gtx, m1_3_2, acc[101]);
-        acc[102] = __ffma2_rn(gtx, m1_2_3, acc[102]);
-        acc[103] = __ffma2_rn(gtx, m1_1_4, acc[103]);
-        acc[104] = __ffma2_rn(gtx, m1_0_5, acc[104]);
-        acc[105] = __ffma2_rn(gtx, m0_6_0, acc[105]);
-        acc[106] = __ffma2_rn(gtx, m0_5_1, acc[106]);
-        acc[107] = __ffma2_rn(gtx, m0_4_2, acc[107]);
-        acc[108] = __ffma2_rn(gtx, m0_3_3, acc[108]);
-        acc[109] = __ffma2_rn(gtx, m0_2_4, acc[109]);
-        acc[110] = __ffma2_rn(gtx, m0_1_5, acc[110]);
-        acc[111] = __ffma2_rn(gtx, m0_0_6, acc[111]);
-        acc[112] = __ffma2_rn(gty, m0_6_0, acc[112]);
-        acc[113] = __ffma2_rn(gty, m0_5_1, acc[113]);
-        acc[114] = __ffma2_rn(gty, m0_4_2, acc[114]);
-        acc[115] = __ffma2_rn(gty, m0_3_3, acc[115]);
-        acc[116] = __ffma2_rn(gty, m0_2_4, acc[116]);
-        acc[117] = __ffma2_rn(gty, m0_1_5, acc[117]);
-        acc[118] = __ffma2_rn(gty, m0_0_6, acc[118]);
-        acc[119] = __ffma2_rn(gtz, m0_0_6, acc[119]);
-    }
-    __device__ __forceinline__ static void mono_to_f(const float* acc, float* f) {
-        f[0] = 1.0f * acc[0];
-        f[1] = 1.0f * acc[2];
-        f[2] = 1.0f * acc[3];
-        f[3] = 1.0f * acc[1];
-        f[4] = 6.0f * acc[5];
-        f[5] = 3.0f * acc[8];
-        f[6] = ((1.0f * acc[9] + -0.5f * acc[7]) + -0.5f * acc[4]);
-        f[7] = 3.0f * acc[6];
-        f[8] = (-3.0f * acc[7] + 3.0f * acc[4]);
-        f[9] = (-15.0f * acc[16] + 45.0f * acc[11]);
-        f[10] = 30.0f * acc[14];
-        f[11] = ((6.0f * acc[18] + -1.5f * acc[16]) + -1.5f * acc[11]);
-        f[12] = ((1.0f * acc[19] + -1.5f * acc[17]) + -1.5f * acc[12]);
-        f[13] = ((6.0f * acc[15] + -1.5f * acc[13]) + -1.5f * acc[10]);
-        f[14] = (-15.0f * acc[17] + 15.0f * acc[12]);
-        f[15] = (-45.0f * acc[13] + 15.0f * acc[10]);
-        f[16] = (-420.0f * acc[26] + 420.0f * acc[21]);
-        f[17] = (-105.0f * acc[31] + 315.0f * acc[24]);
-        f[18] = ((90.0f * acc[28] + -15.0f * acc[26]) + -15.0f * acc[21]);
-        f[19] = ((10.0f * acc[33] + -7.5f * acc[31]) + -7.5f * acc[24]);
-        f[20] = ((fmaf(0.75f, acc[23], 1.0f * acc[34]) + fmaf(0.375f, acc[20], -3.0f * acc[32])) + (0.375f * acc[30] + -3.0f * acc[25]));
-        f[21] = ((10.0f * acc[29] + -7.5f * acc[27]) + -7.5f * acc[22]);
-        f[22] = ((-45.0f * acc[32] + 7.5f * acc[30]) + (45.0f * acc[25] + -7.5f * acc[20]));
-        f[23] = (-315.0f * acc[27] + 105.0f * acc[22]);
-        f[24] = ((105.0f * acc[30] + -630.0f * acc[23]) + 105.0f * acc[20]);
-        f[25] = ((945.0f * acc[50] + -9450.0f * acc[41]) + 4725.0f * acc[36]);
-        f[26] = (-3780.0f * acc[46] + 3780.0f * acc[39]);
-        f[27] = ((fmaf(-157.5f, acc[36], -420.0f * acc[52]) + 52.5f * acc[50]) + (1260.0f * acc[43] + -105.0f * acc[41]));
-        f[28] = ((210.0f * acc[48] + -105.0f * acc[46]) + -105.0f * acc[39]);
-        f[29] = ((fmaf(3.75f, acc[41], 15.0f * acc[54]) + fmaf(1.875f, acc[36], -22.5f * acc[52])) + (1.875f * acc[50] + -22.5f * acc[43]));
-        f[30] = ((fmaf(3.75f, acc[42], 1.0f * acc[55]) + fmaf(1.875f, acc[37], -5.0f * acc[53])) + (1.875f * acc[51] + -5.0f * acc[44]));
-        f[31] = ((fmaf(3.75f, acc[38], 15.0f * acc[49]) + fmaf(1.875f, acc[35], -22.5f * acc[47])) + (1.875f * acc[45] + -22.5f * acc[40]));
-        f[32] = ((-105.0f * acc[53] + 52.5f * acc[51]) + (105.0f * acc[44] + -52.5f * acc[37]));
-        f[33] = ((fmaf(-52.5f, acc[35], -1260.0f * acc[47]) + 157.5f * acc[45]) + (420.0f * acc[40] + 105.0f * acc[38]));
-        f[34] = ((945.0f * acc[51] + -5670.0f * acc[42]) + 945.0f * acc[37]);
-        f[35] = ((4725.0f * acc[45] + -9450.0f * acc[38]) + 945.0f * acc[35]);
-        f[36] = ((62370.0f * acc[71] + -207900.0f * acc[62]) + 62370.0f * acc[57]);
-        f[37] = ((10395.0f * acc[78] + -103950.0f * acc[67]) + 51975.0f * acc[60]);
-        f[38] = ((-18900.0f * acc[73] + 1890.0f * acc[71]) + (18900.0f * acc[64] + -1890.0f * acc[57]));
-        f[39] = ((fmaf(-1417.5f, acc[60], -1260.0f * acc[80]) + 472.5f * acc[78]) + (3780.0f * acc[69] + -945.0f * acc[67]));
-        f[40] = ((fmaf(52.5f, acc[62], 420.0f * acc[75]) + fmaf(26.25f, acc[57], -420.0f * acc[73])) + (26.25f * acc[71] + -420.0f * acc[64]));
-        f[41] = ((fmaf(26.25f, acc[67], 21.0f * acc[82]) + fmaf(13.125f, acc[60], -52.5f * acc[80])) + (13.125f * acc[78] + -52.5f * acc[69]));
-        f[42] = ((fmaf(-0.9375f, acc[59], fmaf(-7.5f, acc[70], 1.0f * acc[83])) + fmaf(-0.3125f, acc[56], fmaf(11.25f, acc[68], -7.5f * acc[81]))) + (fmaf(-0.9375f, acc[66], 5.625f * acc[79]) + fmaf(5.625f, acc[61], -0.3125f * acc[77])));
-        f[43] = ((fmaf(26.25f, acc[63], 21.0f * acc[76]) + fmaf(13.125f, acc[58], -52.5f * acc[74])) + (13.125f * acc[72] + -52.5f * acc[65]));
-        f[44] = ((fmaf(-13.125f, acc[66], -210.0f * acc[81]) + fmaf(-210.0f, acc[61], 210.0f * acc[79])) + (fmaf(13.125f, acc[59], -13.125f * acc[77]) + fmaf(13.125f, acc[56], 210.0f * acc[70])));
-        f[45] = ((fmaf(-472.5f, acc[58], -3780.0f * acc[74]) + 1417.5f * acc[72]) + (1260.0f * acc[65] + 945.0f * acc[63]));
-        f[46] = ((fmaf(4725.0f, acc[61], 4725.0f * acc[79]) + fmaf(2362.5f, acc[59], -472.5f * acc[77])) + (fmaf(-472.5f, acc[56], -28350.0f * acc[68]) + 2362.5f * acc[66]));
-        f[47] = ((51975.0f * acc[72] + -103950.0f * acc[63]) + 10395.0f * acc[58]);
-        f[48] = ((-10395.0f * acc[77] + 155925.0f * acc[66]) + (-155925.0f * acc[59] + 10395.0f * acc[56]));
-        f[49] = ((-135135.0f * acc[112] + 2837835.0f * acc[99]) + (-4729725.0f * acc[90] + 945945.0f * acc[85]));
-        f[50] = ((810810.0f * acc[106] + -2702700.0f * acc[95]) + 810810.0f * acc[88]);
-        f[51] = ((fmaf(311850.0f, acc[92], 62370.0f * acc[114]) + fmaf(25987.5f, acc[90], -5197.5f * acc[112])) + (fmaf(-25987.5f, acc[85], -623700.0f * acc[101]) + 46777.5f * acc[99]));
-        f[52] = ((-69300.0f * acc[108] + 20790.0f * acc[106]) + (69300.0f * acc[97] + -20790.0f * acc[88]));
-        f[53] = ((fmaf(354.375f, acc[85], fmaf(-4725.0f, acc[101], -3150.0f * acc[116])) + fmaf(118.125f, acc[99], 2362.5f * acc[114])) + (fmaf(-7087.5f, acc[92], -118.125f * acc[112]) + fmaf(590.625f, acc[90], 9450.0f * acc[103])));
-        f[54] = ((fmaf(472.5f, acc[95], 756.0f * acc[110]) + fmaf(236.25f, acc[88], -1260.0f * acc[108])) + (236.25f * acc[106] + -1260.0f * acc[97]));
-        f[55] = ((fmaf(-6.5625f, acc[90], fmaf(-105.0f, acc[103], 28.0f * acc[118])) + fmaf(-2.1875f, acc[85], fmaf(105.0f, acc[101], -105.0f * acc[116]))) + (fmaf(-6.5625f, acc[99], 52.5f * acc[114]) + fmaf(52.5f, acc[92], -2.1875f * acc[112])));
-        f[56] = ((fmaf(-6.5625f, acc[91], fmaf(-10.5f, acc[104], 1.0f * acc[119])) + fmaf(-2.1875f, acc[86], fmaf(26.25f, acc[102], -10.5f * acc[117]))) + (fmaf(-6.5625f, acc[100], 13.125f * acc[115]) + fmaf(13.125f, acc[93], -2.1875f * acc[113])));
-        f[57] = ((fmaf(-6.5625f, acc[87], fmaf(-105.0f, acc[98], 28.0f * acc[111])) + fmaf(-2.1875f, acc[84], fmaf(105.0f, acc[96], -105.0f * acc[109]))) + (fmaf(-6.5625f, acc[94], 52.5f * acc[107]) + fmaf(52.5f, acc[89], -2.1875f * acc[105])));
-        f[58] = ((fmaf(-118.125f, acc[100], -378.0f * acc[117]) + fmaf(-630.0f, acc[93], 630.0f * acc[115])) + (fmaf(118.125f, acc[91], -118.125f * acc[113]) + fmaf(118.125f, acc[86], 378.0f * acc[104])));
-        f[59] = ((fmaf(118.125f, acc[84], fmaf(4725.0f, acc[96], -9450.0f * acc[109])) + fmaf(-590.625f, acc[94], 7087.5f * acc[107])) + (fmaf(-2362.5f, acc[89], -354.375f * acc[105]) + fmaf(-118.125f, acc[87], 3150.0f * acc[98])));
-        f[60] = ((fmaf(17325.0f, acc[93], 17325.0f * acc[115]) + fmaf(25987.5f, acc[91], -5197.5f * acc[113])) + (fmaf(-5197.5f, acc[86], -103950.0f * acc[102]) + 25987.5f * acc[100]));
-        f[61] = ((fmaf(62370.0f, acc[89], 311850.0f * acc[107]) + fmaf(46777.5f, acc[87], -25987.5f * acc[105])) + (fmaf(-5197.5f, acc[84], -623700.0f * acc[96]) + 25987.5f * acc[94]));
-        f[62] = ((-135135.0f * acc[113] + 2027025.0f * acc[100]) + (-2027025.0f * acc[91] + 135135.0f * acc[86]));
-        f[63] = ((-945945.0f * acc[105] + 4729725.0f * acc[94]) + (-2837835.0f * acc[87] + 135135.0f * acc[84]));
-    }
-    __device__ __forceinline__ static void grad_coeffs(const float* w, float* gq) {
-        (void)w; (void)gq;
-        gq[0] = 1.0f * w[3];
-        gq[1] = 1.0f * w[1];
-        gq[2] = 1.0f * w[2];
-        gq[3] = (-1.0f * w[6] + 6.0f * w[8]);
-        gq[4] = 6.0f * w[4];
-        gq[5] = 3.0f * w[7];
-        gq[6] = 6.0f * w[4];
-        gq[7] = (-1.0f * w[6] + -6.0f * w[8]);
-        gq[8] = 3.0f * w[5];
-        gq[9] = 3.0f * w[7];
-        gq[10] = 3.0f * w[5];
-        gq[11] = 2.0f * w[6];
-        gq[12] = (-4.5f * w[13] + 45.0f * w[15]);
-        gq[13] = (90.0f * w[9] + -3.0f * w[11]);
-        gq[14] = (-3.0f * w[12] + 30.0f * w[14]);
-        gq[15] = (-1.5f * w[13] + -45.0f * w[15]);
-        gq[16] = 30.0f * w[10];
-        gq[17] = 6.0f * w[13];
-        gq[18] = (45.0f * w[9] + -1.5f * w[11]);
-        gq[19] = (-3.0f * w[13] + -90.0f * w[15]);
-        gq[20] = 30.0f * w[10];
-        gq[21] = (-45.0f * w[9] + -4.5f * w[11]);
-        gq[22] = (-3.0f * w[12] + -30.0f * w[14]);
-        gq[23] = 6.0f * w[11];
-        gq[24] = (-1.5f * w[12] + 15.0f * w[14]);
-        gq[25] = 30.0f * w[10];
-        gq[26] = 12.0f * w[13];
-        gq[27] = (-1.5f * w[12] + -15.0f * w[14]);
-        gq[28] = 12.0f * w[11];
-        gq[29] = 3.0f * w[12];
-        gq[30] = ((1.5f * w[20] + -30.0f * w[22]) + 420.0f * w[24]);
-        gq[31] = (1260.0f * w[16] + -45.0f * w[18]);
-        gq[32] = (-22.5f * w[21] + 315.0f * w[23]);
-        gq[33] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[34] = (630.0f * w[17] + -15.0f * w[19]);
-        gq[35] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[36] = (-420.0f * w[16] + -15.0f * w[18]);
-        gq[37] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[38] = 90.0f * w[18];
-        gq[39] = 10.0f * w[21];
-        gq[40] = (420.0f * w[16] + -15.0f * w[18]);
-        gq[41] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[42] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[43] = (-1260.0f * w[16] + -45.0f * w[18]);
-        gq[44] = (-15.0f * w[21] + -630.0f * w[23]);
-        gq[45] = 90.0f * w[18];
-        gq[46] = ((1.5f * w[20] + 30.0f * w[22]) + 420.0f * w[24]);
-        gq[47] = (-315.0f * w[17] + -22.5f * w[19]);
-        gq[48] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[49] = 10.0f * w[19];
-        gq[50] = (-7.5f * w[21] + 105.0f * w[23]);
-        gq[51] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[52] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[53] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[54] = 180.0f * w[18];
-        gq[55] = 30.0f * w[21];
-        gq[56] = (-105.0f * w[17] + -7.5f * w[19]);
-        gq[57] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[58] = 30.0f * w[19];
-        gq[59] = 4.0f * w[20];
-        gq[60] = ((9.375f * w[31] + -262.5f * w[33]) + 4725.0f * w[35]);
-        gq[61] = ((18900.0f * w[25] + -630.0f * w[27]) + 7.5f * w[29]);
-        gq[62] = ((7.5f * w[30] + -210.0f * w[32]) + 3780.0f * w[34]);
-        gq[63] = ((11.25f * w[31] + 315.0f * w[33]) + -28350.0f * w[35]);
-        gq[64] = (11340.0f * w[26] + -315.0f * w[28]);
-        gq[65] = (-67.5f * w[31] + 1260.0f * w[33]);
-        gq[66] = ((-18900.0f * w[25] + -210.0f * w[27]) + 7.5f * w[29]);
-        gq[67] = (7.5f * w[30] + -11340.0f * w[34]);
-        gq[68] = (2520.0f * w[27] + -45.0f * w[29]);
-        gq[69] = (-10.0f * w[30] + 210.0f * w[32]);
-        gq[70] = ((1.875f * w[31] + 157.5f * w[33]) + 4725.0f * w[35]);
-        gq[71] = (-3780.0f * w[26] + -105.0f * w[28]);
-        gq[72] = (-22.5f * w[31] + -1260.0f * w[33]);
-        gq[73] = 210.0f * w[28];
-        gq[74] = 15.0f * w[31];
-        gq[75] = ((4725.0f * w[25] + -157.5f * w[27]) + 1.875f * w[29]);
-        gq[76] = ((7.5f * w[31] + 210.0f * w[33]) + -18900.0f * w[35]);
-        gq[77] = (3780.0f * w[26] + -105.0f * w[28]);
-        gq[78] = ((-28350.0f * w[25] + -315.0f * w[27]) + 11.25f * w[29]);
-        gq[79] = (7.5f * w[30] + -11340.0f * w[34]);
-        gq[80] = (1260.0f * w[27] + -22.5f * w[29]);
-        gq[81] = ((7.5f * w[31] + 630.0f * w[33]) + 18900.0f * w[35]);
-        gq[82] = (-11340.0f * w[26] + -315.0f * w[28]);
-        gq[83] = (-45.0f * w[31] + -2520.0f * w[33]);
-        gq[84] = 210.0f * w[28];
-        gq[85] = ((4725.0f * w[25] + 262.5f * w[27]) + 9.375f * w[29]);
-        gq[86] = ((7.5f * w[30] + 210.0f * w[32]) + 3780.0f * w[34]);
-        gq[87] = (-1260.0f * w[27] + -67.5f * w[29]);
-        gq[88] = (-10.0f * w[30] + -210.0f * w[32]);
-        gq[89] = 15.0f * w[29];
-        gq[90] = ((1.875f * w[30] + -52.5f * w[32]) + 945.0f * w[34]);
-        gq[91] = (3780.0f * w[26] + -105.0f * w[28]);
-        gq[92] = (-45.0f * w[31] + 840.0f * w[33]);
-        gq[93] = (3.75f * w[30] + -5670.0f * w[34]);
-        gq[94] = (2520.0f * w[27] + -45.0f * w[29]);
-        gq[95] = (-15.0f * w[30] + 315.0f * w[32]);
-        gq[96] = (-3780.0f * w[26] + -105.0f * w[28]);
-        gq[97] = (-45.0f * w[31] + -2520.0f * w[33]);
-        gq[98] = 630.0f * w[28];
-        gq[99] = 60.0f * w[31];
-        gq[100] = ((1.875f * w[30] + 52.5f * w[32]) + 945.0f * w[34]);
-        gq[101] = (-840.0f * w[27] + -45.0f * w[29]);
-        gq[102] = (-15.0f * w[30] + -315.0f * w[32]);
-        gq[103] = 60.0f * w[29];
-        gq[104] = 5.0f * w[30];
-        gq[105] = ((-1.875f * w[42] + 78.75f * w[44]) + (-2835.0f * w[46] + 62370.0f * w[48]));
-        gq[106] = ((311850.0f * w[36] + -9450.0f * w[38]) + 131.25f * w[40]);
-        gq[107] = ((65.625f * w[43] + -2362.5f * w[45]) + 51975.0f * w[47]);
-        gq[108] = ((-3.75f * w[42] + 52.5f * w[44]) + (9450.0f * w[46] + -623700.0f * w[48]));
-        gq[109] = ((207900.0f * w[37] + -5670.0f * w[39]) + 52.5f * w[41]);
-        gq[110] = ((22.5f * w[42] + -840.0f * w[44]) + 18900.0f * w[46]);
-        gq[111] = (-623700.0f * w[36] + 157.5f * w[40]);
-        gq[112] = ((78.75f * w[43] + 2835.0f * w[45]) + -311850.0f * w[47]);
-        gq[113] = (56700.0f * w[38] + -1260.0f * w[40]);
-        gq[114] = (-157.5f * w[43] + 3780.0f * w[45]);
-        gq[115] = ((-1.875f * w[42] + -26.25f * w[44]) + (4725.0f * w[46] + 311850.0f * w[48]));
-        gq[116] = ((-207900.0f * w[37] + -1890.0f * w[39]) + 52.5f * w[41]);
-        gq[117] = (22.5f * w[42] + -56700.0f * w[46]);
-        gq[118] = (7560.0f * w[39] + -105.0f * w[41]);
-        gq[119] = (-15.0f * w[42] + 420.0f * w[44]);
-        gq[120] = ((62370.0f * w[36] + 1890.0f * w[38]) + 26.25f * w[40]);
-        gq[121] = ((13.125f * w[43] + 1417.5f * w[45]) + 51975.0f * w[47]);
-        gq[122] = (-18900.0f * w[38] + -420.0f * w[40]);
-        gq[123] = (-52.5f * w[43] + -3780.0f * w[45]);
-        gq[124] = 420.0f * w[40];
-        gq[125] = 21.0f * w[43];
-        gq[126] = ((62370.0f * w[36] + -1890.0f * w[38]) + 26.25f * w[40]);
-        gq[127] = ((-1.875f * w[42] + 26.25f * w[44]) + (4725.0f * w[46] + -311850.0f * w[48]));
-        gq[128] = ((51975.0f * w[37] + -1417.5f * w[39]) + 13.125f * w[41]);
-        gq[129] = (-623700.0f * w[36] + 157.5f * w[40]);
-        gq[130] = ((52.5f * w[43] + 1890.0f * w[45]) + -207900.0f * w[47]);
-        gq[131] = (18900.0f * w[38] + -420.0f * w[40]);
-        gq[132] = ((-3.75f * w[42] + -52.5f * w[44]) + (9450.0f * w[46] + 623700.0f * w[48]));
-        gq[133] = ((-311850.0f * w[37] + -2835.0f * w[39]) + 78.75f * w[41]);
-        gq[134] = (22.5f * w[42] + -56700.0f * w[46]);
-        gq[135] = (3780.0f * w[39] + -52.5f * w[41]);
-        gq[136] = ((311850.0f * w[36] + 9450.0f * w[38]) + 131.25f * w[40]);
-        gq[137] = ((52.5f * w[43] + 5670.0f * w[45]) + 207900.0f * w[47]);
-        gq[138] = (-56700.0f * w[38] + -1260.0f * w[40]);
-        gq[139] = (-105.0f * w[43] + -7560.0f * w[45]);
-        gq[140] = 420.0f * w[40];
-        gq[141] = ((-1.875f * w[42] + -78.75f * w[44]) + (-2835.0f * w[46] + -62370.0f * w[48]));
-        gq[142] = ((51975.0f * w[37] + 2362.5f * w[39]) + 65.625f * w[41]);
-        gq[143] = ((22.5f * w[42] + 840.0f * w[44]) + 18900.0f * w[46]);
-        gq[144] = (-3780.0f * w[39] + -157.5f * w[41]);
-        gq[145] = (-15.0f * w[42] + -420.0f * w[44]);
-        gq[146] = 21.0f * w[41];
-        gq[147] = ((13.125f * w[43] + -472.5f * w[45]) + 10395.0f * w[47]);
-        gq[148] = ((51975.0f * w[37] + -1417.5f * w[39]) + 13.125f * w[41]);
-        gq[149] = ((11.25f * w[42] + -420.0f * w[44]) + 9450.0f * w[46]);
-        gq[150] = ((26.25f * w[43] + 945.0f * w[45]) + -103950.0f * w[47]);
-        gq[151] = (37800.0f * w[38] + -840.0f * w[40]);
-        gq[152] = (-157.5f * w[43] + 3780.0f * w[45]);
-        gq[153] = ((-103950.0f * w[37] + -945.0f * w[39]) + 26.25f * w[41]);
-        gq[154] = (22.5f * w[42] + -56700.0f * w[46]);
-        gq[155] = (11340.0f * w[39] + -157.5f * w[41]);
-        gq[156] = (-30.0f * w[42] + 840.0f * w[44]);
-        gq[157] = ((13.125f * w[43] + 1417.5f * w[45]) + 51975.0f * w[47]);
-        gq[158] = (-37800.0f * w[38] + -840.0f * w[40]);
-        gq[159] = (-157.5f * w[43] + -11340.0f * w[45]);
-        gq[160] = 1680.0f * w[40];
-        gq[161] = 105.0f * w[43];
-        gq[162] = ((10395.0f * w[37] + 472.5f * w[39]) + 13.125f * w[41]);
-        gq[163] = ((11.25f * w[42] + 420.0f * w[44]) + 9450.0f * w[46]);
-        gq[164] = (-3780.0f * w[39] + -157.5f * w[41]);
-        gq[165] = (-30.0f * w[42] + -840.0f * w[44]);
-        gq[166] = 105.0f * w[41];
-        gq[167] = 6.0f * w[42];
-        gq[168] = ((-15.3125f * w[57] + 826.875f * w[59]) + (-36382.5f * w[61] + 945945.0f * w[63]));
-        gq[169] = ((5675670.0f * w[49] + -155925.0f * w[51]) + (2126.25f * w[53] + -13.125f * w[55]));
-        gq[170] = ((-13.125f * w[56] + 708.75f * w[58]) + (-31185.0f * w[60] + 810810.0f * w[62]));
-        gq[171] = ((-32.8125f * w[57] + -590.625f * w[59]) + (233887.5f * w[61] + -14189175.0f * w[63]));
-        gq[172] = ((4054050.0f * w[50] + -103950.0f * w[52]) + 1181.25f * w[54]);
-        gq[173] = ((262.5f * w[57] + -11812.5f * w[59]) + 311850.0f * w[61]);
-        gq[174] = ((-18918900.0f * w[49] + 103950.0f * w[51]) + (2362.5f * w[53] + -26.25f * w[55]));
-        gq[175] = ((-26.25f * w[56] + 472.5f * w[58]) + (103950.0f * w[60] + -8108100.0f * w[62]));
-        gq[176] = ((1247400.0f * w[51] + -28350.0f * w[53]) + 210.0f * w[55]);
-        gq[177] = ((52.5f * w[56] + -2520.0f * w[58]) + 69300.0f * w[60]);
-        gq[178] = ((-19.6875f * w[57] + -1771.875f * w[59]) + (77962.5f * w[61] + 14189175.0f * w[63]));
-        gq[179] = (-8108100.0f * w[50] + 1417.5f * w[54]);
-        gq[180] = ((315.0f * w[57] + 14175.0f * w[59]) + -1871100.0f * w[61]);
-        gq[181] = (207900.0f * w[52] + -3780.0f * w[54]);
-        gq[182] = (-315.0f * w[57] + 9450.0f * w[59]);
-        gq[183] = ((5675670.0f * w[49] + 93555.0f * w[51]) + (236.25f * w[53] + -13.125f * w[55]));
-        gq[184] = ((-13.125f * w[56] + -236.25f * w[58]) + (51975.0f * w[60] + 4054050.0f * w[62]));
-        gq[185] = ((-1247400.0f * w[51] + -9450.0f * w[53]) + 210.0f * w[55]);
-        gq[186] = (52.5f * w[56] + -207900.0f * w[60]);
-        gq[187] = (18900.0f * w[53] + -210.0f * w[55]);
-        gq[188] = (-21.0f * w[56] + 756.0f * w[58]);
-        gq[189] = ((-2.1875f * w[57] + -354.375f * w[59]) + (-25987.5f * w[61] + -945945.0f * w[63]));
-        gq[190] = ((810810.0f * w[50] + 20790.0f * w[52]) + 236.25f * w[54]);
-        gq[191] = ((52.5f * w[57] + 7087.5f * w[59]) + 311850.0f * w[61]);
-        gq[192] = (-69300.0f * w[52] + -1260.0f * w[54]);
-        gq[193] = (-105.0f * w[57] + -9450.0f * w[59]);
-        gq[194] = 756.0f * w[54];
-        gq[195] = 28.0f * w[57];
-        gq[196] = ((945945.0f * w[49] + -25987.5f * w[51]) + (354.375f * w[53] + -2.1875f * w[55]));
-        gq[197] = ((-13.125f * w[57] + -236.25f * w[59]) + (93555.0f * w[61] + -5675670.0f * w[63]));
-        gq[198] = ((810810.0f * w[50] + -20790.0f * w[52]) + 236.25f * w[54]);
-        gq[199] = ((-14189175.0f * w[49] + 77962.5f * w[51]) + (1771.875f * w[53] + -19.6875f * w[55]));
-        gq[200] = ((-13.125f * w[56] + 236.25f * w[58]) + (51975.0f * w[60] + -4054050.0f * w[62]));
-        gq[201] = ((311850.0f * w[51] + -7087.5f * w[53]) + 52.5f * w[55]);
-        gq[202] = ((-26.25f * w[57] + -2362.5f * w[59]) + (103950.0f * w[61] + 18918900.0f * w[63]));
-        gq[203] = (-8108100.0f * w[50] + 1417.5f * w[54]);
-        gq[204] = ((210.0f * w[57] + 9450.0f * w[59]) + -1247400.0f * w[61]);
-        gq[205] = (69300.0f * w[52] + -1260.0f * w[54]);
-        gq[206] = ((14189175.0f * w[49] + 233887.5f * w[51]) + (590.625f * w[53] + -32.8125f * w[55]));
-        gq[207] = ((-26.25f * w[56] + -472.5f * w[58]) + (103950.0f * w[60] + 8108100.0f * w[62]));
-        gq[208] = ((-1871100.0f * w[51] + -14175.0f * w[53]) + 315.0f * w[55]);
-        gq[209] = (52.5f * w[56] + -207900.0f * w[60]);
-        gq[210] = (9450.0f * w[53] + -105.0f * w[55]);
-        gq[211] = ((-13.125f * w[57] + -2126.25f * w[59]) + (-155925.0f * w[61] + -5675670.0f * w[63]));
-        gq[212] = ((4054050.0f * w[50] + 103950.0f * w[52]) + 1181.25f * w[54]);
-        gq[213] = ((210.0f * w[57] + 28350.0f * w[59]) + 1247400.0f * w[61]);
-        gq[214] = (-207900.0f * w[52] + -3780.0f * w[54]);
-        gq[215] = (-210.0f * w[57] + -18900.0f * w[59]);
-        gq[216] = 756.0f * w[54];
-        gq[217] = ((-945945.0f * w[49] + -36382.5f * w[51]) + (-826.875f * w[53] + -15.3125f * w[55]));
-        gq[218] = ((-13.125f * w[56] + -708.75f * w[58]) + (-31185.0f * w[60] + -810810.0f * w[62]));
-        gq[219] = ((311850.0f * w[51] + 11812.5f * w[53]) + 262.5f * w[55]);
-        gq[220] = ((52.5f * w[56] + 2520.0f * w[58]) + 69300.0f * w[60]);
-        gq[221] = (-9450.0f * w[53] + -315.0f * w[55]);
-        gq[222] = (-21.0f * w[56] + -756.0f * w[58]);
-        gq[223] = 28.0f * w[55];
-        gq[224] = ((-2.1875f * w[56] + 118.125f * w[58]) + (-5197.5f * w[60] + 135135.0f * w[62]));
-        gq[225] = ((810810.0f * w[50] + -20790.0f * w[52]) + 236.25f * w[54]);
-        gq[226] = ((105.0f * w[57] + -4725.0f * w[59]) + 124740.0f * w[61]);
-        gq[227] = ((-6.5625f * w[56] + 118.125f * w[58]) + (25987.5f * w[60] + -2027025.0f * w[62]));
-        gq[228] = ((623700.0f * w[51] + -14175.0f * w[53]) + 105.0f * w[55]);
-        gq[229] = ((39.375f * w[56] + -1890.0f * w[58]) + 51975.0f * w[60]);
-        gq[230] = (-2702700.0f * w[50] + 472.5f * w[54]);
-        gq[231] = ((210.0f * w[57] + 9450.0f * w[59]) + -1247400.0f * w[61]);
-        gq[232] = (207900.0f * w[52] + -3780.0f * w[54]);
-        gq[233] = (-420.0f * w[57] + 12600.0f * w[59]);
-        gq[234] = ((-6.5625f * w[56] + -118.125f * w[58]) + (25987.5f * w[60] + 2027025.0f * w[62]));
-        gq[235] = ((-1247400.0f * w[51] + -9450.0f * w[53]) + 210.0f * w[55]);
-        gq[236] = (78.75f * w[56] + -311850.0f * w[60]);
-        gq[237] = (37800.0f * w[53] + -420.0f * w[55]);
-        gq[238] = (-52.5f * w[56] + 1890.0f * w[58]);
-        gq[239] = ((810810.0f * w[50] + 20790.0f * w[52]) + 236.25f * w[54]);
-        gq[240] = ((105.0f * w[57] + 14175.0f * w[59]) + 623700.0f * w[61]);
-        gq[241] = (-207900.0f * w[52] + -3780.0f * w[54]);
-        gq[242] = (-420.0f * w[57] + -37800.0f * w[59]);
-        gq[243] = 3780.0f * w[54];
-        gq[244] = 168.0f * w[57];
-        gq[245] = ((-2.1875f * w[56] + -118.125f * w[58]) + (-5197.5f * w[60] + -135135.0f * w[62]));
-        gq[246] = ((124740.0f * w[51] + 4725.0f * w[53]) + 105.0f * w[55]);
-        gq[247] = ((39.375f * w[56] + 1890.0f * w[58]) + 51975.0f * w[60]);
-        gq[248] = (-12600.0f * w[53] + -420.0f * w[55]);
-        gq[249] = (-52.5f * w[56] + -1890.0f * w[58]);
-        gq[250] = 168.0f * w[55];
-        gq[251] = 7.0f * w[56];
-    }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
-        (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        const float u1_0_0 = x;
-        const float u0_1_0 = y;
-        const float u0_0_1 = z;
-        const float u2_0_0 = x * u1_0_0;
-        const float u1_1_0 = x * u0_1_0;
-        const float u1_0_1 = x * u0_0_1;
-        const float u0_2_0 = y * u0_1_0;
-        const float u0_1_1 = y * u0_0_1;
-        const float u0_0_2 = z * u0_0_1;
-        const float u3_0_0 = x * u2_0_0;
-        const float u2_1_0 = x * u1_1_0;
-        const float u2_0_1 = x * u1_0_1;
-        const float u1_2_0 = x * u0_2_0;
-        const float u1_1_1 = x * u0_1_1;
-        const float u1_0_2 = x * u0_0_2;
-        const float u0_3_0 = y * u0_2_0;
-        const float u0_2_1 = y * u0_1_1;
-        const float u0_1_2 = y * u0_0_2;
-        const float u0_0_3 = z * u0_0_2;
-        const float u4_0_0 = x * u3_0_0;
-        const float u3_1_0 = x * u2_1_0;
-        const float u3_0_1 = x * u2_0_1;
-        const float u2_2_0 = x * u1_2_0;
-        const float u2_1_1 = x * u1_1_1;
-        const float u2_0_2 = x * u1_0_2;
-        const float u1_3_0 = x * u0_3_0;
-        const float u1_2_1 = x * u0_2_1;
-        const float u1_1_2 = x * u0_1_2;
-        const float u1_0_3 = x * u0_0_3;
-        const float u0_4_0 = y * u0_3_0;
-        const float u0_3_1 = y * u0_2_1;
-        const float u0_2_2 = y * u0_1_2;
-        const float u0_1_3 = y * u0_0_3;
-        const float u0_0_4 = z * u0_0_3;
-        const float u5_0_0 = x * u4_0_0;
-        const float u4_1_0 = x * u3_1_0;
-        const float u4_0_1 = x * u3_0_1;
-        const float u3_2_0 = x * u2_2_0;
-        const float u3_1_1 = x * u2_1_1;
-        const float u3_0_2 = x * u2_0_2;
-        const float u2_3_0 = x * u1_3_0;
-        const float u2_2_1 = x * u1_2_1;
-        const float u2_1_2 = x * u1_1_2;
-        const float u2_0_3 = x * u1_0_3;
-        const float u1_4_0 = x * u0_4_0;
-        const float u1_3_1 = x * u0_3_1;
-        const float u1_2_2 = x * u0_2_2;
-        const float u1_1_3 = x * u0_1_3;
-        const float u1_0_4 = x * u0_0_4;
-        const float u0_5_0 = y * u0_4_0;
-        const float u0_4_1 = y * u0_3_1;
-        const float u0_3_2 = y * u0_2_2;
-        const float u0_2_3 = y * u0_1_3;
-        const float u0_1_4 = y * u0_0_4;
-        const float u0_0_5 = z * u0_0_4;
-        const float u6_0_0 = x * u5_0_0;
-        const float u5_1_0 = x * u4_1_0;
-        const float u5_0_1 = x * u4_0_1;
-        const float u4_2_0 = x * u3_2_0;
-        const float u4_1_1 = x * u3_1_1;
-        const float u4_0_2 = x * u3_0_2;
-        const float u3_3_0 = x * u2_3_0;
-        const float u3_2_1 = x * u2_2_1;
-        const float u3_1_2 = x * u2_1_2;
-        const float u3_0_3 = x * u2_0_3;
-        const float u2_4_0 = x * u1_4_0;
-        const float u2_3_1 = x * u1_3_1;
-        const float u2_2_2 = x * u1_2_2;
-        const float u2_1_3 = x * u1_1_3;
-        const float u2_0_4 = x * u1_0_4;
-        const float u1_5_0 = x * u0_5_0;
-        const float u1_4_1 = x * u0_4_1;
-        const float u1_3_2 = x * u0_3_2;
-        const float u1_2_3 = x * u0_2_3;
-        const float u1_1_4 = x * u0_1_4;
-        const float u1_0_5 = x * u0_0_5;
-        const float u0_6_0 = y * u0_5_0;
-        const float u0_5_1 = y * u0_4_1;
-        const float u0_4_2 = y * u0_3_2;
-        const float u0_3_3 = y * u0_2_3;
-        const float u0_2_4 = y * u0_1_4;
-        const float u0_1_5 = y * u0_0_5;
-        const float u0_0_6 = z * u0_0_5;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
-        gx[1] = gq[3] * u1_0_0 + gq[4] * u0_1_0 + gq[5] * u0_0_1;
-        gy[1] = gq[6] * u1_0_0 + gq[7] * u0_1_0 + gq[8] * u0_0_1;
-        gz[1] = gq[9] * u1_0_0 + gq[10] * u0_1_0 + gq[11] * u0_0_1;
-        gx[2] = gq[12] * u2_0_0 + gq[13] * u1_1_0 + gq[14] * u1_0_1 + gq[15] * u0_2_0 + gq[16] * u0_1_1 + gq[17] * u0_0_2;
-        gy[2] = gq[18] * u2_0_0 + gq[19] * u1_1_0 + gq[20] * u1_0_1 + gq[21] * u0_2_0 + gq[22] * u0_1_1 + gq[23] * u0_0_2;
-        gz[2] = gq[24] * u2_0_0 + gq[25] * u1_1_0 + gq[26] * u1_0_1 + gq[27] * u0_2_0 + gq[28] * u0_1_1 + gq[29] * u0_0_2;
-        gx[3] = gq[30] * u3_0_0 + gq[31] * u2_1_0 + gq[32] * u2_0_1 + gq[33] * u1_2_0 + gq[34] * u1_1_1 + gq[35] * u1_0_2 + gq[36] * u0_3_0 + gq[37] * u0_2_1 + gq[38] * u0_1_2 + gq[39] * u0_0_3;
-        gy[3] = gq[40] * u3_0_0 + gq[41] * u2_1_0 + gq[42] * u2_0_1 + gq[43] * u1_2_0 + gq[44] * u1_1_1 + gq[45] * u1_0_2 + gq[46] * u0_3_0 + gq[47] * u0_2_1 + gq[48] * u0_1_2 + gq[49] * u0_0_3;
-        gz[3] = gq[50] * u3_0_0 + gq[51] * u2_1_0 + gq[52] * u2_0_1 + gq[53] * u1_2_0 + gq[54] * u1_1_1 + gq[55] * u1_0_2 + gq[56] * u0_3_0 + gq[57] * u0_2_1 + gq[58] * u0_1_2 + gq[59] * u0_0_3;
-        gx[4] = gq[60] * u4_0_0 + gq[61] * u3_1_0 + gq[62] * u3_0_1 + gq[63] * u2_2_0 + gq[64] * u2_1_1 + gq[65] * u2_0_2 + gq[66] * u1_3_0 + gq[67] * u1_2_1 + gq[68] * u1_1_2 + gq[69] * u1_0_3 + gq[70] * u0_4_0 + gq[71] * u0_3_1 + gq[72] * u0_2_2 + gq[73] * u0_1_3 + gq[74] * u0_0_4;
-        gy[4] = gq[75] * u4_0_0 + gq[76] * u3_1_0 + gq[77] * u3_0_1 + gq[78] * u2_2_0 + gq[79] * u2_1_1 + gq[80] * u2_0_2 + gq[81] * u1_3_0 + gq[82] * u1_2_1 + gq[83] * u1_1_2 + gq[84] * u1_0_3 + gq[85] * u0_4_0 + gq[86] * u0_3_1 + gq[87] * u0_2_2 + gq[88] * u0_1_3 + gq[89] * u0_0_4;
-        gz[4] = gq[90] * u4_0_0 + gq[91] * u3_1_0 + gq[92] * u3_0_1 + gq[93] * u2_2_0 + gq[94] * u2_1_1 + gq[95] * u2_0_2 + gq[96] * u1_3_0 + gq[97] * u1_2_1 + gq[98] * u1_1_2 + gq[99] * u1_0_3 + gq[100] * u0_4_0 + gq[101] * u0_3_1 + gq[102] * u0_2_2 + gq[103] * u0_1_3 + gq[104] * u0_0_4;
-        gx[5] = gq[105] * u5_0_0 + gq[106] * u4_1_0 + gq[107] * u4_0_1 + gq[108] * u3_2_0 + gq[109] * u3_1_1 + gq[110] * u3_0_2 + gq[111] * u2_3_0 + gq[112] * u2_2_1 + gq[113] * u2_1_2 + gq[114] * u2_0_3 + gq[115] * u1_4_0 + gq[116] * u1_3_1 + gq[117] * u1_2_2 + gq[118] * u1_1_3 + gq[119] * u1_0_4 + gq[120] * u0_5_0 + gq[121] * u0_4_1 + gq[122] * u0_3_2 + gq[123] * u0_2_3 + gq[124] * u0_1_4 + gq[125] * u0_0_5;
-        gy[5] = gq[126] * u5_0_0 + gq[127] * u4_1_0 + gq[128] * u4_0_1 + gq[129] * u3_2_0 + gq[130] * u3_1_1 + gq[131] * u3_0_2 + gq[132] * u2_3_0 + gq[133] * u2_2_1 + gq[134] * u2_1_2 + gq[135] * u2_0_3 + gq[136] * u1_4_0 + gq[137] * u1_3_1 + gq[138] * u1_2_2 + gq[139] * u1_1_3 + gq[140] * u1_0_4 + gq[141] * u0_5_0 + gq[142] * u0_4_1 + gq[143] * u0_3_2 + gq[144] * u0_2_3 + gq[145] * u0_1_4 + gq[146] * u0_0_5;
-        gz[5] = gq[147] * u5_0_0 + gq[148] * u4_1_0 + gq[149] * u4_0_1 + gq[150] * u3_2_0 + gq[151] * u3_1_1 + gq[152] * u3_0_2 + gq[153] * u2_3_0 + gq[154] * u2_2_1 + gq[155] * u2_1_2 + gq[156] * u2_0_3 + gq[157] * u1_4_0 + gq[158] * u1_3_1 + gq[159] * u1_2_2 + gq[160] * u1_1_3 + gq[161] * u1_0_4 + gq[162] * u0_5_0 + gq[163] * u0_4_1 + gq[164] * u0_3_2 + gq[165] * u0_2_3 + gq[166] * u0_1_4 + gq[167] * u0_0_5;
-        gx[6] = gq[168] * u6_0_0 + gq[169] * u5_1_0 + gq[170] * u5_0_1 + gq[171] * u4_2_0 + gq[172] * u4_1_1 + gq[173] * u4_0_2 + gq[174] * u3_3_0 + gq[175] * u3_2_1 + gq[176] * u3_1_2 + gq[177] * u3_0_3 + gq[178] * u2_4_0 + gq[179] * u2_3_1 + gq[180] * u2_2_2 + gq[181] * u2_1_3 + gq[182] * u2_0_4 + gq[183] * u1_5_0 + gq[184] * u1_4_1 + gq[185] * u1_3_2 + gq[186] * u1_2_3 + gq[187] * u1_1_4 + gq[188] * u1_0_5 + gq[189] * u0_6_0 + gq[190] * u0_5_1 + gq[191] * u0_4_2 + gq[192] * u0_3_3 + gq[193] * u0_2_4 + gq[194] * u0_1_5 + gq[195] * u0_0_6;
-        gy[6] = gq[196] * u6_0_0 + gq[197] * u5_1_0 + gq[198] * u5_0_1 + gq[199] * u4_2_0 + gq[200] * u4_1_1 + gq[201] * u4_0_2 + gq[202] * u3_3_0 + gq[203] * u3_2_1 + gq[204] * u3_1_2 + gq[205] * u3_0_3 + gq[206] * u2_4_0 + gq[207] * u2_3_1 + gq[208] * u2_2_2 + gq[209] * u2_1_3 + gq[210] * u2_0_4 + gq[211] * u1_5_0 + gq[212] * u1_4_1 + gq[213] * u1_3_2 + gq[214] * u1_2_3 + gq[215] * u1_1_4 + gq[216] * u1_0_5 + gq[217] * u0_6_0 + gq[218] * u0_5_1 + gq[219] * u0_4_2 + gq[220] * u0_3_3 + gq[221] * u0_2_4 + gq[222] * u0_1_5 + gq[223] * u0_0_6;
-        gz[6] = gq[224] * u6_0_0 + gq[225] * u5_1_0 + gq[226] * u5_0_1 + gq[227] * u4_2_0 + gq[228] * u4_1_1 + gq[229] * u4_0_2 + gq[230] * u3_3_0 + gq[231] * u3_2_1 + gq[232] * u3_1_2 + gq[233] * u3_0_3 + gq[234] * u2_4_0 + gq[235] * u2_3_1 + gq[236] * u2_2_2 + gq[237] * u2_1_3 + gq[238] * u2_0_4 + gq[239] * u1_5_0 + gq[240] * u1_4_1 + gq[241] * u1_3_2 + gq[242] * u1_2_3 + gq[243] * u1_1_4 + gq[244] * u1_0_5 + gq[245] * u0_6_0 + gq[246] * u0_5_1 + gq[247] * u0_4_2 + gq[248] * u0_3_3 + gq[249] * u0_2_4 + gq[250] * u0_1_5 + gq[251] * u0_0_6;
-    }
-    static constexpr int QZ = 11;    // Gauss-Legendre nodes in cos(theta)
-    static constexpr int QP = 22;    // uniform azimuths
-    static constexpr int QF = 15;    // azimuthal harmonics 1, cos m phi, sin m phi
+    static constexpr int LPS = 6;   // lane-pair product rule: node pairs
+    static constexpr int LPQ = 6;   // ... and azimuth quads
+    static constexpr int LES = 8;   // lane-pair projected-exponential rule: node pairs
+    static constexpr int LEQ = 8;   // ... and azimuth quads
 #if defined(SHS_NB) && SHS_NB == 8
-    __device__ __forceinline__ static const float* qleg() { return kQuadLeg8; }
-    __device__ __forceinline__ static const float* qtrig() { return kQuadTrig8; }
-    __device__ __forceinline__ static const float* qw() { return kQuadW8; }
+    __device__ __forceinline__ static const float* lp_leg() { return kLpLeg8; }
+    __device__ __forceinline__ static const float* le_leg() { return kLeLeg8; }
+    __device__ __forceinline__ static const float* lp_trig_row(int b) { return kLpTrig8 + b * 15; }
 #endif
+    __device__ __forceinline__ static float lp_trig(int b, int h) {   // h = 2m - 1: cos(m phi_b), 2m: sin
+        switch (b * 15 + h) {
+            case 1: return 0.9914448857307434f;
+            case 2: return 0.13052618503570557f;
+            case 3: return 0.9659258127212524f;
+            case 4: return 0.258819043636322f;
+            case 5: return 0.9238795042037964f;
+            case 6: return 0.3826834261417389f;
+            case 7: return 0.8660253882408142f;
+            case 8: return 0.5f;
+            case 9: return 0.7933533191680908f;
+            case 10: return 0.6087614297866821f;
+            case 11: return 0.7071067690849304f;
+            case 12: return 0.7071067690849304f;
+            case 13: return 0.6087614297866821f;
+            case 14: return 0.7933533191680908f;
+            case 16: return 0.9238795042037964f;
+            case 17: return 0.3826834261417389f;
+            case 18: return 0.7071067690849304f;
+            case 19: return 0.7071067690849304f;
+            case 20: return 0.3826834261417389f;
+            case 21: return 0.9238795042037964f;
+            case 22: return 6.123234262925839e-17f;
+            case 23: return 1.0f;
+            case 24: return -0.3826834261417389f;
+            case 25: return 0.9238795042037964f;
+            case 26: return -0.7071067690849304f;
+            case 27: return 0.7071067690849304f;
+            case 28: return -0.9238795042037964f;
+            case 29: return 0.3826834261417389f;
+            case 31: return 0.7933533191680908f;
+            case 32: return 0.6087614297866821f;
+            case 33: return 0.258819043636322f;
+            case 34: return 0.9659258127212524f;
+            case 35: return -0.3826834261417389f;
+            case 36: return 0.9238795042037964f;
+            case 37: return -0.8660253882408142f;
+            case 38: return 0.5f;
+            case 39: return -0.9914448857307434f;
+            case 40: return -0.13052618503570557f;
+            case 41: return -0.7071067690849304f;
+            case 42: return -0.7071067690849304f;
+            case 43: return -0.13052618503570557f;
+            case 44: return -0.9914448857307434f;
+            case 46: return 0.6087614297866821f;
+            case 47: return 0.7933533191680908f;
+            case 48: return -0.258819043636322f;
+            case 49: return 0.9659258127212524f;
+            case 50: return -0.9238795042037964f;
+            case 51: return 0.3826834261417389f;
+            case 52: return -0.8660253882408142f;
+            case 53: return -0.5f;
+            case 54: return -0.13052618503570557f;
+            case 55: return -0.9914448857307434f;
+            case 56: return 0.7071067690849304f;
+            case 57: return -0.7071067690849304f;
+            case 58: return 0.9914448857307434f;
+            case 59: return 0.13052618503570557f;
+            case 61: return 0.3826834261417389f;
+            case 62: return 0.9238795042037964f;
+            case 63: return -0.7071067690849304f;
+            case 64: return 0.7071067690849304f;
+            case 65: return -0.9238795042037964f;
+            case 66: return -0.3826834261417389f;
+            case 67: return -1.8369701465288538e-16f;
+            case 68: return -1.0f;
+            case 69: return 0.9238795042037964f;
+            case 70: return -0.3826834261417389f;
+            case 71: return 0.7071067690849304f;
+            case 72: return 0.7071067690849304f;
+            case 73: return -0.3826834261417389f;
+            case 74: return 0.9238795042037964f;
+            case 76: return 0.13052618503570557f;
+            case 77: return 0.9914448857307434f;
+            case 78: return -0.9659258127212524f;
+            case 79: return 0.258819043636322f;
+            case 80: return -0.3826834261417389f;
+            case 81: return -0.9238795042037964f;
+            case 82: return 0.8660253882408142f;
+            case 83: return -0.5f;
+            case 84: return 0.6087614297866821f;
+            case 85: return 0.7933533191680908f;
+            case 86: return -0.7071067690849304f;
+            case 87: return 0.7071067690849304f;
+            case 88: return -0.7933533191680908f;
+            case 89: return -0.6087614297866821f;
+            default: return 1.0f;
+        }
+    }
+    __device__ __forceinline__ static float le_trig(int b, int h) {   // h = 2m - 1: cos(m phi_b), 2m: sin
+        switch (b * 15 + h) {
+            case 1: return 0.9951847195625305f;
+            case 2: return 0.0980171412229538f;
+            case 3: return 0.9807852506637573f;
+            case 4: return 0.19509032368659973f;
+            case 5: return 0.9569403529167175f;
+            case 6: return 0.290284663438797f;
+            case 7: return 0.9238795042037964f;
+            case 8: return 0.3826834261417389f;
+            case 9: return 0.8819212913513184f;
+            case 10: return 0.4713967442512512f;
+            case 11: return 0.8314695954322815f;
+            case 12: return 0.5555702447891235f;
+            case 13: return 0.7730104327201843f;
+            case 14: return 0.6343932747840881f;
+            case 16: return 0.9569403529167175f;
+            case 17: return 0.290284663438797f;
+            case 18: return 0.8314695954322815f;
+            case 19: return 0.5555702447891235f;
+            case 20: return 0.6343932747840881f;
+            case 21: return 0.7730104327201843f;
+            case 22: return 0.3826834261417389f;
+            case 23: return 0.9238795042037964f;
+            case 24: return 0.0980171412229538f;
+            case 25: return 0.9951847195625305f;
+            case 26: return -0.19509032368659973f;
+            case 27: return 0.9807852506637573f;
+            case 28: return -0.4713967442512512f;
+            case 29: return 0.8819212913513184f;
+            case 31: return 0.8819212913513184f;
+            case 32: return 0.4713967442512512f;
+            case 33: return 0.5555702447891235f;
+            case 34: return 0.8314695954322815f;
+            case 35: return 0.0980171412229538f;
+            case 36: return 0.9951847195625305f;
+            case 37: return -0.3826834261417389f;
+            case 38: return 0.9238795042037964f;
+            case 39: return -0.7730104327201843f;
+            case 40: return 0.6343932747840881f;
+            case 41: return -0.9807852506637573f;
+            case 42: return 0.19509032368659973f;
+            case 43: return -0.9569403529167175f;
+            case 44: return -0.290284663438797f;
+            case 46: return 0.7730104327201843f;
+            case 47: return 0.6343932747840881f;
+            case 48: return 0.19509032368659973f;
+            case 49: return 0.9807852506637573f;
+            case 50: return -0.4713967442512512f;
+            case 51: return 0.8819212913513184f;
+            case 52: return -0.9238795042037964f;
+            case 53: return 0.3826834261417389f;
+            case 54: return -0.9569403529167175f;
+            case 55: return -0.290284663438797f;
+            case 56: return -0.5555702447891235f;
+            case 57: return -0.8314695954322815f;
+            case 58: return 0.0980171412229538f;
+            case 59: return -0.9951847195625305f;
+            case 61: return 0.6343932747840881f;
+            case 62: return 0.7730104327201843f;
+            case 63: return -0.19509032368659973f;
+            case 64: return 0.9807852506637573f;
+            case 65: return -0.8819212913513184f;
+            case 66: return 0.4713967442512512f;
+            case 67: return -0.9238795042037964f;
+            case 68: return -0.3826834261417389f;
+            case 69: return -0.290284663438797f;
+            case 70: return -0.9569403529167175f;
+            case 71: return 0.5555702447891235f;
+            case 72: return -0.8314695954322815f;
+            case 73: return 0.9951847195625305f;
+            case 74: return -0.0980171412229538f;
+            case 76: return 0.4713967442512512f;
+            case 77: return 0.8819212913513184f;
+            case 78: return -0.5555702447891235f;
+            case 79: return 0.8314695954322815f;
+            case 80: return -0.9951847195625305f;
+            case 81: return -0.0980171412229538f;
+            case 82: return -0.3826834261417389f;
+            case 83: return -0.9238795042037964f;
+            case 84: return 0.6343932747840881f;
+            case 85: return -0.7730104327201843f;
+            case 86: return 0.9807852506637573f;
+            case 87: return 0.19509032368659973f;
+            case 88: return 0.290284663438797f;
+            case 89: return 0.9569403529167175f;
+            case 91: return 0.290284663438797f;
+            case 92: return 0.9569403529167175f;
+            case 93: return -0.8314695954322815f;
+            case 94: return 0.5555702447891235f;
+            case 95: return -0.7730104327201843f;
+            case 96: return -0.6343932747840881f;
+            case 97: return 0.3826834261417389f;
+            case 98: return -0.9238795042037964f;
+            case 99: return 0.9951847195625305f;
+            case 100: return 0.0980171412229538f;
+            case 101: return 0.19509032368659973f;
+            case 102: return 0.9807852506637573f;
+            case 103: return -0.8819212913513184f;
+            case 104: return 0.4713967442512512f;
+            case 106: return 0.0980171412229538f;
+            case 107: return 0.9951847195625305f;
+            case 108: return -0.9807852506637573f;
+            case 109: return 0.19509032368659973f;
+            case 110: return -0.290284663438797f;
+            case 111: return -0.9569403529167175f;
+            case 112: return 0.9238795042037964f;
+            case 113: return -0.3826834261417389f;
+            case 114: return 0.4713967442512512f;
+            case 115: return 0.8819212913513184f;
+            case 116: return -0.8314695954322815f;
+            case 117: return 0.5555702447891235f;
+            case 118: return -0.6343932747840881f;
+            case 119: return -0.7730104327201843f;
+            default: return 1.0f;
+        }
+    }
 };
 
 }  // namespace shsgen

@@ -69,7 +69,8 @@ struct shs_scene_s {
     int n_spheres;
     int K, Kpad;
     int device;
-    int max_grid;          // persistent backward grid
+    int grid, tail_grid;   // persistent adjoint grids: one launch or the pair pass; the tail's launch (from 6 bands)
+    int max_grid;          // the larger one
     int partial_stride;    // floats per block partial
     float4* spheres;       // [max(N,1)]
     float* light;          // [3][Kpad]
@@ -80,7 +81,7 @@ struct shs_scene_s {
     unsigned int* batch_counter;
     float* fwork;          // f storage when shs_shade gets no saved buffer (tensor-core path)
     int64_t fwork_points;
-    float* bwork;          // [K][P] adjoint coefficients of the split backward (>= 6 bands)
+    float* bwork;          // [K][P] adjoint coefficients between the tail and the pair pass (from 6 bands)
     int64_t bwork_points;
     float* hwork;          // tensor-core adjoint: squaring operands per block [grid][kMaxK][K + 2][128]
     float2* ol_table;      // exp_mode 2: (a, b) per node
@@ -89,7 +90,7 @@ struct shs_scene_s {
 };
 
 struct shs_batch_s {
-    unsigned int* queues;  // [16] tile counters: forward / backward x n_bands
+    unsigned int* queues;  // [64] tile counters: forward / backward x n_bands x variant
 };
 
 namespace {
@@ -126,7 +127,7 @@ template <int NB> struct Bwd {
     static cudaError_t run(const BwdArgs& a, cudaStream_t s) { return shs::launch_backward<NB>(a, s); }
 };
 
-int blocks_per_sm(int nb, int n) {
+shs::BwdBlocks blocks_per_sm(int nb, int n) {
     switch (nb) {
         case 1: return shs::backward_blocks_per_sm<1>(n);
         case 2: return shs::backward_blocks_per_sm<2>(n);
@@ -136,7 +137,7 @@ int blocks_per_sm(int nb, int n) {
         case 6: return shs::backward_blocks_per_sm<6>(n);
         case 7: return shs::backward_blocks_per_sm<7>(n);
         case 8: return shs::backward_blocks_per_sm<8>(n);
-        default: return 1;
+        default: return {1, 1, 1};
     }
 }
 
@@ -180,6 +181,8 @@ SceneView view_of(const shs_scene_s* s) {
     v.status = s->status;
     return v;
 }
+
+int variant_of(const shs_scene_s* s) { return shs::batch_variant(view_of(s), s->cfg.n_bands); }
 
 bool tensor_core_precision(const shs_config& c) { return c.precision != SHS_FP32; }
 
@@ -451,7 +454,7 @@ int report_cuda(cudaError_t e, const char* what) { return cuda_fail(e, what); }
 cudaError_t launch_backward_nb(int n_bands, const BwdArgs& a, cudaStream_t s) {
     return dispatch<Bwd>(n_bands, a, s);
 }
-int backward_blocks_per_sm_nb(int n_bands, int n_spheres) { return blocks_per_sm(n_bands, n_spheres); }
+int backward_blocks_per_sm_nb(int n_bands, int n_spheres) { return blocks_per_sm(n_bands, n_spheres).both; }
 }  // namespace shs
 
 extern "C" {
@@ -495,7 +498,10 @@ shs_status shs_scene_create(const shs_config* cfg, int32_t n_spheres, const floa
         delete sc;
         return cuda_fail(e, "query device");
     }
-    sc->max_grid = sms * blocks_per_sm(cfg->n_bands, n_spheres);
+    const shs::BwdBlocks blocks = blocks_per_sm(cfg->n_bands, n_spheres);
+    sc->tail_grid = sms * blocks.tail;
+    sc->grid = sms * (cfg->n_bands >= 6 ? blocks.pairs : blocks.both);
+    sc->max_grid = sc->grid > sc->tail_grid ? sc->grid : sc->tail_grid;
     sc->partial_stride = static_cast<int>(align_up(3 * sc->K + 1 + 4 * n_spheres, 4));
     const size_t partial_floats =
         cfg->deterministic ? static_cast<size_t>(sc->max_grid) * sc->partial_stride : sc->partial_stride;
@@ -751,8 +757,12 @@ static shs_status backward_common(shs_scene_t sc, int64_t n_points, const float*
     a.counter = sc->cfg.deterministic ? nullptr : sc->counter;
     a.partial_stride = sc->partial_stride;
     a.dfp_ws = nullptr;
+    const int per_tile = shs::tile_points(sc->cfg.n_bands);
+    const int64_t tiles = (n_points + per_tile - 1) / per_tile;
+    a.grid = static_cast<int>(tiles < sc->grid ? tiles : sc->grid);
+    a.tail_grid = static_cast<int>(tiles < sc->tail_grid ? tiles : sc->tail_grid);
     if (sc->cfg.n_bands >= 6) {
-        // split backward: per-point tail pass, then a sphere-per-lane pair pass
+        // the tail and the pair pass as two launches
         if (sc->bwork_points < n_points) {
             cudaError_t e = cudaStreamSynchronize(s);
             cudaFree(sc->bwork);
@@ -764,9 +774,6 @@ static shs_status backward_common(shs_scene_t sc, int64_t n_points, const float*
         }
         a.dfp_ws = sc->bwork;
     }
-    const int64_t tiles = (n_points + shs::kBlock - 1) / shs::kBlock;
-    a.grid = static_cast<int>(tiles < sc->max_grid ? tiles : sc->max_grid);
-    a.skip_tail = 0;
     if (tensor_core_precision(sc->cfg)) {
         // the exponential's and the shading's adjoint on the tensor cores, then
         // the float32 pair pass of the split backward
@@ -831,7 +838,7 @@ static shs_status backward_common(shs_scene_t sc, int64_t n_points, const float*
         t.hist = sc->hwork;
         cudaError_t e = shs::launch_tail_tc_bwd(t, s);
         if (e != cudaSuccess) return cuda_fail(e, "launch tensor-core adjoint tail");
-        a.skip_tail = 1;
+        a.tail_grid = 0;
     }
     cudaError_t e = dispatch<Bwd>(sc->cfg.n_bands, a, s);
     return e == cudaSuccess ? SHS_OK : cuda_fail(e, "launch backward");
@@ -862,7 +869,7 @@ shs_status shs_batch_create(shs_batch_t* out) {
     *out = nullptr;
     shs_batch_s* b = new (std::nothrow) shs_batch_s();
     if (!b) return fail(SHS_ERR_OOM, "host allocation failed");
-    cudaError_t e = cudaMalloc(&b->queues, 16 * sizeof(unsigned int));
+    cudaError_t e = cudaMalloc(&b->queues, 64 * sizeof(unsigned int));
     if (e != cudaSuccess) {
         delete b;
         return cuda_fail(e, "allocate batch queues");
@@ -903,16 +910,19 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
                 return fail(SHS_ERR_INVALID_ARG, "requests %d and %d share a scene", j, i);
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(batch->queues, 0, 16 * sizeof(unsigned int), s);
+    cudaError_t e = cudaMemsetAsync(batch->queues, 0, 64 * sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_fail(e, "reset batch queues");
-    for (int nb = 1; nb <= 8 && e == cudaSuccess; ++nb) {
+    for (int g = 0; g < 32 && e == cudaSuccess; ++g) {
+        const int nb = g / 4 + 1, variant = g % 4;
+        if (variant >= shs::batch_variants(nb)) continue;
         shs::FwdBatch fb;
         fb.n = 0;
         fb.total_tiles = 0;
-        fb.queue = batch->queues + (nb - 1);
+        fb.variant = variant;
+        fb.queue = batch->queues + g;
         for (int i = 0; i < n_reqs; ++i) {
             const shs_request& r = reqs[i];
-            if (r.scene->cfg.n_bands != nb || r.n_points == 0 || !r.radiance) continue;
+            if (r.scene->cfg.n_bands != nb || variant_of(r.scene) != variant || r.n_points == 0 || !r.radiance) continue;
             shs::FwdArgs& a = fb.r[fb.n];
             a = shs::FwdArgs{};
             a.sc = view_of(r.scene);
@@ -923,22 +933,25 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
             a.radiance = r.radiance;
             split_saved(r.scene, r.n_points, r.saved, &a.saved_f, &a.saved_k);
             fb.tile_begin[fb.n] = fb.total_tiles;
-            fb.total_tiles += (r.n_points + shs::kBlock - 1) / shs::kBlock;
+            fb.total_tiles += (r.n_points + shs::tile_points(nb) - 1) / shs::tile_points(nb);
             ++fb.n;
         }
         fb.tile_begin[fb.n] = fb.total_tiles;
         if (fb.n) e = dispatch<FwdB>(nb, fb, s);
     }
-    for (int nb = 1; nb <= 8 && e == cudaSuccess; ++nb) {
+    for (int g = 0; g < 32 && e == cudaSuccess; ++g) {
+        const int nb = g / 4 + 1, variant = g % 4;
+        if (variant >= shs::batch_variants(nb)) continue;
         shs::BwdBatch bb;
         bb.n = 0;
         bb.max_spheres = 0;
         bb.total_tiles = 0;
-        bb.queue = batch->queues + 8 + (nb - 1);
+        bb.variant = variant;
+        bb.queue = batch->queues + 32 + g;
         for (int i = 0; i < n_reqs && e == cudaSuccess; ++i) {
             const shs_request& r = reqs[i];
             shs_scene_s* sc = r.scene;
-            if (sc->cfg.n_bands != nb || (!r.target && !r.d_radiance)) continue;
+            if (sc->cfg.n_bands != nb || variant_of(sc) != variant || (!r.target && !r.d_radiance)) continue;
             if (r.n_points == 0) {
                 if (r.d_light) e = cudaMemsetAsync(r.d_light, 0, sizeof(float) * 3 * sc->K, s);
                 if (e == cudaSuccess && r.d_centers && sc->n_spheres) e = cudaMemsetAsync(r.d_centers, 0, sizeof(float) * 3 * sc->n_spheres, s);
@@ -972,7 +985,7 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
             a.counter = sc->batch_counter;
             a.partial_stride = sc->partial_stride;
             bb.tile_begin[bb.n] = bb.total_tiles;
-            bb.total_tiles += (r.n_points + shs::kBlock - 1) / shs::kBlock;
+            bb.total_tiles += (r.n_points + shs::tile_points(nb) - 1) / shs::tile_points(nb);
             if (sc->n_spheres > bb.max_spheres) bb.max_spheres = sc->n_spheres;
             ++bb.n;
         }

@@ -1,0 +1,666 @@
+// Adjoint shading kernels for 6, 7 and 8 bands, compiled once per n_bands with
+// -DSHS_NB=n (shs_hi.cuh).
+//
+// Adjoint of the pair terms: one sphere per lane.  A warp owns the 16 points
+// whose tail adjoint it has just run; their coefficients go through shared
+// memory (read back as broadcasts), each lane keeps its sphere's geometry and
+// sums over the 16 points in registers, and the warp walks the spheres in
+// groups of 32, so every warp of a block has the same share of the work.
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "shs_hi.cuh"
+#include "shs_warp.cuh"
+
+namespace shs {
+namespace {
+
+// ---------------------------------------------------------------------------
+// pair adjoint
+// ---------------------------------------------------------------------------
+
+// A point's adjoint coefficients in shared memory: column m holds
+// w_lm = dLoss/df_lm (-2 pi eps) NORM_lm (2l - 1)!! / (l (l + 1)) for l = m ..
+// NB - 1 (l = 0: without the division), for m > 0 as (cos, sin) pairs; columns start
+// at multiples of four floats.
+__host__ __device__ constexpr int wcol(int m) {
+    int b = 0;
+    for (int k = 0; k < m; ++k) b += ((k ? 2 : 1) * (NB - k) + 3) / 4 * 4;
+    return b;
+}
+constexpr int WST = wcol(NB) + 4;
+constexpr int kWarpRegion = kWarpPoints * WST > 64 * NS ? kWarpPoints * WST : 64 * NS;   // floats
+
+// Adjoint of one pair's Psi = sum_l G_l(c) Phi_l(s_hat), Phi_l = sum_m w_lm
+// Ybar_lm: the gradients with respect to the sphere's centre (the point gets
+// the negative) and radius.  Per order m, with R_lm and d/dz R_lm = R_l,m+1:
+//   alpha = sum_l P_l' R_lm w_lm           -> d/dx, d/dy of C_m + i S_m
+//   beta  = sum_l P_l' R_l,m+1 w_lm        -> d/dz
+//   gamma = sum_l l (l + 1) P_l R_lm w_lm  -> -dPsi/dc
+// (the factor s2 of G_l is applied at the end).  The products P_l' R_l,m+1 of
+// one order are the next order's P_l' R_lm.  At 8 bands about 440 FP32
+// instructions a pair, where the evaluation and reverse sweep of all 64
+// harmonics took about 800.
+template <bool CULL>
+__device__ __forceinline__ void pair_backward(float px, float py, float pz, float4 sp, const float* w, float& gcx,
+                                              float& gcy, float& gcz, float& gr, Normal u) {
+    const PairGeom g = pair_geometry<CULL>(px, py, pz, sp, u);
+    float P[NB], dP[NB];
+    legendre(g.c, P, dP);
+#pragma unroll
+    for (int l = 1; l < NB; ++l) P[l] *= float(l * (l + 1));
+    const float sx = g.dx * g.invD, sy = g.dy * g.invD, sz = g.dz * g.invD;
+    float zi[NB], col[NB], nxt[NB], e[NB], C = 1.f, S = 0.f;
+    float gx = 0.f, gy = 0.f, gz = 0.f, ga = 0.f;
+    sh_column_factors(sz, zi);
+    sh_column<0>(zi, col);
+    static_for<NB>([&](auto mm) {
+        constexpr int m = mm;
+        float wm[((m ? 2 : 1) * (NB - m) + 3) / 4 * 4];
+        const float4* w4 = reinterpret_cast<const float4*>(w + wcol(m));
+#pragma unroll
+        for (int i = 0; i < ((m ? 2 : 1) * (NB - m) + 3) / 4; ++i) {
+            const float4 v = w4[i];
+            wm[4 * i] = v.x;
+            wm[4 * i + 1] = v.y;
+            wm[4 * i + 2] = v.z;
+            wm[4 * i + 3] = v.w;
+        }
+        sh_column<m + 1>(zi, nxt);
+        float ac = 0.f, as = 0.f, bc = 0.f, bs = 0.f, cc = 0.f, cs = 0.f;
+#pragma unroll
+        for (int i = 0; i < NB - m; ++i) {   // l = m + i
+            const float h = P[m + i] * col[i];
+            const float wc = wm[m ? 2 * i : i], ws = wm[m ? 2 * i + 1 : 0];
+            cc = fmaf(h, wc, cc);
+            if (m) {
+                ac = fmaf(e[i], wc, ac);
+                as = fmaf(e[i], ws, as);
+                cs = fmaf(h, ws, cs);
+            }
+            if (i) {
+                e[i - 1] = dP[m + i] * nxt[i - 1];
+                bc = fmaf(e[i - 1], wc, bc);
+                if (m) bs = fmaf(e[i - 1], ws, bs);
+            }
+        }
+        if (m) {
+            const float fm = static_cast<float>(m);   // C, S still hold order m - 1
+            gx = fmaf(fm, fmaf(ac, C, as * S), gx);
+            gy = fmaf(fm, fmaf(as, C, -(ac * S)), gy);
+            const float c1 = fmaf(sx, C, -(sy * S)), s1 = fmaf(sx, S, sy * C);
+            C = c1;
+            S = s1;
+            gz = fmaf(bc, C, fmaf(bs, S, gz));
+            ga = fmaf(cc, C, fmaf(cs, S, ga));
+        } else {
+            gz = bc;
+            ga = cc;
+        }
+#pragma unroll
+        for (int i = 0; i + 1 < NB - m; ++i) col[i] = nxt[i];
+    });
+    gx *= g.s2;
+    gy *= g.s2;
+    gz *= g.s2;
+    // dPsi/dc = -ga; c = sqrt(1 - s2): d c / d s2 = -1 / (2 c); clamped caps carry no gradient
+    const float ds2 = g.open ? __fdividef(0.5f * ga, g.c) : 0.f;
+    gr = ds2 * 2.f * sp.w * g.invD2;                 // s2 = r^2 / D^2
+    const float dD2 = -ds2 * g.s2 * g.invD2;
+    const float sg = sx * gx + sy * gy + sz * gz;    // s_hat = d / D: tangential part
+    gcx = fmaf(gx - sx * sg, g.invD, 2.f * dD2 * g.dx);
+    gcy = fmaf(gy - sy * sg, g.invD, 2.f * dD2 * g.dy);
+    gcz = fmaf(gz - sz * sg, g.invD, 2.f * dD2 * g.dz);
+}
+
+// ---------------------------------------------------------------------------
+// adjoint
+// ---------------------------------------------------------------------------
+
+constexpr int kDl = (3 * NS + 15) / 16 * 16;   // a lane parity's lighting sums, 16 at a time
+
+struct BwdShared {
+    float4* sph;                 // [N]
+    float4* acc;                 // [NWARP][N] (d cx, d cy, d cz, d r)
+    const float (*lt)[3][NSP];
+    const float* leg;
+    float (*dl)[2][kDl];         // [NWARP]
+    float* loss;                 // [NWARP]
+    float* w;                    // per warp: the operands of its products, then its points' rows [16][WST]
+    int region;                  // floats of w per warp
+    float4* pt;                  // [kTile]
+    float4* nrm;                 // [kTile] (horizon culling)
+};
+
+// Adjoint of the exponential and the shading at the lane pair's point: the
+// per-point outputs, the lighting and loss sums, and dLoss/df_i (-2 pi eps)
+// NORM_i of the lane's slots in dfp.
+template <bool EXP, bool CULL>
+__device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShared& sh, int64_t p, float* dfp) {
+    const LanePair lp = lane_pair();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = lp.odd ? 1 : 0;
+    const int64_t P = a.n_points;
+    const bool live = p < P;
+    const int64_t q = live ? p : 0;
+    const Normal nn{load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
+                    load_or(a.normals, 3 * q + 2, live)};
+    const float* legs = sh.leg + (lp.odd ? NL : 0);
+    float f[NS];
+    int k;
+    if (a.saved_f) {
+        lp_load(a.saved_f, P, q, live, lp, f);
+        k = live ? min(max(a.saved_k[q], 0), kMaxK) : 0;   // a foreign buffer cannot overrun hist
+    } else {
+        lp_log_visibility<CULL>(a.sc, sh.sph, load_or(a.points, 3 * q, live), load_or(a.points, 3 * q + 1, live),
+                                load_or(a.points, 3 * q + 2, live),
+                                CULL ? unit_normal(nn.x, nn.y, nn.z) : Normal{}, lp, f);
+        k = -1;
+    }
+    const float n2 = lp_norm2(f, lp);
+    if (k < 0) k = scaling_k(a.sc, n2);
+
+    // ---- the exponential again, keeping in local memory f, the operand of
+    // every squaring and S with V = e0 S (EXP: U).  The operands of the
+    // products sit in the warp's columns of shared memory, X and Y (a product's
+    // result and work arrays fill the registers).  kmax: the warp's largest k;
+    // a pair past its own k keeps S.
+    float* X = sh.w + warp * sh.region + lane;
+    float* Y = X + 32 * NS;
+    float fh[NS], hist[EXP ? 1 : kMaxK + 1][NS];
+    float scale = 1.f;
+    OLCoef ol{1.f, 1.f, 0.f, 0.f};
+    const float e0 = expf(lp_even(f[0]) * kInvSqrt4Pi);
+    const int kmax = EXP ? 0 : __reduce_max_sync(0xffffffffu, k);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) fh[s] = f[s];
+    {
+        float S[NS];
+        if constexpr (EXP) {
+            lp_proj_exp(f, legs + kLegProduct, lp, S);
+        } else {
+            scale = ldexpf(1.f, -k);
+            ol = ol_coef(a.sc, n2 * scale * scale);
+#pragma unroll
+            for (int s = 0; s < NS; ++s) S[s] = ol.b * (f[s] * scale);
+            S[0] = lp.odd ? S[0] : ol.a * kSqrt4Pi;
+        }
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            X[32 * s] = S[s];
+            hist[0][s] = S[s];
+        }
+    }
+#pragma unroll 1
+    for (int t = 0; t < kmax; ++t) {
+        float T[NS];
+        lp_product<true, true, 32>(X, nullptr, legs, lp, T);
+        const bool on = t < k;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            T[s] = on ? T[s] : X[32 * s];
+            X[32 * s] = T[s];
+            hist[t + 1][s] = T[s];
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < NS; ++s) X[32 * s] *= e0;
+
+    // ---- loss, dLoss/dB, and u_c = a_c dLoss/dB_c
+    float dB[3], uc[3], loss = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (a.target) {
+            const float r = load_or(a.radiance, 3 * q + c, live) - load_or(a.target, 3 * q + c, live);
+            dB[c] = r;
+            loss = fmaf(0.5f * r, r, loss);
+        } else {
+            dB[c] = load_or(a.d_radiance, 3 * q + c, live);
+        }
+        uc[c] = load_or(a.albedo, 3 * q + c, live) * dB[c];
+    }
+    if (a.target) {
+        const float v = warp_sum(lp.odd ? 0.f : loss);
+        if (lane == 0) sh.loss[warp] += v;
+    }
+
+    // ---- every two-operand product of the adjoint through one loop body (six
+    // inlined products would not fit the instruction cache):
+    //   step 0: W = V * H            -> d_albedo, d_light
+    //   step 1: dH = dW * V          -> d_normals (C is symmetric: the adjoint of a * b is d * b)
+    //   step 2: dV = dW * H
+    //   step 3 + i: dS = 2 dS * (operand of squaring kmax - 1 - i)
+    const Normal u = unit_normal(nn.x, nn.y, nn.z);
+    float de0 = 0.f;   // X: V, then dW, then dV and dS
+#pragma unroll 1
+    for (int step = 0; step < 3 + kmax; ++step) {
+        if (step == 1 && !a.d_normals) continue;
+        const int t = kmax + 2 - step;   // squaring, from step 3
+        float T[NS];
+        if (step == 0 || step == 2) {
+            float H[NS];
+            lp_cosine_lobe(u.x, u.y, u.z, lp, H);
+#pragma unroll
+            for (int s = 0; s < NS; ++s) Y[32 * s] = H[s];
+        } else {
+            const float* h = &hist[step == 1 ? kmax : t][0];
+            const float v = step == 1 ? e0 : 1.f;
+#pragma unroll
+            for (int s = 0; s < NS; ++s) Y[32 * s] = v * h[s];
+        }
+        lp_product<false, true, 32>(X, Y, legs, lp, T);
+        if (step == 0) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float lw = 0.f;
+#pragma unroll
+                for (int s = 0; s < NS; ++s) lw = fmaf(sh.lt[b][c][s], T[s], lw);
+                lw = lp_sum(lw);
+                if (live && !lp.odd && a.d_albedo) a.d_albedo[3 * q + c] = dB[c] * lw;
+            }
+            if (a.d_light) {
+#pragma unroll
+                for (int base = 0; base < 3 * NS; base += 16) {
+                    float v[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        v[i] = base + i < 3 * NS ? uc[(base + i) / NS] * T[(base + i) % NS] : 0.f;
+                    lp_halve<16, 16>(v, lane);
+                    sh.dl[warp][b][base + (lane >> 1)] += v[0];
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < NS; ++s)
+                X[32 * s] = fmaf(uc[0], sh.lt[b][0][s], fmaf(uc[1], sh.lt[b][1][s], uc[2] * sh.lt[b][2][s]));
+        } else if (step == 1) {
+            float gx, gy, gz;
+            lp_lobe_adjoint(u.x, u.y, u.z, T, lp, gx, gy, gz);
+            const float n2v = fmaf(nn.x, nn.x, fmaf(nn.y, nn.y, nn.z * nn.z)), il = n2v > 0.f ? rsqrtf(n2v) : 0.f;
+            const float ug = u.x * gx + u.y * gy + u.z * gz;
+            if (live && !lp.odd) {
+                a.d_normals[3 * q] = (gx - u.x * ug) * il;
+                a.d_normals[3 * q + 1] = (gy - u.y * ug) * il;
+                a.d_normals[3 * q + 2] = (gz - u.z * ug) * il;
+            }
+        } else if (step == 2) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                de0 = fmaf(T[s], hist[kmax][s], de0);
+                X[32 * s] = EXP ? T[s] : e0 * T[s];
+            }
+        } else {
+            if (t < k) {
+#pragma unroll
+                for (int s = 0; s < NS; ++s) X[32 * s] = 2.f * T[s];
+            }
+        }
+    }
+
+    // ---- exponent
+    if constexpr (EXP) {
+        float dV[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) dV[s] = X[32 * s];
+        lp_proj_exp_adjoint(fh, dV, e0, legs + kLegProduct, lp, dfp);
+    } else {
+        // S_0 = a(s) sqrt(4 pi), S_i = b(s) g_i: dg_i = b dS_i + (dA a'/s + dB b'/s) g_i
+        const float dA = lp_even(X[0]) * kSqrt4Pi;
+        float dBs = lp.odd ? X[0] * (fh[0] * scale) : 0.f;
+#pragma unroll
+        for (int s = 1; s < NS; ++s) dBs = fmaf(X[32 * s], fh[s] * scale, dBs);
+        dBs = lp_sum(dBs);
+        const float cg = fmaf(dA, ol.ca, dBs * ol.cb);
+#pragma unroll
+        for (int s = 0; s < NS; ++s) dfp[s] = fmaf(ol.b, X[32 * s], cg * (fh[s] * scale)) * scale;
+    }
+    de0 = lp_sum(de0);
+    dfp[0] = lp.odd ? dfp[0] : de0 * e0 * kInvSqrt4Pi;
+    static_for<NS>([&](auto s) {
+        constexpr int i0 = lp_index(s, 0), i1 = lp_index(s, 1);
+        dfp[s] *= a.sc.neg_2pi_eps * (lp.odd ? SH::norm(i1 < 0 ? 0 : i1) : SH::norm(i0));
+    });
+}
+
+// The lane's coefficients into its point's row of shared memory.
+__device__ __forceinline__ void lp_store_row(const float* dfp, float* row, const LanePair& lp) {
+    static_for<NS>([&](auto s) {
+        constexpr int m = lp_m(s), l0 = lp_l(s, 0), l1 = lp_l(s, 1), sn = lp_sin(s);
+        constexpr int o0 = wcol(m) + (m ? 2 * (l0 - m) + sn : l0), o1 = wcol(m) + (m ? 2 * (l1 - m) + sn : l1);
+        constexpr float c0 = dfact(l0) / float(l0 ? l0 * (l0 + 1) : 1), c1 = dfact(l1) / float(l1 * (l1 + 1));
+        if (l1 < NB || !lp.odd) row[lp.odd ? o1 : o0] = dfp[s] * (lp.odd ? c1 : c0);
+    });
+}
+
+// Pair adjoints of the warp's 16 points, one sphere per lane; with fewer than
+// 17 (9) spheres the lanes take two (four) points at once.
+template <bool CULL>
+__device__ __forceinline__ void lp_pairs(const BwdArgs& a, const BwdShared& sh, int64_t tile) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = a.sc.n_spheres;
+    const int width = N > 16 ? 32 : N > 8 ? 16 : 8, sub = lane / width, stride = 32 / width;
+    float4* acc_row = sh.acc + warp * N;
+    const float* rows = sh.w + warp * sh.region;
+    const bool want_pts = a.d_points != nullptr;
+    float gp[3] = {0.f, 0.f, 0.f};   // lane t < 16: gradient of the warp's point t
+    for (int j0 = 0; j0 < N; j0 += width) {
+        const int j = j0 + lane % width;
+        const bool has = j < N;
+        const float4 sp = has ? sh.sph[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int t = 0; t < kWarpPoints; t += stride) {
+            const int r = warp * kWarpPoints + t + sub;
+            const float4 pt = sh.pt[r];
+            Normal u{};
+            if (CULL) u = Normal{sh.nrm[r].x, sh.nrm[r].y, sh.nrm[r].z};
+            float gcx, gcy, gcz, gr;
+            pair_backward<CULL>(pt.x, pt.y, pt.z, sp, rows + (r - warp * kWarpPoints) * WST, gcx, gcy, gcz, gr, u);
+            if (!has) gcx = gcy = gcz = gr = 0.f;
+            acc.x += gcx;
+            acc.y += gcy;
+            acc.z += gcz;
+            acc.w += gr;
+            if (want_pts) {
+                for (int o = 1; o < width; o <<= 1) {
+                    gcx += __shfl_xor_sync(0xffffffffu, gcx, o);
+                    gcy += __shfl_xor_sync(0xffffffffu, gcy, o);
+                    gcz += __shfl_xor_sync(0xffffffffu, gcz, o);
+                }
+                // lane t + i takes the sum its sub-group i holds
+                const int src = ((lane - t) & (stride - 1)) * width;
+                const float x = __shfl_sync(0xffffffffu, gcx, src), y = __shfl_sync(0xffffffffu, gcy, src),
+                            z = __shfl_sync(0xffffffffu, gcz, src);
+                if (lane >= t && lane < t + stride) {
+                    gp[0] -= x;
+                    gp[1] -= y;
+                    gp[2] -= z;
+                }
+            }
+        }
+        for (int o = width; o < 32; o <<= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+            acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+        }
+        if (has && sub == 0) {
+            float4 v = acc_row[j];
+            v.x += acc.x;
+            v.y += acc.y;
+            v.z += acc.z;
+            v.w += acc.w;
+            acc_row[j] = v;
+        }
+    }
+    const int64_t p = tile * kTile + warp * kWarpPoints + lane;
+    if (want_pts && lane < kWarpPoints && p < a.n_points) {
+        a.d_points[3 * p] = gp[0];
+        a.d_points[3 * p + 1] = gp[1];
+        a.d_points[3 * p + 2] = gp[2];
+    }
+}
+
+// One tile: tail adjoint, then the pair adjoints.  A warp reads only the rows
+// it wrote, so warps need no block barrier between the two.  With a workspace
+// the two run as launches of their own (kPhaseTail stores the coefficients in
+// dfp_ws, kPhasePairs reads them), each of which keeps to one region of code:
+// as one launch (kPhaseBoth, for callers without a workspace) the kernel waits
+// on instruction fetch (1.1 stalled warps per issue; 1M points, 300 spheres, 8
+// bands: 10.5 ms against 4.0 + 5.4 ms).
+constexpr int kPhaseBoth = 0, kPhaseTail = 1, kPhasePairs = 2;
+
+template <bool EXP, bool CULL, int PHASE>
+__device__ __forceinline__ void lp_backward_tile(const BwdArgs& a, const BwdShared& sh, int64_t tile) {
+    const LanePair lp = lane_pair();
+    const int row = threadIdx.x >> 1;
+    const int64_t p = tile * kTile + row;
+    const bool live = p < a.n_points;
+    const bool pairs = a.d_centers || a.d_radii || a.d_points;
+    float dfp[NS];
+    if constexpr (PHASE == kPhasePairs) {
+        lp_load(a.dfp_ws, a.n_points, live ? p : 0, live, lp, dfp);
+    } else {
+        lp_tail_adjoint<EXP, CULL>(a, sh, p, dfp);
+    }
+    if constexpr (PHASE == kPhaseTail) {
+        if (pairs && live) lp_store(dfp, a.n_points, p, lp, a.dfp_ws);
+        return;
+    }
+    if (!pairs) return;
+    __syncwarp();   // the region held the tail's operands
+    lp_store_row(dfp, sh.w + (row >> 4) * sh.region + (row & 15) * WST, lp);
+    if (!lp.odd) {
+        const int64_t q = live ? p : 0;
+        sh.pt[row] = make_float4(load_or(a.points, 3 * q, live), load_or(a.points, 3 * q + 1, live),
+                                 load_or(a.points, 3 * q + 2, live), 0.f);
+        if (CULL) {
+            const Normal u = unit_normal(load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
+                                         load_or(a.normals, 3 * q + 2, live));
+            sh.nrm[row] = make_float4(u.x, u.y, u.z, 0.f);
+        }
+    }
+    __syncwarp();
+    lp_pairs<CULL>(a, sh, tile);
+    __syncwarp();
+}
+
+// Block total of entry e of the scene-level sums (d_light, loss, spheres).
+__device__ __forceinline__ float lp_block_sum(const BwdShared& sh, int N, int e) {
+    float v = 0.f;
+    if (e < 3 * K) {
+        const int c = e / K, i = e % K;
+        int l = 0;
+        while ((l + 1) * (l + 1) <= i) ++l;
+        const int m = i - l * (l + 1), am = m < 0 ? -m : m, b = (l + am) & 1;
+        const int s = c * NS + lp_slot(am, m < 0, (l - am - b) >> 1);
+#pragma unroll
+        for (int w = 0; w < NWARP; ++w) v += sh.dl[w][b][s];
+    } else if (e == 3 * K) {
+#pragma unroll
+        for (int w = 0; w < NWARP; ++w) v += sh.loss[w];
+    } else {
+        const int q = e - (3 * K + 1);
+        const float* acc = reinterpret_cast<const float*>(sh.acc);
+#pragma unroll
+        for (int w = 0; w < NWARP; ++w) v += acc[w * 4 * N + q];
+    }
+    return v;
+}
+
+#define SHS_LP_BWD_SHARED(EXP, PHASE)                                                        \
+    extern __shared__ __align__(16) float4 dyn[];                                            \
+    __shared__ __align__(16) float s_light[3 * KPAD];                                        \
+    __shared__ __align__(16) float s_lt[2][3][NSP];                                          \
+    __shared__ __align__(16) float s_leg[kLegProduct + ((EXP) ? kLegExp : 0)];               \
+    __shared__ __align__(16) float s_w[NWARP * ((PHASE) == kPhasePairs ? kWarpPoints * WST : kWarpRegion)];                 \
+    __shared__ __align__(16) float4 s_pt[(PHASE) == kPhaseTail ? 1 : kTile], s_nrm[(PHASE) == kPhaseTail ? 1 : kTile]; \
+    __shared__ float s_dl[NWARP][2][kDl], s_loss[NWARP];                                     \
+    __shared__ __align__(8) uint64_t s_bar;                                                  \
+    __shared__ bool s_last
+
+__device__ __forceinline__ void clear_sums(const BwdShared& sh, int N) {
+    float* acc = reinterpret_cast<float*>(sh.acc);
+    for (int e = threadIdx.x; e < NWARP * 4 * N; e += kBlock) acc[e] = 0.f;
+    for (int e = threadIdx.x; e < NWARP * 2 * kDl; e += kBlock) (&sh.dl[0][0][0])[e] = 0.f;
+    if (threadIdx.x < NWARP) sh.loss[threadIdx.x] = 0.f;
+}
+
+// Layout of one block's reduced scene gradient (E floats):
+//   [0, 3K)          d_light, channel-major
+//   [3K]             loss
+//   [3K+1, 3K+1+4N)  per sphere (d cx, d cy, d cz, d r)
+template <bool EXP, bool CULL, int PHASE>
+__global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_lp_kernel(BwdArgs a) {
+    SHS_LP_BWD_SHARED(EXP, PHASE);
+    const int N = a.sc.n_spheres;
+    const BwdShared sh{dyn, dyn + N, s_lt, s_leg, s_dl, s_loss, s_w, PHASE == kPhasePairs ? kWarpPoints * WST : kWarpRegion,
+                       s_pt, s_nrm};
+    if (PHASE != kPhasePairs) load_rules(s_leg, EXP);
+    if (!stage_scene(a.sc, sh.sph, s_light, &s_bar)) return;
+    clear_sums(sh, PHASE == kPhaseTail ? 0 : N);
+    slot_lighting(s_light, s_lt);
+
+    const int64_t ntiles = (a.n_points + kTile - 1) / kTile;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+        lp_backward_tile<EXP, CULL, PHASE>(a, sh, tile);
+
+    // ---- block reduction of the phase's entries, then one scene-level
+    // reduction (by the last launch)
+    __syncthreads();
+    const int E = 3 * K + 1 + 4 * N, begin = PHASE == kPhasePairs ? 3 * K + 1 : 0,
+              end = PHASE == kPhaseTail ? 3 * K + 1 : E;
+    float* out = a.partials + static_cast<size_t>(blockIdx.x) * a.partial_stride;
+    const bool det = a.counter == nullptr;
+    for (int e = begin + threadIdx.x; e < end; e += kBlock) {
+        const float v = lp_block_sum(sh, N, e);
+        if (det) out[e] = v;
+        else atomicAdd(a.partials + e, v);
+    }
+    if (det || PHASE == kPhaseTail) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    finish_scene_sums(a, E);
+}
+
+// ---------------------------------------------------------------------------
+// batched persistent kernel (serving): many requests, one launch
+// ---------------------------------------------------------------------------
+
+// Adjoint for every tile of every request in the batch.  Each tile's scene
+// sums go to its request's accumulator with atomics; the tile that completes a
+// request writes that request's outputs.
+template <bool EXP, bool CULL>
+__global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_batch_kernel(const __grid_constant__ BwdBatch b) {
+    SHS_LP_BWD_SHARED(EXP, kPhaseBoth);
+    __shared__ long long s_tile;
+    const BwdShared sh{dyn, dyn + b.max_spheres, s_lt, s_leg, s_dl, s_loss, s_w, kWarpRegion, s_pt, s_nrm};
+    load_rules(s_leg, EXP);
+    mbar_init(&s_bar);
+    int staged = -1;
+    uint32_t parity = 0;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = static_cast<long long>(atomicAdd(b.queue, 1u));
+        __syncthreads();
+        const int64_t tile = s_tile;
+        if (tile >= b.total_tiles) break;
+        const int r = find_request(b.tile_begin, b.n, tile);
+        const BwdArgs& a = b.r[r];
+        const int N = a.sc.n_spheres;
+        if (r != staged) {
+            if (!stage_copy(a.sc, sh.sph, s_light, &s_bar, parity)) return;
+            parity ^= 1u;
+            staged = r;
+            slot_lighting(s_light, s_lt);
+        }
+        clear_sums(sh, N);
+        __syncthreads();
+        lp_backward_tile<EXP, CULL, kPhaseBoth>(a, sh, tile - b.tile_begin[r]);
+        __syncthreads();
+        const int E = 3 * K + 1 + 4 * N;
+        for (int e = threadIdx.x; e < E; e += kBlock) atomicAdd(a.partials + e, lp_block_sum(sh, N, e));
+        __threadfence();
+        __syncthreads();
+        const int64_t ntiles_r = b.tile_begin[r + 1] - b.tile_begin[r];
+        if (threadIdx.x == 0) s_last = atomicAdd(a.counter, 1u) == static_cast<unsigned>(ntiles_r - 1);
+        __syncthreads();
+        if (s_last) finish_scene_sums(a, E);
+    }
+}
+
+size_t backward_dyn_smem(int n_spheres) { return static_cast<size_t>(n_spheres) * 16u * (1 + NWARP); }
+
+// The tail launch stages the spheres only to recompute f; it has no sphere sums.
+size_t phase_dyn_smem(int phase, int n_spheres) {
+    return phase == kPhaseTail ? static_cast<size_t>(n_spheres) * 16u : backward_dyn_smem(n_spheres);
+}
+
+template <bool EXP, bool CULL, int PHASE>
+cudaError_t launch_backward_lp(const BwdArgs& a, int grid, cudaStream_t s) {
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(backward_lp_kernel<EXP, CULL, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(phase_dyn_smem(PHASE, kMaxSpheres)));
+    if (attr != cudaSuccess) return attr;
+    backward_lp_kernel<EXP, CULL, PHASE>
+        <<<static_cast<unsigned>(grid), kBlock, phase_dyn_smem(PHASE, a.sc.n_spheres), s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
+template <int PHASE>
+cudaError_t launch_phase(const BwdArgs& a, int grid, cudaStream_t s) {
+    const bool cull = a.sc.horizon_cull != 0, exp1 = PHASE != kPhasePairs && a.sc.exp_mode == 1;
+    if (exp1) {
+        return cull ? launch_backward_lp<PHASE != kPhasePairs, true, PHASE>(a, grid, s)
+                    : launch_backward_lp<PHASE != kPhasePairs, false, PHASE>(a, grid, s);
+    }
+    return cull ? launch_backward_lp<false, true, PHASE>(a, grid, s) : launch_backward_lp<false, false, PHASE>(a, grid, s);
+}
+
+template <int PHASE>
+int phase_blocks(int n_spheres) {
+    cudaFuncSetAttribute(backward_lp_kernel<false, false, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         static_cast<int>(phase_dyn_smem(PHASE, kMaxSpheres)));
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, backward_lp_kernel<false, false, PHASE>, kBlock,
+                                                      phase_dyn_smem(PHASE, n_spheres)) != cudaSuccess || nb < 1)
+        nb = 1;
+    return nb;
+}
+
+template <bool EXP, bool CULL>
+cudaError_t launch_backward_batch_lp(const BwdBatch& b, cudaStream_t s) {
+    const size_t smem = backward_dyn_smem(b.max_spheres);
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(backward_batch_kernel<EXP, CULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(backward_dyn_smem(kMaxSpheres)));
+    if (attr != cudaSuccess) return attr;
+    int grid = 0;
+    const cudaError_t e = one_wave(backward_batch_kernel<EXP, CULL>, smem, b.total_tiles, &grid);
+    if (e != cudaSuccess) return e;
+    backward_batch_kernel<EXP, CULL><<<grid, kBlock, smem, s>>>(b);
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+template <>
+BwdBlocks backward_blocks_per_sm<NB>(int n_spheres) {
+    return BwdBlocks{phase_blocks<kPhaseBoth>(n_spheres), phase_blocks<kPhaseTail>(n_spheres),
+                     phase_blocks<kPhasePairs>(n_spheres)};
+}
+
+template <>
+cudaError_t launch_backward_batch<NB>(const BwdBatch& b, cudaStream_t s) {
+    if (b.total_tiles <= 0) return cudaSuccess;
+    switch (b.variant) {
+        case 0: return launch_backward_batch_lp<false, false>(b, s);
+        case 1: return launch_backward_batch_lp<false, true>(b, s);
+        case 2: return launch_backward_batch_lp<true, false>(b, s);
+        default: return launch_backward_batch_lp<true, true>(b, s);
+    }
+}
+
+template <>
+cudaError_t launch_backward<NB>(const BwdArgs& a, cudaStream_t s) {
+    if (a.n_points <= 0) return cudaSuccess;
+    cudaError_t err = cudaSuccess;
+    if (a.dfp_ws) {
+        if (a.tail_grid) err = launch_phase<kPhaseTail>(a, a.tail_grid, s);   // else: ran on the tensor cores
+        const bool need_pairs = a.d_centers || a.d_radii || a.d_points;
+        if (err == cudaSuccess && (need_pairs || a.counter != nullptr)) err = launch_phase<kPhasePairs>(a, a.grid, s);
+    } else {
+        err = launch_phase<kPhaseBoth>(a, a.grid, s);
+    }
+    if (err != cudaSuccess || a.counter != nullptr) return err;
+    const int E = 3 * K + 1 + 4 * a.sc.n_spheres;
+    reduce_partials_kernel<<<(E + 31) / 32, 32 * kReduceWarps, 0, s>>>(a, a.dfp_ws && a.tail_grid ? a.tail_grid : a.grid,
+                                                                       a.grid);
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace shs

@@ -7,7 +7,9 @@
 
 namespace shs {
 
-constexpr int kBlock = 128;          // threads per block, one shading point each
+constexpr int kBlock = 128;          // threads per block
+// Points per block: two lanes share a point from 6 bands.
+constexpr int tile_points(int n_bands) { return n_bands >= 6 ? kBlock / 2 : kBlock; }
 constexpr int kMaxSpheres = 1024;    // spheres staged in shared memory at once
 constexpr int kMaxK = 16;            // cap on the number of squarings
 
@@ -64,20 +66,31 @@ struct BwdArgs {
     float* d_radii;
     float* d_points;
     float* d_normals;
-    float* dfp_ws;           // [K][P] pair-adjoint coefficients (split backward, >= 6 bands)
+    float* dfp_ws;           // [K][P] pair-adjoint coefficients between the tail's launch and the pair
+                             // pass (from 6 bands), or null: one launch
     float* partials;         // [grid][stride] scratch
     unsigned int* counter;   // scratch, zero between launches
     int partial_stride;
-    int grid;                // persistent grid size
-    int skip_tail;           // split backward: dfp_ws and the lighting / loss rows are already written
+    int grid;                // persistent grid size (of the pair pass when there are two launches)
+    int tail_grid;           // grid of the tail's launch; 0: the tail ran before (tensor cores), its coefficients
+                             // and lighting / loss rows are written
 };
 
 // A batch: up to kMaxBatch requests (of one band count) whose 128-point tiles
 // form one work list; a persistent grid pulls tiles from a device counter.
 constexpr int kMaxBatch = 32;
 
+// From 6 bands the requests of one batch kernel also share a variant (bit 0:
+// horizon culling, bit 1: projected exponential), which the kernel is compiled
+// for.
+constexpr int batch_variants(int n_bands) { return n_bands >= 6 ? 4 : 1; }
+inline int batch_variant(const SceneView& sc, int n_bands) {
+    return n_bands >= 6 ? (sc.horizon_cull ? 1 : 0) + (sc.exp_mode == 1 ? 2 : 0) : 0;
+}
+
 struct FwdBatch {
     int n;
+    int variant;
     int64_t total_tiles;
     int64_t tile_begin[kMaxBatch + 1];   // prefix sums of tiles per request
     unsigned int* queue;                  // zero before launch
@@ -86,6 +99,7 @@ struct FwdBatch {
 
 struct BwdBatch {
     int n;
+    int variant;
     int max_spheres;
     int64_t total_tiles;
     int64_t tile_begin[kMaxBatch + 1];
@@ -146,7 +160,12 @@ template <int NB> cudaError_t launch_forward_batch(const FwdBatch& b, cudaStream
 template <int NB> cudaError_t launch_backward_batch(const BwdBatch& b, cudaStream_t s);
 template <int NB> cudaError_t launch_forward(const FwdArgs& a, cudaStream_t s);
 template <int NB> cudaError_t launch_backward(const BwdArgs& a, cudaStream_t s);
-template <int NB> int backward_blocks_per_sm(int n_spheres);
+// Resident blocks per SM of the adjoint kernels: as one launch, and (from 6
+// bands) of the tail's and the pair pass's own launches.
+struct BwdBlocks {
+    int both, tail, pairs;
+};
+template <int NB> BwdBlocks backward_blocks_per_sm(int n_spheres);
 cudaError_t launch_pack_spheres(const float* centers, const float* radii, float4* out, int n,
                                 bool has_c, bool has_r, cudaStream_t s);
 

@@ -162,7 +162,8 @@ extern "C" shs_status shs_shade_backward_noalloc(
     a.partials = acc;            // one accumulator, finished by the last block
     a.counter = counter;
     a.partial_stride = E;
-    const int64_t tiles = (n_points + shs::kBlock - 1) / shs::kBlock;
+    const int per_tile = shs::tile_points(cfg->n_bands);
+    const int64_t tiles = (n_points + per_tile - 1) / per_tile;
     const int64_t max_grid = static_cast<int64_t>(sms) * shs::backward_blocks_per_sm_nb(cfg->n_bands, n_spheres);
     a.grid = static_cast<int>(tiles < max_grid ? tiles : max_grid);
     e = shs::launch_backward_nb(cfg->n_bands, a, s);

@@ -1,0 +1,229 @@
+// Shared by the kernels of every band count: staging of a scene into shared
+// memory, the geometry of a point-sphere pair, and the scene-level sums'
+// finish.  Included by translation units compiled with -DSHS_NB=n.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "generated/shs_sh_gen.cuh"
+#include "shs_internal.h"
+
+#ifndef SHS_NB
+#error "compile with -DSHS_NB=<n_bands>"
+#endif
+
+namespace shs {
+namespace {
+
+constexpr int NB = SHS_NB;
+constexpr int K = NB * NB;
+constexpr int KPAD = (K + 3) / 4 * 4;
+constexpr int NWARP = kBlock / 32;
+using SH = shsgen::SH<NB>;
+
+
+__host__ __device__ constexpr int band_of(int i) {
+    int l = 0;
+    while ((l + 1) * (l + 1) <= i) ++l;
+    return l;
+}
+
+__device__ __forceinline__ float fast_sqrt(float x) {   // sqrt(x) = x / sqrt(x), x >= 0
+    return x * rsqrtf(fmaxf(x, 1e-30f));
+}
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+__device__ __forceinline__ uint64_t global_ns() {
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// One mbarrier per block tracks the bulk copies that stage a scene (sphere
+// array + lighting) into shared memory.  Initialise it once per block.
+__device__ void mbar_init(uint64_t* bar) {
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncthreads();
+}
+
+// Stage a scene with bulk asynchronous copies completing on `bar` (phase
+// `parity`, alternating between stagings).  Every thread waits with a bound of
+// about one second; the result is block-uniform: false means the copy did not
+// complete, the status word is set and the block must not use the data.  The
+// caller must have synchronised the block if shared memory held a previous
+// scene that threads may still read.
+__device__ bool stage_copy(const SceneView& sc, float4* s_sph, float* s_light, uint64_t* bar,
+                           uint32_t parity) {
+    const uint32_t sph_bytes = static_cast<uint32_t>(sc.n_spheres) * 16u;
+    const uint32_t light_bytes = 3u * KPAD * 4u;
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                     ::"r"(smem_addr(bar)), "r"(sph_bytes + light_bytes) : "memory");
+        if (sph_bytes)
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                ::"r"(smem_addr(s_sph)), "l"(sc.spheres), "r"(sph_bytes), "r"(smem_addr(bar))
+                : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+            ::"r"(smem_addr(s_light)), "l"(sc.light), "r"(light_bytes), "r"(smem_addr(bar))
+            : "memory");
+    }
+    bool done = false;
+    const uint64_t t0 = global_ns();
+    for (uint32_t it = 0; it < (1u << 26) && !done; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            " selp.b32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+        done = ok != 0;
+        if (!done && global_ns() - t0 > 1000000000ull) break;
+    }
+    const bool any_failed = __syncthreads_or(!done);
+    if (any_failed && threadIdx.x == 0) atomicExch(sc.status, kDevTimeout);
+    return !any_failed;
+}
+
+__device__ bool stage_scene(const SceneView& sc, float4* s_sph, float* s_light, uint64_t* bar) {
+    mbar_init(bar);
+    return stage_copy(sc, s_sph, s_light, bar, 0u);
+}
+
+struct PairGeom {
+    float dx, dy, dz, invD, invD2, s2, c;
+    bool open;
+};
+
+// Unit normal of the shading point, used by horizon culling.
+struct Normal {
+    float x = 0.f, y = 0.f, z = 0.f;
+};
+
+__device__ __forceinline__ Normal unit_normal(float nx, float ny, float nz) {
+    const float n2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
+    const float il = n2 > 0.f ? rsqrtf(n2) : 0.f;
+    return Normal{nx * il, ny * il, nz * il};
+}
+
+// With CULL (the optional horizon-culling reading), a sphere entirely below
+// the tangent plane at x, (c - x) . n_hat < -r, becomes an empty cap: s2 = 0
+// and c = 1 make every G_l zero, and a closed cap carries no gradient.
+template <bool CULL = false>
+__device__ __forceinline__ PairGeom pair_geometry(float px, float py, float pz, float4 sp, Normal u = {}) {
+    PairGeom g;
+    g.dx = sp.x - px;
+    g.dy = sp.y - py;
+    g.dz = sp.z - pz;
+    const float D2 = fmaf(g.dx, g.dx, fmaf(g.dy, g.dy, g.dz * g.dz));
+    g.invD = D2 > 0.f ? rsqrtf(D2) : 0.f;     // D = 0: every term below vanishes
+    g.invD2 = g.invD * g.invD;
+    const float r2i = sp.w * sp.w * g.invD2;
+    g.open = r2i < 1.f;
+    g.s2 = fminf(r2i, 1.f);                   // point inside the sphere: hemisphere cap
+    g.c = fast_sqrt(1.f - g.s2);
+    if constexpr (CULL) {
+        if (fmaf(g.dx, u.x, fmaf(g.dy, u.y, g.dz * u.z)) < -sp.w) {
+            g.s2 = 0.f;
+            g.c = 1.f;
+            g.open = false;
+        }
+    }
+    return g;
+}
+
+__device__ __forceinline__ float load_or(const float* p, int64_t i, bool live) {
+    return live ? __ldg(p + i) : 0.f;
+}
+
+// Parts of the forward pass a kernel runs: everything; the log-visibility f
+// only, stored; or, from a stored f, the exponential and shading.
+constexpr int kFwdFull = 0, kFwdPairs = 1, kFwdTail = 2;
+
+// The last contributor copies the accumulated scene-level sums to the
+// outputs and re-zeroes the accumulator and its counter for the next launch.
+__device__ void finish_scene_sums(const BwdArgs& a, int E) {
+    __threadfence();
+    for (int e = threadIdx.x; e < E; e += kBlock) {
+        const float v = __ldcg(a.partials + e);
+        a.partials[e] = 0.f;
+        if (e < 3 * K) {
+            if (a.d_light) a.d_light[e] = v;
+        } else if (e == 3 * K) {
+            if (a.loss) *a.loss = v;
+        } else {
+            const int s = e - (3 * K + 1), j = s >> 2, comp = s & 3;
+            if (comp < 3) {
+                if (a.d_centers) a.d_centers[3 * j + comp] = v;
+            } else if (a.d_radii) {
+                a.d_radii[j] = v;
+            }
+        }
+    }
+    if (threadIdx.x == 0) *a.counter = 0u;
+}
+
+__device__ __forceinline__ int find_request(const int64_t* tb, int n, int64_t tile) {
+    int r = 0;
+    while (r + 1 < n && tile >= tb[r + 1]) ++r;
+    return r;
+}
+
+// Deterministic finish: fixed-order sum of the blocks' partial rows (the
+// lighting and loss entries and the sphere entries may come from launches with
+// different grids).  One block per 32 entries;
+// its 32 warps stride over the rows with four independent loads in flight
+// each (the sum is latency-bound: ~450 rows of 32 floats per block).
+constexpr int kReduceWarps = 32;
+
+__global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(BwdArgs a, int light_rows,
+                                                                            int sphere_rows) {
+    __shared__ float s[kReduceWarps][33];
+    const int N = a.sc.n_spheres;
+    const int E = 3 * K + 1 + 4 * N;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
+    float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
+    const int nblk = e <= 3 * K ? light_rows : sphere_rows;
+    if (e < E) {
+        const float* col = a.partials + e;
+        const size_t st = static_cast<size_t>(a.partial_stride);
+        int b = warp;
+        for (; b + 3 * kReduceWarps < nblk; b += 4 * kReduceWarps) {
+            v0 += __ldcg(col + b * st);
+            v1 += __ldcg(col + (b + kReduceWarps) * st);
+            v2 += __ldcg(col + (b + 2 * kReduceWarps) * st);
+            v3 += __ldcg(col + (b + 3 * kReduceWarps) * st);
+        }
+        for (; b < nblk; b += kReduceWarps) v0 += __ldcg(col + b * st);
+    }
+    s[warp][lane] = (v0 + v1) + (v2 + v3);
+    __syncthreads();
+    if (warp != 0 || e >= E) return;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < kReduceWarps; ++w) t += s[w][lane];
+    if (e < 3 * K) {
+        if (a.d_light) a.d_light[e] = t;
+    } else if (e == 3 * K) {
+        if (a.loss) *a.loss = t;
+    } else {
+        const int q = e - (3 * K + 1), j = q >> 2, comp = q & 3;
+        if (comp < 3) {
+            if (a.d_centers) a.d_centers[3 * j + comp] = t;
+        } else if (a.d_radii) {
+            a.d_radii[j] = t;
+        }
+    }
+}
+
+}  // namespace
+}  // namespace shs

@@ -1,0 +1,82 @@
+"""Kernels of 6 to 8 bands (a lane pair per point, one sphere per lane in the
+pair adjoint) at the edges of their tiles: 64-point tiles, 16 points per warp,
+8 / 16 / 32 spheres per warp step, against the FP64 oracle; every variant of
+the batched kernels against the single calls."""
+
+import ctypes
+
+import numpy as np
+import pytest
+
+from oracle import shs_oracle as O
+from paper_2104_00359_gb300 import synthetic as S
+
+from gpu_helpers import FIELDS, GRADS, gpu_run, grad_err, rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+def _tol(n):
+    return 1e-4 if n < 7 else 3e-4   # float32 gradients from 7 bands (squarings double the rounding error)
+
+
+@pytest.mark.parametrize("n", [6, 7, 8])
+@pytest.mark.parametrize("points,spheres", [(1, 1), (15, 7), (16, 8), (17, 9), (63, 16), (64, 17), (65, 31), (127, 32),
+                                            (129, 33), (70, 65)])
+def test_tile_edges(n, points, spheres):
+    sc = S.random_scene(9000 + 100 * n + points, points, spheres, n, inside_fraction=0.0)
+    cfg = O.Config(n_bands=n)
+    dB = np.random.default_rng(points).normal(size=(points, 3)).astype(np.float32)
+    for saved in (True, False):
+        B, k, f, g, status = gpu_run(sc, cfg, dB=dB, saved=saved)
+        assert status == 0
+        args = [sc[x] for x in FIELDS]
+        ref = O.shade_backward(cfg, *args, dB, k=k)
+        assert rel_err(B, ref["forward"]["radiance"]).max() <= 1e-4
+        for name in GRADS:
+            err = grad_err(name, g[name], ref)
+            assert err.max() <= _tol(n), f"{name}: {err.max():.3e}"
+
+
+@pytest.mark.parametrize("n", [6, 8])
+def test_batch_variants_match_single_calls(n):
+    """One batch over the four kernel variants (horizon culling x projected
+    exponential) and two sizes; float32 sums in another order only."""
+    import torch
+    from paper_2104_00359_gb300 import Config, Scene, _lib
+    dev = torch.device("cuda:0")
+    lib = _lib.load()
+    jobs = []
+    for i, (cull, mode, P, N) in enumerate([(0, 0, 130, 33), (1, 0, 64, 9), (0, 1, 65, 20), (1, 1, 200, 5),
+                                            (0, 0, 1, 1), (1, 1, 63, 40)]):
+        sc = S.random_scene(9900 + i, P, N, n)
+        T = {k: torch.from_numpy(sc[k]).to(dev) for k in FIELDS}
+        T["target"] = torch.rand((P, 3), device=dev, generator=torch.Generator(dev).manual_seed(i))
+        cfg = Config(n_bands=n, horizon_cull=bool(cull), exp_mode=mode)
+        single = Scene(T["centers"], T["radii"], T["light"], cfg)
+        sv = single.new_saved(P, dev)
+        B = single.shade(T["points"], T["normals"], T["albedo"], saved=sv)
+        g = single.backward_l2(T["points"], T["normals"], T["albedo"], B, T["target"], saved=sv)
+        batched = Scene(T["centers"], T["radii"], T["light"], cfg)
+        out = dict(radiance=torch.zeros((P, 3), device=dev), saved=batched.new_saved(P, dev),
+                   loss=torch.zeros((), device=dev), **batched._grad_buffers(P, dev, batched.ALL))
+        r = _lib.ShsRequest()
+        r.scene, r.n_points = batched.handle.value, P
+        for k in ("points", "normals", "albedo", "target"):
+            setattr(r, k, T[k].data_ptr())
+        for k, v in out.items():
+            setattr(r, k, v.data_ptr())
+        jobs.append((r, B, g, out, (T, single, batched)))
+    h = ctypes.c_void_p()
+    _lib.check(lib.shs_batch_create(ctypes.byref(h)), "shs_batch_create")
+    arr = (_lib.ShsRequest * len(jobs))(*[j[0] for j in jobs])
+    for _ in range(2):   # the accumulators are clean again for a second call
+        _lib.check(lib.shs_shade_batch(h, arr, len(jobs), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)),
+                   "shs_shade_batch")
+        torch.cuda.synchronize()
+        for r, B, g, out, _ in jobs:
+            assert torch.equal(out["radiance"], B)
+            for k in ("loss",) + GRADS:
+                x, y = out[k].double(), g[k].double()
+                assert (x - y).abs().max() <= 2e-6 * max(float(y.abs().max()), 1e-6), k
+    _lib.check(lib.shs_batch_destroy(h), "shs_batch_destroy")
