@@ -124,6 +124,12 @@ shs_status shs_scene_create(const shs_config* cfg, int32_t n_spheres,
 shs_status shs_scene_update(shs_scene_t scene, const float* centers,
                             const float* radii, const float* light, void* stream);
 
+/* The same for n_scenes scenes of one sphere and band count in one launch (per
+ * 32 scenes): centers [n_scenes][N][3]; radii [N] and light [3,K] shared by
+ * all; NULL = unchanged. */
+shs_status shs_scenes_update(const shs_scene_t* scenes, int32_t n_scenes, const float* centers,
+                             const float* radii, const float* light, void* stream);
+
 /* Optimal linear step of the SH exponential (Sec. 3.3.2, after Ren et al.'s
  * scaling / squaring setting): with g the scaled exponent (zero DC) and
  * s = |g| its coefficient norm, exp*(g) ~ a(s) sqrt(4 pi) e_0 + b(s) g.

@@ -11,6 +11,8 @@ import ctypes
 import os
 from ctypes import POINTER, c_char_p, c_float, c_int32, c_int64, c_size_t, c_void_p
 
+import torch
+
 LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "lib", "libshshadow.so")
 
 SHS_OK = 0
@@ -54,6 +56,7 @@ _SIGS = {
     "shs_scene_create": (c_int32, [POINTER(ShsConfig), c_int32, c_void_p, c_void_p, c_void_p, c_void_p,
                                    POINTER(c_void_p)]),
     "shs_scene_update": (c_int32, [c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]),
+    "shs_scenes_update": (c_int32, [POINTER(c_void_p), c_int32, c_void_p, c_void_p, c_void_p, c_void_p]),
     "shs_scene_set_ol_table": (c_int32, [c_void_p, _F, c_int32, c_float]),
     "shs_scene_destroy": (c_int32, [c_void_p]),
     "shs_scene_info": (c_int32, [c_void_p, POINTER(ShsConfig), POINTER(c_int32)]),
@@ -126,5 +129,13 @@ def check(status, where):
 
 
 def ptr(t):
-    """Device (or host) address of a tensor, or None."""
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    """Device (or host) address of a tensor, or None (the declared argument
+    types turn it into a pointer)."""
+    return None if t is None else t.data_ptr()
+
+
+def current_stream(index=None):
+    """Handle of torch's current stream on device ``index`` (default: the
+    current device), without building a torch.cuda.Stream object (0.1 against
+    3 us per call)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice() if index is None else index)

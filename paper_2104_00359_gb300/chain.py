@@ -18,18 +18,14 @@ import ctypes
 import torch
 
 from . import _lib
-from ._lib import check, ptr
+from ._lib import check, current_stream, ptr
 from .shade import Scene, shade
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-
-
 def _dev(t, name):
-    if not (t.is_cuda and t.dtype == torch.float32):
+    if not (t.is_cuda and t.dtype is torch.float32):
         raise TypeError(f"{name} must be a float32 CUDA tensor")
-    return t.contiguous()
+    return t if t.is_contiguous() else t.contiguous()
 
 
 class DeformPose(torch.autograd.Function):
@@ -40,14 +36,14 @@ class DeformPose(torch.autograd.Function):
     @staticmethod
     def forward(ctx, base, basis, p, pose, direction):
         lib = _lib.load()
-        base, basis, p, pose = (_dev(t.detach(), n) for t, n in
+        base, basis, p, pose = (_dev(t, n) for t, n in
                                 ((base, "base"), (basis, "basis"), (p, "p"), (pose, "pose")))
         M, D = int(base.shape[0]), int(p.shape[0])
         if tuple(basis.shape) != (M, 3, D) or tuple(pose.shape) != (6,):
             raise ValueError(f"basis {tuple(basis.shape)} / pose {tuple(pose.shape)} do not match M={M}, D={D}")
         x = torch.empty((M, 3), dtype=torch.float32, device=base.device)
         check(lib.shs_chain_forward(ptr(base), ptr(basis), M, D, ptr(p), ptr(pose), int(direction), None, ptr(x),
-                                    _stream()), "shs_chain_forward")
+                                    current_stream()), "shs_chain_forward")
         ctx.save_for_backward(base, basis, p, pose)
         ctx.direction = int(direction)
         return x
@@ -63,7 +59,7 @@ class DeformPose(torch.autograd.Function):
         nbytes = int(lib.shs_chain_workspace_bytes(M, D))
         ws = torch.empty((max(nbytes, 16) + 3) // 4, dtype=torch.float32, device=base.device)
         check(lib.shs_chain_backward(ptr(base), ptr(basis), M, D, ptr(p), ptr(pose), ctx.direction, ptr(dx),
-                                     ptr(d_p), ptr(d_pose), ptr(ws), ws.numel() * 4, _stream()),
+                                     ptr(d_p), ptr(d_pose), ptr(ws), ws.numel() * 4, current_stream()),
               "shs_chain_backward")
         return None, None, d_p, d_pose, None
 
@@ -129,14 +125,14 @@ class DeformPoseViews(torch.autograd.Function):
     @staticmethod
     def forward(ctx, base, basis, p, poses, direction):
         lib = _lib.load()
-        base, basis, p, poses = (_dev(t.detach(), n) for t, n in
+        base, basis, p, poses = (_dev(t, n) for t, n in
                                  ((base, "base"), (basis, "basis"), (p, "p"), (poses, "poses")))
         M, D, V = int(base.shape[0]), int(p.shape[0]), int(poses.shape[0])
         if tuple(basis.shape) != (M, 3, D) or tuple(poses.shape) != (V, 6):
             raise ValueError(f"basis {tuple(basis.shape)} / poses {tuple(poses.shape)} do not match M={M}, D={D}")
         x = torch.empty((V, M, 3), dtype=torch.float32, device=base.device)
         check(lib.shs_chain_forward_views(ptr(base), ptr(basis), M, D, ptr(p), ptr(poses), V, int(direction), None,
-                                          ptr(x), _stream()), "shs_chain_forward_views")
+                                          ptr(x), current_stream()), "shs_chain_forward_views")
         ctx.save_for_backward(base, basis, p, poses)
         ctx.direction = int(direction)
         return x
@@ -152,7 +148,7 @@ class DeformPoseViews(torch.autograd.Function):
         nbytes = int(lib.shs_chain_views_workspace_bytes(M, D, V))
         ws = torch.empty((max(nbytes, 16) + 3) // 4, dtype=torch.float32, device=base.device)
         check(lib.shs_chain_backward_views(ptr(base), ptr(basis), M, D, ptr(p), ptr(poses), V, ctx.direction,
-                                           ptr(dx), ptr(d_p), ptr(d_poses), ptr(ws), ws.numel() * 4, _stream()),
+                                           ptr(dx), ptr(d_p), ptr(d_poses), ptr(ws), ws.numel() * 4, current_stream()),
               "shs_chain_backward_views")
         return None, None, d_p, d_poses, None
 
@@ -195,9 +191,24 @@ class ViewBatch:
         except Exception:
             pass
 
+    def requests(self, pts, nrm, alb):
+        """One request per view over [V, P, 3] points and normals."""
+        arr = (_lib.ShsRequest * self.V)()
+        p, n, a, step = pts.data_ptr(), nrm.data_ptr(), alb.data_ptr(), self.P * 12
+        for v, r in enumerate(arr):
+            r.scene, r.n_points, r.saved = self.scenes[v].handle.value, self.P, self.saved[v].data_ptr()
+            r.points, r.normals, r.albedo = p + v * step, n + v * step, a
+        return arr
+
+    def update(self, centers, radii, light):
+        """Every view's sphere centres [V, N, 3], the shared radii and lighting."""
+        handles = (ctypes.c_void_p * self.V)(*[sc.handle.value for sc in self.scenes])
+        check(self.lib.shs_scenes_update(handles, self.V, ptr(centers), ptr(radii), ptr(light), current_stream()),
+              "shs_scenes_update")
+
     def run(self, reqs):
-        arr = (_lib.ShsRequest * len(reqs))(*reqs)
-        check(self.lib.shs_shade_batch(self.batch, arr, len(reqs), _stream()), "shs_shade_batch")
+        arr = reqs if isinstance(reqs, ctypes.Array) else (_lib.ShsRequest * len(reqs))(*reqs)
+        check(self.lib.shs_shade_batch(self.batch, arr, len(reqs), current_stream()), "shs_shade_batch")
 
 
 class ShadeViews(torch.autograd.Function):
@@ -207,20 +218,18 @@ class ShadeViews(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, points, normals, albedo, centers, radii, light, views):
-        V, P = views.V, views.P
-        pts, nrm = _dev(points.detach(), "points"), _dev(normals.detach(), "normals")
-        alb, ctr = _dev(albedo.detach(), "albedo"), _dev(centers.detach(), "centers")
-        rad_, lgt = _dev(radii.detach(), "radii"), _dev(light.detach(), "light")
-        for v, sc in enumerate(views.scenes):
-            sc.update(centers=ctr[v], radii=rad_, light=lgt)
+        V, P, N, K = views.V, views.P, views.N, views.K
+        pts, nrm, alb = _dev(points, "points"), _dev(normals, "normals"), _dev(albedo, "albedo")
+        ctr, rad_, lgt = _dev(centers, "centers"), _dev(radii, "radii"), _dev(light, "light")
+        for t, shape, name in ((ctr, (V, N, 3), "centers"), (rad_, (N,), "radii"), (lgt, (3, K), "light")):
+            if t.shape != shape and (N or t is lgt):
+                raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {shape}")
+        views.update(ctr, rad_, lgt)
         out = torch.empty((V, P, 3), dtype=torch.float32, device=pts.device)
-        reqs = []
-        for v, sc in enumerate(views.scenes):
-            r = _lib.ShsRequest()
-            r.scene, r.n_points = sc.handle.value, P
-            r.points, r.normals, r.albedo = pts[v].data_ptr(), nrm[v].data_ptr(), alb.data_ptr()
-            r.radiance, r.saved = out[v].data_ptr(), views.saved[v].data_ptr()
-            reqs.append(r)
+        reqs = views.requests(pts, nrm, alb)
+        base = out.data_ptr()
+        for v, r in enumerate(reqs):
+            r.radiance = base + v * P * 12
         views.run(reqs)
         ctx.save_for_backward(pts, nrm, alb)
         ctx.views = views
@@ -236,17 +245,14 @@ class ShadeViews(torch.autograd.Function):
         z = lambda *s: torch.empty(s, dtype=torch.float32, device=dev)
         g = dict(d_points=z(V, P, 3), d_normals=z(V, P, 3), d_albedo=z(V, P, 3), d_centers=z(V, max(N, 1), 3),
                  d_radii=z(V, max(N, 1)), d_light=z(V, 3, K))
-        reqs = []
-        for v, sc in enumerate(views.scenes):
-            r = _lib.ShsRequest()
-            r.scene, r.n_points = sc.handle.value, P
-            r.points, r.normals, r.albedo = pts[v].data_ptr(), nrm[v].data_ptr(), alb.data_ptr()
-            r.saved, r.d_radiance = views.saved[v].data_ptr(), dB[v].data_ptr()
-            r.d_light, r.d_albedo = g["d_light"][v].data_ptr(), g["d_albedo"][v].data_ptr()
-            r.d_points, r.d_normals = g["d_points"][v].data_ptr(), g["d_normals"][v].data_ptr()
-            if N:
-                r.d_centers, r.d_radii = g["d_centers"][v].data_ptr(), g["d_radii"][v].data_ptr()
-            reqs.append(r)
+        reqs = views.requests(pts, nrm, alb)
+        step = {k: t.stride(0) * 4 for k, t in g.items()}
+        base = {k: t.data_ptr() for k, t in g.items() if N or k not in ("d_centers", "d_radii")}
+        d = dB.data_ptr()
+        for v, r in enumerate(reqs):
+            r.d_radiance = d + v * P * 12
+            for k, b in base.items():
+                setattr(r, k, b + v * step[k])
         views.run(reqs)
         d_centers = g["d_centers"][:, :N] if N else None
         d_radii = g["d_radii"][:, :N].sum(0) if N else None

@@ -53,6 +53,33 @@ __global__ void pack_spheres_kernel(const float* c, const float* r, float4* out,
     if (has_r) v.w = r[j];
     out[j] = v;
 }
+
+// Spheres and lighting of up to kMaxBatch scenes of one size in one launch
+// (scene y of the grid): lighting rows go to Kpad floats, the padding stays.
+struct UpdateArgs {
+    const float* centers;   // [scene][n][3] or null
+    const float* radii;     // [n] or null
+    const float* light;     // [3][K] or null
+    int n, K, Kpad;
+    float4* spheres[kMaxBatch];
+    float* lights[kMaxBatch];
+};
+__global__ void update_scenes_kernel(const __grid_constant__ UpdateArgs a) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, v = blockIdx.y;
+    if (i < a.n && (a.centers || a.radii)) {
+        float4* s = a.spheres[v] + i;
+        float4 q = *s;
+        if (a.centers) {
+            const float* c = a.centers + (static_cast<size_t>(v) * a.n + i) * 3;
+            q.x = c[0];
+            q.y = c[1];
+            q.z = c[2];
+        }
+        if (a.radii) q.w = a.radii[i];
+        *s = q;
+    }
+    if (a.light && i < 3 * a.K) a.lights[v][i / a.K * a.Kpad + i % a.K] = a.light[i];
+}
 }  // namespace
 
 cudaError_t launch_pack_spheres(const float* centers, const float* radii, float4* out, int n,
@@ -536,16 +563,49 @@ shs_status shs_scene_create(const shs_config* cfg, int32_t n_spheres, const floa
     return SHS_OK;
 }
 
+static shs_status update_scenes(const shs_scene_t* scenes, int n_scenes, const float* centers, const float* radii,
+                                const float* light, cudaStream_t s) {
+    shs::UpdateArgs u;
+    const shs_scene_s* sc = scenes[0];
+    u.n = sc->n_spheres;
+    u.centers = u.n > 0 ? centers : nullptr;
+    u.radii = u.n > 0 ? radii : nullptr;
+    u.light = light;
+    u.K = sc->K;
+    u.Kpad = sc->Kpad;
+    for (int i = 0; i < n_scenes; ++i) {
+        u.spheres[i] = scenes[i]->spheres;
+        u.lights[i] = scenes[i]->light;
+    }
+    const int spheres = u.centers || u.radii ? u.n : 0, lights = light ? 3 * u.K : 0;
+    const int items = spheres > lights ? spheres : lights;
+    if (items == 0) return SHS_OK;
+    shs::update_scenes_kernel<<<dim3((items + 127) / 128, n_scenes), 128, 0, s>>>(u);
+    shs::count_launch();
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? SHS_OK : cuda_fail(e, "update scene");
+}
+
 shs_status shs_scene_update(shs_scene_t sc, const float* centers, const float* radii,
                             const float* light, void* stream) {
     if (!sc) return fail(SHS_ERR_INVALID_ARG, "scene is NULL");
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if ((centers || radii) && sc->n_spheres > 0) {
-        cudaError_t e = shs::launch_pack_spheres(centers, radii, sc->spheres, sc->n_spheres,
-                                                 centers != nullptr, radii != nullptr, s);
-        if (e != cudaSuccess) return cuda_fail(e, "pack spheres");
+    return update_scenes(&sc, 1, centers, radii, light, static_cast<cudaStream_t>(stream));
+}
+
+shs_status shs_scenes_update(const shs_scene_t* scenes, int32_t n_scenes, const float* centers, const float* radii,
+                             const float* light, void* stream) {
+    if (n_scenes < 0 || (n_scenes > 0 && !scenes)) return fail(SHS_ERR_INVALID_ARG, "bad scene list");
+    for (int i = 0; i < n_scenes; ++i) {
+        if (!scenes[i]) return fail(SHS_ERR_INVALID_ARG, "scene %d is NULL", i);
+        if (scenes[i]->n_spheres != scenes[0]->n_spheres || scenes[i]->K != scenes[0]->K)
+            return fail(SHS_ERR_INVALID_ARG, "scene %d differs in size from scene 0", i);
     }
-    if (light) return set_light(sc, light, s);
+    for (int i = 0; i < n_scenes; i += shs::kMaxBatch) {
+        const int n = n_scenes - i < shs::kMaxBatch ? n_scenes - i : shs::kMaxBatch;
+        const float* c = centers ? centers + static_cast<size_t>(i) * scenes[0]->n_spheres * 3 : nullptr;
+        const shs_status st = update_scenes(scenes + i, n, c, radii, light, static_cast<cudaStream_t>(stream));
+        if (st != SHS_OK) return st;
+    }
     return SHS_OK;
 }
 

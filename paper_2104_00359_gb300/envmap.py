@@ -3,12 +3,10 @@ by the library's projection kernel (``shs_project_envmap``)."""
 
 from __future__ import annotations
 
-import ctypes
-
 import torch
 
 from . import _lib
-from ._lib import check, ptr
+from ._lib import check, current_stream, ptr
 
 
 def project_envmap(env, n_bands, out=None, workspace=None):
@@ -25,7 +23,7 @@ def project_envmap(env, n_bands, out=None, workspace=None):
     need = int(lib.shs_envmap_workspace_bytes(H, W, int(n_bands)))
     if workspace is None or workspace.numel() * workspace.element_size() < need:
         workspace = torch.empty(max(need, 4) // 4, dtype=torch.float32, device=env.device)
-    stream = ctypes.c_void_p(torch.cuda.current_stream(env.device).cuda_stream)
     check(lib.shs_project_envmap(ptr(env), H, W, int(n_bands), ptr(light), ptr(workspace),
-                                 workspace.numel() * workspace.element_size(), stream), "shs_project_envmap")
+                                 workspace.numel() * workspace.element_size(), current_stream(env.device.index)),
+          "shs_project_envmap")
     return light

@@ -15,7 +15,7 @@ import numpy as np
 import torch
 
 from . import _lib
-from ._lib import check, ptr
+from ._lib import check, current_stream, ptr
 
 
 def _proj_host(proj):
@@ -33,15 +33,15 @@ class Rasterize(torch.autograd.Function):
     @staticmethod
     def forward(ctx, vertices, radiance, faces, proj, height, width):
         lib = _lib.load()
-        v = vertices.detach().contiguous().float()
-        b = radiance.detach().contiguous().float()
+        v = vertices.contiguous().float()
+        b = radiance.contiguous().float()
         f = faces.contiguous().to(torch.int32)
         H, W = int(height), int(width)
         P, Pp = _proj_host(proj)
         image = torch.empty((H, W, 3), dtype=torch.float32, device=v.device)
         face_index = torch.empty((H, W), dtype=torch.int32, device=v.device)
         ws, need = _workspace(lib, v.shape[0], H, W, v.device)
-        stream = ctypes.c_void_p(torch.cuda.current_stream(v.device).cuda_stream)
+        stream = current_stream(v.device.index)
         check(lib.shs_rasterize(ptr(v), v.shape[0], ptr(f), f.shape[0], Pp, ptr(b), H, W, ptr(image),
                                 ptr(face_index), ptr(ws), need, stream), "shs_rasterize")
         ctx.save_for_backward(v, b, f, face_index)
@@ -61,7 +61,7 @@ class Rasterize(torch.autograd.Function):
         if not (want_v or want_b):
             return None, None, None, None, None, None
         ws, need = _workspace(lib, v.shape[0], H, W, v.device)
-        stream = ctypes.c_void_p(torch.cuda.current_stream(v.device).cuda_stream)
+        stream = current_stream(v.device.index)
         P = ctx.P
         check(lib.shs_rasterize_backward(ptr(v), v.shape[0], ptr(f), f.shape[0], P.ctypes.data_as(ctypes.c_void_p),
                                          ptr(b), H, W, ptr(face_index), ptr(d_image.contiguous().float()),

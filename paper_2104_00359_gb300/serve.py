@@ -131,13 +131,14 @@ class Job:
         c = self.chunks[chunk] if self.chunks else None
         r.scene = (c["scene"] if c else self.scene).handle.value
         r.n_points = p1 - p0
-        r.points, r.normals, r.albedo = (t[p0:p1].data_ptr() for t in (self.points, self.normals, self.albedo))
-        r.radiance = self.radiance[p0:p1].data_ptr()
+        at = 12 * p0   # bytes of p0 rows of three floats
+        r.points, r.normals, r.albedo = (t.data_ptr() + at for t in (self.points, self.normals, self.albedo))
+        r.radiance = self.radiance.data_ptr() + at
         r.saved = (c["saved"] if c else self.saved).data_ptr()
         if op == "fwdbwd":
-            r.target = self.target[p0:p1].data_ptr()
+            r.target = self.target.data_ptr() + at
             r.loss = (c["loss"] if c else self.loss).data_ptr()
-            r.d_albedo = self.grads["d_albedo"][p0:p1].data_ptr()
+            r.d_albedo = self.grads["d_albedo"].data_ptr() + at
             for k in ("d_light", "d_centers", "d_radii"):
                 v = self.grads[k]
                 if v is None:

@@ -16,7 +16,7 @@ import numpy as np
 import torch
 
 from . import _lib
-from ._lib import ShsConfig, check, ptr
+from ._lib import ShsConfig, check, current_stream, ptr
 
 
 @dataclass
@@ -41,17 +41,14 @@ class Config:
                          int(bool(self.horizon_cull)), int(self.exp_mode))
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-
-
 def _dev_f32(t, shape, name):
     if t is None:
         return None
-    if not (t.is_cuda and t.dtype == torch.float32):
+    if not (t.is_cuda and t.dtype is torch.float32):
         raise TypeError(f"{name} must be a float32 CUDA tensor")
-    t = t.contiguous()
-    if tuple(t.shape) != tuple(shape):
+    if not t.is_contiguous():
+        t = t.contiguous()
+    if t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t
 
@@ -69,7 +66,7 @@ class Scene:
         L = _dev_f32(light, (3, self.K), "light")
         h = ctypes.c_void_p()
         cfg = self.config.to_c()
-        check(self.lib.shs_scene_create(ctypes.byref(cfg), self.n_spheres, ptr(c), ptr(r), ptr(L), _stream(),
+        check(self.lib.shs_scene_create(ctypes.byref(cfg), self.n_spheres, ptr(c), ptr(r), ptr(L), current_stream(),
                                         ctypes.byref(h)), "shs_scene_create")
         self.handle = h
         if self.config.exp_mode == 2 and self.config.ol_table is not None:
@@ -79,7 +76,7 @@ class Scene:
         c = _dev_f32(centers, (self.n_spheres, 3), "centers") if centers is not None and self.n_spheres else None
         r = _dev_f32(radii, (self.n_spheres,), "radii") if radii is not None and self.n_spheres else None
         L = _dev_f32(light, (3, self.K), "light") if light is not None else None
-        check(self.lib.shs_scene_update(self.handle, ptr(c), ptr(r), ptr(L), _stream()), "shs_scene_update")
+        check(self.lib.shs_scene_update(self.handle, ptr(c), ptr(r), ptr(L), current_stream()), "shs_scene_update")
 
     def set_ol_table(self, a, b, s_max):
         """Optimal linear coefficients a(s), b(s) at the nodes s_i = i s_max / (m-1)
@@ -104,7 +101,7 @@ class Scene:
             pass
 
     def saved_bytes(self, n_points):
-        return int(self.lib.shs_saved_bytes(self.handle, int(n_points)))
+        return self.lib.shs_saved_bytes(self.handle, int(n_points))
 
     def saved_views(self, saved, n_points):
         """(f [P, K] float32 view, k [P] int32 view) of a saved buffer, with the
@@ -125,7 +122,7 @@ class Scene:
         nrm = _dev_f32(normals, (P, 3), "normals")
         alb = _dev_f32(albedo, (P, 3), "albedo")
         rad = out if out is not None else torch.empty((P, 3), dtype=torch.float32, device=pts.device)
-        check(self.lib.shs_shade(self.handle, P, ptr(pts), ptr(nrm), ptr(alb), ptr(rad), ptr(saved), _stream()),
+        check(self.lib.shs_shade(self.handle, P, ptr(pts), ptr(nrm), ptr(alb), ptr(rad), ptr(saved), current_stream()),
               "shs_shade")
         return rad
 
@@ -137,12 +134,12 @@ class Scene:
         nrm = _dev_f32(normals, (P, 3), "normals")
         alb = _dev_f32(albedo, (P, 3), "albedo")
         rad = out if out is not None else torch.empty((P, 3), dtype=torch.float32, device=nrm.device)
-        check(self.lib.shs_shade_tail(self.handle, P, ptr(nrm), ptr(alb), ptr(saved), ptr(rad), _stream()),
+        check(self.lib.shs_shade_tail(self.handle, P, ptr(nrm), ptr(alb), ptr(saved), ptr(rad), current_stream()),
               "shs_shade_tail")
         return rad
 
     def _grad_buffers(self, P, device, want):
-        z = lambda *s: torch.empty(s, dtype=torch.float32, device=device)
+        z = lambda *s: torch.empty(s, dtype=torch.float32, device=device)   # noqa: E731
         N = self.n_spheres
         return dict(
             d_light=z(3, self.K) if "light" in want else None,
@@ -165,7 +162,7 @@ class Scene:
         check(self.lib.shs_shade_backward(self.handle, P, ptr(pts), ptr(nrm), ptr(alb), ptr(saved), ptr(dB),
                                           ptr(g["d_light"]), ptr(g["d_albedo"]), ptr(g["d_centers"]),
                                           ptr(g["d_radii"]), ptr(g["d_points"]), ptr(g["d_normals"]),
-                                          _stream()), "shs_shade_backward")
+                                          current_stream()), "shs_shade_backward")
         return g
 
     def backward_l2(self, points, normals, albedo, radiance, target, saved=None, want=ALL):
@@ -181,12 +178,12 @@ class Scene:
         check(self.lib.shs_shade_backward_l2(self.handle, P, ptr(pts), ptr(nrm), ptr(alb), ptr(saved), ptr(rad),
                                              ptr(tgt), ptr(g["loss"]), ptr(g["d_light"]), ptr(g["d_albedo"]),
                                              ptr(g["d_centers"]), ptr(g["d_radii"]), ptr(g["d_points"]),
-                                             ptr(g["d_normals"]), _stream()), "shs_shade_backward_l2")
+                                             ptr(g["d_normals"]), current_stream()), "shs_shade_backward_l2")
         return g
 
     def device_status(self):
         st = ctypes.c_int32(0)
-        check(self.lib.shs_scene_device_status(self.handle, _stream(), ctypes.byref(st)), "shs_scene_device_status")
+        check(self.lib.shs_scene_device_status(self.handle, current_stream(), ctypes.byref(st)), "shs_scene_device_status")
         return int(st.value)
 
 
@@ -198,9 +195,10 @@ class ShadeFunction(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, points, normals, albedo, centers, radii, light, scene):
-        scene.update(centers.detach(), radii.detach(), light.detach())
+        # (a Function's forward and backward run without gradient recording)
+        scene.update(centers, radii, light)
         saved = scene.new_saved(points.shape[0], points.device)
-        B = scene.shade(points.detach(), normals.detach(), albedo.detach(), saved=saved)
+        B = scene.shade(points, normals, albedo, saved=saved)
         ctx.scene = scene
         ctx.save_for_backward(points, normals, albedo, saved)
         return B
@@ -210,8 +208,7 @@ class ShadeFunction(torch.autograd.Function):
         points, normals, albedo, saved = ctx.saved_tensors
         names = ("points", "normals", "albedo", "centers", "radii", "light")
         want = tuple(n for n, need in zip(names, ctx.needs_input_grad[:6]) if need)
-        g = ctx.scene.backward(points.detach(), normals.detach(), albedo.detach(), dB.contiguous(),
-                               saved=saved, want=want)
+        g = ctx.scene.backward(points, normals, albedo, dB, saved=saved, want=want)
         return (g["d_points"], g["d_normals"], g["d_albedo"], g["d_centers"], g["d_radii"], g["d_light"], None)
 
 
