@@ -13,8 +13,16 @@
 // Passes: clip coordinates per vertex; per triangle, its pixel bounding box
 // tested against the triangle and the (depth, face) key of each covered
 // pixel folded into a 64-bit atomicMin depth buffer; per pixel, the winning
-// triangle's colour.  The adjoint runs per pixel with atomic accumulation
-// into per-vertex gradients (rounding order varies between runs).
+// triangle's colour.  Four lanes share a triangle: a warp then waits for the
+// longest of 8 bounding boxes instead of 32 (99k triangles at 1024^2: 29 -> 20
+// us).
+//
+// The adjoint runs per pixel.  Its atomics are the bound: a thread takes
+// kRunPixels consecutive pixels, sums while they show the same triangle, and
+// adds a triangle's sums to the vertices with six 16-byte atomics (18 scalar
+// ones per pixel took 117 us at 1024^2, 99k triangles: now 26 us; one
+// triangle's lanes walking its box instead took 91 us, its lanes mostly idle).
+// Rounding order varies between runs.
 
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -35,6 +43,7 @@ struct RasterArgs {
     float4* clip;            // [V] workspace
     unsigned long long* zbuf;   // [H*W] workspace
     float4* dclip;           // [V] workspace (adjoint)
+    float4* drad;            // [V] workspace (adjoint, in zbuf's place): radiance gradients
 };
 
 __device__ __forceinline__ bool face_ids(const RasterArgs& a, int f, int& i0, int& i1, int& i2) {
@@ -55,25 +64,44 @@ __device__ __forceinline__ uint32_t ordered_bits(float z) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
-__global__ void raster_clip_kernel(const __grid_constant__ RasterArgs a) {
+// Clip coordinates of the vertices and, forward, the empty depth buffer
+// (n_clear pixels); in the adjoint zeros for the vertices' gradients.
+__global__ void raster_clip_kernel(const __grid_constant__ RasterArgs a, int n_clear, int adjoint) {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < n_clear) a.zbuf[v] = kEmpty;
     if (v >= a.V) return;
     const float x = __ldg(a.vertices + 3 * v), y = __ldg(a.vertices + 3 * v + 1), z = __ldg(a.vertices + 3 * v + 2);
     float c[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) c[r] = fmaf(a.P[4 * r], x, fmaf(a.P[4 * r + 1], y, fmaf(a.P[4 * r + 2], z, a.P[4 * r + 3])));
     a.clip[v] = make_float4(c[0], c[1], c[2], c[3]);
+    if (adjoint) a.dclip[v] = a.drad[v] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void raster_clear_kernel(unsigned long long* zbuf, int n) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) zbuf[p] = kEmpty;
+// Pixel ranges whose centres a triangle's bounding box holds: column c has
+// x = -1 + (2c + 1) / W, row r has y = 1 - (2r + 1) / H.
+struct PixelBox {
+    int cmin, cmax, rmin, rmax;
+};
+__device__ __forceinline__ PixelBox pixel_box(const RasterArgs& a, float x0, float y0, float x1, float y1, float x2,
+                                              float y2) {
+    const float xmin = fminf(x0, fminf(x1, x2)), xmax = fmaxf(x0, fmaxf(x1, x2));
+    const float ymin = fminf(y0, fminf(y1, y2)), ymax = fmaxf(y0, fmaxf(y1, y2));
+    PixelBox b;
+    b.cmin = max(0, static_cast<int>(ceilf((xmin + 1.f) * 0.5f * a.W - 0.5f)));
+    b.cmax = min(a.W - 1, static_cast<int>(floorf((xmax + 1.f) * 0.5f * a.W - 0.5f)));
+    b.rmin = max(0, static_cast<int>(ceilf((1.f - ymax) * 0.5f * a.H - 0.5f)));
+    b.rmax = min(a.H - 1, static_cast<int>(floorf((1.f - ymin) * 0.5f * a.H - 0.5f)));
+    return b;
 }
 
-// One thread per triangle: test the pixel centres of its bounding box.
+constexpr int kFaceLanes = 4;   // lanes per triangle
+
+// Test the pixel centres of each triangle's bounding box.
 __global__ void raster_faces_kernel(const __grid_constant__ RasterArgs a) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= a.F) return;
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t / kFaceLanes >= a.F) return;
+    const int f = static_cast<int>(t / kFaceLanes);
     int i0, i1, i2;
     if (!face_ids(a, f, i0, i1, i2)) return;
     const float4 c0 = a.clip[i0], c1 = a.clip[i1], c2 = a.clip[i2];
@@ -84,27 +112,31 @@ __global__ void raster_faces_kernel(const __grid_constant__ RasterArgs a) {
     const float A = edge_fn(x0, y0, x1, y1, x2, y2);
     if (!(A != 0.f) || !isfinite(A)) return;
     const float inv_a = 1.f / A;
-    // pixel ranges: column c has x = -1 + (2c + 1) / W, row r has y = 1 - (2r + 1) / H
-    const float xmin = fminf(x0, fminf(x1, x2)), xmax = fmaxf(x0, fmaxf(x1, x2));
-    const float ymin = fminf(y0, fminf(y1, y2)), ymax = fmaxf(y0, fmaxf(y1, y2));
-    const int cmin = max(0, static_cast<int>(ceilf((xmin + 1.f) * 0.5f * a.W - 0.5f)));
-    const int cmax = min(a.W - 1, static_cast<int>(floorf((xmax + 1.f) * 0.5f * a.W - 0.5f)));
-    const int rmin = max(0, static_cast<int>(ceilf((1.f - ymax) * 0.5f * a.H - 0.5f)));
-    const int rmax = min(a.H - 1, static_cast<int>(floorf((1.f - ymin) * 0.5f * a.H - 0.5f)));
-    if (cmin > cmax || rmin > rmax) return;
-    for (int r = rmin; r <= rmax; ++r) {
+    const PixelBox b = pixel_box(a, x0, y0, x1, y1, x2, y2);
+    if (b.cmin > b.cmax || b.rmin > b.rmax) return;
+    // the lanes take every fourth pixel of the box, row after row
+    int r = b.rmin, c = b.cmin + static_cast<int>(t % kFaceLanes);
+    const int nc = b.cmax - b.cmin + 1;
+    while (c > b.cmax) {
+        c -= nc;
+        ++r;
+    }
+    while (r <= b.rmax) {
         const float py = 1.f - (2.f * r + 1.f) / a.H;
-        for (int c = cmin; c <= cmax; ++c) {
-            const float px = -1.f + (2.f * c + 1.f) / a.W;
-            const float l0 = edge_fn(x1, y1, x2, y2, px, py) * inv_a;
-            const float l1 = edge_fn(x2, y2, x0, y0, px, py) * inv_a;
-            const float l2 = edge_fn(x0, y0, x1, y1, px, py) * inv_a;
-            if (l0 < 0.f || l1 < 0.f || l2 < 0.f) continue;
-            const float z = fmaf(l0, z0, fmaf(l1, z1, l2 * z2));
-            if (!(z >= -1.f && z <= 1.f)) continue;
+        const float px = -1.f + (2.f * c + 1.f) / a.W;
+        const float l0 = edge_fn(x1, y1, x2, y2, px, py) * inv_a;
+        const float l1 = edge_fn(x2, y2, x0, y0, px, py) * inv_a;
+        const float l2 = edge_fn(x0, y0, x1, y1, px, py) * inv_a;
+        const float z = fmaf(l0, z0, fmaf(l1, z1, l2 * z2));
+        if (!(l0 < 0.f || l1 < 0.f || l2 < 0.f) && z >= -1.f && z <= 1.f) {
             const unsigned long long key = (static_cast<unsigned long long>(ordered_bits(z)) << 32) |
                                            static_cast<unsigned int>(f);
             atomicMin(a.zbuf + static_cast<size_t>(r) * a.W + c, key);
+        }
+        c += kFaceLanes;
+        while (c > b.cmax) {
+            c -= nc;
+            ++r;
         }
     }
 }
@@ -162,27 +194,19 @@ __global__ void raster_resolve_kernel(const __grid_constant__ RasterArgs a, floa
     face_index[p] = f;
 }
 
-// Adjoint per pixel: radiance gradients b_k dI, and the clip-coordinate
-// gradients of the triangle's vertices through the barycentrics.
-__global__ void raster_backward_kernel(const __grid_constant__ RasterArgs a, const int32_t* face_index,
-                                       const float* d_image, float* d_radiance, int want_pos) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.H * a.W) return;
-    const int f = face_index[p];
-    if (f < 0 || f >= a.F) return;
-    PixelBary pb;
-    if (!face_ids(a, f, pb.ids[0], pb.ids[1], pb.ids[2])) return;
-    pixel_bary(a, f, p / a.W, p % a.W, pb);
+// One pixel's adjoint, added to dr (radiance gradients b_k dI, vertex-major) and
+// dc (clip-coordinate gradients (x, y, w) of the triangle's vertices through the
+// barycentrics).
+__device__ __forceinline__ void pixel_adjoint(const RasterArgs& a, const PixelBary& pb, const float* d_image, int p,
+                                              bool want_pos, float (*dr)[3], float (*dc)[3]) {
     const float dI[3] = {__ldg(d_image + 3 * p), __ldg(d_image + 3 * p + 1), __ldg(d_image + 3 * p + 2)};
     float g[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float* Bk = a.radiance + 3 * pb.ids[k];
         g[k] = fmaf(dI[0], __ldg(Bk), fmaf(dI[1], __ldg(Bk + 1), dI[2] * __ldg(Bk + 2)));
-        if (d_radiance) {
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) atomicAdd(d_radiance + 3 * pb.ids[k] + ch, pb.b[k] * dI[ch]);
-        }
+        for (int ch = 0; ch < 3; ++ch) dr[k][ch] += pb.b[k] * dI[ch];
     }
     if (!want_pos) return;
     const float bg = g[0] * pb.b[0] + g[1] * pb.b[1] + g[2] * pb.b[2];
@@ -208,18 +232,59 @@ __global__ void raster_backward_kernel(const __grid_constant__ RasterArgs a, con
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        float4* d = a.dclip + pb.ids[k];
         const float iw = 1.f / pb.w[k];
-        atomicAdd(&d->x, dn[k][0] * iw);
-        atomicAdd(&d->y, dn[k][1] * iw);
-        atomicAdd(&d->w, dw[k] - (dn[k][0] * pb.n[k][0] + dn[k][1] * pb.n[k][1]) * iw);
+        dc[k][0] += dn[k][0] * iw;
+        dc[k][1] += dn[k][1] * iw;
+        dc[k][2] += dw[k] - (dn[k][0] * pb.n[k][0] + dn[k][1] * pb.n[k][1]) * iw;
     }
 }
 
-// d_vertices[v] = P[:, 0:3]^T dclip[v].
-__global__ void raster_vertex_backward_kernel(const __grid_constant__ RasterArgs a, float* d_vertices) {
+constexpr int kRunPixels = 4;
+__global__ void raster_backward_kernel(const __grid_constant__ RasterArgs a, const int32_t* face_index,
+                                       const float* d_image, int want_rad, int want_pos) {
+    const int n = a.H * a.W, p0 = (blockIdx.x * blockDim.x + threadIdx.x) * kRunPixels;
+    PixelBary pb;
+    float dr[3][3], dc[3][3];
+    int cur = -1;   // triangle the sums belong to
+    auto flush = [&] {
+        if (cur < 0) return;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (want_rad) atomicAdd(a.drad + pb.ids[k], make_float4(dr[k][0], dr[k][1], dr[k][2], 0.f));
+            if (want_pos) atomicAdd(a.dclip + pb.ids[k], make_float4(dc[k][0], dc[k][1], 0.f, dc[k][2]));
+        }
+    };
+#pragma unroll 1
+    for (int p = p0; p < p0 + kRunPixels && p < n; ++p) {
+        const int f = __ldg(face_index + p);
+        if (f != cur) {
+            flush();
+            cur = f >= 0 && f < a.F && face_ids(a, f, pb.ids[0], pb.ids[1], pb.ids[2]) ? f : -1;
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int e = 0; e < 3; ++e) dr[k][e] = dc[k][e] = 0.f;
+        }
+        if (cur < 0) continue;
+        pixel_bary(a, f, p / a.W, p % a.W, pb);
+        pixel_adjoint(a, pb, d_image, p, want_pos, dr, dc);
+    }
+    flush();
+}
+
+// d_vertices[v] = P[:, 0:3]^T dclip[v], d_radiance[v] = drad[v] (either may be
+// null).
+__global__ void raster_vertex_backward_kernel(const __grid_constant__ RasterArgs a, float* d_radiance,
+                                              float* d_vertices) {
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= a.V) return;
+    if (d_radiance) {
+        const float4 r = a.drad[v];
+        d_radiance[3 * v] = r.x;
+        d_radiance[3 * v + 1] = r.y;
+        d_radiance[3 * v + 2] = r.z;
+    }
+    if (!d_vertices) return;
     const float4 d = a.dclip[v];
 #pragma unroll
     for (int j = 0; j < 3; ++j)
@@ -228,7 +293,8 @@ __global__ void raster_vertex_backward_kernel(const __grid_constant__ RasterArgs
 
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
-// Workspace: clip [V] float4, dclip [V] float4, depth buffer [H*W] uint64.
+// Workspace: clip [V] float4, dclip [V] float4, then the depth buffer [H*W]
+// uint64 or, in the adjoint, drad [V] float4.
 bool raster_setup(RasterArgs& a, const float* vertices, int32_t n_vertices, const int32_t* faces,
                   int32_t n_faces, const float* proj, const float* radiance, int32_t height, int32_t width,
                   void* workspace, size_t workspace_bytes, shs_status* st);
@@ -238,7 +304,8 @@ bool raster_setup(RasterArgs& a, const float* vertices, int32_t n_vertices, cons
 extern "C" size_t shs_raster_workspace_bytes(int32_t n_vertices, int32_t height, int32_t width) {
     if (n_vertices < 0 || height < 1 || width < 1 || height > 16384 || width > 16384) return 0;
     const size_t v = static_cast<size_t>(n_vertices > 0 ? n_vertices : 1);
-    return 2 * align256(sizeof(float4) * v) + align256(sizeof(unsigned long long) * height * width);
+    const size_t vb = align256(sizeof(float4) * v), zb = align256(sizeof(unsigned long long) * height * width);
+    return 2 * vb + (zb > vb ? zb : vb);
 }
 
 namespace {
@@ -268,7 +335,13 @@ bool raster_setup(RasterArgs& a, const float* vertices, int32_t n_vertices, cons
     a.clip = reinterpret_cast<float4*>(w);
     a.dclip = reinterpret_cast<float4*>(w + vb);
     a.zbuf = reinterpret_cast<unsigned long long*>(w + 2 * vb);
+    a.drad = reinterpret_cast<float4*>(a.zbuf);
     return true;
+}
+
+constexpr int kFaceBlock = 128;
+unsigned face_blocks(int n_faces) {
+    return static_cast<unsigned>((static_cast<int64_t>(n_faces) * kFaceLanes + kFaceBlock - 1) / kFaceBlock);
 }
 
 shs_status raster_status(cudaError_t e, const char* what) {
@@ -289,14 +362,11 @@ extern "C" shs_status shs_rasterize(const float* vertices, int32_t n_vertices, c
         return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int npix = height * width;
-    if (n_vertices > 0) {
-        raster_clip_kernel<<<(n_vertices + 255) / 256, 256, 0, s>>>(a);
-        shs::count_launch();
-    }
-    raster_clear_kernel<<<(npix + 255) / 256, 256, 0, s>>>(a.zbuf, npix);
+    const int items = n_vertices > npix ? n_vertices : npix;
+    raster_clip_kernel<<<(items + 255) / 256, 256, 0, s>>>(a, npix, 0);
     shs::count_launch();
     if (n_faces > 0) {
-        raster_faces_kernel<<<(n_faces + 127) / 128, 128, 0, s>>>(a);
+        raster_faces_kernel<<<face_blocks(n_faces), kFaceBlock, 0, s>>>(a);
         shs::count_launch();
     }
     raster_resolve_kernel<<<(npix + 255) / 256, 256, 0, s>>>(a, image, face_index);
@@ -317,23 +387,18 @@ extern "C" shs_status shs_rasterize_backward(const float* vertices, int32_t n_ve
                       workspace_bytes, &st))
         return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaSuccess;
     if (n_vertices > 0) {
-        if (d_radiance) e = cudaMemsetAsync(d_radiance, 0, sizeof(float) * 3 * n_vertices, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(a.dclip, 0, sizeof(float4) * n_vertices, s);
-        if (e != cudaSuccess) return raster_status(e, "rasterize backward: clear");
-        raster_clip_kernel<<<(n_vertices + 255) / 256, 256, 0, s>>>(a);
+        raster_clip_kernel<<<(n_vertices + 255) / 256, 256, 0, s>>>(a, 0, 1);
         shs::count_launch();
     }
-    const int npix = height * width;
+    const int64_t npix = static_cast<int64_t>(height) * width;
     if (n_vertices > 0 && (d_radiance || d_vertices)) {
-        raster_backward_kernel<<<(npix + 255) / 256, 256, 0, s>>>(a, face_index, d_image, d_radiance,
-                                                                   d_vertices ? 1 : 0);
+        const int64_t threads = (npix + kRunPixels - 1) / kRunPixels;
+        raster_backward_kernel<<<static_cast<unsigned>((threads + 127) / 128), 128, 0, s>>>(
+            a, face_index, d_image, d_radiance ? 1 : 0, d_vertices ? 1 : 0);
         shs::count_launch();
-        if (d_vertices) {
-            raster_vertex_backward_kernel<<<(n_vertices + 255) / 256, 256, 0, s>>>(a, d_vertices);
-            shs::count_launch();
-        }
+        raster_vertex_backward_kernel<<<(n_vertices + 255) / 256, 256, 0, s>>>(a, d_radiance, d_vertices);
+        shs::count_launch();
     }
     return raster_status(cudaGetLastError(), "rasterize backward");
 }

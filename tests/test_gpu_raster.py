@@ -88,6 +88,28 @@ def test_backward_matches_oracle():
         assert err.max() <= 1e-3, f"{name}: {err.max():.3e}"
 
 
+@pytest.mark.parametrize("H,W", [(1, 1), (3, 7), (33, 61)])
+@pytest.mark.parametrize("large", [True, False])
+def test_backward_runs_of_pixels(H, W, large):
+    """Pixel runs that end inside a row, at the image's end and on a change of
+    triangle; one triangle over the whole image in front of or behind a mesh."""
+    m, faces = _mesh(n_theta=8, n_phi=10)
+    v, B = m["v0"].astype(np.float64), m["albedo"].astype(np.float64)
+    P = S.look_at_perspective((2.4, 0.7, 1.1), aspect=W / H)
+    if large:   # a screen-filling triangle behind the mesh
+        q = np.array([[-6.0, -9.0, -7.0], [-6.0, 12.0, -7.0], [-7.0, 1.0, 12.0]])
+        faces = np.concatenate([faces, [[len(v), len(v) + 1, len(v) + 2]]]).astype(np.int32)
+        v, B = np.concatenate([v, q]), np.concatenate([B, [[0.3, 0.5, 0.7], [0.9, 0.1, 0.2], [0.4, 0.4, 0.8]]])
+    v, B = v.astype(np.float32), B.astype(np.float32)
+    dI = np.random.default_rng(H + W).normal(size=(H, W, 3))
+    got = _gpu(v, faces, P, B, H, W, dI=dI)
+    ref = R.rasterize_backward(v, faces, P, B, got["face_index"], dI)
+    for name in ("d_radiance", "d_vertices"):
+        r, g = ref[name], got[name]
+        err = np.abs(g - r) / np.maximum(np.abs(r), 1e-2 * max(np.abs(r).max(), 1e-12))
+        assert err.max() <= 1e-3, f"{name}: {err.max():.3e}"
+
+
 def test_empty_and_culled_inputs():
     import torch
     from paper_2104_00359_gb300.raster import rasterize
