@@ -371,6 +371,34 @@ def emit_gaunt(n, C):
     return mul_lines, sqr_lines
 
 
+def emit_lobe_products(n, C):
+    """Products with the clamped-cosine lobe H, whose bands l = 3, 5, .. vanish:
+    mul_lobe: o = a * b for b without those bands; mul_onto_lobe: only the
+    lobe's bands of o = a * b (the others are set to zero)."""
+    K = n * n
+    on = [l < 2 or l % 2 == 0 for l in range(n) for _ in range(2 * l + 1)]
+    by_i = {i: [] for i in range(K)}
+    for (i, j, k), v in sorted(C.items()):
+        by_i[i].append((j, k, v))
+    lobe, onto = [], []
+    for i in range(K):
+        t_lobe, t_onto = [], []
+        for j, k, v in by_i[i]:
+            c = fmt(("c", v))
+            both = f"a[{j}] * b[{j}]" if j == k else f"(a[{j}] * b[{k}] + a[{k}] * b[{j}])"
+            t_onto.append((c, both))
+            if j == k:
+                if on[j]:
+                    t_lobe.append((c, both))
+            elif on[j] and on[k]:
+                t_lobe.append((c, both))
+            elif on[j] or on[k]:
+                t_lobe.append((c, f"a[{j}] * b[{k}]" if on[k] else f"a[{k}] * b[{j}]"))
+        lobe.append(f"o[{i}] = {balanced_sum(t_lobe)};" if t_lobe else f"o[{i}] = 0.0f;")
+        onto.append(f"o[{i}] = {balanced_sum(t_onto)};" if t_onto and on[i] else f"o[{i}] = 0.0f;")
+    return lobe, onto
+
+
 def balanced_sum(terms, chains=4):
     """sum of c * t over (c, t) as up to ``chains`` interleaved FMA chains added
     pairwise: rounding error grows with len/chains instead of len, and the
@@ -415,9 +443,10 @@ def emit_monomial_route(n):
       every monomial of degree l < n (forward pair term in monomial form).
     mono_to_f(acc, f): f_i = sum_a Hbar_i[a] acc[off_l + a], Hbar_i the
       homogeneous Ybar_i, i.e. the un-normalised log-visibility coefficients.
-    grad_coeffs(w, gq): for bands l >= 1, the coefficients over monomials of
-      degree l-1 of the three partial derivatives of Phi_l = sum_m w_lm Hbar_lm.
-    grad_eval(x, y, z, gq, gx, gy, gz): (gx, gy, gz)[l-1] = grad Phi_l(x, y, z).
+    grad_coeffs(w, gq): for bands l >= 1, the entries of the symmetric tensor of
+      Phi_l = sum_m w_lm Hbar_lm, scaled by l.
+    grad_eval2(x, y, z, gq, gx, gy, gz): (gx, gy, gz)[l-1] = grad Phi_l(x, y, z)
+      of two points at once, gq(o) their entry o.
     """
     H = homogeneous_polys(n)
     offs, na = [], 0
@@ -449,37 +478,44 @@ def emit_monomial_route(n):
         terms = [(fmt(("c", float(v))), f"acc[{offs[l] + monomials(l).index(mono)}]")
                  for mono, v in sorted(H[i].items()) if v != 0]
         m2f.append(f"f[{i}] = {balanced_sum(terms)};")
+    # adjoint: symmetric tensor entries T_alpha = l coef_alpha / multinomial(alpha)
+    # of Phi_l, and the gradient dPhi_l/dv = sum_beta multinomial(beta) s^beta T_{beta+e_v}
     goffs, ng = [], 0
     for l in range(1, n):
         goffs.append(ng)
-        ng += 3 * len(monomials(l - 1))
+        ng += len(monomials(l))
     gc = []
     for l in range(1, n):
-        lower = monomials(l - 1)
-        for comp in range(3):
-            for bi, beta in enumerate(lower):
+        for ai, alpha in enumerate(monomials(l)):
+            mult = math.factorial(l) // math.prod(math.factorial(e) for e in alpha)
+            terms = []
+            for m in range(-l, l + 1):
+                i = l * l + l + m
+                v = H[i].get(alpha, 0)
+                if v != 0:
+                    terms.append((fmt(("c", float(v) * l / mult)), f"w[{i}]"))
+            gc.append(f"gq[{goffs[l - 1] + ai}] = {balanced_sum(terms) if terms else '0.0f'};")
+    ge, uname = [], {(0, 0, 0): None, (1, 0, 0): "x", (0, 1, 0): "y", (0, 0, 1): "z"}
+    for d in range(2, n - 1):   # weighted monomials of degree d
+        for v in "xyz":
+            ge.append(f"const float2 {v}{d} = __fmul2_rn(make_float2({d}.0f, {d}.0f), {v});")
+        for beta in monomials(d):
+            v = next(i for i in range(3) if beta[i] in (1, d))
+            low = list(beta)
+            low[v] -= 1
+            var = "xyz"[v] + ("" if beta[v] == d else str(d))
+            uname[beta] = "u{}_{}_{}".format(*beta)
+            ge.append(f"const float2 {uname[beta]} = __fmul2_rn({uname[tuple(low)]}, {var});")
+    for l in range(1, n):
+        for comp, g in ((0, "gx"), (1, "gy"), (2, "gz")):
+            expr = None
+            for beta in monomials(l - 1):
                 up = list(beta)
                 up[comp] += 1
-                up = tuple(up)
-                factor = up[comp]
-                terms = []
-                for m in range(-l, l + 1):
-                    i = l * l + l + m
-                    v = H[i].get(up, 0)
-                    if v != 0:
-                        terms.append((fmt(("c", float(v) * factor)), f"w[{i}]"))
-                o = goffs[l - 1] + comp * len(lower) + bi
-                gc.append(f"gq[{o}] = {balanced_sum(terms) if terms else '0.0f'};")
-    ge_m, gname = _mono_lines(max(n - 2, 0), prefix="u")
-    ge = list(ge_m)
-    for l in range(1, n):
-        lower = monomials(l - 1)
-        for comp, g in ((0, "gx"), (1, "gy"), (2, "gz")):
-            terms = []
-            for bi, beta in enumerate(lower):
-                o = goffs[l - 1] + comp * len(lower) + bi
-                terms.append(f"gq[{o}]" + ("" if beta == (0, 0, 0) else f" * {gname[beta]}"))
-            ge.append(f"{g}[{l - 1}] = {' + '.join(terms)};")
+                t = f"gq({goffs[l - 1] + monomials(l).index(tuple(up))})"
+                u = uname[beta]
+                expr = t if u is None else (f"__fmul2_rn({t}, {u})" if expr is None else f"__ffma2_rn({t}, {u}, {expr})")
+            ge.append(f"{g}[{l - 1}] = {expr};")
     return na, ng, ml, acc, m2f, gc, ge
 
 
@@ -739,7 +775,7 @@ def generate():
         if n < LANE_PAIR_FROM:
             na, ng, ml, acc_l, m2f_l, gc_l, ge_l = emit_monomial_route(n)
             parts.append(f"    static constexpr int NA = {na};   // monomials of degree < n")
-            parts.append(f"    static constexpr int NG = {max(ng, 1)};   // gradient coefficients, bands >= 1")
+            parts.append(f"    static constexpr int NG = {ng};   // symmetric tensor entries, bands >= 1")
             parts.append("    __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {")
             parts.append("        (void)x; (void)y; (void)z;")
             parts.append(indent(ml + acc_l))
@@ -757,8 +793,9 @@ def generate():
             parts.append("        (void)w; (void)gq;")
             parts.append(indent(gc_l))
             parts.append("    }")
-            parts.append("    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,")
-            parts.append("                                                     float* gx, float* gy, float* gz) {")
+            parts.append("    template <class Q>")
+            parts.append("    __device__ __forceinline__ static void grad_eval2(float2 x, float2 y, float2 z, Q&& gq,")
+            parts.append("                                                      float2* gx, float2* gy, float2* gz) {")
             parts.append("        (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;")
             parts.append(indent(ge_l))
             parts.append("    }")
@@ -767,6 +804,11 @@ def generate():
             parts.append("                                               float* __restrict__ o) {")
             parts.append(indent(mul_l))
             parts.append("    }")
+            for nm, lines in zip(("mul_lobe", "mul_onto_lobe"), emit_lobe_products(n, C)):
+                parts.append(f"    __device__ __forceinline__ static void {nm}(const float* __restrict__ a, const float* __restrict__ b,")
+                parts.append("                                               float* __restrict__ o) {")
+                parts.append(indent(lines))
+                parts.append("    }")
             parts.append("    __device__ __forceinline__ static void sqr(const float* __restrict__ a, float* __restrict__ o) {")
             parts.append(indent(sqr_l))
             parts.append("    }")

@@ -47,7 +47,7 @@ template <> struct SH<1> {
         gz = 0.0f;
     }
     static constexpr int NA = 1;   // monomials of degree < n
-    static constexpr int NG = 1;   // gradient coefficients, bands >= 1
+    static constexpr int NG = 0;   // symmetric tensor entries, bands >= 1
     __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
         (void)x; (void)y; (void)z;
         acc[0] = fmaf(G[0], 1.0f, acc[0]);
@@ -65,12 +65,21 @@ template <> struct SH<1> {
         (void)w; (void)gq;
 
     }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
+    template <class Q>
+    __device__ __forceinline__ static void grad_eval2(float2 x, float2 y, float2 z, Q&& gq,
+                                                      float2* gx, float2* gy, float2* gz) {
         (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
 
     }
     __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = 0.282094806432724f * a[0] * b[0];
+    }
+    __device__ __forceinline__ static void mul_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = 0.282094806432724f * a[0] * b[0];
+    }
+    __device__ __forceinline__ static void mul_onto_lobe(const float* __restrict__ a, const float* __restrict__ b,
                                                float* __restrict__ o) {
         o[0] = 0.282094806432724f * a[0] * b[0];
     }
@@ -125,7 +134,7 @@ template <> struct SH<2> {
         gz = w[2];
     }
     static constexpr int NA = 4;   // monomials of degree < n
-    static constexpr int NG = 3;   // gradient coefficients, bands >= 1
+    static constexpr int NG = 3;   // symmetric tensor entries, bands >= 1
     __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
         (void)x; (void)y; (void)z;
         const float m1_0_0 = x;
@@ -160,14 +169,29 @@ template <> struct SH<2> {
         gq[1] = 1.0f * w[1];
         gq[2] = 1.0f * w[2];
     }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
+    template <class Q>
+    __device__ __forceinline__ static void grad_eval2(float2 x, float2 y, float2 z, Q&& gq,
+                                                      float2* gx, float2* gy, float2* gz) {
         (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
+        gx[0] = gq(0);
+        gy[0] = gq(1);
+        gz[0] = gq(2);
     }
     __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((0.282094806432724f * a[0] * b[0] + 0.282094806432724f * a[1] * b[1]) + (0.282094806432724f * a[2] * b[2] + 0.282094806432724f * a[3] * b[3]));
+        o[1] = 0.282094806432724f * (a[0] * b[1] + a[1] * b[0]);
+        o[2] = 0.282094806432724f * (a[0] * b[2] + a[2] * b[0]);
+        o[3] = 0.282094806432724f * (a[0] * b[3] + a[3] * b[0]);
+    }
+    __device__ __forceinline__ static void mul_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((0.282094806432724f * a[0] * b[0] + 0.282094806432724f * a[1] * b[1]) + (0.282094806432724f * a[2] * b[2] + 0.282094806432724f * a[3] * b[3]));
+        o[1] = 0.282094806432724f * (a[0] * b[1] + a[1] * b[0]);
+        o[2] = 0.282094806432724f * (a[0] * b[2] + a[2] * b[0]);
+        o[3] = 0.282094806432724f * (a[0] * b[3] + a[3] * b[0]);
+    }
+    __device__ __forceinline__ static void mul_onto_lobe(const float* __restrict__ a, const float* __restrict__ b,
                                                float* __restrict__ o) {
         o[0] = ((0.282094806432724f * a[0] * b[0] + 0.282094806432724f * a[1] * b[1]) + (0.282094806432724f * a[2] * b[2] + 0.282094806432724f * a[3] * b[3]));
         o[1] = 0.282094806432724f * (a[0] * b[1] + a[1] * b[0]);
@@ -281,7 +305,7 @@ template <> struct SH<3> {
         gz = w[2] + 3.0f * a_t9 + z * a_t6 + z * a_t6;
     }
     static constexpr int NA = 10;   // monomials of degree < n
-    static constexpr int NG = 12;   // gradient coefficients, bands >= 1
+    static constexpr int NG = 9;   // symmetric tensor entries, bands >= 1
     __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
         (void)x; (void)y; (void)z;
         const float m1_0_0 = x;
@@ -341,27 +365,46 @@ template <> struct SH<3> {
         gq[3] = (-1.0f * w[6] + 6.0f * w[8]);
         gq[4] = 6.0f * w[4];
         gq[5] = 3.0f * w[7];
-        gq[6] = 6.0f * w[4];
-        gq[7] = (-1.0f * w[6] + -6.0f * w[8]);
-        gq[8] = 3.0f * w[5];
-        gq[9] = 3.0f * w[7];
-        gq[10] = 3.0f * w[5];
-        gq[11] = 2.0f * w[6];
+        gq[6] = (-1.0f * w[6] + -6.0f * w[8]);
+        gq[7] = 3.0f * w[5];
+        gq[8] = 2.0f * w[6];
     }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
+    template <class Q>
+    __device__ __forceinline__ static void grad_eval2(float2 x, float2 y, float2 z, Q&& gq,
+                                                      float2* gx, float2* gy, float2* gz) {
         (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        const float u1_0_0 = x;
-        const float u0_1_0 = y;
-        const float u0_0_1 = z;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
-        gx[1] = gq[3] * u1_0_0 + gq[4] * u0_1_0 + gq[5] * u0_0_1;
-        gy[1] = gq[6] * u1_0_0 + gq[7] * u0_1_0 + gq[8] * u0_0_1;
-        gz[1] = gq[9] * u1_0_0 + gq[10] * u0_1_0 + gq[11] * u0_0_1;
+        gx[0] = gq(0);
+        gy[0] = gq(1);
+        gz[0] = gq(2);
+        gx[1] = __ffma2_rn(gq(5), z, __ffma2_rn(gq(4), y, __fmul2_rn(gq(3), x)));
+        gy[1] = __ffma2_rn(gq(7), z, __ffma2_rn(gq(6), y, __fmul2_rn(gq(4), x)));
+        gz[1] = __ffma2_rn(gq(8), z, __ffma2_rn(gq(7), y, __fmul2_rn(gq(5), x)));
     }
     __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])) + fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1])) + (fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]) + fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])));
+        o[1] = ((fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0])) + -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1])) + (-0.21850968897342682f * (a[1] * b[8] + a[8] * b[1]) + 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2])));
+        o[2] = ((0.282094806432724f * (a[0] * b[2] + a[2] * b[0]) + 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1])) + (0.2523132562637329f * (a[2] * b[6] + a[6] * b[2]) + 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3])));
+        o[3] = ((fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0])) + 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1])) + (0.21850968897342682f * (a[2] * b[7] + a[7] * b[2]) + -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3])));
+        o[4] = ((0.282094806432724f * (a[0] * b[4] + a[4] * b[0]) + 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1])) + (-0.180223748087883f * (a[4] * b[6] + a[6] * b[4]) + 0.15607835352420807f * (a[5] * b[7] + a[7] * b[5])));
+        o[5] = ((fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), 0.282094806432724f * (a[0] * b[5] + a[5] * b[0])) + 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1])) + (0.15607835352420807f * (a[4] * b[7] + a[7] * b[4]) + 0.0901118740439415f * (a[5] * b[6] + a[6] * b[5])));
+        o[6] = ((fmaf(-0.180223748087883f, a[8] * b[8], fmaf(-0.180223748087883f, a[4] * b[4], 0.282094806432724f * (a[0] * b[6] + a[6] * b[0]))) + fmaf(0.0901118740439415f, a[5] * b[5], -0.12615662813186646f * a[1] * b[1])) + (fmaf(0.180223748087883f, a[6] * b[6], 0.2523132562637329f * a[2] * b[2]) + fmaf(0.0901118740439415f, a[7] * b[7], -0.12615662813186646f * a[3] * b[3])));
+        o[7] = ((fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), 0.282094806432724f * (a[0] * b[7] + a[7] * b[0])) + 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2])) + (0.15607835352420807f * (a[4] * b[5] + a[5] * b[4]) + 0.0901118740439415f * (a[6] * b[7] + a[7] * b[6])));
+        o[8] = ((fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), 0.282094806432724f * (a[0] * b[8] + a[8] * b[0])) + fmaf(0.15607835352420807f, a[7] * b[7], -0.21850968897342682f * a[1] * b[1])) + (0.21850968897342682f * a[3] * b[3] + -0.15607835352420807f * a[5] * b[5]));
+    }
+    __device__ __forceinline__ static void mul_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])) + fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1])) + (fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]) + fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])));
+        o[1] = ((fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0])) + -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1])) + (-0.21850968897342682f * (a[1] * b[8] + a[8] * b[1]) + 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2])));
+        o[2] = ((0.282094806432724f * (a[0] * b[2] + a[2] * b[0]) + 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1])) + (0.2523132562637329f * (a[2] * b[6] + a[6] * b[2]) + 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3])));
+        o[3] = ((fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0])) + 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1])) + (0.21850968897342682f * (a[2] * b[7] + a[7] * b[2]) + -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3])));
+        o[4] = ((0.282094806432724f * (a[0] * b[4] + a[4] * b[0]) + 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1])) + (-0.180223748087883f * (a[4] * b[6] + a[6] * b[4]) + 0.15607835352420807f * (a[5] * b[7] + a[7] * b[5])));
+        o[5] = ((fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), 0.282094806432724f * (a[0] * b[5] + a[5] * b[0])) + 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1])) + (0.15607835352420807f * (a[4] * b[7] + a[7] * b[4]) + 0.0901118740439415f * (a[5] * b[6] + a[6] * b[5])));
+        o[6] = ((fmaf(-0.180223748087883f, a[8] * b[8], fmaf(-0.180223748087883f, a[4] * b[4], 0.282094806432724f * (a[0] * b[6] + a[6] * b[0]))) + fmaf(0.0901118740439415f, a[5] * b[5], -0.12615662813186646f * a[1] * b[1])) + (fmaf(0.180223748087883f, a[6] * b[6], 0.2523132562637329f * a[2] * b[2]) + fmaf(0.0901118740439415f, a[7] * b[7], -0.12615662813186646f * a[3] * b[3])));
+        o[7] = ((fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), 0.282094806432724f * (a[0] * b[7] + a[7] * b[0])) + 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2])) + (0.15607835352420807f * (a[4] * b[5] + a[5] * b[4]) + 0.0901118740439415f * (a[6] * b[7] + a[7] * b[6])));
+        o[8] = ((fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), 0.282094806432724f * (a[0] * b[8] + a[8] * b[0])) + fmaf(0.15607835352420807f, a[7] * b[7], -0.21850968897342682f * a[1] * b[1])) + (0.21850968897342682f * a[3] * b[3] + -0.15607835352420807f * a[5] * b[5]));
+    }
+    __device__ __forceinline__ static void mul_onto_lobe(const float* __restrict__ a, const float* __restrict__ b,
                                                float* __restrict__ o) {
         o[0] = ((fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])) + fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1])) + (fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]) + fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])));
         o[1] = ((fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0])) + -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1])) + (-0.21850968897342682f * (a[1] * b[8] + a[8] * b[1]) + 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2])));
@@ -563,7 +606,7 @@ template <> struct SH<4> {
         gz = w[2] + 3.0f * a_t23 + t19 * a_t20 + 3.0f * a_t19 + 0.6666666865348816f * a_t17 + t14 * a_t15 + z * a_t12 + z * a_t12;
     }
     static constexpr int NA = 20;   // monomials of degree < n
-    static constexpr int NG = 30;   // gradient coefficients, bands >= 1
+    static constexpr int NG = 19;   // symmetric tensor entries, bands >= 1
     __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
         (void)x; (void)y; (void)z;
         const float m1_0_0 = x;
@@ -662,52 +705,42 @@ template <> struct SH<4> {
         gq[3] = (-1.0f * w[6] + 6.0f * w[8]);
         gq[4] = 6.0f * w[4];
         gq[5] = 3.0f * w[7];
-        gq[6] = 6.0f * w[4];
-        gq[7] = (-1.0f * w[6] + -6.0f * w[8]);
-        gq[8] = 3.0f * w[5];
-        gq[9] = 3.0f * w[7];
-        gq[10] = 3.0f * w[5];
-        gq[11] = 2.0f * w[6];
-        gq[12] = (-4.5f * w[13] + 45.0f * w[15]);
-        gq[13] = (90.0f * w[9] + -3.0f * w[11]);
-        gq[14] = (-3.0f * w[12] + 30.0f * w[14]);
-        gq[15] = (-1.5f * w[13] + -45.0f * w[15]);
-        gq[16] = 30.0f * w[10];
-        gq[17] = 6.0f * w[13];
-        gq[18] = (45.0f * w[9] + -1.5f * w[11]);
-        gq[19] = (-3.0f * w[13] + -90.0f * w[15]);
-        gq[20] = 30.0f * w[10];
-        gq[21] = (-45.0f * w[9] + -4.5f * w[11]);
-        gq[22] = (-3.0f * w[12] + -30.0f * w[14]);
-        gq[23] = 6.0f * w[11];
-        gq[24] = (-1.5f * w[12] + 15.0f * w[14]);
-        gq[25] = 30.0f * w[10];
-        gq[26] = 12.0f * w[13];
-        gq[27] = (-1.5f * w[12] + -15.0f * w[14]);
-        gq[28] = 12.0f * w[11];
-        gq[29] = 3.0f * w[12];
+        gq[6] = (-1.0f * w[6] + -6.0f * w[8]);
+        gq[7] = 3.0f * w[5];
+        gq[8] = 2.0f * w[6];
+        gq[9] = (-4.5f * w[13] + 45.0f * w[15]);
+        gq[10] = (45.0f * w[9] + -1.5f * w[11]);
+        gq[11] = (-1.5f * w[12] + 15.0f * w[14]);
+        gq[12] = (-1.5f * w[13] + -45.0f * w[15]);
+        gq[13] = 15.0f * w[10];
+        gq[14] = 6.0f * w[13];
+        gq[15] = (-45.0f * w[9] + -4.5f * w[11]);
+        gq[16] = (-1.5f * w[12] + -15.0f * w[14]);
+        gq[17] = 6.0f * w[11];
+        gq[18] = 3.0f * w[12];
     }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
+    template <class Q>
+    __device__ __forceinline__ static void grad_eval2(float2 x, float2 y, float2 z, Q&& gq,
+                                                      float2* gx, float2* gy, float2* gz) {
         (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        const float u1_0_0 = x;
-        const float u0_1_0 = y;
-        const float u0_0_1 = z;
-        const float u2_0_0 = x * u1_0_0;
-        const float u1_1_0 = x * u0_1_0;
-        const float u1_0_1 = x * u0_0_1;
-        const float u0_2_0 = y * u0_1_0;
-        const float u0_1_1 = y * u0_0_1;
-        const float u0_0_2 = z * u0_0_1;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
-        gx[1] = gq[3] * u1_0_0 + gq[4] * u0_1_0 + gq[5] * u0_0_1;
-        gy[1] = gq[6] * u1_0_0 + gq[7] * u0_1_0 + gq[8] * u0_0_1;
-        gz[1] = gq[9] * u1_0_0 + gq[10] * u0_1_0 + gq[11] * u0_0_1;
-        gx[2] = gq[12] * u2_0_0 + gq[13] * u1_1_0 + gq[14] * u1_0_1 + gq[15] * u0_2_0 + gq[16] * u0_1_1 + gq[17] * u0_0_2;
-        gy[2] = gq[18] * u2_0_0 + gq[19] * u1_1_0 + gq[20] * u1_0_1 + gq[21] * u0_2_0 + gq[22] * u0_1_1 + gq[23] * u0_0_2;
-        gz[2] = gq[24] * u2_0_0 + gq[25] * u1_1_0 + gq[26] * u1_0_1 + gq[27] * u0_2_0 + gq[28] * u0_1_1 + gq[29] * u0_0_2;
+        const float2 x2 = __fmul2_rn(make_float2(2.0f, 2.0f), x);
+        const float2 y2 = __fmul2_rn(make_float2(2.0f, 2.0f), y);
+        const float2 z2 = __fmul2_rn(make_float2(2.0f, 2.0f), z);
+        const float2 u2_0_0 = __fmul2_rn(x, x);
+        const float2 u1_1_0 = __fmul2_rn(y, x2);
+        const float2 u1_0_1 = __fmul2_rn(z, x2);
+        const float2 u0_2_0 = __fmul2_rn(y, y);
+        const float2 u0_1_1 = __fmul2_rn(z, y2);
+        const float2 u0_0_2 = __fmul2_rn(z, z);
+        gx[0] = gq(0);
+        gy[0] = gq(1);
+        gz[0] = gq(2);
+        gx[1] = __ffma2_rn(gq(5), z, __ffma2_rn(gq(4), y, __fmul2_rn(gq(3), x)));
+        gy[1] = __ffma2_rn(gq(7), z, __ffma2_rn(gq(6), y, __fmul2_rn(gq(4), x)));
+        gz[1] = __ffma2_rn(gq(8), z, __ffma2_rn(gq(7), y, __fmul2_rn(gq(5), x)));
+        gx[2] = __ffma2_rn(gq(14), u0_0_2, __ffma2_rn(gq(13), u0_1_1, __ffma2_rn(gq(12), u0_2_0, __ffma2_rn(gq(11), u1_0_1, __ffma2_rn(gq(10), u1_1_0, __fmul2_rn(gq(9), u2_0_0))))));
+        gy[2] = __ffma2_rn(gq(17), u0_0_2, __ffma2_rn(gq(16), u0_1_1, __ffma2_rn(gq(15), u0_2_0, __ffma2_rn(gq(13), u1_0_1, __ffma2_rn(gq(12), u1_1_0, __fmul2_rn(gq(10), u2_0_0))))));
+        gz[2] = __ffma2_rn(gq(18), u0_0_2, __ffma2_rn(gq(17), u0_1_1, __ffma2_rn(gq(16), u0_2_0, __ffma2_rn(gq(14), u1_0_1, __ffma2_rn(gq(13), u1_1_0, __fmul2_rn(gq(11), u2_0_0))))));
     }
     __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,
                                                float* __restrict__ o) {
@@ -727,6 +760,44 @@ template <> struct SH<4> {
         o[13] = ((fmaf(-0.09403159469366074f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.12615662813186646f, (a[6] * b[13] + a[13] * b[6]), fmaf(-0.05839917063713074f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[13] + a[13] * b[0])))) + fmaf(0.059470802545547485f, (a[7] * b[12] + a[12] * b[7]), fmaf(-0.09403159469366074f, (a[4] * b[9] + a[9] * b[4]), -0.05839917063713074f * (a[1] * b[4] + a[4] * b[1])))) + (fmaf(0.11516471952199936f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.14567312598228455f, (a[4] * b[11] + a[11] * b[4]), 0.23359668254852295f * (a[2] * b[7] + a[7] * b[2]))) + fmaf(0.14567312598228455f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.11516471952199936f, (a[5] * b[10] + a[10] * b[5]), 0.20230065286159515f * (a[3] * b[6] + a[6] * b[3])))));
         o[14] = ((fmaf(-0.18806318938732147f, (a[8] * b[12] + a[12] * b[8]), fmaf(0.1486770063638687f, (a[5] * b[9] + a[9] * b[5]), 0.282094806432724f * (a[0] * b[14] + a[14] * b[0]))) + fmaf(-0.11516471952199936f, (a[5] * b[11] + a[11] * b[5]), -0.18467439711093903f * (a[1] * b[5] + a[5] * b[1]))) + (fmaf(0.11516471952199936f, (a[7] * b[13] + a[13] * b[7]), 0.18467439711093903f * (a[2] * b[8] + a[8] * b[2])) + fmaf(0.1486770063638687f, (a[7] * b[15] + a[15] * b[7]), 0.18467439711093903f * (a[3] * b[7] + a[7] * b[3]))));
         o[15] = ((fmaf(-0.1486770063638687f, (a[5] * b[10] + a[10] * b[5]), 0.282094806432724f * (a[0] * b[15] + a[15] * b[0])) + fmaf(-0.2102610468864441f, (a[6] * b[15] + a[15] * b[6]), -0.22617901861667633f * (a[1] * b[4] + a[4] * b[1]))) + (fmaf(0.1486770063638687f, (a[7] * b[14] + a[14] * b[7]), 0.22617901861667633f * (a[3] * b[8] + a[8] * b[3])) + fmaf(-0.09403159469366074f, (a[8] * b[13] + a[13] * b[8]), 0.09403159469366074f * (a[4] * b[11] + a[11] * b[4]))));
+    }
+    __device__ __forceinline__ static void mul_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])) + fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1])) + (fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]) + fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])));
+        o[1] = ((fmaf(0.05839917063713074f, a[11] * b[8], fmaf(-0.18467439711093903f, a[14] * b[5], fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0])))) + fmaf(0.20230065286159515f, a[11] * b[6], fmaf(-0.05839917063713074f, a[13] * b[4], -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1])))) + (fmaf(0.18467439711093903f, a[10] * b[7], fmaf(-0.22617901861667633f, a[15] * b[4], -0.21850968897342682f * (a[1] * b[8] + a[8] * b[1]))) + fmaf(0.22617901861667633f, a[9] * b[8], fmaf(-0.14304816722869873f, a[12] * b[5], 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2])))));
+        o[2] = ((fmaf(0.18467439711093903f, a[14] * b[8], fmaf(0.18467439711093903f, a[10] * b[4], 0.282094806432724f * (a[0] * b[2] + a[2] * b[0]))) + fmaf(0.23359668254852295f, a[11] * b[5], 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1]))) + (fmaf(0.24776668846607208f, a[12] * b[6], 0.2523132562637329f * (a[2] * b[6] + a[6] * b[2])) + fmaf(0.23359668254852295f, a[13] * b[7], 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3]))));
+        o[3] = ((fmaf(0.22617901861667633f, a[15] * b[8], fmaf(0.20230065286159515f, a[13] * b[6], fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0])))) + fmaf(-0.14304816722869873f, a[12] * b[7], fmaf(0.22617901861667633f, a[9] * b[4], 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1])))) + (fmaf(0.18467439711093903f, a[14] * b[7], fmaf(-0.05839917063713074f, a[11] * b[4], 0.21850968897342682f * (a[2] * b[7] + a[7] * b[2]))) + fmaf(-0.05839917063713074f, a[13] * b[8], fmaf(0.18467439711093903f, a[10] * b[5], -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3])))));
+        o[4] = ((fmaf(0.15607835352420807f, (a[5] * b[7] + a[7] * b[5]), fmaf(0.18467439711093903f, a[10] * b[2], 0.282094806432724f * (a[0] * b[4] + a[4] * b[0]))) + fmaf(0.22617901861667633f, a[9] * b[3], 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1]))) + (fmaf(-0.05839917063713074f, a[11] * b[3], -0.05839917063713074f * a[13] * b[1]) + fmaf(-0.180223748087883f, (a[4] * b[6] + a[6] * b[4]), -0.22617901861667633f * a[15] * b[1])));
+        o[5] = ((fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), fmaf(0.23359668254852295f, a[11] * b[2], 0.282094806432724f * (a[0] * b[5] + a[5] * b[0]))) + fmaf(0.18467439711093903f, a[10] * b[3], 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1]))) + (fmaf(0.15607835352420807f, (a[4] * b[7] + a[7] * b[4]), -0.14304816722869873f * a[12] * b[1]) + fmaf(0.0901118740439415f, (a[5] * b[6] + a[6] * b[5]), -0.18467439711093903f * a[14] * b[1])));
+        o[6] = ((fmaf(0.0901118740439415f, a[5] * b[5], fmaf(0.24776668846607208f, a[12] * b[2], 0.282094806432724f * (a[0] * b[6] + a[6] * b[0]))) + fmaf(0.180223748087883f, a[6] * b[6], fmaf(-0.12615662813186646f, a[3] * b[3], -0.12615662813186646f * a[1] * b[1]))) + (fmaf(0.0901118740439415f, a[7] * b[7], fmaf(0.20230065286159515f, a[13] * b[3], 0.20230065286159515f * a[11] * b[1])) + fmaf(-0.180223748087883f, a[8] * b[8], fmaf(-0.180223748087883f, a[4] * b[4], 0.2523132562637329f * a[2] * b[2]))));
+        o[7] = ((fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), fmaf(-0.14304816722869873f, a[12] * b[3], 0.282094806432724f * (a[0] * b[7] + a[7] * b[0]))) + fmaf(0.18467439711093903f, a[14] * b[3], 0.18467439711093903f * a[10] * b[1])) + (fmaf(0.15607835352420807f, (a[4] * b[5] + a[5] * b[4]), 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2])) + fmaf(0.0901118740439415f, (a[6] * b[7] + a[7] * b[6]), 0.23359668254852295f * a[13] * b[2])));
+        o[8] = ((fmaf(-0.15607835352420807f, a[5] * b[5], fmaf(0.18467439711093903f, a[14] * b[2], 0.282094806432724f * (a[0] * b[8] + a[8] * b[0]))) + fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), fmaf(0.21850968897342682f, a[3] * b[3], -0.21850968897342682f * a[1] * b[1]))) + (fmaf(0.15607835352420807f, a[7] * b[7], fmaf(-0.05839917063713074f, a[13] * b[3], 0.22617901861667633f * a[9] * b[1])) + fmaf(0.22617901861667633f, a[15] * b[3], 0.05839917063713074f * a[11] * b[1])));
+        o[9] = ((fmaf(0.1486770063638687f, a[14] * b[5], 0.282094806432724f * a[9] * b[0]) + fmaf(-0.2102610468864441f, a[9] * b[6], 0.22617901861667633f * (a[1] * b[8] + a[8] * b[1]))) + (fmaf(0.1486770063638687f, a[10] * b[7], 0.22617901861667633f * (a[3] * b[4] + a[4] * b[3])) + fmaf(-0.09403159469366074f, a[11] * b[8], -0.09403159469366074f * a[13] * b[4])));
+        o[10] = ((fmaf(0.11516471952199936f, a[11] * b[7], fmaf(-0.18806318938732147f, a[12] * b[4], 0.282094806432724f * a[10] * b[0])) + fmaf(0.11516471952199936f, a[13] * b[5], 0.18467439711093903f * (a[1] * b[7] + a[7] * b[1]))) + (fmaf(-0.1486770063638687f, a[15] * b[5], 0.18467439711093903f * (a[2] * b[4] + a[4] * b[2])) + fmaf(0.1486770063638687f, a[9] * b[7], 0.18467439711093903f * (a[3] * b[5] + a[5] * b[3]))));
+        o[11] = ((fmaf(-0.14567312598228455f, a[11] * b[8], fmaf(-0.11516471952199936f, a[14] * b[5], fmaf(-0.05839917063713074f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * a[11] * b[0]))) + fmaf(0.12615662813186646f, a[11] * b[6], fmaf(0.14567312598228455f, a[13] * b[4], 0.20230065286159515f * (a[1] * b[6] + a[6] * b[1])))) + (fmaf(0.11516471952199936f, a[10] * b[7], fmaf(0.09403159469366074f, a[15] * b[4], 0.05839917063713074f * (a[1] * b[8] + a[8] * b[1]))) + fmaf(-0.09403159469366074f, a[9] * b[8], fmaf(0.059470802545547485f, a[12] * b[5], 0.23359668254852295f * (a[2] * b[5] + a[5] * b[2])))));
+        o[12] = ((fmaf(-0.18806318938732147f, a[14] * b[8], fmaf(-0.18806318938732147f, a[10] * b[4], 0.282094806432724f * a[12] * b[0])) + fmaf(0.059470802545547485f, a[11] * b[5], -0.14304816722869873f * (a[1] * b[5] + a[5] * b[1]))) + (fmaf(0.16820883750915527f, a[12] * b[6], 0.24776668846607208f * (a[2] * b[6] + a[6] * b[2])) + fmaf(0.059470802545547485f, a[13] * b[7], -0.14304816722869873f * (a[3] * b[7] + a[7] * b[3]))));
+        o[13] = ((fmaf(-0.09403159469366074f, a[15] * b[8], fmaf(0.12615662813186646f, a[13] * b[6], fmaf(-0.05839917063713074f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * a[13] * b[0]))) + fmaf(0.059470802545547485f, a[12] * b[7], fmaf(-0.09403159469366074f, a[9] * b[4], -0.05839917063713074f * (a[1] * b[4] + a[4] * b[1])))) + (fmaf(0.11516471952199936f, a[14] * b[7], fmaf(0.14567312598228455f, a[11] * b[4], 0.23359668254852295f * (a[2] * b[7] + a[7] * b[2]))) + fmaf(0.14567312598228455f, a[13] * b[8], fmaf(0.11516471952199936f, a[10] * b[5], 0.20230065286159515f * (a[3] * b[6] + a[6] * b[3])))));
+        o[14] = ((fmaf(-0.18806318938732147f, a[12] * b[8], fmaf(0.1486770063638687f, a[9] * b[5], 0.282094806432724f * a[14] * b[0])) + fmaf(-0.11516471952199936f, a[11] * b[5], -0.18467439711093903f * (a[1] * b[5] + a[5] * b[1]))) + (fmaf(0.11516471952199936f, a[13] * b[7], 0.18467439711093903f * (a[2] * b[8] + a[8] * b[2])) + fmaf(0.1486770063638687f, a[15] * b[7], 0.18467439711093903f * (a[3] * b[7] + a[7] * b[3]))));
+        o[15] = ((fmaf(-0.1486770063638687f, a[10] * b[5], 0.282094806432724f * a[15] * b[0]) + fmaf(-0.2102610468864441f, a[15] * b[6], -0.22617901861667633f * (a[1] * b[4] + a[4] * b[1]))) + (fmaf(0.1486770063638687f, a[14] * b[7], 0.22617901861667633f * (a[3] * b[8] + a[8] * b[3])) + fmaf(-0.09403159469366074f, a[13] * b[8], 0.09403159469366074f * a[11] * b[4])));
+    }
+    __device__ __forceinline__ static void mul_onto_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((fmaf(0.282094806432724f, a[12] * b[12], fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0]))) + fmaf(0.282094806432724f, a[13] * b[13], fmaf(0.282094806432724f, a[9] * b[9], fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1])))) + (fmaf(0.282094806432724f, a[14] * b[14], fmaf(0.282094806432724f, a[10] * b[10], fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]))) + fmaf(0.282094806432724f, a[15] * b[15], fmaf(0.282094806432724f, a[11] * b[11], fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])))));
+        o[1] = ((fmaf(0.05839917063713074f, (a[8] * b[11] + a[11] * b[8]), fmaf(-0.18467439711093903f, (a[5] * b[14] + a[14] * b[5]), fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0])))) + fmaf(0.20230065286159515f, (a[6] * b[11] + a[11] * b[6]), fmaf(-0.05839917063713074f, (a[4] * b[13] + a[13] * b[4]), -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1])))) + (fmaf(0.18467439711093903f, (a[7] * b[10] + a[10] * b[7]), fmaf(-0.22617901861667633f, (a[4] * b[15] + a[15] * b[4]), -0.21850968897342682f * (a[1] * b[8] + a[8] * b[1]))) + fmaf(0.22617901861667633f, (a[8] * b[9] + a[9] * b[8]), fmaf(-0.14304816722869873f, (a[5] * b[12] + a[12] * b[5]), 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2])))));
+        o[2] = ((fmaf(0.18467439711093903f, (a[8] * b[14] + a[14] * b[8]), fmaf(0.18467439711093903f, (a[4] * b[10] + a[10] * b[4]), 0.282094806432724f * (a[0] * b[2] + a[2] * b[0]))) + fmaf(0.23359668254852295f, (a[5] * b[11] + a[11] * b[5]), 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1]))) + (fmaf(0.24776668846607208f, (a[6] * b[12] + a[12] * b[6]), 0.2523132562637329f * (a[2] * b[6] + a[6] * b[2])) + fmaf(0.23359668254852295f, (a[7] * b[13] + a[13] * b[7]), 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3]))));
+        o[3] = ((fmaf(0.22617901861667633f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.20230065286159515f, (a[6] * b[13] + a[13] * b[6]), fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0])))) + fmaf(-0.14304816722869873f, (a[7] * b[12] + a[12] * b[7]), fmaf(0.22617901861667633f, (a[4] * b[9] + a[9] * b[4]), 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1])))) + (fmaf(0.18467439711093903f, (a[7] * b[14] + a[14] * b[7]), fmaf(-0.05839917063713074f, (a[4] * b[11] + a[11] * b[4]), 0.21850968897342682f * (a[2] * b[7] + a[7] * b[2]))) + fmaf(-0.05839917063713074f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.18467439711093903f, (a[5] * b[10] + a[10] * b[5]), -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3])))));
+        o[4] = ((fmaf(0.09403159469366074f, (a[11] * b[15] + a[15] * b[11]), fmaf(0.15607835352420807f, (a[5] * b[7] + a[7] * b[5]), fmaf(0.18467439711093903f, (a[2] * b[10] + a[10] * b[2]), 0.282094806432724f * (a[0] * b[4] + a[4] * b[0])))) + fmaf(-0.09403159469366074f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.22617901861667633f, (a[3] * b[9] + a[9] * b[3]), 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1])))) + (fmaf(-0.18806318938732147f, (a[10] * b[12] + a[12] * b[10]), fmaf(-0.05839917063713074f, (a[3] * b[11] + a[11] * b[3]), -0.05839917063713074f * (a[1] * b[13] + a[13] * b[1]))) + fmaf(0.14567312598228455f, (a[11] * b[13] + a[13] * b[11]), fmaf(-0.180223748087883f, (a[4] * b[6] + a[6] * b[4]), -0.22617901861667633f * (a[1] * b[15] + a[15] * b[1])))));
+        o[5] = ((fmaf(0.059470802545547485f, (a[11] * b[12] + a[12] * b[11]), fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), fmaf(0.23359668254852295f, (a[2] * b[11] + a[11] * b[2]), 0.282094806432724f * (a[0] * b[5] + a[5] * b[0])))) + fmaf(-0.11516471952199936f, (a[11] * b[14] + a[14] * b[11]), fmaf(0.1486770063638687f, (a[9] * b[14] + a[14] * b[9]), fmaf(0.18467439711093903f, (a[3] * b[10] + a[10] * b[3]), 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1]))))) + (fmaf(0.11516471952199936f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.15607835352420807f, (a[4] * b[7] + a[7] * b[4]), -0.14304816722869873f * (a[1] * b[12] + a[12] * b[1]))) + fmaf(-0.1486770063638687f, (a[10] * b[15] + a[15] * b[10]), fmaf(0.0901118740439415f, (a[5] * b[6] + a[6] * b[5]), -0.18467439711093903f * (a[1] * b[14] + a[14] * b[1])))));
+        o[6] = ((fmaf(-0.2102610468864441f, a[15] * b[15], fmaf(-0.2102610468864441f, a[9] * b[9], fmaf(0.0901118740439415f, a[5] * b[5], fmaf(0.24776668846607208f, (a[2] * b[12] + a[12] * b[2]), 0.282094806432724f * (a[0] * b[6] + a[6] * b[0]))))) + fmaf(0.12615662813186646f, a[11] * b[11], fmaf(0.180223748087883f, a[6] * b[6], fmaf(-0.12615662813186646f, a[3] * b[3], -0.12615662813186646f * a[1] * b[1])))) + (fmaf(0.16820883750915527f, a[12] * b[12], fmaf(0.0901118740439415f, a[7] * b[7], fmaf(0.20230065286159515f, (a[3] * b[13] + a[13] * b[3]), 0.20230065286159515f * (a[1] * b[11] + a[11] * b[1])))) + fmaf(0.12615662813186646f, a[13] * b[13], fmaf(-0.180223748087883f, a[8] * b[8], fmaf(-0.180223748087883f, a[4] * b[4], 0.2523132562637329f * a[2] * b[2])))));
+        o[7] = ((fmaf(0.11516471952199936f, (a[13] * b[14] + a[14] * b[13]), fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), fmaf(-0.14304816722869873f, (a[3] * b[12] + a[12] * b[3]), 0.282094806432724f * (a[0] * b[7] + a[7] * b[0])))) + fmaf(0.1486770063638687f, (a[14] * b[15] + a[15] * b[14]), fmaf(0.1486770063638687f, (a[9] * b[10] + a[10] * b[9]), fmaf(0.18467439711093903f, (a[3] * b[14] + a[14] * b[3]), 0.18467439711093903f * (a[1] * b[10] + a[10] * b[1]))))) + (fmaf(0.11516471952199936f, (a[10] * b[11] + a[11] * b[10]), fmaf(0.15607835352420807f, (a[4] * b[5] + a[5] * b[4]), 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2]))) + fmaf(0.059470802545547485f, (a[12] * b[13] + a[13] * b[12]), fmaf(0.0901118740439415f, (a[6] * b[7] + a[7] * b[6]), 0.23359668254852295f * (a[2] * b[13] + a[13] * b[2])))));
+        o[8] = ((fmaf(-0.14567312598228455f, a[11] * b[11], fmaf(-0.15607835352420807f, a[5] * b[5], fmaf(0.18467439711093903f, (a[2] * b[14] + a[14] * b[2]), 0.282094806432724f * (a[0] * b[8] + a[8] * b[0])))) + fmaf(-0.18806318938732147f, (a[12] * b[14] + a[14] * b[12]), fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), fmaf(0.21850968897342682f, a[3] * b[3], -0.21850968897342682f * a[1] * b[1])))) + (fmaf(0.14567312598228455f, a[13] * b[13], fmaf(0.15607835352420807f, a[7] * b[7], fmaf(-0.05839917063713074f, (a[3] * b[13] + a[13] * b[3]), 0.22617901861667633f * (a[1] * b[9] + a[9] * b[1])))) + fmaf(-0.09403159469366074f, (a[13] * b[15] + a[15] * b[13]), fmaf(-0.09403159469366074f, (a[9] * b[11] + a[11] * b[9]), fmaf(0.22617901861667633f, (a[3] * b[15] + a[15] * b[3]), 0.05839917063713074f * (a[1] * b[11] + a[11] * b[1]))))));
+        o[9] = 0.0f;
+        o[10] = 0.0f;
+        o[11] = 0.0f;
+        o[12] = 0.0f;
+        o[13] = 0.0f;
+        o[14] = 0.0f;
+        o[15] = 0.0f;
     }
     __device__ __forceinline__ static void sqr(const float* __restrict__ a, float* __restrict__ o) {
         o[0] = ((fmaf(0.282094806432724f, a[12] * a[12], fmaf(0.282094806432724f, a[8] * a[8], fmaf(0.282094806432724f, a[4] * a[4], 0.282094806432724f * a[0] * a[0]))) + fmaf(0.282094806432724f, a[13] * a[13], fmaf(0.282094806432724f, a[9] * a[9], fmaf(0.282094806432724f, a[5] * a[5], 0.282094806432724f * a[1] * a[1])))) + (fmaf(0.282094806432724f, a[14] * a[14], fmaf(0.282094806432724f, a[10] * a[10], fmaf(0.282094806432724f, a[6] * a[6], 0.282094806432724f * a[2] * a[2]))) + fmaf(0.282094806432724f, a[15] * a[15], fmaf(0.282094806432724f, a[11] * a[11], fmaf(0.282094806432724f, a[7] * a[7], 0.282094806432724f * a[3] * a[3])))));
@@ -1025,7 +1096,7 @@ template <> struct SH<5> {
         gz = w[2] + 15.0f * a_t42 + t38 * a_t39 + 3.0f * a_t37 + t32 * a_t33 + t29 * a_t30 + 3.0f * a_t29 + t24 * a_t25 + 0.6666666865348816f * a_t23 + t20 * a_t21 + z * a_t18 + z * a_t18;
     }
     static constexpr int NA = 35;   // monomials of degree < n
-    static constexpr int NG = 60;   // gradient coefficients, bands >= 1
+    static constexpr int NG = 34;   // symmetric tensor entries, bands >= 1
     __device__ __forceinline__ static void accumulate(const float* G, float x, float y, float z, float* acc) {
         (void)x; (void)y; (void)z;
         const float m1_0_0 = x;
@@ -1183,95 +1254,73 @@ template <> struct SH<5> {
         gq[3] = (-1.0f * w[6] + 6.0f * w[8]);
         gq[4] = 6.0f * w[4];
         gq[5] = 3.0f * w[7];
-        gq[6] = 6.0f * w[4];
-        gq[7] = (-1.0f * w[6] + -6.0f * w[8]);
-        gq[8] = 3.0f * w[5];
-        gq[9] = 3.0f * w[7];
-        gq[10] = 3.0f * w[5];
-        gq[11] = 2.0f * w[6];
-        gq[12] = (-4.5f * w[13] + 45.0f * w[15]);
-        gq[13] = (90.0f * w[9] + -3.0f * w[11]);
-        gq[14] = (-3.0f * w[12] + 30.0f * w[14]);
-        gq[15] = (-1.5f * w[13] + -45.0f * w[15]);
-        gq[16] = 30.0f * w[10];
-        gq[17] = 6.0f * w[13];
-        gq[18] = (45.0f * w[9] + -1.5f * w[11]);
-        gq[19] = (-3.0f * w[13] + -90.0f * w[15]);
-        gq[20] = 30.0f * w[10];
-        gq[21] = (-45.0f * w[9] + -4.5f * w[11]);
-        gq[22] = (-3.0f * w[12] + -30.0f * w[14]);
-        gq[23] = 6.0f * w[11];
-        gq[24] = (-1.5f * w[12] + 15.0f * w[14]);
-        gq[25] = 30.0f * w[10];
-        gq[26] = 12.0f * w[13];
-        gq[27] = (-1.5f * w[12] + -15.0f * w[14]);
-        gq[28] = 12.0f * w[11];
-        gq[29] = 3.0f * w[12];
-        gq[30] = ((1.5f * w[20] + -30.0f * w[22]) + 420.0f * w[24]);
-        gq[31] = (1260.0f * w[16] + -45.0f * w[18]);
-        gq[32] = (-22.5f * w[21] + 315.0f * w[23]);
-        gq[33] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[34] = (630.0f * w[17] + -15.0f * w[19]);
-        gq[35] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[36] = (-420.0f * w[16] + -15.0f * w[18]);
-        gq[37] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[38] = 90.0f * w[18];
-        gq[39] = 10.0f * w[21];
-        gq[40] = (420.0f * w[16] + -15.0f * w[18]);
-        gq[41] = (1.5f * w[20] + -1260.0f * w[24]);
-        gq[42] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[43] = (-1260.0f * w[16] + -45.0f * w[18]);
-        gq[44] = (-15.0f * w[21] + -630.0f * w[23]);
-        gq[45] = 90.0f * w[18];
-        gq[46] = ((1.5f * w[20] + 30.0f * w[22]) + 420.0f * w[24]);
-        gq[47] = (-315.0f * w[17] + -22.5f * w[19]);
-        gq[48] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[49] = 10.0f * w[19];
-        gq[50] = (-7.5f * w[21] + 105.0f * w[23]);
-        gq[51] = (315.0f * w[17] + -7.5f * w[19]);
-        gq[52] = (-6.0f * w[20] + 90.0f * w[22]);
-        gq[53] = (-7.5f * w[21] + -315.0f * w[23]);
-        gq[54] = 180.0f * w[18];
-        gq[55] = 30.0f * w[21];
-        gq[56] = (-105.0f * w[17] + -7.5f * w[19]);
-        gq[57] = (-6.0f * w[20] + -90.0f * w[22]);
-        gq[58] = 30.0f * w[19];
-        gq[59] = 4.0f * w[20];
+        gq[6] = (-1.0f * w[6] + -6.0f * w[8]);
+        gq[7] = 3.0f * w[5];
+        gq[8] = 2.0f * w[6];
+        gq[9] = (-4.5f * w[13] + 45.0f * w[15]);
+        gq[10] = (45.0f * w[9] + -1.5f * w[11]);
+        gq[11] = (-1.5f * w[12] + 15.0f * w[14]);
+        gq[12] = (-1.5f * w[13] + -45.0f * w[15]);
+        gq[13] = 15.0f * w[10];
+        gq[14] = 6.0f * w[13];
+        gq[15] = (-45.0f * w[9] + -4.5f * w[11]);
+        gq[16] = (-1.5f * w[12] + -15.0f * w[14]);
+        gq[17] = 6.0f * w[11];
+        gq[18] = 3.0f * w[12];
+        gq[19] = ((1.5f * w[20] + -30.0f * w[22]) + 420.0f * w[24]);
+        gq[20] = (420.0f * w[16] + -15.0f * w[18]);
+        gq[21] = (-7.5f * w[21] + 105.0f * w[23]);
+        gq[22] = (0.5f * w[20] + -420.0f * w[24]);
+        gq[23] = (105.0f * w[17] + -2.5f * w[19]);
+        gq[24] = (-2.0f * w[20] + 30.0f * w[22]);
+        gq[25] = (-420.0f * w[16] + -15.0f * w[18]);
+        gq[26] = (-2.5f * w[21] + -105.0f * w[23]);
+        gq[27] = 30.0f * w[18];
+        gq[28] = 10.0f * w[21];
+        gq[29] = ((1.5f * w[20] + 30.0f * w[22]) + 420.0f * w[24]);
+        gq[30] = (-105.0f * w[17] + -7.5f * w[19]);
+        gq[31] = (-2.0f * w[20] + -30.0f * w[22]);
+        gq[32] = 10.0f * w[19];
+        gq[33] = 4.0f * w[20];
     }
-    __device__ __forceinline__ static void grad_eval(float x, float y, float z, const float* gq,
-                                                     float* gx, float* gy, float* gz) {
+    template <class Q>
+    __device__ __forceinline__ static void grad_eval2(float2 x, float2 y, float2 z, Q&& gq,
+                                                      float2* gx, float2* gy, float2* gz) {
         (void)x; (void)y; (void)z; (void)gq; (void)gx; (void)gy; (void)gz;
-        const float u1_0_0 = x;
-        const float u0_1_0 = y;
-        const float u0_0_1 = z;
-        const float u2_0_0 = x * u1_0_0;
-        const float u1_1_0 = x * u0_1_0;
-        const float u1_0_1 = x * u0_0_1;
-        const float u0_2_0 = y * u0_1_0;
-        const float u0_1_1 = y * u0_0_1;
-        const float u0_0_2 = z * u0_0_1;
-        const float u3_0_0 = x * u2_0_0;
-        const float u2_1_0 = x * u1_1_0;
-        const float u2_0_1 = x * u1_0_1;
-        const float u1_2_0 = x * u0_2_0;
-        const float u1_1_1 = x * u0_1_1;
-        const float u1_0_2 = x * u0_0_2;
-        const float u0_3_0 = y * u0_2_0;
-        const float u0_2_1 = y * u0_1_1;
-        const float u0_1_2 = y * u0_0_2;
-        const float u0_0_3 = z * u0_0_2;
-        gx[0] = gq[0];
-        gy[0] = gq[1];
-        gz[0] = gq[2];
-        gx[1] = gq[3] * u1_0_0 + gq[4] * u0_1_0 + gq[5] * u0_0_1;
-        gy[1] = gq[6] * u1_0_0 + gq[7] * u0_1_0 + gq[8] * u0_0_1;
-        gz[1] = gq[9] * u1_0_0 + gq[10] * u0_1_0 + gq[11] * u0_0_1;
-        gx[2] = gq[12] * u2_0_0 + gq[13] * u1_1_0 + gq[14] * u1_0_1 + gq[15] * u0_2_0 + gq[16] * u0_1_1 + gq[17] * u0_0_2;
-        gy[2] = gq[18] * u2_0_0 + gq[19] * u1_1_0 + gq[20] * u1_0_1 + gq[21] * u0_2_0 + gq[22] * u0_1_1 + gq[23] * u0_0_2;
-        gz[2] = gq[24] * u2_0_0 + gq[25] * u1_1_0 + gq[26] * u1_0_1 + gq[27] * u0_2_0 + gq[28] * u0_1_1 + gq[29] * u0_0_2;
-        gx[3] = gq[30] * u3_0_0 + gq[31] * u2_1_0 + gq[32] * u2_0_1 + gq[33] * u1_2_0 + gq[34] * u1_1_1 + gq[35] * u1_0_2 + gq[36] * u0_3_0 + gq[37] * u0_2_1 + gq[38] * u0_1_2 + gq[39] * u0_0_3;
-        gy[3] = gq[40] * u3_0_0 + gq[41] * u2_1_0 + gq[42] * u2_0_1 + gq[43] * u1_2_0 + gq[44] * u1_1_1 + gq[45] * u1_0_2 + gq[46] * u0_3_0 + gq[47] * u0_2_1 + gq[48] * u0_1_2 + gq[49] * u0_0_3;
-        gz[3] = gq[50] * u3_0_0 + gq[51] * u2_1_0 + gq[52] * u2_0_1 + gq[53] * u1_2_0 + gq[54] * u1_1_1 + gq[55] * u1_0_2 + gq[56] * u0_3_0 + gq[57] * u0_2_1 + gq[58] * u0_1_2 + gq[59] * u0_0_3;
+        const float2 x2 = __fmul2_rn(make_float2(2.0f, 2.0f), x);
+        const float2 y2 = __fmul2_rn(make_float2(2.0f, 2.0f), y);
+        const float2 z2 = __fmul2_rn(make_float2(2.0f, 2.0f), z);
+        const float2 u2_0_0 = __fmul2_rn(x, x);
+        const float2 u1_1_0 = __fmul2_rn(y, x2);
+        const float2 u1_0_1 = __fmul2_rn(z, x2);
+        const float2 u0_2_0 = __fmul2_rn(y, y);
+        const float2 u0_1_1 = __fmul2_rn(z, y2);
+        const float2 u0_0_2 = __fmul2_rn(z, z);
+        const float2 x3 = __fmul2_rn(make_float2(3.0f, 3.0f), x);
+        const float2 y3 = __fmul2_rn(make_float2(3.0f, 3.0f), y);
+        const float2 z3 = __fmul2_rn(make_float2(3.0f, 3.0f), z);
+        const float2 u3_0_0 = __fmul2_rn(u2_0_0, x);
+        const float2 u2_1_0 = __fmul2_rn(u2_0_0, y3);
+        const float2 u2_0_1 = __fmul2_rn(u2_0_0, z3);
+        const float2 u1_2_0 = __fmul2_rn(u0_2_0, x3);
+        const float2 u1_1_1 = __fmul2_rn(u0_1_1, x3);
+        const float2 u1_0_2 = __fmul2_rn(u0_0_2, x3);
+        const float2 u0_3_0 = __fmul2_rn(u0_2_0, y);
+        const float2 u0_2_1 = __fmul2_rn(u0_2_0, z3);
+        const float2 u0_1_2 = __fmul2_rn(u0_0_2, y3);
+        const float2 u0_0_3 = __fmul2_rn(u0_0_2, z);
+        gx[0] = gq(0);
+        gy[0] = gq(1);
+        gz[0] = gq(2);
+        gx[1] = __ffma2_rn(gq(5), z, __ffma2_rn(gq(4), y, __fmul2_rn(gq(3), x)));
+        gy[1] = __ffma2_rn(gq(7), z, __ffma2_rn(gq(6), y, __fmul2_rn(gq(4), x)));
+        gz[1] = __ffma2_rn(gq(8), z, __ffma2_rn(gq(7), y, __fmul2_rn(gq(5), x)));
+        gx[2] = __ffma2_rn(gq(14), u0_0_2, __ffma2_rn(gq(13), u0_1_1, __ffma2_rn(gq(12), u0_2_0, __ffma2_rn(gq(11), u1_0_1, __ffma2_rn(gq(10), u1_1_0, __fmul2_rn(gq(9), u2_0_0))))));
+        gy[2] = __ffma2_rn(gq(17), u0_0_2, __ffma2_rn(gq(16), u0_1_1, __ffma2_rn(gq(15), u0_2_0, __ffma2_rn(gq(13), u1_0_1, __ffma2_rn(gq(12), u1_1_0, __fmul2_rn(gq(10), u2_0_0))))));
+        gz[2] = __ffma2_rn(gq(18), u0_0_2, __ffma2_rn(gq(17), u0_1_1, __ffma2_rn(gq(16), u0_2_0, __ffma2_rn(gq(14), u1_0_1, __ffma2_rn(gq(13), u1_1_0, __fmul2_rn(gq(11), u2_0_0))))));
+        gx[3] = __ffma2_rn(gq(28), u0_0_3, __ffma2_rn(gq(27), u0_1_2, __ffma2_rn(gq(26), u0_2_1, __ffma2_rn(gq(25), u0_3_0, __ffma2_rn(gq(24), u1_0_2, __ffma2_rn(gq(23), u1_1_1, __ffma2_rn(gq(22), u1_2_0, __ffma2_rn(gq(21), u2_0_1, __ffma2_rn(gq(20), u2_1_0, __fmul2_rn(gq(19), u3_0_0))))))))));
+        gy[3] = __ffma2_rn(gq(32), u0_0_3, __ffma2_rn(gq(31), u0_1_2, __ffma2_rn(gq(30), u0_2_1, __ffma2_rn(gq(29), u0_3_0, __ffma2_rn(gq(27), u1_0_2, __ffma2_rn(gq(26), u1_1_1, __ffma2_rn(gq(25), u1_2_0, __ffma2_rn(gq(23), u2_0_1, __ffma2_rn(gq(22), u2_1_0, __fmul2_rn(gq(20), u3_0_0))))))))));
+        gz[3] = __ffma2_rn(gq(33), u0_0_3, __ffma2_rn(gq(32), u0_1_2, __ffma2_rn(gq(31), u0_2_1, __ffma2_rn(gq(30), u0_3_0, __ffma2_rn(gq(28), u1_0_2, __ffma2_rn(gq(27), u1_1_1, __ffma2_rn(gq(26), u1_2_0, __ffma2_rn(gq(24), u2_0_1, __ffma2_rn(gq(23), u2_1_0, __fmul2_rn(gq(21), u3_0_0))))))))));
     }
     __device__ __forceinline__ static void mul(const float* __restrict__ a, const float* __restrict__ b,
                                                float* __restrict__ o) {
@@ -1291,6 +1340,62 @@ template <> struct SH<5> {
         o[13] = ((fmaf(-0.11752006411552429f, (a[15] * b[24] + a[24] * b[15]), fmaf(0.11468784511089325f, (a[13] * b[22] + a[22] * b[13]), fmaf(0.10257992148399353f, (a[10] * b[19] + a[19] * b[10]), fmaf(-0.09403159469366074f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.12615662813186646f, (a[6] * b[13] + a[13] * b[6]), fmaf(0.16858388483524323f, (a[3] * b[22] + a[22] * b[3]), fmaf(0.23841361701488495f, (a[2] * b[21] + a[21] * b[2]), 0.282094806432724f * (a[0] * b[13] + a[13] * b[0])))))))) + fmaf(0.10257992148399353f, (a[14] * b[21] + a[21] * b[14]), fmaf(0.11468784511089325f, (a[11] * b[18] + a[18] * b[11]), fmaf(-0.11752006411552429f, (a[9] * b[16] + a[16] * b[9]), fmaf(0.059470802545547485f, (a[7] * b[12] + a[12] * b[7]), fmaf(-0.09403159469366074f, (a[4] * b[9] + a[9] * b[4]), fmaf(0.20230065286159515f, (a[3] * b[6] + a[6] * b[3]), -0.05839917063713074f * (a[1] * b[4] + a[4] * b[1])))))))) + (fmaf(0.06785023957490921f, (a[14] * b[23] + a[23] * b[14]), fmaf(0.09932258725166321f, (a[12] * b[21] + a[21] * b[12]), fmaf(0.1332552284002304f, (a[9] * b[18] + a[18] * b[9]), fmaf(0.11516471952199936f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.14567312598228455f, (a[4] * b[11] + a[11] * b[4]), fmaf(-0.05839917063713074f, (a[3] * b[8] + a[8] * b[3]), 0.16858388483524323f * (a[1] * b[18] + a[18] * b[1]))))))) + fmaf(0.1332552284002304f, (a[15] * b[22] + a[22] * b[15]), fmaf(0.025644980370998383f, (a[13] * b[20] + a[20] * b[13]), fmaf(0.06785023957490921f, (a[10] * b[17] + a[17] * b[10]), fmaf(0.14567312598228455f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.11516471952199936f, (a[5] * b[10] + a[10] * b[5]), fmaf(-0.15078601241111755f, (a[3] * b[20] + a[20] * b[3]), 0.23359668254852295f * (a[2] * b[7] + a[7] * b[2])))))))));
         o[14] = ((fmaf(0.06785023957490921f, (a[13] * b[23] + a[23] * b[13]), fmaf(0.06785023957490921f, (a[11] * b[17] + a[17] * b[11]), fmaf(0.1486770063638687f, (a[7] * b[15] + a[15] * b[7]), fmaf(0.1994711458683014f, (a[3] * b[23] + a[23] * b[3]), fmaf(0.18467439711093903f, (a[2] * b[8] + a[8] * b[2]), 0.282094806432724f * (a[0] * b[14] + a[14] * b[0])))))) + fmaf(-0.17951487004756927f, (a[14] * b[20] + a[20] * b[14]), fmaf(-0.10257992148399353f, (a[11] * b[19] + a[19] * b[11]), fmaf(-0.18806318938732147f, (a[8] * b[12] + a[12] * b[8]), fmaf(0.1486770063638687f, (a[5] * b[9] + a[9] * b[5]), fmaf(0.21324361860752106f, (a[2] * b[22] + a[22] * b[2]), -0.18467439711093903f * (a[1] * b[5] + a[5] * b[1]))))))) + (fmaf(0.15171775221824646f, (a[14] * b[24] + a[24] * b[14]), fmaf(-0.04441840946674347f, (a[12] * b[22] + a[22] * b[12]), fmaf(-0.09932258725166321f, (a[9] * b[19] + a[19] * b[9]), fmaf(-0.11516471952199936f, (a[5] * b[11] + a[11] * b[5]), fmaf(0.18467439711093903f, (a[3] * b[7] + a[7] * b[3]), 0.1994711458683014f * (a[1] * b[17] + a[17] * b[1])))))) + fmaf(-0.09932258725166321f, (a[15] * b[21] + a[21] * b[15]), fmaf(0.10257992148399353f, (a[13] * b[21] + a[21] * b[13]), fmaf(0.15171775221824646f, (a[10] * b[16] + a[16] * b[10]), fmaf(0.11516471952199936f, (a[7] * b[13] + a[13] * b[7]), fmaf(-0.07539300620555878f, (a[3] * b[21] + a[21] * b[3]), 0.07539300620555878f * (a[1] * b[19] + a[19] * b[1]))))))));
         o[15] = ((fmaf(0.07693494111299515f, (a[15] * b[20] + a[20] * b[15]), fmaf(-0.20355072617530823f, (a[12] * b[23] + a[23] * b[12]), fmaf(-0.09403159469366074f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.09403159469366074f, (a[4] * b[11] + a[11] * b[4]), fmaf(0.1628675013780594f, (a[2] * b[23] + a[23] * b[2]), 0.282094806432724f * (a[0] * b[15] + a[15] * b[0])))))) + fmaf(0.1332552284002304f, (a[13] * b[22] + a[22] * b[13]), fmaf(0.09932258725166321f, (a[10] * b[19] + a[19] * b[10]), fmaf(-0.1486770063638687f, (a[5] * b[10] + a[10] * b[5]), fmaf(0.22617901861667633f, (a[3] * b[8] + a[8] * b[3]), -0.22617901861667633f * (a[1] * b[4] + a[4] * b[1])))))) + (fmaf(-0.11752006411552429f, (a[13] * b[24] + a[24] * b[13]), fmaf(-0.11752006411552429f, (a[11] * b[16] + a[16] * b[11]), fmaf(-0.2102610468864441f, (a[6] * b[15] + a[15] * b[6]), fmaf(-0.04352817311882973f, (a[3] * b[22] + a[22] * b[3]), 0.23032943904399872f * (a[1] * b[16] + a[16] * b[1]))))) + fmaf(-0.09932258725166321f, (a[14] * b[21] + a[21] * b[14]), fmaf(-0.1332552284002304f, (a[11] * b[18] + a[18] * b[11]), fmaf(0.1486770063638687f, (a[7] * b[14] + a[14] * b[7]), fmaf(0.23032943904399872f, (a[3] * b[24] + a[24] * b[3]), 0.04352817311882973f * (a[1] * b[18] + a[18] * b[1])))))));
+        o[16] = ((fmaf(0.10652530938386917f, (a[16] * b[20] + a[20] * b[16]), fmaf(-0.07508081942796707f, (a[8] * b[18] + a[18] * b[8]), fmaf(-0.07508081942796707f, (a[4] * b[22] + a[22] * b[4]), 0.282094806432724f * (a[0] * b[16] + a[16] * b[0])))) + fmaf(-0.11909890919923782f, (a[17] * b[21] + a[21] * b[17]), fmaf(-0.11752006411552429f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.14046335220336914f, (a[5] * b[23] + a[23] * b[5]), 0.23032943904399872f * (a[1] * b[15] + a[15] * b[1]))))) + (fmaf(0.13504546880722046f, (a[18] * b[22] + a[22] * b[18]), fmaf(0.15171775221824646f, (a[10] * b[14] + a[14] * b[10]), fmaf(-0.2293756902217865f, (a[6] * b[16] + a[16] * b[6]), 0.23032943904399872f * (a[3] * b[9] + a[9] * b[3])))) + fmaf(-0.11909890919923782f, (a[19] * b[23] + a[23] * b[19]), fmaf(-0.11752006411552429f, (a[11] * b[15] + a[15] * b[11]), fmaf(0.14046335220336914f, (a[7] * b[17] + a[17] * b[7]), 0.23841361701488495f * (a[4] * b[8] + a[8] * b[4]))))));
+        o[17] = ((fmaf(0.11909890919923782f, (a[19] * b[24] + a[24] * b[19]), fmaf(-0.11909890919923782f, (a[16] * b[21] + a[21] * b[16]), fmaf(-0.11262122541666031f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[24] + a[24] * b[5]), fmaf(0.16858388483524323f, (a[4] * b[7] + a[7] * b[4]), 0.282094806432724f * (a[0] * b[17] + a[17] * b[0])))))) + fmaf(-0.15978795289993286f, (a[17] * b[20] + a[20] * b[17]), fmaf(-0.20355072617530823f, (a[9] * b[12] + a[12] * b[9]), fmaf(-0.057343922555446625f, (a[6] * b[17] + a[17] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[21] + a[21] * b[4]), 0.1994711458683014f * (a[1] * b[14] + a[14] * b[1])))))) + (fmaf(0.045015156269073486f, (a[18] * b[21] + a[21] * b[18]), fmaf(0.06785023957490921f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.14046335220336914f, (a[7] * b[16] + a[16] * b[7]), fmaf(0.16858388483524323f, (a[5] * b[8] + a[8] * b[5]), 0.1628675013780594f * (a[2] * b[9] + a[9] * b[2]))))) + fmaf(0.045015156269073486f, (a[19] * b[22] + a[22] * b[19]), fmaf(0.06785023957490921f, (a[11] * b[14] + a[14] * b[11]), fmaf(0.13272538781166077f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.13272538781166077f, (a[5] * b[22] + a[22] * b[5]), 0.1994711458683014f * (a[3] * b[10] + a[10] * b[3])))))));
+        o[18] = ((fmaf(0.10208478569984436f, (a[19] * b[21] + a[21] * b[19]), fmaf(0.13504546880722046f, (a[16] * b[22] + a[22] * b[16]), fmaf(0.1332552284002304f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.06553591042757034f, (a[6] * b[18] + a[18] * b[6]), fmaf(0.07508081942796707f, (a[4] * b[24] + a[24] * b[4]), fmaf(-0.04352817311882973f, (a[3] * b[9] + a[9] * b[3]), 0.282094806432724f * (a[0] * b[18] + a[18] * b[0]))))))) + fmaf(-0.045015156269073486f, (a[19] * b[23] + a[23] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[21] + a[21] * b[17]), fmaf(-0.04441840946674347f, (a[10] * b[12] + a[12] * b[10]), fmaf(0.13272538781166077f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.180223748087883f, (a[5] * b[7] + a[7] * b[5]), fmaf(0.16858388483524323f, (a[3] * b[11] + a[11] * b[3]), 0.16858388483524323f * (a[1] * b[13] + a[13] * b[1])))))))) + (fmaf(-0.08369845151901245f, (a[18] * b[20] + a[20] * b[18]), fmaf(0.11468784511089325f, (a[11] * b[13] + a[13] * b[11]), fmaf(0.09029786288738251f, (a[7] * b[19] + a[19] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[21] + a[21] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[6] + a[6] * b[4]), 0.04352817311882973f * (a[1] * b[15] + a[15] * b[1])))))) + fmaf(-0.13504546880722046f, (a[18] * b[24] + a[24] * b[18]), fmaf(-0.1332552284002304f, (a[11] * b[15] + a[15] * b[11]), fmaf(-0.07508081942796707f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.13272538781166077f, (a[5] * b[23] + a[23] * b[5]), fmaf(-0.19036461412906647f, (a[4] * b[20] + a[20] * b[4]), 0.21324361860752106f * (a[2] * b[10] + a[10] * b[2]))))))));
+        o[19] = ((fmaf(0.10208478569984436f, (a[18] * b[21] + a[21] * b[18]), fmaf(-0.10257992148399353f, (a[11] * b[14] + a[14] * b[11]), fmaf(-0.09932258725166321f, (a[9] * b[14] + a[14] * b[9]), fmaf(0.1392638087272644f, (a[6] * b[19] + a[19] * b[6]), fmaf(0.22072811424732208f, (a[5] * b[6] + a[6] * b[5]), fmaf(-0.07539300620555878f, (a[3] * b[10] + a[10] * b[3]), 0.282094806432724f * (a[0] * b[19] + a[19] * b[0]))))))) + fmaf(-0.045015156269073486f, (a[18] * b[23] + a[23] * b[18]), fmaf(-0.11909890919923782f, (a[16] * b[23] + a[23] * b[16]), fmaf(0.10257992148399353f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.09029786288738251f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.06371872127056122f, (a[5] * b[8] + a[8] * b[5]), fmaf(-0.06371872127056122f, (a[4] * b[7] + a[7] * b[4]), 0.1946638971567154f * (a[1] * b[12] + a[12] * b[1])))))))) + (fmaf(0.06848055124282837f, (a[19] * b[20] + a[20] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[22] + a[22] * b[17]), fmaf(0.09932258725166321f, (a[10] * b[15] + a[15] * b[10]), fmaf(-0.11262122541666031f, (a[8] * b[17] + a[17] * b[8]), fmaf(0.04486937075853348f, (a[5] * b[20] + a[20] * b[5]), fmaf(0.14188940823078156f, (a[4] * b[21] + a[21] * b[4]), 0.07539300620555878f * (a[1] * b[14] + a[14] * b[1]))))))) + fmaf(-0.10208478569984436f, (a[19] * b[22] + a[22] * b[19]), fmaf(0.11909890919923782f, (a[17] * b[24] + a[24] * b[17]), fmaf(0.09932258725166321f, (a[11] * b[12] + a[12] * b[11]), fmaf(-0.14188940823078156f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.09029786288738251f, (a[5] * b[22] + a[22] * b[5]), fmaf(0.11262122541666031f, (a[4] * b[23] + a[23] * b[4]), 0.23841361701488495f * (a[2] * b[11] + a[11] * b[2])))))))));
+        o[20] = ((fmaf(-0.15978795289993286f, a[23] * b[23], fmaf(0.06848055124282837f, a[19] * b[19], fmaf(0.07693494111299515f, a[15] * b[15], fmaf(0.025644980370998383f, a[11] * b[11], fmaf(0.04029925540089607f, a[8] * b[8], fmaf(0.24179553985595703f, a[6] * b[6], fmaf(0.04029925540089607f, a[4] * b[4], 0.282094806432724f * (a[0] * b[20] + a[20] * b[0])))))))) + fmaf(0.10652530938386917f, a[24] * b[24], fmaf(0.13696110248565674f, a[20] * b[20], fmaf(0.10652530938386917f, a[16] * b[16], fmaf(0.1538698822259903f, a[12] * b[12], fmaf(-0.19036461412906647f, (a[8] * b[22] + a[22] * b[8]), fmaf(0.16383977234363556f, (a[6] * b[20] + a[20] * b[6]), fmaf(-0.19036461412906647f, (a[4] * b[18] + a[18] * b[4]), -0.15078601241111755f * (a[1] * b[11] + a[11] * b[1]))))))))) + (fmaf(0.06848055124282837f, a[21] * b[21], fmaf(-0.15978795289993286f, a[17] * b[17], fmaf(0.025644980370998383f, a[13] * b[13], fmaf(0.07693494111299515f, a[9] * b[9], fmaf(-0.1611970216035843f, a[7] * b[7], fmaf(-0.1611970216035843f, a[5] * b[5], 0.2462325245141983f * (a[2] * b[12] + a[12] * b[2]))))))) + fmaf(-0.08369845151901245f, a[22] * b[22], fmaf(-0.08369845151901245f, a[18] * b[18], fmaf(-0.17951487004756927f, a[14] * b[14], fmaf(-0.17951487004756927f, a[10] * b[10], fmaf(0.04486937075853348f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.04486937075853348f, (a[5] * b[19] + a[19] * b[5]), -0.15078601241111755f * (a[3] * b[13] + a[13] * b[3])))))))));
+        o[21] = ((fmaf(0.06848055124282837f, (a[20] * b[21] + a[21] * b[20]), fmaf(-0.09932258725166321f, (a[14] * b[15] + a[15] * b[14]), fmaf(-0.09932258725166321f, (a[9] * b[10] + a[10] * b[9]), fmaf(0.04486937075853348f, (a[7] * b[20] + a[20] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[18] + a[18] * b[5]), fmaf(-0.07539300620555878f, (a[3] * b[14] + a[14] * b[3]), 0.282094806432724f * (a[0] * b[21] + a[21] * b[0]))))))) + fmaf(0.10208478569984436f, (a[21] * b[22] + a[22] * b[21]), fmaf(-0.11909890919923782f, (a[16] * b[17] + a[17] * b[16]), fmaf(0.10257992148399353f, (a[10] * b[11] + a[11] * b[10]), fmaf(0.09029786288738251f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.22072811424732208f, (a[6] * b[7] + a[7] * b[6]), fmaf(-0.06371872127056122f, (a[4] * b[5] + a[5] * b[4]), -0.07539300620555878f * (a[1] * b[10] + a[10] * b[1])))))))) + (fmaf(0.045015156269073486f, (a[22] * b[23] + a[23] * b[22]), fmaf(0.045015156269073486f, (a[17] * b[18] + a[18] * b[17]), fmaf(0.09932258725166321f, (a[12] * b[13] + a[13] * b[12]), fmaf(0.14188940823078156f, (a[8] * b[21] + a[21] * b[8]), fmaf(0.1392638087272644f, (a[6] * b[21] + a[21] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[17] + a[17] * b[4]), 0.23841361701488495f * (a[2] * b[13] + a[13] * b[2]))))))) + fmaf(-0.11909890919923782f, (a[23] * b[24] + a[24] * b[23]), fmaf(0.10208478569984436f, (a[18] * b[19] + a[19] * b[18]), fmaf(0.10257992148399353f, (a[13] * b[14] + a[14] * b[13]), fmaf(-0.11262122541666031f, (a[8] * b[23] + a[23] * b[8]), fmaf(-0.06371872127056122f, (a[7] * b[8] + a[8] * b[7]), fmaf(0.14188940823078156f, (a[4] * b[19] + a[19] * b[4]), 0.1946638971567154f * (a[3] * b[12] + a[12] * b[3])))))))));
+        o[22] = ((fmaf(0.13504546880722046f, (a[22] * b[24] + a[24] * b[22]), fmaf(-0.10208478569984436f, a[19] * b[19], fmaf(0.11468784511089325f, a[13] * b[13], fmaf(-0.07508081942796707f, (a[8] * b[24] + a[24] * b[8]), fmaf(0.180223748087883f, a[7] * b[7], fmaf(0.13272538781166077f, (a[5] * b[17] + a[17] * b[5]), fmaf(0.16858388483524323f, (a[3] * b[13] + a[13] * b[3]), 0.282094806432724f * (a[0] * b[22] + a[22] * b[0])))))))) + fmaf(-0.08369845151901245f, (a[20] * b[22] + a[22] * b[20]), fmaf(0.1332552284002304f, (a[13] * b[15] + a[15] * b[13]), fmaf(0.1332552284002304f, (a[9] * b[11] + a[11] * b[9]), fmaf(0.09029786288738251f, (a[7] * b[21] + a[21] * b[7]), fmaf(-0.09029786288738251f, (a[5] * b[19] + a[19] * b[5]), fmaf(-0.04352817311882973f, (a[3] * b[15] + a[15] * b[3]), -0.04352817311882973f * (a[1] * b[9] + a[9] * b[1])))))))) + (fmaf(0.10208478569984436f, a[21] * b[21], fmaf(0.13504546880722046f, (a[16] * b[18] + a[18] * b[16]), fmaf(-0.11468784511089325f, a[11] * b[11], fmaf(0.13272538781166077f, (a[7] * b[23] + a[23] * b[7]), fmaf(0.15607835352420807f, (a[6] * b[8] + a[8] * b[6]), fmaf(-0.07508081942796707f, (a[4] * b[16] + a[16] * b[4]), -0.16858388483524323f * (a[1] * b[11] + a[11] * b[1]))))))) + fmaf(0.045015156269073486f, (a[21] * b[23] + a[23] * b[21]), fmaf(0.045015156269073486f, (a[17] * b[19] + a[19] * b[17]), fmaf(-0.04441840946674347f, (a[12] * b[14] + a[14] * b[12]), fmaf(-0.19036461412906647f, (a[8] * b[20] + a[20] * b[8]), fmaf(0.06553591042757034f, (a[6] * b[22] + a[22] * b[6]), fmaf(-0.180223748087883f, a[5] * b[5], 0.21324361860752106f * (a[2] * b[14] + a[14] * b[2])))))))));
+        o[23] = ((fmaf(-0.11909890919923782f, (a[21] * b[24] + a[24] * b[21]), fmaf(-0.11909890919923782f, (a[16] * b[19] + a[19] * b[16]), fmaf(-0.11262122541666031f, (a[8] * b[21] + a[21] * b[8]), fmaf(-0.057343922555446625f, (a[6] * b[23] + a[23] * b[6]), fmaf(-0.16858388483524323f, (a[4] * b[5] + a[5] * b[4]), 0.282094806432724f * (a[0] * b[23] + a[23] * b[0])))))) + fmaf(-0.045015156269073486f, (a[18] * b[19] + a[19] * b[18]), fmaf(-0.06785023957490921f, (a[10] * b[11] + a[11] * b[10]), fmaf(0.16858388483524323f, (a[7] * b[8] + a[8] * b[7]), fmaf(0.11262122541666031f, (a[4] * b[19] + a[19] * b[4]), -0.1994711458683014f * (a[1] * b[10] + a[10] * b[1])))))) + (fmaf(-0.15978795289993286f, (a[20] * b[23] + a[23] * b[20]), fmaf(-0.20355072617530823f, (a[12] * b[15] + a[15] * b[12]), fmaf(0.13272538781166077f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.14046335220336914f, (a[5] * b[16] + a[16] * b[5]), 0.1628675013780594f * (a[2] * b[15] + a[15] * b[2]))))) + fmaf(0.045015156269073486f, (a[21] * b[22] + a[22] * b[21]), fmaf(0.06785023957490921f, (a[13] * b[14] + a[14] * b[13]), fmaf(0.14046335220336914f, (a[7] * b[24] + a[24] * b[7]), fmaf(-0.13272538781166077f, (a[5] * b[18] + a[18] * b[5]), 0.1994711458683014f * (a[3] * b[14] + a[14] * b[3])))))));
+        o[24] = ((fmaf(0.10652530938386917f, (a[20] * b[24] + a[24] * b[20]), fmaf(-0.11752006411552429f, (a[13] * b[15] + a[15] * b[13]), fmaf(0.23841361701488495f, a[8] * b[8], fmaf(0.07508081942796707f, (a[4] * b[18] + a[18] * b[4]), 0.282094806432724f * (a[0] * b[24] + a[24] * b[0]))))) + fmaf(-0.11909890919923782f, (a[21] * b[23] + a[23] * b[21]), fmaf(0.15171775221824646f, a[14] * b[14], fmaf(-0.07508081942796707f, (a[8] * b[22] + a[22] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[17] + a[17] * b[5]), -0.23032943904399872f * (a[1] * b[9] + a[9] * b[1])))))) + (fmaf(0.13504546880722046f, a[22] * b[22], fmaf(0.11909890919923782f, (a[17] * b[19] + a[19] * b[17]), fmaf(0.11752006411552429f, (a[9] * b[11] + a[11] * b[9]), fmaf(-0.2293756902217865f, (a[6] * b[24] + a[24] * b[6]), 0.23032943904399872f * (a[3] * b[15] + a[15] * b[3]))))) + fmaf(-0.13504546880722046f, a[18] * b[18], fmaf(-0.15171775221824646f, a[10] * b[10], fmaf(0.14046335220336914f, (a[7] * b[23] + a[23] * b[7]), -0.23841361701488495f * a[4] * b[4])))));
+    }
+    __device__ __forceinline__ static void mul_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((fmaf(0.282094806432724f, a[23] * b[23], fmaf(0.282094806432724f, a[19] * b[19], fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])))) + fmaf(0.282094806432724f, a[24] * b[24], fmaf(0.282094806432724f, a[20] * b[20], fmaf(0.282094806432724f, a[16] * b[16], fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1]))))) + (fmaf(0.282094806432724f, a[21] * b[21], fmaf(0.282094806432724f, a[17] * b[17], fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]))) + fmaf(0.282094806432724f, a[22] * b[22], fmaf(0.282094806432724f, a[18] * b[18], fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])))));
+        o[1] = ((fmaf(0.04352817311882973f, a[15] * b[18], fmaf(0.16858388483524323f, a[13] * b[18], fmaf(-0.1994711458683014f, a[10] * b[23], fmaf(0.05839917063713074f, a[11] * b[8], fmaf(-0.18467439711093903f, a[14] * b[5], fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0]))))))) + fmaf(0.1994711458683014f, a[14] * b[17], fmaf(-0.15078601241111755f, a[11] * b[20], fmaf(-0.04352817311882973f, a[9] * b[22], fmaf(0.20230065286159515f, a[11] * b[6], fmaf(-0.05839917063713074f, a[13] * b[4], -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1]))))))) + (fmaf(0.07539300620555878f, a[14] * b[19], fmaf(-0.16858388483524323f, a[11] * b[22], fmaf(-0.23032943904399872f, a[9] * b[24], fmaf(0.18467439711093903f, a[10] * b[7], fmaf(-0.22617901861667633f, a[15] * b[4], -0.21850968897342682f * (a[1] * b[8] + a[8] * b[1])))))) + fmaf(0.23032943904399872f, a[15] * b[16], fmaf(0.1946638971567154f, a[12] * b[19], fmaf(-0.07539300620555878f, a[10] * b[21], fmaf(0.22617901861667633f, a[9] * b[8], fmaf(-0.14304816722869873f, a[12] * b[5], 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2]))))))));
+        o[2] = ((fmaf(0.2462325245141983f, a[12] * b[20], fmaf(0.18467439711093903f, a[14] * b[8], fmaf(0.18467439711093903f, a[10] * b[4], 0.282094806432724f * (a[0] * b[2] + a[2] * b[0])))) + fmaf(0.23841361701488495f, a[13] * b[21], fmaf(0.1628675013780594f, a[9] * b[17], fmaf(0.23359668254852295f, a[11] * b[5], 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1]))))) + (fmaf(0.21324361860752106f, a[14] * b[22], fmaf(0.21324361860752106f, a[10] * b[18], fmaf(0.24776668846607208f, a[12] * b[6], 0.2523132562637329f * (a[2] * b[6] + a[6] * b[2])))) + fmaf(0.1628675013780594f, a[15] * b[23], fmaf(0.23841361701488495f, a[11] * b[19], fmaf(0.23359668254852295f, a[13] * b[7], 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3]))))));
+        o[3] = ((fmaf(0.23032943904399872f, a[15] * b[24], fmaf(0.16858388483524323f, a[13] * b[22], fmaf(-0.07539300620555878f, a[10] * b[19], fmaf(0.22617901861667633f, a[15] * b[8], fmaf(0.20230065286159515f, a[13] * b[6], fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0]))))))) + fmaf(-0.07539300620555878f, a[14] * b[21], fmaf(0.16858388483524323f, a[11] * b[18], fmaf(0.23032943904399872f, a[9] * b[16], fmaf(-0.14304816722869873f, a[12] * b[7], fmaf(0.22617901861667633f, a[9] * b[4], 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1]))))))) + (fmaf(0.1994711458683014f, a[14] * b[23], fmaf(0.1946638971567154f, a[12] * b[21], fmaf(-0.04352817311882973f, a[9] * b[18], fmaf(0.18467439711093903f, a[14] * b[7], fmaf(-0.05839917063713074f, a[11] * b[4], 0.21850968897342682f * (a[2] * b[7] + a[7] * b[2])))))) + fmaf(-0.04352817311882973f, a[15] * b[22], fmaf(-0.15078601241111755f, a[13] * b[20], fmaf(0.1994711458683014f, a[10] * b[17], fmaf(-0.05839917063713074f, a[13] * b[8], fmaf(0.18467439711093903f, a[10] * b[5], -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3]))))))));
+        o[4] = ((fmaf(0.07508081942796707f, (a[18] * b[24] + a[24] * b[18]), fmaf(0.23841361701488495f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.16858388483524323f, (a[5] * b[23] + a[23] * b[5]), fmaf(0.04029925540089607f, (a[4] * b[20] + a[20] * b[4]), fmaf(0.18467439711093903f, a[10] * b[2], 0.282094806432724f * (a[0] * b[4] + a[4] * b[0])))))) + fmaf(0.14188940823078156f, (a[19] * b[21] + a[21] * b[19]), fmaf(-0.07508081942796707f, (a[16] * b[22] + a[22] * b[16]), fmaf(0.15607835352420807f, (a[6] * b[18] + a[18] * b[6]), fmaf(-0.23841361701488495f, (a[4] * b[24] + a[24] * b[4]), fmaf(0.22617901861667633f, a[9] * b[3], 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1]))))))) + (fmaf(0.11262122541666031f, (a[19] * b[23] + a[23] * b[19]), fmaf(-0.11262122541666031f, (a[17] * b[21] + a[21] * b[17]), fmaf(0.16858388483524323f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.15607835352420807f, (a[5] * b[7] + a[7] * b[5]), fmaf(-0.05839917063713074f, a[11] * b[3], -0.05839917063713074f * a[13] * b[1]))))) + fmaf(-0.19036461412906647f, (a[18] * b[20] + a[20] * b[18]), fmaf(-0.06371872127056122f, (a[7] * b[19] + a[19] * b[7]), fmaf(-0.06371872127056122f, (a[5] * b[21] + a[21] * b[5]), fmaf(-0.180223748087883f, (a[4] * b[6] + a[6] * b[4]), -0.22617901861667633f * a[15] * b[1]))))));
+        o[5] = ((fmaf(0.09029786288738251f, (a[18] * b[21] + a[21] * b[18]), fmaf(0.06371872127056122f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.180223748087883f, (a[5] * b[22] + a[22] * b[5]), fmaf(-0.16858388483524323f, (a[4] * b[23] + a[23] * b[4]), fmaf(0.23359668254852295f, a[11] * b[2], 0.282094806432724f * (a[0] * b[5] + a[5] * b[0])))))) + fmaf(-0.13272538781166077f, (a[18] * b[23] + a[23] * b[18]), fmaf(0.14046335220336914f, (a[16] * b[23] + a[23] * b[16]), fmaf(0.22072811424732208f, (a[6] * b[19] + a[19] * b[6]), fmaf(0.0901118740439415f, (a[5] * b[6] + a[6] * b[5]), fmaf(0.18467439711093903f, a[10] * b[3], 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1]))))))) + (fmaf(0.04486937075853348f, (a[19] * b[20] + a[20] * b[19]), fmaf(0.13272538781166077f, (a[17] * b[22] + a[22] * b[17]), fmaf(0.180223748087883f, (a[7] * b[18] + a[18] * b[7]), fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[7] + a[7] * b[4]), -0.14304816722869873f * a[12] * b[1]))))) + fmaf(-0.09029786288738251f, (a[19] * b[22] + a[22] * b[19]), fmaf(-0.14046335220336914f, (a[17] * b[24] + a[24] * b[17]), fmaf(0.16858388483524323f, (a[8] * b[17] + a[17] * b[8]), fmaf(-0.1611970216035843f, (a[5] * b[20] + a[20] * b[5]), fmaf(-0.06371872127056122f, (a[4] * b[21] + a[21] * b[4]), -0.18467439711093903f * a[14] * b[1])))))));
+        o[6] = ((fmaf(-0.057343922555446625f, a[23] * b[23], fmaf(0.1392638087272644f, a[19] * b[19], fmaf(0.15607835352420807f, (a[8] * b[22] + a[22] * b[8]), fmaf(0.24179553985595703f, (a[6] * b[20] + a[20] * b[6]), fmaf(0.15607835352420807f, (a[4] * b[18] + a[18] * b[4]), fmaf(0.24776668846607208f, a[12] * b[2], 0.282094806432724f * (a[0] * b[6] + a[6] * b[0]))))))) + fmaf(-0.2293756902217865f, a[24] * b[24], fmaf(0.16383977234363556f, a[20] * b[20], fmaf(-0.2293756902217865f, a[16] * b[16], fmaf(0.0901118740439415f, a[7] * b[7], fmaf(0.0901118740439415f, a[5] * b[5], fmaf(-0.12615662813186646f, a[3] * b[3], -0.12615662813186646f * a[1] * b[1]))))))) + (fmaf(0.1392638087272644f, a[21] * b[21], fmaf(-0.057343922555446625f, a[17] * b[17], fmaf(0.22072811424732208f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.22072811424732208f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.20230065286159515f, a[13] * b[3], 0.20230065286159515f * a[11] * b[1]))))) + fmaf(0.06553591042757034f, a[22] * b[22], fmaf(0.06553591042757034f, a[18] * b[18], fmaf(-0.180223748087883f, a[8] * b[8], fmaf(0.180223748087883f, a[6] * b[6], fmaf(-0.180223748087883f, a[4] * b[4], 0.2523132562637329f * a[2] * b[2])))))));
+        o[7] = ((fmaf(0.04486937075853348f, (a[20] * b[21] + a[21] * b[20]), fmaf(0.16858388483524323f, (a[8] * b[23] + a[23] * b[8]), fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), fmaf(-0.06371872127056122f, (a[4] * b[19] + a[19] * b[4]), fmaf(-0.14304816722869873f, a[12] * b[3], 0.282094806432724f * (a[0] * b[7] + a[7] * b[0])))))) + fmaf(0.09029786288738251f, (a[21] * b[22] + a[22] * b[21]), fmaf(0.14046335220336914f, (a[16] * b[17] + a[17] * b[16]), fmaf(-0.1611970216035843f, (a[7] * b[20] + a[20] * b[7]), fmaf(0.180223748087883f, (a[5] * b[18] + a[18] * b[5]), fmaf(0.18467439711093903f, a[14] * b[3], 0.18467439711093903f * a[10] * b[1])))))) + (fmaf(0.13272538781166077f, (a[22] * b[23] + a[23] * b[22]), fmaf(0.13272538781166077f, (a[17] * b[18] + a[18] * b[17]), fmaf(0.180223748087883f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.0901118740439415f, (a[6] * b[7] + a[7] * b[6]), fmaf(0.15607835352420807f, (a[4] * b[5] + a[5] * b[4]), 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2])))))) + fmaf(0.14046335220336914f, (a[23] * b[24] + a[24] * b[23]), fmaf(0.09029786288738251f, (a[18] * b[19] + a[19] * b[18]), fmaf(-0.06371872127056122f, (a[8] * b[21] + a[21] * b[8]), fmaf(0.22072811424732208f, (a[6] * b[21] + a[21] * b[6]), fmaf(0.16858388483524323f, (a[4] * b[17] + a[17] * b[4]), 0.23359668254852295f * a[13] * b[2])))))));
+        o[8] = ((fmaf(-0.11262122541666031f, (a[21] * b[23] + a[23] * b[21]), fmaf(-0.11262122541666031f, (a[17] * b[19] + a[19] * b[17]), fmaf(0.16858388483524323f, (a[7] * b[23] + a[23] * b[7]), fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), fmaf(0.23841361701488495f, (a[4] * b[16] + a[16] * b[4]), fmaf(0.18467439711093903f, a[14] * b[2], 0.282094806432724f * (a[0] * b[8] + a[8] * b[0]))))))) + fmaf(-0.07508081942796707f, (a[22] * b[24] + a[24] * b[22]), fmaf(-0.14188940823078156f, a[19] * b[19], fmaf(0.04029925540089607f, (a[8] * b[20] + a[20] * b[8]), fmaf(0.15607835352420807f, (a[6] * b[22] + a[22] * b[6]), fmaf(-0.15607835352420807f, a[5] * b[5], fmaf(0.21850968897342682f, a[3] * b[3], -0.21850968897342682f * a[1] * b[1]))))))) + (fmaf(-0.19036461412906647f, (a[20] * b[22] + a[22] * b[20]), fmaf(0.23841361701488495f, (a[8] * b[24] + a[24] * b[8]), fmaf(0.15607835352420807f, a[7] * b[7], fmaf(0.16858388483524323f, (a[5] * b[17] + a[17] * b[5]), fmaf(-0.05839917063713074f, a[13] * b[3], 0.22617901861667633f * a[9] * b[1]))))) + fmaf(0.14188940823078156f, a[21] * b[21], fmaf(-0.07508081942796707f, (a[16] * b[18] + a[18] * b[16]), fmaf(-0.06371872127056122f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.06371872127056122f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.22617901861667633f, a[15] * b[3], 0.05839917063713074f * a[11] * b[1])))))));
+        o[9] = ((fmaf(-0.09932258725166321f, a[14] * b[19], fmaf(0.11752006411552429f, a[11] * b[24], fmaf(-0.09403159469366074f, a[11] * b[8], fmaf(-0.09403159469366074f, a[13] * b[4], fmaf(0.1628675013780594f, (a[2] * b[17] + a[17] * b[2]), 0.282094806432724f * a[9] * b[0]))))) + fmaf(-0.20355072617530823f, a[12] * b[17], fmaf(0.07693494111299515f, a[9] * b[20], fmaf(0.1486770063638687f, a[14] * b[5], fmaf(0.22617901861667633f, (a[3] * b[4] + a[4] * b[3]), 0.22617901861667633f * (a[1] * b[8] + a[8] * b[1])))))) + (fmaf(-0.11752006411552429f, a[13] * b[16], fmaf(-0.09932258725166321f, a[10] * b[21], fmaf(-0.2102610468864441f, a[9] * b[6], fmaf(0.23032943904399872f, (a[3] * b[16] + a[16] * b[3]), -0.04352817311882973f * (a[1] * b[22] + a[22] * b[1]))))) + fmaf(0.1332552284002304f, a[13] * b[18], fmaf(0.1332552284002304f, a[11] * b[22], fmaf(0.1486770063638687f, a[10] * b[7], fmaf(-0.04352817311882973f, (a[3] * b[18] + a[18] * b[3]), -0.23032943904399872f * (a[1] * b[24] + a[24] * b[1])))))));
+        o[10] = ((fmaf(0.06785023957490921f, a[13] * b[17], fmaf(-0.15171775221824646f, a[10] * b[24], fmaf(0.1486770063638687f, a[9] * b[7], fmaf(-0.07539300620555878f, (a[3] * b[19] + a[19] * b[3]), fmaf(0.18467439711093903f, (a[2] * b[4] + a[4] * b[2]), 0.282094806432724f * a[10] * b[0]))))) + fmaf(0.10257992148399353f, a[13] * b[19], fmaf(0.10257992148399353f, a[11] * b[21], fmaf(0.11516471952199936f, a[11] * b[7], fmaf(-0.18806318938732147f, a[12] * b[4], fmaf(0.21324361860752106f, (a[2] * b[18] + a[18] * b[2]), 0.18467439711093903f * (a[1] * b[7] + a[7] * b[1]))))))) + (fmaf(0.15171775221824646f, a[14] * b[16], fmaf(-0.06785023957490921f, a[11] * b[23], fmaf(-0.09932258725166321f, a[9] * b[21], fmaf(0.11516471952199936f, a[13] * b[5], fmaf(0.18467439711093903f, (a[3] * b[5] + a[5] * b[3]), -0.07539300620555878f * (a[1] * b[21] + a[21] * b[1])))))) + fmaf(0.09932258725166321f, a[15] * b[19], fmaf(-0.04441840946674347f, a[12] * b[18], fmaf(-0.17951487004756927f, a[10] * b[20], fmaf(-0.1486770063638687f, a[15] * b[5], fmaf(0.1994711458683014f, (a[3] * b[17] + a[17] * b[3]), -0.1994711458683014f * (a[1] * b[23] + a[23] * b[1]))))))));
+        o[11] = ((fmaf(-0.1332552284002304f, a[15] * b[18], fmaf(0.11468784511089325f, a[13] * b[18], fmaf(-0.06785023957490921f, a[10] * b[23], fmaf(-0.14567312598228455f, a[11] * b[8], fmaf(-0.11516471952199936f, a[14] * b[5], fmaf(0.16858388483524323f, (a[3] * b[18] + a[18] * b[3]), fmaf(-0.16858388483524323f, (a[1] * b[22] + a[22] * b[1]), 0.282094806432724f * a[11] * b[0]))))))) + fmaf(0.06785023957490921f, a[14] * b[17], fmaf(0.025644980370998383f, a[11] * b[20], fmaf(0.1332552284002304f, a[9] * b[22], fmaf(0.12615662813186646f, a[11] * b[6], fmaf(0.14567312598228455f, a[13] * b[4], fmaf(0.23359668254852295f, (a[2] * b[5] + a[5] * b[2]), 0.20230065286159515f * (a[1] * b[6] + a[6] * b[1])))))))) + (fmaf(-0.10257992148399353f, a[14] * b[19], fmaf(-0.11468784511089325f, a[11] * b[22], fmaf(0.11752006411552429f, a[9] * b[24], fmaf(0.11516471952199936f, a[10] * b[7], fmaf(0.09403159469366074f, a[15] * b[4], fmaf(0.23841361701488495f, (a[2] * b[19] + a[19] * b[2]), 0.05839917063713074f * (a[1] * b[8] + a[8] * b[1]))))))) + fmaf(-0.11752006411552429f, a[15] * b[16], fmaf(0.09932258725166321f, a[12] * b[19], fmaf(0.10257992148399353f, a[10] * b[21], fmaf(-0.09403159469366074f, a[9] * b[8], fmaf(0.059470802545547485f, a[12] * b[5], fmaf(-0.05839917063713074f, (a[3] * b[4] + a[4] * b[3]), -0.15078601241111755f * (a[1] * b[20] + a[20] * b[1])))))))));
+        o[12] = ((fmaf(0.09932258725166321f, a[13] * b[21], fmaf(-0.20355072617530823f, a[9] * b[17], fmaf(0.059470802545547485f, a[11] * b[5], fmaf(0.2462325245141983f, (a[2] * b[20] + a[20] * b[2]), 0.282094806432724f * a[12] * b[0])))) + fmaf(-0.04441840946674347f, a[14] * b[22], fmaf(-0.04441840946674347f, a[10] * b[18], fmaf(0.16820883750915527f, a[12] * b[6], fmaf(-0.14304816722869873f, (a[3] * b[7] + a[7] * b[3]), -0.14304816722869873f * (a[1] * b[5] + a[5] * b[1])))))) + (fmaf(-0.20355072617530823f, a[15] * b[23], fmaf(0.09932258725166321f, a[11] * b[19], fmaf(0.059470802545547485f, a[13] * b[7], fmaf(0.1946638971567154f, (a[3] * b[21] + a[21] * b[3]), 0.1946638971567154f * (a[1] * b[19] + a[19] * b[1]))))) + fmaf(0.1538698822259903f, a[12] * b[20], fmaf(-0.18806318938732147f, a[14] * b[8], fmaf(-0.18806318938732147f, a[10] * b[4], 0.24776668846607208f * (a[2] * b[6] + a[6] * b[2]))))));
+        o[13] = ((fmaf(-0.11752006411552429f, a[15] * b[24], fmaf(0.11468784511089325f, a[13] * b[22], fmaf(0.10257992148399353f, a[10] * b[19], fmaf(-0.09403159469366074f, a[15] * b[8], fmaf(0.12615662813186646f, a[13] * b[6], fmaf(0.16858388483524323f, (a[3] * b[22] + a[22] * b[3]), fmaf(0.23841361701488495f, (a[2] * b[21] + a[21] * b[2]), 0.282094806432724f * a[13] * b[0]))))))) + fmaf(0.10257992148399353f, a[14] * b[21], fmaf(0.11468784511089325f, a[11] * b[18], fmaf(-0.11752006411552429f, a[9] * b[16], fmaf(0.059470802545547485f, a[12] * b[7], fmaf(-0.09403159469366074f, a[9] * b[4], fmaf(0.20230065286159515f, (a[3] * b[6] + a[6] * b[3]), -0.05839917063713074f * (a[1] * b[4] + a[4] * b[1])))))))) + (fmaf(0.06785023957490921f, a[14] * b[23], fmaf(0.09932258725166321f, a[12] * b[21], fmaf(0.1332552284002304f, a[9] * b[18], fmaf(0.11516471952199936f, a[14] * b[7], fmaf(0.14567312598228455f, a[11] * b[4], fmaf(-0.05839917063713074f, (a[3] * b[8] + a[8] * b[3]), 0.16858388483524323f * (a[1] * b[18] + a[18] * b[1]))))))) + fmaf(0.1332552284002304f, a[15] * b[22], fmaf(0.025644980370998383f, a[13] * b[20], fmaf(0.06785023957490921f, a[10] * b[17], fmaf(0.14567312598228455f, a[13] * b[8], fmaf(0.11516471952199936f, a[10] * b[5], fmaf(-0.15078601241111755f, (a[3] * b[20] + a[20] * b[3]), 0.23359668254852295f * (a[2] * b[7] + a[7] * b[2])))))))));
+        o[14] = ((fmaf(0.06785023957490921f, a[13] * b[23], fmaf(0.06785023957490921f, a[11] * b[17], fmaf(0.1486770063638687f, a[15] * b[7], fmaf(0.1994711458683014f, (a[3] * b[23] + a[23] * b[3]), fmaf(0.18467439711093903f, (a[2] * b[8] + a[8] * b[2]), 0.282094806432724f * a[14] * b[0]))))) + fmaf(-0.17951487004756927f, a[14] * b[20], fmaf(-0.10257992148399353f, a[11] * b[19], fmaf(-0.18806318938732147f, a[12] * b[8], fmaf(0.1486770063638687f, a[9] * b[5], fmaf(0.21324361860752106f, (a[2] * b[22] + a[22] * b[2]), -0.18467439711093903f * (a[1] * b[5] + a[5] * b[1]))))))) + (fmaf(0.15171775221824646f, a[14] * b[24], fmaf(-0.04441840946674347f, a[12] * b[22], fmaf(-0.09932258725166321f, a[9] * b[19], fmaf(-0.11516471952199936f, a[11] * b[5], fmaf(0.18467439711093903f, (a[3] * b[7] + a[7] * b[3]), 0.1994711458683014f * (a[1] * b[17] + a[17] * b[1])))))) + fmaf(-0.09932258725166321f, a[15] * b[21], fmaf(0.10257992148399353f, a[13] * b[21], fmaf(0.15171775221824646f, a[10] * b[16], fmaf(0.11516471952199936f, a[13] * b[7], fmaf(-0.07539300620555878f, (a[3] * b[21] + a[21] * b[3]), 0.07539300620555878f * (a[1] * b[19] + a[19] * b[1]))))))));
+        o[15] = ((fmaf(0.07693494111299515f, a[15] * b[20], fmaf(-0.20355072617530823f, a[12] * b[23], fmaf(-0.09403159469366074f, a[13] * b[8], fmaf(0.09403159469366074f, a[11] * b[4], fmaf(0.1628675013780594f, (a[2] * b[23] + a[23] * b[2]), 0.282094806432724f * a[15] * b[0]))))) + fmaf(0.1332552284002304f, a[13] * b[22], fmaf(0.09932258725166321f, a[10] * b[19], fmaf(-0.1486770063638687f, a[10] * b[5], fmaf(0.22617901861667633f, (a[3] * b[8] + a[8] * b[3]), -0.22617901861667633f * (a[1] * b[4] + a[4] * b[1])))))) + (fmaf(-0.11752006411552429f, a[13] * b[24], fmaf(-0.11752006411552429f, a[11] * b[16], fmaf(-0.2102610468864441f, a[15] * b[6], fmaf(-0.04352817311882973f, (a[3] * b[22] + a[22] * b[3]), 0.23032943904399872f * (a[1] * b[16] + a[16] * b[1]))))) + fmaf(-0.09932258725166321f, a[14] * b[21], fmaf(-0.1332552284002304f, a[11] * b[18], fmaf(0.1486770063638687f, a[14] * b[7], fmaf(0.23032943904399872f, (a[3] * b[24] + a[24] * b[3]), 0.04352817311882973f * (a[1] * b[18] + a[18] * b[1])))))));
+        o[16] = ((fmaf(-0.11909890919923782f, (a[19] * b[23] + a[23] * b[19]), fmaf(-0.07508081942796707f, (a[8] * b[18] + a[18] * b[8]), fmaf(-0.07508081942796707f, (a[4] * b[22] + a[22] * b[4]), 0.282094806432724f * (a[0] * b[16] + a[16] * b[0])))) + fmaf(0.10652530938386917f, (a[16] * b[20] + a[20] * b[16]), fmaf(0.14046335220336914f, (a[5] * b[23] + a[23] * b[5]), 0.23032943904399872f * a[15] * b[1]))) + (fmaf(-0.11909890919923782f, (a[17] * b[21] + a[21] * b[17]), fmaf(-0.2293756902217865f, (a[6] * b[16] + a[16] * b[6]), 0.23032943904399872f * a[9] * b[3])) + fmaf(0.13504546880722046f, (a[18] * b[22] + a[22] * b[18]), fmaf(0.14046335220336914f, (a[7] * b[17] + a[17] * b[7]), 0.23841361701488495f * (a[4] * b[8] + a[8] * b[4])))));
+        o[17] = ((fmaf(0.045015156269073486f, (a[19] * b[22] + a[22] * b[19]), fmaf(-0.11262122541666031f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[24] + a[24] * b[5]), fmaf(0.16858388483524323f, (a[4] * b[7] + a[7] * b[4]), 0.282094806432724f * (a[0] * b[17] + a[17] * b[0]))))) + fmaf(0.11909890919923782f, (a[19] * b[24] + a[24] * b[19]), fmaf(-0.11909890919923782f, (a[16] * b[21] + a[21] * b[16]), fmaf(-0.057343922555446625f, (a[6] * b[17] + a[17] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[21] + a[21] * b[4]), 0.1994711458683014f * a[14] * b[1]))))) + (fmaf(-0.15978795289993286f, (a[17] * b[20] + a[20] * b[17]), fmaf(0.14046335220336914f, (a[7] * b[16] + a[16] * b[7]), fmaf(0.16858388483524323f, (a[5] * b[8] + a[8] * b[5]), 0.1628675013780594f * a[9] * b[2]))) + fmaf(0.045015156269073486f, (a[18] * b[21] + a[21] * b[18]), fmaf(0.13272538781166077f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.13272538781166077f, (a[5] * b[22] + a[22] * b[5]), 0.1994711458683014f * a[10] * b[3])))));
+        o[18] = ((fmaf(0.10208478569984436f, (a[19] * b[21] + a[21] * b[19]), fmaf(0.13504546880722046f, (a[16] * b[22] + a[22] * b[16]), fmaf(0.06553591042757034f, (a[6] * b[18] + a[18] * b[6]), fmaf(0.07508081942796707f, (a[4] * b[24] + a[24] * b[4]), fmaf(-0.04352817311882973f, a[9] * b[3], 0.282094806432724f * (a[0] * b[18] + a[18] * b[0])))))) + fmaf(-0.045015156269073486f, (a[19] * b[23] + a[23] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[21] + a[21] * b[17]), fmaf(0.13272538781166077f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.180223748087883f, (a[5] * b[7] + a[7] * b[5]), fmaf(0.16858388483524323f, a[11] * b[3], 0.16858388483524323f * a[13] * b[1])))))) + (fmaf(-0.08369845151901245f, (a[18] * b[20] + a[20] * b[18]), fmaf(0.09029786288738251f, (a[7] * b[19] + a[19] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[21] + a[21] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[6] + a[6] * b[4]), 0.04352817311882973f * a[15] * b[1])))) + fmaf(-0.13504546880722046f, (a[18] * b[24] + a[24] * b[18]), fmaf(-0.07508081942796707f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.13272538781166077f, (a[5] * b[23] + a[23] * b[5]), fmaf(-0.19036461412906647f, (a[4] * b[20] + a[20] * b[4]), 0.21324361860752106f * a[10] * b[2]))))));
+        o[19] = ((fmaf(-0.045015156269073486f, (a[18] * b[23] + a[23] * b[18]), fmaf(-0.11909890919923782f, (a[16] * b[23] + a[23] * b[16]), fmaf(0.1392638087272644f, (a[6] * b[19] + a[19] * b[6]), fmaf(0.22072811424732208f, (a[5] * b[6] + a[6] * b[5]), fmaf(-0.07539300620555878f, a[10] * b[3], 0.282094806432724f * (a[0] * b[19] + a[19] * b[0])))))) + fmaf(0.06848055124282837f, (a[19] * b[20] + a[20] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[22] + a[22] * b[17]), fmaf(0.09029786288738251f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.06371872127056122f, (a[5] * b[8] + a[8] * b[5]), fmaf(-0.06371872127056122f, (a[4] * b[7] + a[7] * b[4]), 0.1946638971567154f * a[12] * b[1])))))) + (fmaf(-0.10208478569984436f, (a[19] * b[22] + a[22] * b[19]), fmaf(0.11909890919923782f, (a[17] * b[24] + a[24] * b[17]), fmaf(-0.11262122541666031f, (a[8] * b[17] + a[17] * b[8]), fmaf(0.04486937075853348f, (a[5] * b[20] + a[20] * b[5]), fmaf(0.14188940823078156f, (a[4] * b[21] + a[21] * b[4]), 0.07539300620555878f * a[14] * b[1]))))) + fmaf(0.10208478569984436f, (a[18] * b[21] + a[21] * b[18]), fmaf(-0.14188940823078156f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.09029786288738251f, (a[5] * b[22] + a[22] * b[5]), fmaf(0.11262122541666031f, (a[4] * b[23] + a[23] * b[4]), 0.23841361701488495f * a[11] * b[2]))))));
+        o[20] = ((fmaf(-0.08369845151901245f, a[22] * b[22], fmaf(-0.08369845151901245f, a[18] * b[18], fmaf(0.04029925540089607f, a[8] * b[8], fmaf(0.24179553985595703f, a[6] * b[6], fmaf(0.04029925540089607f, a[4] * b[4], 0.282094806432724f * (a[0] * b[20] + a[20] * b[0])))))) + fmaf(-0.15978795289993286f, a[23] * b[23], fmaf(0.06848055124282837f, a[19] * b[19], fmaf(-0.19036461412906647f, (a[8] * b[22] + a[22] * b[8]), fmaf(0.16383977234363556f, (a[6] * b[20] + a[20] * b[6]), fmaf(-0.19036461412906647f, (a[4] * b[18] + a[18] * b[4]), -0.15078601241111755f * a[11] * b[1])))))) + (fmaf(0.10652530938386917f, a[24] * b[24], fmaf(0.13696110248565674f, a[20] * b[20], fmaf(0.10652530938386917f, a[16] * b[16], fmaf(-0.1611970216035843f, a[7] * b[7], fmaf(-0.1611970216035843f, a[5] * b[5], 0.2462325245141983f * a[12] * b[2]))))) + fmaf(0.06848055124282837f, a[21] * b[21], fmaf(-0.15978795289993286f, a[17] * b[17], fmaf(0.04486937075853348f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.04486937075853348f, (a[5] * b[19] + a[19] * b[5]), -0.15078601241111755f * a[13] * b[3]))))));
+        o[21] = ((fmaf(0.10208478569984436f, (a[21] * b[22] + a[22] * b[21]), fmaf(-0.11909890919923782f, (a[16] * b[17] + a[17] * b[16]), fmaf(0.04486937075853348f, (a[7] * b[20] + a[20] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[18] + a[18] * b[5]), fmaf(-0.07539300620555878f, a[14] * b[3], 0.282094806432724f * (a[0] * b[21] + a[21] * b[0])))))) + fmaf(0.045015156269073486f, (a[22] * b[23] + a[23] * b[22]), fmaf(0.045015156269073486f, (a[17] * b[18] + a[18] * b[17]), fmaf(0.09029786288738251f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.22072811424732208f, (a[6] * b[7] + a[7] * b[6]), fmaf(-0.06371872127056122f, (a[4] * b[5] + a[5] * b[4]), -0.07539300620555878f * a[10] * b[1])))))) + (fmaf(-0.11909890919923782f, (a[23] * b[24] + a[24] * b[23]), fmaf(0.10208478569984436f, (a[18] * b[19] + a[19] * b[18]), fmaf(0.14188940823078156f, (a[8] * b[21] + a[21] * b[8]), fmaf(0.1392638087272644f, (a[6] * b[21] + a[21] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[17] + a[17] * b[4]), 0.23841361701488495f * a[13] * b[2]))))) + fmaf(0.06848055124282837f, (a[20] * b[21] + a[21] * b[20]), fmaf(-0.11262122541666031f, (a[8] * b[23] + a[23] * b[8]), fmaf(-0.06371872127056122f, (a[7] * b[8] + a[8] * b[7]), fmaf(0.14188940823078156f, (a[4] * b[19] + a[19] * b[4]), 0.1946638971567154f * a[12] * b[3]))))));
+        o[22] = ((fmaf(-0.08369845151901245f, (a[20] * b[22] + a[22] * b[20]), fmaf(-0.07508081942796707f, (a[8] * b[24] + a[24] * b[8]), fmaf(0.180223748087883f, a[7] * b[7], fmaf(0.13272538781166077f, (a[5] * b[17] + a[17] * b[5]), fmaf(0.16858388483524323f, a[13] * b[3], 0.282094806432724f * (a[0] * b[22] + a[22] * b[0])))))) + fmaf(0.10208478569984436f, a[21] * b[21], fmaf(0.13504546880722046f, (a[16] * b[18] + a[18] * b[16]), fmaf(0.09029786288738251f, (a[7] * b[21] + a[21] * b[7]), fmaf(-0.09029786288738251f, (a[5] * b[19] + a[19] * b[5]), fmaf(-0.04352817311882973f, a[15] * b[3], -0.04352817311882973f * a[9] * b[1])))))) + (fmaf(0.045015156269073486f, (a[21] * b[23] + a[23] * b[21]), fmaf(0.045015156269073486f, (a[17] * b[19] + a[19] * b[17]), fmaf(0.13272538781166077f, (a[7] * b[23] + a[23] * b[7]), fmaf(0.15607835352420807f, (a[6] * b[8] + a[8] * b[6]), fmaf(-0.07508081942796707f, (a[4] * b[16] + a[16] * b[4]), -0.16858388483524323f * a[11] * b[1]))))) + fmaf(0.13504546880722046f, (a[22] * b[24] + a[24] * b[22]), fmaf(-0.10208478569984436f, a[19] * b[19], fmaf(-0.19036461412906647f, (a[8] * b[20] + a[20] * b[8]), fmaf(0.06553591042757034f, (a[6] * b[22] + a[22] * b[6]), fmaf(-0.180223748087883f, a[5] * b[5], 0.21324361860752106f * a[14] * b[2])))))));
+        o[23] = ((fmaf(0.045015156269073486f, (a[21] * b[22] + a[22] * b[21]), fmaf(-0.11262122541666031f, (a[8] * b[21] + a[21] * b[8]), fmaf(-0.057343922555446625f, (a[6] * b[23] + a[23] * b[6]), fmaf(-0.16858388483524323f, (a[4] * b[5] + a[5] * b[4]), 0.282094806432724f * (a[0] * b[23] + a[23] * b[0]))))) + fmaf(-0.11909890919923782f, (a[21] * b[24] + a[24] * b[21]), fmaf(-0.11909890919923782f, (a[16] * b[19] + a[19] * b[16]), fmaf(0.16858388483524323f, (a[7] * b[8] + a[8] * b[7]), fmaf(0.11262122541666031f, (a[4] * b[19] + a[19] * b[4]), -0.1994711458683014f * a[10] * b[1]))))) + (fmaf(-0.045015156269073486f, (a[18] * b[19] + a[19] * b[18]), fmaf(0.13272538781166077f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.14046335220336914f, (a[5] * b[16] + a[16] * b[5]), 0.1628675013780594f * a[15] * b[2]))) + fmaf(-0.15978795289993286f, (a[20] * b[23] + a[23] * b[20]), fmaf(0.14046335220336914f, (a[7] * b[24] + a[24] * b[7]), fmaf(-0.13272538781166077f, (a[5] * b[18] + a[18] * b[5]), 0.1994711458683014f * a[14] * b[3])))));
+        o[24] = ((fmaf(0.10652530938386917f, (a[20] * b[24] + a[24] * b[20]), fmaf(0.23841361701488495f, a[8] * b[8], fmaf(0.07508081942796707f, (a[4] * b[18] + a[18] * b[4]), 0.282094806432724f * (a[0] * b[24] + a[24] * b[0])))) + fmaf(-0.11909890919923782f, (a[21] * b[23] + a[23] * b[21]), fmaf(-0.07508081942796707f, (a[8] * b[22] + a[22] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[17] + a[17] * b[5]), -0.23032943904399872f * a[9] * b[1])))) + (fmaf(0.13504546880722046f, a[22] * b[22], fmaf(0.11909890919923782f, (a[17] * b[19] + a[19] * b[17]), fmaf(-0.2293756902217865f, (a[6] * b[24] + a[24] * b[6]), 0.23032943904399872f * a[15] * b[3]))) + fmaf(-0.13504546880722046f, a[18] * b[18], fmaf(0.14046335220336914f, (a[7] * b[23] + a[23] * b[7]), -0.23841361701488495f * a[4] * b[4]))));
+    }
+    __device__ __forceinline__ static void mul_onto_lobe(const float* __restrict__ a, const float* __restrict__ b,
+                                               float* __restrict__ o) {
+        o[0] = ((fmaf(0.282094806432724f, a[24] * b[24], fmaf(0.282094806432724f, a[20] * b[20], fmaf(0.282094806432724f, a[16] * b[16], fmaf(0.282094806432724f, a[12] * b[12], fmaf(0.282094806432724f, a[8] * b[8], fmaf(0.282094806432724f, a[4] * b[4], 0.282094806432724f * a[0] * b[0])))))) + fmaf(0.282094806432724f, a[21] * b[21], fmaf(0.282094806432724f, a[17] * b[17], fmaf(0.282094806432724f, a[13] * b[13], fmaf(0.282094806432724f, a[9] * b[9], fmaf(0.282094806432724f, a[5] * b[5], 0.282094806432724f * a[1] * b[1])))))) + (fmaf(0.282094806432724f, a[22] * b[22], fmaf(0.282094806432724f, a[18] * b[18], fmaf(0.282094806432724f, a[14] * b[14], fmaf(0.282094806432724f, a[10] * b[10], fmaf(0.282094806432724f, a[6] * b[6], 0.282094806432724f * a[2] * b[2]))))) + fmaf(0.282094806432724f, a[23] * b[23], fmaf(0.282094806432724f, a[19] * b[19], fmaf(0.282094806432724f, a[15] * b[15], fmaf(0.282094806432724f, a[11] * b[11], fmaf(0.282094806432724f, a[7] * b[7], 0.282094806432724f * a[3] * b[3])))))));
+        o[1] = ((fmaf(0.04352817311882973f, (a[15] * b[18] + a[18] * b[15]), fmaf(0.16858388483524323f, (a[13] * b[18] + a[18] * b[13]), fmaf(-0.1994711458683014f, (a[10] * b[23] + a[23] * b[10]), fmaf(0.05839917063713074f, (a[8] * b[11] + a[11] * b[8]), fmaf(-0.18467439711093903f, (a[5] * b[14] + a[14] * b[5]), fmaf(0.21850968897342682f, (a[3] * b[4] + a[4] * b[3]), 0.282094806432724f * (a[0] * b[1] + a[1] * b[0]))))))) + fmaf(0.1994711458683014f, (a[14] * b[17] + a[17] * b[14]), fmaf(-0.15078601241111755f, (a[11] * b[20] + a[20] * b[11]), fmaf(-0.04352817311882973f, (a[9] * b[22] + a[22] * b[9]), fmaf(0.20230065286159515f, (a[6] * b[11] + a[11] * b[6]), fmaf(-0.05839917063713074f, (a[4] * b[13] + a[13] * b[4]), -0.12615662813186646f * (a[1] * b[6] + a[6] * b[1]))))))) + (fmaf(0.07539300620555878f, (a[14] * b[19] + a[19] * b[14]), fmaf(-0.16858388483524323f, (a[11] * b[22] + a[22] * b[11]), fmaf(-0.23032943904399872f, (a[9] * b[24] + a[24] * b[9]), fmaf(0.18467439711093903f, (a[7] * b[10] + a[10] * b[7]), fmaf(-0.22617901861667633f, (a[4] * b[15] + a[15] * b[4]), -0.21850968897342682f * (a[1] * b[8] + a[8] * b[1])))))) + fmaf(0.23032943904399872f, (a[15] * b[16] + a[16] * b[15]), fmaf(0.1946638971567154f, (a[12] * b[19] + a[19] * b[12]), fmaf(-0.07539300620555878f, (a[10] * b[21] + a[21] * b[10]), fmaf(0.22617901861667633f, (a[8] * b[9] + a[9] * b[8]), fmaf(-0.14304816722869873f, (a[5] * b[12] + a[12] * b[5]), 0.21850968897342682f * (a[2] * b[5] + a[5] * b[2]))))))));
+        o[2] = ((fmaf(0.2462325245141983f, (a[12] * b[20] + a[20] * b[12]), fmaf(0.18467439711093903f, (a[8] * b[14] + a[14] * b[8]), fmaf(0.18467439711093903f, (a[4] * b[10] + a[10] * b[4]), 0.282094806432724f * (a[0] * b[2] + a[2] * b[0])))) + fmaf(0.23841361701488495f, (a[13] * b[21] + a[21] * b[13]), fmaf(0.1628675013780594f, (a[9] * b[17] + a[17] * b[9]), fmaf(0.23359668254852295f, (a[5] * b[11] + a[11] * b[5]), 0.21850968897342682f * (a[1] * b[5] + a[5] * b[1]))))) + (fmaf(0.21324361860752106f, (a[14] * b[22] + a[22] * b[14]), fmaf(0.21324361860752106f, (a[10] * b[18] + a[18] * b[10]), fmaf(0.24776668846607208f, (a[6] * b[12] + a[12] * b[6]), 0.2523132562637329f * (a[2] * b[6] + a[6] * b[2])))) + fmaf(0.1628675013780594f, (a[15] * b[23] + a[23] * b[15]), fmaf(0.23841361701488495f, (a[11] * b[19] + a[19] * b[11]), fmaf(0.23359668254852295f, (a[7] * b[13] + a[13] * b[7]), 0.21850968897342682f * (a[3] * b[7] + a[7] * b[3]))))));
+        o[3] = ((fmaf(0.23032943904399872f, (a[15] * b[24] + a[24] * b[15]), fmaf(0.16858388483524323f, (a[13] * b[22] + a[22] * b[13]), fmaf(-0.07539300620555878f, (a[10] * b[19] + a[19] * b[10]), fmaf(0.22617901861667633f, (a[8] * b[15] + a[15] * b[8]), fmaf(0.20230065286159515f, (a[6] * b[13] + a[13] * b[6]), fmaf(0.21850968897342682f, (a[3] * b[8] + a[8] * b[3]), 0.282094806432724f * (a[0] * b[3] + a[3] * b[0]))))))) + fmaf(-0.07539300620555878f, (a[14] * b[21] + a[21] * b[14]), fmaf(0.16858388483524323f, (a[11] * b[18] + a[18] * b[11]), fmaf(0.23032943904399872f, (a[9] * b[16] + a[16] * b[9]), fmaf(-0.14304816722869873f, (a[7] * b[12] + a[12] * b[7]), fmaf(0.22617901861667633f, (a[4] * b[9] + a[9] * b[4]), 0.21850968897342682f * (a[1] * b[4] + a[4] * b[1]))))))) + (fmaf(0.1994711458683014f, (a[14] * b[23] + a[23] * b[14]), fmaf(0.1946638971567154f, (a[12] * b[21] + a[21] * b[12]), fmaf(-0.04352817311882973f, (a[9] * b[18] + a[18] * b[9]), fmaf(0.18467439711093903f, (a[7] * b[14] + a[14] * b[7]), fmaf(-0.05839917063713074f, (a[4] * b[11] + a[11] * b[4]), 0.21850968897342682f * (a[2] * b[7] + a[7] * b[2])))))) + fmaf(-0.04352817311882973f, (a[15] * b[22] + a[22] * b[15]), fmaf(-0.15078601241111755f, (a[13] * b[20] + a[20] * b[13]), fmaf(0.1994711458683014f, (a[10] * b[17] + a[17] * b[10]), fmaf(-0.05839917063713074f, (a[8] * b[13] + a[13] * b[8]), fmaf(0.18467439711093903f, (a[5] * b[10] + a[10] * b[5]), -0.12615662813186646f * (a[3] * b[6] + a[6] * b[3]))))))));
+        o[4] = ((fmaf(0.07508081942796707f, (a[18] * b[24] + a[24] * b[18]), fmaf(0.09403159469366074f, (a[11] * b[15] + a[15] * b[11]), fmaf(0.23841361701488495f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.16858388483524323f, (a[5] * b[23] + a[23] * b[5]), fmaf(0.04029925540089607f, (a[4] * b[20] + a[20] * b[4]), fmaf(0.18467439711093903f, (a[2] * b[10] + a[10] * b[2]), 0.282094806432724f * (a[0] * b[4] + a[4] * b[0]))))))) + fmaf(0.14188940823078156f, (a[19] * b[21] + a[21] * b[19]), fmaf(-0.07508081942796707f, (a[16] * b[22] + a[22] * b[16]), fmaf(-0.09403159469366074f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.15607835352420807f, (a[6] * b[18] + a[18] * b[6]), fmaf(-0.23841361701488495f, (a[4] * b[24] + a[24] * b[4]), fmaf(0.22617901861667633f, (a[3] * b[9] + a[9] * b[3]), 0.21850968897342682f * (a[1] * b[3] + a[3] * b[1])))))))) + (fmaf(0.11262122541666031f, (a[19] * b[23] + a[23] * b[19]), fmaf(-0.11262122541666031f, (a[17] * b[21] + a[21] * b[17]), fmaf(-0.18806318938732147f, (a[10] * b[12] + a[12] * b[10]), fmaf(0.16858388483524323f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.15607835352420807f, (a[5] * b[7] + a[7] * b[5]), fmaf(-0.05839917063713074f, (a[3] * b[11] + a[11] * b[3]), -0.05839917063713074f * (a[1] * b[13] + a[13] * b[1]))))))) + fmaf(-0.19036461412906647f, (a[18] * b[20] + a[20] * b[18]), fmaf(0.14567312598228455f, (a[11] * b[13] + a[13] * b[11]), fmaf(-0.06371872127056122f, (a[7] * b[19] + a[19] * b[7]), fmaf(-0.06371872127056122f, (a[5] * b[21] + a[21] * b[5]), fmaf(-0.180223748087883f, (a[4] * b[6] + a[6] * b[4]), -0.22617901861667633f * (a[1] * b[15] + a[15] * b[1]))))))));
+        o[5] = ((fmaf(-0.09029786288738251f, (a[19] * b[22] + a[22] * b[19]), fmaf(-0.14046335220336914f, (a[17] * b[24] + a[24] * b[17]), fmaf(0.059470802545547485f, (a[11] * b[12] + a[12] * b[11]), fmaf(0.06371872127056122f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.180223748087883f, (a[5] * b[22] + a[22] * b[5]), fmaf(-0.16858388483524323f, (a[4] * b[23] + a[23] * b[4]), fmaf(0.23359668254852295f, (a[2] * b[11] + a[11] * b[2]), 0.282094806432724f * (a[0] * b[5] + a[5] * b[0])))))))) + fmaf(0.09029786288738251f, (a[18] * b[21] + a[21] * b[18]), fmaf(-0.11516471952199936f, (a[11] * b[14] + a[14] * b[11]), fmaf(0.1486770063638687f, (a[9] * b[14] + a[14] * b[9]), fmaf(0.22072811424732208f, (a[6] * b[19] + a[19] * b[6]), fmaf(0.0901118740439415f, (a[5] * b[6] + a[6] * b[5]), fmaf(0.18467439711093903f, (a[3] * b[10] + a[10] * b[3]), 0.21850968897342682f * (a[1] * b[2] + a[2] * b[1])))))))) + (fmaf(-0.13272538781166077f, (a[18] * b[23] + a[23] * b[18]), fmaf(0.14046335220336914f, (a[16] * b[23] + a[23] * b[16]), fmaf(0.11516471952199936f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.180223748087883f, (a[7] * b[18] + a[18] * b[7]), fmaf(-0.15607835352420807f, (a[5] * b[8] + a[8] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[7] + a[7] * b[4]), -0.14304816722869873f * (a[1] * b[12] + a[12] * b[1]))))))) + fmaf(0.04486937075853348f, (a[19] * b[20] + a[20] * b[19]), fmaf(0.13272538781166077f, (a[17] * b[22] + a[22] * b[17]), fmaf(-0.1486770063638687f, (a[10] * b[15] + a[15] * b[10]), fmaf(0.16858388483524323f, (a[8] * b[17] + a[17] * b[8]), fmaf(-0.1611970216035843f, (a[5] * b[20] + a[20] * b[5]), fmaf(-0.06371872127056122f, (a[4] * b[21] + a[21] * b[4]), -0.18467439711093903f * (a[1] * b[14] + a[14] * b[1])))))))));
+        o[6] = ((fmaf(0.06553591042757034f, a[22] * b[22], fmaf(0.06553591042757034f, a[18] * b[18], fmaf(0.12615662813186646f, a[13] * b[13], fmaf(0.15607835352420807f, (a[8] * b[22] + a[22] * b[8]), fmaf(0.24179553985595703f, (a[6] * b[20] + a[20] * b[6]), fmaf(0.15607835352420807f, (a[4] * b[18] + a[18] * b[4]), fmaf(0.24776668846607208f, (a[2] * b[12] + a[12] * b[2]), 0.282094806432724f * (a[0] * b[6] + a[6] * b[0])))))))) + fmaf(-0.057343922555446625f, a[23] * b[23], fmaf(0.1392638087272644f, a[19] * b[19], fmaf(-0.2102610468864441f, a[15] * b[15], fmaf(-0.2102610468864441f, a[9] * b[9], fmaf(0.0901118740439415f, a[7] * b[7], fmaf(0.0901118740439415f, a[5] * b[5], fmaf(-0.12615662813186646f, a[3] * b[3], -0.12615662813186646f * a[1] * b[1])))))))) + (fmaf(-0.2293756902217865f, a[24] * b[24], fmaf(0.16383977234363556f, a[20] * b[20], fmaf(-0.2293756902217865f, a[16] * b[16], fmaf(0.12615662813186646f, a[11] * b[11], fmaf(0.22072811424732208f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.22072811424732208f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.20230065286159515f, (a[3] * b[13] + a[13] * b[3]), 0.20230065286159515f * (a[1] * b[11] + a[11] * b[1])))))))) + fmaf(0.1392638087272644f, a[21] * b[21], fmaf(-0.057343922555446625f, a[17] * b[17], fmaf(0.16820883750915527f, a[12] * b[12], fmaf(-0.180223748087883f, a[8] * b[8], fmaf(0.180223748087883f, a[6] * b[6], fmaf(-0.180223748087883f, a[4] * b[4], 0.2523132562637329f * a[2] * b[2]))))))));
+        o[7] = ((fmaf(0.14046335220336914f, (a[23] * b[24] + a[24] * b[23]), fmaf(0.09029786288738251f, (a[18] * b[19] + a[19] * b[18]), fmaf(0.11516471952199936f, (a[13] * b[14] + a[14] * b[13]), fmaf(0.16858388483524323f, (a[8] * b[23] + a[23] * b[8]), fmaf(0.15607835352420807f, (a[7] * b[8] + a[8] * b[7]), fmaf(-0.06371872127056122f, (a[4] * b[19] + a[19] * b[4]), fmaf(-0.14304816722869873f, (a[3] * b[12] + a[12] * b[3]), 0.282094806432724f * (a[0] * b[7] + a[7] * b[0])))))))) + fmaf(0.04486937075853348f, (a[20] * b[21] + a[21] * b[20]), fmaf(0.1486770063638687f, (a[14] * b[15] + a[15] * b[14]), fmaf(0.1486770063638687f, (a[9] * b[10] + a[10] * b[9]), fmaf(-0.1611970216035843f, (a[7] * b[20] + a[20] * b[7]), fmaf(0.180223748087883f, (a[5] * b[18] + a[18] * b[5]), fmaf(0.18467439711093903f, (a[3] * b[14] + a[14] * b[3]), 0.18467439711093903f * (a[1] * b[10] + a[10] * b[1])))))))) + (fmaf(0.09029786288738251f, (a[21] * b[22] + a[22] * b[21]), fmaf(0.14046335220336914f, (a[16] * b[17] + a[17] * b[16]), fmaf(0.11516471952199936f, (a[10] * b[11] + a[11] * b[10]), fmaf(0.180223748087883f, (a[7] * b[22] + a[22] * b[7]), fmaf(0.0901118740439415f, (a[6] * b[7] + a[7] * b[6]), fmaf(0.15607835352420807f, (a[4] * b[5] + a[5] * b[4]), 0.21850968897342682f * (a[2] * b[3] + a[3] * b[2]))))))) + fmaf(0.13272538781166077f, (a[22] * b[23] + a[23] * b[22]), fmaf(0.13272538781166077f, (a[17] * b[18] + a[18] * b[17]), fmaf(0.059470802545547485f, (a[12] * b[13] + a[13] * b[12]), fmaf(-0.06371872127056122f, (a[8] * b[21] + a[21] * b[8]), fmaf(0.22072811424732208f, (a[6] * b[21] + a[21] * b[6]), fmaf(0.16858388483524323f, (a[4] * b[17] + a[17] * b[4]), 0.23359668254852295f * (a[2] * b[13] + a[13] * b[2])))))))));
+        o[8] = ((fmaf(0.14188940823078156f, a[21] * b[21], fmaf(-0.07508081942796707f, (a[16] * b[18] + a[18] * b[16]), fmaf(-0.14567312598228455f, a[11] * b[11], fmaf(0.16858388483524323f, (a[7] * b[23] + a[23] * b[7]), fmaf(-0.180223748087883f, (a[6] * b[8] + a[8] * b[6]), fmaf(0.23841361701488495f, (a[4] * b[16] + a[16] * b[4]), fmaf(0.18467439711093903f, (a[2] * b[14] + a[14] * b[2]), 0.282094806432724f * (a[0] * b[8] + a[8] * b[0])))))))) + fmaf(-0.11262122541666031f, (a[21] * b[23] + a[23] * b[21]), fmaf(-0.11262122541666031f, (a[17] * b[19] + a[19] * b[17]), fmaf(-0.18806318938732147f, (a[12] * b[14] + a[14] * b[12]), fmaf(0.04029925540089607f, (a[8] * b[20] + a[20] * b[8]), fmaf(0.15607835352420807f, (a[6] * b[22] + a[22] * b[6]), fmaf(-0.15607835352420807f, a[5] * b[5], fmaf(0.21850968897342682f, a[3] * b[3], -0.21850968897342682f * a[1] * b[1])))))))) + (fmaf(-0.07508081942796707f, (a[22] * b[24] + a[24] * b[22]), fmaf(-0.14188940823078156f, a[19] * b[19], fmaf(0.14567312598228455f, a[13] * b[13], fmaf(0.23841361701488495f, (a[8] * b[24] + a[24] * b[8]), fmaf(0.15607835352420807f, a[7] * b[7], fmaf(0.16858388483524323f, (a[5] * b[17] + a[17] * b[5]), fmaf(-0.05839917063713074f, (a[3] * b[13] + a[13] * b[3]), 0.22617901861667633f * (a[1] * b[9] + a[9] * b[1])))))))) + fmaf(-0.19036461412906647f, (a[20] * b[22] + a[22] * b[20]), fmaf(-0.09403159469366074f, (a[13] * b[15] + a[15] * b[13]), fmaf(-0.09403159469366074f, (a[9] * b[11] + a[11] * b[9]), fmaf(-0.06371872127056122f, (a[7] * b[21] + a[21] * b[7]), fmaf(0.06371872127056122f, (a[5] * b[19] + a[19] * b[5]), fmaf(0.22617901861667633f, (a[3] * b[15] + a[15] * b[3]), 0.05839917063713074f * (a[1] * b[11] + a[11] * b[1])))))))));
+        o[9] = 0.0f;
+        o[10] = 0.0f;
+        o[11] = 0.0f;
+        o[12] = 0.0f;
+        o[13] = 0.0f;
+        o[14] = 0.0f;
+        o[15] = 0.0f;
         o[16] = ((fmaf(0.10652530938386917f, (a[16] * b[20] + a[20] * b[16]), fmaf(-0.07508081942796707f, (a[8] * b[18] + a[18] * b[8]), fmaf(-0.07508081942796707f, (a[4] * b[22] + a[22] * b[4]), 0.282094806432724f * (a[0] * b[16] + a[16] * b[0])))) + fmaf(-0.11909890919923782f, (a[17] * b[21] + a[21] * b[17]), fmaf(-0.11752006411552429f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.14046335220336914f, (a[5] * b[23] + a[23] * b[5]), 0.23032943904399872f * (a[1] * b[15] + a[15] * b[1]))))) + (fmaf(0.13504546880722046f, (a[18] * b[22] + a[22] * b[18]), fmaf(0.15171775221824646f, (a[10] * b[14] + a[14] * b[10]), fmaf(-0.2293756902217865f, (a[6] * b[16] + a[16] * b[6]), 0.23032943904399872f * (a[3] * b[9] + a[9] * b[3])))) + fmaf(-0.11909890919923782f, (a[19] * b[23] + a[23] * b[19]), fmaf(-0.11752006411552429f, (a[11] * b[15] + a[15] * b[11]), fmaf(0.14046335220336914f, (a[7] * b[17] + a[17] * b[7]), 0.23841361701488495f * (a[4] * b[8] + a[8] * b[4]))))));
         o[17] = ((fmaf(0.11909890919923782f, (a[19] * b[24] + a[24] * b[19]), fmaf(-0.11909890919923782f, (a[16] * b[21] + a[21] * b[16]), fmaf(-0.11262122541666031f, (a[8] * b[19] + a[19] * b[8]), fmaf(-0.14046335220336914f, (a[5] * b[24] + a[24] * b[5]), fmaf(0.16858388483524323f, (a[4] * b[7] + a[7] * b[4]), 0.282094806432724f * (a[0] * b[17] + a[17] * b[0])))))) + fmaf(-0.15978795289993286f, (a[17] * b[20] + a[20] * b[17]), fmaf(-0.20355072617530823f, (a[9] * b[12] + a[12] * b[9]), fmaf(-0.057343922555446625f, (a[6] * b[17] + a[17] * b[6]), fmaf(-0.11262122541666031f, (a[4] * b[21] + a[21] * b[4]), 0.1994711458683014f * (a[1] * b[14] + a[14] * b[1])))))) + (fmaf(0.045015156269073486f, (a[18] * b[21] + a[21] * b[18]), fmaf(0.06785023957490921f, (a[10] * b[13] + a[13] * b[10]), fmaf(0.14046335220336914f, (a[7] * b[16] + a[16] * b[7]), fmaf(0.16858388483524323f, (a[5] * b[8] + a[8] * b[5]), 0.1628675013780594f * (a[2] * b[9] + a[9] * b[2]))))) + fmaf(0.045015156269073486f, (a[19] * b[22] + a[22] * b[19]), fmaf(0.06785023957490921f, (a[11] * b[14] + a[14] * b[11]), fmaf(0.13272538781166077f, (a[7] * b[18] + a[18] * b[7]), fmaf(0.13272538781166077f, (a[5] * b[22] + a[22] * b[5]), 0.1994711458683014f * (a[3] * b[10] + a[10] * b[3])))))));
         o[18] = ((fmaf(0.10208478569984436f, (a[19] * b[21] + a[21] * b[19]), fmaf(0.13504546880722046f, (a[16] * b[22] + a[22] * b[16]), fmaf(0.1332552284002304f, (a[9] * b[13] + a[13] * b[9]), fmaf(0.06553591042757034f, (a[6] * b[18] + a[18] * b[6]), fmaf(0.07508081942796707f, (a[4] * b[24] + a[24] * b[4]), fmaf(-0.04352817311882973f, (a[3] * b[9] + a[9] * b[3]), 0.282094806432724f * (a[0] * b[18] + a[18] * b[0]))))))) + fmaf(-0.045015156269073486f, (a[19] * b[23] + a[23] * b[19]), fmaf(0.045015156269073486f, (a[17] * b[21] + a[21] * b[17]), fmaf(-0.04441840946674347f, (a[10] * b[12] + a[12] * b[10]), fmaf(0.13272538781166077f, (a[7] * b[17] + a[17] * b[7]), fmaf(0.180223748087883f, (a[5] * b[7] + a[7] * b[5]), fmaf(0.16858388483524323f, (a[3] * b[11] + a[11] * b[3]), 0.16858388483524323f * (a[1] * b[13] + a[13] * b[1])))))))) + (fmaf(-0.08369845151901245f, (a[18] * b[20] + a[20] * b[18]), fmaf(0.11468784511089325f, (a[11] * b[13] + a[13] * b[11]), fmaf(0.09029786288738251f, (a[7] * b[19] + a[19] * b[7]), fmaf(0.09029786288738251f, (a[5] * b[21] + a[21] * b[5]), fmaf(0.15607835352420807f, (a[4] * b[6] + a[6] * b[4]), 0.04352817311882973f * (a[1] * b[15] + a[15] * b[1])))))) + fmaf(-0.13504546880722046f, (a[18] * b[24] + a[24] * b[18]), fmaf(-0.1332552284002304f, (a[11] * b[15] + a[15] * b[11]), fmaf(-0.07508081942796707f, (a[8] * b[16] + a[16] * b[8]), fmaf(-0.13272538781166077f, (a[5] * b[23] + a[23] * b[5]), fmaf(-0.19036461412906647f, (a[4] * b[20] + a[20] * b[4]), 0.21324361860752106f * (a[2] * b[10] + a[10] * b[2]))))))));

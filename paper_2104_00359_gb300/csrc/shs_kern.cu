@@ -120,46 +120,77 @@ __device__ __forceinline__ void interleave_sphere_pairs(float4* s_sph, int N) {
     }
 }
 
-// Adjoint of one pair given dfp_i = dLoss/df_i * (-2 pi eps) * NORM_i: the
-// gradients with respect to the sphere centre (the point gets the negative)
-// and the radius, through the per-band homogeneous polynomials
-// Phi_l(s) = sum_m dfp_lm Hbar_lm(s) (degree l).  The pair's loss term is
-// Psi = sum_l G_l(c) Phi_l(s_hat).  Euler's identity s . grad Phi_l = l Phi_l
-// makes every needed quantity a dot product with the per-band gradients:
+// Adjoint of two pairs, one sphere with two points (one per half of every
+// float2), in the packed float32x2 instructions.  The pair's loss term is
+// Psi = sum_l G_l(c) Phi_l(s_hat) with the per-band homogeneous polynomials
+// Phi_l(s) = sum_m dfp_lm Hbar_lm(s) (degree l), dfp_i = dLoss/df_i (-2 pi eps)
+// NORM_i.  Euler's identity s . grad Phi_l = l Phi_l makes every needed
+// quantity a dot product with the per-band gradients:
 //   a = sum_l G_l grad Phi_l,    b = sum_l (P_l / l) grad Phi_l   (l >= 1)
 //   dPsi/dc = -sum_l P_l Phi_l = -(s_hat . b) - Phi_0
 //   dPsi/dd = (a - (s_hat . a) s_hat) / D + 2 (dPsi/dD^2) d
-// so only the gradient polynomials (degree l-1) are evaluated per pair.
-template <bool CULL = false>
-__device__ __forceinline__ void pair_backward_grad(float px, float py, float pz, float4 sp,
-                                                   const float* gq, float q0, float& gcx,
-                                                   float& gcy, float& gcz, float& gr, Normal u = {}) {
-    const PairGeom g = pair_geometry<CULL>(px, py, pz, sp, u);
-    float P[NB], G[NB];
-    cap_closed(g.c, g.s2, G, P);
-    const float sx = g.dx * g.invD, sy = g.dy * g.invD, sz = g.dz * g.invD;
-    float gx[NB], gy[NB], gz[NB];
-    SH::grad_eval(sx, sy, sz, gq, gx, gy, gz);
-    float ax = 0.f, ay = 0.f, az = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
+// so only the gradient polynomials (degree l-1) are evaluated per pair.  q:
+// the two points' x, y, z, Phi_0 and tensor entries.  The results
+// are the gradients with respect to the sphere's centre (the points get the
+// negatives) and radius.
+template <bool CULL>
+__device__ __forceinline__ void pair_backward2(float4 sp, const float2* q, float2* d, const float2* u) {
+    const float2 one = make_float2(1.f, 1.f);
+    const PairGeom2 g = pair_geometry2<CULL>(q[0], q[1], q[2], sp, u);
+    const float2 s2 = g.s2, c = g.c, sx = __fmul2_rn(g.dx, g.invD), sy = __fmul2_rn(g.dy, g.invD),
+                 sz = __fmul2_rn(g.dz, g.invD);
+    float2 dc = q[3], ax{}, ay{}, az{};   // dc: -dPsi/dc
+    if constexpr (NB > 1) {
+        float2 gx[NB - 1], gy[NB - 1], gz[NB - 1], G[NB], Pl[NB];   // Pl: P_l / l
+        SH::grad_eval2(sx, sy, sz, [&](int o) { return q[4 + o]; }, gx, gy, gz);
+        auto k2 = [](float v) { return make_float2(v, v); };
+        G[1] = __fmul2_rn(k2(0.5f), s2);
+        Pl[1] = c;
+        if constexpr (NB > 2) {
+            G[2] = __fmul2_rn(G[1], c);
+            Pl[2] = __ffma2_rn(k2(-0.75f), s2, k2(0.5f));
+        }
+        if constexpr (NB > 3) {
+            G[3] = __fmul2_rn(s2, __ffma2_rn(k2(-0.625f), s2, k2(0.5f)));
+            Pl[3] = __fmul2_rn(c, __ffma2_rn(k2(-2.5f / 3.f), s2, k2(1.f / 3.f)));
+        }
+        if constexpr (NB > 4) {
+            G[4] = __fmul2_rn(G[2], __ffma2_rn(k2(-1.75f), s2, one));
+            Pl[4] = __ffma2_rn(s2, __ffma2_rn(k2(4.375f / 4.f), s2, k2(-1.25f)), k2(0.25f));
+        }
+        ax = __fmul2_rn(G[1], gx[0]);
+        ay = __fmul2_rn(G[1], gy[0]);
+        az = __fmul2_rn(G[1], gz[0]);
+        float2 bx = __fmul2_rn(Pl[1], gx[0]), by = __fmul2_rn(Pl[1], gy[0]), bz = __fmul2_rn(Pl[1], gz[0]);
 #pragma unroll
-    for (int l = 1; l < NB; ++l) {
-        ax = fmaf(G[l], gx[l - 1], ax);
-        ay = fmaf(G[l], gy[l - 1], ay);
-        az = fmaf(G[l], gz[l - 1], az);
-        const float pl = P[l] * (1.f / float(l));
-        bx = fmaf(pl, gx[l - 1], bx);
-        by = fmaf(pl, gy[l - 1], by);
-        bz = fmaf(pl, gz[l - 1], bz);
+        for (int l = 2; l < NB; ++l) {
+            ax = __ffma2_rn(G[l], gx[l - 1], ax);
+            ay = __ffma2_rn(G[l], gy[l - 1], ay);
+            az = __ffma2_rn(G[l], gz[l - 1], az);
+            bx = __ffma2_rn(Pl[l], gx[l - 1], bx);
+            by = __ffma2_rn(Pl[l], gy[l - 1], by);
+            bz = __ffma2_rn(Pl[l], gz[l - 1], bz);
+        }
+        dc = __ffma2_rn(sx, bx, __ffma2_rn(sy, by, __ffma2_rn(sz, bz, dc)));
     }
-    const float rad = fmaf(sx, ax, fmaf(sy, ay, sz * az));
-    const float dc = -fmaf(sx, bx, fmaf(sy, by, fmaf(sz, bz, q0)));
-    // c = sqrt(1 - s2): d c / d s2 = -1 / (2 c); clamped caps carry no gradient
-    const float ds2 = g.open ? __fdividef(-0.5f * dc, g.c) : 0.f;
-    gr = ds2 * 2.f * sp.w * g.invD2;                      // s2 = r^2 / D^2
-    const float coef = -2.f * ds2 * g.s2 * g.invD2;        // 2 dPsi/dD^2
-    gcx = fmaf(fmaf(-rad, sx, ax), g.invD, coef * g.dx);
-    gcy = fmaf(fmaf(-rad, sy, ay), g.invD, coef * g.dy);
-    gcz = fmaf(fmaf(-rad, sz, az), g.invD, coef * g.dz);
+    pair_finish2(g, sp.w, sx, sy, sz, ax, ay, az, dc, d);
+}
+
+// A warp's 32 points for the pair adjoint: 16 rows of two points each, per row
+// x, y, z, Phi_0 and the NG tensor entries as float2; the row length (in
+// float2, 2 mod 4) spreads the lanes' writes over the banks.
+constexpr int kRowUsed = 4 + SH::NG;
+constexpr int kRow = kRowUsed + (6 - kRowUsed % 4) % 4;
+constexpr int kWarpRows = 16;
+static_assert(kRow % 4 == 2 && kRow >= kRowUsed, "row length");
+
+__device__ __forceinline__ void load_row(const float4* row, float2* q) {
+#pragma unroll
+    for (int i = 0; i < (kRowUsed + 1) / 2; ++i) {
+        const float4 v = row[i];
+        q[2 * i] = make_float2(v.x, v.y);
+        q[2 * i + 1] = make_float2(v.z, v.w);
+    }
 }
 
 __host__ __device__ constexpr int harm_of(int i) {   // 0: 1, 2m-1: cos m phi, 2m: sin m phi
@@ -375,7 +406,7 @@ __device__ __forceinline__ void forward_point(const FwdArgs& a, const float4* s_
     cosine_lobe(__ldg(a.normals + 3 * p), __ldg(a.normals + 3 * p + 1), __ldg(a.normals + 3 * p + 2),
                 H, ux, uy, uz, il);
     float W[K];
-    SH::mul(V, H, W);
+    SH::mul_lobe(V, H, W);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         float d = 0.f;
@@ -414,19 +445,106 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? SHS_FWD_MINB : 1) forward_ke
 // backward kernel
 // ---------------------------------------------------------------------------
 
-// Sum four values over the warp; lane l returns the total of value (l >> 3).
-__device__ __forceinline__ float warp_sum4(float v0, float v1, float v2, float v3, int lane) {
-    const bool h16 = lane & 16;
-    float ka = h16 ? v2 : v0, kb = h16 ? v3 : v1;
-    ka += __shfl_xor_sync(0xffffffffu, h16 ? v0 : v2, 16);
-    kb += __shfl_xor_sync(0xffffffffu, h16 ? v1 : v3, 16);
-    const bool h8 = lane & 8;
-    float k = h8 ? kb : ka;
-    k += __shfl_xor_sync(0xffffffffu, h8 ? ka : kb, 8);
-    k += __shfl_xor_sync(0xffffffffu, k, 4);
-    k += __shfl_xor_sync(0xffffffffu, k, 2);
-    k += __shfl_xor_sync(0xffffffffu, k, 1);
-    return k;
+// Pair adjoints of the warp's 32 points from 32 spheres on.  A pair of lanes
+// holds a row's coefficients in registers and takes every second sphere; the
+// rows walk the spheres at different offsets, so the 32 lanes update 32
+// distinct slots of the warp's sphere sums with plain shared-memory
+// read-modify-writes, and the point gradients stay in registers.  (Spheres on
+// the lanes and the rows' coefficients read as broadcasts measured the same
+// without point gradients and 35 % slower with them: those need a sum over the
+// lanes per row, and the last step idles lanes.)
+template <bool CULL>
+__device__ __forceinline__ void warp_pairs(const BwdArgs& a, const float4* s_sph, const float4* rows,
+                                           const float2 (*nrm)[3], float4* acc_row, int64_t p0, int lane) {
+    const int N = a.sc.n_spheres, M = (N + 1) >> 1, r = lane >> 1, h = lane & 1;
+    float2 q[kRowUsed + 1], u[3] = {}, gp[3] = {};
+    load_row(rows + r * (kRow / 2), q);
+    if constexpr (CULL) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e) u[e] = nrm[r][e];
+    }
+    int m = r;   // M >= 16 rows
+#pragma unroll 1
+    for (int t = 0; t < M; ++t) {
+        const int j = 2 * m + h;
+        const bool has = j < N;
+        const float4 sp = has ? s_sph[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float2 d[4];
+        pair_backward2<CULL>(sp, q, d, u);
+        if (has) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) gp[e] = __fadd2_rn(gp[e], d[e]);
+            float4 v = acc_row[j];
+            v.x += d[0].x + d[0].y;
+            v.y += d[1].x + d[1].y;
+            v.z += d[2].x + d[2].y;
+            v.w += d[3].x + d[3].y;
+            acc_row[j] = v;
+        }
+        __syncwarp();
+        m = m + 1 == M ? 0 : m + 1;
+    }
+    if (!a.d_points) return;
+    // the row's point h is this lane's
+    const int64_t p = p0 + lane;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        gp[e].x += __shfl_xor_sync(0xffffffffu, gp[e].x, 1);
+        gp[e].y += __shfl_xor_sync(0xffffffffu, gp[e].y, 1);
+        if (p < a.n_points) a.d_points[3 * p + e] = -(h ? gp[e].y : gp[e].x);
+    }
+}
+
+// Fewer than 32 spheres: the lanes hold `width` spheres (32, 16 or 8, then one,
+// two or four rows at once); a row's sums stay in registers over the spheres
+// and are summed over the lanes once.
+template <bool CULL>
+__device__ __forceinline__ void warp_pairs_few(const BwdArgs& a, const float4* s_sph, const float4* rows,
+                                               const float2 (*nrm)[3], float4* acc_row, int64_t p0, int lane) {
+    const int N = a.sc.n_spheres, width = N > 16 ? 32 : N > 8 ? 16 : 8, sub = lane / width, stride = 32 / width;
+    const int j = lane % width;
+    const bool has = j < N;
+    const float4 sp = has ? s_sph[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 acc[4] = {};
+#pragma unroll 1
+    for (int t = 0; t < kWarpRows; t += stride) {
+        const int r = t + sub;
+        float2 q[kRowUsed + 1], d[4];
+        load_row(rows + r * (kRow / 2), q);
+        pair_backward2<CULL>(sp, q, d, nrm[CULL ? r : 0]);
+        if (!has) d[0] = d[1] = d[2] = d[3] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[e] = __fadd2_rn(acc[e], d[e]);
+        if (a.d_points) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+                for (int o = 1; o < width; o <<= 1) {
+                    d[e].x += __shfl_xor_sync(0xffffffffu, d[e].x, o);
+                    d[e].y += __shfl_xor_sync(0xffffffffu, d[e].y, o);
+                }
+            // six lanes of the sub-group write the row's two points
+            const int64_t p = p0 + 2 * r + j / 3;
+            if (j < 6 && p < a.n_points) {
+                const float2 v = j % 3 == 0 ? d[0] : j % 3 == 1 ? d[1] : d[2];
+                a.d_points[3 * p + j % 3] = -(j < 3 ? v.x : v.y);
+            }
+        }
+    }
+    float s[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        s[e] = acc[e].x + acc[e].y;
+        for (int o = width; o < 32; o <<= 1) s[e] += __shfl_xor_sync(0xffffffffu, s[e], o);
+    }
+    if (has && sub == 0) {
+        float4 v = acc_row[j];
+        v.x += s[0];
+        v.y += s[1];
+        v.z += s[2];
+        v.w += s[3];
+        acc_row[j] = v;
+    }
+    __syncwarp();
 }
 
 // Adjoint of one 128-point tile of one request: per-point outputs are written,
@@ -438,8 +556,8 @@ __device__ __forceinline__ float warp_sum4(float v0, float v1, float v2, float v
 // scene's exp_mode read per call (2).
 template <int CULLM = 2, int EXPM = 2>
 __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_sph, const float* s_light,
-                                              float* s_acc, float (*s_dl)[3 * K + 1], int64_t tile,
-                                              int lane, int warp) {
+                                              float* s_acc, float (*s_dl)[3 * K + 1], float4* s_rows,
+                                              float2 (*s_nrm)[3], int64_t tile, int lane, int warp) {
     const int N = a.sc.n_spheres;
     const int64_t P = a.n_points;
     const int64_t p = tile * kBlock + threadIdx.x;
@@ -511,7 +629,7 @@ __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_
     cosine_lobe(load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
                 load_or(a.normals, 3 * q + 2, live), H, ux, uy, uz, il);
     float W[K];
-    SH::mul(V, H, W);
+    SH::mul_lobe(V, H, W);
 
     // ---- shading adjoint: B_c = a_c L_c . W
     float dB[3], alb[3], loss = 0.f;
@@ -556,8 +674,8 @@ __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_
         if (lane == 0) s_dl[warp][3 * K] += v;
     }
     float dV[K], dH[K];
-    SH::mul(dW, H, dV);                     // C is symmetric: adjoint of a*b is d*b
-    SH::mul(dW, V, dH);
+    SH::mul_lobe(dW, H, dV);                // C is symmetric: adjoint of a*b is d*b
+    SH::mul_onto_lobe(dW, V, dH);           // the normal adjoint scales the other bands by zero
 
     // ---- normal adjoint through H = A_hat_l NORM_i Ybar_i(n / |n|)
     if (live && a.d_normals) {
@@ -604,70 +722,44 @@ __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_
 #pragma unroll
     for (int i = 0; i < K; ++i) dfp[i] *= a.sc.neg_2pi_eps * SH::norm(i);
 
-    // ---- pair adjoints
-    const bool want_sph = a.d_centers || a.d_radii;
-    if (want_sph || a.d_points) {
-        float gq[SH::NG];
+    // ---- pair adjoints: the warp's points go through shared memory, two per
+    // row; the warp reads only its own rows
+    if (!(a.d_centers || a.d_radii || a.d_points) || N == 0) {
+        if (live && a.d_points)
+            for (int c = 0; c < 3; ++c) a.d_points[3 * q + c] = 0.f;
+        return;
+    }
+    __syncwarp();   // the previous tile's rows have been read
+    float* row = reinterpret_cast<float*>(s_rows + warp * (kWarpRows * kRow / 2)) + (lane >> 1) * (2 * kRow) + (lane & 1);
+    row[0] = px;
+    row[2] = py;
+    row[4] = pz;
+    row[6] = dfp[0];
+    {
+        float gq[SH::NG > 0 ? SH::NG : 1];
         SH::grad_coeffs(dfp, gq);
-        const float q0 = dfp[0];
-        const Normal u{ux, uy, uz};
-        float gpx = 0.f, gpy = 0.f, gpz = 0.f;
-        float* my_acc = s_acc + warp * 4 * N;
-        // the pair loops, instantiated with and without horizon culling so the
-        // selection costs nothing per pair when it is off
-        auto loops = [&](auto cull_tag) {
-            constexpr bool CULL = decltype(cull_tag)::value;
-            auto pair = [&](float4 sp, float& gcx, float& gcy, float& gcz, float& gr) {
-                pair_backward_grad<CULL>(px, py, pz, sp, gq, q0, gcx, gcy, gcz, gr, u);
-            };
-            if (want_sph && N >= 32) {
-                // Skewed order: at step t lane l handles sphere (l + t) mod N, so the
-                // 32 lanes update 32 distinct slots of the warp's accumulator row
-                // with plain shared-memory read-modify-writes (no cross-lane sums).
-                float4* row = reinterpret_cast<float4*>(my_acc);
-                int j = lane;
-#pragma unroll 1
-                for (int t = 0; t < N; ++t) {
-                    float gcx, gcy, gcz, gr;
-                    pair(s_sph[j], gcx, gcy, gcz, gr);
-                    gpx -= gcx;
-                    gpy -= gcy;
-                    gpz -= gcz;
-                    float4 acc = row[j];
-                    acc.x += gcx;
-                    acc.y += gcy;
-                    acc.z += gcz;
-                    acc.w += gr;
-                    row[j] = acc;
-                    __syncwarp();
-                    j = (j + 1 == N) ? 0 : j + 1;
-                }
-            } else {
-#pragma unroll 1
-                for (int j = 0; j < N; ++j) {
-                    float gcx, gcy, gcz, gr;
-                    pair(s_sph[j], gcx, gcy, gcz, gr);
-                    gpx -= gcx;
-                    gpy -= gcy;
-                    gpz -= gcz;
-                    if (want_sph) {
-                        const float v = warp_sum4(gcx, gcy, gcz, gr, lane);
-                        if ((lane & 7) == 0) my_acc[4 * j + (lane >> 3)] += v;
-                    }
-                }
-            }
-        };
-        if constexpr (CULLM == 2) {
-            if (a.sc.horizon_cull) loops(std::true_type{});
-            else loops(std::false_type{});
-        } else {
-            loops(std::integral_constant<bool, CULLM == 1>{});
-        }
-        if (live && a.d_points) {
-            a.d_points[3 * q] = gpx;
-            a.d_points[3 * q + 1] = gpy;
-            a.d_points[3 * q + 2] = gpz;
-        }
+#pragma unroll
+        for (int o = 0; o < SH::NG; ++o) row[8 + 2 * o] = gq[o];
+    }
+    float* nr = reinterpret_cast<float*>(&s_nrm[warp * kWarpRows + (lane >> 1)][0]) + (lane & 1);
+    nr[0] = ux;
+    nr[2] = uy;
+    nr[4] = uz;
+    __syncwarp();
+    const float4* rows = s_rows + warp * (kWarpRows * kRow / 2);
+    const float2(*nrm)[3] = s_nrm + warp * kWarpRows;
+    float4* acc_row = reinterpret_cast<float4*>(s_acc) + warp * N;
+    auto loops = [&](auto cull_tag) {
+        constexpr bool CULL = decltype(cull_tag)::value;
+        const int64_t p0 = tile * kBlock + warp * 32;
+        if (N >= 32) warp_pairs<CULL>(a, s_sph, rows, nrm, acc_row, p0, lane);
+        else warp_pairs_few<CULL>(a, s_sph, rows, nrm, acc_row, p0, lane);
+    };
+    if constexpr (CULLM == 2) {
+        if (a.sc.horizon_cull) loops(std::true_type{});
+        else loops(std::false_type{});
+    } else {
+        loops(std::integral_constant<bool, CULLM == 1>{});
     }
 }
 
@@ -683,6 +775,8 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? SHS_BWD_MINB : 1) backward_k
     __shared__ __align__(16) float s_light[3 * KPAD];
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ float s_dl[NWARP][3 * K + 1];
+    __shared__ __align__(16) float4 s_rows[NWARP * kWarpRows * kRow / 2];
+    __shared__ __align__(8) float2 s_nrm[NWARP * kWarpRows][3];
     __shared__ bool s_last;
     const int N = a.sc.n_spheres;
     float4* s_sph = dyn;                  // [N]
@@ -696,7 +790,7 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? SHS_BWD_MINB : 1) backward_k
 
     const int64_t ntiles = (a.n_points + kBlock - 1) / kBlock;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-        backward_tile<CULLM, EXPM>(a, s_sph, s_light, s_acc, s_dl, tile, lane, warp);
+        backward_tile<CULLM, EXPM>(a, s_sph, s_light, s_acc, s_dl, s_rows, s_nrm, tile, lane, warp);
 
     // ---- block reduction, then one scene-level reduction
     __syncthreads();
@@ -768,6 +862,8 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? 4 : 1)
     __shared__ __align__(16) float s_light[3 * KPAD];
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ float s_dl[NWARP][3 * K + 1];
+    __shared__ __align__(16) float4 s_rows[NWARP * kWarpRows * kRow / 2];
+    __shared__ __align__(8) float2 s_nrm[NWARP * kWarpRows][3];
     __shared__ bool s_last;
     __shared__ long long s_tile;
     float4* s_sph = dyn;                                        // [max N]
@@ -793,7 +889,7 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? 4 : 1)
         for (int e = threadIdx.x; e < NWARP * 4 * N; e += kBlock) s_acc[e] = 0.f;
         for (int e = threadIdx.x; e < NWARP * (3 * K + 1); e += kBlock) (&s_dl[0][0])[e] = 0.f;
         __syncthreads();
-        backward_tile(a, s_sph, s_light, s_acc, s_dl, tile - b.tile_begin[r], lane, warp);
+        backward_tile(a, s_sph, s_light, s_acc, s_dl, s_rows, s_nrm, tile - b.tile_begin[r], lane, warp);
         __syncthreads();
         const int E = 3 * K + 1 + 4 * N;
         for (int e = threadIdx.x; e < E; e += kBlock) {

@@ -140,6 +140,63 @@ __device__ __forceinline__ PairGeom pair_geometry(float px, float py, float pz, 
     return g;
 }
 
+// The same for one sphere and two points, one per half of every float2, in the
+// packed float32x2 instructions (identical arithmetic per half).  ic = 1 / c.
+struct PairGeom2 {
+    float2 dx, dy, dz, invD, invD2, s2, c, ic;
+    bool open0, open1;
+};
+
+template <bool CULL>
+__device__ __forceinline__ PairGeom2 pair_geometry2(float2 px, float2 py, float2 pz, float4 sp, const float2* u) {
+    const float2 one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f);
+    PairGeom2 g;
+    g.dx = make_float2(sp.x - px.x, sp.x - px.y);
+    g.dy = make_float2(sp.y - py.x, sp.y - py.y);
+    g.dz = make_float2(sp.z - pz.x, sp.z - pz.y);
+    const float2 D2 = __ffma2_rn(g.dx, g.dx, __ffma2_rn(g.dy, g.dy, __fmul2_rn(g.dz, g.dz)));
+    g.invD = make_float2(D2.x > 0.f ? rsqrtf(D2.x) : 0.f, D2.y > 0.f ? rsqrtf(D2.y) : 0.f);
+    g.invD2 = __fmul2_rn(g.invD, g.invD);
+    const float r2 = sp.w * sp.w;
+    const float2 r2i = __fmul2_rn(make_float2(r2, r2), g.invD2);
+    g.open0 = r2i.x < 1.f;
+    g.open1 = r2i.y < 1.f;
+    g.s2 = make_float2(fminf(r2i.x, 1.f), fminf(r2i.y, 1.f));
+    const float2 om = __ffma2_rn(g.s2, mone, one);
+    g.ic = make_float2(rsqrtf(fmaxf(om.x, 1e-30f)), rsqrtf(fmaxf(om.y, 1e-30f)));
+    g.c = __fmul2_rn(om, g.ic);
+    if constexpr (CULL) {   // u: the points' unit normals
+        const float2 h = __ffma2_rn(g.dx, u[0], __ffma2_rn(g.dy, u[1], __fmul2_rn(g.dz, u[2])));
+        if (h.x < -sp.w) {
+            g.s2.x = 0.f;
+            g.c.x = 1.f;
+            g.open0 = false;
+        }
+        if (h.y < -sp.w) {
+            g.s2.y = 0.f;
+            g.c.y = 1.f;
+            g.open1 = false;
+        }
+    }
+    return g;
+}
+
+// dPsi/dd and dPsi/dr of two pairs from s_hat, s_hat's gradient a (its radial
+// part is removed here) and ga = -dPsi/dc.
+__device__ __forceinline__ void pair_finish2(const PairGeom2& g, float r, float2 sx, float2 sy, float2 sz, float2 ax,
+                                             float2 ay, float2 az, float2 ga, float2* d) {
+    const float2 mone = make_float2(-1.f, -1.f);
+    // c = sqrt(1 - s2): d c / d s2 = -1 / (2 c); clamped caps carry no gradient
+    const float2 h = __fmul2_rn(ga, g.ic);
+    const float2 t = __fmul2_rn(make_float2(g.open0 ? h.x : 0.f, g.open1 ? h.y : 0.f), g.invD2);   // 2 dPsi/ds2 / D^2
+    const float2 coef = __fmul2_rn(__fmul2_rn(t, mone), g.s2);                                     // 2 dPsi/dD^2
+    const float2 nrad = __fmul2_rn(mone, __ffma2_rn(sx, ax, __ffma2_rn(sy, ay, __fmul2_rn(sz, az))));
+    d[0] = __ffma2_rn(__ffma2_rn(nrad, sx, ax), g.invD, __fmul2_rn(coef, g.dx));
+    d[1] = __ffma2_rn(__ffma2_rn(nrad, sy, ay), g.invD, __fmul2_rn(coef, g.dy));
+    d[2] = __ffma2_rn(__ffma2_rn(nrad, sz, az), g.invD, __fmul2_rn(coef, g.dz));
+    d[3] = __fmul2_rn(t, make_float2(r, r));                                                       // s2 = r^2 / D^2
+}
+
 __device__ __forceinline__ float load_or(const float* p, int64_t i, bool live) {
     return live ? __ldg(p + i) : 0.f;
 }

@@ -1,7 +1,7 @@
-"""Kernels of 6 to 8 bands (a lane pair per point, one sphere per lane in the
-pair adjoint) at the edges of their tiles: 64-point tiles, 16 points per warp,
-8 / 16 / 32 spheres per warp step; every variant of the batched kernels against
-the single calls."""
+"""The adjoint kernels at the edges of their tiles: 6 to 8 bands (a lane pair
+per point, 64-point tiles, 16 points per warp, 8 / 16 / 32 spheres per warp
+step) and 1 to 5 bands; every variant of the batched kernels of 6 and more
+bands against the single calls."""
 
 import ctypes
 
@@ -41,6 +41,15 @@ def test_tile_edges(n, points, spheres):
         for name in ("d_light", "d_centers", "d_radii"):
             err = grad_err(name, g[name], ref)
             assert err.max() <= _tol(n), f"{name}: {err.max():.3e}"
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("points,spheres", [(1, 1), (31, 8), (32, 9), (33, 17), (127, 31), (129, 32), (65, 33),
+                                            (97, 64), (128, 71)])
+def test_tile_edges_low_bands(n, points, spheres):
+    """1 to 5 bands: two points per row of the pair adjoint, a lane pair per row
+    from 32 spheres on, spheres on the lanes below."""
+    test_tile_edges(n, points, spheres)
 
 
 @pytest.mark.parametrize("n", [6, 8])
