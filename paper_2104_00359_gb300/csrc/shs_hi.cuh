@@ -18,20 +18,6 @@ constexpr int kTile = tile_points(NB);        // points per block tile
 constexpr int kWarpPoints = kTile / NWARP;    // points per warp
 static_assert(kTile * 2 == kBlock && kWarpPoints == 16, "a lane pair per point");
 
-// Legendre P_l(c) and P_l'(c) for l < NB (Bonnet recurrence and
-// P'_{l+1} = P'_{l-1} + (2l+1) P_l).
-__device__ __forceinline__ void legendre(float c, float* P, float* dP) {
-    P[0] = 1.f;
-    P[1] = c;
-    dP[0] = 0.f;
-    dP[1] = 1.f;
-#pragma unroll
-    for (int l = 1; l + 1 < NB; ++l) {
-        P[l + 1] = fmaf((2.f * l + 1.f) / (l + 1.f) * c, P[l], -(float(l) / (l + 1.f)) * P[l - 1]);
-        dP[l + 1] = fmaf(2.f * l + 1.f, P[l], dP[l - 1]);
-    }
-}
-
 // One pair's log-visibility terms in the lanes' column form, added to acc:
 // acc[m, i] += s2 P_l'(c) R_lm(s_hat) (C_m, S_m), l = m + i (l = 0: 1 - c); the
 // factors 1 / (l (l + 1)), (2l - 1)!!, NORM and -2 pi eps follow once per

@@ -20,98 +20,126 @@ namespace {
 // pair adjoint
 // ---------------------------------------------------------------------------
 
-// A point's adjoint coefficients in shared memory: column m holds
+// Two points' adjoint coefficients in shared memory, one row per pair of
+// points and one point per half of every float2: x, y, z, then (horizon culling)
+// the unit normals, then for column m
 // w_lm = dLoss/df_lm (-2 pi eps) NORM_lm (2l - 1)!! / (l (l + 1)) for l = m ..
-// NB - 1 (l = 0: without the division), for m > 0 as (cos, sin) pairs; columns start
-// at multiples of four floats.
+// NB - 1 (l = 0: without the division), for m > 0 as (cos, sin) pairs; columns
+// start at multiples of two entries (16 bytes).
 __host__ __device__ constexpr int wcol(int m) {
-    int b = 0;
-    for (int k = 0; k < m; ++k) b += ((k ? 2 : 1) * (NB - k) + 3) / 4 * 4;
+    int b = 6;
+    for (int k = 0; k < m; ++k) b += ((k ? 2 : 1) * (NB - k) + 1) / 2 * 2;
     return b;
 }
-constexpr int WST = wcol(NB) + 4;
-constexpr int kWarpRegion = kWarpPoints * WST > 64 * NS ? kWarpPoints * WST : 64 * NS;   // floats
+constexpr int kWarpRows = kWarpPoints / 2;
+constexpr int WST = wcol(NB) + 2;   // entries per row
+constexpr int kRowFloats = kWarpRows * 2 * WST;
+constexpr int kWarpRegion = kRowFloats > 64 * NS ? kRowFloats : 64 * NS;   // floats
 
-// Adjoint of one pair's Psi = sum_l G_l(c) Phi_l(s_hat), Phi_l = sum_m w_lm
-// Ybar_lm: the gradients with respect to the sphere's centre (the point gets
-// the negative) and radius.  Per order m, with R_lm and d/dz R_lm = R_l,m+1:
+// Adjoint of two pairs (one sphere, two points) Psi = sum_l G_l(c)
+// Phi_l(s_hat), Phi_l = sum_m w_lm Ybar_lm: the gradients with respect to the
+// sphere's centre (the points get the negatives) and radius.  Per order m, with
+// R_lm and d/dz R_lm = R_l,m+1:
 //   alpha = sum_l P_l' R_lm w_lm           -> d/dx, d/dy of C_m + i S_m
 //   beta  = sum_l P_l' R_l,m+1 w_lm        -> d/dz
 //   gamma = sum_l l (l + 1) P_l R_lm w_lm  -> -dPsi/dc
 // (the factor s2 of G_l is applied at the end).  The products P_l' R_l,m+1 of
 // one order are the next order's P_l' R_lm.  At 8 bands about 440 FP32
-// instructions a pair, where the evaluation and reverse sweep of all 64
-// harmonics took about 800.
-template <bool CULL>
-__device__ __forceinline__ void pair_backward(float px, float py, float pz, float4 sp, const float* w, float& gcx,
-                                              float& gcy, float& gcz, float& gr, Normal u) {
-    const PairGeom g = pair_geometry<CULL>(px, py, pz, sp, u);
-    float P[NB], dP[NB];
-    legendre(g.c, P, dP);
+// operations a pair, where the evaluation and reverse sweep of all 64
+// harmonics took about 800.  Packed, because a scalar multiply-add with three
+// different registers issues at 70 - 110 of 128 lanes a clock on this chip
+// (register ports), a packed one at 120.
+__device__ __forceinline__ float2 k2(float v) { return make_float2(v, v); }
+
+template <int M>
+__device__ __forceinline__ void sh_column2(const float2* zi, float2* col) {
+    if constexpr (M < NB) {
+        col[0] = k2(1.f);
+        if constexpr (M + 1 < NB) col[1] = zi[0];
 #pragma unroll
-    for (int l = 1; l < NB; ++l) P[l] *= float(l * (l + 1));
-    const float sx = g.dx * g.invD, sy = g.dy * g.invD, sz = g.dz * g.invD;
-    float zi[NB], col[NB], nxt[NB], e[NB], C = 1.f, S = 0.f;
-    float gx = 0.f, gy = 0.f, gz = 0.f, ga = 0.f;
-    sh_column_factors(sz, zi);
-    sh_column<0>(zi, col);
-    static_for<NB>([&](auto mm) {
-        constexpr int m = mm;
-        float wm[((m ? 2 : 1) * (NB - m) + 3) / 4 * 4];
-        const float4* w4 = reinterpret_cast<const float4*>(w + wcol(m));
-#pragma unroll
-        for (int i = 0; i < ((m ? 2 : 1) * (NB - m) + 3) / 4; ++i) {
-            const float4 v = w4[i];
-            wm[4 * i] = v.x;
-            wm[4 * i + 1] = v.y;
-            wm[4 * i + 2] = v.z;
-            wm[4 * i + 3] = v.w;
+        for (int i = 1; i + 1 < NB - M; ++i) {
+            const int l = M + i;
+            col[i + 1] = __ffma2_rn(zi[i], col[i],
+                                    __fmul2_rn(k2(-(float(l + M) / float((4 * l * l - 1) * (i + 1)))), col[i - 1]));
         }
-        sh_column<m + 1>(zi, nxt);
-        float ac = 0.f, as = 0.f, bc = 0.f, bs = 0.f, cc = 0.f, cs = 0.f;
+    }
+}
+
+template <bool CULL>
+__device__ __forceinline__ void pair_backward2(float4 sp, const float2* row, float2* d) {
+    const PairGeom2 g = pair_geometry2<CULL>(row[0], row[1], row[2], sp, row + 3);
+    float2 P[NB], dP[NB];   // P_l (times l (l + 1) below) and P_l'
+    P[0] = k2(1.f);
+    P[1] = g.c;
+    dP[1] = k2(1.f);
+#pragma unroll
+    for (int l = 1; l + 1 < NB; ++l) {
+        P[l + 1] = __ffma2_rn(__fmul2_rn(k2((2.f * l + 1.f) / (l + 1.f)), g.c), P[l],
+                              __fmul2_rn(k2(-(float(l) / (l + 1.f))), P[l - 1]));
+        dP[l + 1] = l == 1 ? __fmul2_rn(k2(3.f), P[1]) : __ffma2_rn(k2(2.f * l + 1.f), P[l], dP[l - 1]);
+    }
+#pragma unroll
+    for (int l = 1; l < NB; ++l) P[l] = __fmul2_rn(P[l], k2(float(l * (l + 1))));
+    const float2 sx = __fmul2_rn(g.dx, g.invD), sy = __fmul2_rn(g.dy, g.invD), sz = __fmul2_rn(g.dz, g.invD);
+    const float2 nsy = __fmul2_rn(sy, k2(-1.f));
+    float2 zi[NB], col[NB], nxt[NB], e[NB], C = k2(1.f), S = k2(0.f);
+    float2 gx = k2(0.f), gy = k2(0.f), gz = k2(0.f), ga = k2(0.f);
+#pragma unroll
+    for (int i = 0; i + 1 < NB; ++i) zi[i] = __fmul2_rn(sz, k2(1.f / float(i + 1)));
+    sh_column2<0>(zi, col);
+    static_for<NB>([&](auto mm) {
+        constexpr int m = mm, n = (m ? 2 : 1) * (NB - m);
+        float2 wm[(n + 1) / 2 * 2];
+        const float4* w4 = reinterpret_cast<const float4*>(row + wcol(m));
+#pragma unroll
+        for (int i = 0; i < (n + 1) / 2; ++i) {
+            const float4 v = w4[i];
+            wm[2 * i] = make_float2(v.x, v.y);
+            wm[2 * i + 1] = make_float2(v.z, v.w);
+        }
+        sh_column2<m + 1>(zi, nxt);
+        float2 ac{}, as{}, bc{}, bs{}, cc{}, cs{};
 #pragma unroll
         for (int i = 0; i < NB - m; ++i) {   // l = m + i
-            const float h = P[m + i] * col[i];
-            const float wc = wm[m ? 2 * i : i], ws = wm[m ? 2 * i + 1 : 0];
-            cc = fmaf(h, wc, cc);
+            const float2 h = i ? __fmul2_rn(P[m + i], col[i]) : P[m];
+            const float2 wc = wm[m ? 2 * i : i], ws = wm[m ? 2 * i + 1 : 0];
+            cc = i ? __ffma2_rn(h, wc, cc) : __fmul2_rn(h, wc);
             if (m) {
-                ac = fmaf(e[i], wc, ac);
-                as = fmaf(e[i], ws, as);
-                cs = fmaf(h, ws, cs);
+                ac = i ? __ffma2_rn(e[i], wc, ac) : __fmul2_rn(e[i], wc);
+                as = i ? __ffma2_rn(e[i], ws, as) : __fmul2_rn(e[i], ws);
+                cs = i ? __ffma2_rn(h, ws, cs) : __fmul2_rn(h, ws);
             }
             if (i) {
-                e[i - 1] = dP[m + i] * nxt[i - 1];
-                bc = fmaf(e[i - 1], wc, bc);
-                if (m) bs = fmaf(e[i - 1], ws, bs);
+                e[i - 1] = i == 1 ? dP[m + i] : __fmul2_rn(dP[m + i], nxt[i - 1]);
+                bc = i > 1 ? __ffma2_rn(e[i - 1], wc, bc) : __fmul2_rn(e[i - 1], wc);
+                if (m) bs = i > 1 ? __ffma2_rn(e[i - 1], ws, bs) : __fmul2_rn(e[i - 1], ws);
             }
         }
-        if (m) {
-            const float fm = static_cast<float>(m);   // C, S still hold order m - 1
-            gx = fmaf(fm, fmaf(ac, C, as * S), gx);
-            gy = fmaf(fm, fmaf(as, C, -(ac * S)), gy);
-            const float c1 = fmaf(sx, C, -(sy * S)), s1 = fmaf(sx, S, sy * C);
-            C = c1;
-            S = s1;
-            gz = fmaf(bc, C, fmaf(bs, S, gz));
-            ga = fmaf(cc, C, fmaf(cs, S, ga));
-        } else {
+        if constexpr (m == 0) {
             gz = bc;
             ga = cc;
+        } else {
+            // C, S still hold order m - 1
+            if constexpr (m == 1) {
+                gx = ac;
+                gy = as;
+                C = sx;
+                S = sy;
+            } else {
+                const float2 fc = __fmul2_rn(k2(float(m)), C), fs = __fmul2_rn(k2(float(m)), S);
+                gx = __ffma2_rn(ac, fc, __ffma2_rn(as, fs, gx));
+                gy = __ffma2_rn(as, fc, __ffma2_rn(__fmul2_rn(ac, k2(-1.f)), fs, gy));
+                const float2 c1 = __ffma2_rn(sx, C, __fmul2_rn(nsy, S)), s1 = __ffma2_rn(sx, S, __fmul2_rn(sy, C));
+                C = c1;
+                S = s1;
+            }
+            if constexpr (m + 1 < NB) gz = __ffma2_rn(bc, C, __ffma2_rn(bs, S, gz));
+            ga = __ffma2_rn(cc, C, __ffma2_rn(cs, S, ga));
         }
 #pragma unroll
         for (int i = 0; i + 1 < NB - m; ++i) col[i] = nxt[i];
     });
-    gx *= g.s2;
-    gy *= g.s2;
-    gz *= g.s2;
-    // dPsi/dc = -ga; c = sqrt(1 - s2): d c / d s2 = -1 / (2 c); clamped caps carry no gradient
-    const float ds2 = g.open ? __fdividef(0.5f * ga, g.c) : 0.f;
-    gr = ds2 * 2.f * sp.w * g.invD2;                 // s2 = r^2 / D^2
-    const float dD2 = -ds2 * g.s2 * g.invD2;
-    const float sg = sx * gx + sy * gy + sz * gz;    // s_hat = d / D: tangential part
-    gcx = fmaf(gx - sx * sg, g.invD, 2.f * dD2 * g.dx);
-    gcy = fmaf(gy - sy * sg, g.invD, 2.f * dD2 * g.dy);
-    gcz = fmaf(gz - sz * sg, g.invD, 2.f * dD2 * g.dz);
+    pair_finish2(g, sp.w, sx, sy, sz, __fmul2_rn(gx, g.s2), __fmul2_rn(gy, g.s2), __fmul2_rn(gz, g.s2), ga, d);
 }
 
 // ---------------------------------------------------------------------------
@@ -127,10 +155,8 @@ struct BwdShared {
     const float* leg;
     float (*dl)[2][kDl];         // [NWARP]
     float* loss;                 // [NWARP]
-    float* w;                    // per warp: the operands of its products, then its points' rows [16][WST]
+    float* w;                    // per warp: the operands of its products, then its points' rows
     int region;                  // floats of w per warp
-    float4* pt;                  // [kTile]
-    float4* nrm;                 // [kTile] (horizon culling)
 };
 
 // Adjoint of the exponential and the shading at the lane pair's point: the
@@ -321,73 +347,65 @@ __device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShare
     });
 }
 
-// The lane's coefficients into its point's row of shared memory.
-__device__ __forceinline__ void lp_store_row(const float* dfp, float* row, const LanePair& lp) {
+// The lane's coefficients into its half of its points' row of shared memory
+// (half: a float pointer to the row's entry 0, first or second point).
+__device__ __forceinline__ void lp_store_row(const float* dfp, float* half, const LanePair& lp) {
     static_for<NS>([&](auto s) {
         constexpr int m = lp_m(s), l0 = lp_l(s, 0), l1 = lp_l(s, 1), sn = lp_sin(s);
         constexpr int o0 = wcol(m) + (m ? 2 * (l0 - m) + sn : l0), o1 = wcol(m) + (m ? 2 * (l1 - m) + sn : l1);
         constexpr float c0 = dfact(l0) / float(l0 ? l0 * (l0 + 1) : 1), c1 = dfact(l1) / float(l1 * (l1 + 1));
-        if (l1 < NB || !lp.odd) row[lp.odd ? o1 : o0] = dfp[s] * (lp.odd ? c1 : c0);
+        if (l1 < NB || !lp.odd) half[2 * (lp.odd ? o1 : o0)] = dfp[s] * (lp.odd ? c1 : c0);
     });
 }
 
-// Pair adjoints of the warp's 16 points, one sphere per lane; with fewer than
-// 17 (9) spheres the lanes take two (four) points at once.
+// Pair adjoints of the warp's 16 points (eight rows of two), one sphere per
+// lane; with fewer than 17 (9) spheres the lanes take two (four) rows at once.
 template <bool CULL>
 __device__ __forceinline__ void lp_pairs(const BwdArgs& a, const BwdShared& sh, int64_t tile) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = a.sc.n_spheres;
     const int width = N > 16 ? 32 : N > 8 ? 16 : 8, sub = lane / width, stride = 32 / width;
     float4* acc_row = sh.acc + warp * N;
-    const float* rows = sh.w + warp * sh.region;
+    const float2* rows = reinterpret_cast<const float2*>(sh.w + warp * sh.region);
     const bool want_pts = a.d_points != nullptr;
     float gp[3] = {0.f, 0.f, 0.f};   // lane t < 16: gradient of the warp's point t
     for (int j0 = 0; j0 < N; j0 += width) {
         const int j = j0 + lane % width;
         const bool has = j < N;
         const float4 sp = has ? sh.sph[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float2 acc[4] = {};
 #pragma unroll 1
-        for (int t = 0; t < kWarpPoints; t += stride) {
-            const int r = warp * kWarpPoints + t + sub;
-            const float4 pt = sh.pt[r];
-            Normal u{};
-            if (CULL) u = Normal{sh.nrm[r].x, sh.nrm[r].y, sh.nrm[r].z};
-            float gcx, gcy, gcz, gr;
-            pair_backward<CULL>(pt.x, pt.y, pt.z, sp, rows + (r - warp * kWarpPoints) * WST, gcx, gcy, gcz, gr, u);
-            if (!has) gcx = gcy = gcz = gr = 0.f;
-            acc.x += gcx;
-            acc.y += gcy;
-            acc.z += gcz;
-            acc.w += gr;
+        for (int t = 0; t < kWarpRows; t += stride) {
+            float2 d[4];
+            pair_backward2<CULL>(sp, rows + (t + sub) * WST, d);
+            if (!has) d[0] = d[1] = d[2] = d[3] = k2(0.f);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[e] = __fadd2_rn(acc[e], d[e]);
             if (want_pts) {
-                for (int o = 1; o < width; o <<= 1) {
-                    gcx += __shfl_xor_sync(0xffffffffu, gcx, o);
-                    gcy += __shfl_xor_sync(0xffffffffu, gcy, o);
-                    gcz += __shfl_xor_sync(0xffffffffu, gcz, o);
-                }
-                // lane t + i takes the sum its sub-group i holds
-                const int src = ((lane - t) & (stride - 1)) * width;
-                const float x = __shfl_sync(0xffffffffu, gcx, src), y = __shfl_sync(0xffffffffu, gcy, src),
-                            z = __shfl_sync(0xffffffffu, gcz, src);
-                if (lane >= t && lane < t + stride) {
-                    gp[0] -= x;
-                    gp[1] -= y;
-                    gp[2] -= z;
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    for (int o = 1; o < width; o <<= 1) {
+                        d[e].x += __shfl_xor_sync(0xffffffffu, d[e].x, o);
+                        d[e].y += __shfl_xor_sync(0xffffffffu, d[e].y, o);
+                    }
+                    // lane 2 (t + i) + h takes half h of the sum its sub-group i holds
+                    const int src = (((lane >> 1) - t) & (stride - 1)) * width;
+                    const float x = __shfl_sync(0xffffffffu, d[e].x, src), y = __shfl_sync(0xffffffffu, d[e].y, src);
+                    if ((lane >> 1) >= t && (lane >> 1) < t + stride) gp[e] -= lane & 1 ? y : x;
                 }
             }
         }
-        for (int o = width; o < 32; o <<= 1) {
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-            acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
-            acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+        float s[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            s[e] = acc[e].x + acc[e].y;
+            for (int o = width; o < 32; o <<= 1) s[e] += __shfl_xor_sync(0xffffffffu, s[e], o);
         }
         if (has && sub == 0) {
             float4 v = acc_row[j];
-            v.x += acc.x;
-            v.y += acc.y;
-            v.z += acc.z;
-            v.w += acc.w;
+            v.x += s[0];
+            v.y += s[1];
+            v.z += s[2];
+            v.w += s[3];
             acc_row[j] = v;
         }
     }
@@ -427,16 +445,18 @@ __device__ __forceinline__ void lp_backward_tile(const BwdArgs& a, const BwdShar
     }
     if (!pairs) return;
     __syncwarp();   // the region held the tail's operands
-    lp_store_row(dfp, sh.w + (row >> 4) * sh.region + (row & 15) * WST, lp);
+    float* half = sh.w + (row >> 4) * sh.region + ((row & 15) >> 1) * (2 * WST) + (row & 1);
+    lp_store_row(dfp, half, lp);
+    const int64_t q = live ? p : 0;
     if (!lp.odd) {
-        const int64_t q = live ? p : 0;
-        sh.pt[row] = make_float4(load_or(a.points, 3 * q, live), load_or(a.points, 3 * q + 1, live),
-                                 load_or(a.points, 3 * q + 2, live), 0.f);
-        if (CULL) {
-            const Normal u = unit_normal(load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
-                                         load_or(a.normals, 3 * q + 2, live));
-            sh.nrm[row] = make_float4(u.x, u.y, u.z, 0.f);
-        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) half[2 * c] = load_or(a.points, 3 * q + c, live);
+    } else if (CULL) {
+        const Normal u = unit_normal(load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
+                                     load_or(a.normals, 3 * q + 2, live));
+        half[6] = u.x;
+        half[8] = u.y;
+        half[10] = u.z;
     }
     __syncwarp();
     lp_pairs<CULL>(a, sh, tile);
@@ -471,8 +491,7 @@ __device__ __forceinline__ float lp_block_sum(const BwdShared& sh, int N, int e)
     __shared__ __align__(16) float s_light[3 * KPAD];                                        \
     __shared__ __align__(16) float s_lt[2][3][NSP];                                          \
     __shared__ __align__(16) float s_leg[kLegProduct + ((EXP) ? kLegExp : 0)];               \
-    __shared__ __align__(16) float s_w[NWARP * ((PHASE) == kPhasePairs ? kWarpPoints * WST : kWarpRegion)];                 \
-    __shared__ __align__(16) float4 s_pt[(PHASE) == kPhaseTail ? 1 : kTile], s_nrm[(PHASE) == kPhaseTail ? 1 : kTile]; \
+    __shared__ __align__(16) float s_w[NWARP * ((PHASE) == kPhasePairs ? kRowFloats : kWarpRegion)];                       \
     __shared__ float s_dl[NWARP][2][kDl], s_loss[NWARP];                                     \
     __shared__ __align__(8) uint64_t s_bar;                                                  \
     __shared__ bool s_last
@@ -492,8 +511,7 @@ template <bool EXP, bool CULL, int PHASE>
 __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_lp_kernel(BwdArgs a) {
     SHS_LP_BWD_SHARED(EXP, PHASE);
     const int N = a.sc.n_spheres;
-    const BwdShared sh{dyn, dyn + N, s_lt, s_leg, s_dl, s_loss, s_w, PHASE == kPhasePairs ? kWarpPoints * WST : kWarpRegion,
-                       s_pt, s_nrm};
+    const BwdShared sh{dyn, dyn + N, s_lt, s_leg, s_dl, s_loss, s_w, PHASE == kPhasePairs ? kRowFloats : kWarpRegion};
     if (PHASE != kPhasePairs) load_rules(s_leg, EXP);
     if (!stage_scene(a.sc, sh.sph, s_light, &s_bar)) return;
     clear_sums(sh, PHASE == kPhaseTail ? 0 : N);
@@ -535,7 +553,7 @@ template <bool EXP, bool CULL>
 __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_batch_kernel(const __grid_constant__ BwdBatch b) {
     SHS_LP_BWD_SHARED(EXP, kPhaseBoth);
     __shared__ long long s_tile;
-    const BwdShared sh{dyn, dyn + b.max_spheres, s_lt, s_leg, s_dl, s_loss, s_w, kWarpRegion, s_pt, s_nrm};
+    const BwdShared sh{dyn, dyn + b.max_spheres, s_lt, s_leg, s_dl, s_loss, s_w, kWarpRegion};
     load_rules(s_leg, EXP);
     mbar_init(&s_bar);
     int staged = -1;
