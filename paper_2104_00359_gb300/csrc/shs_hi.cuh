@@ -166,18 +166,5 @@ __device__ __forceinline__ float lp_norm2(const float* f, const LanePair& lp) {
 #define SHS_LP_MINB 3
 #endif
 
-// Blocks of a persistent kernel one wave holds (at least one per SM).
-template <class Kern>
-cudaError_t one_wave(Kern kernel, size_t smem, int64_t tiles, int* grid) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, smem);
-    if (e != cudaSuccess) return e;
-    const int64_t cap = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
-    *grid = static_cast<int>(tiles < cap ? tiles : cap);
-    return cudaSuccess;
-}
-
 }  // namespace
 }  // namespace shs

@@ -220,7 +220,7 @@ __device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShare
 #pragma unroll 1
     for (int t = 0; t < kmax; ++t) {
         float T[NS];
-        lp_product<true, true, 32>(X, nullptr, legs, lp, T);
+        lp_product<true, false, 32>(X, nullptr, legs, lp, T);
         const bool on = t < k;
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
@@ -635,8 +635,9 @@ cudaError_t launch_backward_batch_lp(const BwdBatch& b, cudaStream_t s) {
         cudaFuncSetAttribute(backward_batch_kernel<EXP, CULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(backward_dyn_smem(kMaxSpheres)));
     if (attr != cudaSuccess) return attr;
+    static WaveCache wave;
     int grid = 0;
-    const cudaError_t e = one_wave(backward_batch_kernel<EXP, CULL>, smem, b.total_tiles, &grid);
+    const cudaError_t e = one_wave(backward_batch_kernel<EXP, CULL>, smem, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
     backward_batch_kernel<EXP, CULL><<<grid, kBlock, smem, s>>>(b);
     count_launch();

@@ -134,8 +134,9 @@ cudaError_t launch_forward_lp(const FwdArgs& a, cudaStream_t s) {
 
 template <bool EXP, bool CULL>
 cudaError_t launch_forward_batch_lp(const FwdBatch& b, cudaStream_t s) {
+    static WaveCache wave;
     int grid = 0;
-    const cudaError_t e = one_wave(forward_batch_kernel<EXP, CULL>, 0, b.total_tiles, &grid);
+    const cudaError_t e = one_wave(forward_batch_kernel<EXP, CULL>, 0, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
     forward_batch_kernel<EXP, CULL><<<grid, kBlock, 0, s>>>(b);
     count_launch();

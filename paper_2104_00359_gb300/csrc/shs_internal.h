@@ -2,6 +2,7 @@
 // kernel translation units (shs_kern.cu compiled once per n_bands).
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -170,6 +171,32 @@ cudaError_t launch_pack_spheres(const float* centers, const float* radii, float4
                                 bool has_c, bool has_r, cudaStream_t s);
 
 void count_launch();
+
+// Blocks one wave of `kernel` holds on the current device at `smem` dynamic
+// bytes; the last answer per device is kept (an occupancy query takes longer
+// than a launch).
+struct WaveCache {
+    std::atomic<uint64_t> slot[64];   // (smem + 1) << 32 | blocks
+};
+template <class Kern>
+cudaError_t one_wave(Kern kernel, size_t smem, int64_t tiles, WaveCache& cache, int* grid) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t key = static_cast<uint64_t>(smem + 1) << 32;
+    uint64_t v = dev < 64 ? cache.slot[dev].load(std::memory_order_relaxed) : 0;
+    if ((v & ~0xffffffffull) != key) {
+        int sms = 0, per_sm = 0;
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, smem);
+        if (e != cudaSuccess) return e;
+        v = key | static_cast<uint32_t>(sms * (per_sm > 0 ? per_sm : 1));
+        if (dev < 64) cache.slot[dev].store(v, std::memory_order_relaxed);
+    }
+    const int64_t cap = static_cast<int64_t>(v & 0xffffffffull);
+    *grid = static_cast<int>(tiles < cap ? tiles : cap);
+    return cudaSuccess;
+}
 
 // Shared by every entry point of the C ABI (defined in shs_api.cu).
 int validate_config(const void* cfg);                    // shs_status of a shs_config*

@@ -933,13 +933,10 @@ BwdBlocks backward_blocks_per_sm<NB>(int n_spheres) {
 template <>
 cudaError_t launch_forward_batch<NB>(const FwdBatch& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, forward_batch_kernel, kBlock, 0);
+    static WaveCache wave;
+    int grid = 0;
+    const cudaError_t e = one_wave(forward_batch_kernel, 0, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
-    const int64_t cap = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
-    const int grid = static_cast<int>(b.total_tiles < cap ? b.total_tiles : cap);
     forward_batch_kernel<<<grid, kBlock, 0, s>>>(b);
     count_launch();
     return cudaGetLastError();
@@ -953,13 +950,10 @@ cudaError_t launch_backward_batch<NB>(const BwdBatch& b, cudaStream_t s) {
         backward_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
         static_cast<int>(backward_dyn_smem(kMaxSpheres)));
     if (attr != cudaSuccess) return attr;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward_batch_kernel, kBlock, smem);
+    static WaveCache wave;
+    int grid = 0;
+    const cudaError_t e = one_wave(backward_batch_kernel, smem, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
-    const int64_t cap = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
-    const int grid = static_cast<int>(b.total_tiles < cap ? b.total_tiles : cap);
     backward_batch_kernel<<<grid, kBlock, smem, s>>>(b);
     count_launch();
     return cudaGetLastError();
