@@ -676,7 +676,7 @@ cudaError_t launch_backward<NB>(const BwdArgs& a, cudaStream_t s) {
     }
     if (err != cudaSuccess || a.counter != nullptr) return err;
     const int E = 3 * K + 1 + 4 * a.sc.n_spheres;
-    reduce_partials_kernel<<<(E + 31) / 32, 32 * kReduceWarps, 0, s>>>(a, a.dfp_ws && a.tail_grid ? a.tail_grid : a.grid,
+    reduce_partials_kernel<<<reduce_blocks(E), kReduceThreads, 0, s>>>(a, a.dfp_ws && a.tail_grid ? a.tail_grid : a.grid,
                                                                        a.grid);
     count_launch();
     return cudaGetLastError();

@@ -1003,7 +1003,7 @@ cudaError_t launch_backward<NB>(const BwdArgs& a, cudaStream_t s) {
     err = cudaGetLastError();
     if (err != cudaSuccess || a.counter != nullptr) return err;
     const int E = 3 * K + 1 + 4 * a.sc.n_spheres;
-    reduce_partials_kernel<<<(E + 31) / 32, 32 * kReduceWarps, 0, s>>>(a, a.grid, a.grid);
+    reduce_partials_kernel<<<reduce_blocks(E), kReduceThreads, 0, s>>>(a, a.grid, a.grid);
     count_launch();
     return cudaGetLastError();
 }
