@@ -70,9 +70,9 @@ def flop_model(n, n_spheres, k_mean):
     return dict(fwd=n_spheres * pf + tf, bwd=n_spheres * pb + tb)
 
 
-KERNEL_SOURCES = ("paper_2104_00359_gb300/csrc/shs_kern.cu", "paper_2104_00359_gb300/csrc/shs_internal.h",
-                  "paper_2104_00359_gb300/csrc/shs_exp.cuh", "paper_2104_00359_gb300/csrc/shs_warp.cuh",
-                  "paper_2104_00359_gb300/csrc/generated/shs_sh_gen.cuh")
+KERNEL_SOURCES = tuple("paper_2104_00359_gb300/csrc/" + f for f in (
+    "shs_kern.cu", "shs_hi_forward.cu", "shs_hi_backward.cu", "shs_hi.cuh", "shs_lanepair.cuh", "shs_point.cuh",
+    "shs_internal.h", "shs_exp.cuh", "shs_warp.cuh", "generated/shs_sh_gen.cuh"))
 
 
 def kernel_source_hash():
@@ -795,9 +795,9 @@ def _fp32_roofline_n8(P, N, k_mean, fwd_ms, bwd_ms, fma_peak):
     fm = flop_model(8, N, k_mean)
     peak = SMS * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
     pts512 = 512 * 512
-    ex_f = profiled_value("flops", "forward_kernel_t", "heightfield512_n8")
-    ex_t = profiled_value("flops", "backward_kernel_t", "heightfield512_n8")
-    ex_p = profiled_value("flops", "bwd_pairs_t_kernel", "heightfield512_n8")
+    ex_f = profiled_value("flops", "forward_lp_kernel", "heightfield512_n8")
+    ex_t = profiled_value("flops", "backward_lp_kernel_tail", "heightfield512_n8")
+    ex_p = profiled_value("flops", "backward_lp_kernel_pairs", "heightfield512_n8")
     ex_f = ex_f / pts512 if ex_f else None
     ex_b = (ex_t + ex_p) / pts512 if (ex_t and ex_p) else None
     wf = min(fm["fwd"], ex_f) if ex_f else fm["fwd"]
