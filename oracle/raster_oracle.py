@@ -155,3 +155,86 @@ def rasterize_backward(vertices, faces, proj, radiance, face_idx, d_image):
                 dclip[ids[k], 3] += dw[k] - (dn[k, 0] * n[k, 0] + dn[k, 1] * n[k, 1]) / w[k]
     d_vertices = dclip @ P[:, :3]
     return dict(d_radiance=dB, d_vertices=d_vertices)
+
+
+# ---------------------------------------------------------------------------
+# float32 restatement of the coverage pass
+# ---------------------------------------------------------------------------
+
+def _fma32(a, b, c):
+    """float32 fused multiply-add: the product is exact in float64; the sum is
+    rounded to odd there, so the final rounding to float32 is the only one."""
+    p = np.asarray(a, np.float64) * np.asarray(b, np.float64)
+    c = np.asarray(c, np.float64)
+    s = p + c
+    t = s - p
+    err = (p - (s - t)) + (c - t)
+    bits = np.atleast_1d(s).view(np.int64).copy()
+    e = np.atleast_1d(err)
+    fix = (e != 0) & (bits & 1 == 0)
+    bits += np.where(fix, np.where((e > 0) == (np.atleast_1d(s) > 0), 1, -1), 0)
+    return bits.view(np.float64).reshape(np.shape(s)).astype(np.float32)
+
+
+def _edge32(a, b, p, lead):
+    """The edge function in float32: the product that is constant along a row
+    of pixels rounded on its own, the other fused (lead False) or rounded on its
+    own too (True)."""
+    ux, uy, vx, vy = b[0] - a[0], b[1] - a[1], p[0] - a[0], p[1] - a[1]
+    return np.where(lead, ux * vy - uy * vx, _fma32(-uy, vx, ux * vy))
+
+
+def _area32(a, b, p):
+    ux, uy, vx, vy = b[0] - a[0], b[1] - a[1], p[0] - a[0], p[1] - a[1]
+    return _fma32(ux, vy, -(uy * vx))
+
+
+def coverage_f32(vertices, faces, proj, height, width, edge=None):
+    """Face index [H, W] of the device's coverage pass, operation for operation
+    in float32 (no denormals expected): which triangle a pixel whose centre
+    lies on an edge shows depends on how the edge function is rounded.  Of the
+    n pixels of a row of a triangle's bounding box the first n mod 4 are rounded
+    without fusing.  ``edge``: another rounding (a, b, p, lead) -> E to compare
+    with."""
+    edge = edge or _edge32
+    f32 = np.float32
+    v, P = np.asarray(vertices, f32), np.asarray(proj, f32).reshape(4, 4)
+    faces = np.asarray(faces, np.int64).reshape(-1, 3)
+    clip = [_fma32(P[r, 0], v[:, 0], _fma32(P[r, 1], v[:, 1], _fma32(P[r, 2], v[:, 2], P[r, 3]))) for r in range(4)]
+    with np.errstate(all="ignore"):
+        ndc = [c / clip[3] for c in clip[:3]]
+        x, y, z = ([n[faces[:, k]] for k in range(3)] for n in ndc)
+        A = _area32((x[0], y[0]), (x[1], y[1]), (x[2], y[2]))
+        inv = f32(1) / A
+        lo = lambda q: np.fmin(q[0], np.fmin(q[1], q[2]))
+        hi = lambda q: np.fmax(q[0], np.fmax(q[1], q[2]))
+        at = lambda t, n: _fma32(t * f32(0.5), f32(n), f32(-0.5))
+        cmin = np.clip(np.ceil(at(lo(x) + f32(1), width)), 0, width)
+        cmax = np.clip(np.floor(at(hi(x) + f32(1), width)), -1, width - 1)
+        rmin = np.clip(np.ceil(at(f32(1) - hi(y), height)), 0, height)
+        rmax = np.clip(np.floor(at(f32(1) - lo(y), height)), -1, height - 1)
+        ok = np.all(clip[3][faces] > 0, axis=1) & np.isfinite(A) & (A != 0) & (cmin <= cmax) & (rmin <= rmax)
+    f = np.nonzero(ok)[0]
+    cmin, cmax, rmin, rmax = (q[f].astype(np.int64) for q in (cmin, cmax, rmin, rmax))
+    area = (cmax - cmin + 1) * (rmax - rmin + 1)
+    t = np.repeat(np.arange(len(f)), area)                      # (triangle, pixel) pairs of the boxes
+    i = np.arange(int(area.sum())) - np.repeat(np.cumsum(area) - area, area)
+    nc = (cmax - cmin + 1)[t]
+    r, c = rmin[t] + i // nc, cmin[t] + i % nc
+    px = f32(-1) + (f32(2) * c.astype(f32) + f32(1)) / f32(width)
+    py = f32(1) - (f32(2) * r.astype(f32) + f32(1)) / f32(height)
+    F = f[t]
+    n = [(x[k][F], y[k][F]) for k in range(3)]
+    lead = i % nc < nc % 4
+    lam = [edge(n[a], n[b], (px, py), lead) * inv[F] for a, b in ((1, 2), (2, 0), (0, 1))]
+    zz = _fma32(lam[0], z[0][F], _fma32(lam[1], z[1][F], lam[2] * z[2][F]))
+    hit = (lam[0] >= 0) & (lam[1] >= 0) & (lam[2] >= 0) & (zz >= -1) & (zz <= 1)
+    pix, zz, F = (r * width + c)[hit], zz[hit].view(np.uint32), F[hit]
+    key = np.where(zz >> 31 == 1, ~zz, zz | np.uint32(1 << 31))  # the depth key: -0 before +0
+    order = np.lexsort((F, key, pix))                           # nearest first, then the lower face
+    pix, F = pix[order], F[order]
+    first = np.ones(len(pix), bool)
+    first[1:] = pix[1:] != pix[:-1]
+    out = np.full(height * width, -1, np.int64)
+    out[pix[first]] = F[first]
+    return out.reshape(height, width)

@@ -53,9 +53,21 @@ __device__ __forceinline__ bool face_ids(const RasterArgs& a, int f, int& i0, in
     return i0 >= 0 && i1 >= 0 && i2 >= 0 && i0 < a.V && i1 < a.V && i2 < a.V;
 }
 
-// Twice the signed area of (a, b, p): the edge function of edge a -> b.
+// Twice the signed area of (a, b, p): the edge function of edge a -> b.  Which
+// triangle shows a pixel whose centre lies on an edge depends on the last bit
+// of this, so the rounding is spelled out and does not follow the code around
+// a call: one product is rounded on its own, the other is fused.
 __device__ __forceinline__ float edge_fn(float ax, float ay, float bx, float by, float px, float py) {
-    return (bx - ax) * (py - ay) - (by - ay) * (px - ax);
+    return __fmaf_rn(bx - ax, py - ay, -__fmul_rn(by - ay, px - ax));
+}
+// The coverage test's form: the product that is constant along a row of
+// pixels is rounded on its own, the other fused, but for the first n mod 4 of
+// the n pixels of a row of the triangle's box (lead), where both are rounded.
+// The rule is the rounding images have had so far (a walk along the row, in
+// fours after the remainder); another moves pixels on shared edges, 1 in 10^6.
+__device__ __forceinline__ float edge_cover(float ax, float ay, float bx, float by, float px, float py, bool lead) {
+    const float row = __fmul_rn(bx - ax, py - ay), u = by - ay, v = px - ax;
+    return lead ? __fsub_rn(row, __fmul_rn(u, v)) : __fmaf_rn(-u, v, row);
 }
 
 // Order-preserving map of a float to uint32 (for the depth key).
@@ -79,7 +91,8 @@ __global__ void raster_clip_kernel(const __grid_constant__ RasterArgs a, int n_c
 }
 
 // Pixel ranges whose centres a triangle's bounding box holds: column c has
-// x = -1 + (2c + 1) / W, row r has y = 1 - (2r + 1) / H.
+// x = -1 + (2c + 1) / W, row r has y = 1 - (2r + 1) / H (fused steps: a centre
+// may lie on the box).
 struct PixelBox {
     int cmin, cmax, rmin, rmax;
 };
@@ -88,10 +101,10 @@ __device__ __forceinline__ PixelBox pixel_box(const RasterArgs& a, float x0, flo
     const float xmin = fminf(x0, fminf(x1, x2)), xmax = fmaxf(x0, fmaxf(x1, x2));
     const float ymin = fminf(y0, fminf(y1, y2)), ymax = fmaxf(y0, fmaxf(y1, y2));
     PixelBox b;
-    b.cmin = max(0, static_cast<int>(ceilf((xmin + 1.f) * 0.5f * a.W - 0.5f)));
-    b.cmax = min(a.W - 1, static_cast<int>(floorf((xmax + 1.f) * 0.5f * a.W - 0.5f)));
-    b.rmin = max(0, static_cast<int>(ceilf((1.f - ymax) * 0.5f * a.H - 0.5f)));
-    b.rmax = min(a.H - 1, static_cast<int>(floorf((1.f - ymin) * 0.5f * a.H - 0.5f)));
+    b.cmin = max(0, static_cast<int>(ceilf(__fmaf_rn((xmin + 1.f) * 0.5f, a.W, -0.5f))));
+    b.cmax = min(a.W - 1, static_cast<int>(floorf(__fmaf_rn((xmax + 1.f) * 0.5f, a.W, -0.5f))));
+    b.rmin = max(0, static_cast<int>(ceilf(__fmaf_rn((1.f - ymax) * 0.5f, a.H, -0.5f))));
+    b.rmax = min(a.H - 1, static_cast<int>(floorf(__fmaf_rn((1.f - ymin) * 0.5f, a.H, -0.5f))));
     return b;
 }
 
@@ -124,9 +137,10 @@ __global__ void raster_faces_kernel(const __grid_constant__ RasterArgs a) {
     while (r <= b.rmax) {
         const float py = 1.f - (2.f * r + 1.f) / a.H;
         const float px = -1.f + (2.f * c + 1.f) / a.W;
-        const float l0 = edge_fn(x1, y1, x2, y2, px, py) * inv_a;
-        const float l1 = edge_fn(x2, y2, x0, y0, px, py) * inv_a;
-        const float l2 = edge_fn(x0, y0, x1, y1, px, py) * inv_a;
+        const bool lead = c - b.cmin < (nc & 3);
+        const float l0 = edge_cover(x1, y1, x2, y2, px, py, lead) * inv_a;
+        const float l1 = edge_cover(x2, y2, x0, y0, px, py, lead) * inv_a;
+        const float l2 = edge_cover(x0, y0, x1, y1, px, py, lead) * inv_a;
         const float z = fmaf(l0, z0, fmaf(l1, z1, l2 * z2));
         if (!(l0 < 0.f || l1 < 0.f || l2 < 0.f) && z >= -1.f && z <= 1.f) {
             const unsigned long long key = (static_cast<unsigned long long>(ordered_bits(z)) << 32) |
