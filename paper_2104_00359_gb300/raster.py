@@ -24,6 +24,16 @@ def _proj_host(proj):
     return P, P.ctypes.data_as(ctypes.c_void_p)
 
 
+def _one_device(vertices, **others):
+    """The kernels take bare addresses: a host tensor, or one of another device,
+    is refused here."""
+    if not vertices.is_cuda:
+        raise ValueError(f"vertices: expected a CUDA tensor, got one on {vertices.device}")
+    for name, t in others.items():
+        if t.device != vertices.device:
+            raise ValueError(f"{name} is on {t.device}, the vertices on {vertices.device}")
+
+
 def _workspace(lib, V, H, W, device):
     need = int(lib.shs_raster_workspace_bytes(int(V), int(H), int(W)))
     return torch.empty(max(need, 256) // 4, dtype=torch.float32, device=device), need
@@ -32,6 +42,7 @@ def _workspace(lib, V, H, W, device):
 class Rasterize(torch.autograd.Function):
     @staticmethod
     def forward(ctx, vertices, radiance, faces, proj, height, width):
+        _one_device(vertices, radiance=radiance, faces=faces)
         lib = _lib.load()
         v = vertices.contiguous().float()
         b = radiance.contiguous().float()
@@ -60,6 +71,7 @@ class Rasterize(torch.autograd.Function):
         db = torch.empty_like(b) if want_b else None
         if not (want_v or want_b):
             return None, None, None, None, None, None
+        _one_device(v, d_image=d_image)
         ws, need = _workspace(lib, v.shape[0], H, W, v.device)
         stream = current_stream(v.device.index)
         P = ctx.P
