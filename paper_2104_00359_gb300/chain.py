@@ -191,13 +191,33 @@ class ViewBatch:
         except Exception:
             pass
 
+    def check(self, points, normals, albedo, centers, radii, light):
+        """ValueError unless the tensors hold what the views read: [V, P, 3] points
+        and normals, [P, 3] albedo, [V, N, 3] centres (more views or points than
+        that are accepted and not read), [N] radii, [3, K] lighting."""
+        V, P, N = self.V, self.P, self.N
+        for t, name in ((points, "points"), (normals, "normals"), (centers, "centers")):
+            if t.dim() < 1 or t.shape[0] < V:
+                raise ValueError(f"{name} has shape {tuple(t.shape)}: fewer than {V} views")
+        for t, n, name in ((points, points.shape[0], "points"), (normals, normals.shape[0], "normals"),
+                           (albedo, 1, "albedo")):
+            if t.numel() < n * 3 * P:
+                raise ValueError(f"{name} has shape {tuple(t.shape)}: fewer than {P} points")
+        if N and centers.shape[1:] != (N, 3):
+            raise ValueError(f"centers has shape {tuple(centers.shape)}, expected {(V, N, 3)}")
+        if N and radii.shape != (N,):
+            raise ValueError(f"radii has shape {tuple(radii.shape)}, expected {(N,)}")
+        if light.shape != (3, self.K):
+            raise ValueError(f"light has shape {tuple(light.shape)}, expected {(3, self.K)}")
+
     def requests(self, pts, nrm, alb):
-        """One request per view over [V, P, 3] points and normals."""
+        """One request per view over checked points and normals."""
         arr = (_lib.ShsRequest * self.V)()
-        p, n, a, step = pts.data_ptr(), nrm.data_ptr(), alb.data_ptr(), self.P * 12
+        p, n, a = pts.data_ptr(), nrm.data_ptr(), alb.data_ptr()
+        p_step, n_step = pts.stride(0) * 4, nrm.stride(0) * 4
         for v, r in enumerate(arr):
             r.scene, r.n_points, r.saved = self.scenes[v].handle.value, self.P, self.saved[v].data_ptr()
-            r.points, r.normals, r.albedo = p + v * step, n + v * step, a
+            r.points, r.normals, r.albedo = p + v * p_step, n + v * n_step, a
         return arr
 
     def update(self, centers, radii, light):
@@ -218,12 +238,10 @@ class ShadeViews(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, points, normals, albedo, centers, radii, light, views):
-        V, P, N, K = views.V, views.P, views.N, views.K
+        V, P = views.V, views.P
         pts, nrm, alb = _dev(points, "points"), _dev(normals, "normals"), _dev(albedo, "albedo")
         ctr, rad_, lgt = _dev(centers, "centers"), _dev(radii, "radii"), _dev(light, "light")
-        for t, shape, name in ((ctr, (V, N, 3), "centers"), (rad_, (N,), "radii"), (lgt, (3, K), "light")):
-            if t.shape != shape and (N or t is lgt):
-                raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {shape}")
+        views.check(pts, nrm, alb, ctr, rad_, lgt)
         views.update(ctr, rad_, lgt)
         out = torch.empty((V, P, 3), dtype=torch.float32, device=pts.device)
         reqs = views.requests(pts, nrm, alb)
