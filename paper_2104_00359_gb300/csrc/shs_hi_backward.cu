@@ -597,10 +597,9 @@ size_t phase_dyn_smem(int phase, int n_spheres) {
 
 template <bool EXP, bool CULL, int PHASE>
 cudaError_t launch_backward_lp(const BwdArgs& a, int grid, cudaStream_t s) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(backward_lp_kernel<EXP, CULL, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(phase_dyn_smem(PHASE, kMaxSpheres)));
-    if (attr != cudaSuccess) return attr;
+    static DeviceOnce once;
+    const cudaError_t e = allow_dyn_smem(backward_lp_kernel<EXP, CULL, PHASE>, phase_dyn_smem(PHASE, kMaxSpheres), once);
+    if (e != cudaSuccess) return e;
     backward_lp_kernel<EXP, CULL, PHASE>
         <<<static_cast<unsigned>(grid), kBlock, phase_dyn_smem(PHASE, a.sc.n_spheres), s>>>(a);
     count_launch();
@@ -631,13 +630,11 @@ int phase_blocks(int n_spheres) {
 template <bool EXP, bool CULL>
 cudaError_t launch_backward_batch_lp(const BwdBatch& b, cudaStream_t s) {
     const size_t smem = backward_dyn_smem(b.max_spheres);
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(backward_batch_kernel<EXP, CULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(backward_dyn_smem(kMaxSpheres)));
-    if (attr != cudaSuccess) return attr;
+    static DeviceOnce once;
     static WaveCache wave;
     int grid = 0;
-    const cudaError_t e = one_wave(backward_batch_kernel<EXP, CULL>, smem, b.total_tiles, wave, &grid);
+    cudaError_t e = allow_dyn_smem(backward_batch_kernel<EXP, CULL>, backward_dyn_smem(kMaxSpheres), once);
+    if (e == cudaSuccess) e = one_wave(backward_batch_kernel<EXP, CULL>, smem, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
     backward_batch_kernel<EXP, CULL><<<grid, kBlock, smem, s>>>(b);
     count_launch();

@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "shs_device_once.h"
+
 namespace shs {
 
 constexpr int kBlock = 128;          // threads per block
@@ -171,6 +173,18 @@ cudaError_t launch_pack_spheres(const float* centers, const float* radii, float4
                                 bool has_c, bool has_r, cudaStream_t s);
 
 void count_launch();
+
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device;
+// `once` is the kernel's own.
+template <class Kern>
+cudaError_t allow_dyn_smem(Kern kernel, size_t bytes, DeviceOnce& once) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return once.run(dev, [&] {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    });
+}
 
 // Blocks one wave of `kernel` holds on the current device at `smem` dynamic
 // bytes; the last answer per device is kept (an occupancy query takes longer

@@ -917,6 +917,16 @@ size_t backward_dyn_smem(int n_spheres) {
     return static_cast<size_t>(n_spheres) * 16u * (1 + NWARP);
 }
 
+template <int CULLM, int EXPM>
+cudaError_t run_backward(const BwdArgs& a, size_t smem, cudaStream_t s) {
+    static DeviceOnce once;
+    const cudaError_t e = allow_dyn_smem(backward_kernel_t<CULLM, EXPM>, backward_dyn_smem(kMaxSpheres), once);
+    if (e != cudaSuccess) return e;
+    backward_kernel_t<CULLM, EXPM><<<static_cast<unsigned>(a.grid), kBlock, smem, s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 template <>
@@ -946,13 +956,11 @@ template <>
 cudaError_t launch_backward_batch<NB>(const BwdBatch& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
     const size_t smem = backward_dyn_smem(b.max_spheres);
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        backward_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        static_cast<int>(backward_dyn_smem(kMaxSpheres)));
-    if (attr != cudaSuccess) return attr;
+    static DeviceOnce once;
     static WaveCache wave;
     int grid = 0;
-    const cudaError_t e = one_wave(backward_batch_kernel, smem, b.total_tiles, wave, &grid);
+    cudaError_t e = allow_dyn_smem(backward_batch_kernel, backward_dyn_smem(kMaxSpheres), once);
+    if (e == cudaSuccess) e = one_wave(backward_batch_kernel, smem, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
     backward_batch_kernel<<<grid, kBlock, smem, s>>>(b);
     count_launch();
@@ -975,32 +983,11 @@ template <>
 cudaError_t launch_backward<NB>(const BwdArgs& a, cudaStream_t s) {
     if (a.n_points <= 0) return cudaSuccess;
     const size_t smem = backward_dyn_smem(a.sc.n_spheres);
-    static const cudaError_t attr = [] {
-        const int bytes = static_cast<int>(backward_dyn_smem(kMaxSpheres));
-        const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        cudaError_t e = cudaFuncSetAttribute(backward_kernel_t<0, 0>, at, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_kernel_t<1, 0>, at, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_kernel_t<0, 1>, at, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_kernel_t<1, 1>, at, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_kernel_t<0, 3>, at, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(backward_kernel_t<1, 3>, at, bytes);
-        return e;
-    }();
-    cudaError_t err = attr;
-    if (err != cudaSuccess) return err;
-    const dim3 grid(static_cast<unsigned>(a.grid));
-    if (a.sc.exp_mode == 1) {
-        if (a.sc.horizon_cull) backward_kernel_t<1, 1><<<grid, kBlock, smem, s>>>(a);
-        else backward_kernel_t<0, 1><<<grid, kBlock, smem, s>>>(a);
-    } else if (a.sc.exp_mode == 2) {
-        if (a.sc.horizon_cull) backward_kernel_t<1, 3><<<grid, kBlock, smem, s>>>(a);
-        else backward_kernel_t<0, 3><<<grid, kBlock, smem, s>>>(a);
-    } else {
-        if (a.sc.horizon_cull) backward_kernel_t<1, 0><<<grid, kBlock, smem, s>>>(a);
-        else backward_kernel_t<0, 0><<<grid, kBlock, smem, s>>>(a);
-    }
-    count_launch();
-    err = cudaGetLastError();
+    const bool cull = a.sc.horizon_cull != 0;
+    cudaError_t err;
+    if (a.sc.exp_mode == 1) err = cull ? run_backward<1, 1>(a, smem, s) : run_backward<0, 1>(a, smem, s);
+    else if (a.sc.exp_mode == 2) err = cull ? run_backward<1, 3>(a, smem, s) : run_backward<0, 3>(a, smem, s);
+    else err = cull ? run_backward<1, 0>(a, smem, s) : run_backward<0, 0>(a, smem, s);
     if (err != cudaSuccess || a.counter != nullptr) return err;
     const int E = 3 * K + 1 + 4 * a.sc.n_spheres;
     reduce_partials_kernel<<<reduce_blocks(E), kReduceThreads, 0, s>>>(a, a.grid, a.grid);
