@@ -154,16 +154,16 @@ template <int NB> struct Bwd {
     static cudaError_t run(const BwdArgs& a, cudaStream_t s) { return shs::launch_backward<NB>(a, s); }
 };
 
-shs::BwdBlocks blocks_per_sm(int nb, int n) {
+shs::BwdBlocks blocks_per_sm(int nb, int n, bool split) {
     switch (nb) {
-        case 1: return shs::backward_blocks_per_sm<1>(n);
-        case 2: return shs::backward_blocks_per_sm<2>(n);
-        case 3: return shs::backward_blocks_per_sm<3>(n);
-        case 4: return shs::backward_blocks_per_sm<4>(n);
-        case 5: return shs::backward_blocks_per_sm<5>(n);
-        case 6: return shs::backward_blocks_per_sm<6>(n);
-        case 7: return shs::backward_blocks_per_sm<7>(n);
-        case 8: return shs::backward_blocks_per_sm<8>(n);
+        case 1: return shs::backward_blocks_per_sm<1>(n, split);
+        case 2: return shs::backward_blocks_per_sm<2>(n, split);
+        case 3: return shs::backward_blocks_per_sm<3>(n, split);
+        case 4: return shs::backward_blocks_per_sm<4>(n, split);
+        case 5: return shs::backward_blocks_per_sm<5>(n, split);
+        case 6: return shs::backward_blocks_per_sm<6>(n, split);
+        case 7: return shs::backward_blocks_per_sm<7>(n, split);
+        case 8: return shs::backward_blocks_per_sm<8>(n, split);
         default: return {1, 1, 1};
     }
 }
@@ -481,7 +481,7 @@ int report_cuda(cudaError_t e, const char* what) { return cuda_fail(e, what); }
 cudaError_t launch_backward_nb(int n_bands, const BwdArgs& a, cudaStream_t s) {
     return dispatch<Bwd>(n_bands, a, s);
 }
-int backward_blocks_per_sm_nb(int n_bands, int n_spheres) { return blocks_per_sm(n_bands, n_spheres).both; }
+int backward_blocks_per_sm_nb(int n_bands, int n_spheres) { return blocks_per_sm(n_bands, n_spheres, false).both; }
 }  // namespace shs
 
 extern "C" {
@@ -525,7 +525,7 @@ shs_status shs_scene_create(const shs_config* cfg, int32_t n_spheres, const floa
         delete sc;
         return cuda_fail(e, "query device");
     }
-    const shs::BwdBlocks blocks = blocks_per_sm(cfg->n_bands, n_spheres);
+    const shs::BwdBlocks blocks = blocks_per_sm(cfg->n_bands, n_spheres, cfg->n_bands >= 6);
     sc->tail_grid = sms * blocks.tail;
     sc->grid = sms * (cfg->n_bands >= 6 ? blocks.pairs : blocks.both);
     sc->max_grid = sc->grid > sc->tail_grid ? sc->grid : sc->tail_grid;

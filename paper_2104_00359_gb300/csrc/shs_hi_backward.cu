@@ -644,9 +644,9 @@ cudaError_t launch_backward_batch_lp(const BwdBatch& b, cudaStream_t s) {
 }  // namespace
 
 template <>
-BwdBlocks backward_blocks_per_sm<NB>(int n_spheres) {
-    return BwdBlocks{phase_blocks<kPhaseBoth>(n_spheres), phase_blocks<kPhaseTail>(n_spheres),
-                     phase_blocks<kPhasePairs>(n_spheres)};
+BwdBlocks backward_blocks_per_sm<NB>(int n_spheres, bool split) {
+    if (!split) return BwdBlocks{phase_blocks<kPhaseBoth>(n_spheres), 0, 0};
+    return BwdBlocks{0, phase_blocks<kPhaseTail>(n_spheres), phase_blocks<kPhasePairs>(n_spheres)};
 }
 
 template <>

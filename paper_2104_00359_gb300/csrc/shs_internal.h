@@ -163,12 +163,13 @@ template <int NB> cudaError_t launch_forward_batch(const FwdBatch& b, cudaStream
 template <int NB> cudaError_t launch_backward_batch(const BwdBatch& b, cudaStream_t s);
 template <int NB> cudaError_t launch_forward(const FwdArgs& a, cudaStream_t s);
 template <int NB> cudaError_t launch_backward(const BwdArgs& a, cudaStream_t s);
-// Resident blocks per SM of the adjoint kernels: as one launch, and (from 6
-// bands) of the tail's and the pair pass's own launches.
+// Resident blocks per SM of the adjoint kernels: as one launch, or (split, from
+// 6 bands) of the tail's and the pair pass's own launches; only what is asked
+// for is queried.
 struct BwdBlocks {
     int both, tail, pairs;
 };
-template <int NB> BwdBlocks backward_blocks_per_sm(int n_spheres);
+template <int NB> BwdBlocks backward_blocks_per_sm(int n_spheres, bool split);
 cudaError_t launch_pack_spheres(const float* centers, const float* radii, float4* out, int n,
                                 bool has_c, bool has_r, cudaStream_t s);
 

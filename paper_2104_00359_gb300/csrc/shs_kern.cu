@@ -930,7 +930,7 @@ cudaError_t run_backward(const BwdArgs& a, size_t smem, cudaStream_t s) {
 }  // namespace
 
 template <>
-BwdBlocks backward_blocks_per_sm<NB>(int n_spheres) {
+BwdBlocks backward_blocks_per_sm<NB>(int n_spheres, bool) {
     cudaFuncSetAttribute(backward_kernel_t<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          static_cast<int>(backward_dyn_smem(kMaxSpheres)));
     int nb = 0;
