@@ -46,12 +46,11 @@ struct EnvArgs {
 // P_l^m(x) without the Condon-Shortley phase, s = sqrt(1 - x^2) >= 0:
 // P_m^m = (2m-1)!! s^m, P_{m+1}^m = (2m+1) x P_m^m,
 // (l - m) P_l^m = (2l-1) x P_{l-1}^m - (l+m-1) P_{l-2}^m.
-__constant__ float kInverse[8] = {0.f, 1.f, 1.f / 2.f, 1.f / 3.f, 1.f / 4.f, 1.f / 5.f, 1.f / 6.f, 1.f / 7.f};
 __device__ __forceinline__ float assoc_legendre(int l, int m, float x, float s) {
     float p0 = 0.f, p1 = 1.f;
     for (int k = 1; k <= m; ++k) p1 *= (2.f * k - 1.f) * s;
     for (int ll = m + 1; ll <= l; ++ll) {
-        const float p2 = ((2.f * ll - 1.f) * x * p1 - (ll + m - 1.f) * p0) * kInverse[ll - m];
+        const float p2 = ((2.f * ll - 1.f) * x * p1 - (ll + m - 1.f) * p0) / (ll - m);
         p0 = p1;
         p1 = p2;
     }
@@ -263,9 +262,9 @@ __global__ void __launch_bounds__(kEnvBlock, SHS_ENV_MINB) envmap_rows_kernel(co
                 mom[ch * NF + 2 * mm] = acc2[3 * (mm - 1) + ch].y;
             }
         }
-        // the row's weights, one evaluation per (l, m >= 0) and no divisions: per
-        // coefficient and channel they cost 8 us of 79 on a 4096 x 8192 map at 8
-        // bands (every warp's at the same time, with the loads idle)
+        // the row's weights, one evaluation per (l, m >= 0): per coefficient and
+        // channel they cost 8 us of 79 on a 4096 x 8192 map at 8 bands (every
+        // warp's at the same time, with the loads idle)
         float st, ct;
         sincospif((r + 0.5f) / a.H, &st, &ct);
         const float w_row = a.domega_scale * st;
