@@ -104,7 +104,7 @@ struct shs_scene_s {
     int* status;           // device status word
     float* partials;       // [max_grid][partial_stride] (deterministic) or accumulator
     unsigned int* counter;
-    float* batch_acc;      // [partial_stride] accumulator for batched calls (kept zero)
+    float* batch_acc;      // [partial_stride] accumulator for batched calls, then the loss in float64 (kept zero)
     unsigned int* batch_counter;
     float* fwork;          // f storage when shs_shade gets no saved buffer (tensor-core path)
     int64_t fwork_points;
@@ -208,6 +208,8 @@ SceneView view_of(const shs_scene_s* s) {
     v.status = s->status;
     return v;
 }
+
+size_t batch_acc_bytes(const shs_scene_s* s) { return sizeof(float) * s->partial_stride + sizeof(double); }
 
 int variant_of(const shs_scene_s* s) { return shs::batch_variant(view_of(s), s->cfg.n_bands); }
 
@@ -537,9 +539,9 @@ shs_status shs_scene_create(const shs_config* cfg, int32_t n_spheres, const floa
     if (e == cudaSuccess) e = cudaMalloc(&sc->status, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&sc->partials, sizeof(float) * partial_floats);
     if (e == cudaSuccess) e = cudaMalloc(&sc->counter, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMalloc(&sc->batch_acc, sizeof(float) * sc->partial_stride);
+    if (e == cudaSuccess) e = cudaMalloc(&sc->batch_acc, batch_acc_bytes(sc));
     if (e == cudaSuccess) e = cudaMalloc(&sc->batch_counter, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(sc->batch_acc, 0, sizeof(float) * sc->partial_stride, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sc->batch_acc, 0, batch_acc_bytes(sc), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc->batch_counter, 0, sizeof(unsigned int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc->light, 0, sizeof(float) * 3 * sc->Kpad, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(sc->status, 0, sizeof(int), s);
@@ -817,6 +819,7 @@ static shs_status backward_common(shs_scene_t sc, int64_t n_points, const float*
     a.counter = sc->cfg.deterministic ? nullptr : sc->counter;
     a.partial_stride = sc->partial_stride;
     a.dfp_ws = nullptr;
+    a.loss_sum = nullptr;
     const int per_tile = shs::tile_points(sc->cfg.n_bands);
     const int64_t tiles = (n_points + per_tile - 1) / per_tile;
     a.grid = static_cast<int>(tiles < sc->grid ? tiles : sc->grid);
@@ -1042,6 +1045,7 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
             a.d_points = r.d_points;
             a.d_normals = r.d_normals;
             a.partials = sc->batch_acc;
+            a.loss_sum = reinterpret_cast<double*>(sc->batch_acc + sc->partial_stride);
             a.counter = sc->batch_counter;
             a.partial_stride = sc->partial_stride;
             bb.tile_begin[bb.n] = bb.total_tiles;
@@ -1068,7 +1072,7 @@ shs_status shs_scene_device_status(shs_scene_t sc, void* stream, int32_t* device
         // next launch would finish early with stale sums.  Start them afresh.
         e = cudaMemsetAsync(sc->partials, 0, sizeof(float) * sc->partial_stride, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(sc->counter, 0, sizeof(unsigned int), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(sc->batch_acc, 0, sizeof(float) * sc->partial_stride, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(sc->batch_acc, 0, batch_acc_bytes(sc), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(sc->batch_counter, 0, sizeof(unsigned int), s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }

@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_batch_kernel(con
         lp_backward_tile<EXP, CULL, kPhaseBoth>(a, sh, tile - b.tile_begin[r]);
         __syncthreads();
         const int E = 3 * K + 1 + 4 * N;
-        for (int e = threadIdx.x; e < E; e += kBlock) atomicAdd(a.partials + e, lp_block_sum(sh, N, e));
+        for (int e = threadIdx.x; e < E; e += kBlock) add_tile_sum(a, e, lp_block_sum(sh, N, e));
         __threadfence();
         __syncthreads();
         const int64_t ntiles_r = b.tile_begin[r + 1] - b.tile_begin[r];

@@ -73,6 +73,7 @@ struct BwdArgs {
                              // pass (from 6 bands), or null: one launch
     float* partials;         // [grid][stride] scratch
     unsigned int* counter;   // scratch, zero between launches
+    double* loss_sum;        // batch: the loss over the request's tiles, zero between launches; else null
     int partial_stride;
     int grid;                // persistent grid size (of the pair pass when there are two launches)
     int tail_grid;           // grid of the tail's launch; 0: the tail ran before (tensor cores), its coefficients

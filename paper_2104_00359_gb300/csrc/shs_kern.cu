@@ -902,7 +902,7 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? 4 : 1)
 #pragma unroll
                 for (int w = 0; w < NWARP; ++w) v += s_acc[w * 4 * N + q];
             }
-            atomicAdd(a.partials + e, v);
+            add_tile_sum(a, e, v);
         }
         __threadfence();
         __syncthreads();

@@ -205,13 +205,28 @@ __device__ __forceinline__ float load_or(const float* p, int64_t i, bool live) {
 // only, stored; or, from a stored f, the exponential and shading.
 constexpr int kFwdFull = 0, kFwdPairs = 1, kFwdTail = 2;
 
+// Adds the tile's total of entry e to a batch request's accumulator.  The
+// loss, a sum of a thousand terms of one sign and more, is added in float64:
+// in float32 its error grows with the number of tiles (2e-6 at 16k tiles).
+__device__ __forceinline__ void add_tile_sum(const BwdArgs& a, int e, float v) {
+    if (e == 3 * K) {
+        if (a.loss) atomicAdd(a.loss_sum, static_cast<double>(v));
+    } else {
+        atomicAdd(a.partials + e, v);
+    }
+}
+
 // The last contributor copies the accumulated scene-level sums to the
 // outputs and re-zeroes the accumulator and its counter for the next launch.
 __device__ void finish_scene_sums(const BwdArgs& a, int E) {
     __threadfence();
     for (int e = threadIdx.x; e < E; e += kBlock) {
-        const float v = __ldcg(a.partials + e);
+        float v = __ldcg(a.partials + e);
         a.partials[e] = 0.f;
+        if (e == 3 * K && a.loss_sum) {
+            v = static_cast<float>(__ldcg(a.loss_sum));
+            *a.loss_sum = 0.0;
+        }
         if (e < 3 * K) {
             if (a.d_light) a.d_light[e] = v;
         } else if (e == 3 * K) {
