@@ -731,9 +731,6 @@ def generate():
     for n in BANDS:
         K = n * n
         C = gaunt_monomial(n)
-        code, outs = build_ybar(n)
-        fwd = emit_forward(code, outs, "Y")
-        vjp = emit_forward(code, [], "Y") + emit_vjp(code, outs)
         mul_l, sqr_l = emit_gaunt(n, C) if n < LANE_PAIR_FROM else ([], [])
         N = norms(n)
         A = ahat(n)
@@ -741,9 +738,9 @@ def generate():
         parts.append(f"template <> struct SH<{n}> {{")
         parts.append(f"    static constexpr int K = {K};")
         parts.append(f"    static constexpr int NNZ_SYM = {len(C)};   // entries (i, j <= k)")
-        parts.append(f"    static constexpr int EZ = {2 * n};    // projected-exponential rule: Gauss-Legendre nodes")
-        parts.append(f"    static constexpr int EP = {4 * n};    // projected-exponential rule: uniform azimuths")
         if n < LANE_PAIR_FROM:
+            parts.append(f"    static constexpr int EZ = {2 * n};    // projected-exponential rule: Gauss-Legendre nodes")
+            parts.append(f"    static constexpr int EP = {4 * n};    // projected-exponential rule: uniform azimuths")
             parts.append("#if defined(SHS_NB) && SHS_NB == " + str(n))
             parts.append(f"    __device__ __forceinline__ static const float* eleg() {{ return kExpLeg{n}; }}")
             parts.append(f"    __device__ __forceinline__ static const float* etrig() {{ return kExpTrig{n}; }}")
@@ -763,16 +760,19 @@ def generate():
         parts.append("            default: return 0.0f;")
         parts.append("        }")
         parts.append("    }")
-        parts.append("    __device__ __forceinline__ static void ybar(float x, float y, float z, float* Y) {")
-        parts.append("        (void)x; (void)y; (void)z;")
-        parts.append(indent(fwd))
-        parts.append("    }")
-        parts.append("    __device__ __forceinline__ static void ybar_vjp(float x, float y, float z, const float* w,")
-        parts.append("                                                    float& gx, float& gy, float& gz) {")
-        parts.append("        (void)x; (void)y; (void)z; (void)w;")
-        parts.append(indent([ln for ln in vjp if not ln.startswith("Y[")]))
-        parts.append("    }")
         if n < LANE_PAIR_FROM:
+            code, outs = build_ybar(n)
+            fwd = emit_forward(code, outs, "Y")
+            vjp = emit_forward(code, [], "Y") + emit_vjp(code, outs)
+            parts.append("    __device__ __forceinline__ static void ybar(float x, float y, float z, float* Y) {")
+            parts.append("        (void)x; (void)y; (void)z;")
+            parts.append(indent(fwd))
+            parts.append("    }")
+            parts.append("    __device__ __forceinline__ static void ybar_vjp(float x, float y, float z, const float* w,")
+            parts.append("                                                    float& gx, float& gy, float& gz) {")
+            parts.append("        (void)x; (void)y; (void)z; (void)w;")
+            parts.append(indent([ln for ln in vjp if not ln.startswith("Y[")]))
+            parts.append("    }")
             na, ng, ml, acc_l, m2f_l, gc_l, ge_l = emit_monomial_route(n)
             parts.append(f"    static constexpr int NA = {na};   // monomials of degree < n")
             parts.append(f"    static constexpr int NG = {ng};   // symmetric tensor entries, bands >= 1")

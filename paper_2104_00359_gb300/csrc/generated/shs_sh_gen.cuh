@@ -1444,8 +1444,6 @@ static __constant__ float kLpTrig6[44] = {1.0f, 0.9807852506637573f, 0.195090323
 template <> struct SH<6> {
     static constexpr int K = 36;
     static constexpr int NNZ_SYM = 1517;   // entries (i, j <= k)
-    static constexpr int EZ = 12;    // projected-exponential rule: Gauss-Legendre nodes
-    static constexpr int EP = 24;    // projected-exponential rule: uniform azimuths
     __device__ __forceinline__ static float norm(int i) {
         switch (i) {
             case 0: return 0.282094806432724f;
@@ -1497,337 +1495,6 @@ template <> struct SH<6> {
             case 5: return 0.0f;
             default: return 0.0f;
         }
-    }
-    __device__ __forceinline__ static void ybar(float x, float y, float z, float* Y) {
-        (void)x; (void)y; (void)z;
-        const float t0 = x * x;
-        const float t1 = y * y;
-        const float t2 = t0 - t1;
-        const float t3 = x * y;
-        const float t4 = y * x;
-        const float t5 = t3 + t4;
-        const float t6 = x * t2;
-        const float t7 = y * t5;
-        const float t8 = t6 - t7;
-        const float t9 = x * t5;
-        const float t10 = y * t2;
-        const float t11 = t9 + t10;
-        const float t12 = x * t8;
-        const float t13 = y * t11;
-        const float t14 = t12 - t13;
-        const float t15 = x * t11;
-        const float t16 = y * t8;
-        const float t17 = t15 + t16;
-        const float t18 = x * t14;
-        const float t19 = y * t17;
-        const float t20 = t18 - t19;
-        const float t21 = x * t17;
-        const float t22 = y * t14;
-        const float t23 = t21 + t22;
-        const float t24 = z * z;
-        const float t25 = t24 * 1.5f;
-        const float t26 = t25 - 0.5f;
-        const float t27 = z * t26;
-        const float t28 = t27 * 1.6666666269302368f;
-        const float t29 = z * 0.6666666865348816f;
-        const float t30 = t28 - t29;
-        const float t31 = z * t30;
-        const float t32 = t31 * 1.75f;
-        const float t33 = t26 * 0.75f;
-        const float t34 = t32 - t33;
-        const float t35 = z * t34;
-        const float t36 = t35 * 1.7999999523162842f;
-        const float t37 = t30 * 0.800000011920929f;
-        const float t38 = t36 - t37;
-        const float t39 = z * 3.0f;
-        const float t40 = z * t39;
-        const float t41 = t40 * 2.5f;
-        const float t42 = t41 - 1.5f;
-        const float t43 = z * t42;
-        const float t44 = t43 * 2.3333332538604736f;
-        const float t45 = t39 * 1.3333333730697632f;
-        const float t46 = t44 - t45;
-        const float t47 = z * t46;
-        const float t48 = t47 * 2.25f;
-        const float t49 = t42 * 1.25f;
-        const float t50 = t48 - t49;
-        const float t51 = z * 3.0f;
-        const float t52 = t51 * 5.0f;
-        const float t53 = z * t52;
-        const float t54 = t53 * 3.5f;
-        const float t55 = t54 - 7.5f;
-        const float t56 = z * t55;
-        const float t57 = t56 * 3.0f;
-        const float t58 = t52 * 2.0f;
-        const float t59 = t57 - t58;
-        const float t60 = z * 15.0f;
-        const float t61 = t60 * 7.0f;
-        const float t62 = z * t61;
-        const float t63 = t62 * 4.5f;
-        const float t64 = t63 - 52.5f;
-        const float t65 = z * 105.0f;
-        const float t66 = t65 * 9.0f;
-        const float t67 = t39 * x;
-        const float t68 = t39 * y;
-        const float t69 = t2 * 3.0f;
-        const float t70 = t5 * 3.0f;
-        const float t71 = t42 * x;
-        const float t72 = t42 * y;
-        const float t73 = t52 * t2;
-        const float t74 = t52 * t5;
-        const float t75 = t8 * 15.0f;
-        const float t76 = t11 * 15.0f;
-        const float t77 = t46 * x;
-        const float t78 = t46 * y;
-        const float t79 = t55 * t2;
-        const float t80 = t55 * t5;
-        const float t81 = t61 * t8;
-        const float t82 = t61 * t11;
-        const float t83 = t14 * 105.0f;
-        const float t84 = t17 * 105.0f;
-        const float t85 = t50 * x;
-        const float t86 = t50 * y;
-        const float t87 = t59 * t2;
-        const float t88 = t59 * t5;
-        const float t89 = t64 * t8;
-        const float t90 = t64 * t11;
-        const float t91 = t66 * t14;
-        const float t92 = t66 * t17;
-        const float t93 = t20 * 945.0f;
-        const float t94 = t23 * 945.0f;
-        Y[0] = 1.0f;
-        Y[1] = y;
-        Y[2] = z;
-        Y[3] = x;
-        Y[4] = t70;
-        Y[5] = t68;
-        Y[6] = t26;
-        Y[7] = t67;
-        Y[8] = t69;
-        Y[9] = t76;
-        Y[10] = t74;
-        Y[11] = t72;
-        Y[12] = t30;
-        Y[13] = t71;
-        Y[14] = t73;
-        Y[15] = t75;
-        Y[16] = t84;
-        Y[17] = t82;
-        Y[18] = t80;
-        Y[19] = t78;
-        Y[20] = t34;
-        Y[21] = t77;
-        Y[22] = t79;
-        Y[23] = t81;
-        Y[24] = t83;
-        Y[25] = t94;
-        Y[26] = t92;
-        Y[27] = t90;
-        Y[28] = t88;
-        Y[29] = t86;
-        Y[30] = t38;
-        Y[31] = t85;
-        Y[32] = t87;
-        Y[33] = t89;
-        Y[34] = t91;
-        Y[35] = t93;
-    }
-    __device__ __forceinline__ static void ybar_vjp(float x, float y, float z, const float* w,
-                                                    float& gx, float& gy, float& gz) {
-        (void)x; (void)y; (void)z; (void)w;
-        const float t0 = x * x;
-        const float t1 = y * y;
-        const float t2 = t0 - t1;
-        const float t3 = x * y;
-        const float t4 = y * x;
-        const float t5 = t3 + t4;
-        const float t6 = x * t2;
-        const float t7 = y * t5;
-        const float t8 = t6 - t7;
-        const float t9 = x * t5;
-        const float t10 = y * t2;
-        const float t11 = t9 + t10;
-        const float t12 = x * t8;
-        const float t13 = y * t11;
-        const float t14 = t12 - t13;
-        const float t15 = x * t11;
-        const float t16 = y * t8;
-        const float t17 = t15 + t16;
-        const float t18 = x * t14;
-        const float t19 = y * t17;
-        const float t20 = t18 - t19;
-        const float t21 = x * t17;
-        const float t22 = y * t14;
-        const float t23 = t21 + t22;
-        const float t24 = z * z;
-        const float t25 = t24 * 1.5f;
-        const float t26 = t25 - 0.5f;
-        const float t27 = z * t26;
-        const float t28 = t27 * 1.6666666269302368f;
-        const float t29 = z * 0.6666666865348816f;
-        const float t30 = t28 - t29;
-        const float t31 = z * t30;
-        const float t32 = t31 * 1.75f;
-        const float t33 = t26 * 0.75f;
-        const float t34 = t32 - t33;
-        const float t35 = z * t34;
-        const float t36 = t35 * 1.7999999523162842f;
-        const float t37 = t30 * 0.800000011920929f;
-        const float t38 = t36 - t37;
-        const float t39 = z * 3.0f;
-        const float t40 = z * t39;
-        const float t41 = t40 * 2.5f;
-        const float t42 = t41 - 1.5f;
-        const float t43 = z * t42;
-        const float t44 = t43 * 2.3333332538604736f;
-        const float t45 = t39 * 1.3333333730697632f;
-        const float t46 = t44 - t45;
-        const float t47 = z * t46;
-        const float t48 = t47 * 2.25f;
-        const float t49 = t42 * 1.25f;
-        const float t50 = t48 - t49;
-        const float t51 = z * 3.0f;
-        const float t52 = t51 * 5.0f;
-        const float t53 = z * t52;
-        const float t54 = t53 * 3.5f;
-        const float t55 = t54 - 7.5f;
-        const float t56 = z * t55;
-        const float t57 = t56 * 3.0f;
-        const float t58 = t52 * 2.0f;
-        const float t59 = t57 - t58;
-        const float t60 = z * 15.0f;
-        const float t61 = t60 * 7.0f;
-        const float t62 = z * t61;
-        const float t63 = t62 * 4.5f;
-        const float t64 = t63 - 52.5f;
-        const float t65 = z * 105.0f;
-        const float t66 = t65 * 9.0f;
-        const float t67 = t39 * x;
-        const float t68 = t39 * y;
-        const float t69 = t2 * 3.0f;
-        const float t70 = t5 * 3.0f;
-        const float t71 = t42 * x;
-        const float t72 = t42 * y;
-        const float t73 = t52 * t2;
-        const float t74 = t52 * t5;
-        const float t75 = t8 * 15.0f;
-        const float t76 = t11 * 15.0f;
-        const float t77 = t46 * x;
-        const float t78 = t46 * y;
-        const float t79 = t55 * t2;
-        const float t80 = t55 * t5;
-        const float t81 = t61 * t8;
-        const float t82 = t61 * t11;
-        const float t83 = t14 * 105.0f;
-        const float t84 = t17 * 105.0f;
-        const float t85 = t50 * x;
-        const float t86 = t50 * y;
-        const float t87 = t59 * t2;
-        const float t88 = t59 * t5;
-        const float t89 = t64 * t8;
-        const float t90 = t64 * t11;
-        const float t91 = t66 * t14;
-        const float t92 = t66 * t17;
-        const float t93 = t20 * 945.0f;
-        const float t94 = t23 * 945.0f;
-        const float a_t94 = w[25];
-        const float a_t93 = w[35];
-        const float a_t92 = w[26];
-        const float a_t91 = w[34];
-        const float a_t90 = w[27];
-        const float a_t89 = w[33];
-        const float a_t88 = w[28];
-        const float a_t87 = w[32];
-        const float a_t86 = w[29];
-        const float a_t85 = w[31];
-        const float a_t84 = w[16];
-        const float a_t83 = w[24];
-        const float a_t82 = w[17];
-        const float a_t81 = w[23];
-        const float a_t80 = w[18];
-        const float a_t79 = w[22];
-        const float a_t78 = w[19];
-        const float a_t77 = w[21];
-        const float a_t76 = w[9];
-        const float a_t75 = w[15];
-        const float a_t74 = w[10];
-        const float a_t73 = w[14];
-        const float a_t72 = w[11];
-        const float a_t71 = w[13];
-        const float a_t70 = w[4];
-        const float a_t69 = w[8];
-        const float a_t68 = w[5];
-        const float a_t67 = w[7];
-        const float a_t66 = t17 * a_t92 + t14 * a_t91;
-        const float a_t65 = 9.0f * a_t66;
-        const float a_t64 = t11 * a_t90 + t8 * a_t89;
-        const float a_t63 = a_t64;
-        const float a_t62 = 4.5f * a_t63;
-        const float a_t61 = t11 * a_t82 + t8 * a_t81 + z * a_t62;
-        const float a_t60 = 7.0f * a_t61;
-        const float a_t59 = t5 * a_t88 + t2 * a_t87;
-        const float a_t58 = -a_t59;
-        const float a_t57 = a_t59;
-        const float a_t56 = 3.0f * a_t57;
-        const float a_t55 = t5 * a_t80 + t2 * a_t79 + z * a_t56;
-        const float a_t54 = a_t55;
-        const float a_t53 = 3.5f * a_t54;
-        const float a_t52 = t5 * a_t74 + t2 * a_t73 + 2.0f * a_t58 + z * a_t53;
-        const float a_t51 = 5.0f * a_t52;
-        const float a_t50 = y * a_t86 + x * a_t85;
-        const float a_t49 = -a_t50;
-        const float a_t48 = a_t50;
-        const float a_t47 = 2.25f * a_t48;
-        const float a_t46 = y * a_t78 + x * a_t77 + z * a_t47;
-        const float a_t45 = -a_t46;
-        const float a_t44 = a_t46;
-        const float a_t43 = 2.3333332538604736f * a_t44;
-        const float a_t42 = y * a_t72 + x * a_t71 + 1.25f * a_t49 + z * a_t43;
-        const float a_t41 = a_t42;
-        const float a_t40 = 2.5f * a_t41;
-        const float a_t39 = y * a_t68 + x * a_t67 + 1.3333333730697632f * a_t45 + z * a_t40;
-        const float a_t38 = w[30];
-        const float a_t37 = -a_t38;
-        const float a_t36 = a_t38;
-        const float a_t35 = 1.7999999523162842f * a_t36;
-        const float a_t34 = w[20] + z * a_t35;
-        const float a_t33 = -a_t34;
-        const float a_t32 = a_t34;
-        const float a_t31 = 1.75f * a_t32;
-        const float a_t30 = w[12] + 0.800000011920929f * a_t37 + z * a_t31;
-        const float a_t29 = -a_t30;
-        const float a_t28 = a_t30;
-        const float a_t27 = 1.6666666269302368f * a_t28;
-        const float a_t26 = w[6] + 0.75f * a_t33 + z * a_t27;
-        const float a_t25 = a_t26;
-        const float a_t24 = 1.5f * a_t25;
-        const float a_t23 = 945.0f * a_t94;
-        const float a_t22 = a_t23;
-        const float a_t21 = a_t23;
-        const float a_t20 = 945.0f * a_t93;
-        const float a_t19 = -a_t20;
-        const float a_t18 = a_t20;
-        const float a_t17 = t66 * a_t92 + 105.0f * a_t84 + x * a_t21 + y * a_t19;
-        const float a_t16 = a_t17;
-        const float a_t15 = a_t17;
-        const float a_t14 = t66 * a_t91 + 105.0f * a_t83 + y * a_t22 + x * a_t18;
-        const float a_t13 = -a_t14;
-        const float a_t12 = a_t14;
-        const float a_t11 = t64 * a_t90 + t61 * a_t82 + 15.0f * a_t76 + x * a_t15 + y * a_t13;
-        const float a_t10 = a_t11;
-        const float a_t9 = a_t11;
-        const float a_t8 = t64 * a_t89 + t61 * a_t81 + 15.0f * a_t75 + y * a_t16 + x * a_t12;
-        const float a_t7 = -a_t8;
-        const float a_t6 = a_t8;
-        const float a_t5 = t59 * a_t88 + t55 * a_t80 + t52 * a_t74 + 3.0f * a_t70 + x * a_t9 + y * a_t7;
-        const float a_t4 = a_t5;
-        const float a_t3 = a_t5;
-        const float a_t2 = t59 * a_t87 + t55 * a_t79 + t52 * a_t73 + 3.0f * a_t69 + y * a_t10 + x * a_t6;
-        const float a_t1 = -a_t2;
-        const float a_t0 = a_t2;
-        gx = w[3] + t50 * a_t85 + t46 * a_t77 + t42 * a_t71 + t39 * a_t67 + t17 * a_t21 + t14 * a_t18 + t11 * a_t15 + t8 * a_t12 + t5 * a_t9 + t2 * a_t6 + y * a_t4 + y * a_t3 + x * a_t0 + x * a_t0;
-        gy = w[1] + t50 * a_t86 + t46 * a_t78 + t42 * a_t72 + t39 * a_t68 + t14 * a_t22 + t17 * a_t19 + t8 * a_t16 + t11 * a_t13 + t2 * a_t10 + t5 * a_t7 + x * a_t4 + x * a_t3 + y * a_t1 + y * a_t1;
-        gz = w[2] + 105.0f * a_t65 + t61 * a_t62 + 15.0f * a_t60 + t55 * a_t56 + t52 * a_t53 + 3.0f * a_t51 + t46 * a_t47 + t42 * a_t43 + t39 * a_t40 + 3.0f * a_t39 + t34 * a_t35 + t30 * a_t31 + 0.6666666865348816f * a_t29 + t26 * a_t27 + z * a_t24 + z * a_t24;
     }
     static constexpr int LPS = 4;   // lane-pair product rule: node pairs
     static constexpr int LPQ = 4;   // ... and azimuth quads
@@ -1959,8 +1626,6 @@ static __constant__ float kLpTrig7[65] = {1.0f, 0.9876883625984192f, 0.156434461
 template <> struct SH<7> {
     static constexpr int K = 49;
     static constexpr int NNZ_SYM = 3348;   // entries (i, j <= k)
-    static constexpr int EZ = 14;    // projected-exponential rule: Gauss-Legendre nodes
-    static constexpr int EP = 28;    // projected-exponential rule: uniform azimuths
     __device__ __forceinline__ static float norm(int i) {
         switch (i) {
             case 0: return 0.282094806432724f;
@@ -2026,467 +1691,6 @@ template <> struct SH<7> {
             case 6: return 0.04908738657832146f;
             default: return 0.0f;
         }
-    }
-    __device__ __forceinline__ static void ybar(float x, float y, float z, float* Y) {
-        (void)x; (void)y; (void)z;
-        const float t0 = x * x;
-        const float t1 = y * y;
-        const float t2 = t0 - t1;
-        const float t3 = x * y;
-        const float t4 = y * x;
-        const float t5 = t3 + t4;
-        const float t6 = x * t2;
-        const float t7 = y * t5;
-        const float t8 = t6 - t7;
-        const float t9 = x * t5;
-        const float t10 = y * t2;
-        const float t11 = t9 + t10;
-        const float t12 = x * t8;
-        const float t13 = y * t11;
-        const float t14 = t12 - t13;
-        const float t15 = x * t11;
-        const float t16 = y * t8;
-        const float t17 = t15 + t16;
-        const float t18 = x * t14;
-        const float t19 = y * t17;
-        const float t20 = t18 - t19;
-        const float t21 = x * t17;
-        const float t22 = y * t14;
-        const float t23 = t21 + t22;
-        const float t24 = x * t20;
-        const float t25 = y * t23;
-        const float t26 = t24 - t25;
-        const float t27 = x * t23;
-        const float t28 = y * t20;
-        const float t29 = t27 + t28;
-        const float t30 = z * z;
-        const float t31 = t30 * 1.5f;
-        const float t32 = t31 - 0.5f;
-        const float t33 = z * t32;
-        const float t34 = t33 * 1.6666666269302368f;
-        const float t35 = z * 0.6666666865348816f;
-        const float t36 = t34 - t35;
-        const float t37 = z * t36;
-        const float t38 = t37 * 1.75f;
-        const float t39 = t32 * 0.75f;
-        const float t40 = t38 - t39;
-        const float t41 = z * t40;
-        const float t42 = t41 * 1.7999999523162842f;
-        const float t43 = t36 * 0.800000011920929f;
-        const float t44 = t42 - t43;
-        const float t45 = z * t44;
-        const float t46 = t45 * 1.8333333730697632f;
-        const float t47 = t40 * 0.8333333134651184f;
-        const float t48 = t46 - t47;
-        const float t49 = z * 3.0f;
-        const float t50 = z * t49;
-        const float t51 = t50 * 2.5f;
-        const float t52 = t51 - 1.5f;
-        const float t53 = z * t52;
-        const float t54 = t53 * 2.3333332538604736f;
-        const float t55 = t49 * 1.3333333730697632f;
-        const float t56 = t54 - t55;
-        const float t57 = z * t56;
-        const float t58 = t57 * 2.25f;
-        const float t59 = t52 * 1.25f;
-        const float t60 = t58 - t59;
-        const float t61 = z * t60;
-        const float t62 = t61 * 2.200000047683716f;
-        const float t63 = t56 * 1.2000000476837158f;
-        const float t64 = t62 - t63;
-        const float t65 = z * 3.0f;
-        const float t66 = t65 * 5.0f;
-        const float t67 = z * t66;
-        const float t68 = t67 * 3.5f;
-        const float t69 = t68 - 7.5f;
-        const float t70 = z * t69;
-        const float t71 = t70 * 3.0f;
-        const float t72 = t66 * 2.0f;
-        const float t73 = t71 - t72;
-        const float t74 = z * t73;
-        const float t75 = t74 * 2.75f;
-        const float t76 = t69 * 1.75f;
-        const float t77 = t75 - t76;
-        const float t78 = z * 15.0f;
-        const float t79 = t78 * 7.0f;
-        const float t80 = z * t79;
-        const float t81 = t80 * 4.5f;
-        const float t82 = t81 - 52.5f;
-        const float t83 = z * t82;
-        const float t84 = t83 * 3.6666667461395264f;
-        const float t85 = t79 * 2.6666667461395264f;
-        const float t86 = t84 - t85;
-        const float t87 = z * 105.0f;
-        const float t88 = t87 * 9.0f;
-        const float t89 = z * t88;
-        const float t90 = t89 * 5.5f;
-        const float t91 = t90 - 472.5f;
-        const float t92 = z * 945.0f;
-        const float t93 = t92 * 11.0f;
-        const float t94 = t49 * x;
-        const float t95 = t49 * y;
-        const float t96 = t2 * 3.0f;
-        const float t97 = t5 * 3.0f;
-        const float t98 = t52 * x;
-        const float t99 = t52 * y;
-        const float t100 = t66 * t2;
-        const float t101 = t66 * t5;
-        const float t102 = t8 * 15.0f;
-        const float t103 = t11 * 15.0f;
-        const float t104 = t56 * x;
-        const float t105 = t56 * y;
-        const float t106 = t69 * t2;
-        const float t107 = t69 * t5;
-        const float t108 = t79 * t8;
-        const float t109 = t79 * t11;
-        const float t110 = t14 * 105.0f;
-        const float t111 = t17 * 105.0f;
-        const float t112 = t60 * x;
-        const float t113 = t60 * y;
-        const float t114 = t73 * t2;
-        const float t115 = t73 * t5;
-        const float t116 = t82 * t8;
-        const float t117 = t82 * t11;
-        const float t118 = t88 * t14;
-        const float t119 = t88 * t17;
-        const float t120 = t20 * 945.0f;
-        const float t121 = t23 * 945.0f;
-        const float t122 = t64 * x;
-        const float t123 = t64 * y;
-        const float t124 = t77 * t2;
-        const float t125 = t77 * t5;
-        const float t126 = t86 * t8;
-        const float t127 = t86 * t11;
-        const float t128 = t91 * t14;
-        const float t129 = t91 * t17;
-        const float t130 = t93 * t20;
-        const float t131 = t93 * t23;
-        const float t132 = t26 * 10395.0f;
-        const float t133 = t29 * 10395.0f;
-        Y[0] = 1.0f;
-        Y[1] = y;
-        Y[2] = z;
-        Y[3] = x;
-        Y[4] = t97;
-        Y[5] = t95;
-        Y[6] = t32;
-        Y[7] = t94;
-        Y[8] = t96;
-        Y[9] = t103;
-        Y[10] = t101;
-        Y[11] = t99;
-        Y[12] = t36;
-        Y[13] = t98;
-        Y[14] = t100;
-        Y[15] = t102;
-        Y[16] = t111;
-        Y[17] = t109;
-        Y[18] = t107;
-        Y[19] = t105;
-        Y[20] = t40;
-        Y[21] = t104;
-        Y[22] = t106;
-        Y[23] = t108;
-        Y[24] = t110;
-        Y[25] = t121;
-        Y[26] = t119;
-        Y[27] = t117;
-        Y[28] = t115;
-        Y[29] = t113;
-        Y[30] = t44;
-        Y[31] = t112;
-        Y[32] = t114;
-        Y[33] = t116;
-        Y[34] = t118;
-        Y[35] = t120;
-        Y[36] = t133;
-        Y[37] = t131;
-        Y[38] = t129;
-        Y[39] = t127;
-        Y[40] = t125;
-        Y[41] = t123;
-        Y[42] = t48;
-        Y[43] = t122;
-        Y[44] = t124;
-        Y[45] = t126;
-        Y[46] = t128;
-        Y[47] = t130;
-        Y[48] = t132;
-    }
-    __device__ __forceinline__ static void ybar_vjp(float x, float y, float z, const float* w,
-                                                    float& gx, float& gy, float& gz) {
-        (void)x; (void)y; (void)z; (void)w;
-        const float t0 = x * x;
-        const float t1 = y * y;
-        const float t2 = t0 - t1;
-        const float t3 = x * y;
-        const float t4 = y * x;
-        const float t5 = t3 + t4;
-        const float t6 = x * t2;
-        const float t7 = y * t5;
-        const float t8 = t6 - t7;
-        const float t9 = x * t5;
-        const float t10 = y * t2;
-        const float t11 = t9 + t10;
-        const float t12 = x * t8;
-        const float t13 = y * t11;
-        const float t14 = t12 - t13;
-        const float t15 = x * t11;
-        const float t16 = y * t8;
-        const float t17 = t15 + t16;
-        const float t18 = x * t14;
-        const float t19 = y * t17;
-        const float t20 = t18 - t19;
-        const float t21 = x * t17;
-        const float t22 = y * t14;
-        const float t23 = t21 + t22;
-        const float t24 = x * t20;
-        const float t25 = y * t23;
-        const float t26 = t24 - t25;
-        const float t27 = x * t23;
-        const float t28 = y * t20;
-        const float t29 = t27 + t28;
-        const float t30 = z * z;
-        const float t31 = t30 * 1.5f;
-        const float t32 = t31 - 0.5f;
-        const float t33 = z * t32;
-        const float t34 = t33 * 1.6666666269302368f;
-        const float t35 = z * 0.6666666865348816f;
-        const float t36 = t34 - t35;
-        const float t37 = z * t36;
-        const float t38 = t37 * 1.75f;
-        const float t39 = t32 * 0.75f;
-        const float t40 = t38 - t39;
-        const float t41 = z * t40;
-        const float t42 = t41 * 1.7999999523162842f;
-        const float t43 = t36 * 0.800000011920929f;
-        const float t44 = t42 - t43;
-        const float t45 = z * t44;
-        const float t46 = t45 * 1.8333333730697632f;
-        const float t47 = t40 * 0.8333333134651184f;
-        const float t48 = t46 - t47;
-        const float t49 = z * 3.0f;
-        const float t50 = z * t49;
-        const float t51 = t50 * 2.5f;
-        const float t52 = t51 - 1.5f;
-        const float t53 = z * t52;
-        const float t54 = t53 * 2.3333332538604736f;
-        const float t55 = t49 * 1.3333333730697632f;
-        const float t56 = t54 - t55;
-        const float t57 = z * t56;
-        const float t58 = t57 * 2.25f;
-        const float t59 = t52 * 1.25f;
-        const float t60 = t58 - t59;
-        const float t61 = z * t60;
-        const float t62 = t61 * 2.200000047683716f;
-        const float t63 = t56 * 1.2000000476837158f;
-        const float t64 = t62 - t63;
-        const float t65 = z * 3.0f;
-        const float t66 = t65 * 5.0f;
-        const float t67 = z * t66;
-        const float t68 = t67 * 3.5f;
-        const float t69 = t68 - 7.5f;
-        const float t70 = z * t69;
-        const float t71 = t70 * 3.0f;
-        const float t72 = t66 * 2.0f;
-        const float t73 = t71 - t72;
-        const float t74 = z * t73;
-        const float t75 = t74 * 2.75f;
-        const float t76 = t69 * 1.75f;
-        const float t77 = t75 - t76;
-        const float t78 = z * 15.0f;
-        const float t79 = t78 * 7.0f;
-        const float t80 = z * t79;
-        const float t81 = t80 * 4.5f;
-        const float t82 = t81 - 52.5f;
-        const float t83 = z * t82;
-        const float t84 = t83 * 3.6666667461395264f;
-        const float t85 = t79 * 2.6666667461395264f;
-        const float t86 = t84 - t85;
-        const float t87 = z * 105.0f;
-        const float t88 = t87 * 9.0f;
-        const float t89 = z * t88;
-        const float t90 = t89 * 5.5f;
-        const float t91 = t90 - 472.5f;
-        const float t92 = z * 945.0f;
-        const float t93 = t92 * 11.0f;
-        const float t94 = t49 * x;
-        const float t95 = t49 * y;
-        const float t96 = t2 * 3.0f;
-        const float t97 = t5 * 3.0f;
-        const float t98 = t52 * x;
-        const float t99 = t52 * y;
-        const float t100 = t66 * t2;
-        const float t101 = t66 * t5;
-        const float t102 = t8 * 15.0f;
-        const float t103 = t11 * 15.0f;
-        const float t104 = t56 * x;
-        const float t105 = t56 * y;
-        const float t106 = t69 * t2;
-        const float t107 = t69 * t5;
-        const float t108 = t79 * t8;
-        const float t109 = t79 * t11;
-        const float t110 = t14 * 105.0f;
-        const float t111 = t17 * 105.0f;
-        const float t112 = t60 * x;
-        const float t113 = t60 * y;
-        const float t114 = t73 * t2;
-        const float t115 = t73 * t5;
-        const float t116 = t82 * t8;
-        const float t117 = t82 * t11;
-        const float t118 = t88 * t14;
-        const float t119 = t88 * t17;
-        const float t120 = t20 * 945.0f;
-        const float t121 = t23 * 945.0f;
-        const float t122 = t64 * x;
-        const float t123 = t64 * y;
-        const float t124 = t77 * t2;
-        const float t125 = t77 * t5;
-        const float t126 = t86 * t8;
-        const float t127 = t86 * t11;
-        const float t128 = t91 * t14;
-        const float t129 = t91 * t17;
-        const float t130 = t93 * t20;
-        const float t131 = t93 * t23;
-        const float t132 = t26 * 10395.0f;
-        const float t133 = t29 * 10395.0f;
-        const float a_t133 = w[36];
-        const float a_t132 = w[48];
-        const float a_t131 = w[37];
-        const float a_t130 = w[47];
-        const float a_t129 = w[38];
-        const float a_t128 = w[46];
-        const float a_t127 = w[39];
-        const float a_t126 = w[45];
-        const float a_t125 = w[40];
-        const float a_t124 = w[44];
-        const float a_t123 = w[41];
-        const float a_t122 = w[43];
-        const float a_t121 = w[25];
-        const float a_t120 = w[35];
-        const float a_t119 = w[26];
-        const float a_t118 = w[34];
-        const float a_t117 = w[27];
-        const float a_t116 = w[33];
-        const float a_t115 = w[28];
-        const float a_t114 = w[32];
-        const float a_t113 = w[29];
-        const float a_t112 = w[31];
-        const float a_t111 = w[16];
-        const float a_t110 = w[24];
-        const float a_t109 = w[17];
-        const float a_t108 = w[23];
-        const float a_t107 = w[18];
-        const float a_t106 = w[22];
-        const float a_t105 = w[19];
-        const float a_t104 = w[21];
-        const float a_t103 = w[9];
-        const float a_t102 = w[15];
-        const float a_t101 = w[10];
-        const float a_t100 = w[14];
-        const float a_t99 = w[11];
-        const float a_t98 = w[13];
-        const float a_t97 = w[4];
-        const float a_t96 = w[8];
-        const float a_t95 = w[5];
-        const float a_t94 = w[7];
-        const float a_t93 = t23 * a_t131 + t20 * a_t130;
-        const float a_t92 = 11.0f * a_t93;
-        const float a_t91 = t17 * a_t129 + t14 * a_t128;
-        const float a_t90 = a_t91;
-        const float a_t89 = 5.5f * a_t90;
-        const float a_t88 = t17 * a_t119 + t14 * a_t118 + z * a_t89;
-        const float a_t87 = 9.0f * a_t88;
-        const float a_t86 = t11 * a_t127 + t8 * a_t126;
-        const float a_t85 = -a_t86;
-        const float a_t84 = a_t86;
-        const float a_t83 = 3.6666667461395264f * a_t84;
-        const float a_t82 = t11 * a_t117 + t8 * a_t116 + z * a_t83;
-        const float a_t81 = a_t82;
-        const float a_t80 = 4.5f * a_t81;
-        const float a_t79 = t11 * a_t109 + t8 * a_t108 + 2.6666667461395264f * a_t85 + z * a_t80;
-        const float a_t78 = 7.0f * a_t79;
-        const float a_t77 = t5 * a_t125 + t2 * a_t124;
-        const float a_t76 = -a_t77;
-        const float a_t75 = a_t77;
-        const float a_t74 = 2.75f * a_t75;
-        const float a_t73 = t5 * a_t115 + t2 * a_t114 + z * a_t74;
-        const float a_t72 = -a_t73;
-        const float a_t71 = a_t73;
-        const float a_t70 = 3.0f * a_t71;
-        const float a_t69 = t5 * a_t107 + t2 * a_t106 + 1.75f * a_t76 + z * a_t70;
-        const float a_t68 = a_t69;
-        const float a_t67 = 3.5f * a_t68;
-        const float a_t66 = t5 * a_t101 + t2 * a_t100 + 2.0f * a_t72 + z * a_t67;
-        const float a_t65 = 5.0f * a_t66;
-        const float a_t64 = y * a_t123 + x * a_t122;
-        const float a_t63 = -a_t64;
-        const float a_t62 = a_t64;
-        const float a_t61 = 2.200000047683716f * a_t62;
-        const float a_t60 = y * a_t113 + x * a_t112 + z * a_t61;
-        const float a_t59 = -a_t60;
-        const float a_t58 = a_t60;
-        const float a_t57 = 2.25f * a_t58;
-        const float a_t56 = y * a_t105 + x * a_t104 + 1.2000000476837158f * a_t63 + z * a_t57;
-        const float a_t55 = -a_t56;
-        const float a_t54 = a_t56;
-        const float a_t53 = 2.3333332538604736f * a_t54;
-        const float a_t52 = y * a_t99 + x * a_t98 + 1.25f * a_t59 + z * a_t53;
-        const float a_t51 = a_t52;
-        const float a_t50 = 2.5f * a_t51;
-        const float a_t49 = y * a_t95 + x * a_t94 + 1.3333333730697632f * a_t55 + z * a_t50;
-        const float a_t48 = w[42];
-        const float a_t47 = -a_t48;
-        const float a_t46 = a_t48;
-        const float a_t45 = 1.8333333730697632f * a_t46;
-        const float a_t44 = w[30] + z * a_t45;
-        const float a_t43 = -a_t44;
-        const float a_t42 = a_t44;
-        const float a_t41 = 1.7999999523162842f * a_t42;
-        const float a_t40 = w[20] + 0.8333333134651184f * a_t47 + z * a_t41;
-        const float a_t39 = -a_t40;
-        const float a_t38 = a_t40;
-        const float a_t37 = 1.75f * a_t38;
-        const float a_t36 = w[12] + 0.800000011920929f * a_t43 + z * a_t37;
-        const float a_t35 = -a_t36;
-        const float a_t34 = a_t36;
-        const float a_t33 = 1.6666666269302368f * a_t34;
-        const float a_t32 = w[6] + 0.75f * a_t39 + z * a_t33;
-        const float a_t31 = a_t32;
-        const float a_t30 = 1.5f * a_t31;
-        const float a_t29 = 10395.0f * a_t133;
-        const float a_t28 = a_t29;
-        const float a_t27 = a_t29;
-        const float a_t26 = 10395.0f * a_t132;
-        const float a_t25 = -a_t26;
-        const float a_t24 = a_t26;
-        const float a_t23 = t93 * a_t131 + 945.0f * a_t121 + x * a_t27 + y * a_t25;
-        const float a_t22 = a_t23;
-        const float a_t21 = a_t23;
-        const float a_t20 = t93 * a_t130 + 945.0f * a_t120 + y * a_t28 + x * a_t24;
-        const float a_t19 = -a_t20;
-        const float a_t18 = a_t20;
-        const float a_t17 = t91 * a_t129 + t88 * a_t119 + 105.0f * a_t111 + x * a_t21 + y * a_t19;
-        const float a_t16 = a_t17;
-        const float a_t15 = a_t17;
-        const float a_t14 = t91 * a_t128 + t88 * a_t118 + 105.0f * a_t110 + y * a_t22 + x * a_t18;
-        const float a_t13 = -a_t14;
-        const float a_t12 = a_t14;
-        const float a_t11 = t86 * a_t127 + t82 * a_t117 + t79 * a_t109 + 15.0f * a_t103 + x * a_t15 + y * a_t13;
-        const float a_t10 = a_t11;
-        const float a_t9 = a_t11;
-        const float a_t8 = t86 * a_t126 + t82 * a_t116 + t79 * a_t108 + 15.0f * a_t102 + y * a_t16 + x * a_t12;
-        const float a_t7 = -a_t8;
-        const float a_t6 = a_t8;
-        const float a_t5 = t77 * a_t125 + t73 * a_t115 + t69 * a_t107 + t66 * a_t101 + 3.0f * a_t97 + x * a_t9 + y * a_t7;
-        const float a_t4 = a_t5;
-        const float a_t3 = a_t5;
-        const float a_t2 = t77 * a_t124 + t73 * a_t114 + t69 * a_t106 + t66 * a_t100 + 3.0f * a_t96 + y * a_t10 + x * a_t6;
-        const float a_t1 = -a_t2;
-        const float a_t0 = a_t2;
-        gx = w[3] + t64 * a_t122 + t60 * a_t112 + t56 * a_t104 + t52 * a_t98 + t49 * a_t94 + t23 * a_t27 + t20 * a_t24 + t17 * a_t21 + t14 * a_t18 + t11 * a_t15 + t8 * a_t12 + t5 * a_t9 + t2 * a_t6 + y * a_t4 + y * a_t3 + x * a_t0 + x * a_t0;
-        gy = w[1] + t64 * a_t123 + t60 * a_t113 + t56 * a_t105 + t52 * a_t99 + t49 * a_t95 + t20 * a_t28 + t23 * a_t25 + t14 * a_t22 + t17 * a_t19 + t8 * a_t16 + t11 * a_t13 + t2 * a_t10 + t5 * a_t7 + x * a_t4 + x * a_t3 + y * a_t1 + y * a_t1;
-        gz = w[2] + 945.0f * a_t92 + t88 * a_t89 + 105.0f * a_t87 + t82 * a_t83 + t79 * a_t80 + 15.0f * a_t78 + t73 * a_t74 + t69 * a_t70 + t66 * a_t67 + 3.0f * a_t65 + t60 * a_t61 + t56 * a_t57 + t52 * a_t53 + t49 * a_t50 + 3.0f * a_t49 + t44 * a_t45 + t40 * a_t41 + t36 * a_t37 + 0.6666666865348816f * a_t35 + t32 * a_t33 + z * a_t30 + z * a_t30;
     }
     static constexpr int LPS = 5;   // lane-pair product rule: node pairs
     static constexpr int LPQ = 5;   // ... and azimuth quads
@@ -2662,8 +1866,6 @@ static __constant__ float kLpTrig8[90] = {1.0f, 0.9914448857307434f, 0.130526185
 template <> struct SH<8> {
     static constexpr int K = 64;
     static constexpr int NNZ_SYM = 6588;   // entries (i, j <= k)
-    static constexpr int EZ = 16;    // projected-exponential rule: Gauss-Legendre nodes
-    static constexpr int EP = 32;    // projected-exponential rule: uniform azimuths
     __device__ __forceinline__ static float norm(int i) {
         switch (i) {
             case 0: return 0.282094806432724f;
@@ -2745,617 +1947,6 @@ template <> struct SH<8> {
             case 7: return 0.0f;
             default: return 0.0f;
         }
-    }
-    __device__ __forceinline__ static void ybar(float x, float y, float z, float* Y) {
-        (void)x; (void)y; (void)z;
-        const float t0 = x * x;
-        const float t1 = y * y;
-        const float t2 = t0 - t1;
-        const float t3 = x * y;
-        const float t4 = y * x;
-        const float t5 = t3 + t4;
-        const float t6 = x * t2;
-        const float t7 = y * t5;
-        const float t8 = t6 - t7;
-        const float t9 = x * t5;
-        const float t10 = y * t2;
-        const float t11 = t9 + t10;
-        const float t12 = x * t8;
-        const float t13 = y * t11;
-        const float t14 = t12 - t13;
-        const float t15 = x * t11;
-        const float t16 = y * t8;
-        const float t17 = t15 + t16;
-        const float t18 = x * t14;
-        const float t19 = y * t17;
-        const float t20 = t18 - t19;
-        const float t21 = x * t17;
-        const float t22 = y * t14;
-        const float t23 = t21 + t22;
-        const float t24 = x * t20;
-        const float t25 = y * t23;
-        const float t26 = t24 - t25;
-        const float t27 = x * t23;
-        const float t28 = y * t20;
-        const float t29 = t27 + t28;
-        const float t30 = x * t26;
-        const float t31 = y * t29;
-        const float t32 = t30 - t31;
-        const float t33 = x * t29;
-        const float t34 = y * t26;
-        const float t35 = t33 + t34;
-        const float t36 = z * z;
-        const float t37 = t36 * 1.5f;
-        const float t38 = t37 - 0.5f;
-        const float t39 = z * t38;
-        const float t40 = t39 * 1.6666666269302368f;
-        const float t41 = z * 0.6666666865348816f;
-        const float t42 = t40 - t41;
-        const float t43 = z * t42;
-        const float t44 = t43 * 1.75f;
-        const float t45 = t38 * 0.75f;
-        const float t46 = t44 - t45;
-        const float t47 = z * t46;
-        const float t48 = t47 * 1.7999999523162842f;
-        const float t49 = t42 * 0.800000011920929f;
-        const float t50 = t48 - t49;
-        const float t51 = z * t50;
-        const float t52 = t51 * 1.8333333730697632f;
-        const float t53 = t46 * 0.8333333134651184f;
-        const float t54 = t52 - t53;
-        const float t55 = z * t54;
-        const float t56 = t55 * 1.8571428060531616f;
-        const float t57 = t50 * 0.8571428656578064f;
-        const float t58 = t56 - t57;
-        const float t59 = z * 3.0f;
-        const float t60 = z * t59;
-        const float t61 = t60 * 2.5f;
-        const float t62 = t61 - 1.5f;
-        const float t63 = z * t62;
-        const float t64 = t63 * 2.3333332538604736f;
-        const float t65 = t59 * 1.3333333730697632f;
-        const float t66 = t64 - t65;
-        const float t67 = z * t66;
-        const float t68 = t67 * 2.25f;
-        const float t69 = t62 * 1.25f;
-        const float t70 = t68 - t69;
-        const float t71 = z * t70;
-        const float t72 = t71 * 2.200000047683716f;
-        const float t73 = t66 * 1.2000000476837158f;
-        const float t74 = t72 - t73;
-        const float t75 = z * t74;
-        const float t76 = t75 * 2.1666667461395264f;
-        const float t77 = t70 * 1.1666666269302368f;
-        const float t78 = t76 - t77;
-        const float t79 = z * 3.0f;
-        const float t80 = t79 * 5.0f;
-        const float t81 = z * t80;
-        const float t82 = t81 * 3.5f;
-        const float t83 = t82 - 7.5f;
-        const float t84 = z * t83;
-        const float t85 = t84 * 3.0f;
-        const float t86 = t80 * 2.0f;
-        const float t87 = t85 - t86;
-        const float t88 = z * t87;
-        const float t89 = t88 * 2.75f;
-        const float t90 = t83 * 1.75f;
-        const float t91 = t89 - t90;
-        const float t92 = z * t91;
-        const float t93 = t92 * 2.5999999046325684f;
-        const float t94 = t87 * 1.600000023841858f;
-        const float t95 = t93 - t94;
-        const float t96 = z * 15.0f;
-        const float t97 = t96 * 7.0f;
-        const float t98 = z * t97;
-        const float t99 = t98 * 4.5f;
-        const float t100 = t99 - 52.5f;
-        const float t101 = z * t100;
-        const float t102 = t101 * 3.6666667461395264f;
-        const float t103 = t97 * 2.6666667461395264f;
-        const float t104 = t102 - t103;
-        const float t105 = z * t104;
-        const float t106 = t105 * 3.25f;
-        const float t107 = t100 * 2.25f;
-        const float t108 = t106 - t107;
-        const float t109 = z * 105.0f;
-        const float t110 = t109 * 9.0f;
-        const float t111 = z * t110;
-        const float t112 = t111 * 5.5f;
-        const float t113 = t112 - 472.5f;
-        const float t114 = z * t113;
-        const float t115 = t114 * 4.333333492279053f;
-        const float t116 = t110 * 3.3333332538604736f;
-        const float t117 = t115 - t116;
-        const float t118 = z * 945.0f;
-        const float t119 = t118 * 11.0f;
-        const float t120 = z * t119;
-        const float t121 = t120 * 6.5f;
-        const float t122 = t121 - 5197.5f;
-        const float t123 = z * 10395.0f;
-        const float t124 = t123 * 13.0f;
-        const float t125 = t59 * x;
-        const float t126 = t59 * y;
-        const float t127 = t2 * 3.0f;
-        const float t128 = t5 * 3.0f;
-        const float t129 = t62 * x;
-        const float t130 = t62 * y;
-        const float t131 = t80 * t2;
-        const float t132 = t80 * t5;
-        const float t133 = t8 * 15.0f;
-        const float t134 = t11 * 15.0f;
-        const float t135 = t66 * x;
-        const float t136 = t66 * y;
-        const float t137 = t83 * t2;
-        const float t138 = t83 * t5;
-        const float t139 = t97 * t8;
-        const float t140 = t97 * t11;
-        const float t141 = t14 * 105.0f;
-        const float t142 = t17 * 105.0f;
-        const float t143 = t70 * x;
-        const float t144 = t70 * y;
-        const float t145 = t87 * t2;
-        const float t146 = t87 * t5;
-        const float t147 = t100 * t8;
-        const float t148 = t100 * t11;
-        const float t149 = t110 * t14;
-        const float t150 = t110 * t17;
-        const float t151 = t20 * 945.0f;
-        const float t152 = t23 * 945.0f;
-        const float t153 = t74 * x;
-        const float t154 = t74 * y;
-        const float t155 = t91 * t2;
-        const float t156 = t91 * t5;
-        const float t157 = t104 * t8;
-        const float t158 = t104 * t11;
-        const float t159 = t113 * t14;
-        const float t160 = t113 * t17;
-        const float t161 = t119 * t20;
-        const float t162 = t119 * t23;
-        const float t163 = t26 * 10395.0f;
-        const float t164 = t29 * 10395.0f;
-        const float t165 = t78 * x;
-        const float t166 = t78 * y;
-        const float t167 = t95 * t2;
-        const float t168 = t95 * t5;
-        const float t169 = t108 * t8;
-        const float t170 = t108 * t11;
-        const float t171 = t117 * t14;
-        const float t172 = t117 * t17;
-        const float t173 = t122 * t20;
-        const float t174 = t122 * t23;
-        const float t175 = t124 * t26;
-        const float t176 = t124 * t29;
-        const float t177 = t32 * 135135.0f;
-        const float t178 = t35 * 135135.0f;
-        Y[0] = 1.0f;
-        Y[1] = y;
-        Y[2] = z;
-        Y[3] = x;
-        Y[4] = t128;
-        Y[5] = t126;
-        Y[6] = t38;
-        Y[7] = t125;
-        Y[8] = t127;
-        Y[9] = t134;
-        Y[10] = t132;
-        Y[11] = t130;
-        Y[12] = t42;
-        Y[13] = t129;
-        Y[14] = t131;
-        Y[15] = t133;
-        Y[16] = t142;
-        Y[17] = t140;
-        Y[18] = t138;
-        Y[19] = t136;
-        Y[20] = t46;
-        Y[21] = t135;
-        Y[22] = t137;
-        Y[23] = t139;
-        Y[24] = t141;
-        Y[25] = t152;
-        Y[26] = t150;
-        Y[27] = t148;
-        Y[28] = t146;
-        Y[29] = t144;
-        Y[30] = t50;
-        Y[31] = t143;
-        Y[32] = t145;
-        Y[33] = t147;
-        Y[34] = t149;
-        Y[35] = t151;
-        Y[36] = t164;
-        Y[37] = t162;
-        Y[38] = t160;
-        Y[39] = t158;
-        Y[40] = t156;
-        Y[41] = t154;
-        Y[42] = t54;
-        Y[43] = t153;
-        Y[44] = t155;
-        Y[45] = t157;
-        Y[46] = t159;
-        Y[47] = t161;
-        Y[48] = t163;
-        Y[49] = t178;
-        Y[50] = t176;
-        Y[51] = t174;
-        Y[52] = t172;
-        Y[53] = t170;
-        Y[54] = t168;
-        Y[55] = t166;
-        Y[56] = t58;
-        Y[57] = t165;
-        Y[58] = t167;
-        Y[59] = t169;
-        Y[60] = t171;
-        Y[61] = t173;
-        Y[62] = t175;
-        Y[63] = t177;
-    }
-    __device__ __forceinline__ static void ybar_vjp(float x, float y, float z, const float* w,
-                                                    float& gx, float& gy, float& gz) {
-        (void)x; (void)y; (void)z; (void)w;
-        const float t0 = x * x;
-        const float t1 = y * y;
-        const float t2 = t0 - t1;
-        const float t3 = x * y;
-        const float t4 = y * x;
-        const float t5 = t3 + t4;
-        const float t6 = x * t2;
-        const float t7 = y * t5;
-        const float t8 = t6 - t7;
-        const float t9 = x * t5;
-        const float t10 = y * t2;
-        const float t11 = t9 + t10;
-        const float t12 = x * t8;
-        const float t13 = y * t11;
-        const float t14 = t12 - t13;
-        const float t15 = x * t11;
-        const float t16 = y * t8;
-        const float t17 = t15 + t16;
-        const float t18 = x * t14;
-        const float t19 = y * t17;
-        const float t20 = t18 - t19;
-        const float t21 = x * t17;
-        const float t22 = y * t14;
-        const float t23 = t21 + t22;
-        const float t24 = x * t20;
-        const float t25 = y * t23;
-        const float t26 = t24 - t25;
-        const float t27 = x * t23;
-        const float t28 = y * t20;
-        const float t29 = t27 + t28;
-        const float t30 = x * t26;
-        const float t31 = y * t29;
-        const float t32 = t30 - t31;
-        const float t33 = x * t29;
-        const float t34 = y * t26;
-        const float t35 = t33 + t34;
-        const float t36 = z * z;
-        const float t37 = t36 * 1.5f;
-        const float t38 = t37 - 0.5f;
-        const float t39 = z * t38;
-        const float t40 = t39 * 1.6666666269302368f;
-        const float t41 = z * 0.6666666865348816f;
-        const float t42 = t40 - t41;
-        const float t43 = z * t42;
-        const float t44 = t43 * 1.75f;
-        const float t45 = t38 * 0.75f;
-        const float t46 = t44 - t45;
-        const float t47 = z * t46;
-        const float t48 = t47 * 1.7999999523162842f;
-        const float t49 = t42 * 0.800000011920929f;
-        const float t50 = t48 - t49;
-        const float t51 = z * t50;
-        const float t52 = t51 * 1.8333333730697632f;
-        const float t53 = t46 * 0.8333333134651184f;
-        const float t54 = t52 - t53;
-        const float t55 = z * t54;
-        const float t56 = t55 * 1.8571428060531616f;
-        const float t57 = t50 * 0.8571428656578064f;
-        const float t58 = t56 - t57;
-        const float t59 = z * 3.0f;
-        const float t60 = z * t59;
-        const float t61 = t60 * 2.5f;
-        const float t62 = t61 - 1.5f;
-        const float t63 = z * t62;
-        const float t64 = t63 * 2.3333332538604736f;
-        const float t65 = t59 * 1.3333333730697632f;
-        const float t66 = t64 - t65;
-        const float t67 = z * t66;
-        const float t68 = t67 * 2.25f;
-        const float t69 = t62 * 1.25f;
-        const float t70 = t68 - t69;
-        const float t71 = z * t70;
-        const float t72 = t71 * 2.200000047683716f;
-        const float t73 = t66 * 1.2000000476837158f;
-        const float t74 = t72 - t73;
-        const float t75 = z * t74;
-        const float t76 = t75 * 2.1666667461395264f;
-        const float t77 = t70 * 1.1666666269302368f;
-        const float t78 = t76 - t77;
-        const float t79 = z * 3.0f;
-        const float t80 = t79 * 5.0f;
-        const float t81 = z * t80;
-        const float t82 = t81 * 3.5f;
-        const float t83 = t82 - 7.5f;
-        const float t84 = z * t83;
-        const float t85 = t84 * 3.0f;
-        const float t86 = t80 * 2.0f;
-        const float t87 = t85 - t86;
-        const float t88 = z * t87;
-        const float t89 = t88 * 2.75f;
-        const float t90 = t83 * 1.75f;
-        const float t91 = t89 - t90;
-        const float t92 = z * t91;
-        const float t93 = t92 * 2.5999999046325684f;
-        const float t94 = t87 * 1.600000023841858f;
-        const float t95 = t93 - t94;
-        const float t96 = z * 15.0f;
-        const float t97 = t96 * 7.0f;
-        const float t98 = z * t97;
-        const float t99 = t98 * 4.5f;
-        const float t100 = t99 - 52.5f;
-        const float t101 = z * t100;
-        const float t102 = t101 * 3.6666667461395264f;
-        const float t103 = t97 * 2.6666667461395264f;
-        const float t104 = t102 - t103;
-        const float t105 = z * t104;
-        const float t106 = t105 * 3.25f;
-        const float t107 = t100 * 2.25f;
-        const float t108 = t106 - t107;
-        const float t109 = z * 105.0f;
-        const float t110 = t109 * 9.0f;
-        const float t111 = z * t110;
-        const float t112 = t111 * 5.5f;
-        const float t113 = t112 - 472.5f;
-        const float t114 = z * t113;
-        const float t115 = t114 * 4.333333492279053f;
-        const float t116 = t110 * 3.3333332538604736f;
-        const float t117 = t115 - t116;
-        const float t118 = z * 945.0f;
-        const float t119 = t118 * 11.0f;
-        const float t120 = z * t119;
-        const float t121 = t120 * 6.5f;
-        const float t122 = t121 - 5197.5f;
-        const float t123 = z * 10395.0f;
-        const float t124 = t123 * 13.0f;
-        const float t125 = t59 * x;
-        const float t126 = t59 * y;
-        const float t127 = t2 * 3.0f;
-        const float t128 = t5 * 3.0f;
-        const float t129 = t62 * x;
-        const float t130 = t62 * y;
-        const float t131 = t80 * t2;
-        const float t132 = t80 * t5;
-        const float t133 = t8 * 15.0f;
-        const float t134 = t11 * 15.0f;
-        const float t135 = t66 * x;
-        const float t136 = t66 * y;
-        const float t137 = t83 * t2;
-        const float t138 = t83 * t5;
-        const float t139 = t97 * t8;
-        const float t140 = t97 * t11;
-        const float t141 = t14 * 105.0f;
-        const float t142 = t17 * 105.0f;
-        const float t143 = t70 * x;
-        const float t144 = t70 * y;
-        const float t145 = t87 * t2;
-        const float t146 = t87 * t5;
-        const float t147 = t100 * t8;
-        const float t148 = t100 * t11;
-        const float t149 = t110 * t14;
-        const float t150 = t110 * t17;
-        const float t151 = t20 * 945.0f;
-        const float t152 = t23 * 945.0f;
-        const float t153 = t74 * x;
-        const float t154 = t74 * y;
-        const float t155 = t91 * t2;
-        const float t156 = t91 * t5;
-        const float t157 = t104 * t8;
-        const float t158 = t104 * t11;
-        const float t159 = t113 * t14;
-        const float t160 = t113 * t17;
-        const float t161 = t119 * t20;
-        const float t162 = t119 * t23;
-        const float t163 = t26 * 10395.0f;
-        const float t164 = t29 * 10395.0f;
-        const float t165 = t78 * x;
-        const float t166 = t78 * y;
-        const float t167 = t95 * t2;
-        const float t168 = t95 * t5;
-        const float t169 = t108 * t8;
-        const float t170 = t108 * t11;
-        const float t171 = t117 * t14;
-        const float t172 = t117 * t17;
-        const float t173 = t122 * t20;
-        const float t174 = t122 * t23;
-        const float t175 = t124 * t26;
-        const float t176 = t124 * t29;
-        const float t177 = t32 * 135135.0f;
-        const float t178 = t35 * 135135.0f;
-        const float a_t178 = w[49];
-        const float a_t177 = w[63];
-        const float a_t176 = w[50];
-        const float a_t175 = w[62];
-        const float a_t174 = w[51];
-        const float a_t173 = w[61];
-        const float a_t172 = w[52];
-        const float a_t171 = w[60];
-        const float a_t170 = w[53];
-        const float a_t169 = w[59];
-        const float a_t168 = w[54];
-        const float a_t167 = w[58];
-        const float a_t166 = w[55];
-        const float a_t165 = w[57];
-        const float a_t164 = w[36];
-        const float a_t163 = w[48];
-        const float a_t162 = w[37];
-        const float a_t161 = w[47];
-        const float a_t160 = w[38];
-        const float a_t159 = w[46];
-        const float a_t158 = w[39];
-        const float a_t157 = w[45];
-        const float a_t156 = w[40];
-        const float a_t155 = w[44];
-        const float a_t154 = w[41];
-        const float a_t153 = w[43];
-        const float a_t152 = w[25];
-        const float a_t151 = w[35];
-        const float a_t150 = w[26];
-        const float a_t149 = w[34];
-        const float a_t148 = w[27];
-        const float a_t147 = w[33];
-        const float a_t146 = w[28];
-        const float a_t145 = w[32];
-        const float a_t144 = w[29];
-        const float a_t143 = w[31];
-        const float a_t142 = w[16];
-        const float a_t141 = w[24];
-        const float a_t140 = w[17];
-        const float a_t139 = w[23];
-        const float a_t138 = w[18];
-        const float a_t137 = w[22];
-        const float a_t136 = w[19];
-        const float a_t135 = w[21];
-        const float a_t134 = w[9];
-        const float a_t133 = w[15];
-        const float a_t132 = w[10];
-        const float a_t131 = w[14];
-        const float a_t130 = w[11];
-        const float a_t129 = w[13];
-        const float a_t128 = w[4];
-        const float a_t127 = w[8];
-        const float a_t126 = w[5];
-        const float a_t125 = w[7];
-        const float a_t124 = t29 * a_t176 + t26 * a_t175;
-        const float a_t123 = 13.0f * a_t124;
-        const float a_t122 = t23 * a_t174 + t20 * a_t173;
-        const float a_t121 = a_t122;
-        const float a_t120 = 6.5f * a_t121;
-        const float a_t119 = t23 * a_t162 + t20 * a_t161 + z * a_t120;
-        const float a_t118 = 11.0f * a_t119;
-        const float a_t117 = t17 * a_t172 + t14 * a_t171;
-        const float a_t116 = -a_t117;
-        const float a_t115 = a_t117;
-        const float a_t114 = 4.333333492279053f * a_t115;
-        const float a_t113 = t17 * a_t160 + t14 * a_t159 + z * a_t114;
-        const float a_t112 = a_t113;
-        const float a_t111 = 5.5f * a_t112;
-        const float a_t110 = t17 * a_t150 + t14 * a_t149 + 3.3333332538604736f * a_t116 + z * a_t111;
-        const float a_t109 = 9.0f * a_t110;
-        const float a_t108 = t11 * a_t170 + t8 * a_t169;
-        const float a_t107 = -a_t108;
-        const float a_t106 = a_t108;
-        const float a_t105 = 3.25f * a_t106;
-        const float a_t104 = t11 * a_t158 + t8 * a_t157 + z * a_t105;
-        const float a_t103 = -a_t104;
-        const float a_t102 = a_t104;
-        const float a_t101 = 3.6666667461395264f * a_t102;
-        const float a_t100 = t11 * a_t148 + t8 * a_t147 + 2.25f * a_t107 + z * a_t101;
-        const float a_t99 = a_t100;
-        const float a_t98 = 4.5f * a_t99;
-        const float a_t97 = t11 * a_t140 + t8 * a_t139 + 2.6666667461395264f * a_t103 + z * a_t98;
-        const float a_t96 = 7.0f * a_t97;
-        const float a_t95 = t5 * a_t168 + t2 * a_t167;
-        const float a_t94 = -a_t95;
-        const float a_t93 = a_t95;
-        const float a_t92 = 2.5999999046325684f * a_t93;
-        const float a_t91 = t5 * a_t156 + t2 * a_t155 + z * a_t92;
-        const float a_t90 = -a_t91;
-        const float a_t89 = a_t91;
-        const float a_t88 = 2.75f * a_t89;
-        const float a_t87 = t5 * a_t146 + t2 * a_t145 + 1.600000023841858f * a_t94 + z * a_t88;
-        const float a_t86 = -a_t87;
-        const float a_t85 = a_t87;
-        const float a_t84 = 3.0f * a_t85;
-        const float a_t83 = t5 * a_t138 + t2 * a_t137 + 1.75f * a_t90 + z * a_t84;
-        const float a_t82 = a_t83;
-        const float a_t81 = 3.5f * a_t82;
-        const float a_t80 = t5 * a_t132 + t2 * a_t131 + 2.0f * a_t86 + z * a_t81;
-        const float a_t79 = 5.0f * a_t80;
-        const float a_t78 = y * a_t166 + x * a_t165;
-        const float a_t77 = -a_t78;
-        const float a_t76 = a_t78;
-        const float a_t75 = 2.1666667461395264f * a_t76;
-        const float a_t74 = y * a_t154 + x * a_t153 + z * a_t75;
-        const float a_t73 = -a_t74;
-        const float a_t72 = a_t74;
-        const float a_t71 = 2.200000047683716f * a_t72;
-        const float a_t70 = y * a_t144 + x * a_t143 + 1.1666666269302368f * a_t77 + z * a_t71;
-        const float a_t69 = -a_t70;
-        const float a_t68 = a_t70;
-        const float a_t67 = 2.25f * a_t68;
-        const float a_t66 = y * a_t136 + x * a_t135 + 1.2000000476837158f * a_t73 + z * a_t67;
-        const float a_t65 = -a_t66;
-        const float a_t64 = a_t66;
-        const float a_t63 = 2.3333332538604736f * a_t64;
-        const float a_t62 = y * a_t130 + x * a_t129 + 1.25f * a_t69 + z * a_t63;
-        const float a_t61 = a_t62;
-        const float a_t60 = 2.5f * a_t61;
-        const float a_t59 = y * a_t126 + x * a_t125 + 1.3333333730697632f * a_t65 + z * a_t60;
-        const float a_t58 = w[56];
-        const float a_t57 = -a_t58;
-        const float a_t56 = a_t58;
-        const float a_t55 = 1.8571428060531616f * a_t56;
-        const float a_t54 = w[42] + z * a_t55;
-        const float a_t53 = -a_t54;
-        const float a_t52 = a_t54;
-        const float a_t51 = 1.8333333730697632f * a_t52;
-        const float a_t50 = w[30] + 0.8571428656578064f * a_t57 + z * a_t51;
-        const float a_t49 = -a_t50;
-        const float a_t48 = a_t50;
-        const float a_t47 = 1.7999999523162842f * a_t48;
-        const float a_t46 = w[20] + 0.8333333134651184f * a_t53 + z * a_t47;
-        const float a_t45 = -a_t46;
-        const float a_t44 = a_t46;
-        const float a_t43 = 1.75f * a_t44;
-        const float a_t42 = w[12] + 0.800000011920929f * a_t49 + z * a_t43;
-        const float a_t41 = -a_t42;
-        const float a_t40 = a_t42;
-        const float a_t39 = 1.6666666269302368f * a_t40;
-        const float a_t38 = w[6] + 0.75f * a_t45 + z * a_t39;
-        const float a_t37 = a_t38;
-        const float a_t36 = 1.5f * a_t37;
-        const float a_t35 = 135135.0f * a_t178;
-        const float a_t34 = a_t35;
-        const float a_t33 = a_t35;
-        const float a_t32 = 135135.0f * a_t177;
-        const float a_t31 = -a_t32;
-        const float a_t30 = a_t32;
-        const float a_t29 = t124 * a_t176 + 10395.0f * a_t164 + x * a_t33 + y * a_t31;
-        const float a_t28 = a_t29;
-        const float a_t27 = a_t29;
-        const float a_t26 = t124 * a_t175 + 10395.0f * a_t163 + y * a_t34 + x * a_t30;
-        const float a_t25 = -a_t26;
-        const float a_t24 = a_t26;
-        const float a_t23 = t122 * a_t174 + t119 * a_t162 + 945.0f * a_t152 + x * a_t27 + y * a_t25;
-        const float a_t22 = a_t23;
-        const float a_t21 = a_t23;
-        const float a_t20 = t122 * a_t173 + t119 * a_t161 + 945.0f * a_t151 + y * a_t28 + x * a_t24;
-        const float a_t19 = -a_t20;
-        const float a_t18 = a_t20;
-        const float a_t17 = t117 * a_t172 + t113 * a_t160 + t110 * a_t150 + 105.0f * a_t142 + x * a_t21 + y * a_t19;
-        const float a_t16 = a_t17;
-        const float a_t15 = a_t17;
-        const float a_t14 = t117 * a_t171 + t113 * a_t159 + t110 * a_t149 + 105.0f * a_t141 + y * a_t22 + x * a_t18;
-        const float a_t13 = -a_t14;
-        const float a_t12 = a_t14;
-        const float a_t11 = t108 * a_t170 + t104 * a_t158 + t100 * a_t148 + t97 * a_t140 + 15.0f * a_t134 + x * a_t15 + y * a_t13;
-        const float a_t10 = a_t11;
-        const float a_t9 = a_t11;
-        const float a_t8 = t108 * a_t169 + t104 * a_t157 + t100 * a_t147 + t97 * a_t139 + 15.0f * a_t133 + y * a_t16 + x * a_t12;
-        const float a_t7 = -a_t8;
-        const float a_t6 = a_t8;
-        const float a_t5 = t95 * a_t168 + t91 * a_t156 + t87 * a_t146 + t83 * a_t138 + t80 * a_t132 + 3.0f * a_t128 + x * a_t9 + y * a_t7;
-        const float a_t4 = a_t5;
-        const float a_t3 = a_t5;
-        const float a_t2 = t95 * a_t167 + t91 * a_t155 + t87 * a_t145 + t83 * a_t137 + t80 * a_t131 + 3.0f * a_t127 + y * a_t10 + x * a_t6;
-        const float a_t1 = -a_t2;
-        const float a_t0 = a_t2;
-        gx = w[3] + t78 * a_t165 + t74 * a_t153 + t70 * a_t143 + t66 * a_t135 + t62 * a_t129 + t59 * a_t125 + t29 * a_t33 + t26 * a_t30 + t23 * a_t27 + t20 * a_t24 + t17 * a_t21 + t14 * a_t18 + t11 * a_t15 + t8 * a_t12 + t5 * a_t9 + t2 * a_t6 + y * a_t4 + y * a_t3 + x * a_t0 + x * a_t0;
-        gy = w[1] + t78 * a_t166 + t74 * a_t154 + t70 * a_t144 + t66 * a_t136 + t62 * a_t130 + t59 * a_t126 + t26 * a_t34 + t29 * a_t31 + t20 * a_t28 + t23 * a_t25 + t14 * a_t22 + t17 * a_t19 + t8 * a_t16 + t11 * a_t13 + t2 * a_t10 + t5 * a_t7 + x * a_t4 + x * a_t3 + y * a_t1 + y * a_t1;
-        gz = w[2] + 10395.0f * a_t123 + t119 * a_t120 + 945.0f * a_t118 + t113 * a_t114 + t110 * a_t111 + 105.0f * a_t109 + t104 * a_t105 + t100 * a_t101 + t97 * a_t98 + 15.0f * a_t96 + t91 * a_t92 + t87 * a_t88 + t83 * a_t84 + t80 * a_t81 + 3.0f * a_t79 + t74 * a_t75 + t70 * a_t71 + t66 * a_t67 + t62 * a_t63 + t59 * a_t60 + 3.0f * a_t59 + t54 * a_t55 + t50 * a_t51 + t46 * a_t47 + t42 * a_t43 + 0.6666666865348816f * a_t41 + t38 * a_t39 + z * a_t36 + z * a_t36;
     }
     static constexpr int LPS = 6;   // lane-pair product rule: node pairs
     static constexpr int LPQ = 6;   // ... and azimuth quads
