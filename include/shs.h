@@ -251,10 +251,9 @@ shs_status shs_noalloc_device_status(void* stream, int32_t* device_status);
 /* ---- Batched shading for serving many jobs (continuous batching) ----------
  * A batch call runs the forward pass (Eq. 8) of up to 32 requests, each on its
  * own resident scene, and the L2 adjoint (as shs_shade_backward_l2) of those
- * that carry a target, in one persistent launch per band count and pass (from 6
- * bands also per horizon_cull and projected-exponential setting): the requests'
- * tiles form one work list that the resident blocks drain through a device
- * counter.  The paper runs one scene per call; this is
+ * that carry a target, in one persistent launch per band count and pass: the
+ * requests' tiles form one work list that the resident blocks drain through a
+ * device counter.  The paper runs one scene per call; this is
  * the serving form of the same computation (Sec. 3.5's analysis-by-synthesis
  * iterations of many jobs at once). */
 typedef struct shs_batch_s* shs_batch_t;

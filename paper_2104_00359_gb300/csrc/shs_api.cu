@@ -117,7 +117,7 @@ struct shs_scene_s {
 };
 
 struct shs_batch_s {
-    unsigned int* queues;  // [64] tile counters: forward / backward x n_bands x variant
+    unsigned int* queues;  // [16] tile counters: forward / backward x n_bands
 };
 
 namespace {
@@ -210,8 +210,6 @@ SceneView view_of(const shs_scene_s* s) {
 }
 
 size_t batch_acc_bytes(const shs_scene_s* s) { return sizeof(float) * s->partial_stride + sizeof(double); }
-
-int variant_of(const shs_scene_s* s) { return shs::batch_variant(view_of(s), s->cfg.n_bands); }
 
 bool tensor_core_precision(const shs_config& c) { return c.precision != SHS_FP32; }
 
@@ -932,7 +930,7 @@ shs_status shs_batch_create(shs_batch_t* out) {
     *out = nullptr;
     shs_batch_s* b = new (std::nothrow) shs_batch_s();
     if (!b) return fail(SHS_ERR_OOM, "host allocation failed");
-    cudaError_t e = cudaMalloc(&b->queues, 64 * sizeof(unsigned int));
+    cudaError_t e = cudaMalloc(&b->queues, 16 * sizeof(unsigned int));
     if (e != cudaSuccess) {
         delete b;
         return cuda_fail(e, "allocate batch queues");
@@ -973,22 +971,20 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
                 return fail(SHS_ERR_INVALID_ARG, "requests %d and %d share a scene", j, i);
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(batch->queues, 0, 64 * sizeof(unsigned int), s);
+    cudaError_t e = cudaMemsetAsync(batch->queues, 0, 16 * sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_fail(e, "reset batch queues");
-    for (int g = 0; g < 32 && e == cudaSuccess; ++g) {
-        const int nb = g / 4 + 1, variant = g % 4;
-        if (variant >= shs::batch_variants(nb)) continue;
+    for (int nb = 1; nb <= 8 && e == cudaSuccess; ++nb) {
         shs::FwdBatch fb;
         fb.n = 0;
         fb.total_tiles = 0;
-        fb.variant = variant;
-        fb.queue = batch->queues + g;
+        fb.queue = batch->queues + (nb - 1);
         for (int i = 0; i < n_reqs; ++i) {
             const shs_request& r = reqs[i];
-            if (r.scene->cfg.n_bands != nb || variant_of(r.scene) != variant || r.n_points == 0 || !r.radiance) continue;
+            if (r.scene->cfg.n_bands != nb || r.n_points == 0 || !r.radiance) continue;
             shs::FwdArgs& a = fb.r[fb.n];
             a = shs::FwdArgs{};
             a.sc = view_of(r.scene);
+            fb.variant.add(a.sc);
             a.n_points = r.n_points;
             a.points = r.points;
             a.normals = r.normals;
@@ -1002,19 +998,16 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
         fb.tile_begin[fb.n] = fb.total_tiles;
         if (fb.n) e = dispatch<FwdB>(nb, fb, s);
     }
-    for (int g = 0; g < 32 && e == cudaSuccess; ++g) {
-        const int nb = g / 4 + 1, variant = g % 4;
-        if (variant >= shs::batch_variants(nb)) continue;
+    for (int nb = 1; nb <= 8 && e == cudaSuccess; ++nb) {
         shs::BwdBatch bb;
         bb.n = 0;
         bb.max_spheres = 0;
         bb.total_tiles = 0;
-        bb.variant = variant;
-        bb.queue = batch->queues + 32 + g;
+        bb.queue = batch->queues + 8 + (nb - 1);
         for (int i = 0; i < n_reqs && e == cudaSuccess; ++i) {
             const shs_request& r = reqs[i];
             shs_scene_s* sc = r.scene;
-            if (sc->cfg.n_bands != nb || variant_of(sc) != variant || (!r.target && !r.d_radiance)) continue;
+            if (sc->cfg.n_bands != nb || (!r.target && !r.d_radiance)) continue;
             if (r.n_points == 0) {
                 if (r.d_light) e = cudaMemsetAsync(r.d_light, 0, sizeof(float) * 3 * sc->K, s);
                 if (e == cudaSuccess && r.d_centers && sc->n_spheres) e = cudaMemsetAsync(r.d_centers, 0, sizeof(float) * 3 * sc->n_spheres, s);
@@ -1025,6 +1018,7 @@ shs_status shs_shade_batch(shs_batch_t batch, const shs_request* reqs, int32_t n
             shs::BwdArgs& a = bb.r[bb.n];
             a = shs::BwdArgs{};
             a.sc = view_of(sc);
+            bb.variant.add(a.sc);
             a.n_points = r.n_points;
             a.points = r.points;
             a.normals = r.normals;

@@ -115,6 +115,20 @@ __device__ __forceinline__ void lp_store(const float* v, int64_t P, int64_t p, c
     });
 }
 
+// The exponential a kernel is compiled for; kExpAny: asked of each scene.
+constexpr int kExpSquarings = 0, kExpProjected = 1, kExpAny = 2;
+template <int EXPM>
+__device__ __forceinline__ bool projected_exp(const SceneView& sc) {
+    return EXPM == kExpAny ? sc.exp_mode == 1 : EXPM == kExpProjected;
+}
+
+// Unit normal for a kernel compiled with culling: a scene that does not cull
+// gets NaN, which no sphere's test is below.
+__device__ __forceinline__ Normal cull_normal(const SceneView& sc, float nx, float ny, float nz) {
+    const float off = __int_as_float(0x7fffffff);
+    return sc.horizon_cull ? unit_normal(nx, ny, nz) : Normal{off, off, off};
+}
+
 // Log-visibility f of the lane pair's point: each lane sums every second
 // sphere, then the lanes exchange halves and keep their own slots.
 template <bool CULL>

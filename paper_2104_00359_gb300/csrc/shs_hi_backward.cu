@@ -162,9 +162,10 @@ struct BwdShared {
 // Adjoint of the exponential and the shading at the lane pair's point: the
 // per-point outputs, the lighting and loss sums, and dLoss/df_i (-2 pi eps)
 // NORM_i of the lane's slots in dfp.
-template <bool EXP, bool CULL>
+template <int EXPM, bool CULL>
 __device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShared& sh, int64_t p, float* dfp) {
     const LanePair lp = lane_pair();
+    const bool projected = projected_exp<EXPM>(a.sc);   // (one request per tile: uniform)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = lp.odd ? 1 : 0;
     const int64_t P = a.n_points;
     const bool live = p < P;
@@ -180,31 +181,31 @@ __device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShare
     } else {
         lp_log_visibility<CULL>(a.sc, sh.sph, load_or(a.points, 3 * q, live), load_or(a.points, 3 * q + 1, live),
                                 load_or(a.points, 3 * q + 2, live),
-                                CULL ? unit_normal(nn.x, nn.y, nn.z) : Normal{}, lp, f);
+                                CULL ? cull_normal(a.sc, nn.x, nn.y, nn.z) : Normal{}, lp, f);
         k = -1;
     }
     const float n2 = lp_norm2(f, lp);
     if (k < 0) k = scaling_k(a.sc, n2);
 
     // ---- the exponential again, keeping in local memory f, the operand of
-    // every squaring and S with V = e0 S (EXP: U).  The operands of the
+    // every squaring and S with V = e0 S (projected: U).  The operands of the
     // products sit in the warp's columns of shared memory, X and Y (a product's
     // result and work arrays fill the registers).  kmax: the warp's largest k;
     // a pair past its own k keeps S.
     float* X = sh.w + warp * sh.region + lane;
     float* Y = X + 32 * NS;
-    float fh[NS], hist[EXP ? 1 : kMaxK + 1][NS];
+    float fh[NS], hist[EXPM == kExpProjected ? 1 : kMaxK + 1][NS];
     float scale = 1.f;
     OLCoef ol{1.f, 1.f, 0.f, 0.f};
     const float e0 = expf(lp_even(f[0]) * kInvSqrt4Pi);
-    const int kmax = EXP ? 0 : __reduce_max_sync(0xffffffffu, k);
+    const int kmax = projected ? 0 : __reduce_max_sync(0xffffffffu, k);
 #pragma unroll
     for (int s = 0; s < NS; ++s) fh[s] = f[s];
     {
         float S[NS];
-        if constexpr (EXP) {
-            lp_proj_exp(f, legs + kLegProduct, lp, S);
-        } else {
+        if (projected) {
+            if constexpr (EXPM != kExpSquarings) lp_proj_exp(f, legs + kLegProduct, lp, S);
+        } else if constexpr (EXPM != kExpProjected) {
             scale = ldexpf(1.f, -k);
             ol = ol_coef(a.sc, n2 * scale * scale);
 #pragma unroll
@@ -312,7 +313,7 @@ __device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShare
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
                 de0 = fmaf(T[s], hist[kmax][s], de0);
-                X[32 * s] = EXP ? T[s] : e0 * T[s];
+                X[32 * s] = projected ? T[s] : e0 * T[s];
             }
         } else {
             if (t < k) {
@@ -323,12 +324,14 @@ __device__ __forceinline__ void lp_tail_adjoint(const BwdArgs& a, const BwdShare
     }
 
     // ---- exponent
-    if constexpr (EXP) {
-        float dV[NS];
+    if (projected) {
+        if constexpr (EXPM != kExpSquarings) {
+            float dV[NS];
 #pragma unroll
-        for (int s = 0; s < NS; ++s) dV[s] = X[32 * s];
-        lp_proj_exp_adjoint(fh, dV, e0, legs + kLegProduct, lp, dfp);
-    } else {
+            for (int s = 0; s < NS; ++s) dV[s] = X[32 * s];
+            lp_proj_exp_adjoint(fh, dV, e0, legs + kLegProduct, lp, dfp);
+        }
+    } else if constexpr (EXPM != kExpProjected) {
         // S_0 = a(s) sqrt(4 pi), S_i = b(s) g_i: dg_i = b dS_i + (dA a'/s + dB b'/s) g_i
         const float dA = lp_even(X[0]) * kSqrt4Pi;
         float dBs = lp.odd ? X[0] * (fh[0] * scale) : 0.f;
@@ -426,7 +429,7 @@ __device__ __forceinline__ void lp_pairs(const BwdArgs& a, const BwdShared& sh, 
 // bands: 10.5 ms against 4.0 + 5.4 ms).
 constexpr int kPhaseBoth = 0, kPhaseTail = 1, kPhasePairs = 2;
 
-template <bool EXP, bool CULL, int PHASE>
+template <int EXPM, bool CULL, int PHASE>
 __device__ __forceinline__ void lp_backward_tile(const BwdArgs& a, const BwdShared& sh, int64_t tile) {
     const LanePair lp = lane_pair();
     const int row = threadIdx.x >> 1;
@@ -437,7 +440,7 @@ __device__ __forceinline__ void lp_backward_tile(const BwdArgs& a, const BwdShar
     if constexpr (PHASE == kPhasePairs) {
         lp_load(a.dfp_ws, a.n_points, live ? p : 0, live, lp, dfp);
     } else {
-        lp_tail_adjoint<EXP, CULL>(a, sh, p, dfp);
+        lp_tail_adjoint<EXPM, CULL>(a, sh, p, dfp);
     }
     if constexpr (PHASE == kPhaseTail) {
         if (pairs && live) lp_store(dfp, a.n_points, p, lp, a.dfp_ws);
@@ -452,7 +455,7 @@ __device__ __forceinline__ void lp_backward_tile(const BwdArgs& a, const BwdShar
 #pragma unroll
         for (int c = 0; c < 3; ++c) half[2 * c] = load_or(a.points, 3 * q + c, live);
     } else if (CULL) {
-        const Normal u = unit_normal(load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
+        const Normal u = cull_normal(a.sc, load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
                                      load_or(a.normals, 3 * q + 2, live));
         half[6] = u.x;
         half[8] = u.y;
@@ -486,11 +489,11 @@ __device__ __forceinline__ float lp_block_sum(const BwdShared& sh, int N, int e)
     return v;
 }
 
-#define SHS_LP_BWD_SHARED(EXP, PHASE)                                                        \
+#define SHS_LP_BWD_SHARED(EXPM, PHASE)                                                       \
     extern __shared__ __align__(16) float4 dyn[];                                            \
     __shared__ __align__(16) float s_light[3 * KPAD];                                        \
     __shared__ __align__(16) float s_lt[2][3][NSP];                                          \
-    __shared__ __align__(16) float s_leg[kLegProduct + ((EXP) ? kLegExp : 0)];               \
+    __shared__ __align__(16) float s_leg[kLegProduct + ((EXPM) ? kLegExp : 0)];              \
     __shared__ __align__(16) float s_w[NWARP * ((PHASE) == kPhasePairs ? kRowFloats : kWarpRegion)];                       \
     __shared__ float s_dl[NWARP][2][kDl], s_loss[NWARP];                                     \
     __shared__ __align__(8) uint64_t s_bar;                                                  \
@@ -507,19 +510,19 @@ __device__ __forceinline__ void clear_sums(const BwdShared& sh, int N) {
 //   [0, 3K)          d_light, channel-major
 //   [3K]             loss
 //   [3K+1, 3K+1+4N)  per sphere (d cx, d cy, d cz, d r)
-template <bool EXP, bool CULL, int PHASE>
+template <int EXPM, bool CULL, int PHASE>
 __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_lp_kernel(BwdArgs a) {
-    SHS_LP_BWD_SHARED(EXP, PHASE);
+    SHS_LP_BWD_SHARED(EXPM, PHASE);
     const int N = a.sc.n_spheres;
     const BwdShared sh{dyn, dyn + N, s_lt, s_leg, s_dl, s_loss, s_w, PHASE == kPhasePairs ? kRowFloats : kWarpRegion};
-    if (PHASE != kPhasePairs) load_rules(s_leg, EXP);
+    if (PHASE != kPhasePairs) load_rules(s_leg, EXPM != kExpSquarings);
     if (!stage_scene(a.sc, sh.sph, s_light, &s_bar)) return;
     clear_sums(sh, PHASE == kPhaseTail ? 0 : N);
     slot_lighting(s_light, s_lt);
 
     const int64_t ntiles = (a.n_points + kTile - 1) / kTile;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-        lp_backward_tile<EXP, CULL, PHASE>(a, sh, tile);
+        lp_backward_tile<EXPM, CULL, PHASE>(a, sh, tile);
 
     // ---- block reduction of the phase's entries, then one scene-level
     // reduction (by the last launch)
@@ -549,12 +552,12 @@ __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_lp_kernel(BwdArg
 // Adjoint for every tile of every request in the batch.  Each tile's scene
 // sums go to its request's accumulator with atomics; the tile that completes a
 // request writes that request's outputs.
-template <bool EXP, bool CULL>
+template <int EXPM, bool CULL>
 __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_batch_kernel(const __grid_constant__ BwdBatch b) {
-    SHS_LP_BWD_SHARED(EXP, kPhaseBoth);
+    SHS_LP_BWD_SHARED(EXPM, kPhaseBoth);
     __shared__ long long s_tile;
     const BwdShared sh{dyn, dyn + b.max_spheres, s_lt, s_leg, s_dl, s_loss, s_w, kWarpRegion};
-    load_rules(s_leg, EXP);
+    load_rules(s_leg, EXPM != kExpSquarings);
     mbar_init(&s_bar);
     int staged = -1;
     uint32_t parity = 0;
@@ -575,7 +578,7 @@ __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) backward_batch_kernel(con
         }
         clear_sums(sh, N);
         __syncthreads();
-        lp_backward_tile<EXP, CULL, kPhaseBoth>(a, sh, tile - b.tile_begin[r]);
+        lp_backward_tile<EXPM, CULL, kPhaseBoth>(a, sh, tile - b.tile_begin[r]);
         __syncthreads();
         const int E = 3 * K + 1 + 4 * N;
         for (int e = threadIdx.x; e < E; e += kBlock) add_tile_sum(a, e, lp_block_sum(sh, N, e));
@@ -595,12 +598,12 @@ size_t phase_dyn_smem(int phase, int n_spheres) {
     return phase == kPhaseTail ? static_cast<size_t>(n_spheres) * 16u : backward_dyn_smem(n_spheres);
 }
 
-template <bool EXP, bool CULL, int PHASE>
+template <int EXPM, bool CULL, int PHASE>
 cudaError_t launch_backward_lp(const BwdArgs& a, int grid, cudaStream_t s) {
     static DeviceOnce once;
-    const cudaError_t e = allow_dyn_smem(backward_lp_kernel<EXP, CULL, PHASE>, phase_dyn_smem(PHASE, kMaxSpheres), once);
+    const cudaError_t e = allow_dyn_smem(backward_lp_kernel<EXPM, CULL, PHASE>, phase_dyn_smem(PHASE, kMaxSpheres), once);
     if (e != cudaSuccess) return e;
-    backward_lp_kernel<EXP, CULL, PHASE>
+    backward_lp_kernel<EXPM, CULL, PHASE>
         <<<static_cast<unsigned>(grid), kBlock, phase_dyn_smem(PHASE, a.sc.n_spheres), s>>>(a);
     count_launch();
     return cudaGetLastError();
@@ -609,34 +612,33 @@ cudaError_t launch_backward_lp(const BwdArgs& a, int grid, cudaStream_t s) {
 template <int PHASE>
 cudaError_t launch_phase(const BwdArgs& a, int grid, cudaStream_t s) {
     const bool cull = a.sc.horizon_cull != 0, exp1 = PHASE != kPhasePairs && a.sc.exp_mode == 1;
-    if (exp1) {
-        return cull ? launch_backward_lp<PHASE != kPhasePairs, true, PHASE>(a, grid, s)
-                    : launch_backward_lp<PHASE != kPhasePairs, false, PHASE>(a, grid, s);
-    }
-    return cull ? launch_backward_lp<false, true, PHASE>(a, grid, s) : launch_backward_lp<false, false, PHASE>(a, grid, s);
+    constexpr int kExp1 = PHASE != kPhasePairs ? kExpProjected : kExpSquarings;
+    if (exp1) return cull ? launch_backward_lp<kExp1, true, PHASE>(a, grid, s) : launch_backward_lp<kExp1, false, PHASE>(a, grid, s);
+    return cull ? launch_backward_lp<kExpSquarings, true, PHASE>(a, grid, s)
+                : launch_backward_lp<kExpSquarings, false, PHASE>(a, grid, s);
 }
 
 template <int PHASE>
 int phase_blocks(int n_spheres) {
-    cudaFuncSetAttribute(backward_lp_kernel<false, false, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(backward_lp_kernel<kExpSquarings, false, PHASE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          static_cast<int>(phase_dyn_smem(PHASE, kMaxSpheres)));
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, backward_lp_kernel<false, false, PHASE>, kBlock,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, backward_lp_kernel<kExpSquarings, false, PHASE>, kBlock,
                                                       phase_dyn_smem(PHASE, n_spheres)) != cudaSuccess || nb < 1)
         nb = 1;
     return nb;
 }
 
-template <bool EXP, bool CULL>
+template <int EXPM, bool CULL>
 cudaError_t launch_backward_batch_lp(const BwdBatch& b, cudaStream_t s) {
     const size_t smem = backward_dyn_smem(b.max_spheres);
     static DeviceOnce once;
     static WaveCache wave;
     int grid = 0;
-    cudaError_t e = allow_dyn_smem(backward_batch_kernel<EXP, CULL>, backward_dyn_smem(kMaxSpheres), once);
-    if (e == cudaSuccess) e = one_wave(backward_batch_kernel<EXP, CULL>, smem, b.total_tiles, wave, &grid);
+    cudaError_t e = allow_dyn_smem(backward_batch_kernel<EXPM, CULL>, backward_dyn_smem(kMaxSpheres), once);
+    if (e == cudaSuccess) e = one_wave(backward_batch_kernel<EXPM, CULL>, smem, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
-    backward_batch_kernel<EXP, CULL><<<grid, kBlock, smem, s>>>(b);
+    backward_batch_kernel<EXPM, CULL><<<grid, kBlock, smem, s>>>(b);
     count_launch();
     return cudaGetLastError();
 }
@@ -652,12 +654,13 @@ BwdBlocks backward_blocks_per_sm<NB>(int n_spheres, bool split) {
 template <>
 cudaError_t launch_backward_batch<NB>(const BwdBatch& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
-    switch (b.variant) {
-        case 0: return launch_backward_batch_lp<false, false>(b, s);
-        case 1: return launch_backward_batch_lp<false, true>(b, s);
-        case 2: return launch_backward_batch_lp<true, false>(b, s);
-        default: return launch_backward_batch_lp<true, true>(b, s);
+    if (b.variant.squarings && b.variant.projected) return launch_backward_batch_lp<kExpAny, true>(b, s);
+    if (b.variant.projected) {
+        return b.variant.cull ? launch_backward_batch_lp<kExpProjected, true>(b, s)
+                              : launch_backward_batch_lp<kExpProjected, false>(b, s);
     }
+    return b.variant.cull ? launch_backward_batch_lp<kExpSquarings, true>(b, s)
+                          : launch_backward_batch_lp<kExpSquarings, false>(b, s);
 }
 
 template <>

@@ -9,7 +9,7 @@
 namespace shs {
 namespace {
 
-template <int MODE, bool EXP, bool CULL>
+template <int MODE, int EXPM, bool CULL>
 __device__ __forceinline__ void lp_forward_tile(const FwdArgs& a, const float4* s_sph, const float (*s_lt)[3][NSP],
                                                 const float* s_leg, int64_t tile) {
     const LanePair lp = lane_pair();
@@ -27,7 +27,7 @@ __device__ __forceinline__ void lp_forward_tile(const FwdArgs& a, const float4* 
         lp_load(a.saved_f, a.n_points, q, live, lp, f);
     } else {
         lp_log_visibility<CULL>(a.sc, s_sph, load_or(a.points, 3 * q, live), load_or(a.points, 3 * q + 1, live),
-                                load_or(a.points, 3 * q + 2, live), CULL ? unit_normal(nx, ny, nz) : Normal{}, lp, f);
+                                load_or(a.points, 3 * q + 2, live), CULL ? cull_normal(a.sc, nx, ny, nz) : Normal{}, lp, f);
         if (a.saved_f && live) lp_store(f, a.n_points, p, lp, a.saved_f);
         if constexpr (MODE == kFwdPairs) return;
     }
@@ -35,9 +35,10 @@ __device__ __forceinline__ void lp_forward_tile(const FwdArgs& a, const float4* 
     const float e0 = expf(lp_even(f[0]) * kInvSqrt4Pi);
     float V[NS];
     int k = 0;
-    if constexpr (EXP) {
-        lp_proj_exp(f, legs + kLegProduct, lp, V);
-    } else {
+    // (a tile belongs to one request: the branch is uniform)
+    if (projected_exp<EXPM>(a.sc)) {
+        if constexpr (EXPM != kExpSquarings) lp_proj_exp(f, legs + kLegProduct, lp, V);
+    } else if constexpr (EXPM != kExpProjected) {
         const float n2 = lp_norm2(f, lp);
         k = scaling_k(a.sc, n2);
         const float scale = ldexpf(1.f, -k);
@@ -68,18 +69,18 @@ __device__ __forceinline__ void lp_forward_tile(const FwdArgs& a, const float4* 
     }
 }
 
-template <int MODE, bool EXP, bool CULL>
+template <int MODE, int EXPM, bool CULL>
 __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) forward_lp_kernel(FwdArgs a) {
     __shared__ __align__(16) float4 s_sph[MODE == kFwdTail ? 1 : kMaxSpheres];
     __shared__ __align__(16) float s_light[3 * KPAD];
     __shared__ __align__(16) float s_lt[2][3][NSP];
-    __shared__ __align__(16) float s_leg[kLegProduct + (EXP ? kLegExp : 0)];
+    __shared__ __align__(16) float s_leg[kLegProduct + (EXPM ? kLegExp : 0)];
     __shared__ __align__(8) uint64_t s_bar;
     if (MODE == kFwdTail) a.sc.n_spheres = 0;
-    if (MODE != kFwdPairs) load_rules(s_leg, EXP);
+    if (MODE != kFwdPairs) load_rules(s_leg, EXPM != kExpSquarings);
     if (!stage_scene(a.sc, s_sph, s_light, &s_bar)) return;
     if (MODE != kFwdPairs) slot_lighting(s_light, s_lt);
-    lp_forward_tile<MODE, EXP, CULL>(a, s_sph, s_lt, s_leg, blockIdx.x);
+    lp_forward_tile<MODE, EXPM, CULL>(a, s_sph, s_lt, s_leg, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -89,15 +90,15 @@ __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) forward_lp_kernel(FwdArgs
 // Forward for every tile of every request in the batch.  Blocks take tiles
 // from a device counter (consecutive tiles mostly share a request, so a
 // request's scene is staged once per run of its tiles).
-template <bool EXP, bool CULL>
+template <int EXPM, bool CULL>
 __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) forward_batch_kernel(const __grid_constant__ FwdBatch b) {
     __shared__ __align__(16) float4 s_sph[kMaxSpheres];
     __shared__ __align__(16) float s_light[3 * KPAD];
     __shared__ __align__(16) float s_lt[2][3][NSP];
-    __shared__ __align__(16) float s_leg[kLegProduct + (EXP ? kLegExp : 0)];
+    __shared__ __align__(16) float s_leg[kLegProduct + (EXPM ? kLegExp : 0)];
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ long long s_tile;
-    load_rules(s_leg, EXP);
+    load_rules(s_leg, EXPM != kExpSquarings);
     mbar_init(&s_bar);
     int staged = -1;
     uint32_t parity = 0;
@@ -115,7 +116,7 @@ __global__ void __launch_bounds__(kBlock, SHS_LP_MINB) forward_batch_kernel(cons
             staged = r;
             slot_lighting(s_light, s_lt);
         }
-        lp_forward_tile<kFwdFull, EXP, CULL>(a, s_sph, s_lt, s_leg, tile - b.tile_begin[r]);
+        lp_forward_tile<kFwdFull, EXPM, CULL>(a, s_sph, s_lt, s_leg, tile - b.tile_begin[r]);
     }
 }
 
@@ -124,21 +125,22 @@ cudaError_t launch_forward_lp(const FwdArgs& a, cudaStream_t s) {
     const unsigned blocks = static_cast<unsigned>((a.n_points + kTile - 1) / kTile);
     const bool exp1 = MODE != kFwdPairs && a.sc.exp_mode == 1;      // the pair pass has no exponential
     const bool cull = MODE != kFwdTail && a.sc.horizon_cull != 0;   // the tail has no spheres
-    if (exp1 && cull) forward_lp_kernel<MODE, MODE != kFwdPairs, MODE != kFwdTail><<<blocks, kBlock, 0, s>>>(a);
-    else if (exp1) forward_lp_kernel<MODE, MODE != kFwdPairs, false><<<blocks, kBlock, 0, s>>>(a);
-    else if (cull) forward_lp_kernel<MODE, false, MODE != kFwdTail><<<blocks, kBlock, 0, s>>>(a);
-    else forward_lp_kernel<MODE, false, false><<<blocks, kBlock, 0, s>>>(a);
+    constexpr int kExp1 = MODE != kFwdPairs ? kExpProjected : kExpSquarings;
+    if (exp1 && cull) forward_lp_kernel<MODE, kExp1, MODE != kFwdTail><<<blocks, kBlock, 0, s>>>(a);
+    else if (exp1) forward_lp_kernel<MODE, kExp1, false><<<blocks, kBlock, 0, s>>>(a);
+    else if (cull) forward_lp_kernel<MODE, kExpSquarings, MODE != kFwdTail><<<blocks, kBlock, 0, s>>>(a);
+    else forward_lp_kernel<MODE, kExpSquarings, false><<<blocks, kBlock, 0, s>>>(a);
     count_launch();
     return cudaGetLastError();
 }
 
-template <bool EXP, bool CULL>
+template <int EXPM, bool CULL>
 cudaError_t launch_forward_batch_lp(const FwdBatch& b, cudaStream_t s) {
     static WaveCache wave;
     int grid = 0;
-    const cudaError_t e = one_wave(forward_batch_kernel<EXP, CULL>, 0, b.total_tiles, wave, &grid);
+    const cudaError_t e = one_wave(forward_batch_kernel<EXPM, CULL>, 0, b.total_tiles, wave, &grid);
     if (e != cudaSuccess) return e;
-    forward_batch_kernel<EXP, CULL><<<grid, kBlock, 0, s>>>(b);
+    forward_batch_kernel<EXPM, CULL><<<grid, kBlock, 0, s>>>(b);
     count_launch();
     return cudaGetLastError();
 }
@@ -148,12 +150,13 @@ cudaError_t launch_forward_batch_lp(const FwdBatch& b, cudaStream_t s) {
 template <>
 cudaError_t launch_forward_batch<NB>(const FwdBatch& b, cudaStream_t s) {
     if (b.total_tiles <= 0) return cudaSuccess;
-    switch (b.variant) {
-        case 0: return launch_forward_batch_lp<false, false>(b, s);
-        case 1: return launch_forward_batch_lp<false, true>(b, s);
-        case 2: return launch_forward_batch_lp<true, false>(b, s);
-        default: return launch_forward_batch_lp<true, true>(b, s);
+    if (b.variant.squarings && b.variant.projected) return launch_forward_batch_lp<kExpAny, true>(b, s);
+    if (b.variant.projected) {
+        return b.variant.cull ? launch_forward_batch_lp<kExpProjected, true>(b, s)
+                              : launch_forward_batch_lp<kExpProjected, false>(b, s);
     }
+    return b.variant.cull ? launch_forward_batch_lp<kExpSquarings, true>(b, s)
+                          : launch_forward_batch_lp<kExpSquarings, false>(b, s);
 }
 
 template <>

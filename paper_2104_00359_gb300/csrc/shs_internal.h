@@ -80,21 +80,24 @@ struct BwdArgs {
                              // and lighting / loss rows are written
 };
 
-// A batch: up to kMaxBatch requests (of one band count) whose 128-point tiles
-// form one work list; a persistent grid pulls tiles from a device counter.
+// A batch: up to kMaxBatch requests (of one band count) whose tiles of
+// tile_points(n_bands) points form one work list; a persistent grid pulls tiles from a device counter.
 constexpr int kMaxBatch = 32;
 
-// From 6 bands the requests of one batch kernel also share a variant (bit 0:
-// horizon culling, bit 1: projected exponential), which the kernel is compiled
-// for.
-constexpr int batch_variants(int n_bands) { return n_bands >= 6 ? 4 : 1; }
-inline int batch_variant(const SceneView& sc, int n_bands) {
-    return n_bands >= 6 ? (sc.horizon_cull ? 1 : 0) + (sc.exp_mode == 1 ? 2 : 0) : 0;
-}
+// What the requests of a batch ask for, which the kernels from 6 bands are
+// compiled for: horizon culling (no request, or some: the kernel then asks each
+// scene), and the exponential (scaling and squarings; projected; both).
+struct BatchVariant {
+    bool cull = false, squarings = false, projected = false;
+    void add(const SceneView& sc) {
+        cull = cull || sc.horizon_cull;
+        (sc.exp_mode == 1 ? projected : squarings) = true;
+    }
+};
 
 struct FwdBatch {
     int n;
-    int variant;
+    BatchVariant variant;
     int64_t total_tiles;
     int64_t tile_begin[kMaxBatch + 1];   // prefix sums of tiles per request
     unsigned int* queue;                  // zero before launch
@@ -103,7 +106,7 @@ struct FwdBatch {
 
 struct BwdBatch {
     int n;
-    int variant;
+    BatchVariant variant;
     int max_spheres;
     int64_t total_tiles;
     int64_t tile_begin[kMaxBatch + 1];
