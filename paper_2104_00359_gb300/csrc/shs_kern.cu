@@ -58,7 +58,7 @@ __device__ __forceinline__ void cap_closed(float c, float s2, float* G, float* P
 // The pair terms are accumulated in the monomial basis: for each band l the
 // pair adds G_l(c) x^a y^b z^c (a+b+c = l) at s_hat, and the harmonic
 // combination is taken once per point (mono_to_f).
-static_assert(NB <= 5, "from 6 bands: shs_kern_hi.cu");
+static_assert(NB <= 5, "from 6 bands: shs_hi_forward.cu, shs_hi_backward.cu");
 constexpr int NACC = SH::NA;
 
 // One pair's un-normalised log-visibility terms, added to acc.
@@ -767,8 +767,8 @@ __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_
 //   [0, 3K)          d_light, channel-major
 //   [3K]             loss
 //   [3K+1, 3K+1+4N)  per sphere (d cx, d cy, d cz, d r)
-// Up to 4 bands: four resident blocks per SM (<= 128 registers per thread) for
-// the pair loop; above that the tail state needs the registers.
+// Up to 4 bands: three resident blocks per SM (167 or 168 registers per thread)
+// for the pair loop; above that the tail state needs the registers.
 template <int CULLM, int EXPM>
 __global__ void __launch_bounds__(kBlock, NB <= 4 ? SHS_BWD_MINB : 1) backward_kernel_t(BwdArgs a) {
     extern __shared__ __align__(16) float4 dyn[];

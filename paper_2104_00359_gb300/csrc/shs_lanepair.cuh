@@ -17,7 +17,8 @@
 // all four values, so a circle of 24 azimuths takes 6 x 15 multiply-adds where
 // evaluating each azimuth takes 24 x 15.  An 8-band square is about 5.2 k
 // FP32 instructions against 13.7 k for the plain separable rule, and no
-// operand lives in local memory.  Measured against one thread per point with
+// operand of the forward pass lives in local memory (the adjoint keeps f and
+// the operands of the squarings there: 2.8 KB a thread at 8 bands).  Measured against one thread per point with
 // the plain rule (8 bands, 300 spheres, 1M points): forward 5.62 -> 3.1 ms
 // (with the pair terms of shs_hi.cuh), adjoint 17.1 -> 9.3 ms; projected
 // exponential, forward 4.18 -> 2.61 ms; 6 bands (unrolled Gaunt products
