@@ -445,7 +445,19 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? SHS_FWD_MINB : 1) forward_ke
 // backward kernel
 // ---------------------------------------------------------------------------
 
-// Pair adjoints of the warp's 32 points from 32 spheres on.  A pair of lanes
+// The point gradients of lane pairs that each hold a row: sums over the pair's
+// spheres, written by the row's point h on lane 2 r + h.
+__device__ __forceinline__ void store_row_points(const BwdArgs& a, float2* gp, int64_t p0, int lane) {
+    const int64_t p = p0 + lane;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        gp[e].x += __shfl_xor_sync(0xffffffffu, gp[e].x, 1);
+        gp[e].y += __shfl_xor_sync(0xffffffffu, gp[e].y, 1);
+        if (p < a.n_points) a.d_points[3 * p + e] = -((lane & 1) ? gp[e].y : gp[e].x);
+    }
+}
+
+// Pair adjoints of the warp's 32 points from 31 spheres on.  A pair of lanes
 // holds a row's coefficients in registers and takes every second sphere; the
 // rows walk the spheres at different offsets, so the 32 lanes update 32
 // distinct slots of the warp's sphere sums with plain shared-memory
@@ -484,24 +496,61 @@ __device__ __forceinline__ void warp_pairs(const BwdArgs& a, const float4* s_sph
         __syncwarp();
         m = m + 1 == M ? 0 : m + 1;
     }
-    if (!a.d_points) return;
-    // the row's point h is this lane's
-    const int64_t p = p0 + lane;
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-        gp[e].x += __shfl_xor_sync(0xffffffffu, gp[e].x, 1);
-        gp[e].y += __shfl_xor_sync(0xffffffffu, gp[e].y, 1);
-        if (p < a.n_points) a.d_points[3 * p + e] = -(h ? gp[e].y : gp[e].x);
-    }
+    if (a.d_points) store_row_points(a, gp, p0, lane);
 }
 
-// Fewer than 32 spheres: the lanes hold `width` spheres (32, 16 or 8, then one,
-// two or four rows at once); a row's sums stay in registers over the spheres
-// and are summed over the lanes once.
+// Fewer spheres: rows on the lane pairs as above, every row at the same two
+// spheres, whose sums over the rows take five shuffles.  (Spheres on the lanes,
+// below, need 24 or 30 shuffles a row for the points, and as many steps for 17
+// spheres as for 32: 262k points, 4 bands, 20 spheres, adjoint with point
+// gradients 118 against 71 us, without 80 against 70 us.)
+template <bool CULL>
+__device__ __forceinline__ void warp_pairs_rows(const BwdArgs& a, const float4* s_sph, const float4* rows,
+                                                const float2 (*nrm)[3], float4* acc_row, int64_t p0, int lane) {
+    const int N = a.sc.n_spheres, r = lane >> 1, h = lane & 1;
+    float2 q[kRowUsed + 1], u[3] = {}, gp[3] = {};
+    load_row(rows + r * (kRow / 2), q);
+    if constexpr (CULL) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e) u[e] = nrm[r][e];
+    }
+    float* acc = reinterpret_cast<float*>(acc_row);
+#pragma unroll 1
+    for (int j = h; j - h < N; j += 2) {
+        const bool has = j < N;
+        const float4 sp = has ? s_sph[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float2 d[4];
+        pair_backward2<CULL>(sp, q, d, u);
+        if (!has) d[0] = d[1] = d[2] = d[3] = make_float2(0.f, 0.f);
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = d[e].x + d[e].y;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) gp[e] = __fadd2_rn(gp[e], d[e]);
+        // halving exchanges: lane bits 4 and 3 end up with component 0 .. 3
+        const bool up = lane & 16, up2 = lane & 8;
+        const float s0 = up ? v[0] : v[2], s1 = up ? v[1] : v[3];
+        v[0] = (up ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, s0, 16);
+        v[1] = (up ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, s1, 16);
+        const float s2 = up2 ? v[0] : v[1];
+        v[0] = (up2 ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, s2, 8);
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 4);
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+        if (has && (lane & 6) == 0) acc[4 * j + (lane >> 3)] += v[0];
+    }
+    __syncwarp();
+    if (a.d_points) store_row_points(a, gp, p0, lane);
+}
+
+// ... or, without point gradients and with the lanes at least 7/8 full: the lanes
+// hold `width` spheres (32, 16 or 8, then one, two or four rows at once), whose
+// sums stay in registers over the rows (3 bands, 16 spheres, 37 against 40 us).
+__device__ __forceinline__ int few_width(int N) { return N > 16 ? 32 : N > 8 ? 16 : 8; }
+
 template <bool CULL>
 __device__ __forceinline__ void warp_pairs_few(const BwdArgs& a, const float4* s_sph, const float4* rows,
-                                               const float2 (*nrm)[3], float4* acc_row, int64_t p0, int lane) {
-    const int N = a.sc.n_spheres, width = N > 16 ? 32 : N > 8 ? 16 : 8, sub = lane / width, stride = 32 / width;
+                                               const float2 (*nrm)[3], float4* acc_row, int lane) {
+    const int N = a.sc.n_spheres, width = few_width(N), sub = lane / width, stride = 32 / width;
     const int j = lane % width;
     const bool has = j < N;
     const float4 sp = has ? s_sph[j] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -515,20 +564,6 @@ __device__ __forceinline__ void warp_pairs_few(const BwdArgs& a, const float4* s
         if (!has) d[0] = d[1] = d[2] = d[3] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[e] = __fadd2_rn(acc[e], d[e]);
-        if (a.d_points) {
-#pragma unroll
-            for (int e = 0; e < 3; ++e)
-                for (int o = 1; o < width; o <<= 1) {
-                    d[e].x += __shfl_xor_sync(0xffffffffu, d[e].x, o);
-                    d[e].y += __shfl_xor_sync(0xffffffffu, d[e].y, o);
-                }
-            // six lanes of the sub-group write the row's two points
-            const int64_t p = p0 + 2 * r + j / 3;
-            if (j < 6 && p < a.n_points) {
-                const float2 v = j % 3 == 0 ? d[0] : j % 3 == 1 ? d[1] : d[2];
-                a.d_points[3 * p + j % 3] = -(j < 3 ? v.x : v.y);
-            }
-        }
     }
     float s[4];
 #pragma unroll
@@ -752,8 +787,9 @@ __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_
     auto loops = [&](auto cull_tag) {
         constexpr bool CULL = decltype(cull_tag)::value;
         const int64_t p0 = tile * kBlock + warp * 32;
-        if (N >= 32) warp_pairs<CULL>(a, s_sph, rows, nrm, acc_row, p0, lane);
-        else warp_pairs_few<CULL>(a, s_sph, rows, nrm, acc_row, p0, lane);
+        if (N >= 2 * kWarpRows - 1) warp_pairs<CULL>(a, s_sph, rows, nrm, acc_row, p0, lane);
+        else if (a.d_points || 8 * N < 7 * few_width(N)) warp_pairs_rows<CULL>(a, s_sph, rows, nrm, acc_row, p0, lane);
+        else warp_pairs_few<CULL>(a, s_sph, rows, nrm, acc_row, lane);
     };
     if constexpr (CULLM == 2) {
         if (a.sc.horizon_cull) loops(std::true_type{});
