@@ -582,6 +582,14 @@ __device__ __forceinline__ void warp_pairs_few(const BwdArgs& a, const float4* s
     __syncwarp();
 }
 
+// From 4 bands a block's warps start each tile, and go on from the squarings
+// (whose number differs by point), together: the unrolled code is larger than
+// the instruction cache, and warps that drift apart fetch it again and again
+// (1M points, 12 spheres, adjoint: 5 bands 2,113 -> 625 us, 4 bands 242 -> 222).
+__device__ __forceinline__ void keep_together() {
+    if constexpr (NB >= 4) __syncthreads();
+}
+
 // Adjoint of one 128-point tile of one request: per-point outputs are written,
 // the scene-level sums are added to the block's shared accumulators
 // (s_dl: d_light and loss per warp, s_acc: per warp and sphere).
@@ -660,6 +668,7 @@ __device__ __forceinline__ void backward_tile(const BwdArgs& a, const float4* s_
 #pragma unroll
         for (int i = 0; i < K; ++i) V[i] = e0 * S[i];
     }
+    keep_together();
     float H[K], ux, uy, uz, il;
     cosine_lobe(load_or(a.normals, 3 * q, live), load_or(a.normals, 3 * q + 1, live),
                 load_or(a.normals, 3 * q + 2, live), H, ux, uy, uz, il);
@@ -825,8 +834,10 @@ __global__ void __launch_bounds__(kBlock, NB <= 4 ? SHS_BWD_MINB : 1) backward_k
     __syncthreads();
 
     const int64_t ntiles = (a.n_points + kBlock - 1) / kBlock;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        keep_together();
         backward_tile<CULLM, EXPM>(a, s_sph, s_light, s_acc, s_dl, s_rows, s_nrm, tile, lane, warp);
+    }
 
     // ---- block reduction, then one scene-level reduction
     __syncthreads();

@@ -41,3 +41,11 @@ def test_point_gradients_of_few_spheres(n):
     lanes per row of points made them 1.5 to 1.8 times the whole)."""
     sub = _adjoint_us(n, 1 << 18, 20, ("light", "albedo", "centers", "radii"))
     assert _adjoint_us(n, 1 << 18, 20) < 1.3 * sub
+
+
+@pytest.mark.parametrize("n", [4, 5])
+def test_squarings_that_differ_by_point(n):
+    """1M points whose squarings number 0 to 4 against two for each (warps that
+    drift apart in code larger than the instruction cache: 4 times at 5 bands)."""
+    two = _adjoint_us(n, 1 << 20, 12, ("light", "albedo", "centers", "radii"), fixed_k=2)
+    assert _adjoint_us(n, 1 << 20, 12, ("light", "albedo", "centers", "radii")) < 2.0 * two
