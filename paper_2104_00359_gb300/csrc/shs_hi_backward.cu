@@ -426,7 +426,7 @@ __device__ __forceinline__ void lp_pairs(const BwdArgs& a, const BwdShared& sh, 
 // dfp_ws, kPhasePairs reads them), each of which keeps to one region of code:
 // as one launch (kPhaseBoth, for callers without a workspace) the kernel waits
 // on instruction fetch (1.1 stalled warps per issue; 1M points, 300 spheres, 8
-// bands: 10.5 ms against 4.0 + 5.4 ms).
+// bands: 9.2 ms against 8.6 ms).
 constexpr int kPhaseBoth = 0, kPhaseTail = 1, kPhasePairs = 2;
 
 template <int EXPM, bool CULL, int PHASE>

@@ -20,7 +20,7 @@
 // operand of the forward pass lives in local memory (the adjoint keeps f and
 // the operands of the squarings there: 2.8 KB a thread at 8 bands).  Measured against one thread per point with
 // the plain rule (8 bands, 300 spheres, 1M points): forward 5.62 -> 3.1 ms
-// (with the pair terms of shs_hi.cuh), adjoint 17.1 -> 9.3 ms; projected
+// (with the pair terms of shs_hi.cuh), adjoint 17.1 -> 8.6 ms; projected
 // exponential, forward 4.18 -> 2.61 ms; 6 bands (unrolled Gaunt products
 // before), exponential and shading of 200k points 152 -> 75 us.
 #pragma once

@@ -14,7 +14,7 @@
 // tested against the triangle and the (depth, face) key of each covered
 // pixel folded into a 64-bit atomicMin depth buffer; per pixel, the winning
 // triangle's colour.  Four lanes share a triangle: a warp then waits for the
-// longest of 8 bounding boxes instead of 32 (99k triangles at 1024^2: 29 -> 20
+// longest of 8 bounding boxes instead of 32 (99k triangles at 1024^2: 29 -> 21
 // us).
 //
 // The adjoint runs per pixel.  Its atomics are the bound: a thread takes

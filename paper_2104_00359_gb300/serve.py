@@ -67,8 +67,10 @@ SMALL_WORK = 1.0e8
 
 def task_work(points, spheres, n_bands, op):
     """Work estimate of one task: point-sphere pairs weighted by the band
-    count's cost per pair (relative to 4 bands), the adjoint counted as
-    forward + 2.5 x forward."""
+    count's cost per pair (relative to 4 bands: the pair loop's, 0.65, 1.45, 2.0
+    and 3.4 at 3, 5, 6 and 8 bands; whole forward passes of 262k points and 200
+    spheres take 0.66, 1.9, 3.0 and 5.7), the adjoint counted as forward +
+    2.5 x forward (measured 2.4 to 2.7)."""
     per_pair = (n_bands * n_bands + 4.0) / 20.0
     return points * max(spheres, 1) * per_pair * (3.5 if op == "fwdbwd" else 1.0)
 
